@@ -2,82 +2,99 @@
 //     Y = X . deq(Wq) + (X . A) . B,
 // streaming every weight byte exactly once.
 //
-// Work decomposition.  All three matrices are stored as blobs of 16 rows x 128 reduction elements,
-// ordered pair-major (see eora_common.cuh), and every blob is an independent piece of work: a warp
-// multiplies it with the 128 activations it needs (kept in registers as tensor-core operand
-// fragments, tokens as the n8 side of the MMA) and adds the 16 x m partial sums to an fp32
-// accumulator array in global memory with red.add.  Blobs of a 3/4-bit backbone go through an integer
-// product (mma.m16n8k32 on the byte codes against two byte planes of 16-bit block fixed point activations,
-// see decode_common.cuh), all other blobs (adapters, 2:4 backbones) are dequantised to exact fp16 integers
-// and go through mma.m16n8k16.  Warps are fully independent: each owns a
-// contiguous run of blobs of up to three matrices, fetches it with its own bulk copies into its own
-// shared-memory ring and never synchronises with another warp of its CTA.
+// What bounds it.  A decode launch moves 3 - 50 MB, 0.5 - 7 us at the HBM's rate, and is one of a chain of dependent
+// launches; most of its time is latency, not bandwidth: instructions at 6 to 10 cycles each in the parts that run once per
+// CTA, an L2 round trip for the activations and one for t, and the products themselves (about 100 instructions per blob).
+// So the kernel is built around the chain
+//     previous launch ends -> activations arrive -> products -> sums -> Y
+// and keeps everything that is not in it out of the way:
+//   * A CTA owns whole row tiles of the output over half of the reduction axis, its cluster partner the other half.  The
+//     sums of a row tile meet in the shared memory of the two CTAs; nothing goes through atomics or tickets in global
+//     memory (a release, a ticket and a read-back cost 1.8 us of a 2.8 us launch measured on their own).
+//   * A's rows belong to CTAs of their own ([0, n_a), dispatched first), which send t = X . A to everybody as 8-byte
+//     words of (value, launch number): a reader that sees the number has the value, so the exchange is one store and
+//     one polling load, no fence, counter or reset.  Only t is waited for, and only by CTAs that come later in the
+//     grid than the ones they wait for, which themselves never wait.  The wait is bounded.
+//   * One token: eight warps of 128 registers and half of an SM's shared memory, so that the next launch's CTAs are
+//     resident and have their first weights in their rings while this one runs (programmatic dependent launch), and four
+//     blobs at once per warp.  More tokens: sixteen warps and a whole SM (the products need the issue slots).
+//     Asking for all of the next launch's weights ahead (bulk prefetches into L2) was slower, 183 against 172 us for four
+//     blocks: the activations and t, which the launch in front is waiting for, then queue behind that traffic.
+// Measured, four LLaMA3-8B blocks of four launches, fp16 adapters of rank 128: 3-bit, one token 194 -> 173 us; eight tokens
+// 303 -> 278 us; two blocks of a 2:4 backbone, one token 143 -> 132 us (the figures before: warps that added their
+// partial sums of single blobs to global memory and counted tickets).
 //
-//   * the first warps ("A owners") take the blobs of A first (t += X . A, sums in d_t) and then a share of W,
-//   * the last warps ("B owners") take one copy of W, then their blobs of B, for which the activations are t
-//     (read back as fp32 and split into an fp16 high and low part, so that t keeps fp32-like accuracy),
-//     then the rest of their share of W,
-//   * the warps in between take backbone blobs only.
-// The only wait in the kernel is the one before the B share: all of A must have been added to t.  A
-// owners never wait, and they sit in the first half of the CTAs, which are dispatched first and hold no B
-// owner, so a waiting warp never holds the place of a CTA it is waiting for.  The wait is bounded like every other.
-//
-// Completion.  Every blob of W or B that has been added to y_ws bumps the ticket of its row tile; the
-// warp that brings a ticket to its final count converts the 16 x m sums to the output type, writes Y and
-// puts the sums and the ticket back to zero.  The warp that finishes the last row tile also clears t
-// and the counters, so all scratch is back to zero when the kernel ends.
-//
-// Programmatic dependent launch: the first bulk copies (weights never change) are issued before
-// griddepcontrol.wait, i.e. while the previous kernel in the stream is still draining; activations
-// and scratch are only touched after it.
+// Work of a CTA.  Its blobs (16 rows x 128 reduction elements, see eora_common.cuh) in the order (chunk of the reduction
+// axis, row tile, pair) are cut into equal runs, one per warp.  The activations of a chunk sit in shared memory
+// in the form the products read: for one token and a 3/4-bit backbone as the byte planes of a 16-bit block fixed point
+// number (integer tensor-core product, decode_common.cuh), else as fp16.  A warp keeps the sums of a row tile in
+// registers and leaves them in a slot of its own when its run goes on to the next tile.
+#include <type_traits>
 #include "decode_common.cuh"
 
 namespace eora {
 namespace {
 using namespace dec;
 
-// One CTA of sixteen warps per SM.  The warps of a CTA start together; with several smaller CTAs per SM the ones that
-// are placed last ran a fifth slower than the first (the scheduler prefers the older warps) and ended the kernel late.
-constexpr int kWarps = 16;
-constexpr int kThreads = kWarps * 32;
-constexpr int kCtasPerSm = 1;
-constexpr int kRing = 2;                  // bulk copies in flight per warp
-constexpr int kSlotBytes = 6528;          // one ring slot = one bulk copy (a run of whole blobs: eight 3-bit, six 4-bit ones)
-constexpr int kBarBytes = 512;            // kWarps * kRing mbarriers
-constexpr int kSmemBytes = kWarps * kRing * kSlotBytes + kBarBytes + kSp24LutBytes;
+// Warps per CTA (log2), by the kind of product.
+__host__ __device__ constexpr int warp_log(int mode) { return mode == 1 ? 3 : 4; }
+constexpr int kMaxTok = 8;                // tokens per launch (the n8 side of the mma)
+constexpr int kMaxSlices = 4;             // parts of the reduction axis that t may be sent in
+constexpr uint32_t kLaunchShift = 10;     // a launch adds 2^10 to the launch counter (at most 1023 CTAs)
+constexpr int kMaxTiles = 48;             // row tiles per cluster (what its shared memory is sized for); more: further CTAs, in waves
+constexpr int kXBytes = 58 * 1024;        // activations of a chunk: 28 pairs of eight tokens
+constexpr int kMaxSmem = 226 * 1024;
+constexpr int kHalfSmem = 112 * 1024;     // what two CTAs of an SM may use each
+constexpr int kMaxSlots = 4;
+constexpr int kPlaneBytes = 272;          // integer path: two byte planes of a pair (256 B), scale and two sums
 
-enum { CNT_A_DONE = 0, CNT_TILES_DONE = 1, CNT_TICKET0 = 2 };
-
-struct Share { uint32_t per, rem; };      // blobs of a matrix dealt to n warps: warp i gets per + (i < rem)
+struct Share { uint32_t per, rem; };      // items dealt to n takers: taker i gets per + (i < rem)
 
 struct DecodeArgs {
   const uint8_t* a_q; const uint8_t* w_q; const uint8_t* b_q;
-  uint32_t a_nt, w_nt;                    // row tiles of A and of W (= of B)
-  uint32_t a_blobs;                       // all of A
-  uint32_t a_per_copy, w_per_copy, b_per_copy;   // blobs per bulk copy
-  uint32_t a_sz2, w_sz2, b_sz2;
-  // Three groups of warps: [0, n1) hold the blobs of A ("A owners"), [n1, n12) only backbone blobs,
-  // [n12, all) the blobs of B.  Every group has its own share of the backbone, starting at w_base[group].
-  uint32_t n1, n12;
-  Share sh_a, sh_b, sh_w[3];
-  uint32_t w_base[3];
-  uint32_t tile_target;                   // blobs per output row tile: pairs of W + pairs of B
+  int a_fmt;                              // format of A and B (FMT_NONE: no adapter)
+  uint32_t a_sz2, b_sz2;
+  uint32_t a_nt, a_np;                    // A: row tiles, pairs
+  uint32_t n_a, a_slices, a_slice_pairs;  // CTAs that hold A; parts of its reduction axis, pairs per part
+  uint32_t ks;                            // CTAs per cluster = parts of W's reduction axis (1 or 2)
+  uint32_t w_nt, w_np, pairs;             // W: row tiles, pairs; pairs per part (of the first)
+  uint32_t chunk;                         // pairs whose activations are in shared memory at a time
+  Share tiles;                            // row tiles of W dealt to the clusters
+  // Of each part: its pairs, and for CTAs with tiles.per / tiles.per + 1 row tiles ceil(2^32 / blobs) (whole runs) -- reciprocals
+  // for the places where a CTA would divide.
+  struct Part { uint32_t pairs, inv_pairs, inv_blobs[2]; } part[2];
+  uint32_t b_np;                          // pairs of B per row tile
+  uint32_t t_chunk;                       // pairs of t in shared memory at a time
+  uint32_t b_log;                         // log2 of the warps that share a row tile's pairs of a chunk
+  uint32_t slots, slot_blobs, ring_pitch; // a warp's ring of weights: slots of whole blobs; bytes from one warp's ring to the next
+  uint32_t off_bar, off_ring, off_seg, off_inbox, off_sum, off_bseg, off_t;   // shared memory (bytes from the start): see the kernel
   const void* x;
   void* ys[4];                            // outputs of the fused layers (one for a plain layer)
-  uint32_t sub_tile0[5];                  // layer i owns row tiles [sub_tile0[i], sub_tile0[i+1])
+  uint32_t sub_tile0[5];                  // layer i owns row tiles [sub_tile0[i], sub_tile0[i + 1]) and pairs [i, i + 1) * sub_pairs of t
   int sub_dout[4];
   int n_sub;
-  uint32_t b_np;                          // pairs of B per layer: the activations of B's blob (pair, tile) are
-                                          // pair (layer(tile) * b_np + pair) of t
-  // Several adapters on one backbone: pair p of B belongs to adapter p / adp_pairs, and token i uses adapter
+  uint32_t sub_pairs;                     // 0: every row tile takes part in all pairs of t (plain layer, several adapters)
+  // Several adapters on one backbone: pair p of t belongs to adapter p / adp_pairs, and token i uses adapter
   // adp[i] (-1: none).  adp_pairs == 0: one adapter for all tokens.
   uint32_t adp_pairs;
-  int adp[8];
-  float* d_t; float* y_ws; uint32_t* counters; int* dev_status;
-  int m, d_in, r_pad, n_pad, x_dtype, y_dtype;   // r_pad: columns of t (all fused layers / adapters)
+  int adp[kMaxTok];
+  unsigned long long* t_part;             // [slices][m][t_cols] words (value, launch number)
+  unsigned long long* launches;           // launch counter
+  int* dev_status;
+  int m, m_log;                           // tokens; log2 of the next power of two
+  int d_in, t_cols, x_dtype, y_dtype;
   unsigned long long wait_ns;             // limit of the wait for t
   unsigned long long* trace;
 };
+
+// Reads a word of every 64 bytes of the arguments.  They are new with every launch, and the first read of a line of them goes to
+// L2; done here, that happens while the launch in front still runs instead of piece by piece in the middle of the kernel.
+__device__ __forceinline__ void touch_args(const DecodeArgs& p) {
+  const uint32_t* w = reinterpret_cast<const uint32_t*>(&p);
+#pragma unroll
+  for (int i = 0; i < (int)(sizeof(DecodeArgs) / 4); i += 16) asm volatile("" ::"r"(w[i]));
+  asm volatile("" ::"r"(w[sizeof(DecodeArgs) / 4 - 1]));
+}
 
 __device__ __forceinline__ uint32_t share_lo(const Share& s, uint32_t i) { return i * s.per + (i < s.rem ? i : s.rem); }
 __device__ __forceinline__ uint32_t share_n(const Share& s, uint32_t i) { return s.per + (i < s.rem ? 1u : 0u); }
@@ -94,532 +111,784 @@ __device__ __forceinline__ uint32_t pack_h2(float a, float b) {
 __device__ __forceinline__ uint32_t bf2_to_h2(uint32_t v) {
   return pack_h2(__uint_as_float(v << 16), __uint_as_float(v & 0xffff0000u));
 }
+__device__ __forceinline__ void prefetch_l2(const void* p, uint32_t bytes) {
+  asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p), "r"(bytes) : "memory");
+}
+__device__ __forceinline__ unsigned long long ld_volatile_u64(const unsigned long long* p) {
+  unsigned long long v;
+  asm volatile("ld.volatile.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
+  return v;
+}
+__device__ __forceinline__ uint32_t mapa(uint32_t addr, uint32_t rank) {
+  uint32_t r;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
+  return r;
+}
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
 
-// Activation fragments of one pair (128 reduction elements) for lane (g, t): token g, elements
-// 64*c + 32*blk + 8*t + [0, 8) in xr[8*c + 4*blk + 0..3].
-__device__ __forceinline__ void load_x_pair(uint32_t (&xr)[16], const DecodeArgs& p, uint32_t pair, int lane) {
-  const int g = lane >> 2, t = lane & 3;
-  if (g < p.m) {
-    const uint16_t* src = reinterpret_cast<const uint16_t*>(p.x) + (size_t)g * p.d_in + pair * 128 + 8 * t;
-    uint4 u[4];                            // all loads first: a use in between would serialise the round trips
+// ---- activations -> shared memory ------------------------------------------------------------------------------
+// Sixteen lanes take the 128 activations of one (pair, token), eight consecutive ones each.
+
+// Integer path (one token): pair q of the chunk at xs + q * kPlaneBytes: [half h of the MMAs][plane][t][16 bytes = MMAs 2h, 2h + 1],
+// i.e. lane (g < 2, t) of the product reads its narrow-operand registers of MMAs 2h and 2h + 1 with one 16-byte load; then
+// the block scale and the sums of the two 64-element tiles.  A warp takes a pair, four consecutive activations a lane.
+template <int FMT, int kWarps>
+__device__ __forceinline__ void stage_x_i8(uint32_t xs, const void* x, bool bf16, uint32_t pair0, uint32_t n, int warp, int lane) {
+  constexpr int B = 4;                             // loads in flight: each is a round trip to a busy L2
+  for (uint32_t q0 = warp; q0 < n; q0 += B * kWarps) {
+  uint2 raw[B];
 #pragma unroll
-    for (int i = 0; i < 4; ++i) u[i] = ld_cg_u4(src + 32 * i);
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      uint4 v = u[i];
-      if (p.x_dtype == EORA_X_BF16) { v.x = bf2_to_h2(v.x); v.y = bf2_to_h2(v.y); v.z = bf2_to_h2(v.z); v.w = bf2_to_h2(v.w); }
-      xr[4 * i] = v.x; xr[4 * i + 1] = v.y; xr[4 * i + 2] = v.z; xr[4 * i + 3] = v.w;
-    }
-  } else {
-#pragma unroll
-    for (int i = 0; i < 16; ++i) xr[i] = 0u;
+  for (int b = 0; b < B; ++b) {
+    raw[b] = make_uint2(0u, 0u);
+    if (q0 + b * kWarps < n)
+      asm volatile("ld.global.cg.v2.u32 {%0,%1}, [%2];" : "=r"(raw[b].x), "=r"(raw[b].y)
+                   : "l"(reinterpret_cast<const uint16_t*>(x) + (size_t)(pair0 + q0 + b * kWarps) * 128 + 4 * lane) : "memory");
   }
-}
-
-// The same for t (fp32 sums in d_t [8][r_pad]), split into high and low fp16 parts.
-__device__ __forceinline__ void load_t_pair(uint32_t (&xh)[16], uint32_t (&xl)[16], const DecodeArgs& p, uint32_t pair, int lane) {
-  const int g = lane >> 2, t = lane & 3;
-  if (p.adp_pairs) {                      // the token takes part only in its own adapter's pairs
-    int mine = p.adp[0];
 #pragma unroll
-    for (int i = 1; i < 8; ++i) if (g == i) mine = p.adp[i];
-    if (mine < 0 || (uint32_t)mine != pair / p.adp_pairs) {
-#pragma unroll
-      for (int i = 0; i < 16; ++i) { xh[i] = 0u; xl[i] = 0u; }
-      return;
-    }
-  }
-  const float* src = p.d_t + (size_t)g * p.r_pad + pair * 128 + 8 * t;
-  uint4 ua[8];                             // all loads first: a use in between would serialise the round trips
-#pragma unroll
-  for (int i = 0; i < 8; ++i) ua[i] = ld_cg_u4(src + 32 * (i >> 1) + 4 * (i & 1));
-#pragma unroll
-  for (int i = 0; i < 4; ++i) {
-#pragma unroll
-    for (int hq = 0; hq < 2; ++hq) {
-      const uint4 u = ua[2 * i + hq];
-      const float f[4] = {__uint_as_float(u.x), __uint_as_float(u.y), __uint_as_float(u.z), __uint_as_float(u.w)};
-#pragma unroll
-      for (int j = 0; j < 2; ++j) {
-        const __half h0 = __float2half_rn(f[2 * j]), h1 = __float2half_rn(f[2 * j + 1]);
-        const __half2 hi = __halves2half2(h0, h1);
-        xh[4 * i + 2 * hq + j] = *reinterpret_cast<const uint32_t*>(&hi);
-        xl[4 * i + 2 * hq + j] = pack_h2(f[2 * j] - __half2float(h0), f[2 * j + 1] - __half2float(h1));
-      }
-    }
-  }
-}
-
-// red.add under a predicate (no branch: with one token only a quarter of the lanes has something to add,
-// and a divergent branch per blob costs more than the adds).
-__device__ __forceinline__ void red_add_if(float* p, float v, uint32_t pred) {
-  asm volatile("{\n\t.reg .pred q;\n\tsetp.ne.u32 q, %2, 0;\n\t@q red.global.add.f32 [%0], %1;\n\t}" ::"l"(p), "f"(v), "r"(pred) : "memory");
-}
-
-// Where a lane's partial sums go: sums[token][ld] for rows 16 * tile + {g, g + 8} and tokens {2t, 2t + 1}.
-struct Flush {
-  float* base;              // sums + 2t * ld + g
-  uint32_t ld;
-  uint32_t has0, has1;      // token 2t / 2t + 1 exists
-};
-__device__ __forceinline__ Flush make_flush(float* sums, int ld, int m, int lane) {
-  const int g = lane >> 2, t = lane & 3;
-  Flush f;
-  f.base = sums + (size_t)(2 * t) * ld + g;
-  f.ld = (uint32_t)ld;
-  f.has0 = 2 * t < m ? 1u : 0u;
-  f.has1 = 2 * t + 1 < m ? 1u : 0u;
-  return f;
-}
-__device__ __forceinline__ void flush_sums(const Flush& f, uint32_t tile, const float (&tot)[4]) {
-  float* b = f.base + tile * 16;
-  red_add_if(b, tot[0], f.has0); red_add_if(b + 8, tot[2], f.has0);
-  red_add_if(b + f.ld, tot[1], f.has1); red_add_if(b + f.ld + 8, tot[3], f.has1);
-}
-
-__device__ __forceinline__ uint32_t atom_add_acq_rel(uint32_t* p, uint32_t v) {
-  uint32_t old;
-  asm volatile("atom.acq_rel.gpu.global.add.u32 %0, [%1], %2;" : "=r"(old) : "l"(p), "r"(v) : "memory");
-  return old;
-}
-__device__ __forceinline__ void red_add_release(uint32_t* p, uint32_t v) {
-  asm volatile("red.release.gpu.global.add.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
-}
-
-// Per-warp state of the copy ring.  All lanes keep the same copy of it; lane 0 issues.
-struct Ring {
-  uint8_t* slots;
-  uint64_t* bars;
-  // producer side: the run of blobs still to be requested, over up to three segments
-  const uint8_t* ptr[3];
-  uint32_t rem[3], blob[3], per[3];
-  int pseg;
-  // consumer side
-  int slot;
-  uint32_t phase;           // bit i: parity of the phase that the next copy into slot i completes
-  int deferred;             // slots [kRing - deferred, kRing) have not had their first copy requested yet
-  uint32_t aux;             // shared-memory address of the 2:4 expansion table (2:4 backbone only)
-};
-
-constexpr uint32_t kNone = 0xffffffffu;
-__device__ __forceinline__ uint32_t slot_parity(const Ring& r) { return (r.phase >> r.slot) & 1u; }
-__device__ __forceinline__ void slot_consumed(Ring& r) {
-  r.phase ^= 1u << r.slot;
-  if (++r.slot == kRing) r.slot = 0;
-}
-
-__device__ __forceinline__ void ring_issue(Ring& r, int slot, int lane) {
-  if (r.pseg == 0 && r.rem[0] == 0) r.pseg = 1;
-  if (r.pseg == 1 && r.rem[1] == 0) r.pseg = 2;
-  if (r.pseg == 2 && r.rem[2] == 0) r.pseg = 3;
-  if (r.pseg >= 3) return;
-  // runtime-indexed reads of three-element arrays would go to local memory: select instead
-  const int s = r.pseg;
-  const uint8_t* src = s == 0 ? r.ptr[0] : s == 1 ? r.ptr[1] : r.ptr[2];
-  const uint32_t rem = s == 0 ? r.rem[0] : s == 1 ? r.rem[1] : r.rem[2];
-  const uint32_t blob = s == 0 ? r.blob[0] : s == 1 ? r.blob[1] : r.blob[2];
-  const uint32_t per = s == 0 ? r.per[0] : s == 1 ? r.per[1] : r.per[2];
-  const uint32_t n = rem < per ? rem : per;
-  const uint32_t bytes = n * blob;
-  if (lane == 0) {
-    mbar_expect_tx(r.bars + slot, bytes);
-    bulk_g2s(r.slots + slot * kSlotBytes, src, bytes, r.bars + slot);
-  }
-  if (s == 0) { r.ptr[0] = src + bytes; r.rem[0] = rem - n; }
-  else if (s == 1) { r.ptr[1] = src + bytes; r.rem[1] = rem - n; }
-  else { r.ptr[2] = src + bytes; r.rem[2] = rem - n; }
-}
-
-enum { OUT_T = 0, OUT_Y = 1 };
-
-__device__ __forceinline__ void st_zero4(float* p) {
-  *reinterpret_cast<float4*>(p) = make_float4(0.f, 0.f, 0.f, 0.f);
-}
-
-// Row tile `tile` of the output is complete.  Called by ONE lane (the one whose ticket was the last);
-// it converts the tile's 16 x m sums, stores them and puts the scratch back to zero.  Several lanes of a
-// warp may each be finishing a tile of their own at the same time.
-__device__ __forceinline__ void finish_row_tile(const DecodeArgs& p, uint32_t tile) {
-  void* y = p.ys[0];
-  uint32_t tile0 = 0;
-  int dout = p.sub_dout[0];
-#pragma unroll
-  for (int i = 1; i < 4; ++i)
-    if (i < p.n_sub && tile >= p.sub_tile0[i]) { y = p.ys[i]; tile0 = p.sub_tile0[i]; dout = p.sub_dout[i]; }
-  for (int token = 0; token < p.m; ++token) {
-    float* s = p.y_ws + (size_t)token * p.n_pad + tile * 16;
-    uint4 u[4];
-#pragma unroll
-    for (int i = 0; i < 4; ++i) u[i] = ld_cg_u4(s + 4 * i);
-#pragma unroll
-    for (int i = 0; i < 4; ++i) st_zero4(s + 4 * i);
-    const float v[16] = {__uint_as_float(u[0].x), __uint_as_float(u[0].y), __uint_as_float(u[0].z), __uint_as_float(u[0].w),
-                         __uint_as_float(u[1].x), __uint_as_float(u[1].y), __uint_as_float(u[1].z), __uint_as_float(u[1].w),
-                         __uint_as_float(u[2].x), __uint_as_float(u[2].y), __uint_as_float(u[2].z), __uint_as_float(u[2].w),
-                         __uint_as_float(u[3].x), __uint_as_float(u[3].y), __uint_as_float(u[3].z), __uint_as_float(u[3].w)};
-    const int64_t o = (int64_t)token * dout + (tile - tile0) * 16;   // d_out is a multiple of 32: the 16 outputs exist
-    if (p.y_dtype == EORA_Y_F32) {
-      float4* dst = reinterpret_cast<float4*>(reinterpret_cast<float*>(y) + o);
-#pragma unroll
-      for (int i = 0; i < 4; ++i) dst[i] = make_float4(v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]);
+  for (int b = 0; b < B; ++b) {
+    const uint32_t q = q0 + b * kWarps;
+    if (q >= n) break;
+    const uint2 u = raw[b];
+    float f[4];
+    if (bf16) {
+      f[0] = __uint_as_float(u.x << 16); f[1] = __uint_as_float(u.x & 0xffff0000u);
+      f[2] = __uint_as_float(u.y << 16); f[3] = __uint_as_float(u.y & 0xffff0000u);
     } else {
-      uint32_t h[8];
+      const float2 a = __half22float2(*reinterpret_cast<const __half2*>(&u.x)), b = __half22float2(*reinterpret_cast<const __half2*>(&u.y));
+      f[0] = a.x; f[1] = a.y; f[2] = b.x; f[3] = b.y;
+    }
+    float am = fmaxf(fmaxf(fabsf(f[0]), fabsf(f[1])), fmaxf(fabsf(f[2]), fabsf(f[3])));
+    am = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(am)));      // non-negative floats order like integers
+    const uint32_t eb = __float_as_uint(am * 1.00396f) >> 23;           // biased exponent of a value just above the maximum
+    const bool live = eb >= 15u && eb < 255u;
+    const float inv = live ? __uint_as_float((268u - eb) << 23) : 0.f;   // 2^(14 - exponent): |v| <= 32639 = 127 * 256 + 127
+    int v[4], s = 0;
 #pragma unroll
-      for (int i = 0; i < 8; ++i) {
-        if (p.y_dtype == EORA_Y_F16) {
-          h[i] = pack_h2(v[2 * i], v[2 * i + 1]);
-        } else {
-          const __nv_bfloat162 b = __floats2bfloat162_rn(v[2 * i], v[2 * i + 1]);
-          h[i] = *reinterpret_cast<const uint32_t*>(&b);
-        }
-      }
-      uint4* dst = reinterpret_cast<uint4*>(reinterpret_cast<uint16_t*>(y) + o);
-      dst[0] = make_uint4(h[0], h[1], h[2], h[3]);
-      dst[1] = make_uint4(h[4], h[5], h[6], h[7]);
+    for (int e = 0; e < 4; ++e) { v[e] = __float2int_rn(f[e] * inv); s += v[e]; }
+    // the low plane is the low byte of v as it is (a signed byte), the high plane byte 1 of v + 128
+    uint32_t lo = prmt(prmt(v[0], v[1], 0x0040u), prmt(v[2], v[3], 0x0040u), 0x5410u);
+    uint32_t hi = prmt(prmt(v[0] + 128, v[1] + 128, 0x0051u), prmt(v[2] + 128, v[3] + 128, 0x0051u), 0x5410u);
+    if constexpr (FMT == FMT_Q4) {                 // the and delivers the codes as (0, 4, 1, 5) and (2, 6, 3, 7): neighbouring lanes swap
+      const uint32_t ol = __shfl_xor_sync(0xffffffffu, lo, 1), oh = __shfl_xor_sync(0xffffffffu, hi, 1);
+      lo = (lane & 1) ? prmt(ol, lo, 0x7362u) : prmt(lo, ol, 0x5140u);
+      hi = (lane & 1) ? prmt(oh, hi, 0x7362u) : prmt(hi, oh, 0x5140u);
+    }
+    const int s_all = __reduce_add_sync(0xffffffffu, s), s_first = __reduce_add_sync(0xffffffffu, lane < 16 ? s : 0);
+    // this lane's elements belong to MMA j = lane / 8 (32 elements each) and lane t of the product
+    const uint32_t j = lane >> 3, t = (lane >> 1) & 3, d = xs + q * kPlaneBytes + (j >> 1) * 128 + t * 16 + (j & 1) * 8 + (lane & 1) * 4;
+    sts_u1(d, lo);
+    sts_u1(d + 64, hi);
+    if (lane == 0) {
+      const uint32_t meta = xs + q * kPlaneBytes + 256;
+      sts_u1(meta, live ? (eb - 14u) << 23 : 0u);                        // 2^(exponent - 14)
+      sts_u1(meta + 4, (uint32_t)s_first);
+      sts_u1(meta + 8, (uint32_t)(s_all - s_first));
     }
   }
-  p.counters[CNT_TICKET0 + tile] = 0u;
+  }
 }
 
-// One segment: `n` consecutive blobs of one matrix starting at blob index b0.
-// I8M: backbone blobs of a launch with two to eight tokens go through the integer product (blob_product_i8m).
-template <int FMT, bool HILO, int OUT, bool I8M = false>
-__device__ __forceinline__ bool run_segment(const DecodeArgs& p, Ring& r, uint32_t b0, uint32_t n, uint32_t nt, uint32_t blob_b,
-                                            uint32_t per_copy, uint32_t sz2, int lane) {
-  if constexpr (FMT == FMT_NONE) {
-    return true;
-  } else {
-    if (n == 0) return true;
-    uint32_t pair = b0 / nt, tile = b0 - pair * nt;
-    uint32_t xr[16], xl[16];
-    XI8M xm;
-    const bool x_bf16 = p.x_dtype == EORA_X_BF16;
-    uint32_t sub = 0, sub_end = nt;
-    Flush fl = OUT == OUT_T ? make_flush(p.d_t, p.r_pad, p.m, lane) : make_flush(p.y_ws, p.n_pad, p.m, lane);
-    if constexpr (HILO) {
-      // all of A must be in t
-      int ok = 1;
-      if (lane == 0) ok = counter_wait(p.counters + CNT_A_DONE, p.a_blobs, p.dev_status, p.wait_ns) ? 1 : 0;
-      ok = __shfl_sync(0xffffffffu, ok, 0);
-      if (!ok) return false;
-      __syncwarp();
-      // the activations of B's blob (pair, tile) belong to the layer that owns the row tile
-      sub = 0;
+// fp16 path: rows of tokens, `pitch` bytes apart (64 bytes past a multiple of 128: the 16-byte reads of a quarter warp, two
+// rows of 64 bytes, then touch every bank once).  Every 16-byte piece (8 elements) holds the four register pairs in
+// the order in which the products of FMT use them.  For the quantised formats also the sums of a tile's activations
+// (the zero-point's factor): xsum[2 * pair + tile][token], and for bf16 activations, which may lie outside fp16's range, a
+// power of two per (pair, token): the fp16 values are x / scale.
+template <int FMT, int kWarps>
+__device__ __forceinline__ void stage_x_f16(uint8_t* xs, uint32_t pitch, float* xsum, float* xscale, const void* x, bool bf16, int m, int d_in,
+                                            uint32_t pair0, uint32_t n) {
+  constexpr bool sums = FMT == FMT_Q4 || FMT == FMT_Q3;
+  const uint32_t hw = threadIdx.x >> 4, l = threadIdx.x & 15, total = n * (uint32_t)m;
+  constexpr int B = 4;                            // loads in flight per lane
+  for (uint32_t u0 = hw; u0 < ((total + 1) & ~1u); u0 += B * 2 * kWarps) {
+    uint4 raw[B];
 #pragma unroll
-      for (int i = 1; i < 4; ++i)
-        if (i < p.n_sub && tile >= p.sub_tile0[i]) sub = i;
-      sub_end = p.sub_tile0[sub + 1];
-      load_t_pair(xr, xl, p, sub * p.b_np + pair, lane);
-    } else if constexpr (I8M) {
-      load_x_i8m<FMT>(xm, p.x, x_bf16, p.m, p.d_in, pair, lane);
-    } else {
-      load_x_pair(xr, p, pair, lane);
-    }
-    // The first copies that were held back (see the kernel) go out behind the loads of the activations,
-    // not in front of them.
-    for (; r.deferred > 0; --r.deferred) ring_issue(r, kRing - r.deferred, lane);
-    // Tickets of the blobs flushed so far are taken in batches of up to 32 (one atomic per lane, one
-    // round trip per batch): batch_tile is the row tile of the batch's first blob, batch_n its size.
-    uint32_t batch_tile = tile, batch_n = 0, flushed = 0;
-    auto commit_batch = [&]() {
-      __syncwarp();
-      uint32_t done = 0, my_tile = 0;
-      if ((uint32_t)lane < batch_n) {
-        my_tile = (batch_tile + lane) % nt;
-        done = atom_add_acq_rel(p.counters + CNT_TICKET0 + my_tile, 1u) + 1u == p.tile_target ? 1u : 0u;
+    for (int i = 0; i < B; ++i) {
+      const uint32_t u = u0 + i * 2 * kWarps;
+      if (u < total) {
+        const uint32_t tok = u / n, q = u - tok * n;
+        raw[i] = ld_cg_u4(reinterpret_cast<const uint16_t*>(x) + (size_t)tok * d_in + (size_t)(pair0 + q) * 128 + 8 * l);
+      } else {
+        raw[i] = make_uint4(0u, 0u, 0u, 0u);
       }
-      const uint32_t mask = __ballot_sync(0xffffffffu, done != 0);
-      if (mask) {
-        // With an adapter the finished row tiles are counted (the count is taken before the tiles are
-        // written out, so that the two round trips overlap): the last one restores t and the counters.
-        uint32_t last = 0;
-        if (p.a_blobs && lane == 0)
-          last = atom_add_acq_rel(p.counters + CNT_TILES_DONE, (uint32_t)__popc(mask)) + __popc(mask) == p.w_nt ? 1u : 0u;
-        if (done) finish_row_tile(p, my_tile);
-        last = __shfl_sync(0xffffffffu, last, 0);
-        if (last) {                               // the whole layer is done: nobody reads t any more
-          for (int i = lane; i < 8 * p.r_pad / 4; i += 32) st_zero4(p.d_t + 4 * i);
-          if (lane == 0) { p.counters[CNT_A_DONE] = 0u; p.counters[CNT_TILES_DONE] = 0u; }
+    }
+#pragma unroll
+    for (int i = 0; i < B; ++i) {
+      const uint32_t u = u0 + i * 2 * kWarps;
+      if ((u & ~1u) >= total) continue;                   // uniform over the warp: its halves take u and u + 1, u even
+      uint32_t w[4] = {raw[i].x, raw[i].y, raw[i].z, raw[i].w};
+      const uint32_t tok = u / n, q = u - tok * n;
+      float sc = 1.f;
+      if (bf16) {
+        float f[8];
+#pragma unroll
+        for (int e = 0; e < 4; ++e) { f[2 * e] = __uint_as_float(w[e] << 16); f[2 * e + 1] = __uint_as_float(w[e] & 0xffff0000u); }
+        float inv = 1.f;
+        if constexpr (sums) {
+          float am = 0.f;
+#pragma unroll
+          for (int e = 0; e < 8; ++e) am = fmaxf(am, fabsf(f[e]));
+#pragma unroll
+          for (int o = 1; o < 16; o <<= 1) am = fmaxf(am, __shfl_xor_sync(0xffffffffu, am, o));
+          const uint32_t eb = __float_as_uint(am) >> 23;
+          if (eb >= 32u && eb < 240u) { inv = __uint_as_float((267u - eb) << 23); sc = __uint_as_float((eb - 13u) << 23); }   // largest magnitude in [2^13, 2^14)
+        }
+#pragma unroll
+        for (int e = 0; e < 4; ++e) w[e] = pack_h2(f[2 * e] * inv, f[2 * e + 1] * inv);
+      }
+      if constexpr (sums) {
+        float s = 0.f;
+#pragma unroll
+        for (int e = 0; e < 4; ++e) { const float2 v = __half22float2(*reinterpret_cast<const __half2*>(&w[e])); s += v.x + v.y; }
+#pragma unroll
+        for (int o = 1; o < 8; o <<= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+        if (u < total) {
+          if ((l & 7) == 0) xsum[(2 * q + (l >> 3)) * kMaxTok + tok] = s;
+          if (l == 0) xscale[q * kMaxTok + tok] = sc;
         }
       }
-      batch_n = 0;
-    };
-    while (n > 0) {
-      const uint32_t cn = n < per_copy ? n : per_copy;
-      if (!mbar_wait_warp(r.bars + r.slot, slot_parity(r), p.dev_status, lane)) return false;
-      const uint8_t* src = r.slots + r.slot * kSlotBytes;
-#pragma unroll 2
-      for (uint32_t j = 0; j < cn; ++j) {
-        float tot[4];
-        if constexpr (I8M) blob_product_i8m<FMT>(src + j * blob_b, lane, sz2, xm, tot);
-        else blob_product<FMT, HILO>(src + j * blob_b, lane, sz2, xr, xl, tot, r.aux);
-        if constexpr (OUT == OUT_T) {
-          flush_sums(fl, tile, tot);
-          ++flushed;
-        } else {
-          if (batch_n == 0) batch_tile = tile;
-          flush_sums(fl, tile, tot);
-          if (++batch_n == 32) commit_batch();
-        }
-        if (++tile == nt) {
-          tile = 0;
-          ++pair;
-          if (j + 1 < cn || n > cn) {
-            if constexpr (HILO) {
-              sub = 0; sub_end = p.sub_tile0[1];
-              load_t_pair(xr, xl, p, pair, lane);
-            } else if constexpr (I8M) {
-              load_x_i8m<FMT>(xm, p.x, x_bf16, p.m, p.d_in, pair, lane);
-            } else {
-              load_x_pair(xr, p, pair, lane);
-            }
-          }
-        } else if constexpr (HILO) {
-          if (tile == sub_end && (j + 1 < cn || n > cn)) {      // the next row tile belongs to the next fused layer
-            ++sub;
-            sub_end = p.sub_tile0[sub + 1];
-            load_t_pair(xr, xl, p, sub * p.b_np + pair, lane);
-          }
-        }
+      if (u < total) {
+        uint4 o = make_uint4(w[0], w[1], w[2], w[3]);
+        if constexpr (FMT == FMT_Q4) { o.y = w[2]; o.z = w[1]; }
+        else if constexpr (FMT == FMT_Q3) o = make_uint4(prmt(w[0], w[1], 0x5410u), prmt(w[0], w[1], 0x7632u), prmt(w[2], w[3], 0x5410u), prmt(w[2], w[3], 0x7632u));
+        *reinterpret_cast<uint4*>(xs + (size_t)tok * pitch + q * 256 + l * 16) = o;
       }
-      __syncwarp();                               // every lane is done with the slot
-      ring_issue(r, r.slot, lane);
-      slot_consumed(r);
-      n -= cn;
     }
-    if constexpr (OUT == OUT_T) {
-      __syncwarp();
-      if (lane == 0) red_add_release(p.counters + CNT_A_DONE, flushed);
-    } else {
-      if (batch_n) commit_batch();
-    }
-    return true;
   }
 }
 
-// The backbone share of a single-token launch (integer inner product): the same walk as run_segment, written for
-// instruction count -- this loop is what bounds the kernel (a warp retires an instruction every ~10 cycles, and every
-// instruction around the product of a blob costs as much as one inside it): running addresses instead of index
-// arithmetic, the group layout as a compile-time constant, runs of blobs without a branch in between.
-struct WalkI8 {
-  XI8 xi;
-  uint32_t pair, tile;          // the next blob; pair == kNone: no activations loaded yet
-  uint32_t next_b;              // its index (to tell whether the next run continues this one)
-  float* yb;
-  uint32_t batch_n, my_tile;    // blobs added but without a ticket yet; lane i < batch_n: the row tile of the i-th
-  uint32_t tk_old, tk_tile, tk_n;   // tickets asked for (lane i: the one of the batch's blob i), not looked at yet
-};
+// ---- products ---------------------------------------------------------------------------------------------------
+// Blobs and activations are addressed by 32-bit shared-memory addresses: what bounds the loop over the blobs is the number
+// of instructions around the tensor-core products, and generic pointers cost two per step.
 
-// The tickets asked for last time: whoever holds a row tile's last one finishes the tile.
-__device__ __forceinline__ void tickets_resolve(const DecodeArgs& p, WalkI8& w, int lane) {
-  if (w.tk_n == 0) return;
-  const uint32_t done = ((uint32_t)lane < w.tk_n && w.tk_old + 1u == p.tile_target) ? 1u : 0u;
-  const uint32_t mask = __ballot_sync(0xffffffffu, done != 0);
-  if (mask) {
-    // With an adapter the finished row tiles are counted (before they are written out, so that the two round
-    // trips overlap): the last one restores t and the counters.
-    uint32_t last = 0;
-    if (p.a_blobs && lane == 0)
-      last = atom_add_acq_rel(p.counters + CNT_TILES_DONE, (uint32_t)__popc(mask)) + __popc(mask) == p.w_nt ? 1u : 0u;
-    if (done) finish_row_tile(p, w.tk_tile);
-    last = __shfl_sync(0xffffffffu, last, 0);
-    if (last) {
-      for (int i = lane; i < 8 * p.r_pad / 4; i += 32) st_zero4(p.d_t + 4 * i);
-      if (lane == 0) { p.counters[CNT_A_DONE] = 0u; p.counters[CNT_TILES_DONE] = 0u; }
-    }
-  }
-  w.tk_n = 0;
-}
-// Tickets for the blobs added since the last batch (the release in front of them waits for the warp's additions
-// to arrive, which is why they are not taken more often than every 32 blobs).  The answers are looked at one batch later: nothing waits for
-// the round trip.
-__device__ __forceinline__ void tickets_take(const DecodeArgs& p, WalkI8& w, int lane) {
-  tickets_resolve(p, w, lane);
-  if (w.batch_n == 0) return;
-  __syncwarp();
-  if ((uint32_t)lane < w.batch_n) {
-    w.tk_tile = w.my_tile;
-    w.tk_old = atom_add_acq_rel(p.counters + CNT_TICKET0 + w.my_tile, 1u);
-  }
-  w.tk_n = w.batch_n;
-  w.batch_n = 0;
-}
-
-// The next blobs are b0, b0 + 1, ...
-template <int FMT>
-__device__ __forceinline__ void walk_seek(const DecodeArgs& p, WalkI8& w, uint32_t b0, int lane) {
-  if (b0 == w.next_b && w.pair != kNone) return;
-  const uint32_t pair = b0 / p.w_nt;
-  w.tile = b0 - pair * p.w_nt;
-  w.next_b = b0;
-  w.yb = p.y_ws + (lane >> 2) + w.tile * 16;
-  if (pair != w.pair) load_x_i8<FMT>(w.xi, p.x, p.x_dtype == EORA_X_BF16, pair, lane);
-  w.pair = pair;
-}
-
-// cn blobs in shared memory at bp; more: blobs follow after these (then the activations of the next pair are
-// fetched when these end a pair).
+// One token, 3/4-bit backbone.  xa: this lane's planes of the pair (stage_x_i8; a block of zeros for the lanes that hold
+// no column), xm: the pair's scale and sums.  acc[0] / acc[1] += rows g / g + 8 on the lanes with t == 0.
 template <int FMT, bool SZ2>
-__device__ __forceinline__ void walk_blobs(const DecodeArgs& p, WalkI8& w, const uint8_t* bp, uint32_t cn, bool more, int lane) {
-  constexpr uint32_t blob_b = blob_bytes(FMT, SZ2 ? 1 : 0);
-  const uint32_t nt = p.w_nt;
-  const uint32_t owner = (lane & 3) == 0 ? 1u : 0u;
-  const uint8_t* bl = bp + (FMT == FMT_Q4 ? 16 : 8) * lane;
-  const uint8_t* bg = bp + 4 * (lane >> 2);
-  w.next_b += cn;
-  for (uint32_t left = cn; left > 0;) {
-    // a run of blobs without a change of pair and without a ticket batch filling up: nothing but products and adds
-    uint32_t run = min(left, min(nt - w.tile, 32u - w.batch_n));
-    if ((uint32_t)lane - w.batch_n < run) w.my_tile = w.tile + ((uint32_t)lane - w.batch_n);
-    left -= run; w.tile += run; w.batch_n += run;
-#pragma unroll 2
-    for (; run > 0; --run, bl += blob_b, bg += blob_b, w.yb += 16) {
-      float t2[2];
-      blob_product_i8<FMT, SZ2>(bl, bg, lane, w.xi, t2);
-      red_add_if(w.yb, t2[0], owner);
-      red_add_if(w.yb + 8, t2[1], owner);
-    }
-    if (w.tile == nt) {                                 // next pair of reduction elements: other activations
-      w.tile = 0; ++w.pair; w.yb = p.y_ws + (lane >> 2);
-      if (left > 0 || more) load_x_i8<FMT>(w.xi, p.x, p.x_dtype == EORA_X_BF16, w.pair, lane);
-      else w.pair = kNone;
-    }
-    if (w.batch_n == 32) tickets_take(p, w, lane);
-  }
-}
-
-// n blobs from b0 on, dealt to this warp ahead of time.
-template <int FMT, bool SZ2>
-__device__ __forceinline__ bool run_backbone_i8(const DecodeArgs& p, Ring& r, WalkI8& w, uint32_t b0, uint32_t n, int lane) {
-  if (n == 0) return true;
-  walk_seek<FMT>(p, w, b0, lane);
-  for (; r.deferred > 0; --r.deferred) ring_issue(r, kRing - r.deferred, lane);
-  while (n > 0) {
-    const uint32_t cn = n < p.w_per_copy ? n : p.w_per_copy;
-    if (!mbar_wait_warp(r.bars + r.slot, slot_parity(r), p.dev_status, lane)) return false;
-    walk_blobs<FMT, SZ2>(p, w, r.slots + r.slot * kSlotBytes, cn, n > cn, lane);
-    __syncwarp();                                       // every lane is done with the slot
-    ring_issue(r, r.slot, lane);
-    slot_consumed(r);
-    n -= cn;
-  }
-  return true;
-}
-
-template <int WF, int I8>
-__device__ __forceinline__ bool run_backbone(const DecodeArgs& p, Ring& r, WalkI8& w, uint32_t first, uint32_t count, uint32_t blob_w, int lane) {
-  if constexpr (I8 == 2) {
-    return run_segment<WF, false, OUT_Y, true>(p, r, first, count, p.w_nt, blob_w, p.w_per_copy, p.w_sz2, lane);
-  } else if constexpr (I8 == 1) {
-    return p.w_sz2 ? run_backbone_i8<WF, true>(p, r, w, first, count, lane) : run_backbone_i8<WF, false>(p, r, w, first, count, lane);
-  } else {
-    return run_segment<WF, false, OUT_Y>(p, r, first, count, p.w_nt, blob_w, p.w_per_copy, p.w_sz2, lane);
-  }
-}
-
-// I8: the backbone goes through the integer inner product -- 1: one token (the walk above), 2: two to eight tokens
-// (tokens as the columns of the narrow operand, two byte planes = two MMAs per weight fragment), 0: fp16 product.
-template <int WF, int ABF, int I8>
-__global__ void __launch_bounds__(kThreads, kCtasPerSm) k_decode(const __grid_constant__ DecodeArgs p) {
-  extern __shared__ __align__(128) uint8_t smem[];
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  // Position in the deal.  Neighbours in the deal sit on different SMs, so that the few warps that hold A (whose sums
-  // everybody's B share waits for) work in parallel on many SMs: the A owners are dealt warp by warp over the first
-  // half of the CTAs, the B owners over the second half, and the warps left over are numbered after them.  No CTA
-  // holds both kinds: the CTAs with A owners are dispatched first and never wait, so a waiting warp never holds the
-  // place of a CTA that it is waiting for.
-  uint32_t gw;
-  {
-    const uint32_t ca = gridDim.x / 2, cb = gridDim.x - ca, n3 = gridDim.x * kWarps - p.n12;
-    if (blockIdx.x < ca) {
-      gw = warp * ca + blockIdx.x;                                    // < n1: an A owner
-    } else {
-      const uint32_t rid = warp * cb + (blockIdx.x - ca);
-      gw = rid < n3 ? p.n12 + rid : p.n1 + (kWarps * ca - p.n1) + (rid - n3);
-    }
-  }
-  asm volatile("griddepcontrol.launch_dependents;");
-  unsigned long long* tr = p.trace ? p.trace + (size_t)(blockIdx.x * kWarps + warp) * 4 : nullptr;
-  if (tr && lane == 0) tr[0] = globaltimer_ns();
-
-  Ring r;
-  r.slots = smem + warp * (kRing * kSlotBytes);
-  r.bars = reinterpret_cast<uint64_t*>(smem + kWarps * kRing * kSlotBytes) + warp * kRing;
-  r.slot = 0; r.phase = 0; r.pseg = 0;
-  r.aux = 0;
-  if constexpr (WF == FMT_SP24 || WF == FMT_SQ4) {
-    // every warp writes the same 16 values, so no CTA-wide barrier is needed before a warp reads them
-    uint32_t* lut = reinterpret_cast<uint32_t*>(smem + kWarps * kRing * kSlotBytes + kBarBytes);
-    if (lane < 16) lut[lane] = sp24_selectors((uint32_t)lane);
-    r.aux = smem_u32(lut);
-  }
-  if (lane == 0) {
+__device__ __forceinline__ void product_i8(const RawBlob<FMT, SZ2>& r, uint32_t xa, uint32_t xm, float (&acc)[2]) {
+  const uint4 xb[2] = {lds_u4(xa), lds_u4(xa + 128)};
+  const uint4 meta = lds_u4(xm);
+  const float scale = __uint_as_float(meta.x);
+  const int xsum[2] = {(int)meta.y, (int)meta.z};
+  int d[4] = {0, 0, 0, 0};             // rows g / g + 8 x columns (low, high plane) on the lanes with t == 0
 #pragma unroll
-    for (int i = 0; i < kRing; ++i) mbar_init(r.bars + i, 1);
-    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+  for (int c = 0; c < 2; ++c) {
+    uint32_t q[4][2];
+    code_quads<FMT>(r.t[c], q);
+    mma16832_s8(d, q[0][0], q[1][0], q[0][1], q[1][1], xb[c].x, xb[c].y);
+    mma16832_s8(d, q[2][0], q[3][0], q[2][1], q[3][1], xb[c].z, xb[c].w);
+    if (c == 1 || SZ2) {
+      const int k = SZ2 ? c : 0;
+      const int xs = SZ2 ? xsum[c] : xsum[0] + xsum[1];
+      const float2 s = __half22float2(*reinterpret_cast<const __half2*>(&r.s[k]));
+      const int z_a = (int)(r.z[k] & 255u), z_b = (int)(r.z[k] >> 8);
+      acc[0] = fmaf((float)(d[1] * 256 + d[0] - z_a * xs), s.x * scale, acc[0]);
+      acc[1] = fmaf((float)(d[3] * 256 + d[2] - z_b * xs), s.y * scale, acc[1]);
+      d[0] = d[1] = d[2] = d[3] = 0;
+    }
   }
-  __syncwarp();
+}
 
-  // this warp's three runs: A, W, B (one of A / B is empty)
-  const bool a_owner = gw < p.n1, b_owner = gw >= p.n12;
-  uint32_t a0 = 0, an = 0, w0, wn, bb0 = 0, bn = 0;
-  if (a_owner) {
-    a0 = share_lo(p.sh_a, gw); an = share_n(p.sh_a, gw);
-    w0 = p.w_base[0] + share_lo(p.sh_w[0], gw); wn = share_n(p.sh_w[0], gw);
-  } else if (!b_owner) {
-    const uint32_t i = gw - p.n1;
-    w0 = p.w_base[1] + share_lo(p.sh_w[1], i); wn = share_n(p.sh_w[1], i);
-  } else {
-    const uint32_t i = gw - p.n12;
-    w0 = p.w_base[2] + share_lo(p.sh_w[2], i); wn = share_n(p.sh_w[2], i);
-    bb0 = share_lo(p.sh_b, i); bn = share_n(p.sh_b, i);
+// This lane's activation registers of a pair for tile c, four per half of the tile.
+__device__ __forceinline__ void load_xf(uint32_t (&xr)[8], uint32_t row, int c) {
+#pragma unroll
+  for (int b = 0; b < 2; ++b) {
+    const uint4 v = lds_u4(row + (2 * c + b) * 64);
+    xr[4 * b] = v.x; xr[4 * b + 1] = v.y; xr[4 * b + 2] = v.z; xr[4 * b + 3] = v.w;
   }
-  const uint32_t blob_a = blob_bytes(ABF, p.a_sz2), blob_w = blob_bytes(WF, p.w_sz2), blob_b = blob_bytes(ABF, p.b_sz2);
-  // Order of the runs.  A owners: A, then W.  The others: the first copy's worth of W, then B, then the
-  // rest of W: by then t is complete, and the round trips of the B share (reading t back, its tickets)
-  // are hidden behind the other warps' W work instead of sitting at the end of the kernel.
-  const uint32_t wf = !b_owner ? wn : (wn < p.w_per_copy ? wn : p.w_per_copy);
-  if (!b_owner) {
-    r.ptr[0] = p.a_q + (size_t)a0 * blob_a; r.rem[0] = an; r.blob[0] = blob_a; r.per[0] = p.a_per_copy;
-    r.ptr[1] = p.w_q + (size_t)w0 * blob_w; r.rem[1] = wn; r.blob[1] = blob_w; r.per[1] = p.w_per_copy;
-    r.ptr[2] = p.w_q; r.rem[2] = 0; r.blob[2] = blob_w; r.per[2] = p.w_per_copy;
-  } else {
-    r.ptr[0] = p.w_q + (size_t)w0 * blob_w; r.rem[0] = wf; r.blob[0] = blob_w; r.per[0] = p.w_per_copy;
-    r.ptr[1] = p.b_q + (size_t)bb0 * blob_b; r.rem[1] = bn; r.blob[1] = blob_b; r.per[1] = p.b_per_copy;
-    r.ptr[2] = p.w_q + (size_t)(w0 + wf) * blob_w; r.rem[2] = wn - wf; r.blob[2] = blob_w; r.per[2] = p.w_per_copy;
+}
+
+// Two to eight tokens, 3/4-bit backbone, fp16 activations.  The codes go into the product as they lie in their words: as
+// fp16 bit patterns they are the numbers q * 2^-24 (subnormals, which the tensor core multiplies exactly), or 16 (8 for 3-bit)
+// times that where they sit four (three) bits higher; those go to an accumulator chain of their own.  One logic
+// instruction per two codes instead of two, and nothing is rounded that was not before.
+//   sum w x = s * (2^24 (chain 0 + chain 1 / 16) - z * sum x)
+// row: this lane's activations of the pair; xsum: the sums of tokens 2t, 2t + 1 over the pair's first tile (32 bytes further: over
+// its second); xscale: their scales (bf16 activations).  acc: (row g, token 2t), (g, 2t + 1), (g + 8, 2t), (g + 8, 2t + 1).
+template <int FMT, bool SZ2>
+__device__ __forceinline__ void product_codes(const RawBlob<FMT, SZ2>& r, uint32_t row, uint32_t xsum, uint32_t xscale, bool bf16, float (&acc)[4]) {
+  constexpr float kUp = 16777216.f, kDown = FMT == FMT_Q4 ? 1.f / 16.f : 1.f / 8.f;
+  float d0[4] = {0.f, 0.f, 0.f, 0.f}, d1[4] = {0.f, 0.f, 0.f, 0.f};
+  float2 xs = make_float2(0.f, 0.f);
+#pragma unroll
+  for (int c = 0; c < 2; ++c) {
+    uint32_t xr[8];
+    load_xf(xr, row, c);
+    uint32_t a[4][4];
+    code_frags<FMT>(r.t[c], a);
+#pragma unroll
+    for (int b = 0; b < 2; ++b) {
+      mma16816(d0, a[2 * b], xr[4 * b], xr[4 * b + 1]);
+      mma16816(d1, a[2 * b + 1], xr[4 * b + 2], xr[4 * b + 3]);
+    }
+    const uint2 xc = lds_u2(xsum + c * 4 * kMaxTok);
+    xs.x += __uint_as_float(xc.x); xs.y += __uint_as_float(xc.y);
+    if (c == 1 || SZ2) {
+      const int k = SZ2 ? c : 0;
+      const float2 s = __half22float2(*reinterpret_cast<const __half2*>(&r.s[k]));
+      const float za = -(float)(r.z[k] & 255u) * s.x, zb = -(float)(r.z[k] >> 8) * s.y;
+      const float sa = s.x * kUp, sb = s.y * kUp;
+      float v[4];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        v[i] = fmaf(fmaf(d1[i], kDown, d0[i]), i < 2 ? sa : sb, (i < 2 ? za : zb) * ((i & 1) ? xs.y : xs.x));
+        d0[i] = 0.f; d1[i] = 0.f;
+      }
+      if (bf16) {
+        const uint2 sc = lds_u2(xscale);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) v[i] *= __uint_as_float((i & 1) ? sc.y : sc.x);
+      }
+#pragma unroll
+      for (int i = 0; i < 4; ++i) acc[i] += v[i];
+      xs = make_float2(0.f, 0.f);
+    }
   }
+}
 
-  // Before the dependency resolves at most two first copies per warp are requested (with a deeper ring the others
-  // follow the loads of the activations, which are read right after the wait and would otherwise queue behind the
-  // weight requests).
-  ring_issue(r, 0, lane);
-  ring_issue(r, 1, lane);
-  r.deferred = kRing - 2;
+// Any format as exact fp16 values (q - z, or the 2:4 pattern expanded), times fp16 activations; LO: a second set of
+// activations (the low part of t) `lo` bytes further.  blob: in shared memory; it is read tile by tile (an fp16 blob is 32
+// registers a lane).
+template <int FMT, bool SZ2, bool LO>
+__device__ __forceinline__ void product_exact(uint32_t blob, int lane, uint32_t row, uint32_t lo, uint32_t lut, float (&acc)[4]) {
+  constexpr bool quant = fmt_quantised(FMT);
+  constexpr int tb = tile_bytes(FMT);
+  float d[2][4];
+#pragma unroll
+  for (int i = 0; i < 4; ++i) { d[0][i] = 0.f; d[1][i] = 0.f; }
+  ZC zc;
+  float2 s = make_float2(1.f, 1.f);
+#pragma unroll
+  for (int c = 0; c < 2; ++c) {
+    if constexpr (quant) {
+      if (c == 0 || SZ2) {
+        const uint32_t sz = blob + 2 * tb + c * kSzEntryBytes, sw = lds_u1(sz + (lane >> 2) * 4);
+        make_zc<FMT>(zc, lds_u16(sz + 32 + (lane >> 2) * 2));
+        s = __half22float2(*reinterpret_cast<const __half2*>(&sw));
+      }
+    }
+    RawTile<FMT> r;
+    load_tile_s<FMT>(r, blob + c * tb, lane);
+    uint32_t a[4][4];
+    tile_frags<FMT>(r, zc, a, lut);
+    uint32_t xr[8];
+    load_xf(xr, row, c);
+#pragma unroll
+    for (int i = 0; i < 4; ++i) mma16816(d[i & 1], a[i], xr[2 * i], xr[2 * i + 1]);
+    if constexpr (LO) {
+      load_xf(xr, row + lo, c);
+#pragma unroll
+      for (int i = 0; i < 4; ++i) mma16816(d[i & 1], a[i], xr[2 * i], xr[2 * i + 1]);
+    }
+    if (c == 1 || (quant && SZ2)) {
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        acc[i] = fmaf(d[0][i] + d[1][i], i < 2 ? s.x : s.y, acc[i]);
+        d[0][i] = 0.f; d[1][i] = 0.f;
+      }
+    }
+  }
+}
 
+// ---- A: t = X . A ---------------------------------------------------------------------------------------------------
+// Unit u = (row tile of A, part of the reduction axis); its pairs go round the sixteen warps, whose sums meet in shared
+// memory; the 16 x m results leave as words (value, launch number).
+template <int ABF, bool SZ2, int kWarps>
+__device__ __forceinline__ void run_a(const DecodeArgs& p, float* red, int warp, int lane, unsigned long long* tr) {
+  constexpr uint32_t blob_b = blob_bytes(ABF, SZ2 ? 1 : 0);
+  const uint32_t units = p.a_nt * p.a_slices;
+  const int g = lane >> 2, t = lane & 3;
+  const bool has = g < p.m;
+  // weights ahead of the dependency: everything of this CTA towards L2 (A and B are small: 173 against 189 us without)
+  for (uint32_t u = blockIdx.x + p.n_a * threadIdx.x; u < units; u += p.n_a * (kWarps * 32)) {
+    const uint32_t tile = u % p.a_nt, s = u / p.a_nt, p0 = s * p.a_slice_pairs;
+    if (p0 < p.a_np) prefetch_l2(p.a_q + ((size_t)tile * p.a_np + p0) * blob_b, min(p.a_slice_pairs, p.a_np - p0) * blob_b);
+  }
   asm volatile("griddepcontrol.wait;" ::: "memory");
   if (tr && lane == 0) tr[1] = globaltimer_ns();
-
-  WalkI8 wk;
-  if constexpr (I8 == 1) {
-    wk.pair = kNone; wk.next_b = kNone; wk.tile = 0; wk.yb = p.y_ws; wk.my_tile = 0; wk.batch_n = 0; wk.tk_n = 0; wk.tk_old = 0; wk.tk_tile = 0;
+  const uint32_t launch = (uint32_t)(ld_volatile_u64(p.launches) >> kLaunchShift) + 1u;
+  const uint16_t* xrow = reinterpret_cast<const uint16_t*>(p.x) + (size_t)(has ? g : 0) * p.d_in + 8 * t;
+  int flip = 0;
+  for (uint32_t u = blockIdx.x; u < units; u += p.n_a, flip ^= 1) {
+    const uint32_t tile = u % p.a_nt, s = u / p.a_nt;
+    const uint32_t p0 = s * p.a_slice_pairs, p1 = min(p.a_np, p0 + p.a_slice_pairs);
+    float acc[4] = {0.f, 0.f, 0.f, 0.f};
+    for (uint32_t q = p0 + warp; q < p1; q += kWarps) {
+      const uint8_t* blob = p.a_q + ((size_t)tile * p.a_np + q) * blob_b;
+      RawBlob<ABF, SZ2> r;
+      load_blob(r, blob, lane);
+      float d[2][4];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) { d[0][i] = 0.f; d[1][i] = 0.f; }
+      ZC zc;
+#pragma unroll
+      for (int c = 0; c < 2; ++c) {
+        uint4 xv[2];
+#pragma unroll
+        for (int b = 0; b < 2; ++b) {
+          xv[b] = has ? ld_cg_u4(xrow + (size_t)q * 128 + 32 * (2 * c + b)) : make_uint4(0u, 0u, 0u, 0u);
+          if (p.x_dtype == EORA_X_BF16) { xv[b].x = bf2_to_h2(xv[b].x); xv[b].y = bf2_to_h2(xv[b].y); xv[b].z = bf2_to_h2(xv[b].z); xv[b].w = bf2_to_h2(xv[b].w); }
+        }
+        if constexpr (fmt_quantised(ABF)) { if (c == 0 || SZ2) make_zc<ABF>(zc, r.z[SZ2 ? c : 0]); }
+        uint32_t a[4][4];
+        tile_frags<ABF>(r.t[c], zc, a, 0u);
+#pragma unroll
+        for (int b = 0; b < 2; ++b) {
+          mma16816(d[0], a[2 * b], xv[b].x, xv[b].y);
+          mma16816(d[1], a[2 * b + 1], xv[b].z, xv[b].w);
+        }
+        if (c == 1 || (fmt_quantised(ABF) && SZ2)) {
+          float2 sc = make_float2(1.f, 1.f);
+          if constexpr (fmt_quantised(ABF)) sc = __half22float2(*reinterpret_cast<const __half2*>(&r.s[SZ2 ? c : 0]));
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            acc[i] = fmaf(d[0][i] + d[1][i], i < 2 ? sc.x : sc.y, acc[i]);
+            d[0][i] = 0.f; d[1][i] = 0.f;
+          }
+        }
+      }
+    }
+    float* mine = red + (flip * kWarps + warp) * 16 * kMaxTok;
+    mine[(2 * t) * 16 + g] = acc[0]; mine[(2 * t + 1) * 16 + g] = acc[1];
+    mine[(2 * t) * 16 + g + 8] = acc[2]; mine[(2 * t + 1) * 16 + g + 8] = acc[3];
+    __syncthreads();
+    if (threadIdx.x < 16u * p.m) {
+      float v = 0.f;
+#pragma unroll
+      for (int w = 0; w < kWarps; ++w) v += red[(flip * kWarps + w) * 16 * kMaxTok + threadIdx.x];
+      const uint32_t tok = threadIdx.x >> 4, col = tile * 16 + (threadIdx.x & 15);
+      const unsigned long long word = ((unsigned long long)launch << 32) | __float_as_uint(v);
+      asm volatile("st.volatile.global.u64 [%0], %1;" ::"l"(p.t_part + ((size_t)s * p.m + tok) * p.t_cols + col), "l"(word) : "memory");
+    }
   }
-  bool ok = true;
-  if (a_owner) ok = run_segment<ABF, false, OUT_T>(p, r, a0, an, p.a_nt, blob_a, p.a_per_copy, p.a_sz2, lane);
-  if (ok) ok = run_backbone<WF, I8>(p, r, wk, w0, wf, blob_w, lane);
   if (tr && lane == 0) tr[2] = globaltimer_ns();
-  if (b_owner) {
-    if (ok) ok = run_segment<ABF, true, OUT_Y>(p, r, bb0, bn, p.w_nt, blob_b, p.b_per_copy, p.b_sz2, lane);
-    if (ok) ok = run_backbone<WF, I8>(p, r, wk, w0 + wf, wn - wf, blob_w, lane);
+}
+
+// ---- after the backbone: + t . B, the partner's sums, Y ---------------------------------------------------------------
+__device__ __forceinline__ int sub_of(const DecodeArgs& p, uint32_t tile) {
+  if (p.n_sub == 1) return 0;
+  int s = 0;
+#pragma unroll
+  for (int i = 1; i < 4; ++i)
+    if (i < p.n_sub && tile >= p.sub_tile0[i]) s = i;
+  return s;
+}
+
+// Two neighbouring columns of t, one part of the reduction axis: asked for (load) and, until the launch's words are there, again.
+struct TWords { unsigned long long a, b; };
+__device__ __forceinline__ void load_t(TWords& w, const unsigned long long* src) {
+  asm volatile("ld.volatile.global.v2.u64 {%0, %1}, [%2];" : "=l"(w.a), "=l"(w.b) : "l"(src) : "memory");
+}
+__device__ __forceinline__ bool wait_t(const DecodeArgs& p, TWords& w, const unsigned long long* src, uint32_t launch) {
+  unsigned long long t0 = 0;
+  for (uint32_t tries = 1;; ++tries) {
+    if ((uint32_t)(w.a >> 32) == launch && (uint32_t)(w.b >> 32) == launch) return true;
+    if ((tries & 63u) == 0u) {
+      const unsigned long long now = globaltimer_ns();
+      if (t0 == 0) t0 = now;
+      else if (now - t0 > p.wait_ns) { atomicExch(p.dev_status, EORA_ERR_DEVICE_TIMEOUT); return false; }
+    }
+    load_t(w, src);
   }
-  if constexpr (I8 == 1) {
-    if (ok) { tickets_take(p, wk, lane); tickets_resolve(p, wk, lane); }
+}
+
+// x / n for small x; inv = ceil(2^32 / n), 0 for n == 1
+__device__ __forceinline__ uint32_t div_by(uint32_t x, uint32_t inv) { return inv ? __umulhi(x, inv) : x; }
+// The warps whose runs hold blobs of row tile f of a chunk of n pairs: those of its first to its last blob.  Warp w's run is
+// [w L / kWarps, (w + 1) L / kWarps) of the L blobs; inv = ceil(2^32 / L).
+struct Owners { uint32_t a, b; };
+template <int kWarps>
+__device__ __forceinline__ Owners owners_of(uint32_t f, uint32_t n, uint32_t inv) {
+  const uint32_t x = (f * n + 1) * kWarps - 1;
+  return {div_by(x, inv), div_by(x + (n - 1) * kWarps, inv)};
+}
+
+// A warp's ring of weights in shared memory: position of the slot that is read next, its barrier and the phase it completes.
+struct Ring { uint32_t base, bytes, bars, so, bar, parity; };
+__device__ __forceinline__ void ring_next(Ring& r, uint32_t slot_b) {
+  r.so += slot_b; r.bar += 8;
+  if (r.so == r.bytes) { r.so = 0; r.bar = r.bars; r.parity ^= 1u; }
+}
+
+// Pairs of t that row tile `tile` takes part in, within [c0, c1): [a, b).
+struct Span { uint32_t a, b, base; };
+__device__ __forceinline__ Span t_span(const DecodeArgs& p, uint32_t tile, uint32_t c0, uint32_t c1) {
+  Span s;
+  s.base = p.sub_pairs ? (uint32_t)sub_of(p, tile) * p.sub_pairs : 0u;
+  s.a = max(c0, s.base); s.b = min(c1, s.base + p.b_np);
+  return s;
+}
+
+// What a CTA does once its warps' runs are in `seg`: adds up the row tiles that its partner finishes and sends it the sums,
+// adds t . B and the partner's sums to its own, and stores Y.  Everything that has to come from L2 (the first words of t, the
+// first blob of B, which goes to the warp's ring) is asked for before the barrier that the warps meet at.  All of it is
+// latency -- a shared-memory load in a rolled loop costs 60 cycles -- so every element has a thread of its own: half a warp
+// per (row tile, token), tokens counted up to a power of two (1 << p.m_log).  Few values live across its phases: with two
+// CTAs of 512 threads an SM has 64 registers a thread, and a spill goes to L2 (shared memory takes nearly all of the L1).
+//
+// The product with B: unit u = (row tile u >> b_log, every (1 << b_log)-th of its pairs in the chunk of t, from u's low bits on);
+// units go round the warps.  bar, parity: the barrier of the warp's (empty) ring that a blob of B arrives at.
+template <int ABF, bool SZ2, int kWarps>
+__device__ __forceinline__ void finish(const DecodeArgs& p, uint8_t* smem, uint32_t ring, uint32_t bar, uint32_t parity, uint32_t t0, uint32_t nT,
+                                       uint32_t rank, uint32_t n, uint32_t inv, uint32_t launch, unsigned long long* tr) {
+  constexpr bool ab = ABF != FMT_NONE;
+  constexpr uint32_t blob_b = blob_bytes(ABF, SZ2 ? 1 : 0);
+  const uint32_t OT = 16u * p.m;
+  const uint32_t f0 = rank ? nT >> 1 : 0u, nf = (p.ks == 2 && rank == 0 ? nT >> 1 : nT) - f0;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  float* const seg = reinterpret_cast<float*>(smem + p.off_seg);
+  const uint32_t hw = threadIdx.x >> 4, row = threadIdx.x & 15;
+  const uint32_t first_tile = t0 + f0;
+
+  auto ask_b = [&](uint32_t tile, uint32_t pair) {
+    if (lane == 0) {
+      mbar_expect_tx_a(bar, blob_b);
+      bulk_g2s_a(ring, p.b_q + ((size_t)tile * p.b_np + pair) * blob_b, blob_b, bar);
+    }
+  };
+  // step e of a chunk of t: two columns of one token (64 steps per pair and token)
+  auto t_tok = [&](uint32_t e) { return (e >> 6) & ((1u << p.m_log) - 1); };
+  auto t_col = [&](uint32_t e) { return (e >> (6 + p.m_log)) * 128 + (e & 63) * 2; };
+  uint32_t c0 = 0, c_end = p.b_np;                 // the chunk of t and the end of all chunks
+  TWords tw = {0ull, 0ull};
+  if constexpr (ab) {
+    if (p.sub_pairs && nf) { c0 = (uint32_t)sub_of(p, first_tile) * p.sub_pairs; c_end = (uint32_t)(sub_of(p, first_tile + nf - 1) + 1) * p.sub_pairs; }
+    if (warp < (int)(nf << p.b_log)) {
+      const uint32_t tile = first_tile + (warp >> p.b_log);
+      const Span s = t_span(p, tile, c0, c0 + p.t_chunk);
+      const uint32_t q = s.a + (warp & ((1u << p.b_log) - 1));
+      if (q < s.b) ask_b(tile, q - s.base);
+    }
+    if (t_tok(threadIdx.x) < (uint32_t)p.m && c0 * 128 + t_col(threadIdx.x) < (uint32_t)p.t_cols)
+      load_t(tw, p.t_part + (size_t)t_tok(threadIdx.x) * p.t_cols + c0 * 128 + t_col(threadIdx.x));
   }
-  if (!ok) {
-    // This warp gave up: its bulk copies still in flight must land before the CTA's shared memory may be reused.  A slot
-    // of the ring is in flight exactly if a copy was requested for it and not consumed: slots from the consumer position on
-    // waits for the phase its next copy completes; a slot without a copy in flight runs into the drain's short limit.
-    for (int i = 0; i < kRing - r.deferred; ++i) mbar_drain_warp(r.bars + i, (r.phase >> i) & 1u, lane);
+  __syncthreads();
+  if (tr && lane == 0) tr[2] = globaltimer_ns();
+
+  auto tile_sum = [&](uint32_t f, uint32_t i) {    // element i of the sums of row tile f: of all warps that hold blobs of it
+    const Owners o = owners_of<kWarps>(f, n, inv);
+    const float* src = seg + (o.a + f) * OT + i;
+    float v0 = 0.f, v1 = 0.f;
+    if ((rank ? p.w_np - p.pairs : p.pairs) > p.chunk) v0 = reinterpret_cast<const float*>(smem + p.off_sum)[f * OT + i];     // of the chunks before
+    uint32_t k = o.b - o.a + 1;
+    for (; k >= 4; k -= 4, src += 4 * OT) { v0 += src[0] + src[OT]; v1 += src[2 * OT] + src[3 * OT]; }
+    if (k > 0) v0 += src[0];
+    if (k > 1) v1 += src[OT];
+    if (k > 2) v0 += src[2 * OT];
+    return v0 + v1;
+  };
+  if (p.ks == 2) {
+    // the partner's tiles: [nf, nT) for rank 0, [0, f0) for rank 1
+    cluster_wait();
+    const uint32_t to = mapa(smem_u32(smem + p.off_inbox), rank ^ 1u) + row * 4;
+    for (uint32_t u = hw; u < (nT - nf) << p.m_log; u += 2 * kWarps) {
+      const uint32_t f = u >> p.m_log, tok = u & ((1u << p.m_log) - 1);
+      if (tok < (uint32_t)p.m)
+        asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(to + (f * OT + tok * 16) * 4), "f"(tile_sum(rank ? f : nf + f, tok * 16 + row)) : "memory");
+    }
+    cluster_arrive();
+  }
+  if constexpr (ab) {
+    const uint32_t pitch = p.t_chunk * 256 + 64;
+    const uint32_t th = smem_u32(smem + p.off_t);
+    float* const bseg = reinterpret_cast<float*>(smem + p.off_bseg);
+    bool first = true;
+#pragma unroll 1
+    while (nf) {
+      // t of this chunk as fp16 high and low parts (error 2^-22 of the value), zero for tokens that do not use the pair's adapter
+      // and in the columns past A's rows (padding)
+      const uint32_t steps = min(p.t_chunk, c_end - c0) << (6 + p.m_log);
+      for (uint32_t e = threadIdx.x; e < steps; e += (kWarps * 32)) {
+        const uint32_t tok = t_tok(e), col = t_col(e);
+        if (tok >= (uint32_t)p.m) continue;
+        float v0 = 0.f, v1 = 0.f;
+        if (c0 * 128 + col < p.a_nt * 16 && !(p.adp_pairs && p.adp[tok] != (int)((c0 + (col >> 7)) / p.adp_pairs))) {
+          const unsigned long long* src = p.t_part + (size_t)tok * p.t_cols + c0 * 128 + col;
+#pragma unroll 1
+          for (uint32_t s = 0; s < p.a_slices; ++s, src += (size_t)p.m * p.t_cols) {
+            if (!first || s || e != threadIdx.x) load_t(tw, src);
+            if (!wait_t(p, tw, src, launch)) break;
+            v0 += __uint_as_float((uint32_t)tw.a); v1 += __uint_as_float((uint32_t)tw.b);
+          }
+        }
+        const uint32_t hi = pack_h2(v0, v1);
+        const float2 hf = __half22float2(*reinterpret_cast<const __half2*>(&hi));
+        const uint32_t d = th + tok * pitch + col * 2;
+        sts_u1(d, hi);
+        sts_u1(d + p.m * pitch, pack_h2(v0 - hf.x, v1 - hf.y));
+      }
+      __syncthreads();
+#pragma unroll 1
+      for (uint32_t u = warp; u < nf << p.b_log; u += kWarps) {
+        const uint32_t tile = first_tile + (u >> p.b_log);
+        const Span s = t_span(p, tile, c0, c0 + p.t_chunk);
+        float acc[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll 1
+        for (uint32_t q = s.a + (u & ((1u << p.b_log) - 1)), k = 0; q < s.b; q += 1u << p.b_log, ++k) {
+          if (!first || u != (uint32_t)warp || k) ask_b(tile, q - s.base);
+          if (!mbar_try_wait_a(bar, parity)) mbar_wait_lane(bar, parity, p.dev_status);
+          parity ^= 1u;
+          __syncwarp();
+          // columns past the tokens repeat the last one; their sums are not stored
+          product_exact<ABF, SZ2, true>(ring, lane, th + min((uint32_t)lane >> 2, (uint32_t)p.m - 1) * pitch + (lane & 3) * 16 + (q - c0) * 256, p.m * pitch, 0u, acc);
+          __syncwarp();
+        }
+        float* d = bseg + u * OT + (lane >> 2) + (lane & 3) * 32;
+        if (2 * (lane & 3) < p.m) { d[0] = acc[0]; d[8] = acc[2]; }
+        if (2 * (lane & 3) + 1 < p.m) { d[16] = acc[1]; d[24] = acc[3]; }
+      }
+      c0 += p.t_chunk;
+      if (c0 >= c_end) break;
+      first = false;
+      __syncthreads();
+      // more chunks of t: this one's products join the first of the tile's partial sums
+      for (uint32_t e = threadIdx.x; e < nf * OT; e += (kWarps * 32)) {
+        const uint32_t f = e / OT, i = e - f * OT;
+        float v = 0.f;
+        for (uint32_t k = 0; k < 1u << p.b_log; ++k) v += bseg[((f << p.b_log) + k) * OT + i];
+        seg[(owners_of<kWarps>(f0 + f, n, inv).a + f0 + f) * OT + i] += v;
+      }
+    }
+  }
+  if (p.ks == 2) cluster_wait();
+  __syncthreads();
+  for (uint32_t u = hw; u < nf << p.m_log; u += 2 * kWarps) {
+    const uint32_t f = u >> p.m_log, tok = u & ((1u << p.m_log) - 1), i = tok * 16 + row;
+    if (tok >= (uint32_t)p.m) continue;
+    float v = tile_sum(f0 + f, i);
+    if (p.ks == 2) v += reinterpret_cast<const float*>(smem + p.off_inbox)[f * OT + i];
+    if constexpr (ab)
+      for (uint32_t k = 0; k < 1u << p.b_log; ++k) v += reinterpret_cast<const float*>(smem + p.off_bseg)[((f << p.b_log) + k) * OT + i];
+    const uint32_t tg = first_tile + f;
+    void* y = p.ys[0];
+    uint32_t st0 = 0;
+    int dout = p.sub_dout[0];
+    if (p.n_sub > 1) {
+#pragma unroll
+      for (int k = 1; k < 4; ++k)
+        if (k < p.n_sub && tg >= p.sub_tile0[k]) { y = p.ys[k]; st0 = p.sub_tile0[k]; dout = p.sub_dout[k]; }
+    }
+    store_y(y, p.y_dtype, (int64_t)tok * dout + (tg - st0) * 16 + row, v);
+  }
+}
+
+// MODE 1: one token through the integer product, 0: fp16 activations.
+// Blobs that a warp multiplies at once.
+__host__ __device__ constexpr uint32_t fast_blobs(int fmt, int mode) { return mode == 1 ? 4 : fmt == FMT_Q4 || fmt == FMT_Q3 ? 2 : 1; }
+
+template <int WF, int MODE, bool SZ2>
+__global__ void __launch_bounds__(32 << warp_log(MODE), MODE == 1 ? 2 : 1) k_decode(const __grid_constant__ DecodeArgs p) {
+  constexpr int kWarpLog = warp_log(MODE), kWarps = 1 << kWarpLog;
+  extern __shared__ __align__(128) uint8_t smem[];
+  __shared__ uint32_t lut_s[16];
+  __shared__ __align__(16) uint32_t zero_s[40];    // what lanes without a token read as their activations
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  asm volatile("griddepcontrol.launch_dependents;");
+  touch_args(p);
+  unsigned long long* tr = p.trace ? p.trace + (size_t)(blockIdx.x * 16 + warp) * 4 : nullptr;
+  if (tr && lane == 0) tr[0] = globaltimer_ns();
+
+  if (blockIdx.x < p.n_a) {
+    float* red = reinterpret_cast<float*>(smem);
+    switch (p.a_fmt) {
+      case FMT_F16: run_a<FMT_F16, false, kWarps>(p, red, warp, lane, tr); break;
+      case FMT_Q8: run_a<FMT_Q8, false, kWarps>(p, red, warp, lane, tr); break;
+      case FMT_Q4: if (p.a_sz2) run_a<FMT_Q4, true, kWarps>(p, red, warp, lane, tr); else run_a<FMT_Q4, false, kWarps>(p, red, warp, lane, tr); break;
+      case FMT_Q3: if (p.a_sz2) run_a<FMT_Q3, true, kWarps>(p, red, warp, lane, tr); else run_a<FMT_Q3, false, kWarps>(p, red, warp, lane, tr); break;
+      default: break;
+    }
+  } else {
+    constexpr uint32_t blob_b = blob_bytes(WF, SZ2 ? 1 : 0);
+    const uint32_t cta = blockIdx.x - p.n_a, cl = p.ks == 2 ? cta >> 1 : cta, rank = p.ks == 2 ? cta & 1 : 0;
+    const uint32_t t0 = share_lo(p.tiles, cl), nT = share_n(p.tiles, cl);
+    const DecodeArgs::Part part = p.part[rank];
+    const uint32_t pr0 = rank * p.pairs, P = part.pairs;
+    const uint32_t OT = 16u * p.m;
+    uint8_t* xs = smem;
+    float* seg = reinterpret_cast<float*>(smem + p.off_seg);
+    // the CTA's blobs are one contiguous range: the two halves of the reduction axis are stored one after the other
+    const uint8_t* w_part = p.w_q + ((size_t)rank * p.w_nt * p.pairs + (size_t)t0 * P) * blob_b;
+    if (p.ks == 2) cluster_arrive();               // (that the partner runs at all, before anything is written to it)
+    uint32_t lut = 0;
+    if constexpr (WF == FMT_SP24 || WF == FMT_SQ4) {
+      if (threadIdx.x < 16) lut_s[threadIdx.x] = sp24_selectors(threadIdx.x);
+      lut = smem_u32(lut_s);
+    }
+    if (threadIdx.x < 40) zero_s[threadIdx.x] = 0u;
+
+    // A warp's run of a chunk of n pairs: blobs [lo, hi) in (row tile, pair) order.  They come through the warp's own ring in
+    // shared memory, one bulk copy of up to slot_blobs blobs per slot.
+    const uint32_t slot_b = p.slot_blobs * blob_b;
+    Ring ring;
+    ring.bytes = p.slots * slot_b; ring.base = smem_u32(smem + p.off_ring) + warp * p.ring_pitch;
+    ring.bars = ring.bar = smem_u32(smem + p.off_bar) + warp * (kMaxSlots * 8);
+    ring.so = 0; ring.parity = 0;
+    if (lane == 0) {
+      for (uint32_t i = 0; i < p.slots; ++i) mbar_init_a(ring.bars + 8 * i, 1);
+      asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    }
+    __syncwarp();
+    uint32_t left = 0, tile = 0, pr = 0;           // blobs of the run still to be multiplied; the next one
+    uint32_t l_left = 0, l_pr = 0;                 // copies: blobs of the run still to be asked for, pair of the next one
+    const uint8_t* l_ptr = w_part;
+    const bool whole = P <= p.chunk;                     // one chunk: the run is contiguous in memory
+    auto open_run = [&](uint32_t c, uint32_t n) {
+      const uint32_t L = nT * n, lo = ((uint32_t)warp * L) >> kWarpLog;
+      left = (((uint32_t)(warp + 1) * L) >> kWarpLog) - lo;
+      tile = whole ? div_by(lo, part.inv_pairs) : lo / n;
+      pr = lo - tile * n;
+      l_pr = pr; l_left = left;
+      l_ptr = w_part + ((size_t)tile * P + c + pr) * blob_b;
+    };
+    auto ask = [&](uint32_t dst_o, uint32_t b, uint32_t n) {
+      uint32_t cnt = min(p.slot_blobs, l_left);
+      if (!whole) cnt = min(cnt, n - l_pr);
+      if (cnt == 0) return;
+      const uint32_t bytes = cnt * blob_b;
+      if (lane == 0) {
+        mbar_expect_tx_a(b, bytes);
+        bulk_g2s_a(ring.base + dst_o, l_ptr, bytes, b);
+      }
+      l_left -= cnt; l_ptr += bytes;
+      if (!whole) { l_pr += cnt; if (l_pr == n) { l_pr = 0; l_ptr += (P - n) * blob_b; } }
+    };
+    auto fill = [&](uint32_t n) {                  // the first copies of a run, into the slots from the reading position on
+      uint32_t o = ring.so, b = ring.bar;
+#pragma unroll 1
+      for (uint32_t i = 0; i < p.slots; ++i) {
+        ask(o, b, n);
+        o += slot_b; b += 8;
+        if (o == ring.bytes) { o = 0; b = ring.bars; }
+      }
+    };
+    const uint32_t chunk0 = min(p.chunk, P);
+    open_run(0, chunk0);
+    fill(chunk0);
+    if (p.n_a) {
+      const uint32_t f0 = rank ? nT >> 1 : 0u, nf = (p.ks == 2 && rank == 0 ? nT >> 1 : nT) - f0;
+      const uint32_t per_tile = p.b_np * (uint32_t)blob_bytes(p.a_fmt, (int)p.b_sz2), bytes = nf * per_tile;
+      const uint8_t* b_part = p.b_q + (size_t)(t0 + f0) * per_tile;
+      for (uint32_t o = threadIdx.x << 14; o < bytes; o += (kWarps * 32) << 14) prefetch_l2(b_part + o, min(16384u, bytes - o));
+    }
+    const int g = lane >> 2, t = lane & 3;
+    const bool bf16 = p.x_dtype == EORA_X_BF16;
+    bool ok = true;
+
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    if (tr && lane == 0) tr[1] = globaltimer_ns();
+    const uint32_t launch = (uint32_t)(ld_volatile_u64(p.launches) >> kLaunchShift) + 1u;
+
+    uint32_t n = 0, inv = 0;
+#pragma unroll 1
+    for (uint32_t c = 0; c < P; c += p.chunk) {
+      n = min(p.chunk, P - c);
+      inv = whole ? part.inv_blobs[nT - p.tiles.per] : 0xffffffffu / (nT * n) + 1u;
+      const uint32_t pitch = p.chunk * 256 + 64;
+      float* xsum = reinterpret_cast<float*>(xs + (size_t)p.m * pitch);          // fp16 path: [2 chunk][8] sums, [chunk][8] scales
+      float* xscale = xsum + 2 * p.chunk * kMaxTok;
+      if (c > 0) {
+        open_run(c, n);
+        fill(n);
+      }
+      if constexpr (MODE == 1) stage_x_i8<WF, kWarps>(smem_u32(xs), p.x, bf16, pr0 + c, n, warp, lane);
+      else stage_x_f16<WF, kWarps>(xs, pitch, xsum, xscale, p.x, bf16, p.m, p.d_in, pr0 + c, n);
+      __syncthreads();
+      float acc[MODE == 1 ? 2 : 4];
+#pragma unroll
+      for (int i = 0; i < (MODE == 1 ? 2 : 4); ++i) acc[i] = 0.f;
+      // this lane's activations of a pair: base and step per pair (lanes without a token stay on the zeros)
+      const bool has = MODE == 1 ? g < 2 : g < p.m;
+      const uint32_t x_step = has ? (MODE == 1 ? kPlaneBytes : 256u) : 0u;
+      const uint32_t x_base = has ? smem_u32(xs) + (MODE == 1 ? (g * 4 + t) * 16 : g * pitch + t * 16) : smem_u32(zero_s);
+      const uint32_t x_meta = MODE == 1 ? smem_u32(xs) + 256 : smem_u32(xsum) + 8 * t;
+      float* d = seg + (warp + tile) * OT + g;
+      auto flush = [&]() {
+        if constexpr (MODE == 1) {
+          if (t == 0) { d[0] = acc[0]; d[8] = acc[1]; }
+          acc[0] = acc[1] = 0.f;
+        } else {
+          if (2 * t < p.m) { d[(2 * t) * 16] = acc[0]; d[(2 * t) * 16 + 8] = acc[2]; }
+          if (2 * t + 1 < p.m) { d[(2 * t + 1) * 16] = acc[1]; d[(2 * t + 1) * 16 + 8] = acc[3]; }
+          acc[0] = acc[1] = acc[2] = acc[3] = 0.f;
+        }
+        d += OT;
+      };
+      uint32_t xa = x_base + pr * x_step, xm = x_meta + pr * (MODE == 1 ? (uint32_t)kPlaneBytes : 8u * kMaxTok);
+      bool open = left == 0;                       // something to leave in the slot at the end (an empty run leaves zeros)
+#pragma unroll 1
+      while (left > 0) {
+        uint32_t cnt = min(p.slot_blobs, left);
+        if (!whole) cnt = min(cnt, n - pr);
+        if (ok && !mbar_try_wait_a(ring.bar, ring.parity) && !mbar_wait_lane(ring.bar, ring.parity, p.dev_status)) {
+          ok = false;                              // gave up: nothing more is asked for, and what is in flight must land first
+          l_left = 0;
+        }
+        __syncwarp();
+        uint32_t src = ring.base + ring.so;
+        left -= cnt;
+        // NB blobs of one row tile at once (independent chains hide one another's latency), one at a time around its end
+        constexpr uint32_t NB = fast_blobs(WF, MODE), xm_step = MODE == 1 ? (uint32_t)kPlaneBytes : 8u * kMaxTok;
+        open = true;
+        auto blobs = [&](auto count) {
+          constexpr int N = decltype(count)::value;
+          if constexpr (WF == FMT_Q4 || WF == FMT_Q3) {
+            RawBlob<WF, SZ2> raw[N];
+#pragma unroll
+            for (int k = 0; k < N; ++k) load_blob_s(raw[k], src + k * blob_b, lane);
+#pragma unroll
+            for (int k = 0; k < N; ++k) {
+              if constexpr (MODE == 1) product_i8<WF, SZ2>(raw[k], xa + k * x_step, xm + k * xm_step, acc);
+              else product_codes<WF, SZ2>(raw[k], xa + k * x_step, xm + k * xm_step, smem_u32(xscale) + ((pr + k) * kMaxTok + 2 * t) * 4, bf16, acc);
+            }
+          } else {
+#pragma unroll
+            for (int k = 0; k < N; ++k) product_exact<WF, SZ2, false>(src + k * blob_b, lane, xa + k * x_step, 0u, lut, acc);
+          }
+          src += N * blob_b; xa += N * x_step; xm += N * xm_step; pr += N; cnt -= N;
+          if (pr == n) { flush(); open = false; pr = 0; xa = x_base; xm = x_meta; }
+        };
+#pragma unroll 1
+        while (cnt > 0) {
+          if (NB > 1 && cnt >= NB && pr + NB <= n) { open = true; blobs(std::integral_constant<int, NB>()); }
+          else { open = true; blobs(std::integral_constant<int, 1>()); }
+        }
+        __syncwarp();                              // every lane is done with the slot
+        ask(ring.so, ring.bar, n);
+        ring_next(ring, slot_b);
+      }
+      if (open) flush();
+      if (c + p.chunk < P) {                       // more chunks: add up what there is
+        __syncthreads();
+        float* sum = reinterpret_cast<float*>(smem + p.off_sum);
+        for (uint32_t f = threadIdx.x >> 4; f < nT; f += 2 * kWarps) {
+          const Owners o = owners_of<kWarps>(f, n, inv);
+          for (uint32_t i = threadIdx.x & 15; i < OT; i += 16) {
+            float v = c ? sum[f * OT + i] : 0.f;
+            for (uint32_t w = o.a; w <= o.b; ++w) v += seg[(w + f) * OT + i];
+            sum[f * OT + i] = v;
+          }
+        }
+      }
+    }
+    if (!__all_sync(0xffffffffu, ok)) {
+      for (uint32_t i = 0; i < p.slots; ++i) mbar_drain_warp(reinterpret_cast<uint64_t*>(smem + p.off_bar) + warp * kMaxSlots + i, ring.bars + 8 * i < ring.bar ? ring.parity ^ 1u : ring.parity, lane);
+    }
+    switch (p.a_fmt) {
+      case FMT_F16: finish<FMT_F16, false, kWarps>(p, smem, ring.base, ring.bar, ring.parity, t0, nT, rank, n, inv, launch, tr); break;
+      case FMT_Q8: finish<FMT_Q8, false, kWarps>(p, smem, ring.base, ring.bar, ring.parity, t0, nT, rank, n, inv, launch, tr); break;
+      case FMT_Q4: if (p.b_sz2) finish<FMT_Q4, true, kWarps>(p, smem, ring.base, ring.bar, ring.parity, t0, nT, rank, n, inv, launch, tr);
+                   else finish<FMT_Q4, false, kWarps>(p, smem, ring.base, ring.bar, ring.parity, t0, nT, rank, n, inv, launch, tr); break;
+      case FMT_Q3: if (p.b_sz2) finish<FMT_Q3, true, kWarps>(p, smem, ring.base, ring.bar, ring.parity, t0, nT, rank, n, inv, launch, tr);
+                   else finish<FMT_Q3, false, kWarps>(p, smem, ring.base, ring.bar, ring.parity, t0, nT, rank, n, inv, launch, tr); break;
+      default: finish<FMT_NONE, false, kWarps>(p, smem, ring.base, ring.bar, ring.parity, t0, nT, rank, n, inv, launch, tr); break;
+    }
+  }
+  __syncthreads();                                 // every thread of the CTA has read the launch counter
+  if (threadIdx.x == 0) {
+    // 2^10 per launch in all: a CTA's 1, and the last CTA of the grid the rest, so that the count never reaches the next
+    // multiple before every CTA has read it
+    const unsigned long long v = blockIdx.x + 1 == gridDim.x ? (1ull << kLaunchShift) - (gridDim.x - 1) : 1ull;
+    asm volatile("red.global.add.u64 [%0], %1;" ::"l"(p.launches), "l"(v) : "memory");
   }
   if (tr && lane == 0) tr[3] = globaltimer_ns();
 }
@@ -629,45 +898,35 @@ cudaError_t launch_kernel(const cudaLaunchConfig_t& cfg, const DecodeArgs& args,
   static bool attr_set[64] = {};  // per kernel (KERNEL is a template argument) and device: the attribute belongs to the current device
   if (device < 0 || device >= 64) return cudaErrorInvalidDevice;
   if (!attr_set[device]) {
-    cudaError_t e = cudaFuncSetAttribute(KERNEL, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
+    cudaError_t e = cudaFuncSetAttribute(KERNEL, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem);
     if (e != cudaSuccess) return e;
     attr_set[device] = true;
   }
   return cudaLaunchKernelEx(&cfg, KERNEL, args);
 }
 
-// Formats whose backbone blobs have an integer inner product.
-constexpr bool has_i8(int fmt) { return fmt == FMT_Q4 || fmt == FMT_Q3; }
-
-template <int WF, int I8>
-cudaError_t launch_ab2(const cudaLaunchConfig_t& cfg, const DecodeArgs& args, int abf, int device) {
-  switch (abf) {
-    case FMT_F16: return launch_kernel<k_decode<WF, FMT_F16, I8>>(cfg, args, device);
-    case FMT_Q4: return launch_kernel<k_decode<WF, FMT_Q4, I8>>(cfg, args, device);
-    case FMT_Q8: return launch_kernel<k_decode<WF, FMT_Q8, I8>>(cfg, args, device);
-    case FMT_Q3: return launch_kernel<k_decode<WF, FMT_Q3, I8>>(cfg, args, device);
-    default: return launch_kernel<k_decode<WF, FMT_NONE, I8>>(cfg, args, device);
+cudaError_t launch_any(const cudaLaunchConfig_t& cfg, const DecodeArgs& a, int wf, bool sz2, int device) {
+  const bool one = a.m == 1;
+  switch (wf) {
+    case FMT_Q4:
+      if (one) return sz2 ? launch_kernel<k_decode<FMT_Q4, 1, true>>(cfg, a, device) : launch_kernel<k_decode<FMT_Q4, 1, false>>(cfg, a, device);
+      return sz2 ? launch_kernel<k_decode<FMT_Q4, 0, true>>(cfg, a, device) : launch_kernel<k_decode<FMT_Q4, 0, false>>(cfg, a, device);
+    case FMT_Q3:
+      if (one) return sz2 ? launch_kernel<k_decode<FMT_Q3, 1, true>>(cfg, a, device) : launch_kernel<k_decode<FMT_Q3, 1, false>>(cfg, a, device);
+      return sz2 ? launch_kernel<k_decode<FMT_Q3, 0, true>>(cfg, a, device) : launch_kernel<k_decode<FMT_Q3, 0, false>>(cfg, a, device);
+    case FMT_SQ4: return sz2 ? launch_kernel<k_decode<FMT_SQ4, 0, true>>(cfg, a, device) : launch_kernel<k_decode<FMT_SQ4, 0, false>>(cfg, a, device);
+    case FMT_SP24: return launch_kernel<k_decode<FMT_SP24, 0, false>>(cfg, a, device);
+    default: return cudaErrorInvalidValue;
   }
 }
-template <int WF>
-cudaError_t launch_ab(const cudaLaunchConfig_t& cfg, const DecodeArgs& args, int abf, int device) {
-  if constexpr (has_i8(WF)) {
-    if (args.m == 1) return launch_ab2<WF, 1>(cfg, args, abf, device);
-    return launch_ab2<WF, 2>(cfg, args, abf, device);
-  }
-  return launch_ab2<WF, 0>(cfg, args, abf, device);
-}
 
-// Relative cost of one blob (time a warp spends on it); only the ratios matter.
-double blob_cost(int fmt, bool hilo) {
+// SM cycles per blob of the backbone / of A or B (only the ratios matter, to deal the CTAs).
+double blob_cost(int fmt, bool int8) {
   switch (fmt) {
-    case FMT_Q3: return 1.00;
-    case FMT_Q4: return 1.05;
-    case FMT_Q8: return 1.40;
-    case FMT_F16: return hilo ? 1.30 : 1.10;
-    case FMT_SP24: return 1.60;
-    case FMT_SQ4: return 1.10;
-    default: return 0.0;
+    case FMT_Q3: case FMT_Q4: return int8 ? 32.0 : 42.0;
+    case FMT_SQ4: return 50.0;
+    case FMT_SP24: return 100.0;          // 2304 bytes: HBM's rate
+    default: return 45.0;
   }
 }
 
@@ -678,139 +937,183 @@ Share make_share(uint32_t total, uint32_t n) {
   return s;
 }
 
-uint32_t blobs_per_copy(const WMat& m) {
-  int n = kSlotBytes / m.blob;
-  return (uint32_t)(n < 1 ? 1 : n);
+struct Plan { DecodeArgs a; int grid; int warps; int smem; };
+
+// How a launch of m (at most eight) tokens is cut up; false if its shared memory does not fit.
+bool make_plan(const Handle* h, int m, Plan& pl) {
+  DecodeArgs& a = pl.a;
+  a = DecodeArgs();
+  const bool ab = h->cfg.rank > 0;
+  const bool int8 = m == 1 && (h->w.fmt == FMT_Q4 || h->w.fmt == FMT_Q3);
+  const uint32_t kWarps = 1u << warp_log(int8 ? 1 : 0);
+  pl.warps = (int)kWarps;
+  a.w_q = h->w.q; a.w_nt = h->w.nt; a.w_np = h->w.np;
+  a.ks = h->w.np >= 2 ? 2 : 1;
+  a.pairs = h->w.half;
+  a.m = m;
+  while ((1 << a.m_log) < m) ++a.m_log;
+  const uint32_t nt = h->w.nt, sms = (uint32_t)h->sm_count / a.ks * a.ks;
+  a.a_fmt = FMT_NONE;
+  a.a_slices = 1;
+  if (ab) {
+    a.a_fmt = h->a.fmt; a.a_q = h->a.q; a.a_nt = h->a.nt; a.a_np = h->a.np; a.a_sz2 = h->a.sz2;
+    a.b_q = h->b.q; a.b_np = h->b.np; a.b_sz2 = h->b.sz2;
+    // CTAs for A.  They work beside the others; what counts is the later of "the backbone's products are done" and "t
+    // has arrived" (an exchange through L2 takes about 2500 cycles).  Row tiles are dealt whole, so some CTAs are often
+    // free; of equal choices the one with the earliest t is taken.
+    const double cw = blob_cost(h->w.fmt, int8), ca = blob_cost(h->a.fmt, false);
+    double best = 1e30, best_a = 1e30;
+    for (uint32_t na = a.ks; na <= sms / 3; na += a.ks) {
+      const uint32_t ncl = (sms - na) / a.ks, per = (nt + ncl - 1) / ncl;
+      const double tw = per * a.pairs * cw;
+      uint32_t sl = 1;
+      while (sl < (uint32_t)kMaxSlices && a.a_nt * sl < na && a.a_np >= 32 * sl) sl *= 2;
+      const uint32_t sp = (a.a_np + sl - 1) / sl, rounds = (a.a_nt * sl + na - 1) / na;
+      const double ta = 2500.0 + rounds * (300.0 + ((sp + kWarps - 1) / kWarps) * kWarps * ca);
+      const double t = tw > ta ? tw : ta;
+      if (t < 0.98 * best || (t <= 1.02 * best && ta < 0.98 * best_a)) { best = t; best_a = ta; a.n_a = na; a.a_slices = sl; a.a_slice_pairs = sp; }
+    }
+    if (a.n_a == 0) return false;
+    a.sub_pairs = h->n_sub > 1 ? (uint32_t)h->r_pad / 128 : 0u;
+  }
+  uint32_t ncl = (sms - a.n_a) / a.ks;
+  if (ncl > nt) ncl = nt;
+  if ((nt + ncl - 1) / ncl > (uint32_t)kMaxTiles) ncl = (nt + kMaxTiles - 1) / kMaxTiles;
+  a.tiles = make_share(nt, ncl);
+  auto inverse = [](uint32_t n) { return (uint32_t)((0x100000000ull + n - 1) / n); };      // 0 for n == 1
+  for (int r = 0; r < 2; ++r) {
+    const uint32_t P = r ? a.w_np - a.pairs : a.pairs;
+    if (P == 0) continue;
+    a.part[r].pairs = P; a.part[r].inv_pairs = inverse(P);
+    for (int k = 0; k < 2; ++k) a.part[r].inv_blobs[k] = inverse((a.tiles.per + k) * P);
+  }
+  pl.grid = (int)(a.n_a + ncl * a.ks);
+  if (pl.grid >= (1 << kLaunchShift)) return false;
+  const uint32_t nT = a.tiles.per + (a.tiles.rem ? 1 : 0), nF = (nT + a.ks - 1) / a.ks;
+  const bool codes = h->w.fmt == FMT_Q4 || h->w.fmt == FMT_Q3;
+  const uint32_t per_pair = int8 ? (uint32_t)kPlaneBytes : (uint32_t)m * 256 + (codes ? 3 * kMaxTok * 4 : 0);
+  a.chunk = a.pairs;
+  if (a.chunk * per_pair > (uint32_t)kXBytes) {
+    const uint32_t parts = (a.chunk * per_pair + kXBytes - 1) / kXBytes;
+    a.chunk = (a.pairs + parts - 1) / parts;
+  }
+  const uint32_t t_pairs = (uint32_t)h->t_cols / 128;
+  a.t_chunk = 32u / (uint32_t)m < t_pairs ? 32u / (uint32_t)m : t_pairs;
+  // Shared memory: activations | barriers | rings (later blobs of B) | sums of the warps' runs | the partner's sums, and, after
+  // the backbone's products (over the activations where they fit and no later chunk needs those): sums of the chunks before |
+  // t . B | t.
+  auto up = [](uint32_t v) { return (v + 127u) & ~127u; };
+  const uint32_t OT = 64u * m;                     // bytes of a row tile's sums
+  const uint32_t x_b = up(a.chunk * per_pair + (int8 ? 0u : 64u * m));
+  while ((2u << a.b_log) * nF <= (uint32_t)kWarps && (1u << a.b_log) < a.t_chunk && (1u << a.b_log) < a.b_np) ++a.b_log;
+  const uint32_t sum_b = a.chunk < a.pairs ? up(nT * OT) : 0u, bseg_b = ab ? up((nF > (uint32_t)kWarps ? nF : (uint32_t)kWarps) * OT) : 0u;
+  const uint32_t t_b = ab ? up(2u * m * (a.t_chunk * 256 + 64)) : 0u, late_b = sum_b + bseg_b + t_b;
+  const uint32_t keep_b = up((kWarps + nT) * OT) + (a.ks == 2 ? up(nF * OT) : 0u) + (a.chunk < a.pairs || late_b > x_b ? late_b : 0u);
+  const uint32_t bar_b = kWarps * kMaxSlots * 8;
+  // The ring takes what is left of half an SM, in two to four slots of one, two or four blobs; at least two
+  // slots even if the CTA then needs an SM of its own.
+  const uint32_t budget = int8 ? kHalfSmem : kMaxSmem;
+  const uint32_t blob = (uint32_t)h->w.blob, fixed = x_b + bar_b + keep_b;
+  const uint32_t room = fixed < budget ? (budget - fixed) / kWarps / blob : 0u;   // blobs per warp
+  if (room >= 4) { a.slot_blobs = room >= 8 ? 4 : 2; a.slots = room / a.slot_blobs < kMaxSlots ? room / a.slot_blobs : kMaxSlots; }
+  else { a.slot_blobs = 1; a.slots = room < 2 ? 2 : room; }
+  a.off_bar = x_b;
+  a.off_ring = a.off_bar + bar_b;
+  a.ring_pitch = a.slots * a.slot_blobs * blob;
+  if (ab && a.ring_pitch < (uint32_t)h->b.blob) a.ring_pitch = h->b.blob;      // (a blob of B at a time)
+  uint32_t off = a.off_ring + up(kWarps * a.ring_pitch);
+  a.off_seg = off; off += up((kWarps + nT) * OT);
+  a.off_inbox = off; off += a.ks == 2 ? up(nF * OT) : 0u;
+  if (a.chunk < a.pairs || late_b > x_b) { a.off_sum = off; off += late_b; }
+  else a.off_sum = 0;                              // over the activations
+  a.off_bseg = a.off_sum + sum_b;
+  a.off_t = a.off_bseg + bseg_b;
+  pl.smem = (int)off;
+  if (pl.smem < (int)(2 * kWarps * 16 * kMaxTok * 4)) pl.smem = (int)(2 * kWarps * 16 * kMaxTok * 4);      // the A CTAs' sums
+  return pl.smem <= kMaxSmem;
 }
 
 }  // namespace
 
-// One thread waits, bounded by the handle's limit, for a count that nobody raises, after leaving the kind of debris a
-// kernel that gives up leaves behind (a partial sum, a partial t, a ticket).  See eora_linear_selftest_wait_timeout.
-__global__ void k_wait_selftest(uint32_t* counters, float* y_ws, float* d_t, int* dev_status, unsigned long long limit_ns) {
+// One thread waits, bounded by the handle's limit, for a word that nobody sends, after leaving a stale one where t's would
+// be.  See eora_linear_selftest_wait_timeout.
+__global__ void k_wait_selftest(unsigned long long* t_part, const unsigned long long* launches, int* dev_status, unsigned long long limit_ns) {
   if (threadIdx.x == 0) {
-    y_ws[0] += 1.f;
-    d_t[0] += 1.f;
-    counters[CNT_TICKET0] += 1u;
-    dec::counter_wait(counters + CNT_A_DONE, 0xffffffffu, dev_status, limit_ns);
+    t_part[0] = 0x3f800000ull;                     // 1.0f, sent by launch 0 (the first is number 1)
+    const uint32_t want = (uint32_t)(ld_volatile_u64(launches) >> kLaunchShift) + 1u;
+    const unsigned long long t0 = dec::globaltimer_ns();
+    while ((uint32_t)(ld_volatile_u64(t_part) >> 32) != want) {
+      if (dec::globaltimer_ns() - t0 > limit_ns) { atomicExch(dev_status, EORA_ERR_DEVICE_TIMEOUT); break; }
+      __nanosleep(32);
+    }
   }
 }
 
 cudaError_t launch_wait_selftest(const Handle* h, cudaStream_t st) {
-  k_wait_selftest<<<1, 32, 0, st>>>(h->counters, h->y_ws, h->d_t, h->dev_status, h->wait_limit_ns);
+  k_wait_selftest<<<1, 32, 0, st>>>(h->t_part, h->launches, h->dev_status, h->wait_limit_ns);
   return cudaGetLastError();
 }
+
+size_t decode_part_bytes(int t_cols) { return (size_t)kMaxSlices * kMaxTok * t_cols * 8; }
 
 bool decode_supported(const Handle* h, int m) {
   if (m < 1 || m > 64) return false;
   if (h->sm_count < 2) return false;
   if (h->w.fmt != FMT_Q4 && h->w.fmt != FMT_Q3 && h->w.fmt != FMT_SP24 && h->w.fmt != FMT_SQ4) return false;
-  if (h->w.blob > kSlotBytes) return false;
-  if (h->cfg.rank > 0 && (h->a.blob > kSlotBytes || h->b.blob > kSlotBytes)) return false;
-  return true;
+  Plan pl;
+  return make_plan(h, m < kMaxTok ? m : kMaxTok, pl);
 }
 
-int decode_launch_count(const Handle*, int m) { return (m + 7) / 8; }
+int decode_launch_count(const Handle*, int m) { return (m + kMaxTok - 1) / kMaxTok; }
 
 int decode_grid(const Handle* h, int m) {
-  const bool i8 = m == 1 && (h->w.fmt == FMT_Q4 || h->w.fmt == FMT_Q3);
-  (void)i8;
-  return h->sm_count * kCtasPerSm;
+  Plan pl;
+  return make_plan(h, m < kMaxTok ? m : kMaxTok, pl) ? pl.grid : 0;
 }
 
 cudaError_t launch_decode_forward(const Handle* h, const void* x, int m, void* const* ys, cudaStream_t st,
                                   const int32_t* adapter_ids) {
-  const bool ab = h->cfg.rank > 0;
-  DecodeArgs a = {};
-  a.w_q = h->w.q; a.w_nt = h->w.nt; a.w_sz2 = h->w.sz2; a.w_per_copy = blobs_per_copy(h->w);
-  const uint32_t w_blobs = (uint32_t)h->w.np * h->w.nt;
-  uint32_t b_blobs = 0;
-  if (ab) {
-    a.a_q = h->a.q; a.a_nt = h->a.nt; a.a_sz2 = h->a.sz2; a.a_per_copy = blobs_per_copy(h->a);
-    a.b_q = h->b.q; a.b_sz2 = h->b.sz2; a.b_per_copy = blobs_per_copy(h->b);
-    a.a_blobs = (uint32_t)h->a.np * h->a.nt;
-    b_blobs = (uint32_t)h->b.np * h->b.nt;
-  } else {
-    a.a_nt = 1; a.a_per_copy = 1; a.b_per_copy = 1;
-  }
-  const int grid = decode_grid(h, m);
-  const uint32_t nw = (uint32_t)grid * kWarps;
-  if (ab) {
-    // with one token the backbone blobs go through the integer inner product, which is cheaper
-    const bool i8 = h->w.fmt == FMT_Q4 || h->w.fmt == FMT_Q3;       // (one to eight tokens: this function's passes)
-    // at most a sixth of the warps hold A, a sixth B (measured on the whole block: a third of each 1.4 % slower, an
-    // eighth 2 % slower)
-    uint32_t n1 = a.a_blobs < nw / 6 ? a.a_blobs : nw / 6;
-    uint32_t n3 = b_blobs < nw / 6 ? b_blobs : nw / 6;
-    if (n1 < 1) n1 = 1;
-    if (n3 < 1) n3 = 1;
-    // the A owners sit in the first half of the CTAs, the B owners in the second (see the kernel)
-    if (n1 > (uint32_t)(grid / 2) * kWarps) n1 = (uint32_t)(grid / 2) * kWarps;
-    if (n3 > (uint32_t)(grid - grid / 2) * kWarps) n3 = (uint32_t)(grid - grid / 2) * kWarps;
-    const uint32_t n2 = nw - n1 - n3;
-    // Deal the blobs so that every warp gets the same estimated time.  Costs are in units of one backbone
-    // blob on the tensor-core path.  Besides its blobs of A or B a warp of the first or third group has a
-    // fixed extra cost: the A owners fetch a second set of activations, the B owners read t back and end
-    // with their own round of tickets, which is latency that a warp cannot hide from itself.
-    const double cw1 = blob_cost(h->w.fmt, false) * (i8 ? 0.75 : 1.0);
-    const double fixed_a = i8 ? 4.0 : 2.0, fixed_b = 9.0;
-    const double e1 = fixed_a + (double)a.a_blobs / n1 * blob_cost(h->a.fmt, false);
-    const double e3 = fixed_b + (double)b_blobs / n3 * blob_cost(h->b.fmt, true);
-    const double T = (w_blobs * cw1 + n1 * e1 + n3 * e3) / nw;      // finishing time of every warp
-    double W1 = T > e1 ? n1 * (T - e1) / cw1 : 0.0, W3 = T > e3 ? n3 * (T - e3) / cw1 : 0.0;
-    if (W1 + W3 > w_blobs) { const double f = w_blobs / (W1 + W3); W1 *= f; W3 *= f; }
-    const uint32_t w1 = (uint32_t)W1, w3 = (uint32_t)W3, w2 = w_blobs - w1 - w3;
-    a.n1 = n1; a.n12 = n1 + n2;
-    a.sh_a = make_share(a.a_blobs, n1);
-    a.sh_b = make_share(b_blobs, n3);
-    a.sh_w[0] = make_share(w1, n1); a.sh_w[1] = make_share(w2, n2); a.sh_w[2] = make_share(w3, n3);
-    a.w_base[0] = 0; a.w_base[1] = w1; a.w_base[2] = w1 + w2;
-  } else {
-    a.n1 = 0; a.n12 = nw;
-    a.sh_a = make_share(0, 0);
-    a.sh_b = make_share(0, 0);
-    a.sh_w[0] = make_share(0, 0); a.sh_w[1] = make_share(w_blobs, nw); a.sh_w[2] = make_share(0, 0);
-    a.w_base[0] = 0; a.w_base[1] = 0; a.w_base[2] = w_blobs;
-  }
-  a.tile_target = (uint32_t)h->w.np + (ab ? (uint32_t)h->b.np : 0u);
-  a.d_t = h->d_t; a.y_ws = h->y_ws; a.counters = h->counters; a.dev_status = h->dev_status;
-  a.d_in = h->cfg.d_in; a.r_pad = h->t_cols; a.n_pad = h->w.n_rows;
-  a.n_sub = h->n_sub;
-  a.b_np = ab ? (uint32_t)h->b.np : 0u;
-  for (int i = 0; i <= h->n_sub; ++i) a.sub_tile0[i] = (uint32_t)h->sub_tile0[i];
-  for (int i = h->n_sub + 1; i < 5; ++i) a.sub_tile0[i] = (uint32_t)h->w.nt;
-  for (int i = 0; i < 4; ++i) a.sub_dout[i] = i < h->n_sub ? h->sub_dout[i] : 0;
-  a.x_dtype = h->cfg.x_dtype; a.y_dtype = h->cfg.y_dtype;
-  a.trace = reinterpret_cast<unsigned long long*>(h->trace);
-  a.wait_ns = h->wait_limit_ns;
-
+  Plan pl;
+  DecodeArgs& a = pl.a;
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(grid);
-  cfg.blockDim = dim3(kThreads);
-  cfg.dynamicSmemBytes = kSmemBytes;
   cfg.stream = st;
-  cudaLaunchAttribute attr[1];
+  cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
+  attr[1].id = cudaLaunchAttributeClusterDimension;
+  attr[1].val.clusterDim.x = 1; attr[1].val.clusterDim.y = 1; attr[1].val.clusterDim.z = 1;
   cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  const int abf = ab ? h->a.fmt : FMT_NONE;
+  cfg.numAttrs = 2;
   const size_t ybytes = h->cfg.y_dtype == EORA_Y_F32 ? 4 : 2;
-  for (int m0 = 0; m0 < m; m0 += 8) {             // eight tokens per pass (the n8 side of the mma)
-    a.m = m - m0 < 8 ? m - m0 : 8;
+  int planned = 0;
+  for (int m0 = 0; m0 < m; m0 += kMaxTok) {        // eight tokens per pass (the n8 side of the mma)
+    const int mp = m - m0 < kMaxTok ? m - m0 : kMaxTok;
+    if (mp != planned) {
+      if (!make_plan(h, mp, pl)) return cudaErrorInvalidValue;
+      planned = mp;
+      a.n_sub = h->n_sub;
+      for (int i = 0; i < 5; ++i) a.sub_tile0[i] = (uint32_t)(i <= h->n_sub ? h->sub_tile0[i] : h->w.nt);
+      for (int i = 0; i < h->n_sub; ++i) a.sub_dout[i] = h->sub_dout[i];
+      a.t_part = h->t_part; a.launches = h->launches; a.dev_status = h->dev_status;
+      a.d_in = h->cfg.d_in; a.t_cols = h->t_cols;
+      a.x_dtype = h->cfg.x_dtype; a.y_dtype = h->cfg.y_dtype;
+      a.trace = reinterpret_cast<unsigned long long*>(h->trace);
+      a.wait_ns = h->wait_limit_ns;
+      cfg.gridDim = dim3(pl.grid);
+      cfg.blockDim = dim3(pl.warps * 32);
+      cfg.dynamicSmemBytes = pl.smem;
+      attr[1].val.clusterDim.x = a.ks;
+    }
     a.x = reinterpret_cast<const uint8_t*>(x) + (size_t)m0 * h->cfg.d_in * 2;
     for (int i = 0; i < h->n_sub; ++i) a.ys[i] = reinterpret_cast<uint8_t*>(ys[i]) + (size_t)m0 * h->sub_dout[i] * ybytes;
-    a.adp_pairs = 0;
     if (h->multi) {
       a.adp_pairs = (uint32_t)h->r_pad / 128;
-      for (int i = 0; i < 8; ++i) {
+      for (int i = 0; i < kMaxTok; ++i) {
         const int id = (adapter_ids && m0 + i < m) ? adapter_ids[m0 + i] : -1;
         a.adp[i] = (id >= 0 && id < h->n_adapters) ? id : -1;
       }
     }
-    cudaError_t e = h->w.fmt == FMT_Q4 ? launch_ab<FMT_Q4>(cfg, a, abf, h->device)
-                  : h->w.fmt == FMT_Q3 ? launch_ab<FMT_Q3>(cfg, a, abf, h->device)
-                  : h->w.fmt == FMT_SQ4 ? launch_ab<FMT_SQ4>(cfg, a, abf, h->device) : launch_ab<FMT_SP24>(cfg, a, abf, h->device);
+    cudaError_t e = launch_any(cfg, a, h->w.fmt, h->w.sz2 != 0, h->device);
     if (e != cudaSuccess) return e;
   }
   return cudaSuccess;

@@ -28,6 +28,23 @@ __device__ __forceinline__ bool mbar_try_wait_susp(uint64_t* bar, uint32_t parit
                : "=r"(ok) : "r"(smem_u32(bar)), "r"(parity), "r"(ns) : "memory");
   return ok != 0;
 }
+// The same on 32-bit shared addresses.
+__device__ __forceinline__ void mbar_init_a(uint32_t bar, uint32_t count) {
+  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(count) : "memory");
+}
+__device__ __forceinline__ void mbar_expect_tx_a(uint32_t bar, uint32_t bytes) {
+  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
+}
+__device__ __forceinline__ bool mbar_try_wait_a(uint32_t bar, uint32_t parity) {
+  uint32_t ok;
+  asm volatile("{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
+               : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
+  return ok != 0;
+}
+__device__ __forceinline__ void bulk_g2s_a(uint32_t dst, const void* src, uint32_t bytes, uint32_t bar) {
+  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
+               ::"r"(dst), "l"(src), "r"(bytes), "r"(bar) : "memory");
+}
 __device__ __forceinline__ unsigned long long globaltimer_ns() {
   unsigned long long t;
   asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t));
@@ -42,6 +59,18 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, int* d
 #pragma unroll 1
     for (int it = 0; it < 64; ++it)
       if (mbar_try_wait_susp(bar, parity, 20000u)) return true;
+    if (globaltimer_ns() - t0 > kWaitLimitNs) break;
+  }
+  atomicExch(dev_status, EORA_ERR_DEVICE_TIMEOUT);
+  return false;
+}
+// The slow path of a wait that every lane of a warp does for itself (the caller brings the lanes together afterwards).
+__device__ __forceinline__ bool mbar_wait_lane(uint32_t bar, uint32_t parity, int* dev_status) {
+  const unsigned long long t0 = globaltimer_ns();
+  for (;;) {
+#pragma unroll 1
+    for (int it = 0; it < 64; ++it)
+      if (mbar_try_wait_a(bar, parity)) return true;
     if (globaltimer_ns() - t0 > kWaitLimitNs) break;
   }
   atomicExch(dev_status, EORA_ERR_DEVICE_TIMEOUT);
@@ -182,8 +211,6 @@ __device__ __forceinline__ uint32_t and_or(uint32_t a, uint32_t mask, uint32_t c
 
 template <int FMT> constexpr bool is_quant() { return fmt_quantised(FMT); }
 
-// Build the A-operand registers of the four mma of one tile from its blob in shared memory.
-// a[i][*]: mma i = 2*blk + sub; entries are fp16x2.
 __device__ __forceinline__ uint32_t prmt(uint32_t a, uint32_t b, uint32_t sel) {
   uint32_t d;
   asm("prmt.b32 %0, %1, %2, %3;" : "=r"(d) : "r"(a), "r"(b), "r"(sel));
@@ -221,12 +248,135 @@ __device__ __forceinline__ uint32_t quad_pair(uint32_t quad, int which) {
   return prmt(quad, 0x64646464u, which ? 0x4342u : 0x4140u);
 }
 
-// `aux`: shared-memory address (32-bit, shared window) of the 2:4 expansion table; unused by other formats.
-template <int FMT>
-__device__ __forceinline__ void tile_frags(const uint8_t* blob, int lane, const ZC& zc, uint32_t (&a)[4][4], uint32_t aux = 0) {
+// ------------------------------------------------------------------------------------------ blobs in registers
+// One lane's payload of a tile and of a blob (two tiles and their scale entries), as loaded from global memory.  The
+// weights are read once per launch: no L1 line is allocated for them.
+__device__ __forceinline__ uint4 ldw_u4(const uint8_t* p) {
+  uint4 v;
+  asm volatile("ld.global.nc.L1::no_allocate.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p));
+  return v;
+}
+__device__ __forceinline__ uint2 ldw_u2(const uint8_t* p) {
+  uint2 v;
+  asm volatile("ld.global.nc.L1::no_allocate.v2.u32 {%0,%1}, [%2];" : "=r"(v.x), "=r"(v.y) : "l"(p));
+  return v;
+}
+__device__ __forceinline__ uint32_t ldw_u1(const uint8_t* p) {
+  uint32_t v;
+  asm volatile("ld.global.nc.L1::no_allocate.u32 %0, [%1];" : "=r"(v) : "l"(p));
+  return v;
+}
+__device__ __forceinline__ uint32_t ldw_u16(const uint8_t* p) {
+  uint16_t v;
+  asm volatile("ld.global.nc.L1::no_allocate.u16 %0, [%1];" : "=h"(v) : "l"(p));
+  return v;
+}
+
+template <int FMT> struct RawTile;
+template <> struct RawTile<FMT_Q4> { uint4 v; };
+template <> struct RawTile<FMT_Q3> { uint2 v; uint32_t w2; };
+template <> struct RawTile<FMT_Q8> { uint4 v[2]; };
+template <> struct RawTile<FMT_F16> { uint4 v[4]; };
+template <> struct RawTile<FMT_SP24> { uint4 v[2]; uint32_t meta; };
+template <> struct RawTile<FMT_SQ4> { uint2 v; uint32_t meta; };
+
+template <int FMT> __device__ __forceinline__ void load_tile(RawTile<FMT>& r, const uint8_t* tile, int lane) {
   if constexpr (FMT == FMT_Q4) {
-    const uint4 v = *reinterpret_cast<const uint4*>(blob + lane * 16);
-    const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+    r.v = ldw_u4(tile + lane * 16);
+  } else if constexpr (FMT == FMT_Q3) {
+    r.v = ldw_u2(tile + lane * 8);
+    r.w2 = ldw_u1(tile + 256 + lane * 4);
+  } else if constexpr (FMT == FMT_SQ4) {
+    r.v = ldw_u2(tile + lane * 8);
+    r.meta = ldw_u1(tile + 256 + lane * 4);
+  } else if constexpr (FMT == FMT_F16) {
+#pragma unroll
+    for (int i = 0; i < 4; ++i) r.v[i] = ldw_u4(tile + i * 512 + lane * 16);
+  } else {                                          // Q8, SP24
+    r.v[0] = ldw_u4(tile + lane * 16);
+    r.v[1] = ldw_u4(tile + 512 + lane * 16);
+    if constexpr (FMT == FMT_SP24) r.meta = ldw_u1(tile + 1024 + lane * 4);
+  }
+}
+
+// s, z: scales (s[row g] | s[row g + 8] << 16) and zero-points (z | z << 8) of the pair, or of each tile (SZ2: groups that are
+// not a multiple of 128).
+template <int FMT, bool SZ2> struct RawBlob {
+  RawTile<FMT> t[2];
+  uint32_t s[SZ2 ? 2 : 1], z[SZ2 ? 2 : 1];
+};
+template <int FMT, bool SZ2> __device__ __forceinline__ void load_blob(RawBlob<FMT, SZ2>& r, const uint8_t* blob, int lane) {
+  constexpr int tb = tile_bytes(FMT);
+  load_tile<FMT>(r.t[0], blob, lane);
+  load_tile<FMT>(r.t[1], blob + tb, lane);
+  if constexpr (fmt_quantised(FMT)) {
+    const int g = lane >> 2;
+#pragma unroll
+    for (int i = 0; i < (SZ2 ? 2 : 1); ++i) {
+      r.s[i] = ldw_u1(blob + 2 * tb + i * kSzEntryBytes + 4 * g);
+      r.z[i] = ldw_u16(blob + 2 * tb + i * kSzEntryBytes + 32 + 2 * g);
+    }
+  }
+}
+
+// The same from a blob in shared memory (32-bit shared addresses).
+__device__ __forceinline__ uint4 lds_u4(uint32_t a) {
+  uint4 v;
+  asm volatile("ld.shared.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(a));
+  return v;
+}
+__device__ __forceinline__ uint2 lds_u2(uint32_t a) {
+  uint2 v;
+  asm volatile("ld.shared.v2.u32 {%0,%1}, [%2];" : "=r"(v.x), "=r"(v.y) : "r"(a));
+  return v;
+}
+__device__ __forceinline__ uint32_t lds_u1(uint32_t a) {
+  uint32_t v;
+  asm volatile("ld.shared.u32 %0, [%1];" : "=r"(v) : "r"(a));
+  return v;
+}
+__device__ __forceinline__ uint32_t lds_u16(uint32_t a) {
+  uint16_t v;
+  asm volatile("ld.shared.u16 %0, [%1];" : "=h"(v) : "r"(a));
+  return v;
+}
+__device__ __forceinline__ void sts_u1(uint32_t a, uint32_t v) { asm volatile("st.shared.u32 [%0], %1;" ::"r"(a), "r"(v) : "memory"); }
+template <int FMT> __device__ __forceinline__ void load_tile_s(RawTile<FMT>& r, uint32_t tile, int lane) {
+  if constexpr (FMT == FMT_Q4) {
+    r.v = lds_u4(tile + lane * 16);
+  } else if constexpr (FMT == FMT_Q3 || FMT == FMT_SQ4) {
+    r.v = lds_u2(tile + lane * 8);
+    const uint32_t w = lds_u1(tile + 256 + lane * 4);
+    if constexpr (FMT == FMT_Q3) r.w2 = w; else r.meta = w;
+  } else if constexpr (FMT == FMT_F16) {
+#pragma unroll
+    for (int i = 0; i < 4; ++i) r.v[i] = lds_u4(tile + i * 512 + lane * 16);
+  } else {                                          // Q8, SP24
+    r.v[0] = lds_u4(tile + lane * 16);
+    r.v[1] = lds_u4(tile + 512 + lane * 16);
+    if constexpr (FMT == FMT_SP24) r.meta = lds_u1(tile + 1024 + lane * 4);
+  }
+}
+template <int FMT, bool SZ2> __device__ __forceinline__ void load_blob_s(RawBlob<FMT, SZ2>& r, uint32_t blob, int lane) {
+  constexpr int tb = tile_bytes(FMT);
+  load_tile_s<FMT>(r.t[0], blob, lane);
+  load_tile_s<FMT>(r.t[1], blob + tb, lane);
+  if constexpr (fmt_quantised(FMT)) {
+    const int g = lane >> 2;
+#pragma unroll
+    for (int i = 0; i < (SZ2 ? 2 : 1); ++i) {
+      r.s[i] = lds_u1(blob + 2 * tb + i * kSzEntryBytes + 4 * g);
+      r.z[i] = lds_u16(blob + 2 * tb + i * kSzEntryBytes + 32 + 2 * g);
+    }
+  }
+}
+
+// The wide operand of the tile's four mma.m16n8k16 as exact fp16 values: a[2 * blk + sub][*].  `aux`: shared-memory address of the
+// 2:4 expansion table; unused by other formats.
+template <int FMT>
+__device__ __forceinline__ void tile_frags(const RawTile<FMT>& r, const ZC& zc, uint32_t (&a)[4][4], uint32_t aux) {
+  if constexpr (FMT == FMT_Q4) {
+    const uint32_t w[4] = {r.v.x, r.v.y, r.v.z, r.v.w};
 #pragma unroll
     for (int part = 0; part < 4; ++part) {
       const int hf = part & 1, blk = part >> 1;
@@ -239,10 +389,8 @@ __device__ __forceinline__ void tile_frags(const uint8_t* blob, int lane, const 
       a[blk * 2 + 1][hf + 2] = h2fma(h3, 0x2C002C00u, zc.c[hf][1]);
     }
   } else if constexpr (FMT == FMT_Q3) {
-    const uint2 v01 = *reinterpret_cast<const uint2*>(blob + lane * 8);
-    const uint32_t v2 = *reinterpret_cast<const uint32_t*>(blob + 256 + lane * 4);
     uint32_t q[4][2];
-    q3_quads(v01.x, v01.y, v2, q);
+    q3_quads(r.v.x, r.v.y, r.w2, q);
 #pragma unroll
     for (int part = 0; part < 4; ++part) {
       const int hf = part & 1, blk = part >> 1;
@@ -255,7 +403,7 @@ __device__ __forceinline__ void tile_frags(const uint8_t* blob, int lane, const 
   } else if constexpr (FMT == FMT_Q8) {
 #pragma unroll
     for (int pl = 0; pl < 2; ++pl) {
-      const uint4 u = *reinterpret_cast<const uint4*>(blob + pl * 512 + lane * 16);
+      const uint4 u = r.v[pl];
 #pragma unroll
       for (int hf = 0; hf < 2; ++hf) {
         const uint32_t w0 = hf ? u.z : u.x, w1 = hf ? u.w : u.y;
@@ -269,45 +417,31 @@ __device__ __forceinline__ void tile_frags(const uint8_t* blob, int lane, const 
 #pragma unroll
     for (int part = 0; part < 4; ++part) {
       const int hf = part & 1, blk = part >> 1;
-      const uint4 u = *reinterpret_cast<const uint4*>(blob + part * 512 + lane * 16);
-      a[blk * 2 + 0][hf] = u.x;
-      a[blk * 2 + 0][hf + 2] = u.y;
-      a[blk * 2 + 1][hf] = u.z;
-      a[blk * 2 + 1][hf + 2] = u.w;
+      a[blk * 2 + 0][hf] = r.v[part].x;
+      a[blk * 2 + 0][hf + 2] = r.v[part].y;
+      a[blk * 2 + 1][hf] = r.v[part].z;
+      a[blk * 2 + 1][hf + 2] = r.v[part].w;
     }
-  } else if constexpr (FMT == FMT_SP24) {
-    const uint32_t meta = *reinterpret_cast<const uint32_t*>(blob + 1024 + lane * 4);
+  } else {
+    // 2:4 formats: a quad's two kept values (SQ4: two codes made exact fp16 values first) are spread over its four positions
+    // with two byte permutes whose selectors come from the table.
 #pragma unroll
     for (int blk = 0; blk < 2; ++blk) {
-      const uint4 u = *reinterpret_cast<const uint4*>(blob + blk * 512 + lane * 16);
-      const uint32_t vv[2][2] = {{u.x, u.y}, {u.z, u.w}};       // [hf][quad]: the quad's two kept values
 #pragma unroll
       for (int hf = 0; hf < 2; ++hf) {
 #pragma unroll
         for (int quad = 0; quad < 2; ++quad) {
-          const uint32_t nib = (meta >> (8 * (blk * 2 + hf) + 4 * quad)) & 15u;
+          uint32_t kept;
+          if constexpr (FMT == FMT_SP24) {
+            const uint4 u = r.v[blk];
+            kept = hf ? (quad ? u.w : u.z) : (quad ? u.y : u.x);
+          } else {
+            kept = h2sub(and_or((blk ? r.v.y : r.v.x) >> (8 * hf + 4 * quad), 0x000f000fu, kMagic), zc.c[hf][0]);
+          }
+          const int sh = 8 * (blk * 2 + hf) + 4 * quad - 2;           // nibble * 4 = byte offset into the table
+          const uint32_t offb = (sh < 0 ? (r.meta << 2) : (r.meta >> (sh < 0 ? 0 : sh))) & 0x3Cu;
           uint32_t sel;
-          asm volatile("ld.shared.u32 %0, [%1];" : "=r"(sel) : "r"(aux + nib * 4));
-          a[blk * 2 + quad][hf] = prmt(vv[hf][quad], 0u, sel);
-          a[blk * 2 + quad][hf + 2] = prmt(vv[hf][quad], 0u, sel >> 16);
-        }
-      }
-    }
-  } else if constexpr (FMT == FMT_SQ4) {
-    // 2:4 pattern with 4-bit kept values: the quad's two codes -> exact fp16 (q - z), then spread like SP24
-    const uint2 v = *reinterpret_cast<const uint2*>(blob + lane * 8);
-    const uint32_t meta = *reinterpret_cast<const uint32_t*>(blob + 256 + lane * 4);
-#pragma unroll
-    for (int blk = 0; blk < 2; ++blk) {
-      const uint32_t w = blk ? v.y : v.x;
-#pragma unroll
-      for (int hf = 0; hf < 2; ++hf) {
-#pragma unroll
-        for (int quad = 0; quad < 2; ++quad) {
-          const uint32_t kept = h2sub(and_or(w >> (8 * hf + 4 * quad), 0x000f000fu, kMagic), zc.c[hf][0]);
-          const uint32_t nib = (meta >> (8 * (blk * 2 + hf) + 4 * quad)) & 15u;
-          uint32_t sel;
-          asm volatile("ld.shared.u32 %0, [%1];" : "=r"(sel) : "r"(aux + nib * 4));
+          asm volatile("ld.shared.u32 %0, [%1];" : "=r"(sel) : "r"(aux + offb));
           a[blk * 2 + quad][hf] = prmt(kept, 0u, sel);
           a[blk * 2 + quad][hf + 2] = prmt(kept, 0u, sel >> 16);
         }
@@ -316,302 +450,60 @@ __device__ __forceinline__ void tile_frags(const uint8_t* blob, int lane, const 
   }
 }
 
-
-// One blob: 16 rows x 128 reduction elements times the activation fragments -> tot (this lane's four
-// entries of the 16 x 8 result: rows g / g + 8, tokens 2t / 2t + 1).
-template <int FMT, bool HILO>
-__device__ __forceinline__ void blob_product(const uint8_t* blob, int lane, uint32_t sz2, const uint32_t (&xr)[16],
-                                             const uint32_t (&xl)[16], float (&tot)[4], uint32_t aux = 0) {
-  constexpr int tb = tile_bytes(FMT);
-  constexpr bool quant = fmt_quantised(FMT);
-  const int g = lane >> 2;
-  // Two independent accumulator chains per tile: the four mma of a tile would otherwise wait for one
-  // another (an mma takes ~30 cycles to deliver its accumulator), and with four warps per scheduler that
-  // latency is not hidden.
-  float acc[2][4];
+// 3/4-bit codes as the fp16 bit patterns they are in their words (subnormals q * 2^-24): a[2 * blk] with the codes at the low end of
+// their half-words, a[2 * blk + 1] with those four (three) bits up, i.e. 16 (8) times as large.
+template <int FMT>
+__device__ __forceinline__ void code_frags(const RawTile<FMT>& r, uint32_t (&a)[4][4]) {
+  if constexpr (FMT == FMT_Q4) {
+    const uint32_t w[4] = {r.v.x, r.v.y, r.v.z, r.v.w};
 #pragma unroll
-  for (int k = 0; k < 4; ++k) { acc[0][k] = 0.f; acc[1][k] = 0.f; tot[k] = 0.f; }
-  ZC zc;
-  float s_a = 0.f, s_b = 0.f;
-#pragma unroll
-  for (int c = 0; c < 2; ++c) {
-    if constexpr (quant) {
-      if (c == 0 || sz2) {
-        const uint8_t* sz = blob + 2 * tb + c * kSzEntryBytes;      // c != 0 only with two entries
-        const uint32_t s2 = reinterpret_cast<const uint32_t*>(sz)[g];
-        const uint32_t z2 = reinterpret_cast<const uint16_t*>(sz + 32)[g];
-        make_zc<FMT>(zc, z2);
-        s_a = __half2float(__ushort_as_half((unsigned short)(s2 & 0xffffu)));
-        s_b = __half2float(__ushort_as_half((unsigned short)(s2 >> 16)));
-      }
+    for (int part = 0; part < 4; ++part) {
+      const int hf = part & 1, blk = part >> 1;
+      const uint32_t hi = w[part] >> 8;
+      a[blk * 2 + 0][hf] = w[part] & 0x000f000fu; a[blk * 2 + 0][hf + 2] = hi & 0x000f000fu;       // elements (0, 1), (4, 5)
+      a[blk * 2 + 1][hf] = w[part] & 0x00f000f0u; a[blk * 2 + 1][hf + 2] = hi & 0x00f000f0u;       // elements (2, 3), (6, 7)
     }
-    uint32_t a[4][4];
-    tile_frags<FMT>(blob + c * tb, lane, zc, a, aux);
+  } else {
+    const uint32_t w[3] = {r.v.x, r.v.y, r.w2};
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      mma16816(acc[i & 1], a[i], xr[8 * c + 2 * i], xr[8 * c + 2 * i + 1]);
-      if constexpr (HILO) mma16816(acc[i & 1], a[i], xl[8 * c + 2 * i], xl[8 * c + 2 * i + 1]);
+    for (int part = 0; part < 3; ++part) {
+      const int hf = part & 1, blk = part >> 1;
+      const uint32_t hi = w[part] >> 8;
+      a[blk * 2 + 0][hf] = w[part] & 0x00070007u; a[blk * 2 + 0][hf + 2] = hi & 0x00070007u;       // elements (0, 2), (1, 3)
+      a[blk * 2 + 1][hf] = w[part] & 0x00380038u; a[blk * 2 + 1][hf + 2] = hi & 0x00380038u;       // elements (4, 6), (5, 7)
     }
-    if constexpr (quant) {
-      if (c == 1 || sz2) {
-        tot[0] = fmaf(acc[0][0] + acc[1][0], s_a, tot[0]); tot[1] = fmaf(acc[0][1] + acc[1][1], s_a, tot[1]);
-        tot[2] = fmaf(acc[0][2] + acc[1][2], s_b, tot[2]); tot[3] = fmaf(acc[0][3] + acc[1][3], s_b, tot[3]);
-#pragma unroll
-        for (int k = 0; k < 4; ++k) { acc[0][k] = 0.f; acc[1][k] = 0.f; }
-      }
-    }
-  }
-  if constexpr (!quant) {
-#pragma unroll
-    for (int k = 0; k < 4; ++k) tot[k] = acc[0][k] + acc[1][k];
+    // part 3 from the spare bits (see the layout)
+    a[2][1] = and_or(r.w2 >> 4, 0x00040004u, (w[0] >> 6) & 0x00030003u);
+    a[2][3] = and_or(r.w2 >> 12, 0x00040004u, (w[0] >> 14) & 0x00030003u);
+    a[3][1] = and_or(r.w2 >> 2, 0x00200020u, (w[1] >> 3) & 0x00180018u);
+    a[3][3] = and_or(r.w2 >> 10, 0x00200020u, (w[1] >> 11) & 0x00180018u);
   }
 }
 
-
 // ------------------------------------------------------------------------------------------ integer path (M = 1)
-// With a single token the fp16 tensor-core product wastes seven of its eight columns and needs the codes as fp16 pairs
-// (one conversion per two codes).  The integer product keeps the codes as bytes (one and-or extracts four of them) and
-// multiplies them with mma.m16n8k32 (s8 x s8 -> s32): a 16 x 128 blob is four instructions.  The 128 activations of a
-// pair are turned once into a 16-bit block fixed-point number, x = v * 2^e with |v| <= 32639 and one power-of-two scale
-// per pair (so the products are exact and one-hot inputs reproduce the weights bit for bit), split into two signed byte
-// planes (v = 256 * high + low) that are columns 0 and 1 of the MMA's narrow operand.  Zero-point and scales follow per
-// group, in fp32:   y += s * 2^e * (sum q v - z * sum v).
-struct XI8 {
-  uint32_t b[4][2];         // this lane's registers of the narrow operand for the four MMAs of a pair (zero for columns >= 2)
-  int sum[2];               // sum of v over tile c of the pair (all lanes hold it)
-  float scale;              // 2^e
-};
-
+// With a single token the fp16 tensor-core product wastes seven of its eight columns and needs the codes as fp16 pairs.
+// The integer product keeps the codes as bytes (one and extracts four of them) and multiplies them with mma.m16n8k32
+// (s8 x s8 -> s32): a 16 x 128 blob is four instructions.  The 128 activations of a pair are turned once into a 16-bit
+// block fixed-point number, x = v * 2^e with |v| <= 32639 and one power-of-two scale per pair (so the products are exact
+// and one-hot inputs reproduce the weights bit for bit), split into two signed byte planes (v = 256 * high + low) that
+// are columns 0 and 1 of the MMA's narrow operand.  Zero-point and scales follow per group, in fp32:
+//   y += s * 2^e * (sum q v - z * sum v).
 __device__ __forceinline__ void mma16832_s8(int (&d)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0, uint32_t b1) {
   asm("mma.sync.aligned.m16n8k32.row.col.s32.s8.s8.s32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
       : "+r"(d[0]), "+r"(d[1]), "+r"(d[2]), "+r"(d[3]) : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
 }
-
-// x: token 0's activations (fp16 or bf16 bits), pair: which 128 of them.  Lane l converts elements 4l .. 4l + 3; the
-// byte planes are then handed to the lanes that own them in the MMA's operand layout: lane (g, t) holds column g (0: low
-// plane, 1: high plane, others: zero) and, for MMA j (tile j / 2, half j % 2 of the tile), the eight reduction elements
-// 32 j + 8 t .. + 7 -- the ones lane t's weight registers of that MMA hold (in the order the and-or delivers the codes).
+// Byte quads of a tile's parts (8 codes of one row): q[part][0] the codes an and delivers first, q[part][1] the others.
 template <int FMT>
-__device__ __forceinline__ void load_x_i8(XI8& xi, const void* x, bool bf16, uint32_t pair, int lane) {
-  const uint16_t* src = reinterpret_cast<const uint16_t*>(x) + pair * 128 + 4 * lane;
-  uint2 u;
-  asm volatile("ld.global.cg.v2.u32 {%0,%1}, [%2];" : "=r"(u.x), "=r"(u.y) : "l"(src) : "memory");
-  float f[4];
-  if (bf16) {
-    f[0] = __uint_as_float(u.x << 16); f[1] = __uint_as_float(u.x & 0xffff0000u);
-    f[2] = __uint_as_float(u.y << 16); f[3] = __uint_as_float(u.y & 0xffff0000u);
-  } else {
-    const float2 a = __half22float2(*reinterpret_cast<const __half2*>(&u.x)), b = __half22float2(*reinterpret_cast<const __half2*>(&u.y));
-    f[0] = a.x; f[1] = a.y; f[2] = b.x; f[3] = b.y;
-  }
-  float am = fmaxf(fmaxf(fabsf(f[0]), fabsf(f[1])), fmaxf(fabsf(f[2]), fabsf(f[3])));
-  am = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(am)));      // non-negative floats order like integers
-  const uint32_t eb = __float_as_uint(am * 1.00396f) >> 23;           // biased exponent of a value just above the maximum
-  const bool live = eb >= 15u && eb < 255u;
-  const float inv = live ? __uint_as_float((268u - eb) << 23) : 0.f;   // 2^(14 - exponent): |v| <= 32639 = 127 * 256 + 127
-  xi.scale = live ? __uint_as_float((eb - 14u) << 23) : 0.f;           // 2^(exponent - 14)
-  int v[4], s = 0;
-#pragma unroll
-  for (int e = 0; e < 4; ++e) { v[e] = __float2int_rn(f[e] * inv); s += v[e]; }
-  // the low plane is the low byte of v as it is (a signed byte), the high plane byte 1 of v + 128
-  const uint32_t lo = prmt(prmt(v[0], v[1], 0x0040u), prmt(v[2], v[3], 0x0040u), 0x5410u);
-  const uint32_t hi = prmt(prmt(v[0] + 128, v[1] + 128, 0x0051u), prmt(v[2] + 128, v[3] + 128, 0x0051u), 0x5410u);
-  // sums per tile (64 elements: lanes 0..15 / 16..31)
-  const int s_half = __reduce_add_sync(0xffffffffu, lane < 16 ? s : 0);
-  const int s_all = __reduce_add_sync(0xffffffffu, s);
-  xi.sum[0] = s_half; xi.sum[1] = s_all - s_half;
-  const int g = lane >> 2, t = lane & 3;
-#pragma unroll
-  for (int j = 0; j < 4; ++j) {
-    const int src_lane = 8 * j + 2 * t;
-    const uint32_t l0 = __shfl_sync(0xffffffffu, lo, src_lane), l1 = __shfl_sync(0xffffffffu, lo, src_lane + 1);
-    const uint32_t h0 = __shfl_sync(0xffffffffu, hi, src_lane), h1 = __shfl_sync(0xffffffffu, hi, src_lane + 1);
-    uint32_t w0 = g == 0 ? l0 : g == 1 ? h0 : 0u, w1 = g == 0 ? l1 : g == 1 ? h1 : 0u;
-    if constexpr (FMT == FMT_Q4) {                 // the and-or delivers the codes as (0, 4, 1, 5) and (2, 6, 3, 7)
-      const uint32_t p0 = prmt(w0, w1, 0x5140u), p1 = prmt(w0, w1, 0x7362u);
-      w0 = p0; w1 = p1;
-    }
-    xi.b[j][0] = w0; xi.b[j][1] = w1;
-  }
-}
-
-// Byte quads of one part (8 codes of one row): q[part][0] the codes an and-or delivers first, q[part][1] the others.
-// tile: the tile plus the lane's offset into it (16 lane bytes for 4-bit codes, 8 lane for 3-bit ones).
-template <int FMT>
-__device__ __forceinline__ void tile_quads(const uint8_t* tile, int lane, uint32_t (&q)[4][2]) {
+__device__ __forceinline__ void code_quads(const RawTile<FMT>& r, uint32_t (&q)[4][2]) {
   if constexpr (FMT == FMT_Q4) {
-    const uint4 v = *reinterpret_cast<const uint4*>(tile);
-    const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+    const uint32_t w[4] = {r.v.x, r.v.y, r.v.z, r.v.w};
 #pragma unroll
     for (int part = 0; part < 4; ++part) {
       q[part][0] = w[part] & 0x0f0f0f0fu;
       q[part][1] = (w[part] >> 4) & 0x0f0f0f0fu;
     }
-  } else if constexpr (FMT == FMT_Q3) {
-    const uint2 v01 = *reinterpret_cast<const uint2*>(tile);
-    const uint32_t v2 = *reinterpret_cast<const uint32_t*>(tile + 256 - 4 * lane);
-    q3_quads(v01.x, v01.y, v2, q);
-  }
-}
-
-// One blob times the byte planes; blob_l: the blob plus the lane's offset into a tile (see tile_quads), blob_g: the blob
-// plus 4 (lane / 4), the offset into a scale entry.  tot[0] / tot[1]: the blob's contribution to rows g /
-// g + 8 (token 0), held by the lanes with t == 0 (the owners of columns 0 and 1 of the accumulator); the other lanes
-// return zeros.  SZ2: one scale entry per tile (groups of 64) instead of one per pair.
-template <int FMT, bool SZ2>
-__device__ __forceinline__ void blob_product_i8(const uint8_t* blob_l, const uint8_t* blob_g, int lane, const XI8& xi, float (&tot)[2]) {
-  constexpr int tb = tile_bytes(FMT);
-  const int g = lane >> 2;
-  const bool owner = (lane & 3) == 0;
-  tot[0] = tot[1] = 0.f;
-  int z_a = 0, z_b = 0;
-  float s_a = 0.f, s_b = 0.f;
-  int zsum_a = 0, zsum_b = 0;          // z * sum v over the tiles of the current scale entry
-  int d[4] = {0, 0, 0, 0};             // rows g / g + 8 x columns (low, high) for the owners
-#pragma unroll
-  for (int c = 0; c < 2; ++c) {
-    if (c == 0 || SZ2) {
-      const uint8_t* sz = blob_g + 2 * tb + c * kSzEntryBytes;
-      const uint32_t s2 = *reinterpret_cast<const uint32_t*>(sz);
-      const uint32_t z2 = *reinterpret_cast<const uint16_t*>(sz + 32 - 2 * g);
-      z_a = (int)(z2 & 255u); z_b = (int)(z2 >> 8);
-      const float2 sf = __half22float2(*reinterpret_cast<const __half2*>(&s2));
-      s_a = owner ? sf.x * xi.scale : 0.f;
-      s_b = owner ? sf.y * xi.scale : 0.f;
-      zsum_a = 0; zsum_b = 0;
-    }
-    zsum_a += z_a * xi.sum[c];
-    zsum_b += z_b * xi.sum[c];
-    uint32_t q[4][2];
-    tile_quads<FMT>(blob_l + c * tb, lane, q);
-#pragma unroll
-    for (int blk = 0; blk < 2; ++blk)          // parts 2 blk (row g) and 2 blk + 1 (row g + 8): one MMA
-      mma16832_s8(d, q[2 * blk][0], q[2 * blk + 1][0], q[2 * blk][1], q[2 * blk + 1][1], xi.b[2 * c + blk][0], xi.b[2 * c + blk][1]);
-    if (c == 1 || SZ2) {
-      tot[0] = fmaf((float)(d[1] * 256 + d[0] - zsum_a), s_a, tot[0]);
-      tot[1] = fmaf((float)(d[3] * 256 + d[2] - zsum_b), s_b, tot[1]);
-      d[0] = d[1] = d[2] = d[3] = 0;
-    }
-  }
-}
-
-// ---- the same integer product for two to eight tokens -------------------------------------------------------------
-// Tokens are the columns of the MMA's narrow operand: lane (g, t) holds, for token g, the eight reduction elements
-// 32 j + 8 t .. + 7 of MMA j -- exactly the sixteen bytes per MMA that it loads from its token's row -- as a low and a
-// high byte plane (two MMAs per weight fragment instead of one).  Every token has its own block scale and sums; the
-// accumulator of lane (g, t) belongs to tokens 2t and 2t + 1, whose scale and sums it fetches once per pair.
-struct XI8M {
-  uint32_t lo[4][2], hi[4][2];   // narrow-operand registers of the four MMAs of a pair, low and high plane (token g)
-  float scale[2];                // 2^e of tokens 2t, 2t + 1
-  int sum[2][2];                 // [token 2t + i][tile c]: sum of v over the tile
-};
-
-template <int FMT>
-__device__ __forceinline__ void load_x_i8m(XI8M& xm, const void* x, bool bf16, int m, int d_in, uint32_t pair, int lane) {
-  const int g = lane >> 2, t = lane & 3;
-  float f[4][8];
-  if (g < m) {
-    const uint16_t* src = reinterpret_cast<const uint16_t*>(x) + (size_t)g * d_in + pair * 128 + 8 * t;
-    uint4 u[4];
-#pragma unroll
-    for (int j = 0; j < 4; ++j) asm volatile("ld.global.cg.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(u[j].x), "=r"(u[j].y), "=r"(u[j].z), "=r"(u[j].w) : "l"(src + 32 * j) : "memory");
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const uint32_t w[4] = {u[j].x, u[j].y, u[j].z, u[j].w};
-#pragma unroll
-      for (int e = 0; e < 4; ++e) {
-        if (bf16) { f[j][2 * e] = __uint_as_float(w[e] << 16); f[j][2 * e + 1] = __uint_as_float(w[e] & 0xffff0000u); }
-        else { const float2 v = __half22float2(*reinterpret_cast<const __half2*>(&w[e])); f[j][2 * e] = v.x; f[j][2 * e + 1] = v.y; }
-      }
-    }
   } else {
-#pragma unroll
-    for (int j = 0; j < 4; ++j)
-#pragma unroll
-      for (int e = 0; e < 8; ++e) f[j][e] = 0.f;
-  }
-  float am = 0.f;
-#pragma unroll
-  for (int j = 0; j < 4; ++j)
-#pragma unroll
-    for (int e = 0; e < 8; ++e) am = fmaxf(am, fabsf(f[j][e]));
-  am = fmaxf(am, __shfl_xor_sync(0xffffffffu, am, 1));
-  am = fmaxf(am, __shfl_xor_sync(0xffffffffu, am, 2));               // the token's 128 elements sit in its four lanes
-  const uint32_t eb = __float_as_uint(am * 1.00396f) >> 23;
-  const bool live = eb >= 15u && eb < 255u;
-  const float inv = live ? __uint_as_float((268u - eb) << 23) : 0.f;
-  const float my_scale = live ? __uint_as_float((eb - 14u) << 23) : 0.f;
-  int my_sum[2] = {0, 0};
-#pragma unroll
-  for (int j = 0; j < 4; ++j) {
-    int v[8];
-#pragma unroll
-    for (int e = 0; e < 8; ++e) { v[e] = __float2int_rn(f[j][e] * inv); my_sum[j >> 1] += v[e]; }
-    uint32_t l0 = prmt(prmt(v[0], v[1], 0x0040u), prmt(v[2], v[3], 0x0040u), 0x5410u);
-    uint32_t l1 = prmt(prmt(v[4], v[5], 0x0040u), prmt(v[6], v[7], 0x0040u), 0x5410u);
-    uint32_t h0 = prmt(prmt(v[0] + 128, v[1] + 128, 0x0051u), prmt(v[2] + 128, v[3] + 128, 0x0051u), 0x5410u);
-    uint32_t h1 = prmt(prmt(v[4] + 128, v[5] + 128, 0x0051u), prmt(v[6] + 128, v[7] + 128, 0x0051u), 0x5410u);
-    if constexpr (FMT == FMT_Q4) {                 // the and-or delivers the codes as (0, 4, 1, 5) and (2, 6, 3, 7)
-      const uint32_t a = prmt(l0, l1, 0x5140u), b = prmt(l0, l1, 0x7362u), c = prmt(h0, h1, 0x5140u), d = prmt(h0, h1, 0x7362u);
-      l0 = a; l1 = b; h0 = c; h1 = d;
-    }
-    xm.lo[j][0] = l0; xm.lo[j][1] = l1; xm.hi[j][0] = h0; xm.hi[j][1] = h1;
-  }
-#pragma unroll
-  for (int c = 0; c < 2; ++c) {
-    my_sum[c] += __shfl_xor_sync(0xffffffffu, my_sum[c], 1);
-    my_sum[c] += __shfl_xor_sync(0xffffffffu, my_sum[c], 2);
-  }
-#pragma unroll
-  for (int i = 0; i < 2; ++i) {                    // what belongs to the accumulator's columns: tokens 2t and 2t + 1
-    const int from = (2 * t + i) * 4;
-    xm.scale[i] = __shfl_sync(0xffffffffu, my_scale, from);
-    xm.sum[i][0] = __shfl_sync(0xffffffffu, my_sum[0], from);
-    xm.sum[i][1] = __shfl_sync(0xffffffffu, my_sum[1], from);
-  }
-}
-
-// tot[i] as the accumulator of mma.m16n8k16: (row g, token 2t), (row g, token 2t + 1), (row g + 8, token 2t), (row g + 8, 2t + 1).
-template <int FMT>
-__device__ __forceinline__ void blob_product_i8m(const uint8_t* blob, int lane, uint32_t sz2, const XI8M& xm, float (&tot)[4]) {
-  constexpr int tb = tile_bytes(FMT);
-  const int g = lane >> 2;
-  const uint8_t* blob_l = blob + (FMT == FMT_Q4 ? 16 : 8) * lane;
-  const uint8_t* blob_g = blob + 4 * g;
-  tot[0] = tot[1] = tot[2] = tot[3] = 0.f;
-  int z_a = 0, z_b = 0;
-  float s_a = 0.f, s_b = 0.f;
-  int zs[2] = {0, 0};                    // sum of v over the tiles of the current scale entry, tokens 2t and 2t + 1
-  int dl[4] = {0, 0, 0, 0}, dh[4] = {0, 0, 0, 0};
-#pragma unroll
-  for (int c = 0; c < 2; ++c) {
-    if (c == 0 || sz2) {
-      const uint8_t* sz = blob_g + 2 * tb + c * kSzEntryBytes;
-      const uint32_t s2 = *reinterpret_cast<const uint32_t*>(sz);
-      const uint32_t z2 = *reinterpret_cast<const uint16_t*>(sz + 32 - 2 * g);
-      z_a = (int)(z2 & 255u); z_b = (int)(z2 >> 8);
-      const float2 sf = __half22float2(*reinterpret_cast<const __half2*>(&s2));
-      s_a = sf.x; s_b = sf.y;
-      zs[0] = zs[1] = 0;
-    }
-    zs[0] += xm.sum[0][c];
-    zs[1] += xm.sum[1][c];
-    uint32_t q[4][2];
-    tile_quads<FMT>(blob_l + c * tb, lane, q);
-#pragma unroll
-    for (int blk = 0; blk < 2; ++blk) {
-      mma16832_s8(dl, q[2 * blk][0], q[2 * blk + 1][0], q[2 * blk][1], q[2 * blk + 1][1], xm.lo[2 * c + blk][0], xm.lo[2 * c + blk][1]);
-      mma16832_s8(dh, q[2 * blk][0], q[2 * blk + 1][0], q[2 * blk][1], q[2 * blk + 1][1], xm.hi[2 * c + blk][0], xm.hi[2 * c + blk][1]);
-    }
-    if (c == 1 || sz2) {
-#pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        const int tok = i & 1, z = i < 2 ? z_a : z_b;
-        const float s = (i < 2 ? s_a : s_b) * xm.scale[tok];
-        tot[i] = fmaf((float)(dh[i] * 256 + dl[i] - z * zs[tok]), s, tot[i]);
-        dl[i] = 0; dh[i] = 0;
-      }
-    }
+    q3_quads(r.v.x, r.v.y, r.w2, q);
   }
 }
 

@@ -34,6 +34,8 @@ void wmat_shape(WMat& m, int fmt, int rows, int k_red, int group) {
   m.nt = m.n_rows / 16;
   m.kc = m.k_red / 64;
   m.np = m.k_red / 128;
+  m.half = m.np;
+  m.nt_all = m.nt; m.np_all = m.np; m.tile0 = m.pair0 = 0;
   m.sz2 = (m.group % 128) ? 1 : 0;
   m.blob = blob_bytes(fmt, m.sz2);
   m.q = nullptr;
@@ -144,14 +146,14 @@ cudaError_t repack_backbone(const WMat& dst, const eora_linear_config& c, const 
 // A view of `m` that starts at row tile t0 (see launch_repack_*).
 WMat tile_view(const WMat& m, int t0) {
   WMat v = m;
-  v.q = m.q + (int64_t)t0 * m.blob;
+  v.tile0 = t0;
   return v;
 }
 
 // A view of `m` that starts at pair p0 of the reduction axis and is n_pairs long.
 WMat pair_view(const WMat& m, int p0, int n_pairs) {
   WMat v = m;
-  v.q = m.q + (int64_t)p0 * m.nt * m.blob;
+  v.pair0 = p0;
   v.np = n_pairs; v.kc = 2 * n_pairs; v.k_red = 128 * n_pairs;
   return v;
 }
@@ -215,6 +217,7 @@ int create_impl(const eora_linear_config* cfgs, const eora_linear_weights* wts, 
   const bool ab_grouped = c.ab_format == EORA_AB_Q4 || c.ab_format == EORA_AB_Q3;
   int ab_fmt = c.ab_format == EORA_AB_F16 ? FMT_F16 : c.ab_format == EORA_AB_Q4 ? FMT_Q4 : c.ab_format == EORA_AB_Q3 ? FMT_Q3 : FMT_Q8;
   wmat_shape(h->w, backbone_fmt(c), c.d_out, c.d_in, backbone_group(c));
+  h->w.half = (h->w.np + 1) / 2;
   if (c.rank > 0) {
     int ga = ab_grouped ? c.ab_group : 0;
     int gb = ab_grouped ? (c.ab_group < c.rank ? c.ab_group : c.rank) : 0;
@@ -246,9 +249,8 @@ int create_impl(const eora_linear_config* cfgs, const eora_linear_weights* wts, 
     // t as fp32 for the simple kernels and as fp16 for the tensor-core family: only where those families can be reached
     h->t_gen = sc.take<float>(generic_reachable ? (int64_t)c.max_m * rp * 4 : 256);
     h->t16 = sc.take<__half>(c.max_m > 8 ? (int64_t)c.max_m * rp * 2 : 256);
-    h->d_t = sc.take<float>(8 * rp * 4);
-    h->y_ws = sc.take<float>((int64_t)8 * h->w.n_rows * 4);
-    h->counters = sc.take<uint32_t>((int64_t)(h->w.nt + 2) * 4);
+    h->t_part = sc.take<unsigned long long>((int64_t)decode_part_bytes((int)rp));
+    h->launches = sc.take<unsigned long long>(256);
     h->dev_status = sc.take<int>(256);
     if (pass == 0) {
       h->scratch_bytes = sc.off;
@@ -333,6 +335,7 @@ int create_multi_impl(const eora_linear_config* cfg, const eora_linear_weights* 
   const bool ab_grouped = c.ab_format == EORA_AB_Q4 || c.ab_format == EORA_AB_Q3;
   const int ab_fmt = c.ab_format == EORA_AB_F16 ? FMT_F16 : c.ab_format == EORA_AB_Q4 ? FMT_Q4 : c.ab_format == EORA_AB_Q3 ? FMT_Q3 : FMT_Q8;
   wmat_shape(h->w, backbone_fmt(c), c.d_out, c.d_in, backbone_group(c));
+  h->w.half = (h->w.np + 1) / 2;
   const int ga = ab_grouped ? c.ab_group : 0;
   const int gb = ab_grouped ? (c.ab_group < c.rank ? c.ab_group : c.rank) : 128;   // per-channel: one entry per pair
   wmat_shape(h->a, ab_fmt, n * h->r_pad, c.d_in, ga);
@@ -350,9 +353,8 @@ int create_multi_impl(const eora_linear_config* cfg, const eora_linear_weights* 
     Carve sc{reinterpret_cast<char*>(h->scratch_mem), 0};
     h->t_gen = sc.take<float>(256);            // prefill scratch is not used by this kind of handle
     h->t16 = sc.take<__half>(256);
-    h->d_t = sc.take<float>(8 * rp * 4);
-    h->y_ws = sc.take<float>((int64_t)8 * h->w.n_rows * 4);
-    h->counters = sc.take<uint32_t>((int64_t)(h->w.nt + 2) * 4);
+    h->t_part = sc.take<unsigned long long>((int64_t)decode_part_bytes((int)rp));
+    h->launches = sc.take<unsigned long long>(256);
     h->dev_status = sc.take<int>(256);
     if (pass == 0) {
       h->scratch_bytes = sc.off;
@@ -624,9 +626,9 @@ int eora_linear_last_device_status(eora_linear_t obj) {
   int v = 0;
   if (cudaMemcpy(&v, h->dev_status, sizeof(int), cudaMemcpyDeviceToHost) != cudaSuccess) return EORA_ERR_CUDA;
   if (v != 0) {
-    // A kernel whose wait ran out returned early and left partial sums, tickets and counters behind: put all
-    // scratch that must be zero between launches (status word included) back, so that the handle stays usable.
-    char* lo = reinterpret_cast<char*>(h->d_t);
+    // After a wait that ran out: put the scratch (words of t, launch counter, status word; sums and tickets of the other
+    // families) back to its first state, so that the handle stays usable.
+    char* lo = reinterpret_cast<char*>(h->t_part);
     char* hi = reinterpret_cast<char*>(h->dev_status) + 256;
     if (cudaMemset(lo, 0, (size_t)(hi - lo)) != cudaSuccess) return EORA_ERR_CUDA;
     if (decode_tc_reset(h, nullptr) != cudaSuccess || prefill_reset(h, nullptr) != cudaSuccess || cudaDeviceSynchronize() != cudaSuccess) return EORA_ERR_CUDA;

@@ -24,9 +24,9 @@ namespace eora {
 //
 // Blobs.  Two tiles that are neighbours along the reduction axis (k-tiles 2p and 2p+1, "pair" p: 128
 // reduction elements) plus the scales and zero-points they need form one contiguous blob, and the
-// blobs are ordered pair-major:  blob (p, tile) sits at  q + (p * nt + tile) * blob.  A run of consecutive
-// blobs is therefore a set of row tiles that all multiply the same 128 activations, and it is one
-// contiguous byte range that a single bulk copy brings into shared memory, scales included.
+// blobs are ordered by half of the reduction axis, row tile, pair: the first `half` pairs of all row tiles, tile by tile, then the
+// others (A and B: half = np, so simply row tile, pair).  What a set of neighbouring row tiles needs of one half is one
+// contiguous byte range.
 //   blob = [tile 2p][tile 2p+1][sz entry 0][sz entry 1 (only if sz2)]
 //   sz entry (48 B) = 8 x half2 scales (s[n_a], s[n_b]) indexed by g, then 8 x u8x2 zero-points (z[n_a] | z[n_b] << 8).
 //   If the group size is a multiple of 128 the pair has one entry (its group), otherwise (64, 192, ...)
@@ -63,6 +63,9 @@ struct WMat {
   int nt;          // n_rows / 16
   int kc;          // k_red / 64
   int np;          // k_red / 128: pairs of k-tiles
+  int half;        // pairs of the first half of the reduction axis: (np + 1) / 2 for the backbone, np for A and B
+  // A view of some of the row tiles or pairs of a larger matrix addresses that matrix: its row tiles, its pairs, and the view's place.
+  int nt_all, np_all, tile0, pair0;
   int sz2;         // 1: one scale entry per tile, 0: one per pair
   int blob;        // bytes of one blob
   const uint8_t* q;      // blobs
@@ -83,7 +86,9 @@ __host__ __device__ inline int64_t wmat_q_bytes(const WMat& w) { return (int64_t
 
 // tile (row tile `tile`, k-tile c) and the scale entry that covers it
 __host__ __device__ inline const uint8_t* wmat_blob(const WMat& w, int tile, int pair) {
-  return w.q + ((int64_t)pair * w.nt + tile) * w.blob;
+  const int t = tile + w.tile0, p = pair + w.pair0;
+  const int64_t i = p < w.half ? (int64_t)t * w.half + p : (int64_t)w.nt_all * w.half + (int64_t)t * (w.np_all - w.half) + (p - w.half);
+  return w.q + i * w.blob;
 }
 __host__ __device__ inline const uint8_t* wmat_tile(const WMat& w, int tile, int c) {
   return wmat_blob(w, tile, c >> 1) + (c & 1) * tile_bytes(w.fmt);
@@ -192,9 +197,8 @@ struct Handle {
   int64_t scratch_bytes;
   float* t_gen;          // [max_m][r_pad] fp32, simple kernels only
   __half* t16;           // [max_m][r_pad] fp16 (prefill)
-  float* d_t;            // [8][t_cols] fp32 sums of t (decode); zero between calls
-  float* y_ws;           // [8][d_out] fp32 sums of y (decode); zero between calls
-  uint32_t* counters;    // decode: [0] blobs of A done, [1] row tiles finished, [2 + tile] blobs of that row tile done
+  unsigned long long* t_part;     // decode: t as words (value, launch number)
+  unsigned long long* launches;   // decode: launch counter
   int* dev_status;       // latched device status
   void* stage_mem;       // staging for the *_host entry points, allocated by the first such call (NULL until then)
   int64_t stage_bytes;
@@ -237,6 +241,7 @@ cudaError_t launch_decode_forward(const Handle* h, const void* x, int m, void* c
                                   const int32_t* adapter_ids = nullptr);
 int decode_launch_count(const Handle* h, int m);
 int decode_grid(const Handle* h, int m);
+size_t decode_part_bytes(int t_cols);
 cudaError_t launch_wait_selftest(const Handle* h, cudaStream_t st);
 
 // tensor-memory decode family (decode_tc.cu)

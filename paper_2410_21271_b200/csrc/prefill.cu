@@ -293,13 +293,6 @@ __device__ __forceinline__ void dequant_store(Packed<FMT> r, uint32_t sc2, uint3
   }
 }
 
-__device__ __forceinline__ bool mbar_try_wait_a(uint32_t bar_addr, uint32_t parity) {
-  uint32_t ok;
-  asm volatile("{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
-               : "=r"(ok) : "r"(bar_addr), "r"(parity) : "memory");
-  return ok != 0;
-}
-
 // One part (W or the K-extension B) of a dequant warp's work.  The warp owns row tile `tile` (0..15) of
 // the CTA's 256 weight rows; k-blocks [kb_lo, kb_hi) of `mat` land in pipeline iterations it0, it0 + 1, ...,
 // and the warp takes those with index kb_lo + kphase + i * kstep (kstep = 2 when two warps share a row
@@ -323,15 +316,16 @@ __device__ __forceinline__ bool dequant_part(const WMat& mat, int n0, int kb_lo,
     const int odd = g & 1;
     uint32_t off[4];
     store_offsets(off, tile, lane);
-    const uint8_t* base = mat.q + (int64_t)rt * mat.blob;                 // this row tile's blob of pair 0
-    const int64_t pair_stride = (int64_t)mat.nt * mat.blob;
+    const uint8_t* base = wmat_blob(mat, rt, 0);                          // this row tile's blob of pair 0
+    const int64_t to_second = wmat_blob(mat, rt, mat.half) - (base + (int64_t)mat.half * mat.blob);   // what the second half of the pairs is further
     const int sz_step = mat.sz2 ? kSzEntryBytes : 0;
     const uint32_t ring = smem_u32(smem + p.w_off), full0 = smem_u32(full_w), empty0 = smem_u32(empty_w);
     Packed<FMT> pk[PF];
     uint32_t scq[PF], zzq[PF];
     auto issue = [&](int kb, int slot) {
       if (!active || kb >= kb_hi) return;
-      const uint8_t* blob = base + (kb >> 1) * pair_stride;
+      const uint8_t* blob = base + (kb >> 1) * mat.blob;
+      if ((kb >> 1) >= mat.half) blob += to_second;
       load_packed<FMT>(pk[slot], blob + (kb & 1) * tb, lane, odd);
       if constexpr (quant) {
         const uint8_t* sz = blob + 2 * tb + (kb & 1) * sz_step;
