@@ -40,15 +40,12 @@ using namespace dec;
 __host__ __device__ constexpr int warp_log(int mode) { return mode == 1 ? 3 : 4; }
 constexpr int kMaxTok = 8;                // tokens per launch (the n8 side of the mma)
 constexpr int kMaxSlices = 4;             // parts of the reduction axis that t may be sent in
-constexpr uint32_t kLaunchShift = 10;     // a launch adds 2^10 to the launch counter (at most 1023 CTAs)
 constexpr int kMaxTiles = 48;             // row tiles per cluster (what its shared memory is sized for); more: further CTAs, in waves
 constexpr int kXBytes = 58 * 1024;        // activations of a chunk: 28 pairs of eight tokens
 constexpr int kMaxSmem = 226 * 1024;
 constexpr int kHalfSmem = 112 * 1024;     // what two CTAs of an SM may use each
 constexpr int kMaxSlots = 4;
 constexpr int kPlaneBytes = 272;          // integer path: two byte planes of a pair (256 B), scale and two sums
-
-struct Share { uint32_t per, rem; };      // items dealt to n takers: taker i gets per + (i < rem)
 
 struct DecodeArgs {
   const uint8_t* a_q; const uint8_t* w_q; const uint8_t* b_q;
@@ -95,37 +92,6 @@ __device__ __forceinline__ void touch_args(const DecodeArgs& p) {
   for (int i = 0; i < (int)(sizeof(DecodeArgs) / 4); i += 16) asm volatile("" ::"r"(w[i]));
   asm volatile("" ::"r"(w[sizeof(DecodeArgs) / 4 - 1]));
 }
-
-__device__ __forceinline__ uint32_t share_lo(const Share& s, uint32_t i) { return i * s.per + (i < s.rem ? i : s.rem); }
-__device__ __forceinline__ uint32_t share_n(const Share& s, uint32_t i) { return s.per + (i < s.rem ? 1u : 0u); }
-
-__device__ __forceinline__ uint4 ld_cg_u4(const void* p) {
-  uint4 v;
-  asm volatile("ld.global.cg.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p) : "memory");
-  return v;
-}
-__device__ __forceinline__ uint32_t pack_h2(float a, float b) {
-  __half2 h = __floats2half2_rn(a, b);
-  return *reinterpret_cast<uint32_t*>(&h);
-}
-__device__ __forceinline__ uint32_t bf2_to_h2(uint32_t v) {
-  return pack_h2(__uint_as_float(v << 16), __uint_as_float(v & 0xffff0000u));
-}
-__device__ __forceinline__ void prefetch_l2(const void* p, uint32_t bytes) {
-  asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p), "r"(bytes) : "memory");
-}
-__device__ __forceinline__ unsigned long long ld_volatile_u64(const unsigned long long* p) {
-  unsigned long long v;
-  asm volatile("ld.volatile.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
-  return v;
-}
-__device__ __forceinline__ uint32_t mapa(uint32_t addr, uint32_t rank) {
-  uint32_t r;
-  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
-  return r;
-}
-__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
-__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
 
 // ---- activations -> shared memory ------------------------------------------------------------------------------
 // Sixteen lanes take the 128 activations of one (pair, token), eight consecutive ones each.
@@ -405,7 +371,7 @@ __device__ __forceinline__ void run_a(const DecodeArgs& p, float* red, int warp,
   }
   asm volatile("griddepcontrol.wait;" ::: "memory");
   if (tr && lane == 0) tr[1] = globaltimer_ns();
-  const uint32_t launch = (uint32_t)(ld_volatile_u64(p.launches) >> kLaunchShift) + 1u;
+  const uint32_t launch = launch_number(p.launches);
   const uint16_t* xrow = reinterpret_cast<const uint16_t*>(p.x) + (size_t)(has ? g : 0) * p.d_in + 8 * t;
   int flip = 0;
   for (uint32_t u = blockIdx.x; u < units; u += p.n_a, flip ^= 1) {
@@ -473,24 +439,6 @@ __device__ __forceinline__ int sub_of(const DecodeArgs& p, uint32_t tile) {
   return s;
 }
 
-// Two neighbouring columns of t, one part of the reduction axis: asked for (load) and, until the launch's words are there, again.
-struct TWords { unsigned long long a, b; };
-__device__ __forceinline__ void load_t(TWords& w, const unsigned long long* src) {
-  asm volatile("ld.volatile.global.v2.u64 {%0, %1}, [%2];" : "=l"(w.a), "=l"(w.b) : "l"(src) : "memory");
-}
-__device__ __forceinline__ bool wait_t(const DecodeArgs& p, TWords& w, const unsigned long long* src, uint32_t launch) {
-  unsigned long long t0 = 0;
-  for (uint32_t tries = 1;; ++tries) {
-    if ((uint32_t)(w.a >> 32) == launch && (uint32_t)(w.b >> 32) == launch) return true;
-    if ((tries & 63u) == 0u) {
-      const unsigned long long now = globaltimer_ns();
-      if (t0 == 0) t0 = now;
-      else if (now - t0 > p.wait_ns) { atomicExch(p.dev_status, EORA_ERR_DEVICE_TIMEOUT); return false; }
-    }
-    load_t(w, src);
-  }
-}
-
 // x / n for small x; inv = ceil(2^32 / n), 0 for n == 1
 __device__ __forceinline__ uint32_t div_by(uint32_t x, uint32_t inv) { return inv ? __umulhi(x, inv) : x; }
 // The warps whose runs hold blobs of row tile f of a chunk of n pairs: those of its first to its last blob.  Warp w's run is
@@ -500,13 +448,6 @@ template <int kWarps>
 __device__ __forceinline__ Owners owners_of(uint32_t f, uint32_t n, uint32_t inv) {
   const uint32_t x = (f * n + 1) * kWarps - 1;
   return {div_by(x, inv), div_by(x + (n - 1) * kWarps, inv)};
-}
-
-// A warp's ring of weights in shared memory: position of the slot that is read next, its barrier and the phase it completes.
-struct Ring { uint32_t base, bytes, bars, so, bar, parity; };
-__device__ __forceinline__ void ring_next(Ring& r, uint32_t slot_b) {
-  r.so += slot_b; r.bar += 8;
-  if (r.so == r.bytes) { r.so = 0; r.bar = r.bars; r.parity ^= 1u; }
 }
 
 // Pairs of t that row tile `tile` takes part in, within [c0, c1): [a, b).
@@ -606,7 +547,7 @@ __device__ __forceinline__ void finish(const DecodeArgs& p, uint8_t* smem, uint3
 #pragma unroll 1
           for (uint32_t s = 0; s < p.a_slices; ++s, src += (size_t)p.m * p.t_cols) {
             if (!first || s || e != threadIdx.x) load_t(tw, src);
-            if (!wait_t(p, tw, src, launch)) break;
+            if (!wait_t(tw, src, launch, p.wait_ns, p.dev_status)) break;
             v0 += __uint_as_float((uint32_t)tw.a); v1 += __uint_as_float((uint32_t)tw.b);
           }
         }
@@ -776,7 +717,7 @@ __global__ void __launch_bounds__(32 << warp_log(MODE), MODE == 1 ? 2 : 1) k_dec
 
     asm volatile("griddepcontrol.wait;" ::: "memory");
     if (tr && lane == 0) tr[1] = globaltimer_ns();
-    const uint32_t launch = (uint32_t)(ld_volatile_u64(p.launches) >> kLaunchShift) + 1u;
+    const uint32_t launch = launch_number(p.launches);
 
     uint32_t n = 0, inv = 0;
 #pragma unroll 1
@@ -884,12 +825,7 @@ __global__ void __launch_bounds__(32 << warp_log(MODE), MODE == 1 ? 2 : 1) k_dec
     }
   }
   __syncthreads();                                 // every thread of the CTA has read the launch counter
-  if (threadIdx.x == 0) {
-    // 2^10 per launch in all: a CTA's 1, and the last CTA of the grid the rest, so that the count never reaches the next
-    // multiple before every CTA has read it
-    const unsigned long long v = blockIdx.x + 1 == gridDim.x ? (1ull << kLaunchShift) - (gridDim.x - 1) : 1ull;
-    asm volatile("red.global.add.u64 [%0], %1;" ::"l"(p.launches), "l"(v) : "memory");
-  }
+  if (threadIdx.x == 0) count_launch(p.launches);
   if (tr && lane == 0) tr[3] = globaltimer_ns();
 }
 
@@ -1040,7 +976,7 @@ bool make_plan(const Handle* h, int m, Plan& pl) {
 __global__ void k_wait_selftest(unsigned long long* t_part, const unsigned long long* launches, int* dev_status, unsigned long long limit_ns) {
   if (threadIdx.x == 0) {
     t_part[0] = 0x3f800000ull;                     // 1.0f, sent by launch 0 (the first is number 1)
-    const uint32_t want = (uint32_t)(ld_volatile_u64(launches) >> kLaunchShift) + 1u;
+    const uint32_t want = launch_number(launches);
     const unsigned long long t0 = dec::globaltimer_ns();
     while ((uint32_t)(ld_volatile_u64(t_part) >> 32) != want) {
       if (dec::globaltimer_ns() - t0 > limit_ns) { atomicExch(dev_status, EORA_ERR_DEVICE_TIMEOUT); break; }

@@ -507,6 +507,77 @@ __device__ __forceinline__ void code_quads(const RawTile<FMT>& r, uint32_t (&q)[
   }
 }
 
+// ------------------------------------------------------------------------------------------ deal, exchange of t
+struct Share { uint32_t per, rem; };      // items dealt to n takers: taker i gets per + (i < rem)
+__device__ __forceinline__ uint32_t share_lo(const Share& s, uint32_t i) { return i * s.per + (i < s.rem ? i : s.rem); }
+__device__ __forceinline__ uint32_t share_n(const Share& s, uint32_t i) { return s.per + (i < s.rem ? 1u : 0u); }
+
+__device__ __forceinline__ uint4 ld_cg_u4(const void* p) {
+  uint4 v;
+  asm volatile("ld.global.cg.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p) : "memory");
+  return v;
+}
+__device__ __forceinline__ uint32_t pack_h2(float a, float b) {
+  __half2 h = __floats2half2_rn(a, b);
+  return *reinterpret_cast<uint32_t*>(&h);
+}
+__device__ __forceinline__ uint32_t bf2_to_h2(uint32_t v) {
+  return pack_h2(__uint_as_float(v << 16), __uint_as_float(v & 0xffff0000u));
+}
+__device__ __forceinline__ void prefetch_l2(const void* p, uint32_t bytes) {
+  asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p), "r"(bytes) : "memory");
+}
+__device__ __forceinline__ unsigned long long ld_volatile_u64(const unsigned long long* p) {
+  unsigned long long v;
+  asm volatile("ld.volatile.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
+  return v;
+}
+__device__ __forceinline__ uint32_t mapa(uint32_t addr, uint32_t rank) {
+  uint32_t r;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
+  return r;
+}
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
+
+
+// Launches of a handle are numbered from 1 (the kernels of the decode family share the count).  A launch adds 2^10 in all: a
+// CTA's 1, and the last CTA of the grid the rest, so that the count never reaches the next multiple before every CTA has
+// read it (a CTA adds its share after its reads, at most 1023 CTAs).
+constexpr uint32_t kLaunchShift = 10;
+__device__ __forceinline__ uint32_t launch_number(const unsigned long long* launches) {
+  return (uint32_t)(ld_volatile_u64(launches) >> kLaunchShift) + 1u;
+}
+__device__ __forceinline__ void count_launch(unsigned long long* launches) {
+  const unsigned long long v = blockIdx.x + 1 == gridDim.x ? (1ull << kLaunchShift) - (gridDim.x - 1) : 1ull;
+  asm volatile("red.global.add.u64 [%0], %1;" ::"l"(launches), "l"(v) : "memory");
+}
+
+// Two neighbouring columns of t, one part of the reduction axis: asked for (load) and, until the launch's words are there, again.
+struct TWords { unsigned long long a, b; };
+__device__ __forceinline__ void load_t(TWords& w, const unsigned long long* src) {
+  asm volatile("ld.volatile.global.v2.u64 {%0, %1}, [%2];" : "=l"(w.a), "=l"(w.b) : "l"(src) : "memory");
+}
+__device__ __forceinline__ bool wait_t(TWords& w, const unsigned long long* src, uint32_t launch, unsigned long long limit_ns, int* dev_status) {
+  unsigned long long t0 = 0;
+  for (uint32_t tries = 1;; ++tries) {
+    if ((uint32_t)(w.a >> 32) == launch && (uint32_t)(w.b >> 32) == launch) return true;
+    if ((tries & 63u) == 0u) {
+      const unsigned long long now = globaltimer_ns();
+      if (t0 == 0) t0 = now;
+      else if (now - t0 > limit_ns) { atomicExch(dev_status, EORA_ERR_DEVICE_TIMEOUT); return false; }
+    }
+    load_t(w, src);
+  }
+}
+
+// A warp's ring of weights in shared memory: position of the slot that is read next, its barrier and the phase it completes.
+struct Ring { uint32_t base, bytes, bars, so, bar, parity; };
+__device__ __forceinline__ void ring_next(Ring& r, uint32_t slot_b) {
+  r.so += slot_b; r.bar += 8;
+  if (r.so == r.bytes) { r.so = 0; r.bar = r.bars; r.parity ^= 1u; }
+}
+
 __device__ __forceinline__ void store_y(void* y, int dtype, int64_t i, float v) {
   if (dtype == EORA_Y_F16) reinterpret_cast<__half*>(y)[i] = __float2half_rn(v);
   else if (dtype == EORA_Y_BF16) reinterpret_cast<__nv_bfloat16*>(y)[i] = __float2bfloat16_rn(v);

@@ -438,6 +438,8 @@ int eora_linear_forward_multi(eora_linear_t obj, const void* x, int32_t m, const
   if (!on_handle_device(h)) return EORA_ERR_UNSUPPORTED;
   if (!decode_supported(h, m)) return EORA_ERR_UNSUPPORTED;
   void* ys[1] = {y};
+  if (h->cfg.x_dtype == EORA_X_F16 && mid_supported(h, m))
+    return launch_mid_forward(h, x, m, ys, reinterpret_cast<cudaStream_t>(stream), adapter_ids) == cudaSuccess ? EORA_OK : EORA_ERR_CUDA;
   return launch_decode_forward(h, x, m, ys, reinterpret_cast<cudaStream_t>(stream), adapter_ids) == cudaSuccess ? EORA_OK : EORA_ERR_CUDA;
 }
 

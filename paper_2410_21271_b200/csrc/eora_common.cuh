@@ -244,6 +244,11 @@ int decode_grid(const Handle* h, int m);
 size_t decode_part_bytes(int t_cols);
 cudaError_t launch_wait_selftest(const Handle* h, cudaStream_t st);
 
+// medium batches (decode_mid.cu)
+bool mid_supported(const Handle* h, int m);
+int mid_launch_count(const Handle* h, int m);
+cudaError_t launch_mid_forward(const Handle* h, const void* x16, int m, void* const* ys, cudaStream_t st, const int32_t* adapter_ids = nullptr);
+
 // tensor-memory decode family (decode_tc.cu)
 cudaError_t decode_tc_init(Handle* h, cudaStream_t st);
 void decode_tc_free(Handle* h);

@@ -764,8 +764,8 @@ bool prefill_supported(const Handle* h, int m) {
   return encode_fn() != nullptr;
 }
 
-int prefill_launch_count(const Handle* h, int) {
-  return (h->cfg.rank > 0 ? 2 : 1) + (h->cfg.x_dtype == EORA_X_BF16 ? 1 : 0);
+int prefill_launch_count(const Handle* h, int m) {
+  return (mid_supported(h, m) ? mid_launch_count(h, m) : h->cfg.rank > 0 ? 2 : 1) + (h->cfg.x_dtype == EORA_X_BF16 ? 1 : 0);
 }
 
 cudaError_t prefill_init(Handle* h) {
@@ -835,6 +835,7 @@ cudaError_t launch_prefill_forward(const Handle* h, const void* x, int m, void* 
     k_bf16_to_f16<<<(int)blocks, 256, 0, st>>>(reinterpret_cast<const __nv_bfloat16*>(x), ps->x16, n);
     x16 = ps->x16;
   }
+  if (mid_supported(h, m)) return launch_mid_forward(h, x16, m, ys, st);
   const int bt = token_tile(m);
   PrefillState* pst = reinterpret_cast<PrefillState*>(h->prefill_state);
   const bool thin = m <= kThinTokens && pst && pst->split_mem;      // one token tile: split the reduction axis instead
