@@ -371,83 +371,65 @@ template <int FMT, bool SZ2> __device__ __forceinline__ void load_blob_s(RawBlob
   }
 }
 
-// The wide operand of the tile's four mma.m16n8k16 as exact fp16 values: a[2 * blk + sub][*].  `aux`: shared-memory address of the
-// 2:4 expansion table; unused by other formats.
+// The wide operand of two of the tile's four mma.m16n8k16 as exact fp16 values: those of its 32-element block blk (0, 1).  `aux`:
+// shared-memory address of the 2:4 expansion table; unused by other formats.
 template <int FMT>
-__device__ __forceinline__ void tile_frags(const RawTile<FMT>& r, const ZC& zc, uint32_t (&a)[4][4], uint32_t aux) {
-  if constexpr (FMT == FMT_Q4) {
-    const uint32_t w[4] = {r.v.x, r.v.y, r.v.z, r.v.w};
+__device__ __forceinline__ void half_frags(const RawTile<FMT>& r, const ZC& zc, int blk, uint32_t (&a0)[4], uint32_t (&a1)[4], uint32_t aux) {
 #pragma unroll
-    for (int part = 0; part < 4; ++part) {
-      const int hf = part & 1, blk = part >> 1;
-      uint32_t lo = w[part], hi = w[part] >> 8;
-      uint32_t h0 = and_or(lo, 0x000f000fu, kMagic), h1 = and_or(lo, 0x00f000f0u, kMagic);
-      uint32_t h2 = and_or(hi, 0x000f000fu, kMagic), h3 = and_or(hi, 0x00f000f0u, kMagic);
-      a[blk * 2 + 0][hf] = h2sub(h0, zc.c[hf][0]);
-      a[blk * 2 + 0][hf + 2] = h2fma(h1, 0x2C002C00u, zc.c[hf][1]);   // * 1/16
-      a[blk * 2 + 1][hf] = h2sub(h2, zc.c[hf][0]);
-      a[blk * 2 + 1][hf + 2] = h2fma(h3, 0x2C002C00u, zc.c[hf][1]);
-    }
-  } else if constexpr (FMT == FMT_Q3) {
-    uint32_t q[4][2];
-    q3_quads(r.v.x, r.v.y, r.w2, q);
-#pragma unroll
-    for (int part = 0; part < 4; ++part) {
-      const int hf = part & 1, blk = part >> 1;
-#pragma unroll
-      for (int quad = 0; quad < 2; ++quad) {          // quad = which of the part's two mma
-        a[blk * 2 + quad][hf] = h2sub(quad_pair(q[part][quad], 0), zc.c[hf][0]);
-        a[blk * 2 + quad][hf + 2] = h2sub(quad_pair(q[part][quad], 1), zc.c[hf][0]);
+  for (int hf = 0; hf < 2; ++hf) {                   // row g, row g + 8: part 2 * blk + hf
+    if constexpr (FMT == FMT_Q4) {
+      const uint32_t lo = blk ? (hf ? r.v.w : r.v.z) : (hf ? r.v.y : r.v.x), hi = lo >> 8;
+      a0[hf] = h2sub(and_or(lo, 0x000f000fu, kMagic), zc.c[hf][0]);
+      a0[hf + 2] = h2fma(and_or(lo, 0x00f000f0u, kMagic), 0x2C002C00u, zc.c[hf][1]);   // * 1/16
+      a1[hf] = h2sub(and_or(hi, 0x000f000fu, kMagic), zc.c[hf][0]);
+      a1[hf + 2] = h2fma(and_or(hi, 0x00f000f0u, kMagic), 0x2C002C00u, zc.c[hf][1]);
+    } else if constexpr (FMT == FMT_Q3) {
+      uint32_t q0, q1;                               // the part's two byte quads of codes (q3_quads)
+      if (blk == 1 && hf == 1) {
+        q0 = and_or(r.w2 >> 4, 0x04040404u, (r.v.x >> 6) & 0x03030303u);
+        q1 = and_or(r.w2 >> 5, 0x04040404u, (r.v.y >> 6) & 0x03030303u);
+      } else {
+        const uint32_t w = blk ? r.w2 : hf ? r.v.y : r.v.x;
+        q0 = w & 0x07070707u; q1 = (w >> 3) & 0x07070707u;
       }
-    }
-  } else if constexpr (FMT == FMT_Q8) {
+      a0[hf] = h2sub(quad_pair(q0, 0), zc.c[hf][0]); a0[hf + 2] = h2sub(quad_pair(q0, 1), zc.c[hf][0]);
+      a1[hf] = h2sub(quad_pair(q1, 0), zc.c[hf][0]); a1[hf + 2] = h2sub(quad_pair(q1, 1), zc.c[hf][0]);
+    } else if constexpr (FMT == FMT_Q8) {
+      const uint32_t w0 = hf ? r.v[blk].z : r.v[blk].x, w1 = hf ? r.v[blk].w : r.v[blk].y;
+      a0[hf] = h2sub(and_or(w0, 0x00ff00ffu, kMagic), zc.c[hf][0]);
+      a0[hf + 2] = h2sub(and_or(w0 >> 8, 0x00ff00ffu, kMagic), zc.c[hf][0]);
+      a1[hf] = h2sub(and_or(w1, 0x00ff00ffu, kMagic), zc.c[hf][0]);
+      a1[hf + 2] = h2sub(and_or(w1 >> 8, 0x00ff00ffu, kMagic), zc.c[hf][0]);
+    } else if constexpr (FMT == FMT_F16) {
+      const uint4 u = r.v[2 * blk + hf];
+      a0[hf] = u.x; a0[hf + 2] = u.y; a1[hf] = u.z; a1[hf + 2] = u.w;
+    } else {
+      // 2:4 formats: a quad's two kept values (SQ4: two codes made exact fp16 values first) are spread over its four
+      // positions with two byte permutes whose selectors come from the table.
 #pragma unroll
-    for (int pl = 0; pl < 2; ++pl) {
-      const uint4 u = r.v[pl];
-#pragma unroll
-      for (int hf = 0; hf < 2; ++hf) {
-        const uint32_t w0 = hf ? u.z : u.x, w1 = hf ? u.w : u.y;
-        a[pl * 2 + 0][hf] = h2sub(and_or(w0, 0x00ff00ffu, kMagic), zc.c[hf][0]);
-        a[pl * 2 + 0][hf + 2] = h2sub(and_or(w0 >> 8, 0x00ff00ffu, kMagic), zc.c[hf][0]);
-        a[pl * 2 + 1][hf] = h2sub(and_or(w1, 0x00ff00ffu, kMagic), zc.c[hf][0]);
-        a[pl * 2 + 1][hf + 2] = h2sub(and_or(w1 >> 8, 0x00ff00ffu, kMagic), zc.c[hf][0]);
-      }
-    }
-  } else if constexpr (FMT == FMT_F16) {
-#pragma unroll
-    for (int part = 0; part < 4; ++part) {
-      const int hf = part & 1, blk = part >> 1;
-      a[blk * 2 + 0][hf] = r.v[part].x;
-      a[blk * 2 + 0][hf + 2] = r.v[part].y;
-      a[blk * 2 + 1][hf] = r.v[part].z;
-      a[blk * 2 + 1][hf + 2] = r.v[part].w;
-    }
-  } else {
-    // 2:4 formats: a quad's two kept values (SQ4: two codes made exact fp16 values first) are spread over its four positions
-    // with two byte permutes whose selectors come from the table.
-#pragma unroll
-    for (int blk = 0; blk < 2; ++blk) {
-#pragma unroll
-      for (int hf = 0; hf < 2; ++hf) {
-#pragma unroll
-        for (int quad = 0; quad < 2; ++quad) {
-          uint32_t kept;
-          if constexpr (FMT == FMT_SP24) {
-            const uint4 u = r.v[blk];
-            kept = hf ? (quad ? u.w : u.z) : (quad ? u.y : u.x);
-          } else {
-            kept = h2sub(and_or((blk ? r.v.y : r.v.x) >> (8 * hf + 4 * quad), 0x000f000fu, kMagic), zc.c[hf][0]);
-          }
-          const int sh = 8 * (blk * 2 + hf) + 4 * quad - 2;           // nibble * 4 = byte offset into the table
-          const uint32_t offb = (sh < 0 ? (r.meta << 2) : (r.meta >> (sh < 0 ? 0 : sh))) & 0x3Cu;
-          uint32_t sel;
-          asm volatile("ld.shared.u32 %0, [%1];" : "=r"(sel) : "r"(aux + offb));
-          a[blk * 2 + quad][hf] = prmt(kept, 0u, sel);
-          a[blk * 2 + quad][hf + 2] = prmt(kept, 0u, sel >> 16);
+      for (int quad = 0; quad < 2; ++quad) {
+        uint32_t kept;
+        if constexpr (FMT == FMT_SP24) {
+          const uint4 u = r.v[blk];
+          kept = hf ? (quad ? u.w : u.z) : (quad ? u.y : u.x);
+        } else {
+          kept = h2sub(and_or((blk ? r.v.y : r.v.x) >> (8 * hf + 4 * quad), 0x000f000fu, kMagic), zc.c[hf][0]);
         }
+        const int sh = 8 * (blk * 2 + hf) + 4 * quad - 2;           // nibble * 4 = byte offset into the table
+        const uint32_t offb = (sh < 0 ? (r.meta << 2) : (r.meta >> (sh < 0 ? 0 : sh))) & 0x3Cu;
+        uint32_t sel;
+        asm volatile("ld.shared.u32 %0, [%1];" : "=r"(sel) : "r"(aux + offb));
+        (quad ? a1 : a0)[hf] = prmt(kept, 0u, sel);
+        (quad ? a1 : a0)[hf + 2] = prmt(kept, 0u, sel >> 16);
       }
     }
   }
+}
+// All four: a[2 * blk + sub][*].
+template <int FMT>
+__device__ __forceinline__ void tile_frags(const RawTile<FMT>& r, const ZC& zc, uint32_t (&a)[4][4], uint32_t aux) {
+  half_frags<FMT>(r, zc, 0, a[0], a[1], aux);
+  half_frags<FMT>(r, zc, 1, a[2], a[3], aux);
 }
 
 // 3/4-bit codes as the fp16 bit patterns they are in their words (subnormals q * 2^-24): a[2 * blk] with the codes at the low end of

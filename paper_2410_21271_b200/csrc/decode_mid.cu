@@ -10,14 +10,14 @@
 // is cut like in decode.cu: clusters of two CTAs own row tiles and split the reduction axis, sums meet in shared memory,
 // t travels as self-validating words from clusters of its own.
 //
-// Work of a CTA.  Its row tiles go in pairs (32 rows share every activation fragment that is read from shared memory); kWarps / (pairs of
-// row tiles) warps share one and cut the reduction axis among them, chunk by chunk.  A warp keeps its sums in registers
-// from the first chunk to the last.  X comes by TMA in chunks of pairs, double-buffered, as [32 k][token][32 fp16]: the
-// eight tokens x 64 bytes that a fragment load of a warp reads are 512 contiguous bytes.  The weights come
-// through a ring per warp.  Weights are RN((q - z) * s) in fp16, as in prefill.cu, so scales need no accumulators of
-// their own.
+// Work of a CTA.  Its row tiles go in pairs (32 rows share every activation fragment that is read from shared memory); kWarps /
+// (pairs of row tiles) warps share one and take turns along the reduction axis, 128 elements at a time.  A warp keeps its
+// sums in registers to the end; t . B is the end of the reduction axis (a CTA's half of every 128 columns of t).  X comes by TMA
+// into a ring of 128-element slots, laid out as [32 k][token][32 fp16]: the eight tokens x 64 bytes that a
+// fragment load of a warp reads are 512 contiguous bytes.  The warp that is the last to read a slot refills it.  The weights come through a ring per warp.  Weights
+// are RN((q - z) * s) in fp16, as in prefill.cu, or, up to 16 tokens, exact q - z with the scale applied to the group's sums.
 //
-// Measured: four LLaMA3-8B blocks, 4-bit backbone and adapters, 16 tokens 544 -> 270 us (see also mid_supported).
+// Measured: four LLaMA3-8B blocks, 4-bit backbone and adapters, 16 tokens 544 -> 261 us (see also mid_supported).
 #include <cuda.h>
 #include "decode_common.cuh"
 
@@ -25,12 +25,13 @@ namespace eora {
 namespace {
 using namespace dec;
 
-constexpr int kWarpLog = 4, kWarps = 1 << kWarpLog, kThreads = kWarps * 32;
+// Sixteen warps of 128 registers; a seventeenth as the producer of X would leave 96 (five warps share a scheduler's registers).
+constexpr int kWarps = 16, kThreads = kWarps * 32;
 constexpr int kMaxPass = 32;              // tokens per launch
 constexpr int kSegPitch = 36;             // floats from one token's 32 row sums to the next (36: the four token pairs of a store hit different banks)
 constexpr int kMaxSmem = 226 * 1024;
 constexpr int kMaxSlots = 4;
-constexpr uint32_t kBox = 4;              // pairs of X per copy
+constexpr int kMaxXSlots = 32;
 
 struct MidArgs {
   const uint8_t* a_q; const uint8_t* w_q; const uint8_t* b_q;
@@ -42,16 +43,16 @@ struct MidArgs {
   Share a_tiles;                          // row tiles of A dealt to their clusters
   uint32_t w_nt;                          // row tiles of W
   Share w_dbl;                            // pairs of row tiles of W dealt to their clusters
-  uint32_t chunk, a_chunk;                // pairs of X per buffer (W, A)
-  uint32_t slots, slot_pairs, ring_pitch; // ring of a warp (W): slots of slot_pairs pairs of two row tiles
+  uint32_t xslots, a_xslots;              // slots of X, one pair each (W, A)
+  uint32_t slots, ring_pitch;             // ring of a warp (W): slots of one pair of two row tiles
   uint32_t a_slots, a_pitch;              // ring of a warp (A): slots of one blob
-  uint32_t off_ring, off_inbox, off_bseg, off_t;      // shared memory, W (X buffers first; later the warps' sums over them)
-  uint32_t a_off_ring, a_off_inbox;
+  uint32_t off_ring, a_off_ring, off_inbox;      // shared memory: X slots | rings; later, over both, the warps' sums | the partner's sums
   void* ys[4];
   uint32_t sub_tile0[5];                  // layer i owns row tiles [sub_tile0[i], sub_tile0[i + 1]) and pairs [i, i + 1) * sub_pairs of t
   int sub_dout[4];
   int n_sub;
-  uint32_t sub_pairs, b_np, t_chunk, b_log;           // as in decode.cu
+  uint32_t sub_pairs, b_np;               // as in decode.cu
+  uint32_t t_chunk;                       // pairs of t in shared memory at a time
   uint32_t adp_pairs;                     // several adapters: pair p of t belongs to adapter p / adp_pairs (0: one adapter)
   signed char adp[kMaxPass];              // adapter of every token (-1: none)
   unsigned long long* t_part;             // [m][t_cols / 2] words (two columns as fp16, launch number)
@@ -80,22 +81,20 @@ __device__ __forceinline__ void load_sz(SZ& z, uint32_t entry, int lane) {
   make_zc<FMT>(z.zc, lds_u16(entry + 32 + (lane >> 2) * 2));
 }
 
-// The wide operand of the tile's four mma: RN((q - z) * s) in fp16, or (SCALED false) the exact q - z.
+// The wide operand of a 32-element block's two mma: RN((q - z) * s) in fp16, or (SCALED false) the exact q - z.
 template <int FMT, bool SCALED>
-__device__ __forceinline__ void weights_f16(uint32_t tile, int lane, const SZ& z, uint32_t lut, uint32_t (&a)[4][4]) {
-  RawTile<FMT> r;
-  load_tile_s<FMT>(r, tile, lane);
-  tile_frags<FMT>(r, z.zc, a, lut);
+__device__ __forceinline__ void weights_half(const RawTile<FMT>& r, int blk, const SZ& z, uint32_t lut, uint32_t (&a)[2][4]) {
+  half_frags<FMT>(r, z.zc, blk, a[0], a[1], lut);
   if constexpr (SCALED && fmt_quantised(FMT)) {
 #pragma unroll
-    for (int i = 0; i < 4; ++i)
+    for (int i = 0; i < 2; ++i)
 #pragma unroll
       for (int e = 0; e < 4; ++e) a[i][e] = h2mul(a[i][e], z.s[e & 1]);
   }
 }
 
-// One pair of T row tiles (blobs `stride` apart) times the activations at x: [4 blocks of 32 k][8 NT tokens][32 fp16], x already at
-// this lane's token and piece.  Up to 16 tokens the scale of a quantised group is applied to the group's sums (8 NT T multiplications
+// One pair of T row tiles (blobs `stride` apart) times the activations of 8 NT tokens at x: [4 blocks of 32 k][8 NT tokens][32 fp16],
+// x already at this lane's token and piece.  Up to 16 tokens the scale of a quantised group is applied to the group's sums (8 NT T multiplications
 // a lane instead of 32 T on the weights); with more the sums would need as many registers again.
 template <int FMT, bool SZ2, int NT, int T>
 __device__ __forceinline__ void product(uint32_t blob, uint32_t stride, int lane, uint32_t x, uint32_t lut, float (&acc)[T][NT][4]) {
@@ -113,23 +112,24 @@ __device__ __forceinline__ void product(uint32_t blob, uint32_t stride, int lane
   }
 #pragma unroll
   for (int c = 0; c < 2; ++c) {
-    uint32_t a[T][4][4];
+    RawTile<FMT> r[T];
 #pragma unroll
     for (int u = 0; u < T; ++u) {
       if constexpr (fmt_quantised(FMT)) { if (c == 0 || SZ2) load_sz<FMT>(z[u], blob + u * stride + 2 * tb + c * kSzEntryBytes, lane); }
-      weights_f16<FMT, !late>(blob + u * stride + c * tb, lane, z[u], lut, a[u]);
+      load_tile_s<FMT>(r[u], blob + u * stride + c * tb, lane);
     }
 #pragma unroll
-    for (int n = 0; n < NT; ++n) {
+    for (int b = 0; b < 2; ++b) {
+      uint32_t a[T][2][4];
 #pragma unroll
-      for (int b = 0; b < 2; ++b) {
+      for (int u = 0; u < T; ++u) weights_half<FMT, !late>(r[u], b, z[u], lut, a[u]);
+#pragma unroll
+      for (int n = 0; n < NT; ++n) {
         const uint4 v = lds_u4(x + (2 * c + b) * (NT * 512) + n * 512);
 #pragma unroll
-        for (int u = 0; u < T; ++u) {
-          float (&o)[4] = late ? d[late ? u : 0][late ? n : 0] : acc[u][n];
-          mma16816(o, a[u][2 * b], v.x, v.y);
-          mma16816(o, a[u][2 * b + 1], v.z, v.w);
-        }
+        for (int u = 0; u < T; ++u) mma16816(late ? d[late ? u : 0][late ? n : 0] : acc[u][n], a[u][0], v.x, v.y);
+#pragma unroll
+        for (int u = 0; u < T; ++u) mma16816(late ? d[late ? u : 0][late ? n : 0] : acc[u][n], a[u][1], v.z, v.w);
       }
     }
     if constexpr (late) {
@@ -150,35 +150,71 @@ __device__ __forceinline__ void product(uint32_t blob, uint32_t stride, int lane
   }
 }
 
-// A or B: the format is known at run time only (one uniform branch per blob).  x_step: bytes from one block of eight tokens to the
-// next, k_step: from one block of 32 k to the next.
-template <int FMT, bool SZ2, int NT>
-__device__ __forceinline__ void product_ab1(uint32_t blob, int lane, uint32_t x, uint32_t x_step, uint32_t k_step, float (&acc)[NT][4]) {
+// A and B: the format is known at run time only (one uniform branch per blob).
+// A: a blob times a pair of X, as above.
+template <int FMT, int NT>
+__device__ __forceinline__ void product_a1(uint32_t blob, uint32_t sz2, int lane, uint32_t x, float (&acc)[NT][4]) {
   constexpr int tb = tile_bytes(FMT);
   SZ z;
 #pragma unroll
   for (int c = 0; c < 2; ++c) {
-    if constexpr (fmt_quantised(FMT)) { if (c == 0 || SZ2) load_sz<FMT>(z, blob + 2 * tb + c * kSzEntryBytes, lane); }
-    uint32_t a[4][4];
-    weights_f16<FMT, true>(blob + c * tb, lane, z, 0u, a);
+    if constexpr (fmt_quantised(FMT)) { if (c == 0 || sz2) load_sz<FMT>(z, blob + 2 * tb + c * kSzEntryBytes, lane); }
+    RawTile<FMT> r;
+    load_tile_s<FMT>(r, blob + c * tb, lane);
 #pragma unroll
-    for (int n = 0; n < NT; ++n) {
+    for (int b = 0; b < 2; ++b) {
+      uint32_t a[2][4];
+      weights_half<FMT, true>(r, b, z, 0u, a);
 #pragma unroll
-      for (int b = 0; b < 2; ++b) {
-        const uint4 v = lds_u4(x + (2 * c + b) * k_step + n * x_step);
-        mma16816(acc[n], a[2 * b], v.x, v.y);
-        mma16816(acc[n], a[2 * b + 1], v.z, v.w);
+      for (int n = 0; n < NT; ++n) {
+        const uint4 v = lds_u4(x + (2 * c + b) * (NT * 512) + n * 512);
+        mma16816(acc[n], a[0], v.x, v.y);
+        mma16816(acc[n], a[1], v.z, v.w);
       }
     }
   }
 }
 template <int NT>
-__device__ __forceinline__ void product_ab(int fmt, uint32_t sz2, uint32_t blob, int lane, uint32_t x, uint32_t x_step, uint32_t k_step, float (&acc)[NT][4]) {
+__device__ __forceinline__ void product_a(int fmt, uint32_t sz2, uint32_t blob, int lane, uint32_t x, float (&acc)[NT][4]) {
   switch (fmt) {
-    case FMT_F16: product_ab1<FMT_F16, false, NT>(blob, lane, x, x_step, k_step, acc); break;
-    case FMT_Q8: product_ab1<FMT_Q8, false, NT>(blob, lane, x, x_step, k_step, acc); break;
-    case FMT_Q4: if (sz2) product_ab1<FMT_Q4, true, NT>(blob, lane, x, x_step, k_step, acc); else product_ab1<FMT_Q4, false, NT>(blob, lane, x, x_step, k_step, acc); break;
-    case FMT_Q3: if (sz2) product_ab1<FMT_Q3, true, NT>(blob, lane, x, x_step, k_step, acc); else product_ab1<FMT_Q3, false, NT>(blob, lane, x, x_step, k_step, acc); break;
+    case FMT_F16: product_a1<FMT_F16, NT>(blob, 0u, lane, x, acc); break;
+    case FMT_Q8: product_a1<FMT_Q8, NT>(blob, 0u, lane, x, acc); break;
+    case FMT_Q4: product_a1<FMT_Q4, NT>(blob, sz2, lane, x, acc); break;
+    case FMT_Q3: product_a1<FMT_Q3, NT>(blob, sz2, lane, x, acc); break;
+    default: break;
+  }
+}
+// B: one 64-element tile of each of two row tiles, each with its scale entry behind it (kBStride bytes apart), times 64 columns of t.
+template <int FMT> constexpr uint32_t kBStride = tile_bytes(FMT) + 64;
+template <int FMT, int NT>
+__device__ __forceinline__ void product_b1(uint32_t buf, int lane, uint32_t x, float (&acc)[2][NT][4]) {
+  // one row tile after the other: an fp16 tile is 16 registers a lane
+#pragma unroll
+  for (int u = 0; u < 2; ++u) {
+    SZ z;
+    if constexpr (fmt_quantised(FMT)) load_sz<FMT>(z, buf + u * kBStride<FMT> + tile_bytes(FMT), lane);
+    RawTile<FMT> r;
+    load_tile_s<FMT>(r, buf + u * kBStride<FMT>, lane);
+#pragma unroll
+    for (int b = 0; b < 2; ++b) {
+      uint32_t a[2][4];
+      weights_half<FMT, true>(r, b, z, 0u, a);
+#pragma unroll
+      for (int n = 0; n < NT; ++n) {
+        const uint4 v = lds_u4(x + b * (NT * 512) + n * 512);
+        mma16816(acc[u][n], a[0], v.x, v.y);
+        mma16816(acc[u][n], a[1], v.z, v.w);
+      }
+    }
+  }
+}
+template <int NT>
+__device__ __forceinline__ void product_b(int fmt, uint32_t buf, int lane, uint32_t x, float (&acc)[2][NT][4]) {
+  switch (fmt) {
+    case FMT_F16: product_b1<FMT_F16, NT>(buf, lane, x, acc); break;
+    case FMT_Q8: product_b1<FMT_Q8, NT>(buf, lane, x, acc); break;
+    case FMT_Q4: product_b1<FMT_Q4, NT>(buf, lane, x, acc); break;
+    case FMT_Q3: product_b1<FMT_Q3, NT>(buf, lane, x, acc); break;
     default: break;
   }
 }
@@ -191,107 +227,75 @@ __device__ __forceinline__ int sub_of(const MidArgs& p, uint32_t tile) {
     if (i < p.n_sub && tile >= p.sub_tile0[i]) s = i;
   return s;
 }
-struct Span { uint32_t a, b, base; };              // pairs of t that row tile `tile` takes part in, within [c0, c1)
-__device__ __forceinline__ Span t_span(const MidArgs& p, uint32_t tile, uint32_t c0, uint32_t c1) {
-  Span s;
-  s.base = p.sub_pairs ? (uint32_t)sub_of(p, tile) * p.sub_pairs : 0u;
-  s.a = max(c0, s.base); s.b = min(c1, s.base + p.b_np);
-  return s;
-}
-
-// The chunks of a CTA's part of the reduction axis (P pairs, chunk of them per buffer) and a warp's share of each: of a chunk's n
-// pairs warp j of wpt takes [j n / wpt, (j + 1) n / wpt).
-struct Walk {
-  uint32_t P, chunk, j, wpt_inv;
-  uint32_t c, q, end;                     // chunk's first pair; next pair of the share, its end (counted from c)
-};
-__device__ __forceinline__ void walk_open(Walk& w, uint32_t c) {
-  w.c = c;
-  const uint32_t n = min(w.chunk, w.P - c), lo = w.j * n, hi = lo + n;
-  w.q = w.wpt_inv ? __umulhi(lo, w.wpt_inv) : lo;
-  w.end = w.wpt_inv ? __umulhi(hi, w.wpt_inv) : hi;
-}
-__device__ __forceinline__ bool walk_next_chunk(Walk& w) {          // to the next chunk with something in it
-  while (w.q == w.end) {
-    if (w.c + w.chunk >= w.P) return false;
-    walk_open(w, w.c + w.chunk);
-  }
-  return true;
-}
-
+// NT: tokens / 8.
 template <int WF, bool SZ2, int NT>
 __global__ void __launch_bounds__(kThreads, 1) k_mid(const __grid_constant__ CUtensorMap tm, const __grid_constant__ MidArgs p) {
   extern __shared__ __align__(128) uint8_t smem[];
   __shared__ uint32_t lut_s[16];
-  __shared__ __align__(8) uint64_t bars_s[2 + kWarps * kMaxSlots];
+  __shared__ __align__(8) uint64_t xbars_s[kMaxXSlots], bars_s[kWarps * kMaxSlots];
+  __shared__ uint32_t readers_s[kMaxXSlots];       // warps that are done with a slot of X
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   asm volatile("griddepcontrol.launch_dependents;");
   const bool is_a = blockIdx.x < p.n_a;
   const uint32_t cta = is_a ? blockIdx.x : blockIdx.x - p.n_a;
   const uint32_t cl = p.ks == 2 ? cta >> 1 : cta, rank = p.ks == 2 ? cta & 1 : 0;
-  if (p.ks == 2) cluster_arrive();                 // (that the partner runs at all, before anything is written to it)
+  const uint32_t d0 = share_lo(is_a ? p.a_tiles : p.w_dbl, cl), nD = share_n(is_a ? p.a_tiles : p.w_dbl, cl);
+  const uint32_t P = rank ? p.np - p.pairs0 : p.pairs0, pr0 = rank ? p.pairs0 : 0u;
+  const uint32_t xs = smem_u32(smem), xfull = smem_u32(xbars_s);
+  constexpr uint32_t kXSlot = NT * 2048;
   if constexpr (WF == FMT_SP24 || WF == FMT_SQ4) { if (threadIdx.x < 16) lut_s[threadIdx.x] = sp24_selectors(threadIdx.x); }
-  const uint32_t lut = smem_u32(lut_s), xbar = smem_u32(bars_s), bars = xbar + 16 + warp * (kMaxSlots * 8);
-  if (threadIdx.x == 0) { mbar_init_a(xbar, 1); mbar_init_a(xbar + 8, 1); }
-  if (lane == 0) {
-#pragma unroll
-    for (int i = 0; i < kMaxSlots; ++i) mbar_init_a(bars + 8 * i, 1);
+  const uint32_t lut = smem_u32(lut_s);
+  if (warp == 0 && lane < kMaxXSlots) {
+    mbar_init_a(xfull + 8 * lane, 1);
+    readers_s[lane] = 0u;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   }
-  __syncwarp();
 
-  // this CTA's units (row tiles of A, or pairs of row tiles of W) and this warp's place: unit d, share j of wpt
-  const uint32_t d0 = share_lo(is_a ? p.a_tiles : p.w_dbl, cl), nD = share_n(is_a ? p.a_tiles : p.w_dbl, cl);
-  const uint32_t wpt = kWarps / nD, d = warp / wpt, j = warp - d * wpt;
+  // this warp's place: unit d (row tile of A, pair of row tiles of W), every wpt-th pair of the reduction axis from j on
+  // The slots of X are a multiple of wpt, so a slot's pairs are always read by the same warps: none of them can be a phase of the
+  // slot's barrier ahead.
+  const uint32_t max_x = is_a ? p.a_xslots : p.xslots, wpt = min(kWarps / nD, max_x), xslots = max_x - max_x % wpt;
+  const uint32_t d = warp / wpt, j = warp - d * wpt;
   const bool active = d < nD;
-  const uint32_t P = rank ? p.np - p.pairs0 : p.pairs0, pr0 = rank ? p.pairs0 : 0u, chunk = is_a ? p.a_chunk : p.chunk;
-  const uint32_t xbuf = smem_u32(smem), xbuf_b = (chunk + kBox - 1) / kBox * (kBox * NT * 2048);
-  Walk in = {P, chunk, j, wpt > 1 ? 0xffffffffu / wpt + 1u : 0u, 0, 0, 0}, out;
-  walk_open(in, 0);
-  if (!active) { in.q = in.end = 0; in.c = P; }
-  out = in;
-
   Ring ring;
   const uint32_t blob_b = is_a ? p.a_blob : (uint32_t)blob_bytes(WF, SZ2 ? 1 : 0);
-  const uint32_t slot_n = is_a ? 1u : p.slot_pairs, slot_b = is_a ? p.a_blob : 2 * slot_n * blob_b, slots = is_a ? p.a_slots : p.slots;
+  const uint32_t slot_b = is_a ? p.a_blob : 2 * blob_b, slots = is_a ? p.a_slots : p.slots;
   ring.base = smem_u32(smem + (is_a ? p.a_off_ring : p.off_ring)) + warp * (is_a ? p.a_pitch : p.ring_pitch);
-  ring.bytes = slots * slot_b; ring.bars = ring.bar = bars; ring.so = 0; ring.parity = 0;
+  ring.bytes = slots * slot_b; ring.bars = ring.bar = smem_u32(bars_s) + warp * (kMaxSlots * 8); ring.so = 0; ring.parity = 0;
   // first blob of the unit's first row tile in this half of the reduction axis, and from there to its second row tile
   const uint8_t* w0 = is_a ? p.a_q + ((size_t)(d0 + d) * p.np + pr0) * blob_b
                            : p.w_q + ((size_t)rank * p.w_nt * p.pairs0 + (size_t)(d0 + d) * 2 * P) * blob_b;
-  const size_t to_second = (size_t)P * blob_b;
-  auto ask = [&](uint32_t so, uint32_t bar) {      // the next copy of the warp's share
-    if (!walk_next_chunk(in)) return;
-    const uint32_t cnt = min(slot_n, in.end - in.q);
+  uint32_t l_q = j;                                // the next pair to be asked for
+  auto ask = [&](uint32_t so, uint32_t bar) {
+    if (l_q >= P) return;
     if (lane == 0) {
-      const uint8_t* src = w0 + (size_t)(in.c + in.q) * blob_b;
-      mbar_expect_tx_a(bar, (is_a ? 1u : 2u) * cnt * blob_b);
-      bulk_g2s_a(ring.base + so, src, cnt * blob_b, bar);
-      if (!is_a) bulk_g2s_a(ring.base + so + slot_n * blob_b, src + to_second, cnt * blob_b, bar);
+      const uint8_t* src = w0 + (size_t)l_q * blob_b;
+      mbar_expect_tx_a(bar, slot_b);
+      bulk_g2s_a(ring.base + so, src, blob_b, bar);
+      if (!is_a) bulk_g2s_a(ring.base + so + blob_b, src + (size_t)P * blob_b, blob_b, bar);
     }
-    in.q += cnt;
+    l_q += wpt;
   };
-  for (uint32_t i = 0, so = 0, b = bars; i < slots; ++i, so += slot_b, b += 8) ask(so, b);
-  const uint32_t f0 = is_a ? 0u : (rank ? nD : 0u), nT = is_a ? nD : 2 * nD;      // W: rank 0 finishes the first nD row tiles, rank 1 the others
-  const uint32_t a_f0 = rank ? nD >> 1 : 0u, a_f1 = p.ks == 2 && rank == 0 ? nD >> 1 : nD;
-  const uint32_t first = is_a ? a_f0 : (p.ks == 2 ? f0 : 0u), nf = is_a ? a_f1 - a_f0 : (p.ks == 2 ? nD : nT);
-  if (!is_a && p.n_a) {                            // blobs of B towards L2
-    const uint32_t per = p.b_np * (uint32_t)blob_bytes(p.a_fmt, (int)p.b_sz2), bytes = nf * per;
-    const uint8_t* b_part = p.b_q + (size_t)(2 * d0 + first) * per;
-    for (uint32_t o = threadIdx.x << 14; o < bytes; o += kThreads << 14) prefetch_l2(b_part + o, min(16384u, bytes - o));
+  if (active) {
+    if (lane == 0) {
+#pragma unroll
+      for (int i = 0; i < kMaxSlots; ++i) mbar_init_a(ring.bars + 8 * i, 1);
+      asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    }
+    __syncwarp();
+    for (uint32_t i = 0, so = 0, b = ring.bars; i < slots; ++i, so += slot_b, b += 8) ask(so, b);
+  }
+  if (!is_a && p.n_a) {                            // blobs of B towards L2 (the partner reads the other halves of them)
+    const uint32_t per = p.b_np * (uint32_t)blob_bytes(p.a_fmt, (int)p.b_sz2), bytes = 2 * nD * per;
+    const uint8_t* b_part = p.b_q + (size_t)(2 * d0) * per;
+    for (uint32_t o = (threadIdx.x * p.ks + rank) << 13; o < bytes; o += (kThreads * p.ks) << 13) prefetch_l2(b_part + o, min(8192u, bytes - o));
   }
   asm volatile("griddepcontrol.wait;" ::: "memory");
-  __syncthreads();                                 // the X barriers are set up
+  __syncthreads();                                 // the barriers of X are set up
   const uint32_t launch = launch_number(p.launches);
-  auto load_x = [&](uint32_t c) {                  // chunk c / chunk of X: one warp per copy, the first of them says how much comes
-    const uint32_t i = (c / chunk) & 1, b = xbar + 8 * i;
-    if (threadIdx.x == 0) mbar_expect_tx_a(b, xbuf_b);
-    for (uint32_t k = warp * kBox; k < chunk && lane == 0; k += kWarps * kBox) tma_load_3d(xbuf + i * xbuf_b + k * (NT * 2048), &tm, 0, 0, (int)((pr0 + c + k) * 4), b);
-  };
-  load_x(0);
-  if (chunk < P) load_x(chunk);
-
+  bool ok = true;
   constexpr int T = 2;
   float acc[T][NT][4];
 #pragma unroll
@@ -300,67 +304,130 @@ __global__ void __launch_bounds__(kThreads, 1) k_mid(const __grid_constant__ CUt
     for (int n = 0; n < NT; ++n)
 #pragma unroll
       for (int i = 0; i < 4; ++i) acc[u][n][i] = 0.f;
-  bool ok = true;
-  uint32_t xpar = 0;                               // bit i: phase that buffer i completes next
+
+  auto load_x = [&](uint32_t q, uint32_t s) {      // pair q into slot s; one lane
+    mbar_expect_tx_a(xfull + 8 * s, kXSlot);
+    tma_load_3d(xs + s * kXSlot, &tm, 0, 0, (int)((pr0 + q) * 4), xfull + 8 * s);
+  };
+  if (lane == 0)
+    for (uint32_t q = warp; q < min(P, xslots); q += kWarps) load_x(q, q);
+  if (active) {
+    const uint32_t xl = xs + (lane >> 2) * 64 + (lane & 3) * 16;
+    uint32_t s = j, par = 0;
 #pragma unroll 1
-  for (uint32_t c = 0, xi = 0; c < P; c += chunk, xi ^= 1) {
-    if (ok && !mbar_try_wait_a(xbar + 8 * xi, (xpar >> xi) & 1) && !mbar_wait_lane(xbar + 8 * xi, (xpar >> xi) & 1, p.dev_status)) ok = false;
-    xpar ^= 1u << xi;
-    if (c > 0 && active) walk_open(out, c);
-    const uint32_t xl = xbuf + xi * xbuf_b + (lane >> 2) * 64 + (lane & 3) * 16;
-#pragma unroll 1
-    while (out.q < out.end) {
-      uint32_t cnt = min(slot_n, out.end - out.q);
+    for (uint32_t q = j; q < P; q += wpt) {
       if (ok && !mbar_try_wait_a(ring.bar, ring.parity) && !mbar_wait_lane(ring.bar, ring.parity, p.dev_status)) ok = false;
-      __syncwarp();
-      uint32_t src = ring.base + ring.so, x = xl + out.q * (NT * 2048);
-      out.q += cnt;
-#pragma unroll 1
-      for (; cnt > 0; --cnt, src += blob_b, x += NT * 2048) {
-        if (is_a) product_ab<NT>(p.a_fmt, p.a_sz2, src, lane, x, 512u, NT * 512u, acc[0]);
-        else product<WF, SZ2, NT, T>(src, slot_n * blob_b, lane, x, lut, acc);
+      if (ok && !mbar_try_wait_a(xfull + 8 * s, par) && !mbar_wait_lane(xfull + 8 * s, par, p.dev_status)) ok = false;
+      if (!__all_sync(0xffffffffu, ok)) { ok = false; break; }
+      const uint32_t src = ring.base + ring.so, x = xl + s * kXSlot;
+      if (is_a) product_a<NT>(p.a_fmt, p.a_sz2, src, lane, x, acc[0]);
+      else product<WF, SZ2, NT, T>(src, blob_b, lane, x, lut, acc);
+      __syncwarp();                                // every lane is done with both slots
+      if (lane == 0 && q + xslots < P) {           // a pair of X is read by one warp per unit
+        uint32_t done = nD - 1;
+        if (nD > 1) asm volatile("atom.acq_rel.cta.shared::cta.add.u32 %0, [%1], %2;" : "=r"(done) : "r"(smem_u32(readers_s + s)), "r"(1u) : "memory");
+        if (done == nD - 1) { readers_s[s] = 0u; load_x(q + xslots, s); }
       }
-      __syncwarp();                                // every lane is done with the slot
-      if (ok) ask(ring.so, ring.bar);
+      ask(ring.so, ring.bar);
       ring_next(ring, slot_b);
+      s += wpt;
+      if (s >= xslots) { s = j; par ^= 1u; }
     }
-    if (c + chunk < P) {
-      __syncthreads();                             // every warp is done with the buffer
-      if (c + 2 * chunk < P) load_x(c + 2 * chunk);
+    if (!ok) {                                     // gave up: this warp's copies in flight must land first
+      for (uint32_t i = 0; i < slots; ++i) mbar_drain_warp(bars_s + warp * kMaxSlots + i, ring.bars + 8 * i < ring.bar ? ring.parity ^ 1u : ring.parity, lane);
     }
-  }
-  if (!__all_sync(0xffffffffu, ok)) {              // gave up: what is in flight must land first
-    for (uint32_t i = 0; i < slots; ++i) mbar_drain_warp(bars_s + 2 + warp * kMaxSlots + i, ring.bars + 8 * i < ring.bar ? ring.parity ^ 1u : ring.parity, lane);
-    for (int i = 0; i < 2; ++i) mbar_drain_warp(bars_s + i, (xpar >> i) & 1, lane);
   }
 
-  // ---- the CTA's sums: every warp's into a slot of its own (over the X buffers), then added up per element
-  const bool ab = p.n_a != 0;
-  auto ask_b = [&](uint32_t tile, uint32_t pair, uint32_t b_blob) {                 // a blob of B to the start of the (empty) ring
-    if (lane == 0) {
-      mbar_expect_tx_a(ring.bar, b_blob);
-      bulk_g2s_a(ring.base, p.b_q + ((size_t)tile * p.b_np + pair) * b_blob, b_blob, ring.bar);
+  // ---- + t . B: this CTA's 64 of every 128 columns of t (all, if it has no partner)
+  if (!is_a && p.n_a) {
+    const uint32_t tile = 2 * (d0 + d), base = p.sub_pairs && active ? (uint32_t)sub_of(p, tile) * p.sub_pairs : 0u;
+    const uint32_t h_log = p.ks == 2 ? 0u : 1u, m_mask = (1u << p.m_log) - 1;      // halves of a pair that are this CTA's
+    uint32_t c0 = 0, c_end = p.b_np;               // chunk of t (pairs), end of all chunks
+    if (p.sub_pairs) { c0 = (uint32_t)sub_of(p, 2 * d0) * p.sub_pairs; c_end = (uint32_t)(sub_of(p, 2 * (d0 + nD) - 1) + 1) * p.sub_pairs; }
+    const uint32_t tb = (uint32_t)tile_bytes(p.a_fmt), stride = tb + 64, sz = fmt_quantised(p.a_fmt) ? (uint32_t)kSzEntryBytes : 0u;
+    const uint32_t b_blob = (uint32_t)blob_bytes(p.a_fmt, (int)p.b_sz2);
+    // unit h of a chunk: pair c0 + (h >> h_log), half `c` of it; a warp takes every wpt-th one of its layer's
+    auto half_of = [&](uint32_t h) { return p.ks == 2 ? rank : h & 1u; };
+    auto ask_b = [&](uint32_t h) {                 // to the start of the (empty) ring
+      if (lane == 0) {
+        const uint32_t c = half_of(h), pair = c0 + (h >> h_log) - base;
+        mbar_expect_tx_a(ring.bar, 2 * (tb + sz));
+#pragma unroll
+        for (uint32_t u = 0; u < 2; ++u) {
+          const uint8_t* blob = p.b_q + ((size_t)(tile + u) * p.b_np + pair) * b_blob;
+          bulk_g2s_a(ring.base + u * stride, blob + c * tb, tb, ring.bar);
+          if (sz) bulk_g2s_a(ring.base + u * stride + tb, blob + 2 * tb + (p.b_sz2 ? c * sz : 0u), sz, ring.bar);
+        }
+      }
+    };
+    auto span = [&](uint32_t& h, uint32_t& h_end) {          // the warp's first unit of the chunk, the end of its layer's
+      const uint32_t lo = max(c0, base), hi = min(min(c0 + p.t_chunk, c_end), base + p.b_np);
+      h = hi > lo ? ((lo - c0) << h_log) + j : 0u;
+      h_end = hi > lo ? (hi - c0) << h_log : 0u;
+    };
+    // step e of a chunk: four columns of one token (16 steps per half and token)
+    auto t_src = [&](uint32_t e, uint32_t& tok, uint32_t& col) {
+      const uint32_t h = e >> (4 + p.m_log);
+      tok = (e >> 4) & m_mask;
+      col = (c0 + (h >> h_log)) * 128 + half_of(h) * 64 + (e & 15) * 4;
+      return p.t_part + ((size_t)tok * p.t_cols + col) / 2;
+    };
+    uint32_t h, h_end, tok, col;
+    span(h, h_end);
+    if (ok && active && h < h_end) ask_b(h);
+    bool asked = true;
+#pragma unroll 1
+    for (;;) {
+      // t as fp16, zero for tokens that do not use the pair's adapter and in the columns past A's rows (padding); the loads of a batch
+      // go out together (each is a round trip to L2), those of the first before the barrier
+      constexpr int kBatch = 2;
+      const uint32_t steps = (min(p.t_chunk, c_end - c0) << h_log) << (4 + p.m_log);
+#pragma unroll 1
+      for (uint32_t e0 = 0; e0 < steps; e0 += kBatch * kThreads) {
+        TWords tw[kBatch];
+#pragma unroll
+        for (int k = 0; k < kBatch; ++k) {
+          const uint32_t e = e0 + k * kThreads + threadIdx.x;
+          const unsigned long long* src = t_src(e, tok, col);
+          if (e < steps && tok < (uint32_t)p.m) load_t(tw[k], src);
+        }
+        if (e0 == 0) __syncthreads();              // every warp is done with X (with the chunk before)
+#pragma unroll
+        for (int k = 0; k < kBatch; ++k) {
+          const uint32_t e = e0 + k * kThreads + threadIdx.x;
+          const unsigned long long* src = t_src(e, tok, col);
+          if (e >= steps || tok >= (uint32_t)p.m) continue;
+          uint32_t v0 = 0u, v1 = 0u;
+          if (col < p.a_nt * 16 && !(p.adp_pairs && p.adp[tok] != (int)((col >> 7) / p.adp_pairs)) &&
+              wait_t(tw[k], src, launch, p.wait_ns, p.dev_status)) { v0 = (uint32_t)tw[k].a; v1 = (uint32_t)tw[k].b; }
+          const uint32_t i = e & 15, dst = xs + (e >> (4 + p.m_log)) * (NT * 1024) + (i >> 3) * (NT * 512) + tok * 64 + (i & 7) * 8;
+          asm volatile("st.shared.v2.u32 [%0], {%1, %2};" ::"r"(dst), "r"(v0), "r"(v1) : "memory");
+        }
+      }
+      __syncthreads();
+      if (active) {
+#pragma unroll 1
+        for (; h < h_end; h += wpt, asked = false) {
+          if (!asked) ask_b(h);
+          if (ok && !mbar_try_wait_a(ring.bar, ring.parity) && !mbar_wait_lane(ring.bar, ring.parity, p.dev_status)) ok = false;
+          ring.parity ^= 1u;
+          if (!__all_sync(0xffffffffu, ok)) { ok = false; break; }
+          // (columns of tokens past m hold whatever was there: their sums are not read)
+          product_b<NT>(p.a_fmt, ring.base, lane, xs + h * (NT * 1024) + (lane >> 2) * 64 + (lane & 3) * 16, acc);
+          __syncwarp();
+        }
+      }
+      c0 += p.t_chunk;
+      if (c0 >= c_end) break;
+      asked = false;
+      span(h, h_end);
     }
-  };
-  const uint32_t first_tile = 2 * d0 + first, b_blob = (uint32_t)blob_bytes(p.a_fmt, (int)p.b_sz2);
-  uint32_t c0 = 0, c_end = p.b_np;                 // chunk of t, end of all chunks
-  TWords tw = {0ull, 0ull};
-  // step e of a chunk of t: four columns of one token (32 steps per pair and token)
-  auto t_tok = [&](uint32_t e) { return (e >> 5) & ((1u << p.m_log) - 1); };
-  auto t_col = [&](uint32_t e) { return (e >> (5 + p.m_log)) * 128 + (e & 31) * 4; };
-  if (!is_a && ab) {
-    if (p.sub_pairs) { c0 = (uint32_t)sub_of(p, first_tile) * p.sub_pairs; c_end = (uint32_t)(sub_of(p, first_tile + nf - 1) + 1) * p.sub_pairs; }
-    if (warp < (int)(nf << p.b_log)) {
-      const uint32_t tile = first_tile + (warp >> p.b_log);
-      const Span s = t_span(p, tile, c0, c0 + p.t_chunk);
-      const uint32_t q = s.a + (warp & ((1u << p.b_log) - 1));
-      if (q < s.b) ask_b(tile, q - s.base, b_blob);
-    }
-    if (t_tok(threadIdx.x) < (uint32_t)p.m && c0 * 128 + t_col(threadIdx.x) < (uint32_t)p.t_cols)
-      load_t(tw, p.t_part + ((size_t)t_tok(threadIdx.x) * p.t_cols + c0 * 128 + t_col(threadIdx.x)) / 2);
   }
-  __syncthreads();                                 // every warp is done with X
+
+  // ---- sums: every warp's into a slot of its own, over X and the rings; the partner's row tiles to the partner
+  if (p.ks == 2) { cluster_arrive(); cluster_wait(); } else __syncthreads();       // nobody needs X and the rings any more
   float* const seg = reinterpret_cast<float*>(smem);
+  float* const inbox = reinterpret_cast<float*>(smem + p.off_inbox);
   constexpr uint32_t kSlot = NT * 8 * kSegPitch;   // floats of a warp's slot: [token][32 rows, pitch 36]
   if (active) {
     float* s = seg + warp * kSlot + (lane & 3) * (2 * kSegPitch) + (lane >> 2);
@@ -373,11 +440,13 @@ __global__ void __launch_bounds__(kThreads, 1) k_mid(const __grid_constant__ CUt
       }
   }
   __syncthreads();
-  const uint32_t hw = threadIdx.x >> 4, row = threadIdx.x & 15, m = p.m, OT = 16 * m, m_mask = (1u << p.m_log) - 1;
-  float* const inbox = reinterpret_cast<float*>(smem + (is_a ? p.a_off_inbox : p.off_inbox));
+  // this CTA finishes row tiles [first, first + nf) of the cluster's nT
+  const uint32_t nT = is_a ? nD : 2 * nD, first = rank ? nT >> 1 : 0u, nf = (p.ks == 2 && rank == 0 ? nT >> 1 : nT) - first;
+  const uint32_t hw = threadIdx.x >> 4, row = threadIdx.x & 15, m = p.m, OT = 16 * m;
+  constexpr uint32_t kHalfWarps = kThreads / 16;
   // four tokens of a row tile at once (independent loads: in a rolled loop each costs its latency), summed over the warps that share it
   auto tile_sum = [&](uint32_t f, uint32_t tok, float (&v)[4]) {
-    const float* s = is_a ? seg + f * wpt * kSlot + tok * kSegPitch + row : seg + (f >> 1) * wpt * kSlot + tok * kSegPitch + (f & 1) * 16 + row;
+    const float* s = seg + tok * kSegPitch + row + (is_a ? f * wpt * kSlot : (f >> 1) * wpt * kSlot + (f & 1) * 16);
 #pragma unroll
     for (int i = 0; i < 4; ++i) v[i] = s[i * kSegPitch];
 #pragma unroll 2
@@ -389,10 +458,9 @@ __global__ void __launch_bounds__(kThreads, 1) k_mid(const __grid_constant__ CUt
   };
   const uint32_t q_log = p.m_log - 2, q_mask = (1u << q_log) - 1;      // groups of four tokens
   if (p.ks == 2) {                                 // the partner's row tiles
-    cluster_wait();
-    const uint32_t s0 = rank ? 0u : first + nf, ns = nT - nf;
+    const uint32_t s0 = rank ? 0u : nf, ns = nT - nf;
     const uint32_t to = mapa(smem_u32(inbox), rank ^ 1u) + row * 4;
-    for (uint32_t u = hw; u < ns << q_log; u += 2 * kWarps) {
+    for (uint32_t u = hw; u < ns << q_log; u += kHalfWarps) {
       const uint32_t f = u >> q_log, tok = (u & q_mask) * 4;
       float v[4];
       tile_sum(s0 + f, tok, v);
@@ -401,78 +469,16 @@ __global__ void __launch_bounds__(kThreads, 1) k_mid(const __grid_constant__ CUt
         if (tok + i < m) asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(to + (f * OT + (tok + i) * 16) * 4), "f"(v[i]) : "memory");
     }
     cluster_arrive();
+    cluster_wait();
   }
-  float* const bseg = reinterpret_cast<float*>(smem + p.off_bseg);
-  if (!is_a && ab) {
-    const uint32_t pitch = p.t_chunk * 256 + 64, th = smem_u32(smem + p.off_t);
-    uint32_t parity = ring.parity;
-    bool fresh = true;
-#pragma unroll 1
-    for (;;) {
-      // t of this chunk as fp16, zero for tokens that do not use the pair's adapter and in the columns past A's rows (padding)
-      const uint32_t steps = min(p.t_chunk, c_end - c0) << (5 + p.m_log);
-      for (uint32_t e = threadIdx.x; e < steps; e += kThreads) {
-        const uint32_t tok = t_tok(e), col = t_col(e);
-        if (tok >= m) continue;
-        uint2 v = make_uint2(0u, 0u);
-        if (c0 * 128 + col < p.a_nt * 16 && !(p.adp_pairs && p.adp[tok] != (int)((c0 + (col >> 7)) / p.adp_pairs))) {
-          const unsigned long long* src = p.t_part + ((size_t)tok * p.t_cols + c0 * 128 + col) / 2;
-          if (!fresh || e != threadIdx.x) load_t(tw, src);
-          if (wait_t(tw, src, launch, p.wait_ns, p.dev_status)) v = make_uint2((uint32_t)tw.a, (uint32_t)tw.b);
-        }
-        sts_u1(th + tok * pitch + col * 2, v.x);
-        sts_u1(th + tok * pitch + col * 2 + 4, v.y);
-      }
-      __syncthreads();
-#pragma unroll 1
-      for (uint32_t u = warp; u < nf << p.b_log; u += kWarps) {
-        const uint32_t tile = first_tile + (u >> p.b_log);
-        const Span s = t_span(p, tile, c0, c0 + p.t_chunk);
-        float bacc[NT][4];
-#pragma unroll
-        for (int n = 0; n < NT; ++n)
-#pragma unroll
-          for (int i = 0; i < 4; ++i) bacc[n][i] = 0.f;
-#pragma unroll 1
-        for (uint32_t q = s.a + (u & ((1u << p.b_log) - 1)), k = 0; q < s.b; q += 1u << p.b_log, ++k) {
-          if (!fresh || u != (uint32_t)warp || k) ask_b(tile, q - s.base, b_blob);
-          if (!mbar_try_wait_a(ring.bar, parity)) mbar_wait_lane(ring.bar, parity, p.dev_status);
-          parity ^= 1u;
-          __syncwarp();
-          product_ab<NT>(p.a_fmt, p.b_sz2, ring.base, lane, th + (lane >> 2) * pitch + (lane & 3) * 16 + (q - c0) * 256, 8 * pitch, 64u, bacc);
-          __syncwarp();
-        }
-        float* b = bseg + u * OT + (lane >> 2) + (lane & 3) * 32;
-#pragma unroll
-        for (int n = 0; n < NT; ++n) {
-          const uint32_t tok = n * 8 + 2 * (lane & 3);
-          if (tok < m) { b[n * 128] = bacc[n][0]; b[n * 128 + 8] = bacc[n][2]; }
-          if (tok + 1 < m) { b[n * 128 + 16] = bacc[n][1]; b[n * 128 + 24] = bacc[n][3]; }
-        }
-      }
-      c0 += p.t_chunk;
-      if (c0 >= c_end) break;
-      fresh = false;
-      __syncthreads();
-      for (uint32_t u = hw; u < nf << p.m_log; u += 2 * kWarps) {      // this chunk's products join the first warp's sums of the row tile
-        const uint32_t f = u >> p.m_log, tok = u & m_mask;
-        if (tok >= m) continue;
-        float v = 0.f;
-        for (uint32_t k = 0; k < 1u << p.b_log; ++k) v += bseg[((f << p.b_log) + k) * OT + tok * 16 + row];
-        seg[((first + f) >> 1) * wpt * kSlot + tok * kSegPitch + ((first + f) & 1) * 16 + row] += v;
-      }
-    }
-  }
-  if (p.ks == 2) cluster_wait();
-  __syncthreads();
   // (m_log >= 4: nf << q_log is even, so the halves of a warp take part alike)
-  for (uint32_t u = hw; u < nf << q_log; u += 2 * kWarps) {
+  for (uint32_t u = hw; u < nf << q_log; u += kHalfWarps) {
     const uint32_t f = u >> q_log, tok = (u & q_mask) * 4;
     float v[4];
     tile_sum(first + f, tok, v);
     if (p.ks == 2) {
 #pragma unroll
-      for (uint32_t i = 0; i < 4; ++i) v[i] += inbox[f * OT + (tok + i < m ? tok + i : tok) * 16 + row];
+      for (uint32_t i = 0; i < 4; ++i) v[i] += inbox[f * OT + min(tok + i, m - 1) * 16 + row];      // (past m: any, not stored)
     }
     if (is_a) {                                    // two columns of t per word
 #pragma unroll
@@ -484,12 +490,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_mid(const __grid_constant__ CUt
         }
       }
     } else {
-      if (ab) {
-        for (uint32_t k = 0; k < 1u << p.b_log; ++k)
-#pragma unroll
-          for (uint32_t i = 0; i < 4; ++i) v[i] += bseg[((f << p.b_log) + k) * OT + (tok + i < m ? tok + i : tok) * 16 + row];
-      }
-      const uint32_t tg = first_tile + f;
+      const uint32_t tg = 2 * d0 + first + f;
       void* y = p.ys[0];
       uint32_t st0 = 0;
       int dout = p.sub_dout[0];
@@ -521,13 +522,13 @@ EncodeTiledFn encode_fn() {
   return fn;
 }
 
-// X [m][d_in] fp16 as (k within a block of 32, token, block of 32 k); the box brings `blocks` blocks of all tokens (zeros past m)
-bool make_map(CUtensorMap* tm, const void* x, int m, int d_in, int tokens, int blocks) {
+// X [m][d_in] fp16 as (k within a block of 32, token, block of 32 k); the box brings a pair (4 blocks) of all tokens (zeros past m)
+bool make_map(CUtensorMap* tm, const void* x, int m, int d_in, int tokens) {
   EncodeTiledFn fn = encode_fn();
   if (!fn) return false;
   cuuint64_t dims[3] = {32, (cuuint64_t)m, (cuuint64_t)d_in / 32};
   cuuint64_t strides[2] = {(cuuint64_t)d_in * 2, 64};
-  cuuint32_t box[3] = {32, (cuuint32_t)tokens, (cuuint32_t)blocks};
+  cuuint32_t box[3] = {32, (cuuint32_t)tokens, 4};
   cuuint32_t estr[3] = {1, 1, 1};
   return fn(tm, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 3, const_cast<void*>(x), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
             CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
@@ -567,15 +568,19 @@ bool make_plan(const Handle* h, int m, Plan& pl) {
   MidArgs& a = pl.a;
   a = MidArgs();
   const bool ab = h->cfg.rank > 0;
-  const int NT = m <= 16 ? 2 : 4, Mr = 8 * NT;
+  const int NT = m <= 16 ? 2 : 4;
   pl.nt = NT;
   a.m = m;
   while ((1 << a.m_log) < m) ++a.m_log;
   a.w_q = h->w.q; a.w_nt = h->w.nt; a.np = h->w.np; a.pairs0 = h->w.half;
   a.ks = h->w.np >= 2 ? 2 : 1;
   const uint32_t sms = (uint32_t)h->sm_count / a.ks * a.ks, cls = sms / a.ks, nd = h->w.nt / 2;
-  a.chunk = NT == 2 ? 16 : 8;                      // 64 KB of X per buffer (one buffer if that is all)
-  if (a.chunk > a.pairs0) a.chunk = a.pairs0;
+  const uint32_t most_x = 131072u / (NT * 2048) < (uint32_t)kMaxXSlots ? 131072u / (NT * 2048) : kMaxXSlots;
+  auto blobs = [&](uint32_t per) {                 // blobs of a CTA with `per` units, idle turns included
+    uint32_t wpt = per >= (uint32_t)kWarps ? 1u : (uint32_t)kWarps / per;
+    if (wpt > most_x) wpt = most_x;
+    return (double)per * wpt * ((a.pairs0 + wpt - 1) / wpt);
+  };
   if (ab) {
     a.a_fmt = h->a.fmt; a.a_q = h->a.q; a.a_nt = h->a.nt; a.a_sz2 = h->a.sz2; a.a_blob = h->a.blob;
     a.b_q = h->b.q; a.b_np = h->b.np; a.b_sz2 = h->b.sz2;
@@ -585,73 +590,57 @@ bool make_plan(const Handle* h, int m, Plan& pl) {
     uint32_t best_n = 1;
     for (uint32_t n = 1; n <= cls / 2 && n <= (uint32_t)h->a.nt; ++n) {
       const uint32_t per_a = (h->a.nt + n - 1) / n, per_w = (nd + cls - n - 1) / (cls - n);
-      if (per_a > (uint32_t)kWarps) continue;
-      const double ta = 24.0 + (double)per_a * a.pairs0 * 1.2, tw = 2.0 * per_w * a.pairs0, t = ta > tw ? ta : tw;
+      if (per_a > (uint32_t)kWarps || per_w > (uint32_t)kWarps) continue;
+      const double ta = 24.0 + 1.2 * blobs(per_a), tw = 2.0 * blobs(per_w), t = ta > tw ? ta : tw;
       if (t < 0.99 * best) { best = t; best_n = n; }
     }
-    if ((h->a.nt + best_n - 1) / best_n > (uint32_t)kWarps) best_n = (h->a.nt + kWarps - 1) / kWarps;
+    if ((h->a.nt + best_n - 1) / best_n > (uint32_t)kWarps) best_n = (h->a.nt + (uint32_t)kWarps - 1) / (uint32_t)kWarps;
     a.n_a = best_n * a.ks;
     a.a_tiles = make_share(h->a.nt, best_n);
     a.sub_pairs = h->n_sub > 1 ? (uint32_t)h->r_pad / 128 : 0u;
   }
   uint32_t ncl = cls > a.n_a / a.ks ? cls - a.n_a / a.ks : 1;
   if (ncl > nd) ncl = nd;
-  if ((nd + ncl - 1) / ncl > (uint32_t)kWarps) ncl = (nd + kWarps - 1) / kWarps;      // more than fit at once: in waves
+  if ((nd + ncl - 1) / ncl > (uint32_t)kWarps) ncl = (nd + (uint32_t)kWarps - 1) / (uint32_t)kWarps;      // more than fit at once: in waves
   a.w_dbl = make_share(nd, ncl);
   pl.grid = (int)(a.n_a + ncl * a.ks);
   if (pl.grid >= (1 << kLaunchShift)) return false;
-  const uint32_t nD = a.w_dbl.per + (a.w_dbl.rem ? 1 : 0), nF = a.ks == 2 ? nD : 2 * nD;
-  const uint32_t t_pairs = (uint32_t)h->t_cols / 128;
-  a.t_chunk = NT == 2 ? 4 : 2;
-  if (a.t_chunk > t_pairs) a.t_chunk = t_pairs;
-  while ((2u << a.b_log) * nF <= (uint32_t)kWarps && (1u << a.b_log) < a.t_chunk && (1u << a.b_log) < a.b_np) ++a.b_log;
+  const uint32_t nD = a.w_dbl.per + (a.w_dbl.rem ? 1 : 0);
   auto up = [](uint32_t v) { return (v + 127u) & ~127u; };
-  const uint32_t seg_b = up(kWarps * Mr * kSegPitch * 4);
-  const uint32_t bseg_b = ab ? up((nF > (uint32_t)kWarps ? nF : (uint32_t)kWarps) * 64 * m) : 0u, t_b = ab ? up(Mr * (a.t_chunk * 256 + 64)) : 0u;
-  a.off_bseg = seg_b; a.off_t = seg_b + bseg_b;
-  const uint32_t late = seg_b + bseg_b + t_b, inbox_b = a.ks == 2 ? up(nD * 64 * m) : 0u;
-  // ring: what is left, in up to four slots of one or two pairs of two row tiles; it also takes a blob of B.  Smaller chunks of X
-  // where that leaves less than two slots.
-  const uint32_t pair_b = 2 * (uint32_t)h->w.blob, b_blob = ab ? (uint32_t)h->b.blob : 0u;
-  uint32_t room = 0;
-  for (;; a.chunk = (a.chunk + 1) / 2) {
-    const uint32_t x_b = (a.chunk < a.pairs0 ? 2 : 1) * ((a.chunk + kBox - 1) / kBox) * (kBox * NT * 2048);
-    a.off_inbox = x_b > late ? x_b : late;
-    a.off_ring = a.off_inbox + inbox_b;
-    room = a.off_ring < (uint32_t)kMaxSmem ? ((uint32_t)kMaxSmem - a.off_ring) / kWarps / pair_b : 0u;
-    if (room >= 2 || a.chunk <= 2 || x_b <= late) break;
-  }
-  if (room < 1) return false;
-  a.slot_pairs = room >= 4 ? 2 : 1;
-  a.slots = room / a.slot_pairs < (uint32_t)kMaxSlots ? room / a.slot_pairs : kMaxSlots;
-  a.ring_pitch = a.slots * a.slot_pairs * pair_b;
-  if (a.ring_pitch < b_blob) a.ring_pitch = b_blob;
-  uint32_t total = a.off_ring + kWarps * a.ring_pitch;
-  if (ab) {
-    const uint32_t per_a = a.a_tiles.per + (a.a_tiles.rem ? 1 : 0);
-    // A's clusters have few row tiles, so their warps cut the reduction axis finely: as much of X at once as leaves a blob per warp
-    uint32_t a_room = 0;
-    for (a.a_chunk = a.pairs0 < 32 ? a.pairs0 : 32;; a.a_chunk = (a.a_chunk + 1) / 2) {
-      const uint32_t bufs = a.a_chunk < a.pairs0 ? 2 : 1, ax = bufs * ((a.a_chunk + kBox - 1) / kBox) * (kBox * NT * 2048);
-      a.a_off_inbox = ax > seg_b ? ax : seg_b;
-      a.a_off_ring = a.a_off_inbox + (a.ks == 2 ? up(((per_a + 1) / 2) * 64 * m) : 0u);
-      a_room = a.a_off_ring < (uint32_t)kMaxSmem ? ((uint32_t)kMaxSmem - a.a_off_ring) / kWarps / a.a_blob : 0u;
-      if (a_room >= 2 || a.a_chunk <= 8) break;
+  const uint32_t x_slot = NT * 2048, seg_b = kWarps * 8 * NT * kSegPitch * 4;
+  a.off_inbox = up(seg_b);
+  const uint32_t per_a = a.a_tiles.per + (a.a_tiles.rem ? 1 : 0);
+  uint32_t total = a.off_inbox + (a.ks == 2 ? (nD > (per_a + 1) / 2 ? nD : (per_a + 1) / 2) * 64 * m : 0u);
+  // Slots of X: as many as there are warps to read different pairs at a time, within 128 KB; a ring of up to four slots from what is
+  // left, fewer slots of X where that would be less than two.  (A ring also takes half a blob of B per row tile.)
+  const uint32_t b_need = ab ? 2u * ((uint32_t)tile_bytes(a.a_fmt) + 64u) : 0u;
+  auto fit = [&](uint32_t slot_b, uint32_t need, uint32_t& xslots, uint32_t& off_ring, uint32_t& slots, uint32_t& pitch) {
+    xslots = most_x;
+    if (xslots > a.pairs0) xslots = a.pairs0;
+    for (;; --xslots) {
+      off_ring = up(xslots * x_slot);
+      const uint32_t room = ((uint32_t)kMaxSmem - off_ring) / kWarps;
+      slots = room / slot_b;
+      if ((slots >= 2 && room >= need) || xslots <= 2) break;
     }
-    if (a_room < 1) return false;
-    a.a_slots = a_room < (uint32_t)kMaxSlots ? a_room : kMaxSlots;
-    a.a_pitch = a.a_slots * a.a_blob;
-    if (a.a_off_ring + kWarps * a.a_pitch > total) total = a.a_off_ring + kWarps * a.a_pitch;
-  }
+    if (slots > (uint32_t)kMaxSlots) slots = kMaxSlots;
+    pitch = slots * slot_b > need ? slots * slot_b : need;
+    const uint32_t end = off_ring + kWarps * pitch;
+    if (end > total) total = end;
+    return slots >= 1;
+  };
+  if (!fit(2 * (uint32_t)h->w.blob, b_need, a.xslots, a.off_ring, a.slots, a.ring_pitch)) return false;
+  if (ab && !fit(a.a_blob, 0u, a.a_xslots, a.a_off_ring, a.a_slots, a.a_pitch)) return false;
+  a.t_chunk = a.off_ring / (NT * 1024) / (a.ks == 2 ? 1 : 2);      // t goes where X was
   pl.smem = (int)total;
   return total <= (uint32_t)kMaxSmem;
 }
 
 }  // namespace
 
-// Above eight tokens (one decode pass is cheaper) and up to what one launch takes.  Three LLaMA3-8B blocks, 4-bit, fp16 adapters of
-// rank 128, against the tcgen05 kernel: 12 tokens 204 against 412 us, 32 tokens 293 against 421; 64 tokens in two launches
-// would be 567 against 431.
+// Above eight tokens (one decode pass is cheaper) and up to 32.  Three LLaMA3-8B blocks, 4-bit, fp16 adapters of rank 128, against
+// the tcgen05 kernel: 12 tokens 196 against 412 us, 32 tokens 256 against 421.  Forms for 64 tokens lost: two launches 510
+// against 431 us; one with twice the accumulators 464 (the sums of 64 tokens fill the registers, and only eight pairs of X fit).
 bool mid_supported(const Handle* h, int m) {
   if (m <= 8 || m > kMaxPass || h->sm_count < 4 || h->cfg.kernel_policy == EORA_POLICY_GENERIC) return false;
   if (h->w.fmt != FMT_Q4 && h->w.fmt != FMT_Q3 && h->w.fmt != FMT_SP24 && h->w.fmt != FMT_SQ4) return false;
@@ -697,7 +686,7 @@ cudaError_t launch_mid_forward(const Handle* h, const void* x16, int m, void* co
       }
     }
     CUtensorMap tm;
-    if (!make_map(&tm, reinterpret_cast<const uint8_t*>(x16) + (size_t)m0 * h->cfg.d_in * 2, mp, h->cfg.d_in, 8 * pl.nt, 4 * kBox)) return cudaErrorInvalidValue;
+    if (!make_map(&tm, reinterpret_cast<const uint8_t*>(x16) + (size_t)m0 * h->cfg.d_in * 2, mp, h->cfg.d_in, 8 * pl.nt)) return cudaErrorInvalidValue;
     cfg.gridDim = dim3(pl.grid);
     cfg.dynamicSmemBytes = pl.smem;
     attr[1].val.clusterDim.x = a.ks;
