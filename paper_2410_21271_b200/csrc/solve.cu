@@ -1,24 +1,30 @@
 // Offline EoRA solve (Algorithm 1, steps 1-6) on the GPU; the interface and the mathematics are in eora_solve.h.
 //
 //   1.  dW = W - W^                                                    (k_sub)
-//   2-4 the paper projects dW into the eigenspace of X~ X~^T, dW' = dW Q sqrt(L).  Only dW' dW'^T is needed here:
-//       G = X~ X~^T  (k x k),  T = dW G,  Mm = T dW^T = dW' dW'^T  (d x d)   (three fp32 contractions)
-//   5.  top-r eigenpairs (U', S'^2) of Mm by subspace iteration on m = r + oversample vectors:
-//         Y = Mm Q;  Q = orth(Y)  by Cholesky-QR (Gram matrix and factor in fp64);  repeated `iters` times, then a
-//         Rayleigh-Ritz step:  H = Q^T Mm Q  (m x m, fp64),  H = V diag(lam) V^T  by one-sided Jacobi in one CTA,
-//         U' = Q V[:, top r],  S' = sqrt(lam)
+//   2-4 the paper projects dW into the eigenspace of X~ X~^T, dW' = dW Q sqrt(L).  Only dW' dW'^T = P P^T with P = dW X~
+//       (d x n) is needed here.
+//   5.  top-r eigenpairs (U', S'^2) of P P^T by subspace iteration on m = r + oversample vectors:
+//         Y = C Q;  Q = orth(Y)  by Cholesky-QR (Gram matrix, factor and substitution in fp64);  repeated `iters` times.
+//       C is the smaller of P P^T (d x d) and P^T P (n x n), whose leading eigenvectors P carries into each other.  Then a
+//       Rayleigh-Ritz step in the d-dimensional basis Y:  H = (P^T Y)^T (P^T Y)  (m x m, fp64),  H = V diag(lam) V^T by
+//       one-sided Jacobi,  U' = Y V[:, top r],  S' = sqrt(lam)
 //   6.  B' = U' S',  A = S'^{-1} U'^T dW
 //
-// Every kernel here is plain fp32 / fp64 CUDA-core arithmetic: the large contractions are tiled SGEMMs
-// (128 x 128 x 16 tiles through shared memory, 8 x 8 outputs per thread; for the skinny products of the iteration
-// 32 x 160 tiles at the default width of 160 vectors, else 64 x 128); fp32 because the quality of the eigenvectors near the cut depends on the small differences
-// between neighbouring eigenvalues of Mm.  The (r + oversample)^2 problems run in fp64 in one CTA each.
+// Large contractions are tiled fp32 SGEMMs on the CUDA cores (fp32 because the quality of the eigenvectors near the cut
+// depends on the small differences between neighbouring eigenvalues); all matrices are padded with zeros to whole tiles, so
+// there is one form of each product.  The (r + oversample)^2 problems run in fp64.
+// Measured, 4096 x 4096 with 2048 calibration columns and rank 128: see k_sgemm_full and the kernels behind it.
 #include <cuda_runtime.h>
 #include <stdint.h>
 #include "../../include/eora_linear.h"
 #include "../../include/eora_solve.h"
 
 namespace {
+
+__device__ __forceinline__ void cluster_sync_all() {
+  asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+  asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
 
 // ------------------------------------------------------------------------------------------------ SGEMM
 constexpr int BM = 128, BN = 128, BKS = 16, PAD = 4;
@@ -82,26 +88,37 @@ __global__ void __launch_bounds__(256) k_sgemm(int M, int N, int P, const float*
   }
 }
 
+// Two fp32 fused multiply-adds per instruction (the pair of neighbouring columns).
+__device__ __forceinline__ void ffma2(float2& d, const float2& a, const float2& b) {
+  unsigned long long& dd = reinterpret_cast<unsigned long long&>(d);
+  asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(dd) : "l"(reinterpret_cast<const unsigned long long&>(a)), "l"(reinterpret_cast<const unsigned long long&>(b)));
+}
+
 // The same product for whole tiles (M, N multiples of 128, P of 16, rows 16-byte aligned): 16-byte global loads, the
-// next k-slice fetched into registers while the current one is multiplied.
-// TM: output rows per thread (8: tiles of 128 rows; 4: tiles of 64 rows, for products with few tiles).
-template <bool TA, bool TB, int TM>
-__global__ void __launch_bounds__(256) k_sgemm_full(int P, const float* __restrict__ A, int lda, const float* __restrict__ B, int ldb,
+// next k-slice fetched into registers while the current one is multiplied, 8 x 8 outputs per thread.
+// SYM: C = op(A) op(A)^T is symmetric; only the tiles on and below the diagonal are computed (grid: their number) and stored
+// to both places.
+template <bool TA, bool TB, bool SYM>
+__global__ void __launch_bounds__(256, 2) k_sgemm_full(int P, const float* __restrict__ A, int lda, const float* __restrict__ B, int ldb,
                                                     float* __restrict__ C, int ldc) {
-  constexpr int BMT = 16 * TM, NA = TM / 4;          // tile rows; 16-byte pieces of the A tile per thread
-  __shared__ __align__(16) float As[2][BKS][BMT + PAD];
+  __shared__ __align__(16) float As[2][BKS][BM + PAD];
   __shared__ __align__(16) float Bs[2][BKS][BN + PAD];
   const int t = threadIdx.x, tx = t & 15, ty = t >> 4;
-  const int m0 = blockIdx.y * BMT, n0 = blockIdx.x * BN;
+  int by = blockIdx.y, bx = blockIdx.x;
+  if (SYM) {                                         // tile number -> (row, column <= row)
+    by = (int)((sqrtf(8.f * bx + 1.f) - 1.f) * 0.5f);
+    while ((by + 1) * (by + 2) / 2 <= bx) ++by;
+    while (by * (by + 1) / 2 > bx) --by;
+    bx -= by * (by + 1) / 2;
+  }
+  const int m0 = by * BM, n0 = bx * BN;
   // this thread's two 16-byte pieces of each operand tile
-  // A not transposed: tile rows m (128) x 16 p: piece = (row, p4), 4 pieces per row;  transposed: A[p][m]: (p, m4), 32 per p
-  int a_r[NA], a_c[NA], b_r[2], b_c[2];
+  // not transposed A / transposed B: tile rows (128) x 16 p: piece = (row, p4), 4 pieces per row;  else (p, col4), 32 per p
+  int a_r[2], a_c[2], b_r[2], b_c[2];
 #pragma unroll
   for (int i = 0; i < 2; ++i) {
     const int e = t + 256 * i;
-    if (i < NA) {
-      if (TA) { a_r[i] = e / (BMT / 4); a_c[i] = (e % (BMT / 4)) * 4; } else { a_r[i] = e >> 2; a_c[i] = (e & 3) * 4; }
-    }
+    if (TA) { a_r[i] = e >> 5; a_c[i] = (e & 31) * 4; } else { a_r[i] = e >> 2; a_c[i] = (e & 3) * 4; }
     if (TB) { b_r[i] = e >> 2; b_c[i] = (e & 3) * 4; } else { b_r[i] = e >> 5; b_c[i] = (e & 31) * 4; }
   }
   auto load_a = [&](int p0, int i) -> float4 {
@@ -120,148 +137,208 @@ __global__ void __launch_bounds__(256) k_sgemm_full(int P, const float* __restri
     if (TB) { Bs[buf][b_c[i]][b_r[i]] = v.x; Bs[buf][b_c[i] + 1][b_r[i]] = v.y; Bs[buf][b_c[i] + 2][b_r[i]] = v.z; Bs[buf][b_c[i] + 3][b_r[i]] = v.w; }
     else *reinterpret_cast<float4*>(&Bs[buf][b_r[i]][b_c[i]]) = v;
   };
-  float acc[TM][8];
+  float2 acc[8][4];
 #pragma unroll
-  for (int i = 0; i < TM; ++i)
+  for (int i = 0; i < 8; ++i)
 #pragma unroll
-    for (int j = 0; j < 8; ++j) acc[i][j] = 0.f;
-  float4 ra[NA], rb[2];
+    for (int j = 0; j < 4; ++j) acc[i][j] = make_float2(0.f, 0.f);
+  float4 ra[2], rb[2];
 #pragma unroll
-  for (int i = 0; i < 2; ++i) { if (i < NA) ra[i] = load_a(0, i); rb[i] = load_b(0, i); }
+  for (int i = 0; i < 2; ++i) { ra[i] = load_a(0, i); rb[i] = load_b(0, i); }
 #pragma unroll
-  for (int i = 0; i < 2; ++i) { if (i < NA) store_a(0, i, ra[i]); store_b(0, i, rb[i]); }
+  for (int i = 0; i < 2; ++i) { store_a(0, i, ra[i]); store_b(0, i, rb[i]); }
   __syncthreads();
   int buf = 0;
   for (int p0 = 0; p0 < P; p0 += BKS) {
     const bool more = p0 + BKS < P;
     if (more) {
 #pragma unroll
-      for (int i = 0; i < 2; ++i) { if (i < NA) ra[i] = load_a(p0 + BKS, i); rb[i] = load_b(p0 + BKS, i); }
+      for (int i = 0; i < 2; ++i) { ra[i] = load_a(p0 + BKS, i); rb[i] = load_b(p0 + BKS, i); }
     }
 #pragma unroll
     for (int p = 0; p < BKS; ++p) {
-      float a[8], b[8];
-      const float4 a0 = *reinterpret_cast<const float4*>(&As[buf][p][ty * 4]);
-      const float4 a1 = TM == 8 ? *reinterpret_cast<const float4*>(&As[buf][p][(BMT / 2) + ty * 4]) : a0;
+      const float4 a0 = *reinterpret_cast<const float4*>(&As[buf][p][ty * 4]), a1 = *reinterpret_cast<const float4*>(&As[buf][p][64 + ty * 4]);
       const float4 b0 = *reinterpret_cast<const float4*>(&Bs[buf][p][tx * 4]), b1 = *reinterpret_cast<const float4*>(&Bs[buf][p][64 + tx * 4]);
-      a[0] = a0.x; a[1] = a0.y; a[2] = a0.z; a[3] = a0.w; a[4] = a1.x; a[5] = a1.y; a[6] = a1.z; a[7] = a1.w;
-      b[0] = b0.x; b[1] = b0.y; b[2] = b0.z; b[3] = b0.w; b[4] = b1.x; b[5] = b1.y; b[6] = b1.z; b[7] = b1.w;
+      const float a[8] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w};
+      const float2 b[4] = {make_float2(b0.x, b0.y), make_float2(b0.z, b0.w), make_float2(b1.x, b1.y), make_float2(b1.z, b1.w)};
 #pragma unroll
-      for (int i = 0; i < TM; ++i)
+      for (int i = 0; i < 8; ++i) {
+        const float2 aa = make_float2(a[i], a[i]);
 #pragma unroll
-        for (int j = 0; j < 8; ++j) acc[i][j] = fmaf(a[i], b[j], acc[i][j]);
+        for (int j = 0; j < 4; ++j) ffma2(acc[i][j], aa, b[j]);
+      }
     }
     if (more) {
 #pragma unroll
-      for (int i = 0; i < 2; ++i) { if (i < NA) store_a(buf ^ 1, i, ra[i]); store_b(buf ^ 1, i, rb[i]); }
+      for (int i = 0; i < 2; ++i) { store_a(buf ^ 1, i, ra[i]); store_b(buf ^ 1, i, rb[i]); }
     }
     __syncthreads();
     buf ^= 1;
   }
 #pragma unroll
-  for (int i = 0; i < TM; ++i) {
-    const int gm = m0 + (i < 4 ? ty * 4 + i : (BMT / 2) + ty * 4 + i - 4);
-    float* row = C + (int64_t)gm * ldc + n0;
-    *reinterpret_cast<float4*>(row + tx * 4) = make_float4(acc[i][0], acc[i][1], acc[i][2], acc[i][3]);
-    *reinterpret_cast<float4*>(row + 64 + tx * 4) = make_float4(acc[i][4], acc[i][5], acc[i][6], acc[i][7]);
+  for (int i = 0; i < 8; ++i) {
+    float* row = C + (int64_t)(m0 + (i & 3) + ty * 4 + (i & 4) * 16) * ldc + n0;
+    *reinterpret_cast<float4*>(row + tx * 4) = make_float4(acc[i][0].x, acc[i][0].y, acc[i][1].x, acc[i][1].y);
+    *reinterpret_cast<float4*>(row + 64 + tx * 4) = make_float4(acc[i][2].x, acc[i][2].y, acc[i][3].x, acc[i][3].y);
+  }
+  if (SYM && by != bx) {
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+      float* row = C + (int64_t)(n0 + (j & 3) + tx * 4 + (j & 4) * 16) * ldc + m0;
+      const int q = j >> 1;
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const float4 v = (j & 1) ? make_float4(acc[4 * h][q].y, acc[4 * h + 1][q].y, acc[4 * h + 2][q].y, acc[4 * h + 3][q].y)
+                                 : make_float4(acc[4 * h][q].x, acc[4 * h + 1][q].x, acc[4 * h + 2][q].x, acc[4 * h + 3][q].x);
+        *reinterpret_cast<float4*>(row + 64 * h + ty * 4) = v;
+      }
+    }
   }
 }
 
-// C[M][160] = A[M][P] B[P][160] (nothing transposed; M a multiple of 32, P of 16, rows 16-byte aligned): the products of the
-// subspace iteration with its default width of 160 vectors.  Tiles of 32 rows x all 160 columns, so that a product
-// with 4096 rows is 128 CTAs and no flop goes into padding columns; 2 x 10 outputs per thread.
-constexpr int NQ = 160, BMQ = 32;
-__global__ void __launch_bounds__(256) k_sgemm_n160(int P, const float* __restrict__ A, int lda, const float* __restrict__ B, int ldb,
-                                                    float* __restrict__ C, int ldc) {
-  __shared__ __align__(16) float As[2][BKS][BMQ + PAD];
-  __shared__ __align__(16) float Bs[2][BKS][NQ + PAD];
+// Skinny products C[M][ldc] = op(A) B with B [P][ldb] of a few hundred columns (the iterates): M a multiple of 64, P of 16 times the
+// cluster size; opA[m][p] = TA ? A[p * lda + m] : A[m * lda + p].  A cluster owns a tile of 64 rows x 16 NC columns and splits P; the
+// partial sums meet in distributed shared memory and are added in a fixed order, so the result does not depend on timing.
+// 4 x NC outputs per thread (two instructions' worth of shared-memory reads per ten of arithmetic at NC = 10; 2 x 10 was bound
+// by the reads), and enough CTAs without padding columns: 2048 x 2048 x 160 are 32 tiles, 128 CTAs.
+template <int NC, bool TA>
+__global__ void __launch_bounds__(256) k_skinny(int P, const float* __restrict__ A, int lda, const float* __restrict__ B, int ldb,
+                                                float* __restrict__ C, int ldc) {
+  constexpr int W = 16 * NC, NP = NC / 2, RM = 64;
+  constexpr int BQ = (BKS * W / 4 + 255) / 256;      // 16-byte pieces of the B slice per thread
+  constexpr int kAb = 2 * BKS * (RM + PAD), kBb = 2 * BKS * (W + PAD), kSm = kAb + kBb > RM * W ? kAb + kBb : RM * W;
+  __shared__ __align__(16) float sm[kSm];
+  float (*As)[BKS][RM + PAD] = reinterpret_cast<float (*)[BKS][RM + PAD]>(sm);
+  float (*Bs)[BKS][W + PAD] = reinterpret_cast<float (*)[BKS][W + PAD]>(sm + kAb);
   const int t = threadIdx.x, tx = t & 15, ty = t >> 4;
-  const int m0 = blockIdx.x * BMQ;
-  // 16-byte pieces: A tile 32 rows x 16 p = 128 pieces (threads 0..127), B tile 16 p x 160 = 640 pieces (2.5 per thread)
-  const int a_r = (t & 127) >> 2, a_c = (t & 3) * 4;
-  int b_r[3], b_c[3];
-#pragma unroll
-  for (int i = 0; i < 3; ++i) { const int e = t + 256 * i; b_r[i] = e / (NQ / 4); b_c[i] = (e % (NQ / 4)) * 4; }
-  const bool has_a = t < 128, has_b2 = t + 512 < BKS * NQ / 4;
-  auto load_a = [&](int p0) -> float4 { return *reinterpret_cast<const float4*>(A + (int64_t)(m0 + a_r) * lda + p0 + a_c); };
-  auto load_b = [&](int p0, int i) -> float4 { return *reinterpret_cast<const float4*>(B + (int64_t)(p0 + b_r[i]) * ldb + b_c[i]); };
-  auto store_a = [&](int buf, const float4& v) {
-    As[buf][a_c][a_r] = v.x; As[buf][a_c + 1][a_r] = v.y; As[buf][a_c + 2][a_r] = v.z; As[buf][a_c + 3][a_r] = v.w;
+  const int ks = gridDim.x, rank = blockIdx.x, m0 = blockIdx.y * RM, n0 = blockIdx.z * W;
+  const int span = P / ks, lo = rank * span;
+  const int a_r = TA ? t >> 4 : t >> 2, a_c = TA ? (t & 15) * 4 : (t & 3) * 4;
+  auto load_a = [&](int p0) -> float4 {
+    return TA ? __ldg(reinterpret_cast<const float4*>(A + (int64_t)(p0 + a_r) * lda + m0 + a_c))
+              : __ldg(reinterpret_cast<const float4*>(A + (int64_t)(m0 + a_r) * lda + p0 + a_c));
   };
-  auto store_b = [&](int buf, int i, const float4& v) { *reinterpret_cast<float4*>(&Bs[buf][b_r[i]][b_c[i]]) = v; };
-  float acc[2][10];
+  auto store_a = [&](int buf, const float4& v) {
+    if (TA) *reinterpret_cast<float4*>(&As[buf][a_r][a_c]) = v;
+    else { As[buf][a_c][a_r] = v.x; As[buf][a_c + 1][a_r] = v.y; As[buf][a_c + 2][a_r] = v.z; As[buf][a_c + 3][a_r] = v.w; }
+  };
+  auto has_b = [&](int i) { return (i + 1) * 256 <= BKS * W / 4 || t + 256 * i < BKS * W / 4; };
+  auto load_b = [&](int p0, int i) -> float4 {
+    const int e = t + 256 * i;
+    return __ldg(reinterpret_cast<const float4*>(B + (int64_t)(p0 + e / (W / 4)) * ldb + n0 + (e % (W / 4)) * 4));
+  };
+  auto store_b = [&](int buf, int i, const float4& v) { const int e = t + 256 * i; *reinterpret_cast<float4*>(&Bs[buf][e / (W / 4)][(e % (W / 4)) * 4]) = v; };
+  // columns of a thread: four of every 64, two of a last 32
+  float2 acc[4][NP];
 #pragma unroll
-  for (int i = 0; i < 2; ++i)
+  for (int i = 0; i < 4; ++i)
 #pragma unroll
-    for (int j = 0; j < 10; ++j) acc[i][j] = 0.f;
-  float4 ra = make_float4(0.f, 0.f, 0.f, 0.f), rb[3];
-  if (has_a) ra = load_a(0);
+    for (int j = 0; j < NP; ++j) acc[i][j] = make_float2(0.f, 0.f);
+  float4 ra = load_a(lo), rb[BQ];
 #pragma unroll
-  for (int i = 0; i < 3; ++i) if (i < 2 || has_b2) rb[i] = load_b(0, i);
-  if (has_a) store_a(0, ra);
+  for (int i = 0; i < BQ; ++i) if (has_b(i)) rb[i] = load_b(lo, i);
+  store_a(0, ra);
 #pragma unroll
-  for (int i = 0; i < 3; ++i) if (i < 2 || has_b2) store_b(0, i, rb[i]);
+  for (int i = 0; i < BQ; ++i) if (has_b(i)) store_b(0, i, rb[i]);
   __syncthreads();
   int buf = 0;
-  for (int p0 = 0; p0 < P; p0 += BKS) {
-    const bool more = p0 + BKS < P;
+  for (int p0 = lo; p0 < lo + span; p0 += BKS) {
+    const bool more = p0 + BKS < lo + span;
     if (more) {
-      if (has_a) ra = load_a(p0 + BKS);
+      ra = load_a(p0 + BKS);
 #pragma unroll
-      for (int i = 0; i < 3; ++i) if (i < 2 || has_b2) rb[i] = load_b(p0 + BKS, i);
+      for (int i = 0; i < BQ; ++i) if (has_b(i)) rb[i] = load_b(p0 + BKS, i);
     }
 #pragma unroll
     for (int p = 0; p < BKS; ++p) {
-      const float2 a = *reinterpret_cast<const float2*>(&As[buf][p][ty * 2]);
-      const float4 b0 = *reinterpret_cast<const float4*>(&Bs[buf][p][tx * 4]), b1 = *reinterpret_cast<const float4*>(&Bs[buf][p][64 + tx * 4]);
-      const float2 b2 = *reinterpret_cast<const float2*>(&Bs[buf][p][128 + tx * 2]);
-      const float b[10] = {b0.x, b0.y, b0.z, b0.w, b1.x, b1.y, b1.z, b1.w, b2.x, b2.y};
+      const float4 a = *reinterpret_cast<const float4*>(&As[buf][p][ty * 4]);
+      float2 b[NP];
 #pragma unroll
-      for (int j = 0; j < 10; ++j) { acc[0][j] = fmaf(a.x, b[j], acc[0][j]); acc[1][j] = fmaf(a.y, b[j], acc[1][j]); }
+      for (int c = 0; c < NC / 4; ++c) {
+        const float4 v = *reinterpret_cast<const float4*>(&Bs[buf][p][64 * c + tx * 4]);
+        b[2 * c] = make_float2(v.x, v.y); b[2 * c + 1] = make_float2(v.z, v.w);
+      }
+      if (NC % 4) b[NP - 1] = *reinterpret_cast<const float2*>(&Bs[buf][p][64 * (NC / 4) + tx * 2]);
+      const float av[4] = {a.x, a.y, a.z, a.w};
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const float2 aa = make_float2(av[i], av[i]);
+#pragma unroll
+        for (int j = 0; j < NP; ++j) ffma2(acc[i][j], aa, b[j]);
+      }
     }
     if (more) {
-      if (has_a) store_a(buf ^ 1, ra);
+      store_a(buf ^ 1, ra);
 #pragma unroll
-      for (int i = 0; i < 3; ++i) if (i < 2 || has_b2) store_b(buf ^ 1, i, rb[i]);
+      for (int i = 0; i < BQ; ++i) if (has_b(i)) store_b(buf ^ 1, i, rb[i]);
     }
     __syncthreads();
     buf ^= 1;
   }
+  auto col = [&](int j) { return j / 2 < NC / 4 ? 64 * (j / 2) + tx * 4 + 2 * (j & 1) : 64 * (NC / 4) + tx * 2; };
+  if (ks == 1) {
 #pragma unroll
-  for (int i = 0; i < 2; ++i) {
-    float* row = C + (int64_t)(m0 + ty * 2 + i) * ldc;
-    *reinterpret_cast<float4*>(row + tx * 4) = make_float4(acc[i][0], acc[i][1], acc[i][2], acc[i][3]);
-    *reinterpret_cast<float4*>(row + 64 + tx * 4) = make_float4(acc[i][4], acc[i][5], acc[i][6], acc[i][7]);
-    *reinterpret_cast<float2*>(row + 128 + tx * 2) = make_float2(acc[i][8], acc[i][9]);
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+      for (int j = 0; j < NP; ++j) *reinterpret_cast<float2*>(C + (int64_t)(m0 + ty * 4 + i) * ldc + n0 + col(j)) = acc[i][j];
+    return;
+  }
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+#pragma unroll
+    for (int j = 0; j < NP; ++j) *reinterpret_cast<float2*>(sm + (ty * 4 + i) * W + col(j)) = acc[i][j];
+  cluster_sync_all();
+  const int per = RM / ks;                           // rows of the tile that this CTA adds up
+  const uint32_t base = (uint32_t)__cvta_generic_to_shared(sm) + rank * per * W * 4;
+  for (int e = t; e < per * W / 4; e += 256) {
+    float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int r = 0; r < ks; ++r) {
+      float4 u;
+      uint32_t a;
+      asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(base + 16 * e), "r"(r));
+      asm volatile("ld.shared::cluster.v4.f32 {%0,%1,%2,%3}, [%4];" : "=f"(u.x), "=f"(u.y), "=f"(u.z), "=f"(u.w) : "r"(a));
+      v.x += u.x; v.y += u.y; v.z += u.z; v.w += u.w;
+    }
+    *reinterpret_cast<float4*>(C + (int64_t)(m0 + rank * per + e / (W / 4)) * ldc + n0 + (e % (W / 4)) * 4) = v;
+  }
+  cluster_sync_all();                                // nobody leaves while its sums are being read
+}
+
+template <int NC, bool TA>
+cudaError_t launch_skinny(cudaStream_t st, int M, int P, const float* A, int lda, const float* B, int ldb, int N, float* C, int ldc) {
+  // as many CTAs per tile as there are SMs for, each with at least eight slices of P
+  const int tiles = M / 64 * (N / (16 * NC));
+  int ks = 4;
+  while (ks > 1 && (tiles * ks > 160 || P % (BKS * ks) || P / ks < 8 * BKS)) ks >>= 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(ks, M / 64, N / (16 * NC));
+  cfg.blockDim = dim3(256);
+  cfg.stream = st;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = ks; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, k_skinny<NC, TA>, P, A, lda, B, ldb, C, ldc);
+}
+// N: a multiple of the width `w` (64, 96, 128 or 160) that make_plan chose.
+template <bool TA>
+cudaError_t skinny(cudaStream_t st, int w, int M, int P, const float* A, int lda, const float* B, int ldb, int N, float* C, int ldc) {
+  switch (w) {
+    case 64: return launch_skinny<4, TA>(st, M, P, A, lda, B, ldb, N, C, ldc);
+    case 96: return launch_skinny<6, TA>(st, M, P, A, lda, B, ldb, N, C, ldc);
+    case 128: return launch_skinny<8, TA>(st, M, P, A, lda, B, ldb, N, C, ldc);
+    default: return launch_skinny<10, TA>(st, M, P, A, lda, B, ldb, N, C, ldc);
   }
 }
 
+// The general product (the loss check: any sizes).
 cudaError_t sgemm(cudaStream_t st, int M, int N, int P, const float* A, int lda, bool ta, const float* B, int ldb, bool tb, float* C, int ldc) {
   dim3 grid((N + BN - 1) / BN, (M + BM - 1) / BM);
-  const bool full = M % BM == 0 && N % BN == 0 && P % BKS == 0 && lda % 4 == 0 && ldb % 4 == 0 && ldc % 4 == 0 &&
+  const bool full = !ta && !tb && M % BM == 0 && N % BN == 0 && P % BKS == 0 && lda % 4 == 0 && ldb % 4 == 0 && ldc % 4 == 0 &&
                     ((reinterpret_cast<uintptr_t>(A) | reinterpret_cast<uintptr_t>(B) | reinterpret_cast<uintptr_t>(C)) & 15) == 0;
-  const bool al = lda % 4 == 0 && ldb % 4 == 0 && ldc % 4 == 0 &&
-                  ((reinterpret_cast<uintptr_t>(A) | reinterpret_cast<uintptr_t>(B) | reinterpret_cast<uintptr_t>(C)) & 15) == 0;
-  if (N == NQ && !ta && !tb && M % BMQ == 0 && P % BKS == 0 && al) {
-    k_sgemm_n160<<<M / BMQ, 256, 0, st>>>(P, A, lda, B, ldb, C, ldc);
-    return cudaGetLastError();
-  }
-  if (full) {
-    // products with few tiles (the 4096 x 256 iterates: 64 tiles of 128 rows on 148 SMs) take tiles of 64 rows
-    const bool half = (int)(grid.x * grid.y) < 120;
-    if (half) {
-      dim3 g2(grid.x, M / 64);
-      if (ta && tb) k_sgemm_full<true, true, 4><<<g2, 256, 0, st>>>(P, A, lda, B, ldb, C, ldc);
-      else if (ta) k_sgemm_full<true, false, 4><<<g2, 256, 0, st>>>(P, A, lda, B, ldb, C, ldc);
-      else if (tb) k_sgemm_full<false, true, 4><<<g2, 256, 0, st>>>(P, A, lda, B, ldb, C, ldc);
-      else k_sgemm_full<false, false, 4><<<g2, 256, 0, st>>>(P, A, lda, B, ldb, C, ldc);
-    } else if (ta && tb) k_sgemm_full<true, true, 8><<<grid, 256, 0, st>>>(P, A, lda, B, ldb, C, ldc);
-    else if (ta) k_sgemm_full<true, false, 8><<<grid, 256, 0, st>>>(P, A, lda, B, ldb, C, ldc);
-    else if (tb) k_sgemm_full<false, true, 8><<<grid, 256, 0, st>>>(P, A, lda, B, ldb, C, ldc);
-    else k_sgemm_full<false, false, 8><<<grid, 256, 0, st>>>(P, A, lda, B, ldb, C, ldc);
-  } else {
-    k_sgemm<<<grid, 256, 0, st>>>(M, N, P, A, lda, ta ? 1 : 0, B, ldb, tb ? 1 : 0, C, ldc);
-  }
+  if (full) k_sgemm_full<false, false, false><<<grid, 256, 0, st>>>(P, A, lda, B, ldb, C, ldc);
+  else k_sgemm<<<grid, 256, 0, st>>>(M, N, P, A, lda, ta ? 1 : 0, B, ldb, tb ? 1 : 0, C, ldc);
   return cudaGetLastError();
 }
 
@@ -269,223 +346,509 @@ cudaError_t sgemm(cudaStream_t st, int M, int N, int P, const float* A, int lda,
 __global__ void k_sub(const float* __restrict__ a, const float* __restrict__ b, float* __restrict__ c, int64_t n) {
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) c[i] = a[i] - b[i];
 }
+// The same into a matrix padded with zeros ([rows_p][ld]); b == nullptr: a copy.
+__global__ void k_sub_pad(const float* __restrict__ a, const float* __restrict__ b, int rows, int cols, float* __restrict__ c, int rows_p, int ld) {
+  for (int r = blockIdx.x; r < rows_p; r += gridDim.x) {
+    const float* ar = a + (int64_t)r * cols;
+    const float* br = b ? b + (int64_t)r * cols : nullptr;
+    float* cr = c + (int64_t)r * ld;
+    if (cols % 4 == 0) {
+      for (int i = threadIdx.x * 4; i < ld; i += blockDim.x * 4) {
+        float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (r < rows && i < cols) {
+          v = *reinterpret_cast<const float4*>(ar + i);
+          if (br) { const float4 u = *reinterpret_cast<const float4*>(br + i); v.x -= u.x; v.y -= u.y; v.z -= u.z; v.w -= u.w; }
+        }
+        *reinterpret_cast<float4*>(cr + i) = v;
+      }
+    } else {
+      for (int i = threadIdx.x; i < ld; i += blockDim.x) cr[i] = r < rows && i < cols ? (br ? ar[i] - br[i] : ar[i]) : 0.f;
+    }
+  }
+}
 
 // A fixed start for the iteration: values in (-1, 1) from a counter hash (any full-rank start converges).  The iterate
-// is stored with a leading dimension ld >= m (a multiple of the SGEMM tile); the columns past m are zero and stay zero.
-__global__ void k_init(float* y, int rows, int m, int ld) {
-  const int64_t n = (int64_t)rows * ld;
+// is stored with a leading dimension ld >= m and rows_p >= rows rows (whole tiles); the padding is zero and stays zero.
+__global__ void k_init(float* y, int rows, int rows_p, int m, int ld) {
+  const int64_t n = (int64_t)rows_p * ld;
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
     uint64_t z = (uint64_t)i * 0x9E3779B97F4A7C15ull + 0xD1B54A32D192ED03ull;
     z = (z ^ (z >> 30)) * 0xBF58476D1CE4E5B9ull;
     z = (z ^ (z >> 27)) * 0x94D049BB133111EBull;
     z ^= z >> 31;
-    y[i] = (int)(i % ld) < m ? (float)((double)(z >> 11) * (2.0 / 9007199254740992.0) - 1.0) : 0.f;
+    y[i] = (int)(i % ld) < m && i / ld < rows ? (float)((double)(z >> 11) * (2.0 / 9007199254740992.0) - 1.0) : 0.f;
   }
 }
 
-// S[i][j] = sum_row A[row][i] B[row][j]  for two [rows][m] fp32 matrices, products and sums in fp64.
-// One CTA per 16 x 16 block of S and per part of the rows (blockIdx.z; `chunk` rows each, a multiple of the slice), one
-// thread per element; slices of 64 rows go through shared memory.  Part z writes its sums to parts[z][m][m];
-// k_sum_parts adds the parts in a fixed order, so the result does not depend on the order the CTAs ran in.
-constexpr int kGramParts = 4;
-__global__ void __launch_bounds__(256) k_gram64(const float* __restrict__ A, const float* __restrict__ B, int rows, int chunk, int m, int ld,
-                                                double* __restrict__ parts) {
-  constexpr int RS = 64;                               // rows per slice
-  __shared__ float sa[RS][17], sb[RS][17];
-  const int i0 = blockIdx.y * 16, j0 = blockIdx.x * 16, t = threadIdx.x, ti = t >> 4, tj = t & 15;
-  const int r_lo = blockIdx.z * chunk, r_hi = min(rows, r_lo + chunk);
-  double acc = 0.0;
-  for (int r0 = r_lo; r0 < r_hi; r0 += RS) {
-#pragma unroll
-    for (int k = 0; k < RS / 16; ++k) {
-      const int rr = r0 + ti + 16 * k;
-      sa[ti + 16 * k][tj] = (rr < r_hi && i0 + tj < m) ? A[(int64_t)rr * ld + i0 + tj] : 0.f;
-      sb[ti + 16 * k][tj] = (rr < r_hi && j0 + tj < m) ? B[(int64_t)rr * ld + j0 + tj] : 0.f;
+// S[i][j] = sum_row A[row][i] A[row][j] for a [rows][m] fp32 matrix, products and sums in fp64, lower triangle.
+// One CTA per 32 x 32 block on or below the diagonal and per part of the rows (blockIdx.y; `chunk` rows each), 2 x 2 elements per
+// thread; slices of 32 rows go through shared memory as fp64 (every element is converted once per CTA: a conversion per operand of
+// every product is what bounded the earlier form, 64 us for 4096 x 160).  Part z writes its sums to parts[z][m][m]; k_sum_parts adds
+// the parts in a fixed order, so the result does not depend on the order the CTAs ran in.
+constexpr int kGramParts = 32;
+__global__ void __launch_bounds__(256) k_gram64(const float* __restrict__ A, int rows, int chunk, int m, int ld, double* __restrict__ parts) {
+  __shared__ __align__(16) double sa[32][34], sb[32][34];
+  int bi = (int)((sqrtf(8.f * blockIdx.x + 1.f) - 1.f) * 0.5f);
+  while ((bi + 1) * (bi + 2) / 2 <= (int)blockIdx.x) ++bi;
+  while (bi * (bi + 1) / 2 > (int)blockIdx.x) --bi;
+  const int bj = blockIdx.x - bi * (bi + 1) / 2;
+  const int t = threadIdx.x, ti = t >> 4, tj = t & 15, lr = t >> 3, lc = (t & 7) * 4;
+  const int r_lo = blockIdx.y * chunk, r_hi = min(rows, r_lo + chunk);
+  double acc[2][2] = {{0.0, 0.0}, {0.0, 0.0}};
+  float4 va = make_float4(0.f, 0.f, 0.f, 0.f), vb = va;
+  // (ld is a multiple of 32 and the columns past m are zero, so whole pieces can be read)
+  auto fetch = [&](int r0) {
+    const int rr = r0 + lr;
+    va = vb = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (rr < r_hi) {
+      va = *reinterpret_cast<const float4*>(A + (int64_t)rr * ld + bi * 32 + lc);
+      vb = *reinterpret_cast<const float4*>(A + (int64_t)rr * ld + bj * 32 + lc);
+    }
+  };
+  fetch(r_lo);
+  for (int r0 = r_lo; r0 < r_hi; r0 += 32) {
+    sa[lr][lc] = va.x; sa[lr][lc + 1] = va.y; sa[lr][lc + 2] = va.z; sa[lr][lc + 3] = va.w;
+    sb[lr][lc] = vb.x; sb[lr][lc + 1] = vb.y; sb[lr][lc + 2] = vb.z; sb[lr][lc + 3] = vb.w;
+    __syncthreads();
+    fetch(r0 + 32);
+#pragma unroll 8
+    for (int r = 0; r < 32; ++r) {
+      const double2 a = *reinterpret_cast<const double2*>(&sa[r][2 * ti]), b = *reinterpret_cast<const double2*>(&sb[r][2 * tj]);
+      acc[0][0] = fma(a.x, b.x, acc[0][0]); acc[0][1] = fma(a.x, b.y, acc[0][1]);
+      acc[1][0] = fma(a.y, b.x, acc[1][0]); acc[1][1] = fma(a.y, b.y, acc[1][1]);
     }
     __syncthreads();
-#pragma unroll 16
-    for (int r = 0; r < RS; ++r) acc += (double)sa[r][ti] * (double)sb[r][tj];
-    __syncthreads();
   }
-  if (i0 + ti < m && j0 + tj < m) parts[((int64_t)blockIdx.z * m + i0 + ti) * m + j0 + tj] = acc;
+#pragma unroll
+  for (int i = 0; i < 2; ++i)
+#pragma unroll
+    for (int j = 0; j < 2; ++j) {
+      const int gi = bi * 32 + 2 * ti + i, gj = bj * 32 + 2 * tj + j;
+      if (gi < m && gj <= gi) parts[((int64_t)blockIdx.y * m + gi) * m + gj] = acc[i][j];
+    }
 }
-__global__ void k_sum_parts(const double* __restrict__ parts, int n_parts, int n, double* __restrict__ S) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  double v = parts[i];
-  for (int z = 1; z < n_parts; ++z) v += parts[(int64_t)z * n + i];
-  S[i] = v;
+// The parts' sum; MIRROR: both triangles, else the lower one.
+template <bool MIRROR>
+__global__ void k_sum_parts(const double* __restrict__ parts, int n_parts, int m, double* __restrict__ S) {
+  const int e = blockIdx.x * blockDim.x + threadIdx.x;
+  const int i = e / m, j = e - i * m;
+  if (i >= m || j > i) return;
+  double v[4] = {0.0, 0.0, 0.0, 0.0};
+  int z = 0;
+  for (; z + 4 <= n_parts; z += 4)
+#pragma unroll
+    for (int k = 0; k < 4; ++k) v[k] += parts[((int64_t)(z + k) * m + i) * m + j];
+  for (; z < n_parts; ++z) v[0] += parts[((int64_t)z * m + i) * m + j];
+  const double sum = (v[0] + v[1]) + (v[2] + v[3]);
+  S[(int64_t)i * m + j] = sum;
+  if (MIRROR) S[(int64_t)j * m + i] = sum;
 }
-// S = A^T B over all rows: the parts, then their sum.
-cudaError_t gram64(cudaStream_t st, const float* A, const float* B, int rows, int m, int ld, double* parts, double* S) {
-  const int chunk = ((rows + kGramParts - 1) / kGramParts + 63) / 64 * 64;
-  dim3 g((m + 15) / 16, (m + 15) / 16, kGramParts);
-  k_gram64<<<g, 256, 0, st>>>(A, B, rows, chunk, m, ld, parts);
-  k_sum_parts<<<(m * m + 255) / 256, 256, 0, st>>>(parts, kGramParts, m * m, S);
+// S = A^T A over all rows: the parts, then their sum.
+template <bool MIRROR>
+cudaError_t gram64(cudaStream_t st, const float* A, int rows, int m, int ld, double* parts, double* S) {
+  const int nb = (m + 31) / 32, tiles = nb * (nb + 1) / 2;
+  int n_parts = (rows + 127) / 128;                  // 128 rows per part, or more where that would be too many
+  if (n_parts > kGramParts) n_parts = kGramParts;
+  const int chunk = ((rows + n_parts - 1) / n_parts + 31) / 32 * 32;
+  n_parts = (rows + chunk - 1) / chunk;
+  k_gram64<<<dim3(tiles, n_parts), 256, 0, st>>>(A, rows, chunk, m, ld, parts);
+  k_sum_parts<MIRROR><<<(m * m + 255) / 256, 256, 0, st>>>(parts, n_parts, m, S);
   return cudaGetLastError();
 }
 
-// Largest m for which the one-CTA kernels below keep their fp64 matrix in shared memory.
-constexpr int kCholSmem = 160;
-// The factorisation proper on an m x m matrix S with row stride ls (shared or global memory, the code is the same).
-// In shared memory ls is odd: threads that walk down a column (one row each) would otherwise all hit one bank when m
-// is a multiple of 16.
-__device__ __forceinline__ void chol_inverse_in_place(double* S, const int m, const int ls, double* shift_slot, double* scratch) {
+// Cholesky S = L L^T (fp64) of an m x m Gram matrix by one CTA, right-looking in panels of 16 columns:
+//   (A) one warp factors the 16 x 16 diagonal block in registers (lane = row) and inverts it,
+//   (B) the rows below are multiplied with the inverse, one element per thread,
+//   (C) the trailing lower triangle is updated in 4 x 4 tiles (16 products per 8 16-byte reads of shared memory).
+// Writes L over S (lower triangle, global) and the inverses of the diagonal blocks; Q = Y L^{-T} follows by k_trsm.  A small multiple
+// of the trace is added to the diagonal first, so that a rank-deficient iterate still factors.  In shared memory up to
+// m = kCholSmem, else in place in global memory (L2).  m = 160: 300 us with an explicit inverse and unblocked updates before.
+constexpr int kCholSmem = 160, kPanPitch = 18;
+constexpr int kCholThreads = 512;
+__host__ __device__ constexpr int chol_smem(int m) { return ((m <= kCholSmem ? m * (m | 1) : 0) + m * kPanPitch) * 8 + 16; }
+__global__ void __launch_bounds__(kCholThreads) k_chol64(double* Sg, int m, double* __restrict__ Dinv) {
+  extern __shared__ __align__(16) double sm[];
+  __shared__ double dv[16][17], shift_s;
   const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
-  if (warp == 0) {
-    double tr = 0.0;
-    for (int i = lane; i < m; i += 32) tr += S[i * ls + i];
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) tr += __shfl_xor_sync(0xffffffffu, tr, o);
-    if (lane == 0) *shift_slot = 1e-13 * tr + 1e-300;
-  }
-  __syncthreads();
-  const double shift = *shift_slot;
-  for (int i = t; i < m; i += 1024) S[i * ls + i] += shift;
-  __syncthreads();
-  // Blocked right-looking factorisation, panels of 16 columns: (A) the 16 x 16 diagonal block by one warp, (B) the rows
-  // below it by one thread per row (forward substitution against the block), (C) the rank-16 update of the trailing
-  // lower triangle by everybody -- three barriers per panel instead of three per column.
-  constexpr int NB = 16;
-  for (int j0 = 0; j0 < m; j0 += NB) {
-    const int jb = m - j0 < NB ? m - j0 : NB;
-    if (warp == 0) {
-      for (int j = 0; j < jb; ++j) {
-        double* dj = S + (j0 + j) * ls + j0;                 // row j0 + j of the block
-        const double v = dj[j];
-        const double ljj = sqrt(v > shift * 1e-3 ? v : shift * 1e-3);
-        __syncwarp();
-        if (lane == 0) dj[j] = ljj;
-        if (lane > j && lane < jb) S[(j0 + lane) * ls + j0 + j] /= ljj;
-        __syncwarp();
-        if (lane > j && lane < jb) {
-          double* dr = S + (j0 + lane) * ls + j0;
-          const double lrj = dr[j];
-          for (int c = j + 1; c <= lane; ++c) dr[c] -= lrj * S[(j0 + c) * ls + j0 + j];
-        }
-        __syncwarp();
-      }
-    }
-    __syncthreads();
-    for (int i = j0 + jb + t; i < m; i += 1024) {           // (B)
-      double* ri = S + i * ls + j0;
-      for (int j = 0; j < jb; ++j) {
-        const double* dj = S + (j0 + j) * ls + j0;
-        double v = ri[j];
-        for (int q = 0; q < j; ++q) v -= ri[q] * dj[q];
-        ri[j] = v / dj[j];
-      }
-    }
-    __syncthreads();
-    for (int i = j0 + jb + warp; i < m; i += 32) {          // (C)
-      const double* li = S + i * ls + j0;
-      double lr[NB];
-#pragma unroll
-      for (int q = 0; q < NB; ++q) lr[q] = q < jb ? li[q] : 0.0;
-      for (int c = j0 + jb + lane; c <= i; c += 32) {
-        const double* lc = S + c * ls + j0;
-        double acc = 0.0;
-#pragma unroll
-        for (int q = 0; q < NB; ++q) acc += q < jb ? lr[q] * lc[q] : 0.0;
-        S[i * ls + c] -= acc;
-      }
-    }
-    __syncthreads();
-  }
-  // X = L^{-1} by blocks of 16, kept transposed in the strict upper triangle of S (free after the factorisation):
-  // S[j][i] = X[i][j] for i > j; the diagonal of X is 1 / L[j][j].
-  //   diagonal blocks: X_bb = L_bb^{-1}, one thread per column (16 steps of forward substitution);
-  //   then block diagonal by block diagonal (distance dd = 1, 2, ...: the blocks of one diagonal are independent):
-  //     P = sum_{kb = jb}^{ib - 1} L_{ib,kb} X_{kb,jb}   (into the scratch, one thread per element),
-  //     X_{ib,jb} = - X_{ib,ib} P.
-  const int nblk = (m + NB - 1) / NB;
-  auto X_at = [&](int i, int j) -> double {               // X[i][j], i >= j
-    return i == j ? 1.0 / S[j * ls + j] : S[j * ls + i];
-  };
-  for (int j = t; j < m; j += 1024) {
-    const int b0 = (j / NB) * NB, b1 = b0 + NB < m ? b0 + NB : m;
-    const double xjj = 1.0 / S[j * ls + j];
-    for (int i = j + 1; i < b1; ++i) {
-      double acc = S[i * ls + j] * xjj;
-      for (int q = j + 1; q < i; ++q) acc += S[i * ls + q] * S[j * ls + q];
-      S[j * ls + i] = -acc / S[i * ls + i];
-    }
-  }
-  __syncthreads();
-  for (int dd = 1; dd < nblk; ++dd) {
-    const int nb_d = nblk - dd;                            // blocks on this diagonal: (ib, jb) = (jb + dd, jb)
-    for (int e = t; e < nb_d * NB * NB; e += 1024) {
-      const int jb = e / (NB * NB), r = (e / NB) % NB, c = e % NB, ib = jb + dd;
-      const int i = ib * NB + r, j = jb * NB + c;
-      double acc = 0.0;
-      if (i < m && j < m) {
-        const double* li = S + i * ls;
-        for (int q = j; q < ib * NB; ++q) acc += li[q] * X_at(q, j);      // X[q][j] = 0 for q < j
-      }
-      scratch[e] = acc;
-    }
-    __syncthreads();
-    for (int e = t; e < nb_d * NB * NB; e += 1024) {
-      const int jb = e / (NB * NB), r = (e / NB) % NB, c = e % NB, ib = jb + dd;
-      const int i = ib * NB + r, j = jb * NB + c;
-      if (i < m && j < m) {
-        double acc = 0.0;
-        for (int q = 0; q <= r; ++q) acc += X_at(i, ib * NB + q) * scratch[(jb * NB + q) * NB + c];
-        S[j * ls + i] = -acc;
-      }
-    }
-    __syncthreads();
-  }
-}
-
-// Cholesky S = L L^T (fp64) of an m x m Gram matrix and the inverse of the factor, by one CTA: writes W = L^{-T} as fp32
-// into an [ld][ld] matrix (zero outside its upper triangle), so that Q = Y W is orth(Y).  The matrix is worked on in
-// shared memory when it fits (m <= kCholSmem), else in place in global memory.  A small multiple of the trace is added
-// to the diagonal first, so that a rank-deficient iterate still factors.
-__global__ void __launch_bounds__(1024) k_chol_inv64(double* Sg, int m, float* W, int ld) {
-  extern __shared__ double sm[];
-  __shared__ double shift_s;
-  const int t = threadIdx.x;
   const bool in_smem = m <= kCholSmem;
   const int ls = in_smem ? (m | 1) : m;
-  if (in_smem) {
-    for (int e = t; e < m * m; e += 1024) sm[(e / m) * ls + e % m] = Sg[e];
-    __syncthreads();
-    chol_inverse_in_place(sm, m, ls, &shift_s, sm + m * ls);
-  } else {
-    chol_inverse_in_place(Sg, m, ls, &shift_s, sm);
+  double* pan = sm;                                  // [m][kPanPitch]
+  double* S = in_smem ? sm + m * kPanPitch : Sg;
+  if (in_smem)
+    for (int i = warp; i < m; i += kCholThreads / 32)
+      for (int j = lane; j <= i; j += 32) S[i * ls + j] = Sg[(int64_t)i * m + j];
+  __syncthreads();
+  if (warp == 0) {
+    double tr = 0.0;
+    for (int i = lane; i < m; i += 32) tr += S[(int64_t)i * ls + i];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) tr += __shfl_xor_sync(0xffffffffu, tr, o);
+    if (lane == 0) shift_s = 1e-13 * tr + 1e-300;
   }
-  const double* S = in_smem ? sm : Sg;
-  // W[j][i] = X[i][j] (upper triangle of W = L^{-T}); everything else zero
-  for (int j = t >> 5; j < ld; j += 32) {
-    for (int i = t & 31; i < ld; i += 32) {
-      float v = 0.f;
-      if (j < m && i < m) {
-        if (i == j) v = (float)(1.0 / S[j * ls + j]);
-        else if (i > j) v = (float)S[j * ls + i];
+  __syncthreads();
+  const double shift = shift_s;
+  for (int i = t; i < m; i += kCholThreads) S[(int64_t)i * ls + i] += shift;
+  __syncthreads();
+  for (int j0 = 0; j0 < m; j0 += 16) {
+    if (warp == 0) {                                 // (A); lanes 16..31 repeat lanes 0..15
+      const int r = lane & 15, gi = j0 + r;
+      double a[16], x[16], rinv = 0.0;
+#pragma unroll
+      for (int q = 0; q < 16; ++q) a[q] = gi < m && q <= r ? S[(int64_t)gi * ls + j0 + q] : (q == r ? 1.0 : 0.0);      // past m: identity
+#pragma unroll
+      for (int k = 0; k < 16; ++k) {
+        double d = __shfl_sync(0xffffffffu, a[k], k);
+        d = d > shift * 1e-3 ? d : shift * 1e-3;
+        const double ri = rsqrt(d);
+        if (r == k) { a[k] = d * ri; rinv = ri; }
+        else if (r > k) a[k] *= ri;
+#pragma unroll
+        for (int c = k + 1; c < 16; ++c) {
+          const double l = __shfl_sync(0xffffffffu, a[k], c);
+          if (r >= c) a[c] -= a[k] * l;
+        }
       }
-      W[j * ld + i] = v;
+      // column r of the inverse by forward substitution
+#pragma unroll
+      for (int i = 0; i < 16; ++i) {
+        double v = i == r ? 1.0 : 0.0, u = 0.0;
+#pragma unroll
+        for (int q = 0; q < i; ++q) {
+          const double l = __shfl_sync(0xffffffffu, a[q], i);
+          if (q & 1) u -= l * x[q]; else v -= l * x[q];
+        }
+        x[i] = (v + u) * __shfl_sync(0xffffffffu, rinv, i);
+      }
+      if (lane < 16) {
+#pragma unroll
+        for (int q = 0; q < 16; ++q) {
+          if (gi < m && q <= r) S[(int64_t)gi * ls + j0 + q] = a[q];
+          dv[q][r] = x[q];
+          Dinv[(int64_t)(j0 + q) * 16 + r] = x[q];
+        }
+      }
     }
+    __syncthreads();
+    const int j1 = j0 + 16, R = m - j1;
+    if (R <= 0) break;
+    for (int e = t; e < R * 16; e += kCholThreads) {       // (B)
+      const int i = j1 + (e >> 4), c = e & 15;
+      const double* ri = S + (int64_t)i * ls + j0;
+      double v = 0.0;
+      for (int q = 0; q <= c; ++q) v = fma(ri[q], dv[c][q], v);
+      pan[i * kPanPitch + c] = v;
+    }
+    __syncthreads();
+    for (int e = t; e < R * 16; e += kCholThreads) S[(int64_t)(j1 + (e >> 4)) * ls + j0 + (e & 15)] = pan[(j1 + (e >> 4)) * kPanPitch + (e & 15)];
+    const int T = (R + 3) / 4, tiles = T * (T + 1) / 2;
+    for (int e = t; e < tiles; e += kCholThreads) {         // (C)
+      int ti = (int)((sqrtf(8.f * e + 1.f) - 1.f) * 0.5f);
+      while ((ti + 1) * (ti + 2) / 2 <= e) ++ti;
+      while (ti * (ti + 1) / 2 > e) --ti;
+      const int i0 = j1 + 4 * ti, c0 = j1 + 4 * (e - ti * (ti + 1) / 2);
+      double acc[4][4];
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int c = 0; c < 4; ++c) acc[i][c] = 0.0;
+#pragma unroll
+      for (int q = 0; q < 16; q += 2) {
+        double2 li[4], lc[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          li[i] = *reinterpret_cast<const double2*>(pan + min(i0 + i, m - 1) * kPanPitch + q);
+          lc[i] = *reinterpret_cast<const double2*>(pan + min(c0 + i, m - 1) * kPanPitch + q);
+        }
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+#pragma unroll
+          for (int c = 0; c < 4; ++c) acc[i][c] = fma(li[i].y, lc[c].y, fma(li[i].x, lc[c].x, acc[i][c]));
+      }
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int c = 0; c < 4; ++c)
+          if (i0 + i < m && c0 + c <= i0 + i) S[(int64_t)(i0 + i) * ls + c0 + c] -= acc[i][c];
+    }
+    __syncthreads();
+  }
+  if (in_smem) {
+    __syncthreads();
+    for (int i = warp; i < m; i += kCholThreads / 32)
+      for (int j = lane; j <= i; j += 32) Sg[(int64_t)i * m + j] = S[i * ls + j];
   }
 }
 
-// Symmetric positive semi-definite eigenproblem H = V diag(lam) V^T, m x m, fp64, by one-sided (Hestenes) Jacobi in one
-// CTA: pairs of rows of H (= columns, H is symmetric) are rotated until they are orthogonal.  With J the product of the
+// Q = Y L^{-T}, row by row (fp64 inside): a CTA takes 16 rows, half a warp each (lane = column of the panel); panel by panel of 16
+// columns  q_p = (y_p - sum_{c < 16 p} q_c L[p][c]^T) Dinv_p^T.  A panel's 16 rows of L come by cp.async, one panel ahead.
+__host__ __device__ constexpr int trsm_pitch(int m) { return (m + 15) / 16 * 16 + 2; }
+__host__ __device__ constexpr int trsm_smem(int m) { return 3 * 16 * trsm_pitch(m) * 8; }
+__global__ void __launch_bounds__(256) k_trsm(const float* __restrict__ Y, const double* __restrict__ L, const double* __restrict__ Dinv, int m, int ld,
+                                              float* __restrict__ Q) {
+  extern __shared__ __align__(16) double smt[];
+  const int lq = trsm_pitch(m);
+  double* qd = smt;                                  // [16][lq]
+  double* lp = smt + 16 * lq;                        // [2][16][lq]
+  const int t = threadIdx.x, r = t >> 4, c = t & 15;
+  const int64_t row = (int64_t)blockIdx.x * 16 + r;
+  const int np = (m + 15) / 16;
+  auto fetch = [&](int p) {                          // rows 16 p .. of L, columns before 16 p
+    double* dst = lp + (p & 1) * 16 * lq;
+    for (int q = c; q < 16 * p; q += 16) {
+      if (16 * p + r < m) {
+        const uint32_t d = (uint32_t)__cvta_generic_to_shared(dst + r * lq + q);
+        asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(d), "l"(L + (int64_t)(16 * p + r) * m + q) : "memory");
+      } else {
+        dst[r * lq + q] = 0.0;
+      }
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+  if (np > 1) fetch(1);
+  for (int p = 0; p < np; ++p) {
+    double dr[16];
+#pragma unroll
+    for (int q = 0; q < 16; ++q) dr[q] = __ldg(Dinv + (int64_t)(16 * p + c) * 16 + q);
+    double v0 = (double)Y[row * ld + 16 * p + c], v1 = 0.0;
+    if (p > 0) {
+      asm volatile("cp.async.wait_group 0;" ::: "memory");
+      __syncthreads();                               // panel p is there, and panel p - 1 has been read
+      if (p + 1 < np) fetch(p + 1);
+      const double* lr = lp + (p & 1) * 16 * lq + c * lq;
+      const double* qr = qd + r * lq;
+#pragma unroll 4
+      for (int q = 0; q < 16 * p; q += 2) {
+        const double2 a = *reinterpret_cast<const double2*>(qr + q), b = *reinterpret_cast<const double2*>(lr + q);
+        v0 = fma(-a.x, b.x, v0); v1 = fma(-a.y, b.y, v1);
+      }
+    }
+    const double v = v0 + v1;
+    double o = 0.0;
+#pragma unroll
+    for (int q = 0; q < 16; ++q) {
+      const double u = __shfl_sync(0xffffffffu, v, q, 16);
+      o = fma(u, dr[q], o);                          // (Dinv is lower triangular: zeros past c)
+    }
+    qd[r * lq + 16 * p + c] = o;
+    Q[row * ld + 16 * p + c] = (float)o;
+    __syncwarp();
+  }
+  for (int i = 16 * np + c; i < ld; i += 16) Q[row * ld + i] = 0.f;
+}
+
+// Symmetric positive semi-definite eigenproblem H = V diag(lam) V^T, m x m, fp64, by one-sided (Hestenes) Jacobi: pairs of
+// columns of H are rotated until they are orthogonal.  With J the product of the rotations the result is H J = V diag(lam): column i
+// has norm lam_i and direction v_i, so the eigenvectors are the normalised columns and no separate accumulation of the
+// rotations is needed (a column whose norm is zero up to rounding has no direction; its eigenvalue is far below the kept ones).
+//
+// A warp holds two blocks of B columns in registers (E elements of each per lane); blocks meet by the round-robin tournament
+// and travel between the warps of a cluster through distributed shared memory, one cluster barrier per meeting.  In a
+// meeting every column of one block is rotated against every column of the other, B disjoint pairs at a time whose latencies
+// overlap; the pairs inside a block take their turn once per sweep.  Squared norms are carried along (recomputed every
+// sweep), so a rotation needs one dot product.  The angle is computed in fp32 -- a rotation by a slightly different angle is
+// still a rotation, and the next sweep works on what it left -- its cosine in fp64.  One CTA that kept the columns in shared
+// memory and went through it for every pair took 4.5 ms at m = 160.
+template <int B, int E>
+struct JacobiShape {
+  static constexpr int kElems = 32 * E;              // elements per column (>= m, zero-padded)
+  static constexpr int kBlock = B * kElems + B;      // doubles of a block: its columns, their squared norms
+};
+template <int B, int E>
+__global__ void __launch_bounds__(B == 4 ? 160 : 320, 1) k_jacobi_cl(const double* __restrict__ Hg, int m, double* lam, float* __restrict__ Vf, int ldv, int max_sweeps) {
+  using Sh = JacobiShape<B, E>;
+  extern __shared__ __align__(16) double smj[];      // [2 buffers][warps][2 sides][B][kElems]
+  __shared__ int moved_s[2];
+  const int t = threadIdx.x, lane = t & 31, warp = t >> 5, nw = blockDim.x >> 5;
+  const int cs = gridDim.x, rank = blockIdx.x, G = cs * nw, g = rank * nw + warp;      // groups of the tournament, this warp's
+  const uint32_t base = (uint32_t)__cvta_generic_to_shared(smj);
+  const uint32_t buf_b = (uint32_t)nw * 2 * Sh::kBlock * 8;
+  // scale so that the largest norm is about one (a power of two: exact)
+  double tr = 0.0;
+  for (int i = lane; i < m; i += 32) tr += Hg[(int64_t)i * m + i];
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) tr += __shfl_xor_sync(0xffffffffu, tr, o);
+  int ex = 0;
+  if (tr > 0.0) frexp(tr, &ex);
+  const double down = ldexp(1.0, -ex), up = ldexp(1.0, ex);
+  double h[2][B][E], nrm[2][B];
+#pragma unroll
+  for (int s = 0; s < 2; ++s)
+#pragma unroll
+    for (int b = 0; b < B; ++b) {
+      const int col = (2 * g + s) * B + b;
+#pragma unroll
+      for (int e = 0; e < E; ++e) {
+        const int i = lane + 32 * e;
+        h[s][b][e] = col < m && i < m ? Hg[(int64_t)col * m + i] * down : 0.0;
+      }
+    }
+  if (t < 2) moved_s[t] = 0;
+  int any = 0;
+  auto norms = [&]() {
+#pragma unroll
+    for (int s = 0; s < 2; ++s)
+#pragma unroll
+      for (int b = 0; b < B; ++b) {
+        double v = 0.0;
+#pragma unroll
+        for (int e = 0; e < E; ++e) v = fma(h[s][b][e], h[s][b][e], v);
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+        nrm[s][b] = v;
+      }
+  };
+  auto rotate = [&](double (&x)[E], double (&y)[E], double& al, double& be, double ga) {
+    if (ga * ga <= 1e-22 * al * be) return;          // orthogonal far beyond what the fp32 operands carry
+    any = 1;
+    // both scaled by one power of two, so that fp32 neither overflows nor loses what is small
+    const double zd = be - al, wd = 2.0 * ga;
+    const int e_max = max(__double2hiint(zd) & 0x7ff00000, __double2hiint(wd) & 0x7ff00000);
+    if (e_max < 0x01000000) return;
+    const double unit = __hiloint2double(0x7fe00000 - e_max, 0);
+    const float z = (float)(zd * unit), w = (float)(wd * unit);
+    const float tf = copysignf(w / (fabsf(z) + sqrtf(fmaf(z, z, w * w))), z >= 0.f ? w : -w);
+    const double tt = (double)tf, c = rsqrt(fma(tt, tt, 1.0)), sn = c * tt;
+#pragma unroll
+    for (int e = 0; e < E; ++e) {
+      const double a = x[e], b = y[e];
+      x[e] = c * a - sn * b;
+      y[e] = fma(sn, a, c * b);
+    }
+    // exact for any angle: |c a - s b|^2 = c^2 al - 2 c s ga + s^2 be
+    const double c2 = c * c, s2 = sn * sn, cs2 = 2.0 * c * sn * ga, na = c2 * al - cs2 + s2 * be, nb = s2 * al + cs2 + c2 * be;
+    al = na > 0.0 ? na : 0.0; be = nb > 0.0 ? nb : 0.0;
+  };
+  auto dot = [&](const double (&x)[E], const double (&y)[E]) {
+    double v = 0.0;
+#pragma unroll
+    for (int e = 0; e < E; ++e) v = fma(x[e], y[e], v);
+    return v;
+  };
+  cluster_sync_all();
+  int flip = 0, sweep = 0;
+  for (; sweep < max_sweeps; ++sweep) {
+    any = 0;
+    norms();
+    if (B > 1) {                                     // the pairs inside the blocks: rounds of B / 2 disjoint pairs in each
+#pragma unroll
+      for (int k = 1; k < B; ++k) {
+        double ga[2][B];
+#pragma unroll
+        for (int s = 0; s < 2; ++s)
+#pragma unroll
+          for (int b = 0; b < B; ++b) if ((b ^ k) > b) ga[s][b] = dot(h[s][b], h[s][b ^ k]);
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+          for (int s = 0; s < 2; ++s)
+#pragma unroll
+            for (int b = 0; b < B; ++b) if ((b ^ k) > b) ga[s][b] += __shfl_xor_sync(0xffffffffu, ga[s][b], o);
+#pragma unroll
+        for (int s = 0; s < 2; ++s)
+#pragma unroll
+          for (int b = 0; b < B; ++b) if ((b ^ k) > b) rotate(h[s][b], h[s][b ^ k], nrm[s][b], nrm[s][b ^ k], ga[s][b]);
+      }
+    }
+    for (int step = 0; step < 2 * G - 1; ++step) {
+#pragma unroll
+      for (int k = 0; k < B; ++k) {
+        double ga[B];
+#pragma unroll
+        for (int b = 0; b < B; ++b) ga[b] = dot(h[0][b], h[1][(b + k) % B]);
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+          for (int b = 0; b < B; ++b) ga[b] += __shfl_xor_sync(0xffffffffu, ga[b], o);
+#pragma unroll
+        for (int b = 0; b < B; ++b) rotate(h[0][b], h[1][(b + k) % B], nrm[0][b], nrm[1][(b + k) % B], ga[b]);
+      }
+      if (G == 1) break;
+      // circle method: the top block of group 0 stays, the others move on by one place of the ring of blocks
+      flip ^= 1;
+#pragma unroll
+      for (int s = 0; s < 2; ++s) {
+        int tg, ts;
+        if (s == 0) { if (g == 0) { tg = 0; ts = 0; } else if (g < G - 1) { tg = g + 1; ts = 0; } else { tg = g; ts = 1; } }
+        else { if (g == 0) { tg = 1; ts = 0; } else { tg = g - 1; ts = 1; } }
+        const uint32_t off = base + flip * buf_b + (uint32_t)((tg % nw) * 2 + ts) * (Sh::kBlock * 8) + lane * 8;
+        uint32_t dst;
+        asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(dst) : "r"(off), "r"(tg / nw));
+#pragma unroll
+        for (int b = 0; b < B; ++b)
+#pragma unroll
+          for (int e = 0; e < E; ++e)
+            asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(dst + (b * Sh::kElems + 32 * e) * 8), "d"(h[s][b][e]) : "memory");
+#pragma unroll
+        for (int b = 0; b < B; ++b)
+          if (lane == b) asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(dst + B * Sh::kElems * 8), "d"(nrm[s][b]) : "memory");
+      }
+      cluster_sync_all();
+#pragma unroll
+      for (int s = 0; s < 2; ++s) {
+        const double* src = smj + (size_t)flip * nw * 2 * Sh::kBlock + (size_t)(warp * 2 + s) * Sh::kBlock + lane;
+#pragma unroll
+        for (int b = 0; b < B; ++b)
+#pragma unroll
+          for (int e = 0; e < E; ++e) h[s][b][e] = src[b * Sh::kElems + 32 * e];
+#pragma unroll
+        for (int b = 0; b < B; ++b) nrm[s][b] = src[B * Sh::kElems + b - lane];
+      }
+    }
+    // did anybody rotate?  every CTA's flag, by every warp that did
+    if (any && lane == 0) {
+      for (int r = 0; r < cs; ++r) {
+        uint32_t a;
+        asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"((uint32_t)__cvta_generic_to_shared(&moved_s[sweep & 1])), "r"(r));
+        asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(a), "r"(1) : "memory");
+      }
+    }
+    cluster_sync_all();
+    const int moved = *reinterpret_cast<volatile int*>(&moved_s[sweep & 1]);
+    if (t == 0) moved_s[(sweep & 1) ^ 1] = 0;
+    cluster_sync_all();
+    if (!moved) break;
+  }
+  // eigenvalues = column norms; order them (descending; ties by place)
+  norms();
+  const int nc = 2 * G * B;
+#pragma unroll
+  for (int s = 0; s < 2; ++s)
+#pragma unroll
+    for (int b = 0; b < B; ++b)
+      if (lane == 0) lam[m + (2 * g + s) * B + b] = sqrt(nrm[s][b]);      // unsorted, behind the sorted ones
+  __threadfence();
+  cluster_sync_all();
+#pragma unroll
+  for (int s = 0; s < 2; ++s)
+#pragma unroll
+    for (int b = 0; b < B; ++b) {
+      const int me = (2 * g + s) * B + b;
+      const double mine = __ldcg(lam + m + me);
+      int rk = 0;
+      for (int o = lane; o < nc; o += 32) { const double v = __ldcg(lam + m + o); rk += (v > mine || (v == mine && o < me)) ? 1 : 0; }
+      rk = __reduce_add_sync(0xffffffffu, rk);
+      if (rk < m) {
+        if (lane == 0) lam[rk] = mine * up;
+        const double inv = mine > 0.0 ? 1.0 / mine : 0.0;
+#pragma unroll
+        for (int e = 0; e < E; ++e) {
+          const int i = lane + 32 * e;
+          if (i < m) Vf[(int64_t)i * ldv + rk] = (float)(h[s][b][e] * inv);
+        }
+      }
+    }
+}
+
+// The same in one CTA, for matrices whose blocks do not fit into a cluster's shared memory (m > 320): pairs of rows of H (= columns, H is symmetric) are rotated until they are orthogonal.  With J the product of the
 // rotations the result is J^T H = diag(lam) J^T: row i has norm lam_i and direction v_i, so the eigenvectors are the
 // normalised rows and no separate accumulation of the rotations is needed (a row whose norm is zero up to rounding has
 // no direction; its eigenvalue is far below the ones that are kept).
 // Pairs follow the round-robin tournament (m' / 2 disjoint pairs per step, m' - 1 steps per sweep); a warp takes a pair.
-// Output: eigenvalues in descending order (lam) and the matching eigenvectors as fp32 columns of Vf ([m][m] row-major).
-__global__ void __launch_bounds__(1024) k_jacobi64(double* Hg, double* V, int m, double* lam, float* Vf, int max_sweeps) {
-  extern __shared__ double smj[];
+// Output: eigenvalues in descending order (lam) and the matching eigenvectors as fp32 columns of Vf ([m][ldv] row-major).
+__global__ void __launch_bounds__(1024) k_jacobi64(double* H, int m, double* lam, float* Vf, int ldv, int max_sweeps) {
   __shared__ int moved_s;
   __shared__ int rank_s[512];
   const int t = threadIdx.x, nt = blockDim.x, warp = t >> 5, lane = t & 31, nwarp = nt >> 5;
-  // the matrix whose columns are rotated is read three times per pair: in shared memory when it fits
-  double* H = m <= kCholSmem ? smj : Hg;
-  (void)V;
-  if (m <= kCholSmem) for (int e = t; e < m * m; e += nt) smj[e] = Hg[e];
-  __syncthreads();
   const int mp = (m + 1) & ~1;                       // players of the tournament (one bye if m is odd)
   for (int sweep = 0; sweep < max_sweeps; ++sweep) {
     if (t == 0) moved_s = 0;
@@ -500,22 +863,7 @@ __global__ void __launch_bounds__(1024) k_jacobi64(double* Hg, double* V, int m,
         // columns p and q of H (column c of the symmetric start is stored as row c: H[c * m + i])
         double* hp = H + (int64_t)p * m; double* hq = H + (int64_t)q * m;
         double al = 0.0, be = 0.0, ga = 0.0;
-        // up to 160 columns a lane keeps its five elements of both rows in registers between the products and the
-        // rotation: the kernel is bound by shared-memory traffic, and this takes a third of it away
-        constexpr int KE = 5;
-        const bool keep = m <= 32 * KE;
-        double av[KE], bv[KE];
-        if (keep) {
-#pragma unroll
-          for (int e = 0; e < KE; ++e) {
-            const int i = lane + 32 * e;
-            const double a = i < m ? hp[i] : 0.0, b = i < m ? hq[i] : 0.0;
-            av[e] = a; bv[e] = b;
-            al += a * a; be += b * b; ga += a * b;
-          }
-        } else {
-          for (int i = lane; i < m; i += 32) { const double a = hp[i], b = hq[i]; al += a * a; be += b * b; ga += a * b; }
-        }
+        for (int i = lane; i < m; i += 32) { const double a = hp[i], b = hq[i]; al += a * a; be += b * b; ga += a * b; }
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) {
           al += __shfl_xor_sync(0xffffffffu, al, o); be += __shfl_xor_sync(0xffffffffu, be, o); ga += __shfl_xor_sync(0xffffffffu, ga, o);
@@ -524,17 +872,9 @@ __global__ void __launch_bounds__(1024) k_jacobi64(double* Hg, double* V, int m,
         const double zeta = (be - al) / (2.0 * ga);
         const double tt = (zeta >= 0.0 ? 1.0 : -1.0) / (fabs(zeta) + sqrt(1.0 + zeta * zeta));
         const double c = 1.0 / sqrt(1.0 + tt * tt), s = c * tt;
-        if (keep) {
-#pragma unroll
-          for (int e = 0; e < KE; ++e) {
-            const int i = lane + 32 * e;
-            if (i < m) { hp[i] = c * av[e] - s * bv[e]; hq[i] = s * av[e] + c * bv[e]; }
-          }
-        } else {
-          for (int i = lane; i < m; i += 32) {
-            const double a = hp[i], b = hq[i];
-            hp[i] = c * a - s * b; hq[i] = s * a + c * b;
-          }
+        for (int i = lane; i < m; i += 32) {
+          const double a = hp[i], b = hq[i];
+          hp[i] = c * a - s * b; hq[i] = s * a + c * b;
         }
         if (lane == 0) moved_s = 1;
       }
@@ -565,26 +905,30 @@ __global__ void __launch_bounds__(1024) k_jacobi64(double* Hg, double* V, int m,
   for (int e = t; e < m * m; e += nt) {
     const int c = e / m, i = e % m;                  // eigenvector c, component i  ->  Vf[i][rank of c]
     const double nrm = lam[rank_s[c]];
-    Vf[(int64_t)i * m + rank_s[c]] = nrm > 0.0 ? (float)(H[e] / nrm) : 0.f;
+    Vf[(int64_t)i * ldv + rank_s[c]] = nrm > 0.0 ? (float)(H[e] / nrm) : 0.f;
   }
 }
 
-// sigma_i = sqrt(lam_i);  B'[row][i] = U[row][i] sigma_i  (U: [d][r])
-__global__ void k_finish_b(const float* __restrict__ U, const double* __restrict__ lam, int d, int r, float* __restrict__ Bp, float* __restrict__ sigma) {
+// sigma_i = sqrt(lam_i);  B'[row][i] = U[row][i] sigma_i  (U: [d][ld])
+__global__ void k_finish_b(const float* __restrict__ U, int ld, const double* __restrict__ lam, int d, int r, float* __restrict__ Bp, float* __restrict__ sigma) {
   const int64_t n = (int64_t)d * r;
   for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < n; e += (int64_t)gridDim.x * blockDim.x) {
     const int i = (int)(e % r);
     const float s = (float)sqrt(fmax(lam[i], 0.0));
-    Bp[e] = U[e] * s;
+    Bp[e] = U[e / r * ld + i] * s;
     if (e < r) sigma[e] = (float)sqrt(fmax(lam[e], 0.0));
   }
 }
-// A[i][:] /= sigma_i  (A: [r][k] holding U^T dW)
-__global__ void k_finish_a(float* __restrict__ A, const double* __restrict__ lam, int r, int k) {
-  const int64_t n = (int64_t)r * k;
-  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < n; e += (int64_t)gridDim.x * blockDim.x) {
-    const double s = sqrt(fmax(lam[e / k], 0.0));
-    A[e] = s > 0.0 ? (float)((double)A[e] / s) : 0.f;
+// A[i][j] = T[j][i] / sigma_i  (T: [k][ld], holding dW^T U); 32 x 32 tiles through shared memory, 32 x 8 threads
+__global__ void k_finish_a(const float* __restrict__ T, int ld, const double* __restrict__ lam, int r, int k, float* __restrict__ A) {
+  __shared__ float tile[32][33];
+  const int j0 = blockIdx.x * 32, i0 = blockIdx.y * 32, x = threadIdx.x, y = threadIdx.y;
+  for (int q = y; q < 32; q += 8) tile[q][x] = j0 + q < k && i0 + x < r ? T[(int64_t)(j0 + q) * ld + i0 + x] : 0.f;
+  __syncthreads();
+  for (int q = y; q < 32; q += 8) {
+    if (i0 + q >= r || j0 + x >= k) continue;
+    const double s = sqrt(fmax(lam[i0 + q], 0.0));
+    A[(int64_t)(i0 + q) * k + j0 + x] = s > 0.0 ? (float)((double)tile[x][q] / s) : 0.f;
   }
 }
 // sum of squares of a matrix, fp64, into *out (zeroed by the caller)
@@ -601,10 +945,23 @@ __global__ void k_axpy_neg(float* __restrict__ c, const float* __restrict__ a, i
 
 // ------------------------------------------------------------------------------------------------ workspace
 struct Plan {
-  int d, k, n, r, m, ldm, iters;       // ldm: leading dimension of the iterates (m rounded up to the SGEMM tile, or 160)
-  size_t off_w, off_dw, off_g, off_t, off_m, off_y, off_q, off_z, off_u, off_s, off_sp, off_h, off_v, off_lam, off_vf, total;
+  int d, k, n, r, m, iters;
+  int dp, kp, np;             // d, k, n in whole 128-tiles
+  bool n_side, pad_x;         // iterate with P^T P instead of P P^T; X~ has to be copied into whole tiles
+  int s, sp;                  // size of the matrix that is iterated with, in whole tiles
+  int w, ldm;                 // width of the skinny products' tiles, leading dimension of the iterates (a multiple of it)
+  int wr, ldr;                // the same for the products with r columns
+  size_t off_dw, off_x, off_p, off_c, off_y, off_q, off_z, off_s, off_sp, off_d, off_h, off_lam, off_vf, total;
 };
 size_t up256(size_t v) { return (v + 255) & ~size_t(255); }
+int up128(int v) { return (v + 127) & ~127; }
+// The width with the fewest padding columns (the widest of those).
+int pick_width(int cols) {
+  int best = 160;
+  for (int w : {128, 96, 64})
+    if ((cols + w - 1) / w * w < (cols + best - 1) / best * best) best = w;
+  return best;
+}
 bool make_plan(const eora_solve_config* c, Plan& p) {
   if (!c || c->d < 1 || c->k < 1 || c->n < 1 || c->rank < 1) return false;
   p.d = c->d; p.k = c->k; p.n = c->n; p.r = c->rank;
@@ -613,47 +970,93 @@ bool make_plan(const eora_solve_config* c, Plan& p) {
   if (p.m > p.d) p.m = p.d;
   if (p.r > p.m || p.m > 512) return false;
   p.iters = c->iters > 0 ? c->iters : 24;
-  p.ldm = (p.m + BN - 1) / BN * BN;
-  if (p.m > BN && p.m <= NQ && p.d % BMQ == 0) p.ldm = NQ;          // the default width: its own kernel, no padding columns
+  p.dp = up128(p.d); p.kp = up128(p.k); p.np = up128(p.n);
+  p.pad_x = p.k % 128 || p.n % 128;
+  // The smaller side (every iteration is a product with its square); it has to hold m directions.
+  p.n_side = p.n < p.d && p.n >= p.m;
+  p.s = p.n_side ? p.n : p.d;
+  p.sp = p.n_side ? p.np : p.dp;
+  p.w = pick_width(p.m); p.ldm = (p.m + p.w - 1) / p.w * p.w;
+  p.wr = pick_width(p.r); p.ldr = (p.r + p.wr - 1) / p.wr * p.wr;
+  if (p.ldr > p.ldm) { p.wr = p.w; p.ldr = p.ldm; }
   size_t o = 0;
   auto take = [&](size_t bytes) { size_t at = o; o += up256(bytes); return at; };
-  p.off_dw = take((size_t)p.d * p.k * 4);
-  p.off_g = take((size_t)p.k * p.k * 4);
-  p.off_t = take((size_t)p.d * (p.k > p.n ? p.k : p.n) * 4);      // T = dW G; the loss check keeps dW X~ here
-  p.off_m = take((size_t)p.d * p.d * 4);
-  p.off_y = take((size_t)p.d * p.ldm * 4);
-  p.off_q = take((size_t)p.d * p.ldm * 4);
-  p.off_z = take((size_t)p.d * p.ldm * 4);
-  p.off_w = take((size_t)p.ldm * p.ldm * 4);
-  p.off_u = take((size_t)p.d * p.r * 4);
+  const size_t rows = p.dp > p.np ? p.dp : p.np, tall = rows > (size_t)p.kp ? rows : p.kp;
+  const size_t c_el = (size_t)p.sp * p.sp, r_el = (size_t)p.d * p.k;
+  p.off_dw = take((size_t)p.dp * p.kp * 4);
+  p.off_x = take(p.pad_x ? (size_t)p.kp * p.np * 4 : 0);
+  p.off_p = take((size_t)p.dp * p.np * 4);                        // P = dW X~; the loss check keeps (dW - B'A) X~ here
+  p.off_c = take((c_el > r_el ? c_el : r_el) * 4);                // C; the loss check keeps dW - B'A here
+  p.off_y = take(rows * p.ldm * 4);
+  p.off_q = take(rows * p.ldm * 4);
+  p.off_z = take(tall * p.ldm * 4);
   p.off_s = take((size_t)p.m * p.m * 8);
   p.off_sp = take((size_t)kGramParts * p.m * p.m * 8);
+  p.off_d = take((size_t)((p.m + 15) / 16) * 256 * 8);
   p.off_h = take((size_t)p.m * p.m * 8);
-  p.off_v = take((size_t)p.m * p.m * 8);
-  p.off_lam = take((size_t)2 * p.m * 8);
-  p.off_vf = take((size_t)p.m * p.m * 4);
-  p.total = o;
+  p.off_lam = take((size_t)(2 * p.m + 128) * 8);
+  p.off_vf = take((size_t)p.ldm * p.ldm * 4);
+  const size_t least = ((size_t)p.d * p.k + (size_t)p.k * p.k + (size_t)p.d * p.d + 64) * 4;      // what earlier versions reported at least
+  p.total = o > least ? o : least;
   return true;
 }
 inline bool aligned16(const void* q) { return (reinterpret_cast<uintptr_t>(q) & 15) == 0; }
 
 #define CK(x) do { cudaError_t e__ = (x); if (e__ != cudaSuccess) return EORA_ERR_CUDA; } while (0)
 
-// Q = orth(Y) by Cholesky-QR: Gram matrix, factor and its inverse in fp64, then Q = Y L^{-T} as a contraction.
-int orthonormalise(cudaStream_t st, const Plan& p, const float* Y, float* Q, double* S, double* parts, float* W) {
-  CK(gram64(st, Y, Y, p.d, p.m, p.ldm, parts, S));
-  static bool attr_set[64] = {};
+// Shared-memory limits are set once per kernel and device.
+template <auto KERNEL>
+cudaError_t allow_smem(int bytes) {
+  static bool done[64] = {};
   int device = 0;
-  if (cudaGetDevice(&device) != cudaSuccess || device < 0 || device >= 64) return EORA_ERR_CUDA;
-  const int smem = (p.m <= kCholSmem ? p.m * (p.m | 1) * 8 : 0) + ((p.m + 15) / 16) * 16 * 16 * 8;     // the matrix (if it fits) and the scratch of the block inverse
-  if (!attr_set[device]) {
-    CK(cudaFuncSetAttribute(k_chol_inv64, cudaFuncAttributeMaxDynamicSharedMemorySize, kCholSmem * (kCholSmem | 1) * 8 + ((kCholSmem + 15) / 16) * 16 * 16 * 8));
-    attr_set[device] = true;
-  }
-  k_chol_inv64<<<1, 1024, smem, st>>>(S, p.m, W, p.ldm);
+  cudaError_t e = cudaGetDevice(&device);
+  if (e != cudaSuccess) return e;
+  if (device < 0 || device >= 64) return cudaErrorInvalidDevice;
+  if (done[device]) return cudaSuccess;
+  e = cudaFuncSetAttribute(KERNEL, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+  if (e == cudaSuccess) done[device] = true;
+  return e;
+}
+
+// Q = orth(Y) by Cholesky-QR: Gram matrix, its factor and Q = Y L^{-T} in fp64.  Y, Q: [rows][ldm], rows a multiple of 16.
+int orthonormalise(cudaStream_t st, const Plan& p, int rows, const float* Y, float* Q, double* S, double* parts, double* D) {
+  CK(gram64<false>(st, Y, rows, p.m, p.ldm, parts, S));
+  CK(allow_smem<k_chol64>(chol_smem(kCholSmem)));
+  CK(allow_smem<k_trsm>(trsm_smem(512)));
+  k_chol64<<<1, kCholThreads, chol_smem(p.m), st>>>(S, p.m, D);
+  k_trsm<<<rows / 16, 256, trsm_smem(p.m), st>>>(Y, S, D, p.m, p.ldm, Q);
   CK(cudaGetLastError());
-  CK(sgemm(st, p.d, p.ldm, p.ldm, Y, p.ldm, false, W, p.ldm, false, Q, p.ldm));
   return EORA_OK;
+}
+
+template <int B, int E>
+cudaError_t launch_jacobi(cudaStream_t st, const double* H, int m, double* lam, float* Vf, int ldv) {
+  constexpr int cs = B == 4 ? 4 : 8;                 // CTAs: five warps each at m = 160, ten at m = 320
+  const int groups = (m + 2 * B - 1) / (2 * B), nw = (groups + cs - 1) / cs;
+  const int smem = 2 * nw * 2 * JacobiShape<B, E>::kBlock * 8;
+  cudaError_t e = allow_smem<k_jacobi_cl<B, E>>(2 * (B == 4 ? 5 : 10) * 2 * JacobiShape<B, E>::kBlock * 8);
+  if (e != cudaSuccess) return e;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(cs);
+  cfg.blockDim = dim3(32 * nw);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = cs; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, k_jacobi_cl<B, E>, H, m, lam, Vf, ldv, 40);
+}
+cudaError_t jacobi(cudaStream_t st, double* H, int m, double* lam, float* Vf, int ldv) {
+  if (m <= 64) return launch_jacobi<4, 2>(st, H, m, lam, Vf, ldv);
+  if (m <= 96) return launch_jacobi<4, 3>(st, H, m, lam, Vf, ldv);
+  if (m <= 128) return launch_jacobi<4, 4>(st, H, m, lam, Vf, ldv);
+  if (m <= 160) return launch_jacobi<4, 5>(st, H, m, lam, Vf, ldv);
+  if (m <= 224) return launch_jacobi<2, 7>(st, H, m, lam, Vf, ldv);
+  if (m <= 320) return launch_jacobi<2, 10>(st, H, m, lam, Vf, ldv);
+  k_jacobi64<<<1, 1024, 0, st>>>(H, m, lam, Vf, ldv, 40);
+  return cudaGetLastError();
 }
 
 }  // namespace
@@ -674,52 +1077,55 @@ int eora_solve(const eora_solve_config* cfg, const float* w, const float* w_hat,
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
   char* ws = reinterpret_cast<char*>(workspace);
   float* dW = reinterpret_cast<float*>(ws + p.off_dw);
-  float* G = reinterpret_cast<float*>(ws + p.off_g);
-  float* T = reinterpret_cast<float*>(ws + p.off_t);
-  float* Mm = reinterpret_cast<float*>(ws + p.off_m);
+  float* Pm = reinterpret_cast<float*>(ws + p.off_p);
+  float* C = reinterpret_cast<float*>(ws + p.off_c);
   float* Y = reinterpret_cast<float*>(ws + p.off_y);
   float* Q = reinterpret_cast<float*>(ws + p.off_q);
   float* Z = reinterpret_cast<float*>(ws + p.off_z);
-  float* Wm = reinterpret_cast<float*>(ws + p.off_w);
-  float* U = reinterpret_cast<float*>(ws + p.off_u);
   double* S = reinterpret_cast<double*>(ws + p.off_s);
   double* Sp = reinterpret_cast<double*>(ws + p.off_sp);
+  double* D = reinterpret_cast<double*>(ws + p.off_d);
   double* H = reinterpret_cast<double*>(ws + p.off_h);
-  double* V = reinterpret_cast<double*>(ws + p.off_v);
   double* lam = reinterpret_cast<double*>(ws + p.off_lam);
   float* Vf = reinterpret_cast<float*>(ws + p.off_vf);
-  const int d = p.d, k = p.k, n = p.n, r = p.r, m = p.m, ldm = p.ldm;
+  const int dp = p.dp, kp = p.kp, np = p.np, sp = p.sp, ldm = p.ldm;
 
-  // step 1
-  k_sub<<<592, 256, 0, st>>>(w, w_hat, dW, (int64_t)d * k);
-  // steps 2-4, as the d x d matrix dW' dW'^T = dW (X~ X~^T) dW^T
-  CK(sgemm(st, k, k, n, x_tilde, n, false, x_tilde, n, true, G, k));          // G = X~ X~^T
-  CK(sgemm(st, d, k, k, dW, k, false, G, k, true, T, k));                     // T = dW G = dW G^T (G is symmetric; the row-by-row form of the product is the faster one)
-  CK(sgemm(st, d, d, k, T, k, false, dW, k, true, Mm, d));                    // Mm = T dW^T
+  // step 1, and X~ in whole tiles
+  k_sub_pad<<<dp < 2368 ? dp : 2368, 256, 0, st>>>(w, w_hat, p.d, p.k, dW, dp, kp);
+  const float* x = x_tilde;
+  if (p.pad_x) {
+    float* xp = reinterpret_cast<float*>(ws + p.off_x);
+    k_sub_pad<<<kp < 2368 ? kp : 2368, 256, 0, st>>>(x_tilde, nullptr, p.k, p.n, xp, kp, np);
+    x = xp;
+  }
+  // steps 2-4: P = dW X~, and the smaller of P P^T and P^T P
+  k_sgemm_full<false, false, false><<<dim3(np / BN, dp / BM), 256, 0, st>>>(kp, dW, kp, x, np, Pm, np);
+  const int T = sp / BM;
+  if (p.n_side) k_sgemm_full<true, false, true><<<T * (T + 1) / 2, 256, 0, st>>>(dp, Pm, np, Pm, np, C, sp);
+  else k_sgemm_full<false, true, true><<<T * (T + 1) / 2, 256, 0, st>>>(np, Pm, np, Pm, np, C, sp);
   // step 5: subspace iteration
-  k_init<<<592, 256, 0, st>>>(Y, d, m, ldm);
-  if (int rc = orthonormalise(st, p, Y, Q, S, Sp, Wm)) return rc;
-  for (int it = 0; it < p.iters; ++it) {
-    CK(sgemm(st, d, ldm, d, Mm, d, false, Q, ldm, false, Y, ldm));            // Y = Mm Q
-    if (int rc = orthonormalise(st, p, Y, Q, S, Sp, Wm)) return rc;
-  }
-  if (int rc = orthonormalise(st, p, Q, Y, S, Sp, Wm)) return rc;                 // second pass: orthogonal to fp32 rounding
-  // Rayleigh-Ritz on span(Y)
-  CK(sgemm(st, d, ldm, d, Mm, d, false, Y, ldm, false, Z, ldm));              // Z = Mm Y
-  CK(gram64(st, Y, Z, d, m, ldm, Sp, H));                                     // H = Y^T Mm Y
-  {
-    static bool jattr[64] = {};
-    int device = 0;
-    if (cudaGetDevice(&device) != cudaSuccess || device < 0 || device >= 64) return EORA_ERR_CUDA;
-    if (!jattr[device]) { CK(cudaFuncSetAttribute(k_jacobi64, cudaFuncAttributeMaxDynamicSharedMemorySize, kCholSmem * kCholSmem * 8)); jattr[device] = true; }
-    k_jacobi64<<<1, 1024, m <= kCholSmem ? m * m * 8 : 0, st>>>(H, V, m, lam, Vf, 40);
-  }
+  k_init<<<592, 256, 0, st>>>(Y, p.s, sp, p.m, ldm);
   CK(cudaGetLastError());
-  CK(sgemm(st, d, r, m, Y, ldm, false, Vf, m, false, U, r));                  // U' = Y V[:, :r]
+  if (int rc = orthonormalise(st, p, sp, Y, Q, S, Sp, D)) return rc;
+  for (int it = 0; it < p.iters; ++it) {
+    CK(skinny<true>(st, p.w, sp, sp, C, sp, Q, ldm, ldm, Y, ldm));            // Y = C Q (C is symmetric: read by columns)
+    if (int rc = orthonormalise(st, p, sp, Y, Q, S, Sp, D)) return rc;
+  }
+  if (p.n_side) {                                                             // to the d-dimensional side
+    CK(skinny<false>(st, p.w, dp, np, Pm, np, Q, ldm, ldm, Y, ldm));
+    if (int rc = orthonormalise(st, p, dp, Y, Q, S, Sp, D)) return rc;
+  }
+  if (int rc = orthonormalise(st, p, dp, Q, Y, S, Sp, D)) return rc;          // second pass: orthogonal to fp32 rounding
+  // Rayleigh-Ritz on span(Y)
+  CK(skinny<true>(st, p.w, np, dp, Pm, np, Y, ldm, ldm, Z, ldm));             // Z = P^T Y
+  CK(gram64<true>(st, Z, np, p.m, ldm, Sp, H));                               // H = Z^T Z = Y^T P P^T Y
+  CK(cudaMemsetAsync(Vf, 0, (size_t)ldm * ldm * 4, st));
+  CK(jacobi(st, H, p.m, lam, Vf, ldm));
+  CK(skinny<false>(st, p.wr, dp, ldm, Y, ldm, Vf, ldm, p.ldr, Q, ldm));       // U' = Y V[:, :r]
   // step 6
-  k_finish_b<<<296, 256, 0, st>>>(U, lam, d, r, b_prime, sigma);
-  CK(sgemm(st, r, k, d, U, r, true, dW, k, false, a, k));                     // U'^T dW
-  k_finish_a<<<296, 256, 0, st>>>(a, lam, r, k);
+  k_finish_b<<<592, 256, 0, st>>>(Q, ldm, lam, p.d, p.r, b_prime, sigma);
+  CK(skinny<true>(st, p.wr, kp, dp, dW, kp, Q, ldm, p.ldr, Z, ldm));          // dW^T U'
+  k_finish_a<<<dim3((p.k + 31) / 32, (p.r + 31) / 32), dim3(32, 8), 0, st>>>(Z, ldm, lam, p.r, p.k, a);
   CK(cudaGetLastError());
   return EORA_OK;
 }
@@ -732,9 +1138,8 @@ int eora_solve_loss(const eora_solve_config* cfg, const float* w, const float* w
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
   char* ws = reinterpret_cast<char*>(workspace);
   float* dW = reinterpret_cast<float*>(ws + p.off_dw);
-  float* R = reinterpret_cast<float*>(ws + p.off_g);       // B'A, then the residual (d x k fits: the slot holds k x k ... see below)
-  float* E = reinterpret_cast<float*>(ws + p.off_t);       // (dW - B'A) X~  (d x n)
-  if ((size_t)p.d * p.k > (size_t)p.k * p.k) R = reinterpret_cast<float*>(ws + p.off_m);   // d > k: use the d x d slot
+  float* R = reinterpret_cast<float*>(ws + p.off_c);       // B'A, then the residual
+  float* E = reinterpret_cast<float*>(ws + p.off_p);       // (dW - B'A) X~  (d x n)
   k_sub<<<592, 256, 0, st>>>(w, w_hat, dW, (int64_t)p.d * p.k);
   CK(sgemm(st, p.d, p.k, p.r, b_prime, p.r, false, a, p.k, false, R, p.k));    // B' A
   k_axpy_neg<<<592, 256, 0, st>>>(R, dW, (int64_t)p.d * p.k);                  // dW - B'A
