@@ -456,24 +456,38 @@ cudaError_t gram64(cudaStream_t st, const float* A, int rows, int m, int ld, dou
   return cudaGetLastError();
 }
 
+// 1 / sqrt(d) in fp64 from the fp32 value by Newton's method (each step doubles the digits; the argument's exponent is taken
+// out first, so every positive d works).
+__device__ __forceinline__ double rsqrt_newton(double d) {
+  const int e = (__double2hiint(d) >> 20) - 1023, half = e >> 1;          // d = 2^(2 half) * [1, 4)
+  const double x = __hiloint2double(__double2hiint(d) - (half << 21), __double2loint(d));
+  double y = (double)rsqrtf((float)x);
+#pragma unroll
+  for (int i = 0; i < 2; ++i) y = fma(y * 0.5, fma(-x * y, y, 1.0), y);
+  return __hiloint2double(__double2hiint(y) - (half << 20), __double2loint(y));
+}
+
 // Cholesky S = L L^T (fp64) of an m x m Gram matrix by one CTA, right-looking in panels of 16 columns:
 //   (A) one warp factors the 16 x 16 diagonal block in registers (lane = row) and inverts it,
 //   (B) the rows below are multiplied with the inverse, one element per thread,
-//   (C) the trailing lower triangle is updated in 4 x 4 tiles (16 products per 8 16-byte reads of shared memory).
+//   (C) the trailing lower triangle is updated in 4 x 4 tiles.  Warp 0 takes the tiles of the next diagonal block first and goes on
+//       with (A) for the next panel while the others update the rest.
+// The chain of (A)s is what bounds it: a pivot, its root, a column and an update, 16 times per panel.
 // Writes L over S (lower triangle, global) and the inverses of the diagonal blocks; Q = Y L^{-T} follows by k_trsm.  A small multiple
 // of the trace is added to the diagonal first, so that a rank-deficient iterate still factors.  In shared memory up to
 // m = kCholSmem, else in place in global memory (L2).  m = 160: 300 us with an explicit inverse and unblocked updates before.
-constexpr int kCholSmem = 160, kPanPitch = 18;
+constexpr int kCholSmem = 160;
 constexpr int kCholThreads = 512;
-__host__ __device__ constexpr int chol_smem(int m) { return ((m <= kCholSmem ? m * (m | 1) : 0) + m * kPanPitch) * 8 + 16; }
+__host__ __device__ constexpr int pan_pitch(int m) { return (m + 5) / 4 * 4 + 2; }      // (even, and rows of the panel on different banks)
+__host__ __device__ constexpr int chol_smem(int m) { return ((m <= kCholSmem ? m * (m | 1) : 0) + 16 * pan_pitch(m)) * 8 + 16; }
 __global__ void __launch_bounds__(kCholThreads) k_chol64(double* Sg, int m, double* __restrict__ Dinv) {
   extern __shared__ __align__(16) double sm[];
   __shared__ double dv[16][17], shift_s;
   const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
   const bool in_smem = m <= kCholSmem;
-  const int ls = in_smem ? (m | 1) : m;
-  double* pan = sm;                                  // [m][kPanPitch]
-  double* S = in_smem ? sm + m * kPanPitch : Sg;
+  const int ls = in_smem ? (m | 1) : m, lp = pan_pitch(m);
+  double* pan = sm;                                  // [16][lp]: the panel by columns
+  double* S = in_smem ? sm + 16 * lp : Sg;
   if (in_smem)
     for (int i = warp; i < m; i += kCholThreads / 32)
       for (int j = lane; j <= i; j += 32) S[i * ls + j] = Sg[(int64_t)i * m + j];
@@ -489,59 +503,57 @@ __global__ void __launch_bounds__(kCholThreads) k_chol64(double* Sg, int m, doub
   const double shift = shift_s;
   for (int i = t; i < m; i += kCholThreads) S[(int64_t)i * ls + i] += shift;
   __syncthreads();
-  for (int j0 = 0; j0 < m; j0 += 16) {
-    if (warp == 0) {                                 // (A); lanes 16..31 repeat lanes 0..15
-      const int r = lane & 15, gi = j0 + r;
-      double a[16], x[16], rinv = 0.0;
+  auto diagonal = [&](int j0) {                      // (A), one warp; lanes 16..31 repeat lanes 0..15
+    const int r = lane & 15, gi = j0 + r;
+    double a[16], x[16], rinv = 0.0;
 #pragma unroll
-      for (int q = 0; q < 16; ++q) a[q] = gi < m && q <= r ? S[(int64_t)gi * ls + j0 + q] : (q == r ? 1.0 : 0.0);      // past m: identity
+    for (int q = 0; q < 16; ++q) a[q] = gi < m && q <= r ? S[(int64_t)gi * ls + j0 + q] : (q == r ? 1.0 : 0.0);      // past m: identity
 #pragma unroll
-      for (int k = 0; k < 16; ++k) {
-        double d = __shfl_sync(0xffffffffu, a[k], k);
-        d = d > shift * 1e-3 ? d : shift * 1e-3;
-        const double ri = rsqrt(d);
-        if (r == k) { a[k] = d * ri; rinv = ri; }
-        else if (r > k) a[k] *= ri;
+    for (int k = 0; k < 16; ++k) {
+      double d = __shfl_sync(0xffffffffu, a[k], k);
+      d = d > shift * 1e-3 ? d : shift * 1e-3;
+      const double ri = rsqrt_newton(d);
+      a[k] = r == k ? d * ri : a[k] * ri;            // (rows above k: never read)
+      if (r == k) rinv = ri;
 #pragma unroll
-        for (int c = k + 1; c < 16; ++c) {
-          const double l = __shfl_sync(0xffffffffu, a[k], c);
-          if (r >= c) a[c] -= a[k] * l;
-        }
+      for (int c = k + 1; c < 16; ++c) a[c] = fma(-a[k], __shfl_sync(0xffffffffu, a[k], c), a[c]);
+    }
+    // column r of the inverse by forward substitution
+#pragma unroll
+    for (int i = 0; i < 16; ++i) {
+      double v = i == r ? 1.0 : 0.0, u = 0.0;
+#pragma unroll
+      for (int q = 0; q < i; ++q) {
+        const double l = __shfl_sync(0xffffffffu, a[q], i);
+        if (q & 1) u = fma(-l, x[q], u); else v = fma(-l, x[q], v);
       }
-      // column r of the inverse by forward substitution
+      x[i] = (v + u) * __shfl_sync(0xffffffffu, rinv, i);
+    }
+    if (lane < 16) {
 #pragma unroll
-      for (int i = 0; i < 16; ++i) {
-        double v = i == r ? 1.0 : 0.0, u = 0.0;
-#pragma unroll
-        for (int q = 0; q < i; ++q) {
-          const double l = __shfl_sync(0xffffffffu, a[q], i);
-          if (q & 1) u -= l * x[q]; else v -= l * x[q];
-        }
-        x[i] = (v + u) * __shfl_sync(0xffffffffu, rinv, i);
-      }
-      if (lane < 16) {
-#pragma unroll
-        for (int q = 0; q < 16; ++q) {
-          if (gi < m && q <= r) S[(int64_t)gi * ls + j0 + q] = a[q];
-          dv[q][r] = x[q];
-          Dinv[(int64_t)(j0 + q) * 16 + r] = x[q];
-        }
+      for (int q = 0; q < 16; ++q) {
+        if (gi < m && q <= r) S[(int64_t)gi * ls + j0 + q] = a[q];
+        dv[q][r] = x[q];
+        Dinv[(int64_t)(j0 + q) * 16 + r] = x[q];
       }
     }
-    __syncthreads();
+  };
+  if (warp == 0) diagonal(0);
+  __syncthreads();
+  for (int j0 = 0; j0 < m; j0 += 16) {
     const int j1 = j0 + 16, R = m - j1;
     if (R <= 0) break;
     for (int e = t; e < R * 16; e += kCholThreads) {       // (B)
       const int i = j1 + (e >> 4), c = e & 15;
       const double* ri = S + (int64_t)i * ls + j0;
-      double v = 0.0;
-      for (int q = 0; q <= c; ++q) v = fma(ri[q], dv[c][q], v);
-      pan[i * kPanPitch + c] = v;
+      double v = 0.0, u = 0.0;
+#pragma unroll
+      for (int q = 0; q < 16; q += 2) { v = fma(ri[q], dv[c][q], v); u = fma(ri[q + 1], dv[c][q + 1], u); }      // (zeros past c)
+      pan[c * lp + i] = v + u;
     }
     __syncthreads();
-    for (int e = t; e < R * 16; e += kCholThreads) S[(int64_t)(j1 + (e >> 4)) * ls + j0 + (e & 15)] = pan[(j1 + (e >> 4)) * kPanPitch + (e & 15)];
-    const int T = (R + 3) / 4, tiles = T * (T + 1) / 2;
-    for (int e = t; e < tiles; e += kCholThreads) {         // (C)
+    const int T = (R + 3) / 4, head = T < 4 ? T * (T + 1) / 2 : 10, tiles = T * (T + 1) / 2;      // the first `head` tiles: the next diagonal block
+    auto update = [&](int e) {                              // (C)
       int ti = (int)((sqrtf(8.f * e + 1.f) - 1.f) * 0.5f);
       while ((ti + 1) * (ti + 2) / 2 <= e) ++ti;
       while (ti * (ti + 1) / 2 > e) --ti;
@@ -551,86 +563,89 @@ __global__ void __launch_bounds__(kCholThreads) k_chol64(double* Sg, int m, doub
       for (int i = 0; i < 4; ++i)
 #pragma unroll
         for (int c = 0; c < 4; ++c) acc[i][c] = 0.0;
-#pragma unroll
-      for (int q = 0; q < 16; q += 2) {
-        double2 li[4], lc[4];
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-          li[i] = *reinterpret_cast<const double2*>(pan + min(i0 + i, m - 1) * kPanPitch + q);
-          lc[i] = *reinterpret_cast<const double2*>(pan + min(c0 + i, m - 1) * kPanPitch + q);
-        }
+#pragma unroll 4
+      for (int q = 0; q < 16; ++q) {                        // (the panel's columns are padded: reading past m is in bounds, the sums are not stored)
+        const double2 l0 = *reinterpret_cast<const double2*>(pan + q * lp + i0), l1 = *reinterpret_cast<const double2*>(pan + q * lp + i0 + 2);
+        const double2 m0 = *reinterpret_cast<const double2*>(pan + q * lp + c0), m1 = *reinterpret_cast<const double2*>(pan + q * lp + c0 + 2);
+        const double li[4] = {l0.x, l0.y, l1.x, l1.y}, lc[4] = {m0.x, m0.y, m1.x, m1.y};
 #pragma unroll
         for (int i = 0; i < 4; ++i)
 #pragma unroll
-          for (int c = 0; c < 4; ++c) acc[i][c] = fma(li[i].y, lc[c].y, fma(li[i].x, lc[c].x, acc[i][c]));
+          for (int c = 0; c < 4; ++c) acc[i][c] = fma(li[i], lc[c], acc[i][c]);
       }
 #pragma unroll
       for (int i = 0; i < 4; ++i)
 #pragma unroll
         for (int c = 0; c < 4; ++c)
           if (i0 + i < m && c0 + c <= i0 + i) S[(int64_t)(i0 + i) * ls + c0 + c] -= acc[i][c];
+    };
+    if (warp == 0) {
+      if (lane < head) update(lane);
+      __syncwarp();
+      diagonal(j1);                                         // (dv was read in (B))
+    } else {
+      const int wt = t - 32;
+      for (int e = wt; e < R * 16; e += kCholThreads - 32) S[(int64_t)(j1 + (e >> 4)) * ls + j0 + (e & 15)] = pan[(e & 15) * lp + j1 + (e >> 4)];
+      for (int e = head + wt; e < tiles; e += kCholThreads - 32) update(e);
     }
     __syncthreads();
   }
-  if (in_smem) {
-    __syncthreads();
+  if (in_smem)
     for (int i = warp; i < m; i += kCholThreads / 32)
       for (int j = lane; j <= i; j += 32) Sg[(int64_t)i * m + j] = S[i * ls + j];
-  }
 }
 
 // Q = Y L^{-T}, row by row (fp64 inside): a CTA takes 16 rows, half a warp each (lane = column of the panel); panel by panel of 16
-// columns  q_p = (y_p - sum_{c < 16 p} q_c L[p][c]^T) Dinv_p^T.  A panel's 16 rows of L come by cp.async, one panel ahead.
+// columns  q_p = (y_p - sum_{c < 16 p} q_c L[p][c]^T) Dinv_p^T.  A panel's 16 rows of L and its Dinv come by cp.async, one panel
+// ahead, its column of Y by a load one panel ahead.
 __host__ __device__ constexpr int trsm_pitch(int m) { return (m + 15) / 16 * 16 + 2; }
-__host__ __device__ constexpr int trsm_smem(int m) { return 3 * 16 * trsm_pitch(m) * 8; }
+__host__ __device__ constexpr int trsm_smem(int m) { return (3 * 16 * trsm_pitch(m) + 2 * 16 * 18) * 8; }
 __global__ void __launch_bounds__(256) k_trsm(const float* __restrict__ Y, const double* __restrict__ L, const double* __restrict__ Dinv, int m, int ld,
                                               float* __restrict__ Q) {
   extern __shared__ __align__(16) double smt[];
   const int lq = trsm_pitch(m);
   double* qd = smt;                                  // [16][lq]
   double* lp = smt + 16 * lq;                        // [2][16][lq]
+  double* di = smt + 48 * lq;                        // [2][16][18]
   const int t = threadIdx.x, r = t >> 4, c = t & 15;
   const int64_t row = (int64_t)blockIdx.x * 16 + r;
   const int np = (m + 15) / 16;
+  auto copy8 = [](double* dst, const double* src) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src) : "memory");
+  };
   auto fetch = [&](int p) {                          // rows 16 p .. of L, columns before 16 p
     double* dst = lp + (p & 1) * 16 * lq;
+    copy8(di + (p & 1) * 16 * 18 + r * 18 + c, Dinv + (int64_t)(16 * p + r) * 16 + c);
     for (int q = c; q < 16 * p; q += 16) {
-      if (16 * p + r < m) {
-        const uint32_t d = (uint32_t)__cvta_generic_to_shared(dst + r * lq + q);
-        asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(d), "l"(L + (int64_t)(16 * p + r) * m + q) : "memory");
-      } else {
-        dst[r * lq + q] = 0.0;
-      }
+      if (16 * p + r < m) copy8(dst + r * lq + q, L + (int64_t)(16 * p + r) * m + q);
+      else dst[r * lq + q] = 0.0;
     }
     asm volatile("cp.async.commit_group;" ::: "memory");
   };
-  if (np > 1) fetch(1);
+  fetch(0);
+  float y = Y[row * ld + c];
   for (int p = 0; p < np; ++p) {
-    double dr[16];
-#pragma unroll
-    for (int q = 0; q < 16; ++q) dr[q] = __ldg(Dinv + (int64_t)(16 * p + c) * 16 + q);
-    double v0 = (double)Y[row * ld + 16 * p + c], v1 = 0.0;
-    if (p > 0) {
-      asm volatile("cp.async.wait_group 0;" ::: "memory");
-      __syncthreads();                               // panel p is there, and panel p - 1 has been read
-      if (p + 1 < np) fetch(p + 1);
-      const double* lr = lp + (p & 1) * 16 * lq + c * lq;
-      const double* qr = qd + r * lq;
+    asm volatile("cp.async.wait_group 0;" ::: "memory");
+    __syncthreads();                                 // panel p is there, and panel p - 1 has been read
+    if (p + 1 < np) fetch(p + 1);
+    double v[4] = {(double)y, 0.0, 0.0, 0.0};
+    if (p + 1 < np) y = Y[row * ld + 16 * (p + 1) + c];
+    const double* lr = lp + (p & 1) * 16 * lq + c * lq;
+    const double* qr = qd + r * lq;
 #pragma unroll 4
-      for (int q = 0; q < 16 * p; q += 2) {
-        const double2 a = *reinterpret_cast<const double2*>(qr + q), b = *reinterpret_cast<const double2*>(lr + q);
-        v0 = fma(-a.x, b.x, v0); v1 = fma(-a.y, b.y, v1);
-      }
+    for (int q = 0; q < 16 * p; q += 4) {
+      const double2 a = *reinterpret_cast<const double2*>(qr + q), b = *reinterpret_cast<const double2*>(lr + q);
+      const double2 a2 = *reinterpret_cast<const double2*>(qr + q + 2), b2 = *reinterpret_cast<const double2*>(lr + q + 2);
+      v[0] = fma(-a.x, b.x, v[0]); v[1] = fma(-a.y, b.y, v[1]); v[2] = fma(-a2.x, b2.x, v[2]); v[3] = fma(-a2.y, b2.y, v[3]);
     }
-    const double v = v0 + v1;
-    double o = 0.0;
+    const double w = (v[0] + v[1]) + (v[2] + v[3]);
+    const double* dr = di + (p & 1) * 16 * 18 + c * 18;
+    double o[4] = {0.0, 0.0, 0.0, 0.0};
 #pragma unroll
-    for (int q = 0; q < 16; ++q) {
-      const double u = __shfl_sync(0xffffffffu, v, q, 16);
-      o = fma(u, dr[q], o);                          // (Dinv is lower triangular: zeros past c)
-    }
-    qd[r * lq + 16 * p + c] = o;
-    Q[row * ld + 16 * p + c] = (float)o;
+    for (int q = 0; q < 16; ++q) o[q & 3] = fma(__shfl_sync(0xffffffffu, w, q, 16), dr[q], o[q & 3]);      // (Dinv is lower triangular: zeros past c)
+    const double res = (o[0] + o[1]) + (o[2] + o[3]);
+    qd[r * lq + 16 * p + c] = res;
+    Q[row * ld + 16 * p + c] = (float)res;
     __syncwarp();
   }
   for (int i = 16 * np + c; i < ld; i += 16) Q[row * ld + i] = 0.f;
