@@ -633,7 +633,7 @@ int eora_linear_last_device_status(eora_linear_t obj) {
     char* lo = reinterpret_cast<char*>(h->t_part);
     char* hi = reinterpret_cast<char*>(h->dev_status) + 256;
     if (cudaMemset(lo, 0, (size_t)(hi - lo)) != cudaSuccess) return EORA_ERR_CUDA;
-    if (decode_tc_reset(h, nullptr) != cudaSuccess || prefill_reset(h, nullptr) != cudaSuccess || cudaDeviceSynchronize() != cudaSuccess) return EORA_ERR_CUDA;
+    if (decode_tc_reset(h, nullptr) != cudaSuccess || cudaDeviceSynchronize() != cudaSuccess) return EORA_ERR_CUDA;
   }
   return v;
 }

@@ -53,10 +53,9 @@ struct PrefillArgs {
   int nkb_w, nkb_b;  // k-blocks of each part
   int sx, sw;        // stages of the ring (sx == sw: token tiles first, weight tiles from w_off on)
   int w_off;         // byte offset of the weight ring (after sx token tiles of bt*128 bytes)
-  // Few tokens (one token tile): the reduction axis is split over ksplit CTAs per tile (kchunk k-blocks each; the
-  // first one also takes the K-extension).  Each adds its accumulator to ws (fp32, [tokens][ld_ws], zero between
-  // launches) and takes a ticket of its tile; the CTA that takes the last one converts the sums to `out` and puts
-  // ws and the ticket back to zero.  ksplit == 1: the accumulator goes straight to `out`.
+  // Where the tiles leave SMs idle, the reduction axis of a tile is split over the ksplit CTAs of a cluster (the first one
+  // also takes the K-extension; split_lo says which backbone k-blocks are whose).  The
+  // partial accumulators meet in distributed shared memory: every CTA finishes every ksplit-th chunk of 32 tokens.
   // Fused layers (stacked along the weight rows): layer i owns rows [sub_row0[i], sub_row0[i + 1]),
   // writes to outs[i] (leading dimension sub_ld[i]) and takes columns [i * t_sub, (i + 1) * t_sub) of t in the
   // K-extension.  A plain layer: n_sub = 1, sub_row0 = {0, n_valid}, outs[0] = out.
@@ -65,10 +64,8 @@ struct PrefillArgs {
   void* outs[4];
   int sub_ld[4];
   int t_sub;
-  int ksplit, kchunk;
-  float* ws;
-  int ld_ws;
-  uint32_t* tickets;
+  int ksplit;
+  int wait_x;          // X comes from the launch in front: wait for it before the first token tile (else only before t)
   int* dev_status;
   long long* trace;  // optional: for CTA (0,0), 4 clock64() stamps per k-block (token copy requested, W ready, X ready, MMA issued),
                      // then one more row: kernel entry, set-up done, accumulators complete, epilogue done
@@ -79,15 +76,16 @@ struct PrefillArgs {
 
 struct PrefillState {
   __half* x16;       // fp16 copy of a bf16 X, [max_m][d_in] (bf16 handles only)
-  // split-K workspace of launches with few tokens (see PrefillArgs::ksplit): sums and tickets of the main product
-  // and of t = X.A; one allocation, zero between launches
-  void* split_mem;
-  size_t split_bytes;
-  float* ws_y; float* ws_t;
-  uint32_t* tk_y; uint32_t* tk_t;
 };
 
-constexpr int kThinTokens = 64;        // launches of up to this many tokens may split the reduction axis
+// First backbone k-block of split s: even shares of all k-blocks, the extension being part of the first; if the extension is more than
+// a share, the others share the backbone.  (each_tiling sees to it that every split has some.)
+__device__ __forceinline__ int split_lo(const PrefillArgs& p, int s) {
+  if (s <= 0) return 0;
+  if (s >= p.ksplit) return p.nkb_w;
+  const int total = p.nkb_w + p.nkb_b;
+  return p.nkb_b > total / p.ksplit ? (s - 1) * p.nkb_w / (p.ksplit - 1) : s * total / p.ksplit - p.nkb_b;
+}
 
 // ---------------------------------------------------------------------------------------------- PTX
 __device__ __forceinline__ void tma_load_2d(void* dst, const CUtensorMap* tm, int c0, int c1, uint64_t* bar) {
@@ -382,20 +380,21 @@ __global__ void __launch_bounds__(kThreadsP, 1) k_prefill(const __grid_constant_
   __shared__ uint32_t tmem_base_s;
   __shared__ uint32_t sp_lut[16];        // 2:4 expansion selectors (2:4 backbones only)
   __shared__ int fail_s;                 // set by an epilogue warp whose bounded wait ran out
-  __shared__ int last_s;                 // split-K: this CTA took its tile's last ticket
   // 1024-byte alignment of the operand tiles (the swizzle pattern is anchored at 1 KB)
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
 
-  // Programmatic dependent launch: a kernel launched behind this one with the serialisation attribute may
-  // start at once (the main product behind the launch that computes t; see launch_prefill_forward).
-  asm volatile("griddepcontrol.launch_dependents;");
+  // Programmatic dependent launch: a kernel launched behind this one with the serialisation attribute may start early.  A launch
+  // that waits for X lets it go only after that wait: the main product behind the launch that computes t starts
+  // without waiting for anything, and reads the same X.
+  if (!p.wait_x) asm volatile("griddepcontrol.launch_dependents;");
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const bool small = (int)blockIdx.x < p.n_small;
   const int big_id = (int)blockIdx.x - p.n_small;
   const int bt = small ? kSmallTile : p.bt;                 // tokens of this CTA's tile (the MMA N)
   const int rows = small ? kSmallTile : p.rows;
-  // big tiles: row tile fastest, then the split of the reduction axis, then the token tile
-  const int tile_x = big_id % p.big_x, split = small ? 0 : (big_id / p.big_x) % p.ksplit, tile_y = big_id / (p.big_x * p.ksplit);
+  // big tiles: the split of the reduction axis fastest (a cluster), then the row tile, then the token tile
+  const int tile = big_id / p.ksplit, split = small ? 0 : big_id - tile * p.ksplit;
+  const int tile_x = tile % p.big_x, tile_y = tile / p.big_x;
   const int n0 = small ? p.n_split + ((int)blockIdx.x % p.small_x) * kSmallTile : tile_x * rows;
   const int m0 = small ? ((int)blockIdx.x / p.small_x) * kSmallTile : tile_y * bt;
   int sub = 0;                                              // fused layers: whose rows these are (tiles never straddle)
@@ -408,7 +407,7 @@ __global__ void __launch_bounds__(kThreadsP, 1) k_prefill(const __grid_constant_
   const int nh = (rows > BN_W && n_end - n0 > BN_W) ? 2 : 1;   // 128-row halves of this CTA that hold real rows
   const CUtensorMap* map_x = small ? &tm_x_small : &tm_x;
   const CUtensorMap* map_t = small ? &tm_t_small : &tm_t;
-  const int kw_lo = split * p.kchunk, kw_hi = min(p.nkb_w, kw_lo + p.kchunk);
+  const int kw_lo = split_lo(p, split), kw_hi = split_lo(p, split + 1);
   const int nkw = kw_hi - kw_lo;
   const int nkb_ext = split == 0 ? p.nkb_b : 0;             // the K-extension goes with the first split
   const int nkb = nkw + nkb_ext;
@@ -441,6 +440,10 @@ __global__ void __launch_bounds__(kThreadsP, 1) k_prefill(const __grid_constant_
   if (warp == 0) {
     // ------------------------------------------------------------------ TMA producer (token tiles)
     if (lane == 0) {
+      if (p.wait_x) {
+        asm volatile("griddepcontrol.wait;" ::: "memory");
+        asm volatile("griddepcontrol.launch_dependents;");
+      }
       int s = 0, wrap = 0;                          // ring slot of iteration `it`, and how often it has been used before
       for (int it = 0; it < nkb; ++it) {
         if (wrap > 0 && !mbar_wait(empty_w + s, (wrap - 1) & 1, p.dev_status)) break;
@@ -451,7 +454,7 @@ __global__ void __launch_bounds__(kThreadsP, 1) k_prefill(const __grid_constant_
           tma_load_2d(xt, map_x, (kw_lo + it) * BK, m0, full_w + s);
         } else {
           // t comes from the previous launch, which may still be running: everything up to here overlapped with it
-          if (it == nkw) asm volatile("griddepcontrol.wait;" ::: "memory");
+          if (it == nkw && !p.wait_x) asm volatile("griddepcontrol.wait;" ::: "memory");
           tma_load_2d(xt, map_t, (it - nkw) * BK + sub * p.t_sub, m0, full_w + s);
         }
         if (++s == p.sw) { s = 0; ++wrap; }
@@ -496,128 +499,82 @@ __global__ void __launch_bounds__(kThreadsP, 1) k_prefill(const __grid_constant_
       ok = dequant_part<WF>(p.w, n0, kw_lo, kw_hi, 0, tile, kphase, kstep, lane, smem, p, full_w, empty_w, lut);
       if (ok && nkb_ext > 0) ok = dequant_part<BF>(p.b, n0, 0, nkb_ext, nkw, tile, kphase, kstep, lane, smem, p, full_w, empty_w, lut);
     }
-    {
-      // Epilogue: all sixteen warps, as four groups of four.  A warp can read the quarter of the TMEM lanes
-      // that its index selects (warp % 4 == dw % 4), i.e. accumulator rows (= weight rows n) 32 * (dw % 4) ...
-      // of each half; columns are tokens.  The chunks of 32 tokens are dealt to the groups round-robin.
-      if (ok) ok = mbar_wait_warp(&acc_full, 0, p.dev_status, lane);
-      // the warps meet at barriers below: they must all take the same way
-      if (!ok) *reinterpret_cast<volatile int*>(&fail_s) = 1;
-      asm volatile("bar.sync 1, 512;" ::: "memory");
-      ok = *reinterpret_cast<volatile int*>(&fail_s) == 0;
-      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-      if (dw == 0 && lane == 0) { PTRACE(nkb, 2); CTRACE(1); }
-      const int grp = dw >> 2, lq = dw & 3;
-      const int nl = lq * 32 + lane;                     // local weight row inside the half = thread index inside the group
-      const int nchunk = (bt + 31) >> 5;
-      const uint32_t lane_base = tmem_d + ((uint32_t)(lq * 32) << 16);
-      if (p.ksplit > 1) {
-        // Split reduction axis: add this CTA's share to the fp32 sums (a thread holds one column n for the 32 tokens of a
-        // chunk; a warp's 32 lanes add 128 contiguous bytes per token), then one ticket per CTA.
-        const int tok_valid = min(bt, p.m - m0);
-        if (ok) {
-          float* wsb = p.ws + (int64_t)m0 * p.ld_ws;
-          for (int hh = 0; hh < nh; ++hh) {
-            const int col = n0 + hh * BN_W + nl;
-            for (int cc = 0; cc < nchunk; ++cc) {
-              if (((hh * nchunk + cc) & 3) != grp) continue;
-              const int c0 = cc * 32;
-              uint32_t v[32];
-              tmem_ld32(lane_base + hh * 256 + (uint32_t)c0, v);
-              asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-              if (col < n_end) {
+    if (ok) ok = mbar_wait_warp(&acc_full, 0, p.dev_status, lane);
+    // the warps meet at barriers below: they must all take the same way
+    if (!ok) *reinterpret_cast<volatile int*>(&fail_s) = 1;
+    asm volatile("bar.sync 1, 512;" ::: "memory");
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    if (dw == 0 && lane == 0) { PTRACE(nkb, 2); CTRACE(1); }
+  }
+
+  // Epilogue: all sixteen dequant warps, as four groups of four.  A warp can read the quarter of the TMEM lanes that its index
+  // selects (warp % 4), i.e. accumulator rows (= weight rows n) 32 * (warp % 4) ... of each half; columns are tokens.  The
+  // accumulator goes out in units of 32 tokens x 128 rows, dealt round-robin to the CTAs of the cluster and to the groups.
+  const int dw = warp - 4, grp = dw >> 2, lq = warp & 3;
+  const int nl = lq * 32 + lane;                         // local weight row inside the half = thread index inside the group
+  const int nchunk = (bt + 31) >> 5, units = nh * nchunk;
+  const uint32_t lane_base = tmem_d + ((uint32_t)(lq * 32) << 16);
+  uint8_t* const parts = smem + 65536;                   // split: the other CTAs' shares of this CTA's units, 16 KB each
+  if (p.ksplit > 1) {
+    __syncwarp();
+    cluster_arrive(); cluster_wait();                    // every CTA's MMAs have completed: the rings are free everywhere
+    const bool live = warp >= 4 && *reinterpret_cast<volatile int*>(&fail_s) == 0;
+    for (int u = grp; live && u < units; u += 4) {
+      const int owner = u % p.ksplit;
+      if (owner == split) continue;
+      const int hh = u / nchunk, c0 = (u - hh * nchunk) * 32;
+      uint32_t v[32];
+      tmem_ld32(lane_base + hh * 256 + (uint32_t)c0, v);
+      asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+      const int slot = (u / p.ksplit) * (p.ksplit - 1) + (split < owner ? split : split - 1);
+      const uint32_t to = mapa(smem_u32(parts + slot * 16384) + nl * 4, (uint32_t)owner);
 #pragma unroll
-                for (int j = 0; j < 32; ++j)
-                  if (c0 + j < tok_valid)
-                    asm volatile("red.global.add.f32 [%0], %1;" ::"l"(wsb + (int64_t)(c0 + j) * p.ld_ws + col), "f"(__uint_as_float(v[j])) : "memory");
-              }
-            }
-          }
-          __threadfence();
-        }
-        asm volatile("bar.sync 1, 512;" ::: "memory");
-        if (dw == 0 && lane == 0) {
-          uint32_t old = 0;
-          uint32_t* tk = p.tickets + tile_y * p.big_x + tile_x;
-          if (ok) asm volatile("atom.acq_rel.gpu.global.add.u32 %0, [%1], %2;" : "=r"(old) : "l"(tk), "r"(1u) : "memory");
-          last_s = (ok && old + 1u == (uint32_t)p.ksplit) ? 1 : 0;
-          if (last_s) *tk = 0u;                          // nobody else touches the ticket any more
-        }
-        asm volatile("bar.sync 1, 512;" ::: "memory");
-        if (*reinterpret_cast<volatile int*>(&last_s)) {
-          __threadfence();
-          // every share is in: sums -> output type, one token row per warp and step, 32 columns per instruction
-          // (all loads of a warp's share first: one round trip to L2, not one per row)
-          const int ncols = min(rows, n_end - n0);
-          const int esz = p.out_dtype == EORA_Y_F32 ? 4 : 2;
-          constexpr int kTok = (kThinTokens + kDqWarps - 1) / kDqWarps, kCol = 2 * BN_W / 32;
-          float f[kTok][kCol];
+      for (int j = 0; j < 32; ++j) asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(to + j * 512), "r"(v[j]) : "memory");
+    }
+    __syncwarp();
+    cluster_arrive(); cluster_wait();
+  }
+  if (warp >= 4 && *reinterpret_cast<volatile int*>(&fail_s) == 0) {
+    // A unit goes through shared memory as [32 tokens][128 n] so that the global stores are 16-byte pieces of rows of Y.
+    // Without a split each group has two buffers of 16 KB and alternates: a buffer is rewritten two units later, after a
+    // barrier that every thread of the group passes only when it has read the buffer out, so one barrier per unit is
+    // enough.  With a split it has one buffer and takes two barriers.
+    const int esz = p.out_dtype == EORA_Y_F32 ? 4 : 2;
+    const int row_sh = esz == 4 ? 5 : 4;                 // log2 of the 16-byte pieces per token row (128 n)
+    uint8_t* const gbuf = smem + grp * (p.ksplit > 1 ? 16384 : 32768);
+    int flip = 0;
+    for (int i = grp; i * p.ksplit + split < units; i += 4) {
+      const int u = i * p.ksplit + split, hh = u / nchunk, c0 = (u - hh * nchunk) * 32;
+      uint8_t* tbuf = gbuf + flip * 16384;
+      if (p.ksplit == 1) flip ^= 1;
+      uint32_t v[32];
+      tmem_ld32(lane_base + hh * 256 + (uint32_t)c0, v);
+      asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+      for (int q = 0; q < p.ksplit - 1; ++q) {
+        const float* src = reinterpret_cast<const float*>(parts + (i * (p.ksplit - 1) + q) * 16384) + nl;
 #pragma unroll
-          for (int i = 0; i < kTok; ++i) {
-            const int tok = dw + i * kDqWarps;
+        for (int j = 0; j < 32; ++j) v[j] = __float_as_uint(__uint_as_float(v[j]) + src[j * 128]);
+      }
 #pragma unroll
-            for (int k = 0; k < kCol; ++k) {
-              const int c = lane + 32 * k;
-              f[i][k] = (tok < tok_valid && c < ncols) ? __ldcg(p.ws + (int64_t)(m0 + tok) * p.ld_ws + n0 + c) : 0.f;
-            }
-          }
-#pragma unroll
-          for (int i = 0; i < kTok; ++i) {
-            const int tok = dw + i * kDqWarps;
-            if (tok >= tok_valid) continue;
-            float* src = p.ws + (int64_t)(m0 + tok) * p.ld_ws + n0;
-            uint8_t* dst = reinterpret_cast<uint8_t*>(out_p) + ((int64_t)(m0 + tok) * ld_o + n0 - col0) * esz;
-#pragma unroll
-            for (int k = 0; k < kCol; ++k) {
-              const int c = lane + 32 * k;
-              if (c >= ncols) continue;
-              src[c] = 0.f;
-              if (p.out_dtype == EORA_Y_F32) reinterpret_cast<float*>(dst)[c] = f[i][k];
-              else if (p.out_dtype == EORA_Y_F16) reinterpret_cast<__half*>(dst)[c] = __float2half_rn(f[i][k]);
-              else reinterpret_cast<__nv_bfloat16*>(dst)[c] = __float2bfloat16_rn(f[i][k]);
-            }
-          }
-        }
-      } else {
-        // A chunk goes through shared memory as [32 tokens][128 n] so that the global stores are 16-byte
-        // pieces of rows of Y.  The rings are free by now (every MMA has completed).  Each group has two
-        // buffers and alternates: a buffer is rewritten two chunks later, after a barrier that every thread of
-        // the group passes only when it has read the buffer out, so one barrier per chunk is enough.
-        const int esz = p.out_dtype == EORA_Y_F32 ? 4 : 2;
-        const int row_sh = esz == 4 ? 5 : 4;             // log2 of the 16-byte pieces per token row (128 n)
-        uint8_t* gbuf = smem + grp * 32768;              // 2 x (32 tokens x 128 n x esz bytes <= 16 KB)
-        int flip = 0;
-        for (int hh = 0; hh < nh && ok; ++hh) {
-          for (int cc = 0; cc < nchunk; ++cc) {
-            if (((hh * nchunk + cc) & 3) != grp) continue;
-            const int c0 = cc * 32;
-            uint8_t* tbuf = gbuf + flip * 16384;
-            flip ^= 1;
-            uint32_t v[32];
-            tmem_ld32(lane_base + hh * 256 + (uint32_t)c0, v);
-            asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-#pragma unroll
-            for (int j = 0; j < 32; ++j) {
-              const float f = __uint_as_float(v[j]);
-              if (p.out_dtype == EORA_Y_F32) reinterpret_cast<float*>(tbuf)[j * BN_W + nl] = f;
-              else if (p.out_dtype == EORA_Y_F16) reinterpret_cast<__half*>(tbuf)[j * BN_W + nl] = __float2half_rn(f);
-              else reinterpret_cast<__nv_bfloat16*>(tbuf)[j * BN_W + nl] = __float2bfloat16_rn(f);
-            }
-            asm volatile("bar.sync %0, 128;" ::"r"(2 + grp) : "memory");
-            const int pieces = 32 << row_sh;
-            for (int i = nl; i < pieces; i += 128) {
-              const int tok = i >> row_sh, piece = i & ((1 << row_sh) - 1);
-              const int row = m0 + c0 + tok, col = n0 + hh * BN_W + piece * (16 / esz);
-              if (c0 + tok < bt && row < p.m && col < n_end) {     // a chunk may reach past the tile's tokens
-                const uint4 val = *reinterpret_cast<const uint4*>(tbuf + (size_t)tok * BN_W * esz + piece * 16);
-                *reinterpret_cast<uint4*>(reinterpret_cast<uint8_t*>(out_p) + ((int64_t)row * ld_o + col - col0) * esz) = val;
-              }
-            }
-          }
+      for (int j = 0; j < 32; ++j) {
+        const float f = __uint_as_float(v[j]);
+        if (p.out_dtype == EORA_Y_F32) reinterpret_cast<float*>(tbuf)[j * BN_W + nl] = f;
+        else if (p.out_dtype == EORA_Y_F16) reinterpret_cast<__half*>(tbuf)[j * BN_W + nl] = __float2half_rn(f);
+        else reinterpret_cast<__nv_bfloat16*>(tbuf)[j * BN_W + nl] = __float2bfloat16_rn(f);
+      }
+      asm volatile("bar.sync %0, 128;" ::"r"(2 + grp) : "memory");
+      const int pieces = 32 << row_sh;
+      for (int e = nl; e < pieces; e += 128) {
+        const int tok = e >> row_sh, piece = e & ((1 << row_sh) - 1);
+        const int row = m0 + c0 + tok, col = n0 + hh * BN_W + piece * (16 / esz);
+        if (c0 + tok < bt && row < p.m && col < n_end) {     // a unit may reach past the tile's tokens
+          const uint4 val = *reinterpret_cast<const uint4*>(tbuf + (size_t)tok * BN_W * esz + piece * 16);
+          *reinterpret_cast<uint4*>(reinterpret_cast<uint8_t*>(out_p) + ((int64_t)row * ld_o + col - col0) * esz) = val;
         }
       }
-      if (dw == 0 && lane == 0) { PTRACE(nkb, 3); CTRACE(2); }
+      if (p.ksplit > 1) asm volatile("bar.sync %0, 128;" ::"r"(2 + grp) : "memory");
     }
+    if (dw == 0 && lane == 0) { PTRACE(nkb, 3); CTRACE(2); }
   }
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
@@ -626,6 +583,8 @@ __global__ void __launch_bounds__(kThreadsP, 1) k_prefill(const __grid_constant_
 
 // n is a multiple of 8 (d_in is a multiple of 128): 16 bytes in, 16 bytes out per step
 __global__ void k_bf16_to_f16(const __nv_bfloat16* in, __half* out, int64_t n) {
+  asm volatile("griddepcontrol.launch_dependents;");
+  asm volatile("griddepcontrol.wait;" ::: "memory");         // `out` may still be read by the launch in front
   for (int64_t i = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) * 8; i < n; i += (int64_t)gridDim.x * blockDim.x * 8) {
     const uint4 v = __ldg(reinterpret_cast<const uint4*>(in + i));
     const uint32_t w[4] = {v.x, v.y, v.z, v.w};
@@ -670,11 +629,11 @@ bool make_map(CUtensorMap* tm, const void* base, int rows, int cols, int ld, int
 
 constexpr int kSmemP = 225 * 1024;
 
-// pdl: the launch may begin while the previous kernel of the stream is still running (it waits, on the
-// device, before it touches what that kernel writes).
+// The launch may begin while the previous kernel of the stream is still running (it waits, on the device, before it touches what
+// that kernel writes).
 template <auto KERNEL>
 cudaError_t launch_p(dim3 grid, int smem, cudaStream_t st, const CUtensorMap& tx, const CUtensorMap& tt, const CUtensorMap& txs,
-                     const CUtensorMap& tts, const PrefillArgs& a, bool pdl) {
+                     const CUtensorMap& tts, const PrefillArgs& a) {
   static bool attr_set[64] = {};   // per kernel and device: the attribute belongs to the device that is current at the call
   int device = 0;
   if (cudaGetDevice(&device) != cudaSuccess || device < 0 || device >= 64) return cudaErrorInvalidDevice;
@@ -688,36 +647,38 @@ cudaError_t launch_p(dim3 grid, int smem, cudaStream_t st, const CUtensorMap& tx
   cfg.blockDim = dim3(kThreadsP);
   cfg.dynamicSmemBytes = (size_t)smem;
   cfg.stream = st;
-  cudaLaunchAttribute attr[1];
+  cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
+  attr[1].id = cudaLaunchAttributeClusterDimension;
+  attr[1].val.clusterDim.x = a.ksplit; attr[1].val.clusterDim.y = 1; attr[1].val.clusterDim.z = 1;
   cfg.attrs = attr;
-  cfg.numAttrs = pdl ? 1 : 0;
+  cfg.numAttrs = 2;
   return cudaLaunchKernelEx(&cfg, KERNEL, tx, tt, txs, tts, a);
 }
 
 template <int WF>
 cudaError_t launch_bf(int bf, dim3 grid, int smem, cudaStream_t st, const CUtensorMap& tx, const CUtensorMap& tt,
-                      const CUtensorMap& txs, const CUtensorMap& tts, const PrefillArgs& a, bool pdl) {
+                      const CUtensorMap& txs, const CUtensorMap& tts, const PrefillArgs& a) {
   switch (bf) {
-    case FMT_F16: return launch_p<k_prefill<WF, FMT_F16>>(grid, smem, st, tx, tt, txs, tts, a, pdl);
-    case FMT_Q4: return launch_p<k_prefill<WF, FMT_Q4>>(grid, smem, st, tx, tt, txs, tts, a, pdl);
-    case FMT_Q8: return launch_p<k_prefill<WF, FMT_Q8>>(grid, smem, st, tx, tt, txs, tts, a, pdl);
-    case FMT_Q3: return launch_p<k_prefill<WF, FMT_Q3>>(grid, smem, st, tx, tt, txs, tts, a, pdl);
-    default: return launch_p<k_prefill<WF, FMT_NONE>>(grid, smem, st, tx, tt, txs, tts, a, pdl);
+    case FMT_F16: return launch_p<k_prefill<WF, FMT_F16>>(grid, smem, st, tx, tt, txs, tts, a);
+    case FMT_Q4: return launch_p<k_prefill<WF, FMT_Q4>>(grid, smem, st, tx, tt, txs, tts, a);
+    case FMT_Q8: return launch_p<k_prefill<WF, FMT_Q8>>(grid, smem, st, tx, tt, txs, tts, a);
+    case FMT_Q3: return launch_p<k_prefill<WF, FMT_Q3>>(grid, smem, st, tx, tt, txs, tts, a);
+    default: return launch_p<k_prefill<WF, FMT_NONE>>(grid, smem, st, tx, tt, txs, tts, a);
   }
 }
 
 cudaError_t launch_any(int wf, int bf, dim3 grid, int smem, cudaStream_t st, const CUtensorMap& tx, const CUtensorMap& tt,
-                       const CUtensorMap& txs, const CUtensorMap& tts, const PrefillArgs& a, bool pdl) {
+                       const CUtensorMap& txs, const CUtensorMap& tts, const PrefillArgs& a) {
   switch (wf) {
-    case FMT_Q4: return launch_bf<FMT_Q4>(bf, grid, smem, st, tx, tt, txs, tts, a, pdl);
-    case FMT_Q3: return launch_bf<FMT_Q3>(bf, grid, smem, st, tx, tt, txs, tts, a, pdl);
-    case FMT_SP24: return launch_bf<FMT_SP24>(bf, grid, smem, st, tx, tt, txs, tts, a, pdl);
-    case FMT_SQ4: return launch_bf<FMT_SQ4>(bf, grid, smem, st, tx, tt, txs, tts, a, pdl);
+    case FMT_Q4: return launch_bf<FMT_Q4>(bf, grid, smem, st, tx, tt, txs, tts, a);
+    case FMT_Q3: return launch_bf<FMT_Q3>(bf, grid, smem, st, tx, tt, txs, tts, a);
+    case FMT_SP24: return launch_bf<FMT_SP24>(bf, grid, smem, st, tx, tt, txs, tts, a);
+    case FMT_SQ4: return launch_bf<FMT_SQ4>(bf, grid, smem, st, tx, tt, txs, tts, a);
     // A as the weight of the first launch (t = X.A): no K-extension there
-    case FMT_F16: return launch_p<k_prefill<FMT_F16, FMT_NONE>>(grid, smem, st, tx, tt, txs, tts, a, pdl);
-    case FMT_Q8: return launch_p<k_prefill<FMT_Q8, FMT_NONE>>(grid, smem, st, tx, tt, txs, tts, a, pdl);
+    case FMT_F16: return launch_p<k_prefill<FMT_F16, FMT_NONE>>(grid, smem, st, tx, tt, txs, tts, a);
+    case FMT_Q8: return launch_p<k_prefill<FMT_Q8, FMT_NONE>>(grid, smem, st, tx, tt, txs, tts, a);
     default: return cudaErrorInvalidValue;
   }
 }
@@ -728,27 +689,68 @@ int fill_stages(PrefillArgs& a) {      // returns the dynamic shared memory to r
   if (a.sw > kMaxWStages) a.sw = kMaxWStages;
   a.sx = a.sw;
   a.w_off = a.sx * a.bt * 128;
-  return a.w_off + a.sw * 2 * BN_W * 128 + 1024;
+  int smem = a.w_off + a.sw * 2 * BN_W * 128;
+  const int units = a.rows / BN_W * ((a.bt + 31) / 32);
+  const int out = a.ksplit > 1 ? 65536 + (units + a.ksplit - 1) / a.ksplit * (a.ksplit - 1) * 16384 : 131072;      // the epilogue's
+  return (out > smem ? out : smem) + 1024;
 }
 
-// Weight rows per CTA: 256 or 128, whichever tiling needs less time counted in waves of sm_count CTAs (a CTA needs an SM
-// of its own).  The dequantisation of a CTA's rows is what bounds its k-block period (1200 cycles for 256 rows, 763 for
-// 128), so a 128-row tile costs 0.64 of a 256-row one.  A last partial wave of 256-row tiles that is at most a quarter
-// of the SMs is covered by small tiles inside the first wave (launch_prefill_forward), counted as half a wave.
-int cta_rows(int n_rows, int m, int bt, int sm_count) {
-  if (n_rows <= BN_W) return 2 * BN_W;
-  const int ty = (m + bt - 1) / bt;
-  const int t256 = ((n_rows + 2 * BN_W - 1) / (2 * BN_W)) * ty, t128 = ((n_rows + BN_W - 1) / BN_W) * ty;
-  const int over = t256 % sm_count;
-  float w256 = (float)(t256 / sm_count);
-  if (over > 0) w256 += (bt == 256 && t256 > sm_count && 4 * over <= sm_count) ? 0.5f : 1.0f;
-  const float w128 = 0.64f * (float)((t128 + sm_count - 1) / sm_count);
-  return w128 < w256 ? BN_W : 2 * BN_W;
+// Tiles of a launch: weight rows and tokens per CTA, CTAs that share a tile's reduction axis.
+struct Tiling { int rows, bt, ks; };
+
+// Shared memory of the split epilogue: four buffers of 16 KB and (ks - 1) shares of every ks-th unit.
+bool split_fits(int rows, int bt, int ks) {
+  const int units = rows / BN_W * ((bt + 31) / 32);
+  return 65536 + (units + ks - 1) / ks * (ks - 1) * 16384 <= kSmemP - 1024;
+}
+// CTAs of clusters of ks that run at once, one per SM (measured: 74 clusters of two, 33 of four, 15 of eight; 148 SMs).
+int at_once(int ks, int sm_count) { return ks == 1 ? sm_count : ks == 2 ? sm_count / 2 * 2 : ks == 4 ? sm_count * 33 / 148 * 4 : sm_count * 15 / 148 * 8; }
+
+// Estimated cycles of a launch.  A k-block takes 1200 cycles with 256 rows and 760 with 128, whatever the tokens (the dequantisation of
+// a CTA's rows and the issue of its MMAs bound it); set-up and first operands 4000; the epilogue 10500 for 256 x 256; meeting in
+// distributed shared memory 3000 more.  A last partial wave of 256-row tiles that is at most a quarter of the SMs is covered by
+// small tiles inside the first wave (launch_prefill_forward), counted as half a wave.
+float tiling_cost(const Tiling& t, int n_rows, int m, int nkb, int sm_count) {
+  const int tiles = (n_rows + t.rows - 1) / t.rows * ((m + t.bt - 1) / t.bt), cap = at_once(t.ks, sm_count), ctas = tiles * t.ks;
+  float waves = (float)((ctas + cap - 1) / cap);
+  const int over = tiles % sm_count;
+  if (t.ks == 1 && t.rows == 2 * BN_W && t.bt == 256 && tiles > sm_count && over > 0 && 4 * over <= sm_count) waves -= 0.5f;
+  return waves * ((float)((nkb + t.ks - 1) / t.ks) * (t.rows == BN_W ? 760.f : 1200.f) + 4000.f + 10500.f * (float)(t.rows * t.bt) / 65536.f +
+                  (t.ks > 1 ? 3000.f : 0.f));
 }
 
-int token_tile(int m) {                // the MMA N: a multiple of 16 up to 256
-  if (m >= 256) return 256;
-  return (m + 15) / 16 * 16;
+int token_tile(int m, int most) {      // the MMA N: a multiple of 16 up to `most`, even tiles
+  const int tiles = (m + most - 1) / most;
+  return ((m + tiles - 1) / tiles + 15) / 16 * 16;
+}
+
+// The tilings of the main product and of t = X.A (t_cols == 0: none) that take least time together.  A CTA of either launch needs
+// an SM of its own and clusters need theirs side by side: if the main launch fits into one wave beside the one for t they
+// overlap to the main product's K-extension; if not, it starts with what t leaves and its last CTAs wait for t.
+struct Tilings { Tiling main, t; };
+template <typename F>
+void each_tiling(int m, int nkb_w, bool only128, F f) {
+  const int bt = m > 1024 ? 256 : token_tile(m, 256);        // (whole tiles for long prompts: a ragged last one costs what a full one does)
+  for (int rows = BN_W; rows <= (only128 ? BN_W : 2 * BN_W); rows += BN_W)
+    for (int ks = 1; ks <= 8 && (ks == 1 || (nkb_w / ks >= 4 && split_fits(rows, bt, ks))); ks *= 2) f(Tiling{rows, bt, ks});
+}
+Tilings pick_tilings(int n_rows, int t_cols, int m, int nkb_w, int nkb_b, int sm_count, bool only128) {
+  Tilings best = {};
+  float best_c = -1.f;
+  auto ctas_of = [&](const Tiling& t, int rows) { return (rows + t.rows - 1) / t.rows * ((m + t.bt - 1) / t.bt) * t.ks; };
+  each_tiling(m, nkb_w, only128, [&](const Tiling& a) {
+    const float cm = tiling_cost(a, n_rows, m, nkb_w + nkb_b, sm_count);
+    const int ctas = ctas_of(a, n_rows);
+    auto take = [&](const Tiling& t, float c) { if (best_c < 0.f || c < best_c) { best_c = c; best = {a, t}; } };
+    if (t_cols == 0) { take(a, cm); return; }
+    each_tiling(m, nkb_w, t_cols <= BN_W, [&](const Tiling& t) {
+      const float ct = tiling_cost(t, t_cols, m, nkb_w, sm_count), tail = (float)nkb_b * (a.rows == BN_W ? 760.f : 1200.f);
+      const int tc = ctas_of(t, t_cols), one_wave = ctas <= at_once(a.ks, sm_count);
+      const bool beside = one_wave && ctas + tc <= at_once(a.ks > t.ks ? a.ks : t.ks, sm_count);
+      take(t, beside ? (cm > ct + tail ? cm : ct + tail) : one_wave ? cm + ct : cm + ct * (float)tc / (float)sm_count);
+    });
+  });
+  return best;
 }
 
 }  // namespace
@@ -775,26 +777,8 @@ cudaError_t prefill_init(Handle* h) {
   *ps = PrefillState();
   cudaError_t e = cudaSuccess;
   if (h->cfg.x_dtype == EORA_X_BF16) e = cudaMalloc(&ps->x16, (size_t)h->cfg.max_m * h->cfg.d_in * 2);
-  if (e == cudaSuccess) {
-    // split-K sums and tickets for launches of up to kThinTokens tokens
-    const size_t tok = (size_t)(h->cfg.max_m < kThinTokens ? h->cfg.max_m : kThinTokens);
-    const size_t rp = (size_t)(h->cfg.rank > 0 ? h->t_cols : 0);
-    const size_t n_all = (size_t)(h->n_sub > 1 ? 16 * h->sub_tile0[h->n_sub] : h->cfg.d_out);
-    const size_t y_b = tok * n_all * 4, t_b = tok * rp * 4;
-    const size_t tky_b = ((n_all + BN_W - 1) / BN_W) * 4, tkt_b = ((rp + BN_W - 1) / BN_W) * 4;
-    auto up = [](size_t v) { return (v + 255) & ~size_t(255); };
-    ps->split_bytes = up(y_b) + up(t_b) + up(tky_b) + up(tkt_b) + 256;
-    e = cudaMalloc(&ps->split_mem, ps->split_bytes);
-    if (e == cudaSuccess) e = cudaMemset(ps->split_mem, 0, ps->split_bytes);
-    char* q = reinterpret_cast<char*>(ps->split_mem);
-    ps->ws_y = reinterpret_cast<float*>(q); q += up(y_b);
-    ps->ws_t = reinterpret_cast<float*>(q); q += up(t_b);
-    ps->tk_y = reinterpret_cast<uint32_t*>(q); q += up(tky_b);
-    ps->tk_t = reinterpret_cast<uint32_t*>(q);
-  }
-  if (e != cudaSuccess) { cudaFree(ps->x16); cudaFree(ps->split_mem); delete ps; return e; }
+  if (e != cudaSuccess) { delete ps; return e; }
   h->prefill_state = ps;
-  h->scratch_bytes += (int64_t)ps->split_bytes;
   return cudaSuccess;
 }
 
@@ -802,25 +786,8 @@ void prefill_free(Handle* h) {
   PrefillState* ps = reinterpret_cast<PrefillState*>(h->prefill_state);
   if (!ps) return;
   cudaFree(ps->x16);
-  cudaFree(ps->split_mem);
   delete ps;
   h->prefill_state = nullptr;
-}
-
-// After a launch that gave up: sums and tickets back to zero.
-cudaError_t prefill_reset(Handle* h, cudaStream_t st) {
-  PrefillState* ps = reinterpret_cast<PrefillState*>(h->prefill_state);
-  if (!ps || !ps->split_mem) return cudaSuccess;
-  return cudaMemsetAsync(ps->split_mem, 0, ps->split_bytes, st);
-}
-
-// How many CTAs share a tile's reduction axis in a launch of few tokens: as many as there are SMs for, each with at
-// least min_kb k-blocks (a CTA's set-up and epilogue are worth about eight of them).
-int pick_ksplit(int tiles, int nkb, int sm_count, int min_kb, int cap) {
-  int s = sm_count / (tiles > 0 ? tiles : 1);
-  if (s > nkb / min_kb) s = nkb / min_kb;
-  if (s > cap) s = cap;
-  return s < 1 ? 1 : s;
 }
 
 cudaError_t launch_prefill_forward(const Handle* h, const void* x, int m, void* const* ys, cudaStream_t st) {
@@ -832,39 +799,36 @@ cudaError_t launch_prefill_forward(const Handle* h, const void* x, int m, void* 
     int64_t n = (int64_t)m * c.d_in;
     int64_t blocks = (n / 8 + 255) / 256;
     if (blocks > h->sm_count * 8) blocks = h->sm_count * 8;
-    k_bf16_to_f16<<<(int)blocks, 256, 0, st>>>(reinterpret_cast<const __nv_bfloat16*>(x), ps->x16, n);
+    cudaLaunchConfig_t cc = {};
+    cc.gridDim = dim3((unsigned)blocks);
+    cc.blockDim = dim3(256);
+    cc.stream = st;
+    cudaLaunchAttribute ca[1];
+    ca[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    ca[0].val.programmaticStreamSerializationAllowed = 1;
+    cc.attrs = ca;
+    cc.numAttrs = 1;
+    cudaError_t e = cudaLaunchKernelEx(&cc, k_bf16_to_f16, reinterpret_cast<const __nv_bfloat16*>(x), ps->x16, n);
+    if (e != cudaSuccess) return e;
     x16 = ps->x16;
   }
   if (mid_supported(h, m)) return launch_mid_forward(h, x16, m, ys, st);
-  const int bt = token_tile(m);
-  PrefillState* pst = reinterpret_cast<PrefillState*>(h->prefill_state);
-  const bool thin = m <= kThinTokens && pst && pst->split_mem;      // one token tile: split the reduction axis instead
+  const bool ab = c.rank > 0;
+  const int nkb_w = c.d_in / BK, nkb_b = ab ? h->r_pad / BK : 0;
+  const int n_rows_all = h->n_sub > 1 ? 16 * h->sub_tile0[h->n_sub] : c.d_out;
+  bool only128 = false;                                       // fused layers: every layer a whole number of tiles
+  for (int i = 0; i < h->n_sub && h->n_sub > 1; ++i) only128 = only128 || h->sub_dout[i] % (2 * BN_W) != 0;
+  const Tilings tls = pick_tilings(n_rows_all, ab ? h->t_cols : 0, m, nkb_w, nkb_b, h->sm_count, only128);
+  const Tiling tl = tls.main;
+  const int bt = tl.bt;
   CUtensorMap tm_x, tm_t;
   if (!make_map(&tm_x, x16, m, c.d_in, c.d_in, bt)) return cudaErrorInvalidValue;
-  const bool ab = c.rank > 0;
   if (ab) {
     if (!make_map(&tm_t, h->t16, m, h->t_cols, h->t_cols, bt)) return cudaErrorInvalidValue;
-    // launch 1: t = X.A with A as the weight (rows = r_pad), written as fp16.  It is a small product (a few
-    // CTAs with token tiles of 128), and the main launch behind it starts at once (programmatic dependent
-    // launch) on the other SMs: the main product needs t only for its last k-blocks and waits for this
-    // launch there, so the two overlap.
-    // Its tile: 128 rows and 128 tokens per CTA give the shortest chain of k-blocks, but a CTA of either
-    // launch needs an SM of its own, so when the main launch fits into one wave the first shape whose CTAs
-    // fit beside it is taken (more rows, then more tokens per CTA: fewer CTAs, longer chain).
-    const int n_rows_all = h->n_sub > 1 ? 16 * h->sub_tile0[h->n_sub] : c.d_out;
-    const int rows_m = thin ? BN_W : cta_rows(n_rows_all, m, bt, h->sm_count);
-    const int main_tiles = ((n_rows_all + rows_m - 1) / rows_m) * ((m + bt - 1) / bt);
-    const int room = main_tiles <= h->sm_count ? h->sm_count - main_tiles : h->sm_count;
-    int rows_t = 2 * BN_W, bt_t = bt;
-    {
-      const int cand[4][2] = {{BN_W, 128}, {2 * BN_W, 128}, {BN_W, 256}, {2 * BN_W, 256}};
-      for (int i = 0; i < 4; ++i) {
-        const int rr = h->t_cols > BN_W ? cand[i][0] : 2 * BN_W;    // one half of rows at most: the tile height does not matter
-        const int tt = cand[i][1] < bt ? cand[i][1] : bt;
-        rows_t = rr; bt_t = tt;
-        if (((h->t_cols + rr - 1) / rr) * ((m + tt - 1) / tt) <= room) break;
-      }
-    }
+    // launch 1: t = X.A with A as the weight (rows = r_pad), written as fp16.  It is a small product, and the main launch
+    // behind it starts on the other SMs while it runs (programmatic dependent launch): the main product needs t only
+    // for its last k-blocks and waits for this launch there.
+    const int rows_t = tls.t.rows, bt_t = tls.t.bt;
     CUtensorMap tm_xt;
     if (!make_map(&tm_xt, x16, m, c.d_in, c.d_in, bt_t)) return cudaErrorInvalidValue;
     PrefillArgs a = {};
@@ -875,19 +839,10 @@ cudaError_t launch_prefill_forward(const Handle* h, const void* x, int m, void* 
     a.n_small = 0; a.small_x = 1; a.n_split = a.n_valid; a.big_x = (h->t_cols + a.rows - 1) / a.rows;
     a.n_sub = 1; a.sub_row0[0] = 0; a.outs[0] = a.out; a.sub_ld[0] = a.ld_out; a.t_sub = 0;
     for (int i = 1; i < 5; ++i) a.sub_row0[i] = a.n_valid;
-    a.ksplit = 1; a.kchunk = a.nkb_w; a.ws = nullptr; a.ld_ws = 0; a.tickets = nullptr;
-    if (thin) {
-      // t is the head of the chain (the main product waits for it in front of its K-extension): as short as possible
-      a.rows = h->t_cols > BN_W ? BN_W : a.rows;
-      a.big_x = (h->t_cols + a.rows - 1) / a.rows;
-      a.ksplit = pick_ksplit(a.big_x, a.nkb_w, h->sm_count / 4, 4, 16);
-      a.kchunk = (a.nkb_w + a.ksplit - 1) / a.ksplit;
-      a.ksplit = (a.nkb_w + a.kchunk - 1) / a.kchunk;
-      a.ws = pst->ws_t; a.ld_ws = h->t_cols; a.tickets = pst->tk_t;
-    }
+    a.ksplit = tls.t.ks; a.wait_x = 1;
     const int smem_t = fill_stages(a);
     dim3 grid(a.big_x * a.ksplit * ((m + bt_t - 1) / bt_t), 1, 1);
-    cudaError_t e = launch_any(h->a.fmt, FMT_NONE, grid, smem_t, st, tm_xt, tm_xt, tm_xt, tm_xt, a, false);
+    cudaError_t e = launch_any(h->a.fmt, FMT_NONE, grid, smem_t, st, tm_xt, tm_xt, tm_xt, tm_xt, a);
     if (e != cudaSuccess) return e;
   } else {
     tm_t = tm_x;
@@ -908,24 +863,9 @@ cudaError_t launch_prefill_forward(const Handle* h, const void* x, int m, void* 
   }
   a.nkb_w = c.d_in / BK; a.nkb_b = ab ? h->r_pad / BK : 0; a.dev_status = h->dev_status;
   a.trace = reinterpret_cast<long long*>(h->trace);
-  a.rows = cta_rows(n_valid, m, bt, h->sm_count);
-  for (int i = 0; i < h->n_sub && h->n_sub > 1; ++i)          // fused layers: every layer a whole number of tiles
-    if (h->sub_dout[i] % (2 * BN_W)) a.rows = BN_W;
+  a.rows = tl.rows;
   a.n_small = 0; a.small_x = 1; a.n_split = n_valid; a.big_x = (n_valid + a.rows - 1) / a.rows;
-  a.ksplit = 1; a.kchunk = a.nkb_w; a.ws = nullptr; a.ld_ws = 0; a.tickets = nullptr;
-  if (thin) {
-    // tiles of 128 rows, unless those need a second wave and tiles of 256 rows do not (fused layers: every layer a whole
-    // number of tiles)
-    bool r256 = (n_valid + BN_W - 1) / BN_W > h->sm_count && (n_valid + 2 * BN_W - 1) / (2 * BN_W) <= h->sm_count;
-    for (int i = 0; i < h->n_sub && h->n_sub > 1; ++i) r256 = r256 && h->sub_dout[i] % (2 * BN_W) == 0;
-    a.rows = n_valid > BN_W && !r256 ? BN_W : 2 * BN_W;
-    a.big_x = (n_valid + a.rows - 1) / a.rows;
-    const int t_ctas = ab ? 16 : 0;                         // leave room for the CTAs of the t launch
-    a.ksplit = pick_ksplit(a.big_x, a.nkb_w, h->sm_count - t_ctas, 8, 16);
-    a.kchunk = (a.nkb_w + a.ksplit - 1) / a.ksplit;
-    a.ksplit = (a.nkb_w + a.kchunk - 1) / a.kchunk;
-    a.ws = pst->ws_y; a.ld_ws = n_valid; a.tickets = pst->tk_y;
-  }
+  a.ksplit = tl.ks; a.wait_x = ab ? 0 : 1;
   const int big_y = (m + bt - 1) / bt;
   // Wave quantisation: a CTA needs an SM of its own, so a few tiles more than a whole number of waves cost a whole
   // wave (gate / up at M = 2048: 448 tiles on 148 SMs).  Then the last row tiles are taken out of the big grid until
@@ -933,7 +873,7 @@ cudaError_t launch_prefill_forward(const Handle* h, const void* x, int m, void* 
   // dispatched first and share the launch's first wave with the big tiles.
   CUtensorMap tm_xs = tm_x, tm_ts = tm_t;
   const int tiles = a.big_x * big_y, over = tiles % h->sm_count;
-  if (a.rows == 2 * BN_W && bt == 256 && tiles > h->sm_count && over > 0 && 4 * over <= h->sm_count) {
+  if (a.ksplit == 1 && a.rows == 2 * BN_W && bt == 256 && tiles > h->sm_count && over > 0 && 4 * over <= h->sm_count) {
     const int peel = (over + big_y - 1) / big_y;                 // row tiles to take out
     if (peel < a.big_x) {
       a.big_x -= peel;
@@ -947,7 +887,7 @@ cudaError_t launch_prefill_forward(const Handle* h, const void* x, int m, void* 
   }
   const int smem_y = fill_stages(a);
   dim3 grid(a.n_small + a.big_x * a.ksplit * big_y, 1, 1);
-  return launch_any(h->w.fmt, ab ? h->b.fmt : FMT_NONE, grid, smem_y, st, tm_x, tm_t, tm_xs, tm_ts, a, ab);
+  return launch_any(h->w.fmt, ab ? h->b.fmt : FMT_NONE, grid, smem_y, st, tm_x, tm_t, tm_xs, tm_ts, a);
 }
 
 }  // namespace eora
