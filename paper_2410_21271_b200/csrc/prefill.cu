@@ -32,9 +32,8 @@ namespace {
 constexpr int BN_W = 128, BK = 64;               // weight rows per MMA (its M), k-block; a CTA owns up to two such halves
 constexpr int kDqWarps = 16;                    // dequant warps (warps 4..19): one 16-row tile of the 256 weight rows each
 constexpr int kThreadsP = (4 + kDqWarps) * 32;  // warp 0: TMA, warp 1: MMA, warp 2: TMEM alloc, warp 3: idle
-constexpr int kMaxWStages = 4;                  // ring of k-block stages (token tile + dequantised weight tile)
+constexpr int kMaxWStages = 6;                  // ring of k-block stages (token tile + dequantised weight tile)
 constexpr int kSmallTile = 128;                // rows and tokens of the small tiles that fill a launch's last wave
-constexpr int kPrefetch = 4;                    // k-blocks of packed weights held in registers ahead of use (2 for fp16)
 
 struct PrefillArgs {
   WMat w;            // weight operand of the first nkb_w k-blocks (rows = output columns)
@@ -52,7 +51,7 @@ struct PrefillArgs {
   int n_small, small_x, n_split, big_x;
   int nkb_w, nkb_b;  // k-blocks of each part
   int sx, sw;        // stages of the ring (sx == sw: token tiles first, weight tiles from w_off on)
-  int w_off;         // byte offset of the weight ring (after sx token tiles of bt*128 bytes)
+  int w_off, w_slot; // byte offset of the weight ring (after sx token tiles of bt*128 bytes), bytes of a weight tile (rows * 128)
   // Where the tiles leave SMs idle, the reduction axis of a tile is split over the ksplit CTAs of a cluster (the first one
   // also takes the K-extension; split_lo says which backbone k-blocks are whose).  The
   // partial accumulators meet in distributed shared memory: every CTA finishes every ksplit-th chunk of 32 tokens.
@@ -83,8 +82,8 @@ struct PrefillState {
 __device__ __forceinline__ int split_lo(const PrefillArgs& p, int s) {
   if (s <= 0) return 0;
   if (s >= p.ksplit) return p.nkb_w;
-  const int total = p.nkb_w + p.nkb_b;
-  return p.nkb_b > total / p.ksplit ? (s - 1) * p.nkb_w / (p.ksplit - 1) : s * total / p.ksplit - p.nkb_b;
+  const int w = p.nkb_w / 2, b = p.nkb_b / 2, total = w + b;      // in pairs: a blob is not split
+  return 2 * (b > total / p.ksplit ? (s - 1) * w / (p.ksplit - 1) : s * total / p.ksplit - b);
 }
 
 // ---------------------------------------------------------------------------------------------- PTX
@@ -292,20 +291,20 @@ __device__ __forceinline__ void dequant_store(Packed<FMT> r, uint32_t sc2, uint3
 }
 
 // One part (W or the K-extension B) of a dequant warp's work.  The warp owns row tile `tile` (0..15) of
-// the CTA's 256 weight rows; k-blocks [kb_lo, kb_hi) of `mat` land in pipeline iterations it0, it0 + 1, ...,
-// and the warp takes those with index kb_lo + kphase + i * kstep (kstep = 2 when two warps share a row
-// tile, which is how a CTA with 128 rows keeps all sixteen warps and twice the loads in flight).
-// Packed weights, scales and zero-points are loaded PF of the warp's k-blocks ahead.  The loop is what bounds the
-// kernel (four of these warps share a scheduler), so everything that does not change per k-block is
-// computed once: the store offsets, the ring position as a running (slot, wrap) pair, shared addresses.
+// the CTA's 256 weight rows; k-blocks [kb_lo, kb_hi) of `mat` (both even) land in pipeline iterations it0, it0 + 1, ...
+// A unit of work is a blob (two k-blocks, one set of scales) or, for fp16 weights, whose blob is 32 registers, one k-block;
+// the warp takes units phase, phase + step, ... (step = 2 when two warps share a row tile, which is how a CTA with 128 rows
+// keeps all sixteen warps and twice the loads in flight).  Units are loaded PF of the warp's own ahead.  The loop is what bounds
+// the kernel (four of these warps share a scheduler), so everything that does not change per k-block is computed once per
+// blob or once altogether: constants from scales and zero-points, running addresses, the ring position as a (slot, wrap) pair.
 template <int FMT>
-__device__ __forceinline__ bool dequant_part(const WMat& mat, int n0, int kb_lo, int kb_hi, int it0, int tile, int kphase,
-                                             int kstep, int lane, uint8_t* smem, const PrefillArgs& p, uint64_t* full_w,
+__device__ __forceinline__ bool dequant_part(const WMat& mat, int n0, int kb_lo, int kb_hi, int it0, int tile, int phase,
+                                             int step, int lane, uint8_t* smem, const PrefillArgs& p, uint64_t* full_w,
                                              uint64_t* empty_w, uint32_t lut) {
   if constexpr (FMT == FMT_NONE) {
     return true;
   } else {
-    constexpr int PF = FMT == FMT_F16 ? 3 : kPrefetch;
+    constexpr int U = FMT == FMT_F16 ? 1 : 2, PF = FMT == FMT_F16 ? 3 : 2;
     constexpr bool quant = fmt_quantised(FMT);
     constexpr int tb = tile_bytes(FMT);
     const int rt = (n0 >> 4) + tile;                     // this warp's row tile of the matrix
@@ -314,51 +313,68 @@ __device__ __forceinline__ bool dequant_part(const WMat& mat, int n0, int kb_lo,
     const int odd = g & 1;
     uint32_t off[4];
     store_offsets(off, tile, lane);
-    const uint8_t* base = wmat_blob(mat, rt, 0);                          // this row tile's blob of pair 0
-    const int64_t to_second = wmat_blob(mat, rt, mat.half) - (base + (int64_t)mat.half * mat.blob);   // what the second half of the pairs is further
-    const int sz_step = mat.sz2 ? kSzEntryBytes : 0;
     const uint32_t ring = smem_u32(smem + p.w_off), full0 = smem_u32(full_w), empty0 = smem_u32(empty_w);
-    Packed<FMT> pk[PF];
-    uint32_t scq[PF], zzq[PF];
-    auto issue = [&](int kb, int slot) {
-      if (!active || kb >= kb_hi) return;
-      const uint8_t* blob = base + (kb >> 1) * mat.blob;
-      if ((kb >> 1) >= mat.half) blob += to_second;
-      load_packed<FMT>(pk[slot], blob + (kb & 1) * tb, lane, odd);
+    const int u_hi = kb_hi / U;                          // units [kb_lo / U + phase, u_hi), every step-th
+    int u_next = kb_lo / U + phase;                      // the next unit to load, and where it is
+    const uint8_t* next = wmat_blob(mat, rt, u_next * U / 2) + (U == 1 ? (u_next & 1) * tb : 0);
+    const int64_t to_second = wmat_blob(mat, rt, mat.half) - (wmat_blob(mat, rt, 0) + (int64_t)mat.half * mat.blob);   // what the second half of the pairs is further
+    const int half_u = u_next * U / 2 < mat.half ? 2 * mat.half / U : 0x7fffffff;      // the unit that the second half begins with, if it is ahead
+    const bool two = mat.sz2 != 0;
+    Packed<FMT> pk[PF][U];
+    uint32_t scq[PF][U], zzq[PF][U];
+    bool crossed = false;
+    auto issue = [&](int slot) {
+      if (!active || u_next >= u_hi) return;
+      if (!crossed && u_next >= half_u) { next += to_second; crossed = true; }
+#pragma unroll
+      for (int c = 0; c < U; ++c) load_packed<FMT>(pk[slot][c], next + c * tb, lane, odd);
       if constexpr (quant) {
-        const uint8_t* sz = blob + 2 * tb + (kb & 1) * sz_step;
-        scq[slot] = __ldg(reinterpret_cast<const uint32_t*>(sz) + g);
-        zzq[slot] = __ldg(reinterpret_cast<const uint16_t*>(sz + 32) + g);
+        const uint8_t* sz = next + 2 * tb + 4 * g;
+        scq[slot][0] = __ldg(reinterpret_cast<const uint32_t*>(sz));
+        zzq[slot][0] = __ldg(reinterpret_cast<const uint16_t*>(sz + 32 - 2 * g));
+        if (two) {
+          scq[slot][U - 1] = __ldg(reinterpret_cast<const uint32_t*>(sz + kSzEntryBytes));
+          zzq[slot][U - 1] = __ldg(reinterpret_cast<const uint16_t*>(sz + kSzEntryBytes + 32 - 2 * g));
+        }
       }
+      u_next += step;
+      next += U == 1 ? (step == 2 ? mat.blob : (u_next & 1) ? tb : mat.blob - tb) : step * mat.blob;
     };
 #pragma unroll
-    for (int j = 0; j < PF; ++j) { scq[j] = 0; zzq[j] = 0; issue(kb_lo + kphase + j * kstep, j); }
-    int it = it0 + kphase;
+    for (int j = 0; j < PF; ++j) issue(j);
+    int it = it0 + phase * U;
     int s = it % p.sw, wrap = it / p.sw;                 // ring slot of iteration `it`, and how often it has been used before
-    for (int kbb = kb_lo + kphase; kbb < kb_hi; kbb += PF * kstep) {
+    auto advance = [&](int by) {                         // by <= 3 <= stages
+      it += by;
+      s += by;
+      if (s >= p.sw) { s -= p.sw; ++wrap; }
+    };
+    for (int ub = kb_lo / U + phase; ub < u_hi; ub += PF * step) {
 #pragma unroll
       for (int j = 0; j < PF; ++j) {
-        const int kb = kbb + j * kstep;
-        if (kb < kb_hi) {
-          if (wrap > 0 && !mbar_try_wait_a(empty0 + 8 * s, (wrap - 1) & 1) &&
-              !mbar_wait_warp(empty_w + s, (wrap - 1) & 1, p.dev_status, lane)) return false;
-          const uint32_t stage = ring + (uint32_t)s * (2 * BN_W * 128);
-          if (active) {
-            dequant_store<FMT>(pk[j], scq[j], zzq[j], stage, off, odd != 0, lut);
-          } else {                                        // rows past the matrix: keep the operand finite
+        if (ub + j * step < u_hi) {
 #pragma unroll
-            for (int k = 0; k < 4; ++k) st_shared_v4(stage + off[k], 0u, 0u, 0u, 0u);
+          for (int c = 0; c < U; ++c) {
+            if (wrap > 0 && !mbar_try_wait_a(empty0 + 8 * s, (wrap - 1) & 1) &&
+                !mbar_wait_warp(empty_w + s, (wrap - 1) & 1, p.dev_status, lane)) return false;
+            const uint32_t stage = ring + (uint32_t)s * p.w_slot;
+            if (active) {
+              const bool own = U == 2 && c == 1 && two;
+              dequant_store<FMT>(pk[j][c], own ? scq[j][U - 1] : scq[j][0], own ? zzq[j][U - 1] : zzq[j][0], stage, off, odd != 0, lut);
+            } else {                                      // rows past the matrix: keep the operand finite
+#pragma unroll
+              for (int k = 0; k < 4; ++k) st_shared_v4(stage + off[k], 0u, 0u, 0u, 0u);
+            }
+            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // generic-proxy stores -> visible to the MMA
+            __syncwarp();
+            if (lane == 0) {
+              asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(full0 + 8 * s) : "memory");
+              if (tile == 0) PTRACE(it, 1);
+            }
+            if (c + 1 < U) advance(1);
           }
-          asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // generic-proxy stores -> visible to the MMA
-          __syncwarp();
-          if (lane == 0) {
-            asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(full0 + 8 * s) : "memory");
-            if (tile == 0) PTRACE(it, 1);
-          }
-          issue(kb + PF * kstep, j);
-          it += kstep;
-          s += kstep;
-          if (s >= p.sw) { s -= p.sw; ++wrap; }             // kstep <= 2 <= stages
+          issue(j);
+          advance(step * U - U + 1);
         }
       }
     }
@@ -474,7 +490,7 @@ __global__ void __launch_bounds__(kThreadsP, 1) k_prefill(const __grid_constant_
         PTRACE(it, 2);
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
         const uint64_t bdesc = make_desc(smem + (size_t)sw * xslot);
-        const uint64_t adesc = make_desc(smem + p.w_off + (size_t)sw * (2 * BN_W * 128));
+        const uint64_t adesc = make_desc(smem + p.w_off + (size_t)sw * p.w_slot);
 #pragma unroll
         for (int j = 0; j < 8; ++j) {
           // half j / 4 of the weight rows is 128 rows = 16 KB further (+1024 in the address field), each K step of
@@ -684,12 +700,13 @@ cudaError_t launch_any(int wf, int bf, dim3 grid, int smem, cudaStream_t st, con
 }
 
 int fill_stages(PrefillArgs& a) {      // returns the dynamic shared memory to request
-  const int stage = a.bt * 128 + 2 * BN_W * 128;       // token tile + weight tile of one k-block
+  a.w_slot = a.rows * 128;
+  const int stage = a.bt * 128 + a.w_slot;             // token tile + weight tile of one k-block
   a.sw = (kSmemP - 1024) / stage;
   if (a.sw > kMaxWStages) a.sw = kMaxWStages;
   a.sx = a.sw;
   a.w_off = a.sx * a.bt * 128;
-  int smem = a.w_off + a.sw * 2 * BN_W * 128;
+  int smem = a.w_off + a.sw * a.w_slot;
   const int units = a.rows / BN_W * ((a.bt + 31) / 32);
   const int out = a.ksplit > 1 ? 65536 + (units + a.ksplit - 1) / a.ksplit * (a.ksplit - 1) * 16384 : 131072;      // the epilogue's
   return (out > smem ? out : smem) + 1024;
