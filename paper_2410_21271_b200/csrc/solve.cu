@@ -473,45 +473,44 @@ __device__ __forceinline__ double rsqrt_newton(double d) {
 //   (C) the trailing lower triangle is updated in 4 x 4 tiles.  Warp 0 takes the tiles of the next diagonal block first and goes on
 //       with (A) for the next panel while the others update the rest.
 // The chain of (A)s is what bounds it: a pivot, its root, a column and an update, 16 times per panel.
-// Writes L over S (lower triangle, global) and the inverses of the diagonal blocks; Q = Y L^{-T} follows by k_trsm.  A small multiple
-// of the trace is added to the diagonal first, so that a rank-deficient iterate still factors.  In shared memory up to
+// Writes L over S (lower triangle, global) and the inverses of the diagonal blocks; Q = Y L^{-T} follows by k_trsm.  Every diagonal
+// element first grows by 1e-13 of itself, so that a rank-deficient iterate still factors; relative to itself, because the columns of
+// an iterate are graded (column j has about the norm of the j-th eigenvalue, or of its square).  In shared memory up to
 // m = kCholSmem, else in place in global memory (L2).  m = 160: 300 us with an explicit inverse and unblocked updates before.
 constexpr int kCholSmem = 160;
 constexpr int kCholThreads = 512;
 __host__ __device__ constexpr int pan_pitch(int m) { return (m + 5) / 4 * 4 + 2; }      // (even, and rows of the panel on different banks)
-__host__ __device__ constexpr int chol_smem(int m) { return ((m <= kCholSmem ? m * (m | 1) : 0) + 16 * pan_pitch(m)) * 8 + 16; }
+__host__ __device__ constexpr int chol_smem(int m) { return ((m <= kCholSmem ? m * (m | 1) : 0) + m + 16 * pan_pitch(m)) * 8 + 16; }
 __global__ void __launch_bounds__(kCholThreads) k_chol64(double* Sg, int m, double* __restrict__ Dinv) {
   extern __shared__ __align__(16) double sm[];
-  __shared__ double dv[16][17], shift_s;
+  __shared__ double dv[16][17];
   const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
   const bool in_smem = m <= kCholSmem;
   const int ls = in_smem ? (m | 1) : m, lp = pan_pitch(m);
   double* pan = sm;                                  // [16][lp]: the panel by columns
-  double* S = in_smem ? sm + 16 * lp : Sg;
+  double* least = sm + 16 * lp;                      // [m]: the smallest pivot of a column that is taken as it is
+  double* S = in_smem ? least + m : Sg;
   if (in_smem)
     for (int i = warp; i < m; i += kCholThreads / 32)
       for (int j = lane; j <= i; j += 32) S[i * ls + j] = Sg[(int64_t)i * m + j];
   __syncthreads();
-  if (warp == 0) {
-    double tr = 0.0;
-    for (int i = lane; i < m; i += 32) tr += S[(int64_t)i * ls + i];
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) tr += __shfl_xor_sync(0xffffffffu, tr, o);
-    if (lane == 0) shift_s = 1e-13 * tr + 1e-300;
+  for (int i = t; i < m; i += kCholThreads) {
+    const double shift = 1e-13 * S[(int64_t)i * ls + i] + 1e-300;
+    S[(int64_t)i * ls + i] += shift;
+    least[i] = 1e-3 * shift;
   }
-  __syncthreads();
-  const double shift = shift_s;
-  for (int i = t; i < m; i += kCholThreads) S[(int64_t)i * ls + i] += shift;
   __syncthreads();
   auto diagonal = [&](int j0) {                      // (A), one warp; lanes 16..31 repeat lanes 0..15
     const int r = lane & 15, gi = j0 + r;
     double a[16], x[16], rinv = 0.0;
+    const double fl = gi < m ? least[gi] : 0.0;
 #pragma unroll
     for (int q = 0; q < 16; ++q) a[q] = gi < m && q <= r ? S[(int64_t)gi * ls + j0 + q] : (q == r ? 1.0 : 0.0);      // past m: identity
 #pragma unroll
     for (int k = 0; k < 16; ++k) {
       double d = __shfl_sync(0xffffffffu, a[k], k);
-      d = d > shift * 1e-3 ? d : shift * 1e-3;
+      const double f = __shfl_sync(0xffffffffu, fl, k);
+      d = d > f ? d : f;
       const double ri = rsqrt_newton(d);
       a[k] = r == k ? d * ri : a[k] * ri;            // (rows above k: never read)
       if (r == k) rinv = ri;
@@ -597,11 +596,11 @@ __global__ void __launch_bounds__(kCholThreads) k_chol64(double* Sg, int m, doub
 
 // Q = Y L^{-T}, row by row (fp64 inside): a CTA takes 16 rows, half a warp each (lane = column of the panel); panel by panel of 16
 // columns  q_p = (y_p - sum_{c < 16 p} q_c L[p][c]^T) Dinv_p^T.  A panel's 16 rows of L and its Dinv come by cp.async, one panel
-// ahead, its column of Y by a load one panel ahead.
+// ahead, its column of Y by a load one panel ahead.  With `scaled`, Q is divided by the power of two next to L[0][0].
 __host__ __device__ constexpr int trsm_pitch(int m) { return (m + 15) / 16 * 16 + 2; }
 __host__ __device__ constexpr int trsm_smem(int m) { return (3 * 16 * trsm_pitch(m) + 2 * 16 * 18) * 8; }
 __global__ void __launch_bounds__(256) k_trsm(const float* __restrict__ Y, const double* __restrict__ L, const double* __restrict__ Dinv, int m, int ld,
-                                              float* __restrict__ Q) {
+                                              float* __restrict__ Q, bool scaled) {
   extern __shared__ __align__(16) double smt[];
   const int lq = trsm_pitch(m);
   double* qd = smt;                                  // [16][lq]
@@ -624,6 +623,8 @@ __global__ void __launch_bounds__(256) k_trsm(const float* __restrict__ Y, const
   };
   fetch(0);
   float y = Y[row * ld + c];
+  const int ex = min(max((__double2hiint(L[0]) >> 20) - 1023, -120), 120);
+  const float scale = scaled ? __int_as_float((127 - ex) << 23) : 1.f;
   for (int p = 0; p < np; ++p) {
     asm volatile("cp.async.wait_group 0;" ::: "memory");
     __syncthreads();                                 // panel p is there, and panel p - 1 has been read
@@ -645,7 +646,7 @@ __global__ void __launch_bounds__(256) k_trsm(const float* __restrict__ Y, const
     for (int q = 0; q < 16; ++q) o[q & 3] = fma(__shfl_sync(0xffffffffu, w, q, 16), dr[q], o[q & 3]);      // (Dinv is lower triangular: zeros past c)
     const double res = (o[0] + o[1]) + (o[2] + o[3]);
     qd[r * lq + 16 * p + c] = res;
-    Q[row * ld + 16 * p + c] = (float)res;
+    Q[row * ld + 16 * p + c] = (float)res * scale;
     __syncwarp();
   }
   for (int i = 16 * np + c; i < ld; i += 16) Q[row * ld + i] = 0.f;
@@ -1033,13 +1034,16 @@ cudaError_t allow_smem(int bytes) {
   return e;
 }
 
+constexpr int kSingleSteps = 4;        // products that are orthogonalised one by one before the pairs begin
+
 // Q = orth(Y) by Cholesky-QR: Gram matrix, its factor and Q = Y L^{-T} in fp64.  Y, Q: [rows][ldm], rows a multiple of 16.
-int orthonormalise(cudaStream_t st, const Plan& p, int rows, const float* Y, float* Q, double* S, double* parts, double* D) {
+int orthonormalise(cudaStream_t st, const Plan& p, int rows, const float* Y, float* Q, double* S, double* parts, double* D,
+                   bool scaled = false) {
   CK(gram64<false>(st, Y, rows, p.m, p.ldm, parts, S));
   CK(allow_smem<k_chol64>(chol_smem(kCholSmem)));
   CK(allow_smem<k_trsm>(trsm_smem(512)));
   k_chol64<<<1, kCholThreads, chol_smem(p.m), st>>>(S, p.m, D);
-  k_trsm<<<rows / 16, 256, trsm_smem(p.m), st>>>(Y, S, D, p.m, p.ldm, Q);
+  k_trsm<<<rows / 16, 256, trsm_smem(p.m), st>>>(Y, S, D, p.m, p.ldm, Q, scaled);
   CK(cudaGetLastError());
   return EORA_OK;
 }
@@ -1122,9 +1126,21 @@ int eora_solve(const eora_solve_config* cfg, const float* w, const float* w_hat,
   k_init<<<592, 256, 0, st>>>(Y, p.s, sp, p.m, ldm);
   CK(cudaGetLastError());
   if (int rc = orthonormalise(st, p, sp, Y, Q, S, Sp, D)) return rc;
-  for (int it = 0; it < p.iters; ++it) {
+  // Orthogonalising costs twice a product with C (a chain of m pivots).  Once the columns are graded -- column j close to the j-th
+  // eigenvector, which the first steps see to -- it is needed only every second product: the part of the larger eigenvectors that
+  // rounding brings into a column stays in the span and is taken out with the next factor, and what lies outside the span
+  // is damped by every product.  The iterate that goes through two products is scaled to norm 1 / lam_1, which keeps
+  // C C Q in the range of the products of one step.  Rank 128, 24 products: 27 -> 17 factorisations of 83 us.
+  for (int it = 0; it < p.iters;) {
+    const bool pair = it >= kSingleSteps && p.iters - it >= 2;
     CK(skinny<true>(st, p.w, sp, sp, C, sp, Q, ldm, ldm, Y, ldm));            // Y = C Q (C is symmetric: read by columns)
-    if (int rc = orthonormalise(st, p, sp, Y, Q, S, Sp, D)) return rc;
+    if (pair) {
+      CK(skinny<true>(st, p.w, sp, sp, C, sp, Y, ldm, ldm, Q, ldm));
+      float* y = Y; Y = Q; Q = y;
+    }
+    it += pair ? 2 : 1;
+    const bool next_pair = it >= kSingleSteps && p.iters - it >= 2;
+    if (int rc = orthonormalise(st, p, sp, Y, Q, S, Sp, D, next_pair)) return rc;
   }
   if (p.n_side) {                                                             // to the d-dimensional side
     CK(skinny<false>(st, p.w, dp, np, Pm, np, Q, ldm, ldm, Y, ldm));
