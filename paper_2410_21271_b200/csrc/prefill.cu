@@ -98,6 +98,22 @@ __device__ __forceinline__ void umma_f16(uint32_t tmem_d, uint64_t adesc, uint64
 __device__ __forceinline__ void umma_commit(uint64_t* bar) {
   asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar)) : "memory");
 }
+// 16 lanes x 32 columns as fragments of 8 x 8 blocks: registers 4 c .. 4 c + 3 hold columns 8 c + 2 (lane % 4) and the next one of
+// lane lane / 4, then of lane lane / 4 + 8.
+__device__ __forceinline__ void tmem_ld16x32(uint32_t taddr, uint32_t* v) {
+  asm volatile("tcgen05.ld.sync.aligned.16x256b.x4.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
+               : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]), "=r"(v[8]), "=r"(v[9]),
+                 "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15])
+               : "r"(taddr));
+}
+__device__ __forceinline__ void stmatrix_x4_trans(uint32_t addr, uint32_t a, uint32_t b, uint32_t c, uint32_t d) {
+  asm volatile("stmatrix.sync.aligned.m8n8.x4.trans.shared.b16 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(a), "r"(b), "r"(c), "r"(d) : "memory");
+}
+__device__ __forceinline__ uint4 lds128(uint32_t addr) {
+  uint4 v;
+  asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(addr) : "memory");
+  return v;
+}
 __device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&v)[32]) {
   asm volatile("tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
                "%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];"
@@ -530,7 +546,18 @@ __global__ void __launch_bounds__(kThreadsP, 1) k_prefill(const __grid_constant_
   const int nl = lq * 32 + lane;                         // local weight row inside the half = thread index inside the group
   const int nchunk = (bt + 31) >> 5, units = nh * nchunk;
   const uint32_t lane_base = tmem_d + ((uint32_t)(lq * 32) << 16);
-  uint8_t* const parts = smem + 65536;                   // split: the other CTAs' shares of this CTA's units, 16 KB each
+  const uint32_t parts = smem_u32(smem) + 65536;         // split: the other CTAs' shares of this CTA's units, 16 KB each
+  const bool out16 = p.out_dtype != EORA_Y_F32;
+  // A unit's accumulators: for a 16-bit Y as fragments of 8 x 8 blocks, for a float Y one row of W per lane (32 tokens).
+  auto load_unit = [&](uint32_t taddr, uint32_t (&v)[32]) {
+    if (out16) {
+      tmem_ld16x32(taddr, v);
+      tmem_ld16x32(taddr + (16u << 16), v + 16);
+    } else {
+      tmem_ld32(taddr, v);
+    }
+    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+  };
   if (p.ksplit > 1) {
     __syncwarp();
     cluster_arrive(); cluster_wait();                    // every CTA's MMAs have completed: the rings are free everywhere
@@ -540,53 +567,74 @@ __global__ void __launch_bounds__(kThreadsP, 1) k_prefill(const __grid_constant_
       if (owner == split) continue;
       const int hh = u / nchunk, c0 = (u - hh * nchunk) * 32;
       uint32_t v[32];
-      tmem_ld32(lane_base + hh * 256 + (uint32_t)c0, v);
-      asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+      load_unit(lane_base + hh * 256 + (uint32_t)c0, v);
       const int slot = (u / p.ksplit) * (p.ksplit - 1) + (split < owner ? split : split - 1);
-      const uint32_t to = mapa(smem_u32(parts + slot * 16384) + nl * 4, (uint32_t)owner);
+      const uint32_t to = mapa(parts + slot * 16384 + nl * 16, (uint32_t)owner);      // (the same thread of the owner adds it to the same registers)
 #pragma unroll
-      for (int j = 0; j < 32; ++j) asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(to + j * 512), "r"(v[j]) : "memory");
+      for (int j = 0; j < 32; j += 4)
+        asm volatile("st.shared::cluster.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(to + j * 512), "r"(v[j]), "r"(v[j + 1]), "r"(v[j + 2]), "r"(v[j + 3]) : "memory");
     }
     __syncwarp();
     cluster_arrive(); cluster_wait();
   }
   if (warp >= 4 && *reinterpret_cast<volatile int*>(&fail_s) == 0) {
-    // A unit goes through shared memory as [32 tokens][128 n] so that the global stores are 16-byte pieces of rows of Y.
-    // Without a split each group has two buffers of 16 KB and alternates: a buffer is rewritten two units later, after a
-    // barrier that every thread of the group passes only when it has read the buffer out, so one barrier per unit is
-    // enough.  With a split it has one buffer and takes two barriers.
-    const int esz = p.out_dtype == EORA_Y_F32 ? 4 : 2;
-    const int row_sh = esz == 4 ? 5 : 4;                 // log2 of the 16-byte pieces per token row (128 n)
-    uint8_t* const gbuf = smem + grp * (p.ksplit > 1 ? 16384 : 32768);
+    // A unit goes through shared memory as [32 tokens][128 n] so that the global stores are 16-byte pieces of rows of Y: a 16-bit
+    // Y by transposing stores of 8 x 8 blocks, rows 16 bytes apart modulo the banks; a float Y word by word.  (Storing it element
+    // by element, the type decided at each, took 7400 of the 10700 cycles of a 256 x 256 tile; the stores to Y take 1000.)
+    // Without a split each group has two buffers of 16 KB (a 32 x 128 block of floats) and alternates: a buffer is rewritten two
+    // units later, after a barrier that every thread of the group passes only when it has read the buffer out, so one barrier
+    // per unit is enough.  With a split it has one buffer and takes two barriers.
+    const uint32_t gbuf = smem_u32(smem) + grp * (p.ksplit > 1 ? 16384 : 32768);
+    const uint32_t pitch = out16 ? 272 : 512;            // bytes from one token's row in the buffer to the next
+    const int esz = out16 ? 2 : 4, row_sh = out16 ? 4 : 5;      // log2 of the 16-byte pieces per token row (128 n)
     int flip = 0;
     for (int i = grp; i * p.ksplit + split < units; i += 4) {
       const int u = i * p.ksplit + split, hh = u / nchunk, c0 = (u - hh * nchunk) * 32;
-      uint8_t* tbuf = gbuf + flip * 16384;
+      const uint32_t tbuf = gbuf + flip * 16384;
       if (p.ksplit == 1) flip ^= 1;
       uint32_t v[32];
-      tmem_ld32(lane_base + hh * 256 + (uint32_t)c0, v);
-      asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+      load_unit(lane_base + hh * 256 + (uint32_t)c0, v);
       for (int q = 0; q < p.ksplit - 1; ++q) {
-        const float* src = reinterpret_cast<const float*>(parts + (i * (p.ksplit - 1) + q) * 16384) + nl;
+        const uint32_t src = parts + (i * (p.ksplit - 1) + q) * 16384 + nl * 16;
 #pragma unroll
-        for (int j = 0; j < 32; ++j) v[j] = __float_as_uint(__uint_as_float(v[j]) + src[j * 128]);
+        for (int j = 0; j < 32; j += 4) {
+          const uint4 o = lds128(src + j * 512);
+          v[j] = __float_as_uint(__uint_as_float(v[j]) + __uint_as_float(o.x));
+          v[j + 1] = __float_as_uint(__uint_as_float(v[j + 1]) + __uint_as_float(o.y));
+          v[j + 2] = __float_as_uint(__uint_as_float(v[j + 2]) + __uint_as_float(o.z));
+          v[j + 3] = __float_as_uint(__uint_as_float(v[j + 3]) + __uint_as_float(o.w));
+        }
       }
+      if (out16) {
+        uint32_t h[16];                                  // pairs of tokens of a row
+        if (p.out_dtype == EORA_Y_F16) {
 #pragma unroll
-      for (int j = 0; j < 32; ++j) {
-        const float f = __uint_as_float(v[j]);
-        if (p.out_dtype == EORA_Y_F32) reinterpret_cast<float*>(tbuf)[j * BN_W + nl] = f;
-        else if (p.out_dtype == EORA_Y_F16) reinterpret_cast<__half*>(tbuf)[j * BN_W + nl] = __float2half_rn(f);
-        else reinterpret_cast<__nv_bfloat16*>(tbuf)[j * BN_W + nl] = __float2bfloat16_rn(f);
+          for (int j = 0; j < 16; ++j) {
+            const __half2 w = __floats2half2_rn(__uint_as_float(v[2 * j]), __uint_as_float(v[2 * j + 1]));
+            h[j] = *reinterpret_cast<const uint32_t*>(&w);
+          }
+        } else {
+#pragma unroll
+          for (int j = 0; j < 16; ++j) {
+            const __nv_bfloat162 w = __floats2bfloat162_rn(__uint_as_float(v[2 * j]), __uint_as_float(v[2 * j + 1]));
+            h[j] = *reinterpret_cast<const uint32_t*>(&w);
+          }
+        }
+        // block q of a store: rows 8 q .. of this warp's 32, tokens 8 c ..;  lane 8 q + i gives the address of token i
+        const uint32_t at = tbuf + (lane & 7) * 272 + (lq * 32 + (lane >> 3) * 8) * 2;
+#pragma unroll
+        for (int c = 0; c < 4; ++c) stmatrix_x4_trans(at + c * 8 * 272, h[2 * c], h[2 * c + 1], h[8 + 2 * c], h[8 + 2 * c + 1]);
+      } else {
+#pragma unroll
+        for (int j = 0; j < 32; ++j) asm volatile("st.shared.u32 [%0], %1;" ::"r"(tbuf + j * 512 + nl * 4), "r"(v[j]) : "memory");
       }
       asm volatile("bar.sync %0, 128;" ::"r"(2 + grp) : "memory");
       const int pieces = 32 << row_sh;
       for (int e = nl; e < pieces; e += 128) {
         const int tok = e >> row_sh, piece = e & ((1 << row_sh) - 1);
         const int row = m0 + c0 + tok, col = n0 + hh * BN_W + piece * (16 / esz);
-        if (c0 + tok < bt && row < p.m && col < n_end) {     // a unit may reach past the tile's tokens
-          const uint4 val = *reinterpret_cast<const uint4*>(tbuf + (size_t)tok * BN_W * esz + piece * 16);
-          *reinterpret_cast<uint4*>(reinterpret_cast<uint8_t*>(out_p) + ((int64_t)row * ld_o + col - col0) * esz) = val;
-        }
+        if (c0 + tok < bt && row < p.m && col < n_end)       // a unit may reach past the tile's tokens
+          *reinterpret_cast<uint4*>(reinterpret_cast<uint8_t*>(out_p) + ((int64_t)row * ld_o + col - col0) * esz) = lds128(tbuf + tok * pitch + piece * 16);
       }
       if (p.ksplit > 1) asm volatile("bar.sync %0, 128;" ::"r"(2 + grp) : "memory");
     }

@@ -1,0 +1,55 @@
+"""GPU parity of the tensor-core path for more than 32 tokens where its cuts can go wrong: clusters that share a reduction axis
+(uneven shares, an extension longer than one share, the fewest k-blocks that are split), token tiles with a remainder, rows that
+end inside a tile, fused layers of 128-row tiles, launches chained back to back.  Tolerance as for every forward (tests/helpers.py)."""
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+from oracle import eora_oracle as orc
+import eora_inputs as gen
+import paper_2410_21271_b200 as eora
+from helpers import make_case, run_layer, check_parity, x_to_torch
+
+
+@pytest.mark.parametrize("w,ab,K,N,r,M,xd,yd,group", [
+    ("q4", "f16", 128, 32, 0, 33, "f16", "f16", 128),       # two k-blocks, one ragged row tile: no split
+    ("q4", "f16", 512, 128, 64, 33, "f16", "f32", 64),      # eight k-blocks: the fewest that two CTAs share
+    ("q4", "f16", 2048, 384, 128, 64, "f16", "f16", 128),
+    ("q3", "q8", 4096, 544, 512, 48, "bf16", "bf16", 128),  # shares of eight CTAs, 544 = 4 * 128 + 32 rows
+    ("q3", "f16", 512, 512, 2048, 70, "f16", "f16", 128),   # the extension is longer than a share of the reduction axis
+    ("sp24", "q4", 1152, 1024, 64, 100, "f16", "f32", 128), # 18 k-blocks: pairs do not divide evenly
+    ("sq4", "f16", 2048, 2080, 0, 257, "f16", "f16", 128),  # two token tiles, the second ragged
+    ("q4", "q3", 14336, 512, 256, 333, "bf16", "f16", 128),
+    ("q4", "f16", 1024, 4096, 24, 700, "f16", "f16", 128),
+])
+def test_prefill_cuts(w, ab, K, N, r, M, xd, yd, group):
+    wf, af, bf = make_case(71, K, N, r, w=w, ab=ab, group=group)
+    x = gen.make_x(72, M, K, xd)
+    L = eora.Layer(wf, af, bf, max_m=M, x_dtype=xd, y_dtype=yd)
+    ref = orc.forward(x, xd, wf, af, bf)
+    for rep in range(2):
+        check_parity(run_layer(L, x, xd), ref, f"{w}/{ab} K{K} N{N} r{r} M{M} call {rep}")
+    L.close()
+
+
+@pytest.mark.parametrize("M", [40, 130])
+def test_prefill_fused_calls_in_a_row(M):
+    """Calls that follow each other without a wait, each reading what the one in front wrote: X of the second is Y of the first."""
+    import torch
+    K, r = 1024, 64
+    layers = [make_case(75 + i, K, N, r, w="q4") for i, N in enumerate((1024, 128, 384))]
+    F = eora.FusedLayers(layers, max_m=M)
+    one = eora.Layer(*layers[0], max_m=M)
+    x = gen.make_x(76, M, K)
+    xt = x_to_torch(x, "f16")
+    for rep in range(3):
+        y = one.forward(xt)
+        ys = F.forward(y)
+    torch.cuda.synchronize()
+    check_parity(y.float().cpu().numpy().astype(np.float64), orc.forward(x, "f16", *layers[0]), "first")
+    x2 = y.cpu().numpy()
+    for i, case in enumerate(layers):
+        check_parity(ys[i].float().cpu().numpy().astype(np.float64), orc.forward(x2, "f16", *case), f"layer {i}")
+    F.close()
+    one.close()
