@@ -485,11 +485,11 @@ static int stage_in(Handle* h, const void* x_host, size_t bytes, int32_t m, cuda
   void* alias = (bytes % 16 == 0 && aligned16(x_host)) ? mapped_alias(const_cast<void*>(x_host), m) : nullptr;
   if (!alias) return cudaMemcpyAsync(h->x_stage, x_host, bytes, cudaMemcpyHostToDevice, s) == cudaSuccess ? EORA_OK : EORA_ERR_CUDA;
   const int64_t n16 = (int64_t)(bytes / 16);
-  int grid = (int)((n16 + 1023) / 1024);
-  if (grid > 64) grid = 64;
+  int grid = (int)((n16 + 127) / 128);            // one 16-byte piece per thread: the link's latency once, not once per piece
+  if (grid > 128) grid = 128;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(grid < 1 ? 1 : grid);
-  cfg.blockDim = dim3(256);
+  cfg.blockDim = dim3(128);
   cfg.stream = s;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
