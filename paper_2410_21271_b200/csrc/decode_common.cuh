@@ -80,9 +80,10 @@ __device__ __forceinline__ bool mbar_wait_lane(uint32_t bar, uint32_t parity, in
 // spin costs a shared-memory access per poll, and a dozen spinning warps are enough to starve the
 // bulk-copy engine and the tensor core of shared-memory bandwidth.  Once lane 0 has seen the phase
 // complete, every lane tests it once itself (which succeeds at once) so that each thread has its own
-// acquire of the data behind the barrier.
+// acquire of the data behind the barrier.  The vote makes the lanes take the same way even if they arrive one after the
+// other: a lane that saw the phase complete and left would miss the shuffle below, whose result would then be undefined.
 __device__ __forceinline__ bool mbar_wait_warp(uint64_t* bar, uint32_t parity, int* dev_status, int lane) {
-  if (mbar_try_wait(bar, parity)) return true;
+  if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity) ? 1 : 0)) return true;
   int ok = 1;
   if (lane == 0) {
     const unsigned long long t0 = globaltimer_ns();
@@ -104,8 +105,6 @@ __device__ __forceinline__ bool mbar_wait_warp(uint64_t* bar, uint32_t parity, i
 // The same without the back-off, for hand-overs that are short and sit on the critical path of a pipeline (a sleeping
 // poll adds up to its period to every hand-over).  The polling try_wait suspends the thread until the phase completes.
 __device__ __forceinline__ bool mbar_wait_warp_fast(uint64_t* bar, uint32_t parity, int* dev_status, int lane) {
-  // The vote makes the lanes take the same way even if they arrive one after the other (a lane that saw the phase
-  // complete and left would leave the others waiting for it in the shuffle below).
   if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity) ? 1 : 0)) return true;
   int ok = 1;
   if (lane == 0) {

@@ -371,7 +371,7 @@ __device__ __forceinline__ bool dequant_part(const WMat& mat, int n0, int kb_lo,
         if (ub + j * step < u_hi) {
 #pragma unroll
           for (int c = 0; c < U; ++c) {
-            if (wrap > 0 && !mbar_try_wait_a(empty0 + 8 * s, (wrap - 1) & 1) &&
+            if (wrap > 0 && !__all_sync(0xffffffffu, mbar_try_wait_a(empty0 + 8 * s, (wrap - 1) & 1)) &&
                 !mbar_wait_warp(empty_w + s, (wrap - 1) & 1, p.dev_status, lane)) return false;
             const uint32_t stage = ring + (uint32_t)s * p.w_slot;
             if (active) {
