@@ -98,6 +98,14 @@ __device__ __forceinline__ void umma_f16(uint32_t tmem_d, uint64_t adesc, uint64
 __device__ __forceinline__ void umma_commit(uint64_t* bar) {
   asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar)) : "memory");
 }
+__device__ __forceinline__ void umma_commit_a(uint32_t bar) {
+  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
+}
+__device__ __forceinline__ bool elect_one() {
+  uint32_t p;
+  asm volatile("{\n\t.reg .pred q;\n\telect.sync _|q, 0xffffffff;\n\tselp.u32 %0, 1, 0, q;\n\t}" : "=r"(p));
+  return p != 0;
+}
 // 16 lanes x 32 columns as fragments of 8 x 8 blocks: registers 4 c .. 4 c + 3 hold columns 8 c + 2 (lane % 4) and the next one of
 // lane lane / 4, then of lane lane / 4 + 8.
 __device__ __forceinline__ void tmem_ld16x32(uint32_t taddr, uint32_t* v) {
@@ -492,21 +500,27 @@ __global__ void __launch_bounds__(kThreadsP, 1) k_prefill(const __grid_constant_
         if (++s == p.sw) { s = 0; ++wrap; }
       }
     }
-  } else if (warp == 1) {
+  } else if (__shfl_sync(0xffffffffu, warp, 0) == 1) {      // (warp-uniform for the compiler)
     // ------------------------------------------------------------------ MMA issuer
-    if (lane == 0) {
-      // instruction descriptor: fp32 accumulate, fp16 x fp16, both operands K-major, M = 128 weight rows, N = bt tokens
-      const uint32_t idesc = (1u << 4) | ((uint32_t)(bt >> 3) << 17) | ((uint32_t)(BN_W >> 4) << 24);
-      bool ok = true;
-      int sw = 0;                                   // ring slot of iteration `it` and its phase
-      uint32_t pw = 0;
-      for (int it = 0; it < nkb && ok; ++it) {
-        ok = mbar_wait(full_w + sw, pw, p.dev_status);   // token tile copied and weight tile dequantised
-        if (!ok) break;
-        PTRACE(it, 2);
-        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        const uint64_t bdesc = make_desc(smem + (size_t)sw * xslot);
-        const uint64_t adesc = make_desc(smem + p.w_off + (size_t)sw * p.w_slot);
+    // The whole warp walks through the loop and one elected lane issues: descriptors and addresses are then warp-uniform values
+    // that stay in uniform registers.  Inside an `if (lane == 0)` every operand of every MMA was moved there first, ~90 cycles
+    // per MMA, which bounded a k-block of 256 rows at 1050 cycles whatever the tokens.
+    // instruction descriptor: fp32 accumulate, fp16 x fp16, both operands K-major, M = 128 weight rows, N = bt tokens
+    const uint32_t idesc = (1u << 4) | ((uint32_t)(bt >> 3) << 17) | ((uint32_t)(BN_W >> 4) << 24);
+    const bool elected = elect_one();
+    const uint64_t bdesc0 = make_desc(smem), adesc0 = make_desc(smem + p.w_off);
+    const uint32_t bstep = xslot >> 4, astep = (uint32_t)p.w_slot >> 4;       // from one ring slot to the next, in 16-byte units
+    const uint32_t full0 = smem_u32(full_w), empty0 = smem_u32(empty_w);
+    bool ok = true;
+    uint32_t sw = 0, pw = 0;                        // ring slot of iteration `it` and its phase
+    for (int it = 0; it < nkb; ++it) {
+      // token tile copied and weight tile dequantised?
+      if (!mbar_try_wait_a(full0 + 8 * sw, pw)) ok = mbar_wait(full_w + sw, pw, p.dev_status);
+      if (!__all_sync(0xffffffffu, ok)) break;
+      if (elected) PTRACE(it, 2);
+      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+      const uint64_t bdesc = bdesc0 + sw * bstep, adesc = adesc0 + sw * astep;
+      if (elected) {
 #pragma unroll
         for (int j = 0; j < 8; ++j) {
           // half j / 4 of the weight rows is 128 rows = 16 KB further (+1024 in the address field), each K step of
@@ -515,12 +529,13 @@ __global__ void __launch_bounds__(kThreadsP, 1) k_prefill(const __grid_constant_
             umma_f16(tmem_d + (j >> 2) * 256, adesc + (uint64_t)((j >> 2) * ((BN_W * 128) >> 4) + 2 * (j & 3)), bdesc + 2 * (j & 3),
                      idesc, (it > 0 || (j & 3) > 0) ? 1u : 0u);
         }
-        umma_commit(empty_w + sw);                  // arrives when these MMAs have finished reading their operands
+        umma_commit_a(empty0 + 8 * sw);             // arrives when these MMAs have finished reading their operands
         PTRACE(it, 3);
-        if (++sw == p.sw) { sw = 0; pw ^= 1u; }
       }
-      umma_commit(&acc_full);                       // arrives when every MMA above has completed
+      if (++sw == (uint32_t)p.sw) { sw = 0; pw ^= 1u; }
     }
+    if (elected) umma_commit(&acc_full);            // arrives when every MMA above has completed
+    __syncwarp();
   } else if (warp >= 4) {
     // ------------------------------------------------------------------ dequant warps, then epilogue
     const int dw = warp - 4;
@@ -771,17 +786,24 @@ bool split_fits(int rows, int bt, int ks) {
 // CTAs of clusters of ks that run at once, one per SM (measured: 74 clusters of two, 33 of four, 15 of eight; 148 SMs).
 int at_once(int ks, int sm_count) { return ks == 1 ? sm_count : ks == 2 ? sm_count / 2 * 2 : ks == 4 ? sm_count * 33 / 148 * 4 : sm_count * 15 / 148 * 8; }
 
-// Estimated cycles of a launch.  A k-block takes 1200 cycles with 256 rows and 760 with 128, whatever the tokens (the dequantisation of
-// a CTA's rows and the issue of its MMAs bound it); set-up and first operands 4000; the epilogue 10500 for 256 x 256; meeting in
-// distributed shared memory 3000 more.  A last partial wave of 256-row tiles that is at most a quarter of the SMs is covered by
-// small tiles inside the first wave (launch_prefill_forward), counted as half a wave.
+// Cycles of a k-block: the dequantisation of the CTA's rows bounds it whatever the tokens (128 rows 525, 256 rows 1030; measured with
+// 64 to 512 tokens) up to 192 of them.  With 256 the eight MMAs of 256 rows alone take 1024 (1150 in all), and the token tiles of
+// 128 rows come close to what L2 delivers (600 in one wave, 740 when the SMs are full throughout several).
+float kblock_cycles(const Tiling& t, bool one_wave) {
+  return t.rows == BN_W ? (t.bt <= 192 ? 525.f : one_wave ? 600.f : 740.f) : (t.bt <= 192 ? 1030.f : 1150.f);
+}
+// Estimated cycles of a launch: its k-blocks, set-up and first operands 3200, the epilogue 900 and 5000 per 256 x 256 of the tile; sharing a
+// reduction axis costs two cluster barriers and the way of the tile's sums through distributed shared memory, 1000 + 1600 per
+// doubling + 5500 per 256 x 256.  A last partial wave of 256-row tiles that is at most a quarter of the SMs is covered by small tiles
+// inside the first wave (launch_prefill_forward), counted as half a wave.
 float tiling_cost(const Tiling& t, int n_rows, int m, int nkb, int sm_count) {
   const int tiles = (n_rows + t.rows - 1) / t.rows * ((m + t.bt - 1) / t.bt), cap = at_once(t.ks, sm_count), ctas = tiles * t.ks;
   float waves = (float)((ctas + cap - 1) / cap);
   const int over = tiles % sm_count;
   if (t.ks == 1 && t.rows == 2 * BN_W && t.bt == 256 && tiles > sm_count && over > 0 && 4 * over <= sm_count) waves -= 0.5f;
-  return waves * ((float)((nkb + t.ks - 1) / t.ks) * (t.rows == BN_W ? 760.f : 1200.f) + 4000.f + 10500.f * (float)(t.rows * t.bt) / 65536.f +
-                  (t.ks > 1 ? 3000.f : 0.f));
+  const float area = (float)(t.rows * t.bt) / 65536.f, doublings = t.ks == 1 ? 0.f : t.ks == 2 ? 1.f : t.ks == 4 ? 2.f : 3.f;
+  return waves * ((float)((nkb + t.ks - 1) / t.ks) * kblock_cycles(t, ctas <= cap) + 4100.f + 5000.f * area +
+                  (t.ks > 1 ? 1000.f + 1600.f * doublings + 5500.f * area : 0.f));
 }
 
 int token_tile(int m, int most) {      // the MMA N: a multiple of 16 up to `most`, even tiles
@@ -793,23 +815,26 @@ int token_tile(int m, int most) {      // the MMA N: a multiple of 16 up to `mos
 // an SM of its own and clusters need theirs side by side: if the main launch fits into one wave beside the one for t they
 // overlap to the main product's K-extension; if not, it starts with what t leaves and its last CTAs wait for t.
 struct Tilings { Tiling main, t; };
+// A reduction axis is shared only by clusters that all run at once: in a second wave a cluster waits for SMs side by side (192 CTAs
+// in pairs take 50 us where 96 take 27).
 template <typename F>
-void each_tiling(int m, int nkb_w, bool only128, F f) {
+void each_tiling(int n_rows, int m, int nkb_w, int sm_count, bool only128, F f) {
   const int bt = m > 1024 ? 256 : token_tile(m, 256);        // (whole tiles for long prompts: a ragged last one costs what a full one does)
   for (int rows = BN_W; rows <= (only128 ? BN_W : 2 * BN_W); rows += BN_W)
-    for (int ks = 1; ks <= 8 && (ks == 1 || (nkb_w / ks >= 4 && split_fits(rows, bt, ks))); ks *= 2) f(Tiling{rows, bt, ks});
+    for (int ks = 1; ks <= 8 && (ks == 1 || (nkb_w / ks >= 4 && split_fits(rows, bt, ks))); ks *= 2)
+      if (ks == 1 || (n_rows + rows - 1) / rows * ((m + bt - 1) / bt) * ks <= at_once(ks, sm_count)) f(Tiling{rows, bt, ks});
 }
 Tilings pick_tilings(int n_rows, int t_cols, int m, int nkb_w, int nkb_b, int sm_count, bool only128) {
   Tilings best = {};
   float best_c = -1.f;
   auto ctas_of = [&](const Tiling& t, int rows) { return (rows + t.rows - 1) / t.rows * ((m + t.bt - 1) / t.bt) * t.ks; };
-  each_tiling(m, nkb_w, only128, [&](const Tiling& a) {
+  each_tiling(n_rows, m, nkb_w, sm_count, only128, [&](const Tiling& a) {
     const float cm = tiling_cost(a, n_rows, m, nkb_w + nkb_b, sm_count);
     const int ctas = ctas_of(a, n_rows);
     auto take = [&](const Tiling& t, float c) { if (best_c < 0.f || c < best_c) { best_c = c; best = {a, t}; } };
     if (t_cols == 0) { take(a, cm); return; }
-    each_tiling(m, nkb_w, t_cols <= BN_W, [&](const Tiling& t) {
-      const float ct = tiling_cost(t, t_cols, m, nkb_w, sm_count), tail = (float)nkb_b * (a.rows == BN_W ? 760.f : 1200.f);
+    each_tiling(t_cols, m, nkb_w, sm_count, t_cols <= BN_W, [&](const Tiling& t) {
+      const float ct = tiling_cost(t, t_cols, m, nkb_w, sm_count), tail = (float)nkb_b * kblock_cycles(a, true);
       const int tc = ctas_of(t, t_cols), one_wave = ctas <= at_once(a.ks, sm_count);
       const bool beside = one_wave && ctas + tc <= at_once(a.ks > t.ks ? a.ks : t.ks, sm_count);
       take(t, beside ? (cm > ct + tail ? cm : ct + tail) : one_wave ? cm + ct : cm + ct * (float)tc / (float)sm_count);
