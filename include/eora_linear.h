@@ -125,10 +125,10 @@ int eora_linear_create(const eora_linear_config* cfg, const eora_linear_weights*
  * x, y: device pointers, row-major, 16-byte aligned, caller-owned; 1 <= m <= max_m; m == 0 is a
  * no-op returning EORA_OK.  Never synchronises and never allocates.  The current device must be the one
  * the handle was created on (EORA_ERR_UNSUPPORTED otherwise).  M <= 8 runs the decode
- * kernel family (one streaming pass over the weights), M > 8 the tensor-core (tcgen05) family, which
- * for up to 64 tokens splits the reduction axis of a tile over several thread blocks (fp32 sums in the
- * handle's scratch, restored by the block that completes a tile); handles that the tensor-core family
- * does not serve run ceil(M / 8) decode passes up to M = 64 (eora_linear_path reports the choice).
+ * kernel family (one streaming pass over the weights), M > 8 the tensor-core family: up to 32 tokens in
+ * one pass on mma.sync, beyond as a tcgen05 product whose tiles may share their reduction axis between
+ * the thread blocks of a cluster.  Handles that the tensor-core family does not serve run ceil(M / 8)
+ * decode passes up to M = 64 (eora_linear_path reports the choice).
  * Asynchronous device-side
  * problems (a bounded wait that ran out) are latched in a status word readable with
  * eora_linear_last_device_status after the caller has synchronised.
@@ -144,7 +144,7 @@ int eora_linear_forward(eora_linear_t h, const void* x, int32_t m, void* y, void
  *     ys[i][M][d_out_i] = X . deq(Wq_i) + (X . A_i) . B_i      for every layer i
  * with ONE kernel launch for up to eight tokens: X is read once, and the launch latency is paid once.
  * ys: host array of n_layers device pointers (16-byte aligned, caller-owned).  M <= 8: the decode
- * family; more tokens: the tensor-core family (two launches, the first for t = X . A of all layers) if
+ * family; more tokens: the tensor-core family (one launch up to 32 tokens, else two, the first for t = X . A) if
  * every d_out_i is a multiple of 128 (and the group size of 64), else ceil(M / 8) decode passes up to
  * M = 64.  max_m > 64 therefore needs the tensor-core family: create returns EORA_ERR_UNSUPPORTED
  * otherwise.  eora_linear_forward / _forward_host on it return
@@ -163,7 +163,7 @@ int eora_linear_forward_fused(eora_linear_t h, const void* x, int32_t m, void* c
  * weights[j]; all adapters have the config's rank and format.  eora_linear_forward_multi computes
  *     y[i] = x[i] . deq(Wq) + (x[i] . A_j) . B_j   with j = adapter_ids[i],   or without the second
  * term if adapter_ids[i] is negative (or not below n_adapters),
- * for M <= max_m <= 64 tokens in one launch per eight tokens.  adapter_ids: HOST array of m int32,
+ * for M <= max_m <= 64 tokens in one launch for up to eight or, with fp16 X, 9 to 32 tokens, else one per eight.  adapter_ids: HOST array of m int32,
  * read before the call returns.  Decode family only; eora_linear_forward on such a handle returns
  * EORA_ERR_UNSUPPORTED.  Cost: every adapter's A and B are streamed once per launch whatever the ids.
  */
@@ -217,14 +217,14 @@ int eora_linear_dump(eora_linear_t h, int32_t what, void* out, void* stream);
 /*
  * Status word latched by the kernels (0 = fine, EORA_ERR_DEVICE_TIMEOUT = a bounded wait ran
  * out).  Reads device memory with a blocking copy: call after synchronising.  Clears the word; if it was
- * not zero, the handle's scratch (partial sums, t, tickets) is put back to its between-calls state as well, so
+ * not zero, the handle's scratch (t, launch numbers) is put back to its between-calls state as well, so
  * that the handle stays usable (the outputs of the call that timed out are undefined).
  */
 int eora_linear_last_device_status(eora_linear_t h);
 
 /*
  * Diagnostics.  eora_linear_decode_grid: how many CTAs a decode forward(m) launches (0 if m is
- * not served by the decode family); each CTA has sixteen warps.  eora_linear_set_trace: give the
+ * not served by the decode family); a CTA has eight or sixteen warps.  eora_linear_set_trace: give the
  * handle a caller-owned device buffer (or NULL to switch tracing off).  A decode forward then
  * records four %globaltimer values (nanoseconds) per warp, at uint64 index
  * 4 * (16 * cta + warp) + k:  k = 0 kernel entry, 1 dependency wait over, 2 first share of the
@@ -268,7 +268,7 @@ int eora_linear_forward_noalloc(const eora_linear_config* cfg, const eora_linear
                                 int32_t m, void* y, void* stream);
 
 /*
- * Bytes of device memory the handle owns: the re-tiled weights; the scratch the kernels need (partial sums, t, tickets:
+ * Bytes of device memory the handle owns: the re-tiled weights; the scratch the kernels need (t, launch numbers:
  * a few hundred KB to a few MB); and the staging buffers of the *_host entry points, [max_m][d_in] + [max_m][d_out],
  * which are allocated by the first *_host call on the handle (0 before that): a model whose activations stay on the
  * device keeps the memory saving that compression buys (paper Section 4.5, the model-size table).
@@ -286,9 +286,9 @@ int64_t eora_linear_staging_bytes(eora_linear_t h);
  */
 int eora_linear_set_wait_limit(eora_linear_t h, uint64_t ns);
 /*
- * Self-test of that path: enqueues a one-warp kernel that leaves a partial sum, a partial t and a ticket in the handle's
- * scratch (what a kernel that gives up leaves behind) and then waits, bounded by the handle's limit, for a count nobody
- * raises.  After synchronising, eora_linear_last_device_status must report EORA_ERR_DEVICE_TIMEOUT, and the next forward
+ * Self-test of that path: enqueues a one-warp kernel that leaves a stale word of t in the handle's
+ * scratch and then waits, bounded by the handle's limit, for one that nobody
+ * sends.  After synchronising, eora_linear_last_device_status must report EORA_ERR_DEVICE_TIMEOUT, and the next forward
  * must be correct again.  Nothing faults or hangs: the wait returns by itself.
  */
 int eora_linear_selftest_wait_timeout(eora_linear_t h, void* stream);

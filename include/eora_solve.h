@@ -9,8 +9,9 @@
  *
  * What is computed.  Steps 2-6 define B' = U' S' and A = S'^{-1} U'^T dW, where U' (d x r) and S'^2 are the top-r
  * eigenpairs of  dW (X~ X~^T) dW^T = dW' dW'^T  (the left singular vectors and squared singular values of dW'):
- * with dW' = U' S' V'^T,  A = V'^T Q'^{-1} = S'^{-1} U'^T dW' Q'^{-1} = S'^{-1} U'^T dW.  The library forms that
- * d x d matrix and takes its top-r eigenpairs by subspace iteration with a Rayleigh-Ritz step, so it needs neither
+ * with dW' = U' S' V'^T,  A = V'^T Q'^{-1} = S'^{-1} U'^T dW' Q'^{-1} = S'^{-1} U'^T dW.  The library takes the
+ * top-r eigenpairs of P P^T, P = dW X~, by subspace iteration with the smaller of P P^T (d x d) and P^T P (n x n), and a
+ * Rayleigh-Ritz step, so it needs neither
  * the k x k eigendecomposition nor the inverse square roots of its (possibly zero) eigenvalues.  B' and A are
  * determined up to one common sign per rank-one pair (as with any SVD); B' A, sigma and the remaining loss are unique
  * where sigma_r > sigma_{r+1}.  Subspace iteration converges like (sigma_{m+1} / sigma_r)^(2 iters), m = r + oversample:

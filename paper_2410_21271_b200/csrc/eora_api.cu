@@ -77,8 +77,8 @@ int y_elem_bytes(int y_dtype) { return y_dtype == EORA_Y_F32 ? 4 : 2; }
 int pick_path(const Handle* h, int m) {
   if (h->cfg.kernel_policy == EORA_POLICY_GENERIC) return EORA_PATH_GENERIC;
   // The decode family streams the weights once per eight tokens.  From two passes on (m > 8) one launch of the
-  // tensor-core family is cheaper: for up to 64 tokens it splits the reduction axis over several CTAs per tile, so it
-  // is no longer a chain over all of d_in (measured, 4-bit q-shaped layer, 16 tokens: 23.6 us in two passes, 17 us so).
+  // tensor-core family is cheaper: up to 32 tokens it takes one pass too (decode_mid.cu: three blocks at 12 tokens 196 us),
+  // beyond, its tiles share their reduction axis between CTAs, so that it is no chain over all of d_in.
   if (decode_tc_supported(h, m)) return EORA_PATH_DECODE;   // EORA_POLICY_TMEM_DECODE: one pass over the weights per sixteen tokens
   const bool dec = m <= 64 && decode_supported(h, m), pre = prefill_supported(h, m);
   if (dec && pre) return EORA_PATH_PREFILL;

@@ -1,4 +1,4 @@
-// Prefill kernel family (M > 64, and 16 < M <= 64 where it beats the decode passes): Y = X.deq(Wq) + (X.A).B
+// Prefill kernel family (more than 32 tokens; fewer where decode_mid.cu does not take the layer): Y = X.deq(Wq) + (X.A).B
 // (paper Eq. 4) as a tcgen05 GEMM.
 //
 // The paper measures only batch-1 decoding (Section 4.5); for many tokens the layer is a dense
@@ -11,8 +11,10 @@
 //   * MMA "B" operand (up to 256 rows): a tile of tokens of X, K-major, brought in by TMA
 //     (cp.async.bulk.tensor, 128-byte swizzle, no multicast) into the same ring of k-block stages as
 //     the dequantised weight tile;
-//   * one thread issues tcgen05.mma (M = 128, N = tokens, K = 16) with the fp32 accumulator in tensor
-//     memory; tcgen05.commit releases the ring slots when the MMAs have drained;
+//   * an elected lane of one warp issues tcgen05.mma (M = 128, N = tokens, K = 16) with the fp32 accumulator in
+//     tensor memory; tcgen05.commit releases the ring slots when the MMAs have drained;
+//   * where whole tiles would leave SMs idle, a cluster of two, four or eight CTAs shares a tile's reduction axis and
+//     adds its parts through distributed shared memory (pick_tilings chooses tile and cluster for both launches);
 //   * the low-rank term is a K-extension: after the d_in/64 backbone k-blocks come r/64 k-blocks whose
 //     token operand is t = X.A (fp16, from a first launch of the same kernel with A as the weight) and
 //     whose weight operand is B, so (X.A).B lands in the same accumulator.  The two launches overlap:
@@ -413,9 +415,8 @@ __global__ void __launch_bounds__(kThreadsP, 1) k_prefill(const __grid_constant_
                                                           const __grid_constant__ CUtensorMap tm_t_small, const PrefillArgs p) {
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   // One ring for both operands: stage s holds the token tile and the dequantised weight tile of a k-block, full_w[s]
-  // collects the copy's bytes and the dequant warps' arrivals, empty_w[s] one commit.  The thread that issues the MMAs
-  // is what bounds a k-block (every MMA blocks it for the ~130 cycles its 128-row operand takes to load), so it gets
-  // one wait and one commit per k-block instead of two of each.
+  // collects the copy's bytes and the dequant warps' arrivals, empty_w[s] one commit: one wait and one commit per k-block for
+  // the warp that issues the MMAs.
   __shared__ __align__(8) uint64_t full_w[kMaxWStages], empty_w[kMaxWStages], acc_full;
   __shared__ uint32_t tmem_base_s;
   __shared__ uint32_t sp_lut[16];        // 2:4 expansion selectors (2:4 backbones only)
