@@ -237,9 +237,14 @@ __device__ __forceinline__ void dequant_store(Packed<FMT> r, uint32_t sc2, uint3
 #pragma unroll
     for (int p = 0; p < 4; ++p) { out[p][0] = r.v[p].x; out[p][1] = r.v[p].y; out[p][2] = r.v[p].z; out[p][3] = r.v[p].w; }
   } else if constexpr (FMT == FMT_SP24 || FMT == FMT_SQ4) {
-    // A quad's two kept values (one register) are spread over its four positions (two registers) with two
-    // byte permutes whose selectors come from a 16-entry table in shared memory indexed by the quad's
-    // position nibble (sp24_selectors).
+    // A quad's two kept values (one register) are spread over its four positions (two registers) with two byte
+    // permutes.  Their selectors (sp24_selectors) are four bytes of 0x44, zero, with 0x10 at the first value's position and 0x32
+    // at the second's: two shifts and one three-input xor.  From a table in shared memory, as in the decode kernels, they cost fewer
+    // instructions, but the loads compete with the MMAs' operands (2:4 14336 x 4096, 2048 tokens: 242 -> 219 us without them).  4-bit
+    // kept values, which need the issue slots more, take every other selector from the table (a block at 2048 tokens 905 -> 880 us,
+    // at 64 tokens 133.5 against 134.3).
+    const uint32_t at0[2] = {(r.meta << 3) & 0x18181818u, (r.meta >> 1) & 0x18181818u};      // 8 * position of the first value, even / odd quads
+    const uint32_t at1[2] = {(r.meta << 1) & 0x18181818u, (r.meta >> 3) & 0x18181818u};      // of the second
     [[maybe_unused]] ZC zc;
     if constexpr (FMT == FMT_SQ4) make_zc_p<FMT>(zc, zz2);
 #pragma unroll
@@ -257,10 +262,12 @@ __device__ __forceinline__ void dequant_store(Packed<FMT> r, uint32_t sc2, uint3
       }
 #pragma unroll
       for (int quad = 0; quad < 2; ++quad) {
-        const int sh = 8 * p + 4 * quad - 2;                                  // nibble * 4 = byte offset into the table
-        const uint32_t offb = (sh < 0 ? (r.meta << 2) : (r.meta >> (sh < 0 ? 0 : sh))) & 0x3Cu;
         uint32_t sel;
-        asm volatile("ld.shared.u32 %0, [%1];" : "=r"(sel) : "r"(lut + offb));
+        if (FMT == FMT_SQ4 && quad == 1) {
+          asm volatile("ld.shared.u32 %0, [%1];" : "=r"(sel) : "r"(lut + ((r.meta >> (8 * p + 2)) & 0x3Cu)));
+        } else {                                                              // (shifts modulo 32: the bits above a byte's position are those of the bytes behind it)
+          sel = 0x44444444u ^ __funnelshift_l(0u, 0x54u, at0[quad] >> (8 * p)) ^ __funnelshift_l(0u, 0x76u, at1[quad] >> (8 * p));
+        }
         out[p][2 * quad] = prmt(vq[quad], 0u, sel);
         out[p][2 * quad + 1] = prmt(vq[quad], 0u, sel >> 16);
       }
@@ -419,7 +426,7 @@ __global__ void __launch_bounds__(kThreadsP, 1) k_prefill(const __grid_constant_
   // the warp that issues the MMAs.
   __shared__ __align__(8) uint64_t full_w[kMaxWStages], empty_w[kMaxWStages], acc_full;
   __shared__ uint32_t tmem_base_s;
-  __shared__ uint32_t sp_lut[16];        // 2:4 expansion selectors (2:4 backbones only)
+  __shared__ uint32_t sp_lut[16];        // 2:4 expansion selectors (2:4 backbones of 4-bit codes only)
   __shared__ int fail_s;                 // set by an epilogue warp whose bounded wait ran out
   // 1024-byte alignment of the operand tiles (the swizzle pattern is anchored at 1 KB)
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -455,7 +462,7 @@ __global__ void __launch_bounds__(kThreadsP, 1) k_prefill(const __grid_constant_
   const uint32_t xbytes = (uint32_t)bt * 128;               // bytes of a token tile; the ring's slots are p.bt * 128 apart
   const uint32_t xslot = (uint32_t)p.bt * 128;
 
-  if constexpr (WF == FMT_SP24 || WF == FMT_SQ4) {
+  if constexpr (WF == FMT_SQ4) {
     if (threadIdx.x >= 32 && threadIdx.x < 48) sp_lut[threadIdx.x - 32] = sp24_selectors(threadIdx.x - 32);
   }
   const uint32_t lut = smem_u32(sp_lut);
