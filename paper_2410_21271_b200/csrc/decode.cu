@@ -620,7 +620,7 @@ template <int WF, int MODE, bool SZ2>
 __global__ void __launch_bounds__(32 << warp_log(MODE), MODE == 1 ? 2 : 1) k_decode(const __grid_constant__ DecodeArgs p) {
   constexpr int kWarpLog = warp_log(MODE), kWarps = 1 << kWarpLog;
   extern __shared__ __align__(128) uint8_t smem[];
-  __shared__ uint32_t lut_s[16];
+  __shared__ __align__(256) uint32_t lut_s[16];
   __shared__ __align__(16) uint32_t zero_s[40];    // what lanes without a token read as their activations
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   asm volatile("griddepcontrol.launch_dependents;");
@@ -650,10 +650,7 @@ __global__ void __launch_bounds__(32 << warp_log(MODE), MODE == 1 ? 2 : 1) k_dec
     const uint8_t* w_part = p.w_q + ((size_t)rank * p.w_nt * p.pairs + (size_t)t0 * P) * blob_b;
     if (p.ks == 2) cluster_arrive();               // (that the partner runs at all, before anything is written to it)
     uint32_t lut = 0;
-    if constexpr (WF == FMT_SP24 || WF == FMT_SQ4) {
-      if (threadIdx.x < 16) lut_s[threadIdx.x] = sp24_selectors(threadIdx.x);
-      lut = smem_u32(lut_s);
-    }
+    if constexpr (WF == FMT_SP24 || WF == FMT_SQ4) lut = sp24_lut(lut_s);
     if (threadIdx.x < 40) zero_s[threadIdx.x] = 0u;
 
     // A warp's run of a chunk of n pairs: blobs [lo, hi) in (row tile, pair) order.  They come through the warp's own ring in

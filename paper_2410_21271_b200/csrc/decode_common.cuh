@@ -229,7 +229,11 @@ __host__ __device__ constexpr uint32_t sp24_selectors(uint32_t nib) {
   }
   return r;
 }
-constexpr int kSp24LutBytes = 64;       // 16 entries; every entry in its own shared-memory bank
+// The table in shared memory: 16 words, each in a bank of its own; `mem` is aligned to 256 bytes (half_frags).  Returns its address.
+__device__ __forceinline__ uint32_t sp24_lut(uint32_t (&mem)[16]) {
+  if (threadIdx.x < 16) mem[threadIdx.x] = sp24_selectors(threadIdx.x);
+  return smem_u32(mem);
+}
 
 // The eight byte quads (one code per byte) of a lane's 32 codes of a 3-bit tile: q[part][quad].
 __device__ __forceinline__ void q3_quads(uint32_t w0, uint32_t w1, uint32_t w2, uint32_t (&q)[4][2]) {
@@ -371,7 +375,7 @@ template <int FMT, bool SZ2> __device__ __forceinline__ void load_blob_s(RawBlob
 }
 
 // The wide operand of two of the tile's four mma.m16n8k16 as exact fp16 values: those of its 32-element block blk (0, 1).  `aux`:
-// shared-memory address of the 2:4 expansion table; unused by other formats.
+// shared-memory address of the 2:4 expansion table (a multiple of 256); unused by other formats.
 template <int FMT>
 __device__ __forceinline__ void half_frags(const RawTile<FMT>& r, const ZC& zc, int blk, uint32_t (&a0)[4], uint32_t (&a1)[4], uint32_t aux) {
 #pragma unroll
@@ -414,10 +418,10 @@ __device__ __forceinline__ void half_frags(const RawTile<FMT>& r, const ZC& zc, 
         } else {
           kept = h2sub(and_or((blk ? r.v.y : r.v.x) >> (8 * hf + 4 * quad), 0x000f000fu, kMagic), zc.c[hf][0]);
         }
-        const int sh = 8 * (blk * 2 + hf) + 4 * quad - 2;           // nibble * 4 = byte offset into the table
-        const uint32_t offb = (sh < 0 ? (r.meta << 2) : (r.meta >> (sh < 0 ? 0 : sh))) & 0x3Cu;
+        // Nibble * 4 = byte offset into the table; one permute puts it under the table's address.
+        const uint32_t offs = (quad ? r.meta >> 2 : r.meta << 2) & 0x3C3C3C3Cu;
         uint32_t sel;
-        asm volatile("ld.shared.u32 %0, [%1];" : "=r"(sel) : "r"(aux + offb));
+        asm volatile("ld.shared.u32 %0, [%1];" : "=r"(sel) : "r"(prmt(offs, aux, 0x7650u + (uint32_t)(blk * 2 + hf))));
         (quad ? a1 : a0)[hf] = prmt(kept, 0u, sel);
         (quad ? a1 : a0)[hf + 2] = prmt(kept, 0u, sel >> 16);
       }

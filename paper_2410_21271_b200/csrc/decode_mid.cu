@@ -231,7 +231,7 @@ __device__ __forceinline__ int sub_of(const MidArgs& p, uint32_t tile) {
 template <int WF, bool SZ2, int NT>
 __global__ void __launch_bounds__(kThreads, 1) k_mid(const __grid_constant__ CUtensorMap tm, const __grid_constant__ MidArgs p) {
   extern __shared__ __align__(128) uint8_t smem[];
-  __shared__ uint32_t lut_s[16];
+  __shared__ __align__(256) uint32_t lut_s[16];
   __shared__ __align__(8) uint64_t xbars_s[kMaxXSlots], bars_s[kWarps * kMaxSlots];
   __shared__ uint32_t readers_s[kMaxXSlots];       // warps that are done with a slot of X
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -243,8 +243,8 @@ __global__ void __launch_bounds__(kThreads, 1) k_mid(const __grid_constant__ CUt
   const uint32_t P = rank ? p.np - p.pairs0 : p.pairs0, pr0 = rank ? p.pairs0 : 0u;
   const uint32_t xs = smem_u32(smem), xfull = smem_u32(xbars_s);
   constexpr uint32_t kXSlot = NT * 2048;
-  if constexpr (WF == FMT_SP24 || WF == FMT_SQ4) { if (threadIdx.x < 16) lut_s[threadIdx.x] = sp24_selectors(threadIdx.x); }
-  const uint32_t lut = smem_u32(lut_s);
+  uint32_t lut = 0;
+  if constexpr (WF == FMT_SP24 || WF == FMT_SQ4) lut = sp24_lut(lut_s);
   if (warp == 0 && lane < kMaxXSlots) {
     mbar_init_a(xfull + 8 * lane, 1);
     readers_s[lane] = 0u;
