@@ -164,7 +164,8 @@ int eora_linear_forward_fused(eora_linear_t h, const void* x, int32_t m, void* c
  *     y[i] = x[i] . deq(Wq) + (x[i] . A_j) . B_j   with j = adapter_ids[i],   or without the second
  * term if adapter_ids[i] is negative (or not below n_adapters),
  * for M <= max_m <= 64 tokens in one launch for up to eight or, with fp16 X, 9 to 32 tokens, else one per eight.  adapter_ids: HOST array of m int32,
- * read before the call returns.  Decode family only; eora_linear_forward on such a handle returns
+ * read before the call returns.  Every operand is multiplied as stored (q - z, t as an fp16 high and low part), whichever kernel serves the
+ * number of tokens, so that a token's result does not lose precision with the size of its batch.  eora_linear_forward on such a handle returns
  * EORA_ERR_UNSUPPORTED.  Cost: every adapter's A and B are streamed once per launch whatever the ids.
  */
 int eora_linear_create_multi(const eora_linear_config* cfg, const eora_linear_weights* weights, int32_t n_adapters,

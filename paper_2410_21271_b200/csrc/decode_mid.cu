@@ -17,6 +17,11 @@
 // fragment load of a warp reads are 512 contiguous bytes.  The warp that is the last to read a slot refills it.  The weights come through a ring per warp.  Weights
 // are RN((q - z) * s) in fp16, as in prefill.cu, or, up to 16 tokens, exact q - z with the scale applied to the group's sums.
 //
+// Several adapters (EXACT): such a batch may as well go through decode.cu, eight tokens at a time, and its results must not
+// depend on how many requests it happens to hold.  All operands are then multiplied as there: exact q - z at every number of tokens, t sent
+// in fp32 and multiplied as an fp16 high and low part.  Rounding t once, and the weights from 17 tokens on, was 2.6 to 2000 times further
+// from float64 (2048 x 1024, three adapters of rank 64, fp32 Y, 9 to 32 tokens: 3e-5 to 2e-4 of Y).
+//
 // Measured: four LLaMA3-8B blocks, 4-bit backbone and adapters, 16 tokens 544 -> 261 us (see also mid_supported).
 #include <cuda.h>
 #include "decode_common.cuh"
@@ -55,7 +60,7 @@ struct MidArgs {
   uint32_t t_chunk;                       // pairs of t in shared memory at a time
   uint32_t adp_pairs;                     // several adapters: pair p of t belongs to adapter p / adp_pairs (0: one adapter)
   signed char adp[kMaxPass];              // adapter of every token (-1: none)
-  unsigned long long* t_part;             // [m][t_cols / 2] words (two columns as fp16, launch number)
+  unsigned long long* t_part;             // [m][t_cols / 2] words (two columns as fp16, launch number); EXACT: [m][t_cols] words (fp32, launch number)
   unsigned long long* launches;
   int* dev_status;
   int m, m_log, t_cols, y_dtype;
@@ -96,10 +101,11 @@ __device__ __forceinline__ void weights_half(const RawTile<FMT>& r, int blk, con
 // One pair of T row tiles (blobs `stride` apart) times the activations of 8 NT tokens at x: [4 blocks of 32 k][8 NT tokens][32 fp16],
 // x already at this lane's token and piece.  Up to 16 tokens the scale of a quantised group is applied to the group's sums (8 NT T multiplications
 // a lane instead of 32 T on the weights); with more the sums would need as many registers again.
-template <int FMT, bool SZ2, int NT, int T>
-__device__ __forceinline__ void product(uint32_t blob, uint32_t stride, int lane, uint32_t x, uint32_t lut, float (&acc)[T][NT][4]) {
+// EXACT: the scale is always applied to the sums.
+template <int FMT, bool SZ2, int NT, int T, bool EXACT>
+__device__ __forceinline__ void product(uint32_t blob, uint32_t stride, int lane, uint32_t x, uint32_t lut, float (*acc)[NT][4]) {
   constexpr int tb = tile_bytes(FMT);
-  constexpr bool late = fmt_quantised(FMT) && NT <= 2;
+  constexpr bool late = fmt_quantised(FMT) && (NT <= 2 || EXACT);
   SZ z[T];
   float d[late ? T : 1][late ? NT : 1][4];
   if constexpr (late) {
@@ -150,11 +156,32 @@ __device__ __forceinline__ void product(uint32_t blob, uint32_t stride, int lane
   }
 }
 
+// The sums of exact products join a row tile's, with the group's scales.
+template <int NT>
+__device__ __forceinline__ void add_scaled(float (&acc)[NT][4], float (&d)[NT][4], const SZ& z) {
+  const float sa = __half2float(__ushort_as_half((unsigned short)z.s[0])), sb = __half2float(__ushort_as_half((unsigned short)z.s[1]));
+#pragma unroll
+  for (int n = 0; n < NT; ++n)
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      acc[n][i] = fmaf(d[n][i], i < 2 ? sa : sb, acc[n][i]);
+      d[n][i] = 0.f;
+    }
+}
+
 // A and B: the format is known at run time only (one uniform branch per blob).
 // A: a blob times a pair of X, as above.
-template <int FMT, int NT>
+template <int FMT, int NT, bool EXACT>
 __device__ __forceinline__ void product_a1(uint32_t blob, uint32_t sz2, int lane, uint32_t x, float (&acc)[NT][4]) {
   constexpr int tb = tile_bytes(FMT);
+  constexpr bool late = EXACT && fmt_quantised(FMT);
+  float d[late ? NT : 1][4];
+  if constexpr (late) {
+#pragma unroll
+    for (int n = 0; n < NT; ++n)
+#pragma unroll
+      for (int i = 0; i < 4; ++i) d[n][i] = 0.f;
+  }
   SZ z;
 #pragma unroll
   for (int c = 0; c < 2; ++c) {
@@ -164,30 +191,40 @@ __device__ __forceinline__ void product_a1(uint32_t blob, uint32_t sz2, int lane
 #pragma unroll
     for (int b = 0; b < 2; ++b) {
       uint32_t a[2][4];
-      weights_half<FMT, true>(r, b, z, 0u, a);
+      weights_half<FMT, !late>(r, b, z, 0u, a);
 #pragma unroll
       for (int n = 0; n < NT; ++n) {
         const uint4 v = lds_u4(x + (2 * c + b) * (NT * 512) + n * 512);
-        mma16816(acc[n], a[0], v.x, v.y);
-        mma16816(acc[n], a[1], v.z, v.w);
+        mma16816(late ? d[late ? n : 0] : acc[n], a[0], v.x, v.y);
+        mma16816(late ? d[late ? n : 0] : acc[n], a[1], v.z, v.w);
       }
     }
+    if constexpr (late) { if (c == 1 || sz2) add_scaled<NT>(acc, d, z); }
   }
 }
-template <int NT>
+template <int NT, bool EXACT>
 __device__ __forceinline__ void product_a(int fmt, uint32_t sz2, uint32_t blob, int lane, uint32_t x, float (&acc)[NT][4]) {
   switch (fmt) {
-    case FMT_F16: product_a1<FMT_F16, NT>(blob, 0u, lane, x, acc); break;
-    case FMT_Q8: product_a1<FMT_Q8, NT>(blob, 0u, lane, x, acc); break;
-    case FMT_Q4: product_a1<FMT_Q4, NT>(blob, sz2, lane, x, acc); break;
-    case FMT_Q3: product_a1<FMT_Q3, NT>(blob, sz2, lane, x, acc); break;
+    case FMT_F16: product_a1<FMT_F16, NT, EXACT>(blob, 0u, lane, x, acc); break;
+    case FMT_Q8: product_a1<FMT_Q8, NT, EXACT>(blob, 0u, lane, x, acc); break;
+    case FMT_Q4: product_a1<FMT_Q4, NT, EXACT>(blob, sz2, lane, x, acc); break;
+    case FMT_Q3: product_a1<FMT_Q3, NT, EXACT>(blob, sz2, lane, x, acc); break;
     default: break;
   }
 }
-// B: one 64-element tile of each of two row tiles, each with its scale entry behind it (kBStride bytes apart), times 64 columns of t.
+// B: one 64-element tile of each of two row tiles, each with its scale entry behind it (kBStride bytes apart), times 64 columns of t
+// (EXACT: their high part, the low part behind it).
 template <int FMT> constexpr uint32_t kBStride = tile_bytes(FMT) + 64;
-template <int FMT, int NT>
+template <int FMT, int NT, bool EXACT>
 __device__ __forceinline__ void product_b1(uint32_t buf, int lane, uint32_t x, float (&acc)[2][NT][4]) {
+  constexpr bool late = EXACT && fmt_quantised(FMT);
+  float d[late ? NT : 1][4];
+  if constexpr (late) {
+#pragma unroll
+    for (int n = 0; n < NT; ++n)
+#pragma unroll
+      for (int i = 0; i < 4; ++i) d[n][i] = 0.f;
+  }
   // one row tile after the other: an fp16 tile is 16 registers a lane
 #pragma unroll
   for (int u = 0; u < 2; ++u) {
@@ -198,23 +235,26 @@ __device__ __forceinline__ void product_b1(uint32_t buf, int lane, uint32_t x, f
 #pragma unroll
     for (int b = 0; b < 2; ++b) {
       uint32_t a[2][4];
-      weights_half<FMT, true>(r, b, z, 0u, a);
+      weights_half<FMT, !late>(r, b, z, 0u, a);
 #pragma unroll
-      for (int n = 0; n < NT; ++n) {
-        const uint4 v = lds_u4(x + b * (NT * 512) + n * 512);
-        mma16816(acc[u][n], a[0], v.x, v.y);
-        mma16816(acc[u][n], a[1], v.z, v.w);
-      }
+      for (int p = 0; p < (EXACT ? 2 : 1); ++p)
+#pragma unroll
+        for (int n = 0; n < NT; ++n) {
+          const uint4 v = lds_u4(x + p * (NT * 1024) + b * (NT * 512) + n * 512);
+          mma16816(late ? d[late ? n : 0] : acc[u][n], a[0], v.x, v.y);
+          mma16816(late ? d[late ? n : 0] : acc[u][n], a[1], v.z, v.w);
+        }
     }
+    if constexpr (late) add_scaled<NT>(acc[u], d, z);
   }
 }
-template <int NT>
+template <int NT, bool EXACT>
 __device__ __forceinline__ void product_b(int fmt, uint32_t buf, int lane, uint32_t x, float (&acc)[2][NT][4]) {
   switch (fmt) {
-    case FMT_F16: product_b1<FMT_F16, NT>(buf, lane, x, acc); break;
-    case FMT_Q8: product_b1<FMT_Q8, NT>(buf, lane, x, acc); break;
-    case FMT_Q4: product_b1<FMT_Q4, NT>(buf, lane, x, acc); break;
-    case FMT_Q3: product_b1<FMT_Q3, NT>(buf, lane, x, acc); break;
+    case FMT_F16: product_b1<FMT_F16, NT, EXACT>(buf, lane, x, acc); break;
+    case FMT_Q8: product_b1<FMT_Q8, NT, EXACT>(buf, lane, x, acc); break;
+    case FMT_Q4: product_b1<FMT_Q4, NT, EXACT>(buf, lane, x, acc); break;
+    case FMT_Q3: product_b1<FMT_Q3, NT, EXACT>(buf, lane, x, acc); break;
     default: break;
   }
 }
@@ -227,8 +267,8 @@ __device__ __forceinline__ int sub_of(const MidArgs& p, uint32_t tile) {
     if (i < p.n_sub && tile >= p.sub_tile0[i]) s = i;
   return s;
 }
-// NT: tokens / 8.
-template <int WF, bool SZ2, int NT>
+// NT: tokens / 8.  EXACT: several adapters (see above).
+template <int WF, bool SZ2, int NT, bool EXACT>
 __global__ void __launch_bounds__(kThreads, 1) k_mid(const __grid_constant__ CUtensorMap tm, const __grid_constant__ MidArgs p) {
   extern __shared__ __align__(128) uint8_t smem[];
   __shared__ __align__(256) uint32_t lut_s[16];
@@ -242,7 +282,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_mid(const __grid_constant__ CUt
   const uint32_t d0 = share_lo(is_a ? p.a_tiles : p.w_dbl, cl), nD = share_n(is_a ? p.a_tiles : p.w_dbl, cl);
   const uint32_t P = rank ? p.np - p.pairs0 : p.pairs0, pr0 = rank ? p.pairs0 : 0u;
   const uint32_t xs = smem_u32(smem), xfull = smem_u32(xbars_s);
-  constexpr uint32_t kXSlot = NT * 2048;
+  constexpr uint32_t kXSlot = NT * 2048, kTHalf = EXACT ? NT * 2048 : NT * 1024;      // bytes of a pair of X; of 64 columns of t
   uint32_t lut = 0;
   if constexpr (WF == FMT_SP24 || WF == FMT_SQ4) lut = sp24_lut(lut_s);
   if (warp == 0 && lane < kMaxXSlots) {
@@ -320,8 +360,14 @@ __global__ void __launch_bounds__(kThreads, 1) k_mid(const __grid_constant__ CUt
       if (ok && !mbar_try_wait_a(xfull + 8 * s, par) && !mbar_wait_lane(xfull + 8 * s, par, p.dev_status)) ok = false;
       if (!__all_sync(0xffffffffu, ok)) { ok = false; break; }
       const uint32_t src = ring.base + ring.so, x = xl + s * kXSlot;
-      if (is_a) product_a<NT>(p.a_fmt, p.a_sz2, src, lane, x, acc[0]);
-      else product<WF, SZ2, NT, T>(src, blob_b, lane, x, lut, acc);
+      if (is_a) {
+        product_a<NT, EXACT>(p.a_fmt, p.a_sz2, src, lane, x, acc[0]);
+      } else if constexpr (EXACT && NT > 2 && fmt_quantised(WF)) {      // one row tile after the other: sums of both would not fit the registers
+#pragma unroll
+        for (int u = 0; u < T; ++u) product<WF, SZ2, NT, 1, true>(src + u * blob_b, blob_b, lane, x, lut, acc + u);
+      } else {
+        product<WF, SZ2, NT, T, EXACT>(src, blob_b, lane, x, lut, acc);
+      }
       __syncwarp();                                // every lane is done with both slots
       if (lane == 0 && q + xslots < P) {           // a pair of X is read by one warp per unit
         uint32_t done = nD - 1;
@@ -365,12 +411,13 @@ __global__ void __launch_bounds__(kThreads, 1) k_mid(const __grid_constant__ CUt
       h = hi > lo ? ((lo - c0) << h_log) + j : 0u;
       h_end = hi > lo ? (hi - c0) << h_log : 0u;
     };
-    // step e of a chunk: four columns of one token (16 steps per half and token)
+    // step e of a chunk: two words of one token, i.e. four columns (16 steps per half and token) or, EXACT, two (32 steps)
+    constexpr uint32_t kSLog = EXACT ? 5 : 4, kSteps = 1u << kSLog, kWordCols = EXACT ? 1 : 2;
     auto t_src = [&](uint32_t e, uint32_t& tok, uint32_t& col) {
-      const uint32_t h = e >> (4 + p.m_log);
-      tok = (e >> 4) & m_mask;
-      col = (c0 + (h >> h_log)) * 128 + half_of(h) * 64 + (e & 15) * 4;
-      return p.t_part + ((size_t)tok * p.t_cols + col) / 2;
+      const uint32_t h = e >> (kSLog + p.m_log);
+      tok = (e >> kSLog) & m_mask;
+      col = (c0 + (h >> h_log)) * 128 + half_of(h) * 64 + (e & (kSteps - 1)) * (2 * kWordCols);
+      return p.t_part + ((size_t)tok * p.t_cols + col) / kWordCols;
     };
     uint32_t h, h_end, tok, col;
     span(h, h_end);
@@ -378,10 +425,10 @@ __global__ void __launch_bounds__(kThreads, 1) k_mid(const __grid_constant__ CUt
     bool asked = true;
 #pragma unroll 1
     for (;;) {
-      // t as fp16, zero for tokens that do not use the pair's adapter and in the columns past A's rows (padding); the loads of a batch
+      // t as fp16 (EXACT: high and low part, error 2^-22 of the value), zero for tokens that do not use the pair's adapter and in the columns past A's rows (padding); the loads of a batch
       // go out together (each is a round trip to L2), those of the first before the barrier
       constexpr int kBatch = 2;
-      const uint32_t steps = (min(p.t_chunk, c_end - c0) << h_log) << (4 + p.m_log);
+      const uint32_t steps = (min(p.t_chunk, c_end - c0) << h_log) << (kSLog + p.m_log);
 #pragma unroll 1
       for (uint32_t e0 = 0; e0 < steps; e0 += kBatch * kThreads) {
         TWords tw[kBatch];
@@ -400,8 +447,17 @@ __global__ void __launch_bounds__(kThreads, 1) k_mid(const __grid_constant__ CUt
           uint32_t v0 = 0u, v1 = 0u;
           if (col < p.a_nt * 16 && !(p.adp_pairs && p.adp[tok] != (int)((col >> 7) / p.adp_pairs)) &&
               wait_t(tw[k], src, launch, p.wait_ns, p.dev_status)) { v0 = (uint32_t)tw[k].a; v1 = (uint32_t)tw[k].b; }
-          const uint32_t i = e & 15, dst = xs + (e >> (4 + p.m_log)) * (NT * 1024) + (i >> 3) * (NT * 512) + tok * 64 + (i & 7) * 8;
-          asm volatile("st.shared.v2.u32 [%0], {%1, %2};" ::"r"(dst), "r"(v0), "r"(v1) : "memory");
+          const uint32_t i = e & (kSteps - 1), blk = i >> (kSLog - 1), in_blk = i & (kSteps / 2 - 1);      // 32 columns = 64 bytes
+          const uint32_t dst = xs + (e >> (kSLog + p.m_log)) * kTHalf + blk * (NT * 512) + tok * 64 + in_blk * (128 / kSteps);
+          if constexpr (EXACT) {
+            const float f0 = __uint_as_float(v0), f1 = __uint_as_float(v1);
+            const uint32_t hi = pack_h2(f0, f1);
+            const float2 hf = __half22float2(*reinterpret_cast<const __half2*>(&hi));
+            sts_u1(dst, hi);
+            sts_u1(dst + NT * 1024, pack_h2(f0 - hf.x, f1 - hf.y));
+          } else {
+            asm volatile("st.shared.v2.u32 [%0], {%1, %2};" ::"r"(dst), "r"(v0), "r"(v1) : "memory");
+          }
         }
       }
       __syncthreads();
@@ -413,7 +469,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_mid(const __grid_constant__ CUt
           ring.parity ^= 1u;
           if (!__all_sync(0xffffffffu, ok)) { ok = false; break; }
           // (columns of tokens past m hold whatever was there: their sums are not read)
-          product_b<NT>(p.a_fmt, ring.base, lane, xs + h * (NT * 1024) + (lane >> 2) * 64 + (lane & 3) * 16, acc);
+          product_b<NT, EXACT>(p.a_fmt, ring.base, lane, xs + h * kTHalf + (lane >> 2) * 64 + (lane & 3) * 16, acc);
           __syncwarp();
         }
       }
@@ -480,7 +536,14 @@ __global__ void __launch_bounds__(kThreads, 1) k_mid(const __grid_constant__ CUt
 #pragma unroll
       for (uint32_t i = 0; i < 4; ++i) v[i] += inbox[f * OT + min(tok + i, m - 1) * 16 + row];      // (past m: any, not stored)
     }
-    if (is_a) {                                    // two columns of t per word
+    if (is_a && EXACT) {                           // a column of t per word
+#pragma unroll
+      for (uint32_t i = 0; i < 4; ++i)
+        if (tok + i < m) {
+          const unsigned long long word = ((unsigned long long)launch << 32) | __float_as_uint(v[i]);
+          asm volatile("st.volatile.global.u64 [%0], %1;" ::"l"(p.t_part + (size_t)(tok + i) * p.t_cols + (d0 + first + f) * 16 + row), "l"(word) : "memory");
+        }
+    } else if (is_a) {                             // two columns of t per word
 #pragma unroll
       for (uint32_t i = 0; i < 4; ++i) {
         const float o = __shfl_down_sync(0xffffffffu, v[i], 1);
@@ -547,7 +610,8 @@ cudaError_t launch_kernel(const cudaLaunchConfig_t& cfg, const CUtensorMap& tm, 
 }
 template <int WF, bool SZ2>
 cudaError_t launch_nt(const cudaLaunchConfig_t& cfg, const CUtensorMap& tm, const MidArgs& a, int nt, int device) {
-  return nt == 2 ? launch_kernel<k_mid<WF, SZ2, 2>>(cfg, tm, a, device) : launch_kernel<k_mid<WF, SZ2, 4>>(cfg, tm, a, device);
+  if (a.adp_pairs) return nt == 2 ? launch_kernel<k_mid<WF, SZ2, 2, true>>(cfg, tm, a, device) : launch_kernel<k_mid<WF, SZ2, 4, true>>(cfg, tm, a, device);
+  return nt == 2 ? launch_kernel<k_mid<WF, SZ2, 2, false>>(cfg, tm, a, device) : launch_kernel<k_mid<WF, SZ2, 4, false>>(cfg, tm, a, device);
 }
 cudaError_t launch_any(const cudaLaunchConfig_t& cfg, const CUtensorMap& tm, const MidArgs& a, int wf, bool sz2, int nt, int device) {
   switch (wf) {
@@ -607,6 +671,7 @@ bool make_plan(const Handle* h, int m, Plan& pl) {
   if (pl.grid >= (1 << kLaunchShift)) return false;
   const uint32_t nD = a.w_dbl.per + (a.w_dbl.rem ? 1 : 0);
   auto up = [](uint32_t v) { return (v + 127u) & ~127u; };
+  const uint32_t t_half = (h->multi ? 2u : 1u) * NT * 1024 * (a.ks == 2 ? 1 : 2);      // bytes of a CTA's part of 128 columns of t
   const uint32_t x_slot = NT * 2048, seg_b = kWarps * 8 * NT * kSegPitch * 4;
   a.off_inbox = up(seg_b);
   const uint32_t per_a = a.a_tiles.per + (a.a_tiles.rem ? 1 : 0);
@@ -614,11 +679,11 @@ bool make_plan(const Handle* h, int m, Plan& pl) {
   // Slots of X: as many as there are warps to read different pairs at a time, within 128 KB; a ring of up to four slots from what is
   // left, fewer slots of X where that would be less than two.  (A ring also takes half a blob of B per row tile.)
   const uint32_t b_need = ab ? 2u * ((uint32_t)tile_bytes(a.a_fmt) + 64u) : 0u;
-  auto fit = [&](uint32_t slot_b, uint32_t need, uint32_t& xslots, uint32_t& off_ring, uint32_t& slots, uint32_t& pitch) {
+  auto fit = [&](uint32_t slot_b, uint32_t need, uint32_t least, uint32_t& xslots, uint32_t& off_ring, uint32_t& slots, uint32_t& pitch) {
     xslots = most_x;
     if (xslots > a.pairs0) xslots = a.pairs0;
     for (;; --xslots) {
-      off_ring = up(xslots * x_slot);
+      off_ring = up(xslots * x_slot > least ? xslots * x_slot : least);
       const uint32_t room = ((uint32_t)kMaxSmem - off_ring) / kWarps;
       slots = room / slot_b;
       if ((slots >= 2 && room >= need) || xslots <= 2) break;
@@ -629,9 +694,9 @@ bool make_plan(const Handle* h, int m, Plan& pl) {
     if (end > total) total = end;
     return slots >= 1;
   };
-  if (!fit(2 * (uint32_t)h->w.blob, b_need, a.xslots, a.off_ring, a.slots, a.ring_pitch)) return false;
-  if (ab && !fit(a.a_blob, 0u, a.a_xslots, a.a_off_ring, a.a_slots, a.a_pitch)) return false;
-  a.t_chunk = a.off_ring / (NT * 1024) / (a.ks == 2 ? 1 : 2);      // t goes where X was
+  if (!fit(2 * (uint32_t)h->w.blob, b_need, ab ? t_half : 0u, a.xslots, a.off_ring, a.slots, a.ring_pitch)) return false;
+  if (ab && !fit(a.a_blob, 0u, 0u, a.a_xslots, a.a_off_ring, a.a_slots, a.a_pitch)) return false;
+  a.t_chunk = a.off_ring / t_half;                 // t goes where X was
   pl.smem = (int)total;
   return total <= (uint32_t)kMaxSmem;
 }

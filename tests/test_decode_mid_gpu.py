@@ -58,3 +58,33 @@ def test_mid_several_adapters():
     torch.cuda.synchronize()
     check_parity(y.float().cpu().numpy().astype(np.float64), reference(x, "f16", wf, adapters, ids), "multi")
     L.close()
+
+
+@pytest.mark.parametrize("w,ab,K,N,r,n,group", [
+    ("q4", "f16", 2048, 512, 64, 3, 128),
+    ("q3", "q4", 2048, 512, 64, 3, 64),
+    ("q4", "q8", 2048, 512, 40, 2, 128),
+    ("sp24", "f16", 2048, 512, 128, 3, 128),
+    ("sq4", "q3", 2048, 512, 64, 3, 128),
+    ("q4", "f16", 128, 32, 64, 2, 128),                  # one pair: no cluster
+    ("q3", "q4", 640, 96, 512, 8, 128),                  # 32 pairs of t, several chunks
+])
+def test_several_adapters_are_as_exact_at_every_number_of_tokens(w, ab, K, N, r, n, group):
+    """A request's result must not depend on how many others share its batch: products of exact operands (fp16 X, integer q - z, t as
+    an fp16 high and low part) summed in fp32, whatever kernel serves the number of tokens.  The bound, against float64 with an fp32 Y:
+    the sums' rounding (a few 2^-24 of the partial sums, which are at most a few times Y) and the low part's (2^-22 of the compensation)
+    stay below 2^-18; t or the weights rounded once to fp16 would show as 2^-13 to 2^-15."""
+    import torch
+    ids = [i % (n + 1) - 1 for i in range(32)]
+    wf, _, _ = make_case(91, K, N, 0, w=w, group=group)
+    adapters = adapters_for(K, N, r, ab, n, 92)
+    x = gen.make_x(93, len(ids), K)
+    ref = reference(x, "f16", wf, adapters, ids)
+    L = eora.MultiAdapterLayer(wf, adapters, max_m=len(ids), y_dtype="f32")
+    for m in (8, 9, 16, 17, 32):
+        y = L.forward(x_to_torch(x[:m], "f16"), ids[:m])
+        torch.cuda.synchronize()
+        assert L.device_status() == 0
+        rel = orc.parity_errors(y.cpu().numpy().astype(np.float64), ref[:m])[0]
+        assert rel <= 2.0 ** -18, (m, rel)
+    L.close()
