@@ -197,7 +197,7 @@ __device__ __forceinline__ void stage_x_f16(uint8_t* xs, uint32_t pitch, float* 
 #pragma unroll
           for (int o = 1; o < 16; o <<= 1) am = fmaxf(am, __shfl_xor_sync(0xffffffffu, am, o));
           const uint32_t eb = __float_as_uint(am) >> 23;
-          if (eb >= 32u && eb < 240u) { inv = __uint_as_float((267u - eb) << 23); sc = __uint_as_float((eb - 13u) << 23); }   // largest magnitude in [2^13, 2^14)
+          if (eb >= 14u && eb < 255u) { inv = __uint_as_float((267u - eb) << 23); sc = __uint_as_float((eb - 13u) << 23); }   // largest magnitude in [2^13, 2^14); both factors are normal numbers
         }
 #pragma unroll
         for (int e = 0; e < 4; ++e) w[e] = pack_h2(f[2 * e] * inv, f[2 * e + 1] * inv);

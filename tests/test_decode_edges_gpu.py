@@ -48,6 +48,23 @@ def test_decode_bf16_beyond_fp16(M):
     L.close()
 
 
+@pytest.mark.parametrize("M", [1, 2, 5, 8])
+def test_decode_bf16_over_its_whole_range(M):
+    """Blocks of bf16 activations whose largest magnitude lies anywhere between 2^-112 and 2^122 (a sum of 256 products with weights
+    below one still fits a float): each is a block of a power of two times fp16 numbers, so none may be lost or overflow."""
+    K, N = 256, 96
+    wf, _, _ = make_case(47, K, N, 0, w="q3")
+    rng = np.random.default_rng(48)
+    L = eora.Layer(wf, None, None, max_m=M, x_dtype="bf16", y_dtype="f32")
+    for e in (-110, -104, -96, -95, 0, 112, 113, 118):
+        x = rng.uniform(1.0, 2.0, (M, K)) * rng.choice([-1.0, 1.0], (M, K))
+        xb = gen.f32_to_bf16_bits(np.ldexp(x, e).astype(np.float32))
+        ref = orc.forward(xb, "bf16", wf, None, None)
+        scale = 2.0 ** -e                                        # (compared near one: squares of 1e-33 would underflow)
+        check_parity(run_layer(L, xb, "bf16") * scale, ref * scale, f"M{M} 2^{e}")
+    L.close()
+
+
 def test_decode_fused_layers_share_a_cta():
     """Four layers of one to five row tiles each: a cluster's row tiles belong to several layers, with different pairs of t."""
     import torch
