@@ -233,8 +233,10 @@ int eora_linear_last_device_status(eora_linear_t h);
  * forward records, for CTA (0, 0) only, four clock64 values per 64-element k-block (token tile
  * requested / first weight tile dequantised / token tile seen by the MMA warp / MMAs issued) at
  * index 4 * k_block + k, k_block < nkb = d_in / 64 + (rank padded to 128) / 64, and one more row at
- * k_block = nkb: kernel entry / set-up done / accumulators complete / epilogue done; the buffer
- * must hold 4 * ((d_in + rank) / 64 + 4) values.  Tracing costs time; leave it off in production.
+ * k_block = nkb: kernel entry / set-up done / accumulators complete / epilogue done (where a cluster shares the
+ * reduction axis, nkb is this CTA's share); the buffer
+ * must hold 4 * ((d_in + rank) / 64 + 4) values.  Forwards of 9 to 32 tokens that take one pass on mma.sync and those of
+ * EORA_POLICY_TMEM_DECODE record nothing.  Tracing costs time; leave it off in production.
  */
 int eora_linear_decode_grid(eora_linear_t h, int32_t m);
 int eora_linear_set_trace(eora_linear_t h, void* trace_buf);

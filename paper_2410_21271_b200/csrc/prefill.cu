@@ -72,7 +72,6 @@ struct PrefillArgs {
                      // then one more row: kernel entry, set-up done, accumulators complete, epilogue done
 };
 
-#define CTRACE(slot) do { if (p.trace) p.trace[1024 + 4 * blockIdx.x + (slot)] = (long long)globaltimer_ns(); } while (0)
 #define PTRACE(it, slot) do { if (p.trace && blockIdx.x == 0 && blockIdx.y == 0) p.trace[(it) * 4 + (slot)] = clock64(); } while (0)
 
 struct PrefillState {
@@ -468,7 +467,6 @@ __global__ void __launch_bounds__(kThreadsP, 1) k_prefill(const __grid_constant_
   const uint32_t lut = smem_u32(sp_lut);
   if (threadIdx.x == 0) {
     PTRACE(nkb, 0);
-    CTRACE(0);
     fail_s = 0;
     for (int i = 0; i < p.sw; ++i) { mbar_init(full_w + i, 8 * nh + 1); mbar_init(empty_w + i, 1); }
     mbar_init(&acc_full, 1);
@@ -559,7 +557,7 @@ __global__ void __launch_bounds__(kThreadsP, 1) k_prefill(const __grid_constant_
     if (!ok) *reinterpret_cast<volatile int*>(&fail_s) = 1;
     asm volatile("bar.sync 1, 512;" ::: "memory");
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-    if (dw == 0 && lane == 0) { PTRACE(nkb, 2); CTRACE(1); }
+    if (dw == 0 && lane == 0) PTRACE(nkb, 2);
   }
 
   // Epilogue: all sixteen dequant warps, as four groups of four.  A warp can read the quarter of the TMEM lanes that its index
@@ -661,7 +659,7 @@ __global__ void __launch_bounds__(kThreadsP, 1) k_prefill(const __grid_constant_
       }
       if (p.ksplit > 1) asm volatile("bar.sync %0, 128;" ::"r"(2 + grp) : "memory");
     }
-    if (dw == 0 && lane == 0) { PTRACE(nkb, 3); CTRACE(2); }
+    if (dw == 0 && lane == 0) PTRACE(nkb, 3);
   }
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
