@@ -1012,8 +1012,7 @@ bool make_plan(const eora_solve_config* c, Plan& p) {
   p.off_h = take((size_t)p.m * p.m * 8);
   p.off_lam = take((size_t)(2 * p.m + 128) * 8);
   p.off_vf = take((size_t)p.ldm * p.ldm * 4);
-  const size_t least = ((size_t)p.d * p.k + (size_t)p.k * p.k + (size_t)p.d * p.d + 64) * 4;      // what earlier versions reported at least
-  p.total = o > least ? o : least;
+  p.total = o;
   return true;
 }
 inline bool aligned16(const void* q) { return (reinterpret_cast<uintptr_t>(q) & 15) == 0; }

@@ -65,6 +65,19 @@ def test_solve_config_layout_and_argument_checks(lib):
     assert lib.eora_solve_loss(None, None, None, None, None, None, None, None, 0, None) == eora.EORA_ERR_NULL_ARG
 
 
+@pytest.mark.parametrize("d,k,n,r", [(4096, 14336, 2048, 128), (8192, 28672, 2048, 128), (14336, 4096, 2048, 128), (256, 8192, 64, 16)])
+def test_solve_workspace_holds_no_unused_squares(lib, d, k, n, r):
+    """What the solve keeps: dW, P = dW X~, the smaller of P P^T and P^T P or (the loss check) dW - B'A, a copy of X~ where it has to be padded, three
+    skinny matrices and the small fp64 problems; each dimension in whole tiles of 128.  No k x k matrix."""
+    up = lambda v: (v + 127) // 128 * 128
+    m, side = r + 32, min(up(d), up(n)) if n >= r + 32 else up(d)
+    widest = max(up(d), up(k), up(n))
+    large = up(d) * up(k) + up(d) * up(n) + max(side * side, d * k) + up(k) * up(n)
+    skinny = 3 * widest * (m + 160)
+    small = 8 * (34 * m * m + 16 * (m + 16) + 2 * m + 128) + 4 * (m + 160) ** 2
+    assert eora.eora_solve_workspace_bytes(eora.eora_solve_config(d, k, n, r, 0, 0)) <= 4 * (large + skinny) + small + 16 * 256
+
+
 def test_status_strings(lib):
     seen = set()
     for s in range(0, -8, -1):

@@ -56,3 +56,25 @@ def test_solve_falling_spectrum(decades, scale):
     opt, got = sol.layer_loss(ref["dW"], ref["B"], ref["A"], x), sol.layer_loss(ref["dW"], b, a, x)
     assert got <= opt * (1 + LOSS_RTOL), (got, opt)
     assert np.allclose(s, ref["sigma"], rtol=SIGMA_RTOL)
+
+
+@pytest.mark.parametrize("d,k,n,r", [(130, 1500, 200, 20), (1500, 130, 200, 20), (256, 512, 1000, 64)])
+def test_solve_needs_no_more_than_the_reported_workspace(d, k, n, r):
+    """Solve and loss check in a workspace of exactly the reported size, with guard bytes behind it."""
+    import torch
+    import paper_2410_21271_b200 as eora
+    w, w_hat, x = gen.make_solve_case(34, d, k, n)
+    cfg = eora.eora_solve_config(d, k, n, r, 0, 0)
+    size = eora.eora_solve_workspace_bytes(cfg)
+    ws = torch.full((size + 65536,), 0xA5, dtype=torch.uint8, device="cuda:0")
+    tw, th, tx = (torch.from_numpy(v).to("cuda:0") for v in (w, w_hat, x))
+    b, a, s = torch.empty((d, r), device="cuda:0"), torch.empty((r, k), device="cuda:0"), torch.empty(r, device="cuda:0")
+    loss = torch.zeros(1, dtype=torch.float64, device="cuda:0")
+    eora.eora_solve(cfg, tw, th, tx, b, a, s, ws[:size])
+    eora.eora_solve_loss(cfg, tw, th, tx, b, a, loss, ws[:size])
+    torch.cuda.synchronize()
+    assert bool((ws[size:] == 0xA5).all())
+    ref = sol.solve(w, w_hat, x, r)
+    opt = sol.layer_loss(ref["dW"], ref["B"], ref["A"], x)
+    assert abs(float(loss.item()) ** 0.5 - opt) <= opt * LOSS_RTOL
+    assert eora.eora_solve(cfg, tw, th, tx, b, a, s, ws[:size - 1], check=False) == eora.EORA_ERR_BAD_SHAPE
