@@ -714,6 +714,11 @@ bool mid_supported(const Handle* h, int m) {
   return make_plan(h, m < kMaxPass ? m : kMaxPass, pl);
 }
 
+int mid_grid(const Handle* h, int m) {
+  Plan pl;
+  return make_plan(h, m < kMaxPass ? m : kMaxPass, pl) ? pl.grid : 0;
+}
+
 int mid_launch_count(const Handle*, int m) { return (m + kMaxPass - 1) / kMaxPass; }
 
 // x16: fp16 activations (device).

@@ -87,6 +87,9 @@ int pick_path(const Handle* h, int m) {
   return EORA_PATH_GENERIC;
 }
 
+// Several adapters: which kernel serves m tokens (of those in reach of the decode family).  The one for 9 to 32 tokens reads X by TMA as fp16.
+bool multi_takes_mid(const Handle* h, int m) { return h->multi && h->cfg.x_dtype == EORA_X_F16 && mid_supported(h, m); }
+
 }  // namespace
 
 extern "C" {
@@ -438,7 +441,7 @@ int eora_linear_forward_multi(eora_linear_t obj, const void* x, int32_t m, const
   if (!on_handle_device(h)) return EORA_ERR_UNSUPPORTED;
   if (!decode_supported(h, m)) return EORA_ERR_UNSUPPORTED;
   void* ys[1] = {y};
-  if (h->cfg.x_dtype == EORA_X_F16 && mid_supported(h, m))
+  if (multi_takes_mid(h, m))
     return launch_mid_forward(h, x, m, ys, reinterpret_cast<cudaStream_t>(stream), adapter_ids) == cudaSuccess ? EORA_OK : EORA_ERR_CUDA;
   return launch_decode_forward(h, x, m, ys, reinterpret_cast<cudaStream_t>(stream), adapter_ids) == cudaSuccess ? EORA_OK : EORA_ERR_CUDA;
 }
@@ -561,6 +564,7 @@ int eora_linear_path(eora_linear_t obj, int32_t m) {
 int eora_linear_launches(eora_linear_t obj, int32_t m) {
   int p = eora_linear_path(obj, m);
   if (p < 0) return p;
+  if (multi_takes_mid(&obj->h, m)) return mid_launch_count(&obj->h, m);
   if (p == EORA_PATH_DECODE) return decode_tc_supported(&obj->h, m) ? decode_tc_launch_count(&obj->h, m) : decode_launch_count(&obj->h, m);
   if (p == EORA_PATH_PREFILL) return prefill_launch_count(&obj->h, m);
   return generic_launch_count(&obj->h);
@@ -663,6 +667,7 @@ int eora_linear_decode_grid(eora_linear_t obj, int32_t m) {
   if (m < 1 || m > 64) return EORA_ERR_BAD_SHAPE;
   if (pick_path(&obj->h, m) != EORA_PATH_DECODE) return 0;
   if (decode_tc_supported(&obj->h, m)) return decode_tc_grid(&obj->h);
+  if (multi_takes_mid(&obj->h, m)) return mid_grid(&obj->h, m);
   return decode_grid(&obj->h, m);
 }
 

@@ -88,3 +88,18 @@ def test_several_adapters_are_as_exact_at_every_number_of_tokens(w, ab, K, N, r,
         rel = orc.parity_errors(y.cpu().numpy().astype(np.float64), ref[:m])[0]
         assert rel <= 2.0 ** -18, (m, rel)
     L.close()
+
+
+@pytest.mark.parametrize("xd", ["f16", "bf16"])
+def test_launches_of_several_adapters(xd):
+    """eora_linear_launches and eora_linear_decode_grid follow the rule that a multi-adapter forward is dispatched by."""
+    K, N, r = 512, 96, 64
+    wf, _, _ = make_case(94, K, N, 0)
+    L = eora.MultiAdapterLayer(wf, adapters_for(K, N, r, "f16", 2, 95), max_m=40, x_dtype=xd)
+    for m in (1, 8, 9, 16, 17, 24, 32, 33, 40):
+        one = xd == "f16" and 9 <= m <= 32
+        assert eora.eora_linear_launches(L.handle, m) == (1 if one else (m + 7) // 8), m
+        grid = eora.eora_linear_decode_grid(L.handle, m)
+        # three pairs of row tiles: a cluster of two each, beside the CTAs that hold A; the kernel for eight tokens has one per row tile
+        assert grid > 0 and (grid != eora.eora_linear_decode_grid(L.handle, 8)) == one, (m, grid)
+    L.close()
