@@ -467,10 +467,11 @@ __device__ __forceinline__ Span t_span(const DecodeArgs& p, uint32_t tile, uint3
 // CTAs of 512 threads an SM has 64 registers a thread, and a spill goes to L2 (shared memory takes nearly all of the L1).
 //
 // The product with B: unit u = (row tile u >> b_log, every (1 << b_log)-th of its pairs in the chunk of t, from u's low bits on);
-// units go round the warps.  bar, parity: the barrier of the warp's (empty) ring that a blob of B arrives at.
+// units go round the warps.  bar, parity: the barrier of the warp's (empty) ring that a blob of B arrives at.  ok: false in a warp whose wait
+// ran out, which asks for nothing more.
 template <int ABF, bool SZ2, int kWarps>
 __device__ __forceinline__ void finish(const DecodeArgs& p, uint8_t* smem, uint32_t ring, uint32_t bar, uint32_t parity, uint32_t t0, uint32_t nT,
-                                       uint32_t rank, uint32_t n, uint32_t inv, uint32_t launch, unsigned long long* tr) {
+                                       uint32_t rank, uint32_t n, uint32_t inv, uint32_t launch, bool ok, unsigned long long* tr) {
   constexpr bool ab = ABF != FMT_NONE;
   constexpr uint32_t blob_b = blob_bytes(ABF, SZ2 ? 1 : 0);
   const uint32_t OT = 16u * p.m;
@@ -493,7 +494,7 @@ __device__ __forceinline__ void finish(const DecodeArgs& p, uint8_t* smem, uint3
   TWords tw = {0ull, 0ull};
   if constexpr (ab) {
     if (p.sub_pairs && nf) { c0 = (uint32_t)sub_of(p, first_tile) * p.sub_pairs; c_end = (uint32_t)(sub_of(p, first_tile + nf - 1) + 1) * p.sub_pairs; }
-    if (warp < (int)(nf << p.b_log)) {
+    if (ok && warp < (int)(nf << p.b_log)) {
       const uint32_t tile = first_tile + (warp >> p.b_log);
       const Span s = t_span(p, tile, c0, c0 + p.t_chunk);
       const uint32_t q = s.a + (warp & ((1u << p.b_log) - 1));
@@ -564,11 +565,11 @@ __device__ __forceinline__ void finish(const DecodeArgs& p, uint8_t* smem, uint3
         const Span s = t_span(p, tile, c0, c0 + p.t_chunk);
         float acc[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll 1
-        for (uint32_t q = s.a + (u & ((1u << p.b_log) - 1)), k = 0; q < s.b; q += 1u << p.b_log, ++k) {
+        for (uint32_t q = s.a + (u & ((1u << p.b_log) - 1)), k = 0; ok && q < s.b; q += 1u << p.b_log, ++k) {
           if (!first || u != (uint32_t)warp || k) ask_b(tile, q - s.base);
-          if (!mbar_try_wait_a(bar, parity)) mbar_wait_lane(bar, parity, p.dev_status);
+          ok = __all_sync(0xffffffffu, mbar_try_wait_a(bar, parity) || mbar_wait_lane(bar, parity, p.dev_status));
+          if (!ok) { mbar_drain_warp(bar, parity, lane); break; }
           parity ^= 1u;
-          __syncwarp();
           // columns past the tokens repeat the last one; their sums are not stored
           product_exact<ABF, SZ2, true>(ring, lane, th + min((uint32_t)lane >> 2, (uint32_t)p.m - 1) * pitch + (lane & 3) * 16 + (q - c0) * 256, p.m * pitch, 0u, acc);
           __syncwarp();
@@ -726,7 +727,7 @@ __global__ void __launch_bounds__(32 << warp_log(MODE), MODE == 1 ? 2 : 1) k_dec
       float* xscale = xsum + 2 * p.chunk * kMaxTok;
       if (c > 0) {
         open_run(c, n);
-        fill(n);
+        if (ok) fill(n); else left = 0;
       }
       if constexpr (MODE == 1) stage_x_i8<WF, kWarps>(smem_u32(xs), p.x, bf16, pr0 + c, n, warp, lane);
       else stage_x_f16<WF, kWarps>(xs, pitch, xsum, xscale, p.x, bf16, p.m, p.d_in, pr0 + c, n);
@@ -757,11 +758,10 @@ __global__ void __launch_bounds__(32 << warp_log(MODE), MODE == 1 ? 2 : 1) k_dec
       while (left > 0) {
         uint32_t cnt = min(p.slot_blobs, left);
         if (!whole) cnt = min(cnt, n - pr);
-        if (ok && !mbar_try_wait_a(ring.bar, ring.parity) && !mbar_wait_lane(ring.bar, ring.parity, p.dev_status)) {
-          ok = false;                              // gave up: nothing more is asked for, and what is in flight must land first
-          l_left = 0;
+        if (!__all_sync(0xffffffffu, mbar_try_wait_a(ring.bar, ring.parity) || mbar_wait_lane(ring.bar, ring.parity, p.dev_status))) {
+          ok = false;                              // gave up: nothing more is asked for (and the ring stays where it is, to say what is in flight)
+          break;
         }
-        __syncwarp();
         uint32_t src = ring.base + ring.so;
         left -= cnt;
         // NB blobs of one row tile at once (independent chains hide one another's latency), one at a time around its end
@@ -808,17 +808,17 @@ __global__ void __launch_bounds__(32 << warp_log(MODE), MODE == 1 ? 2 : 1) k_dec
         }
       }
     }
-    if (!__all_sync(0xffffffffu, ok)) {
-      for (uint32_t i = 0; i < p.slots; ++i) mbar_drain_warp(reinterpret_cast<uint64_t*>(smem + p.off_bar) + warp * kMaxSlots + i, ring.bars + 8 * i < ring.bar ? ring.parity ^ 1u : ring.parity, lane);
+    if (!ok) {                                     // what is in flight must land before its memory is used for anything else
+      for (uint32_t i = 0; i < p.slots; ++i) mbar_drain_warp(ring.bars + 8 * i, ring.bars + 8 * i < ring.bar ? ring.parity ^ 1u : ring.parity, lane);
     }
     switch (p.a_fmt) {
-      case FMT_F16: finish<FMT_F16, false, kWarps>(p, smem, ring.base, ring.bar, ring.parity, t0, nT, rank, n, inv, launch, tr); break;
-      case FMT_Q8: finish<FMT_Q8, false, kWarps>(p, smem, ring.base, ring.bar, ring.parity, t0, nT, rank, n, inv, launch, tr); break;
-      case FMT_Q4: if (p.b_sz2) finish<FMT_Q4, true, kWarps>(p, smem, ring.base, ring.bar, ring.parity, t0, nT, rank, n, inv, launch, tr);
-                   else finish<FMT_Q4, false, kWarps>(p, smem, ring.base, ring.bar, ring.parity, t0, nT, rank, n, inv, launch, tr); break;
-      case FMT_Q3: if (p.b_sz2) finish<FMT_Q3, true, kWarps>(p, smem, ring.base, ring.bar, ring.parity, t0, nT, rank, n, inv, launch, tr);
-                   else finish<FMT_Q3, false, kWarps>(p, smem, ring.base, ring.bar, ring.parity, t0, nT, rank, n, inv, launch, tr); break;
-      default: finish<FMT_NONE, false, kWarps>(p, smem, ring.base, ring.bar, ring.parity, t0, nT, rank, n, inv, launch, tr); break;
+      case FMT_F16: finish<FMT_F16, false, kWarps>(p, smem, ring.base, ring.bar, ring.parity, t0, nT, rank, n, inv, launch, ok, tr); break;
+      case FMT_Q8: finish<FMT_Q8, false, kWarps>(p, smem, ring.base, ring.bar, ring.parity, t0, nT, rank, n, inv, launch, ok, tr); break;
+      case FMT_Q4: if (p.b_sz2) finish<FMT_Q4, true, kWarps>(p, smem, ring.base, ring.bar, ring.parity, t0, nT, rank, n, inv, launch, ok, tr);
+                   else finish<FMT_Q4, false, kWarps>(p, smem, ring.base, ring.bar, ring.parity, t0, nT, rank, n, inv, launch, ok, tr); break;
+      case FMT_Q3: if (p.b_sz2) finish<FMT_Q3, true, kWarps>(p, smem, ring.base, ring.bar, ring.parity, t0, nT, rank, n, inv, launch, ok, tr);
+                   else finish<FMT_Q3, false, kWarps>(p, smem, ring.base, ring.bar, ring.parity, t0, nT, rank, n, inv, launch, ok, tr); break;
+      default: finish<FMT_NONE, false, kWarps>(p, smem, ring.base, ring.bar, ring.parity, t0, nT, rank, n, inv, launch, ok, tr); break;
     }
   }
   __syncthreads();                                 // every thread of the CTA has read the launch counter

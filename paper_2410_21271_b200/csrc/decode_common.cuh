@@ -124,10 +124,10 @@ __device__ __forceinline__ bool mbar_wait_warp_fast(uint64_t* bar, uint32_t pari
 
 // Wait, for at most two milliseconds and without touching the status word, for a bulk copy that may still be in flight:
 // used by a warp that has already given up and only has to let its copies land before it leaves.
-__device__ __forceinline__ void mbar_drain_warp(uint64_t* bar, uint32_t parity, int lane) {
+__device__ __forceinline__ void mbar_drain_warp(uint32_t bar, uint32_t parity, int lane) {
   if (lane == 0) {
     const unsigned long long t0 = globaltimer_ns();
-    while (!mbar_try_wait(bar, parity) && globaltimer_ns() - t0 < 2000000ull) __nanosleep(200);
+    while (!mbar_try_wait_a(bar, parity) && globaltimer_ns() - t0 < 2000000ull) __nanosleep(200);
   }
   __syncwarp();
 }

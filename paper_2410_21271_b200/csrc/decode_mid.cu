@@ -379,8 +379,9 @@ __global__ void __launch_bounds__(kThreads, 1) k_mid(const __grid_constant__ CUt
       s += wpt;
       if (s >= xslots) { s = j; par ^= 1u; }
     }
-    if (!ok) {                                     // gave up: this warp's copies in flight must land first
-      for (uint32_t i = 0; i < slots; ++i) mbar_drain_warp(bars_s + warp * kMaxSlots + i, ring.bars + 8 * i < ring.bar ? ring.parity ^ 1u : ring.parity, lane);
+    if (!ok) {                                     // gave up: what is in flight for this warp must land first, weights and the slots of X that it reads
+      for (uint32_t i = 0; i < slots; ++i) mbar_drain_warp(ring.bars + 8 * i, ring.bars + 8 * i < ring.bar ? ring.parity ^ 1u : ring.parity, lane);
+      for (uint32_t i = j; i < xslots; i += wpt) mbar_drain_warp(xfull + 8 * i, i < s ? par ^ 1u : par, lane);
     }
   }
 
@@ -463,11 +464,15 @@ __global__ void __launch_bounds__(kThreads, 1) k_mid(const __grid_constant__ CUt
       __syncthreads();
       if (active) {
 #pragma unroll 1
-        for (; h < h_end; h += wpt, asked = false) {
+        for (; ok && h < h_end; h += wpt, asked = false) {      // (a warp that gave up asks for nothing more)
           if (!asked) ask_b(h);
-          if (ok && !mbar_try_wait_a(ring.bar, ring.parity) && !mbar_wait_lane(ring.bar, ring.parity, p.dev_status)) ok = false;
+          if (!mbar_try_wait_a(ring.bar, ring.parity) && !mbar_wait_lane(ring.bar, ring.parity, p.dev_status)) ok = false;
+          if (!__all_sync(0xffffffffu, ok)) {
+            ok = false;
+            mbar_drain_warp(ring.bar, ring.parity, lane);
+            break;
+          }
           ring.parity ^= 1u;
-          if (!__all_sync(0xffffffffu, ok)) { ok = false; break; }
           // (columns of tokens past m hold whatever was there: their sums are not read)
           product_b<NT, EXACT>(p.a_fmt, ring.base, lane, xs + h * kTHalf + (lane >> 2) * 64 + (lane & 3) * 16, acc);
           __syncwarp();
