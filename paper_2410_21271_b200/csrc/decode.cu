@@ -429,6 +429,20 @@ __device__ __forceinline__ void run_a(const DecodeArgs& p, float* red, int warp,
   if (tr && lane == 0) tr[2] = globaltimer_ns();
 }
 
+// One token: an SM has room for two CTAs, one of this launch and one of the launch behind it.  A CTA that holds A is done long before the
+// others.  If it left before the launch behind had been placed (calls that are enqueued one by one arrive during the launch in front), that launch
+// would put two of its CTAs on this SM and none on another, would take as long as those two, and hand the imbalance on: gate|up at one token 22
+// us instead of 15, four blocks 248 us enqueued against 178 in a graph.  So the CTA keeps its place until a launch has entered after its own, or the
+// first of the others is about to store its sums, or for kHoldNs (with many streams such CTAs could otherwise fill the chip).  Only timing
+// depends on it.  Kept always until the others' end, four blocks in a graph took 183 us instead of 178: the launch after next is placed later.
+__device__ unsigned long long g_last_entry;        // globaltimer when the last one-token launch on this device entered
+constexpr unsigned long long kHoldNs = 30000ull, kEntrySpreadNs = 1000ull;      // (CTAs of one launch enter within 0.6 us on a free chip)
+__device__ __forceinline__ void hold_place(const unsigned long long* launches, unsigned long long entry) {
+  const unsigned long long t0 = globaltimer_ns();
+  while (ld_volatile_u64(&g_last_entry) <= entry + kEntrySpreadNs && (ld_volatile_u64(launches) & ((1ull << kLaunchShift) - 1)) == 0 &&
+         globaltimer_ns() - t0 < kHoldNs) __nanosleep(100);
+}
+
 // ---- after the backbone: + t . B, the partner's sums, Y ---------------------------------------------------------------
 __device__ __forceinline__ int sub_of(const DecodeArgs& p, uint32_t tile) {
   if (p.n_sub == 1) return 0;
@@ -593,6 +607,7 @@ __device__ __forceinline__ void finish(const DecodeArgs& p, uint8_t* smem, uint3
   }
   if (p.ks == 2) cluster_wait();
   __syncthreads();
+  if (threadIdx.x == 0) count_launch(p.launches);  // (every thread of the CTA has read the counter)
   for (uint32_t u = hw; u < nf << p.m_log; u += 2 * kWarps) {
     const uint32_t f = u >> p.m_log, tok = u & ((1u << p.m_log) - 1), i = tok * 16 + row;
     if (tok >= (uint32_t)p.m) continue;
@@ -626,6 +641,11 @@ __global__ void __launch_bounds__(32 << warp_log(MODE), MODE == 1 ? 2 : 1) k_dec
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   asm volatile("griddepcontrol.launch_dependents;");
   touch_args(p);
+  unsigned long long entry = 0;
+  if (MODE == 1 && threadIdx.x == 0) {
+    entry = globaltimer_ns();
+    if (blockIdx.x == 0) asm volatile("st.volatile.global.u64 [%0], %1;" ::"l"(&g_last_entry), "l"(entry) : "memory");
+  }
   unsigned long long* tr = p.trace ? p.trace + (size_t)(blockIdx.x * 16 + warp) * 4 : nullptr;
   if (tr && lane == 0) tr[0] = globaltimer_ns();
 
@@ -637,6 +657,11 @@ __global__ void __launch_bounds__(32 << warp_log(MODE), MODE == 1 ? 2 : 1) k_dec
       case FMT_Q4: if (p.a_sz2) run_a<FMT_Q4, true, kWarps>(p, red, warp, lane, tr); else run_a<FMT_Q4, false, kWarps>(p, red, warp, lane, tr); break;
       case FMT_Q3: if (p.a_sz2) run_a<FMT_Q3, true, kWarps>(p, red, warp, lane, tr); else run_a<FMT_Q3, false, kWarps>(p, red, warp, lane, tr); break;
       default: break;
+    }
+    __syncthreads();                               // every thread of the CTA has read the launch counter
+    if (threadIdx.x == 0) {
+      if constexpr (MODE == 1) hold_place(p.launches, entry);
+      count_launch(p.launches);
     }
   } else {
     constexpr uint32_t blob_b = blob_bytes(WF, SZ2 ? 1 : 0);
@@ -821,8 +846,6 @@ __global__ void __launch_bounds__(32 << warp_log(MODE), MODE == 1 ? 2 : 1) k_dec
       default: finish<FMT_NONE, false, kWarps>(p, smem, ring.base, ring.bar, ring.parity, t0, nT, rank, n, inv, launch, ok, tr); break;
     }
   }
-  __syncthreads();                                 // every thread of the CTA has read the launch counter
-  if (threadIdx.x == 0) count_launch(p.launches);
   if (tr && lane == 0) tr[3] = globaltimer_ns();
 }
 

@@ -46,3 +46,20 @@ def test_nine_to_32_tokens_record_nothing():
     L = eora.Layer(wf, af, bf, max_m=M)
     assert bool((traced(L, gen.make_x(106, M, K), 0) == GUARD).all())
     L.close()
+
+
+def test_one_token_ctas_of_a_keep_their_place():
+    """The CTAs that hold A are done long before the others and keep their places until a launch behind has entered or the others are about
+    to store, so that a late launch finds one place per SM.  Alone on the chip: CTA 0 (which holds A) leaves after the last CTA's
+    products with the backbone."""
+    import torch
+    K, N, r = 14336, 4096, 128
+    wf, af, bf = make_case(107, K, N, r, w="q3")
+    L = eora.Layer(wf, af, bf, max_m=1)
+    x = gen.make_x(108, 1, K)
+    grid = eora.eora_linear_decode_grid(L.handle, 1)
+    for _ in range(3):
+        t = traced(L, x, 64 * grid).view(grid, 16, 4)
+        torch.cuda.synchronize()
+        assert int(t[0, 0, 3]) >= int(t[grid - 1, 0, 2])
+    L.close()
