@@ -632,8 +632,11 @@ __device__ __forceinline__ void finish(const DecodeArgs& p, uint8_t* smem, uint3
 // Blobs that a warp multiplies at once.
 __host__ __device__ constexpr uint32_t fast_blobs(int fmt, int mode) { return mode == 1 ? 4 : fmt == FMT_Q4 || fmt == FMT_Q3 ? 2 : 1; }
 
+// 120 registers a thread, not 128: two CTAs of the one-token form (one of the larger form) then leave an SM 4096 registers, enough for a CTA
+// of the staging kernel of the host-buffer calls.  With all registers taken, the SMs that held such a CTA had no room for the launch behind it,
+// which put its last CTAs in pairs on other SMs (see hold_place): four 3-bit blocks of host-buffer calls in a graph 264 us, so 214; enqueued 358 and 313.
 template <int WF, int MODE, bool SZ2>
-__global__ void __launch_bounds__(32 << warp_log(MODE), MODE == 1 ? 2 : 1) k_decode(const __grid_constant__ DecodeArgs p) {
+__global__ void __maxnreg__(120) k_decode(const __grid_constant__ DecodeArgs p) {
   constexpr int kWarpLog = warp_log(MODE), kWarps = 1 << kWarpLog;
   extern __shared__ __align__(128) uint8_t smem[];
   __shared__ __align__(256) uint32_t lut_s[16];

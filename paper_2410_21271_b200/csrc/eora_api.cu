@@ -479,7 +479,9 @@ static void* mapped_alias(void* host, int32_t m) {
 // Small activations in mapped page-locked host memory are fetched by a kernel instead of the copy engine: a copy node
 // between two launches costs the stream several microseconds (the engine's start and completion, and no overlap with
 // the launches around it), a programmatic dependent launch that reads 8-28 KB over the link about two.
-__global__ void k_stage_in(const uint4* __restrict__ src, uint4* __restrict__ dst, int64_t n16) {
+// 32 registers x 128 threads are what the decode kernels leave of an SM (see k_decode), so that it never takes the place of one of their CTAs.
+constexpr int kStageThreads = 128;
+__global__ void __launch_bounds__(kStageThreads, 16) k_stage_in(const uint4* __restrict__ src, uint4* __restrict__ dst, int64_t n16) {
   asm volatile("griddepcontrol.launch_dependents;");
   asm volatile("griddepcontrol.wait;" ::: "memory");          // the staging buffer may still be read by the launch in front
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n16; i += (int64_t)gridDim.x * blockDim.x) dst[i] = src[i];
@@ -487,12 +489,18 @@ __global__ void k_stage_in(const uint4* __restrict__ src, uint4* __restrict__ ds
 static int stage_in(Handle* h, const void* x_host, size_t bytes, int32_t m, cudaStream_t s) {
   void* alias = (bytes % 16 == 0 && aligned16(x_host)) ? mapped_alias(const_cast<void*>(x_host), m) : nullptr;
   if (!alias) return cudaMemcpyAsync(h->x_stage, x_host, bytes, cudaMemcpyHostToDevice, s) == cudaSuccess ? EORA_OK : EORA_ERR_CUDA;
+  // An SM cannot change its division into L1 and shared memory while CTAs are on it: the decode kernels' is asked for.
+  static bool carved[64] = {};
+  if (h->device >= 0 && h->device < 64 && !carved[h->device]) {
+    if (cudaFuncSetAttribute(k_stage_in, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared) != cudaSuccess) return EORA_ERR_CUDA;
+    carved[h->device] = true;
+  }
   const int64_t n16 = (int64_t)(bytes / 16);
-  int grid = (int)((n16 + 127) / 128);            // one 16-byte piece per thread: the link's latency once, not once per piece
+  int grid = (int)((n16 + kStageThreads - 1) / kStageThreads);            // one 16-byte piece per thread: the link's latency once, not once per piece
   if (grid > 128) grid = 128;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(grid < 1 ? 1 : grid);
-  cfg.blockDim = dim3(128);
+  cfg.blockDim = dim3(kStageThreads);
   cfg.stream = s;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
