@@ -41,10 +41,10 @@ __host__ __device__ constexpr int warp_log(int mode) { return mode == 1 ? 3 : 4;
 constexpr int kMaxTok = 8;                // tokens per launch (the n8 side of the mma)
 constexpr int kMaxSlices = 4;             // parts of the reduction axis that t may be sent in
 constexpr int kMaxTiles = 48;             // row tiles per cluster (what its shared memory is sized for); more: further CTAs, in waves
-constexpr int kXBytes = 58 * 1024;        // activations of a chunk: 28 pairs of eight tokens
 constexpr int kMaxSmem = 226 * 1024;
 constexpr int kHalfSmem = 112 * 1024;     // what two CTAs of an SM may use each
 constexpr int kMaxSlots = 4;
+constexpr uint32_t kRingLeast = 48 * 1024;      // bytes of weights in flight per CTA that keep HBM busy (148 x 48 KB = 7 MB, a microsecond's worth)
 constexpr int kPlaneBytes = 272;          // integer path: two byte planes of a pair (256 B), scale and two sums
 
 struct DecodeArgs {
@@ -896,10 +896,11 @@ Share make_share(uint32_t total, uint32_t n) {
   return s;
 }
 
-struct Plan { DecodeArgs a; int grid; int warps; int smem; };
+struct Plan { DecodeArgs a; int grid; int warps; int smem; uint32_t ring; };
 
-// How a launch of m (at most eight) tokens is cut up; false if its shared memory does not fit.
-bool make_plan(const Handle* h, int m, Plan& pl) {
+// How a launch of m (at most eight) tokens is cut up, with the activations in `chunks` parts and at most max_tiles row tiles per cluster;
+// false if its shared memory does not fit.
+bool cut(const Handle* h, int m, uint32_t chunks, uint32_t max_tiles, Plan& pl) {
   DecodeArgs& a = pl.a;
   a = DecodeArgs();
   const bool ab = h->cfg.rank > 0;
@@ -937,7 +938,7 @@ bool make_plan(const Handle* h, int m, Plan& pl) {
   }
   uint32_t ncl = (sms - a.n_a) / a.ks;
   if (ncl > nt) ncl = nt;
-  if ((nt + ncl - 1) / ncl > (uint32_t)kMaxTiles) ncl = (nt + kMaxTiles - 1) / kMaxTiles;
+  if ((nt + ncl - 1) / ncl > max_tiles) ncl = (nt + max_tiles - 1) / max_tiles;
   a.tiles = make_share(nt, ncl);
   auto inverse = [](uint32_t n) { return (uint32_t)((0x100000000ull + n - 1) / n); };      // 0 for n == 1
   for (int r = 0; r < 2; ++r) {
@@ -951,11 +952,8 @@ bool make_plan(const Handle* h, int m, Plan& pl) {
   const uint32_t nT = a.tiles.per + (a.tiles.rem ? 1 : 0), nF = (nT + a.ks - 1) / a.ks;
   const bool codes = h->w.fmt == FMT_Q4 || h->w.fmt == FMT_Q3;
   const uint32_t per_pair = int8 ? (uint32_t)kPlaneBytes : (uint32_t)m * 256 + (codes ? 3 * kMaxTok * 4 : 0);
-  a.chunk = a.pairs;
-  if (a.chunk * per_pair > (uint32_t)kXBytes) {
-    const uint32_t parts = (a.chunk * per_pair + kXBytes - 1) / kXBytes;
-    a.chunk = (a.pairs + parts - 1) / parts;
-  }
+  a.chunk = (a.pairs + chunks - 1) / chunks;
+  if ((uint64_t)kWarps * (nT * a.chunk) * (nT * a.chunk) >> 32) return false;      // (div_by is exact below that)
   const uint32_t t_pairs = (uint32_t)h->t_cols / 128;
   a.t_chunk = 32u / (uint32_t)m < t_pairs ? 32u / (uint32_t)m : t_pairs;
   // Shared memory: activations | barriers | rings (later blobs of B) | sums of the warps' runs | the partner's sums, and, after
@@ -974,6 +972,7 @@ bool make_plan(const Handle* h, int m, Plan& pl) {
   const uint32_t budget = int8 ? kHalfSmem : kMaxSmem;
   const uint32_t blob = (uint32_t)h->w.blob, fixed = x_b + bar_b + keep_b;
   const uint32_t room = fixed < budget ? (budget - fixed) / kWarps / blob : 0u;   // blobs per warp
+  pl.ring = room * blob * kWarps;
   if (room >= 4) { a.slot_blobs = room >= 8 ? 4 : 2; a.slots = room / a.slot_blobs < kMaxSlots ? room / a.slot_blobs : kMaxSlots; }
   else { a.slot_blobs = 1; a.slots = room < 2 ? 2 : room; }
   a.off_bar = x_b;
@@ -990,6 +989,23 @@ bool make_plan(const Handle* h, int m, Plan& pl) {
   pl.smem = (int)off;
   if (pl.smem < (int)(2 * kWarps * 16 * kMaxTok * 4)) pl.smem = (int)(2 * kWarps * 16 * kMaxTok * 4);      // the A CTAs' sums
   return pl.smem <= kMaxSmem;
+}
+
+// The fewest parts of the activations with which the rings hold kRingLeast: every further part is a barrier, a round trip to L2 and rings
+// that run empty (3-bit 14336 x 4096 at eight tokens, adapters of rank 128: three parts of 58 KB 24.2 us, one of 118 KB 19.4).  If none does (large blobs,
+// many row tiles), the one with the largest ring; if nothing fits, fewer row tiles per cluster.
+bool make_plan(const Handle* h, int m, Plan& pl) {
+  for (uint32_t max_tiles = kMaxTiles; max_tiles >= 8; max_tiles -= 8) {
+    uint32_t best = 0, best_ring = 0;
+    for (uint32_t chunks = 1; chunks <= (uint32_t)h->w.half && chunks <= 64; ++chunks) {
+      if (!cut(h, m, chunks, max_tiles, pl)) continue;
+      if (pl.ring >= kRingLeast) return true;
+      if (best == 0 || pl.ring > best_ring) { best = chunks; best_ring = pl.ring; }
+      else break;
+    }
+    if (best) return cut(h, m, best, max_tiles, pl);
+  }
+  return false;
 }
 
 }  // namespace

@@ -77,3 +77,31 @@ def test_decode_fused_layers_share_a_cta():
     for i, (wf, af, bf) in enumerate(layers):
         check_parity(ys[i].float().cpu().numpy().astype(np.float64), orc.forward(x, "f16", wf, af, bf), f"layer {i}")
     F.close()
+
+
+def test_decode_of_many_long_2to4_rows():
+    """2:4, eight tokens, a reduction axis in several parts, 48 row tiles per cluster and four pairs of t: with those, activations, sums and rings of
+    large blobs do not fit at once, and the launch is cut finer.  Every quad keeps its first two places, so that a few columns are quickly checked."""
+    import torch
+    K, N, r, M = 14848, 57344, 512, 8
+    g = torch.Generator(device="cuda:0").manual_seed(51)
+    vals = (torch.randn((N, K // 2), device="cuda:0", generator=g) * 0.02).half()
+    meta = torch.full((N, K // 32), 0x44444444, dtype=torch.int32, device="cuda:0")
+    cfg, wts = eora.eora_linear_config(), eora.eora_linear_weights()
+    cfg.d_in, cfg.d_out, cfg.rank, cfg.w_format, cfg.w_bits, cfg.w_group = K, N, r, eora.EORA_W_SPARSE24, 4, 128
+    cfg.ab_format, cfg.ab_group, cfg.x_dtype, cfg.y_dtype, cfg.max_m = eora.EORA_AB_F16, 128, eora.EORA_X_F16, eora.EORA_Y_F32, M
+    a = (torch.randn((K, r), device="cuda:0", generator=g) * 0.02).half()
+    b = (torch.randn((r, N), device="cuda:0", generator=g) * 0.02).half()
+    wts.w_codes, wts.w_zeros, wts.a, wts.b = vals.data_ptr(), meta.data_ptr(), a.data_ptr(), b.data_ptr()
+    h = eora.eora_linear_create(cfg, wts)
+    x = torch.randn((M, K), device="cuda:0", generator=g).half()
+    y = torch.empty((M, N), device="cuda:0")
+    assert eora.eora_linear_path(h, M) == eora.EORA_PATH_DECODE
+    eora.eora_linear_forward(h, x, M, y)
+    torch.cuda.synchronize()
+    assert eora.eora_linear_last_device_status(h) == 0
+    eora.eora_linear_destroy(h)
+    cols = torch.arange(0, N, 331, device="cuda:0")
+    kept = x.double().reshape(M, K // 4, 4)[:, :, :2].reshape(M, K // 2)
+    ref = kept @ vals[cols].double().T + (x.double() @ a.double()) @ b[:, cols].double()
+    check_parity(y[:, cols].double().cpu().numpy(), ref.cpu().numpy())
