@@ -526,10 +526,10 @@ __device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster
 __device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
 
 
-// Launches of a handle are numbered from 1 (the kernels of the decode family share the count).  A launch adds 2^10 in all: a
+// Launches of a handle are numbered from 1 (the kernels of the decode family share the count).  A launch adds 2^16 in all: a
 // CTA's 1, and the last CTA of the grid the rest, so that the count never reaches the next multiple before every CTA has
-// read it (a CTA adds its share after its reads, at most 1023 CTAs).
-constexpr uint32_t kLaunchShift = 10;
+// read it (a CTA adds its share after its reads, at most 65535 CTAs: 25 million outputs).
+constexpr uint32_t kLaunchShift = 16;
 __device__ __forceinline__ uint32_t launch_number(const unsigned long long* launches) {
   return (uint32_t)(ld_volatile_u64(launches) >> kLaunchShift) + 1u;
 }

@@ -79,6 +79,18 @@ def test_decode_fused_layers_share_a_cta():
     F.close()
 
 
+@pytest.mark.parametrize("M", [1, 8])
+def test_decode_of_very_many_outputs(M):
+    """400 000 outputs: more row tiles than a thousand CTAs take, in waves."""
+    K, N = 128, 400000
+    wf, _, _ = make_case(49, K, N, 0, w="q3")
+    x = gen.make_x(50, M, K)
+    L = eora.Layer(wf, None, None, max_m=M)
+    assert L.path(M) == eora.EORA_PATH_DECODE
+    check_parity(run_layer(L, x, "f16"), orc.forward(x, "f16", wf, None, None), f"M{M}")
+    L.close()
+
+
 def test_decode_of_many_long_2to4_rows():
     """2:4, eight tokens, a reduction axis in several parts, 48 row tiles per cluster and four pairs of t: with those, activations, sums and rings of
     large blobs do not fit at once, and the launch is cut finer.  Every quad keeps its first two places, so that a few columns are quickly checked."""
