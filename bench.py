@@ -492,8 +492,8 @@ FP32_PEAK_TFLOPS = 148 * 128 * 2 * 1.965e9 / 1e12
 def time_solve(device: str, d: int = 4096, k: int = 4096, n: int = 2048, r: int = 128, reps: int = 3, cpu: bool = True):
     """Extra: the offline solve (Algorithm 1 steps 1-6) of one q-shaped layer: weight 4096 x 4096, 2048 calibration
     columns, rank 128, library defaults (32 extra vectors, 24 iterations).  Flops = those of the contractions the
-    library runs (Gram matrix, the two products that form dW' dW'^T, one product per iteration plus its
-    orthonormalisation, Rayleigh-Ritz, A); the small fp64 problems are not counted."""
+    library runs, without padding: P = dW X~, the lower half of its smaller square, one product with that per iteration, the way to the d side, P^T Y,
+    Y V and dW^T U'; the factorisations and the small fp64 problems are not counted."""
     import torch
     import paper_2410_21271_b200 as eora
     w, w_hat, x = gen.make_solve_case(31, d, k, n)
@@ -508,8 +508,9 @@ def time_solve(device: str, d: int = 4096, k: int = 4096, n: int = 2048, r: int 
     torch.cuda.synchronize()
     ms = e0.elapsed_time(e1) / reps
     m, iters = r + 32, 24
-    ldm = 160 if (128 < m <= 160 and d % 32 == 0) else (m + 127) // 128 * 128      # width the library's iterates are stored with
-    flops = 2.0 * k * k * n + 2.0 * d * k * k + 2.0 * d * d * k + (iters + 1) * 2.0 * d * d * ldm + (iters + 2) * 2.0 * d * ldm * ldm + 2.0 * r * d * k
+    side, other = (n, d) if m <= n < d else (d, n)        # the library iterates with the smaller square that holds m directions
+    flops = 2.0 * d * k * n + 1.0 * side * side * other + iters * 2.0 * side * side * m + (2.0 * d * n * m if side == n else 0.0) \
+        + 2.0 * d * n * m + 2.0 * d * m * r + 2.0 * r * d * k
     loss = eora.solve_loss(tw, th, tx, b, a)
     uncompensated = float(torch.linalg.norm((tw - th).double() @ tx.double()))
     out = {"workload": f"one layer {d}x{k}, {n} calibration columns, rank {r}", "ms": ms, "layers_per_s": 1e3 / ms,
