@@ -640,7 +640,7 @@ __global__ void __maxnreg__(120) k_decode(const __grid_constant__ DecodeArgs p) 
   constexpr int kWarpLog = warp_log(MODE), kWarps = 1 << kWarpLog;
   extern __shared__ __align__(128) uint8_t smem[];
   __shared__ __align__(256) uint32_t lut_s[16];
-  __shared__ __align__(16) uint32_t zero_s[40];    // what lanes without a token read as their activations
+  __shared__ __align__(16) uint32_t zero_s[52];    // what lanes without a token read as their activations: up to 208 bytes (load_xf)
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   asm volatile("griddepcontrol.launch_dependents;");
   touch_args(p);
@@ -680,7 +680,7 @@ __global__ void __maxnreg__(120) k_decode(const __grid_constant__ DecodeArgs p) 
     if (p.ks == 2) cluster_arrive();               // (that the partner runs at all, before anything is written to it)
     uint32_t lut = 0;
     if constexpr (WF == FMT_SP24 || WF == FMT_SQ4) lut = sp24_lut(lut_s);
-    if (threadIdx.x < 40) zero_s[threadIdx.x] = 0u;
+    if (threadIdx.x < 52) zero_s[threadIdx.x] = 0u;
 
     // A warp's run of a chunk of n pairs: blobs [lo, hi) in (row tile, pair) order.  They come through the warp's own ring in
     // shared memory, one bulk copy of up to slot_blobs blobs per slot.
