@@ -493,7 +493,7 @@ class FusedLayers:
 
 class MultiAdapterLayer:
     """One backbone with several adapters; every token of a forward names the adapter it uses (-1: none).
-    max_m > 64 needs every d_out to be a multiple of 128 (the tensor-core family).  Methods only marshal arguments."""
+    max_m is at most 64.  Methods only marshal arguments."""
 
     def __init__(self, w_fmt: dict, adapters, *, max_m: int, x_dtype: str = "f16", y_dtype: str = "f16", device="cuda:0"):
         import torch

@@ -17,7 +17,8 @@
 //     grid than the ones they wait for, which themselves never wait.  The wait is bounded.
 //   * One token: eight warps of 128 registers and half of an SM's shared memory, so that the next launch's CTAs are
 //     resident and have their first weights in their rings while this one runs (programmatic dependent launch), and four
-//     blobs at once per warp.  More tokens: sixteen warps and a whole SM (the products need the issue slots).
+//     blobs at once per warp.  More tokens: sixteen warps and a whole SM, for the rings beside their activations and
+//     sums.  (The issue slots are not what asks for it: 1.35 of 4 are used at eight tokens, and the first stall is a missing instruction.)
 //     Asking for all of the next launch's weights ahead (bulk prefetches into L2) was slower, 183 against 172 us for four
 //     blocks: the activations and t, which the launch in front is waiting for, then queue behind that traffic.
 // Measured, four LLaMA3-8B blocks of four launches, fp16 adapters of rank 128: 3-bit, one token 194 -> 173 us; eight tokens

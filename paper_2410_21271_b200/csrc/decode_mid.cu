@@ -32,7 +32,7 @@ using namespace dec;
 
 // Sixteen warps of 128 registers; a seventeenth as the producer of X would leave 96 (five warps share a scheduler's registers).
 constexpr int kWarps = 16, kThreads = kWarps * 32;
-constexpr int kMaxPass = 32;              // tokens per launch
+constexpr int kMaxTokens = 32;            // tokens per launch
 constexpr int kSegPitch = 36;             // floats from one token's 32 row sums to the next (36: the four token pairs of a store hit different banks)
 constexpr int kMaxSmem = 226 * 1024;
 constexpr int kMaxSlots = 4;
@@ -59,7 +59,7 @@ struct MidArgs {
   uint32_t sub_pairs, b_np;               // as in decode.cu
   uint32_t t_chunk;                       // pairs of t in shared memory at a time
   uint32_t adp_pairs;                     // several adapters: pair p of t belongs to adapter p / adp_pairs (0: one adapter)
-  signed char adp[kMaxPass];              // adapter of every token (-1: none)
+  signed char adp[kMaxTokens];              // adapter of every token (-1: none)
   unsigned long long* t_part;             // [m][t_cols / 2] words (two columns as fp16, launch number); EXACT: [m][t_cols] words (fp32, launch number)
   unsigned long long* launches;
   int* dev_status;
@@ -712,64 +712,50 @@ bool make_plan(const Handle* h, int m, Plan& pl) {
 // the tcgen05 kernel: 12 tokens 196 against 412 us, 32 tokens 256 against 421.  Forms for 64 tokens lost: two launches 510
 // against 431 us; one with twice the accumulators 464 (the sums of 64 tokens fill the registers, and only eight pairs of X fit).
 bool mid_supported(const Handle* h, int m) {
-  if (m <= 8 || m > kMaxPass || h->sm_count < 4 || h->cfg.kernel_policy == EORA_POLICY_GENERIC) return false;
+  if (m <= 8 || m > kMaxTokens || h->sm_count < 4 || h->cfg.kernel_policy == EORA_POLICY_GENERIC) return false;
   if (h->w.fmt != FMT_Q4 && h->w.fmt != FMT_Q3 && h->w.fmt != FMT_SP24 && h->w.fmt != FMT_SQ4) return false;
   if (!encode_fn()) return false;
   Plan pl;
-  return make_plan(h, m < kMaxPass ? m : kMaxPass, pl);
+  return make_plan(h, m, pl);
 }
 
 int mid_grid(const Handle* h, int m) {
   Plan pl;
-  return make_plan(h, m < kMaxPass ? m : kMaxPass, pl) ? pl.grid : 0;
+  return make_plan(h, m, pl) ? pl.grid : 0;
 }
-
-int mid_launch_count(const Handle*, int m) { return (m + kMaxPass - 1) / kMaxPass; }
 
 // x16: fp16 activations (device).
 cudaError_t launch_mid_forward(const Handle* h, const void* x16, int m, void* const* ys, cudaStream_t st, const int32_t* adapter_ids) {
   Plan pl;
   MidArgs& a = pl.a;
+  if (!make_plan(h, m, pl)) return cudaErrorInvalidValue;
   cudaLaunchConfig_t cfg = {};
   cfg.stream = st;
+  cfg.gridDim = dim3(pl.grid);
   cfg.blockDim = dim3(kThreads);
+  cfg.dynamicSmemBytes = pl.smem;
   cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   attr[1].id = cudaLaunchAttributeClusterDimension;
-  attr[1].val.clusterDim.x = 1; attr[1].val.clusterDim.y = 1; attr[1].val.clusterDim.z = 1;
+  attr[1].val.clusterDim.x = a.ks; attr[1].val.clusterDim.y = 1; attr[1].val.clusterDim.z = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 2;
-  const size_t ybytes = h->cfg.y_dtype == EORA_Y_F32 ? 4 : 2;
-  const int passes = mid_launch_count(h, m);
-  for (int i = 0, m0 = 0; i < passes; ++i) {
-    const int mp = (m - m0 + passes - i - 1) / (passes - i);      // even passes
-    if (!make_plan(h, mp, pl)) return cudaErrorInvalidValue;
-    a.n_sub = h->n_sub;
-    for (int k = 0; k < 5; ++k) a.sub_tile0[k] = (uint32_t)(k <= h->n_sub ? h->sub_tile0[k] : h->w.nt);
-    for (int k = 0; k < h->n_sub; ++k) {
-      a.sub_dout[k] = h->sub_dout[k];
-      a.ys[k] = reinterpret_cast<uint8_t*>(ys[k]) + (size_t)m0 * h->sub_dout[k] * ybytes;
+  a.n_sub = h->n_sub;
+  for (int k = 0; k < 5; ++k) a.sub_tile0[k] = (uint32_t)(k <= h->n_sub ? h->sub_tile0[k] : h->w.nt);
+  for (int k = 0; k < h->n_sub; ++k) { a.sub_dout[k] = h->sub_dout[k]; a.ys[k] = ys[k]; }
+  a.t_part = h->t_part; a.launches = h->launches; a.dev_status = h->dev_status;
+  a.t_cols = h->t_cols; a.y_dtype = h->cfg.y_dtype; a.wait_ns = h->wait_limit_ns;
+  if (h->multi) {
+    a.adp_pairs = (uint32_t)h->r_pad / 128;
+    for (int k = 0; k < m; ++k) {
+      const int id = adapter_ids ? adapter_ids[k] : -1;
+      a.adp[k] = (signed char)(id >= 0 && id < h->n_adapters ? id : -1);
     }
-    a.t_part = h->t_part; a.launches = h->launches; a.dev_status = h->dev_status;
-    a.t_cols = h->t_cols; a.y_dtype = h->cfg.y_dtype; a.wait_ns = h->wait_limit_ns;
-    if (h->multi) {
-      a.adp_pairs = (uint32_t)h->r_pad / 128;
-      for (int k = 0; k < mp; ++k) {
-        const int id = adapter_ids ? adapter_ids[m0 + k] : -1;
-        a.adp[k] = (signed char)(id >= 0 && id < h->n_adapters ? id : -1);
-      }
-    }
-    CUtensorMap tm;
-    if (!make_map(&tm, reinterpret_cast<const uint8_t*>(x16) + (size_t)m0 * h->cfg.d_in * 2, mp, h->cfg.d_in, 8 * pl.nt)) return cudaErrorInvalidValue;
-    cfg.gridDim = dim3(pl.grid);
-    cfg.dynamicSmemBytes = pl.smem;
-    attr[1].val.clusterDim.x = a.ks;
-    cudaError_t e = launch_any(cfg, tm, a, h->w.fmt, h->w.sz2 != 0, pl.nt, h->device);
-    if (e != cudaSuccess) return e;
-    m0 += mp;
   }
-  return cudaSuccess;
+  CUtensorMap tm;
+  if (!make_map(&tm, x16, m, h->cfg.d_in, 8 * pl.nt)) return cudaErrorInvalidValue;
+  return launch_any(cfg, tm, a, h->w.fmt, h->w.sz2 != 0, pl.nt, h->device);
 }
 
 }  // namespace eora

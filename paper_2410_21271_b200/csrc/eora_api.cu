@@ -572,7 +572,7 @@ int eora_linear_path(eora_linear_t obj, int32_t m) {
 int eora_linear_launches(eora_linear_t obj, int32_t m) {
   int p = eora_linear_path(obj, m);
   if (p < 0) return p;
-  if (multi_takes_mid(&obj->h, m)) return mid_launch_count(&obj->h, m);
+  if (multi_takes_mid(&obj->h, m)) return 1;
   if (p == EORA_PATH_DECODE) return decode_tc_supported(&obj->h, m) ? decode_tc_launch_count(&obj->h, m) : decode_launch_count(&obj->h, m);
   if (p == EORA_PATH_PREFILL) return prefill_launch_count(&obj->h, m);
   return generic_launch_count(&obj->h);

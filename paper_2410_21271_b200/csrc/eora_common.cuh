@@ -246,7 +246,6 @@ cudaError_t launch_wait_selftest(const Handle* h, cudaStream_t st);
 
 // medium batches (decode_mid.cu)
 bool mid_supported(const Handle* h, int m);
-int mid_launch_count(const Handle* h, int m);
 int mid_grid(const Handle* h, int m);
 cudaError_t launch_mid_forward(const Handle* h, const void* x16, int m, void* const* ys, cudaStream_t st, const int32_t* adapter_ids = nullptr);
 

@@ -52,8 +52,8 @@ struct PrefillArgs {
   // [0, n_split) (big_x row tiles per token tile).  Without small tiles n_small = 0 and n_split = n_valid.
   int n_small, small_x, n_split, big_x;
   int nkb_w, nkb_b;  // k-blocks of each part
-  int sx, sw;        // stages of the ring (sx == sw: token tiles first, weight tiles from w_off on)
-  int w_off, w_slot; // byte offset of the weight ring (after sx token tiles of bt*128 bytes), bytes of a weight tile (rows * 128)
+  int sw;            // stages of the ring (token tiles first, weight tiles from w_off on)
+  int w_off, w_slot; // byte offset of the weight ring (after sw token tiles of bt*128 bytes), bytes of a weight tile (rows * 128)
   // Where the tiles leave SMs idle, the reduction axis of a tile is split over the ksplit CTAs of a cluster (the first one
   // also takes the K-extension; split_lo says which backbone k-blocks are whose).  The
   // partial accumulators meet in distributed shared memory: every CTA finishes every ksplit-th chunk of 32 tokens.
@@ -773,8 +773,7 @@ int fill_stages(PrefillArgs& a) {      // returns the dynamic shared memory to r
   const int stage = a.bt * 128 + a.w_slot;             // token tile + weight tile of one k-block
   a.sw = (kSmemP - 1024) / stage;
   if (a.sw > kMaxWStages) a.sw = kMaxWStages;
-  a.sx = a.sw;
-  a.w_off = a.sx * a.bt * 128;
+  a.w_off = a.sw * a.bt * 128;
   int smem = a.w_off + a.sw * a.w_slot;
   const int units = a.rows / BN_W * ((a.bt + 31) / 32);
   const int out = a.ksplit > 1 ? 65536 + (units + a.ksplit - 1) / a.ksplit * (a.ksplit - 1) * 16384 : 131072;      // the epilogue's
@@ -863,7 +862,7 @@ bool prefill_supported(const Handle* h, int m) {
 }
 
 int prefill_launch_count(const Handle* h, int m) {
-  return (mid_supported(h, m) ? mid_launch_count(h, m) : h->cfg.rank > 0 ? 2 : 1) + (h->cfg.x_dtype == EORA_X_BF16 ? 1 : 0);
+  return (mid_supported(h, m) ? 1 : h->cfg.rank > 0 ? 2 : 1) + (h->cfg.x_dtype == EORA_X_BF16 ? 1 : 0);
 }
 
 cudaError_t prefill_init(Handle* h) {
