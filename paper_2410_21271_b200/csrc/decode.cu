@@ -22,7 +22,7 @@
 //     Asking for all of the next launch's weights ahead (bulk prefetches into L2) was slower, 183 against 172 us for four
 //     blocks: the activations and t, which the launch in front is waiting for, then queue behind that traffic.
 // Measured, four LLaMA3-8B blocks of four launches, fp16 adapters of rank 128: 3-bit, one token 194 -> 173 us; eight tokens
-// 303 -> 278 us; two blocks of a 2:4 backbone, one token 143 -> 132 us (the figures before: warps that added their
+// 303 -> 259 us; two blocks of a 2:4 backbone, one token 143 -> 132 us (the figures before: warps that added their
 // partial sums of single blobs to global memory and counted tickets).
 //
 // Work of a CTA.  Its blobs (16 rows x 128 reduction elements, see eora_common.cuh) in the order (chunk of the reduction
@@ -359,8 +359,10 @@ __device__ __forceinline__ void product_exact(uint32_t blob, int lane, uint32_t 
 // ---- A: t = X . A ---------------------------------------------------------------------------------------------------
 // Unit u = (row tile of A, part of the reduction axis); its pairs go round the sixteen warps, whose sums meet in shared
 // memory; the 16 x m results leave as words (value, launch number).
+// Returns (thread 0) g_last_entry as it was when the launch in front had ended: asked for here, it costs nothing later (see hold_place).
+__device__ unsigned long long g_last_entry;        // globaltimer when the last one-token launch on this device entered
 template <int ABF, bool SZ2, int kWarps>
-__device__ __forceinline__ void run_a(const DecodeArgs& p, float* red, int warp, int lane, unsigned long long* tr) {
+__device__ __forceinline__ unsigned long long run_a(const DecodeArgs& p, float* red, int warp, int lane, unsigned long long* tr) {
   constexpr uint32_t blob_b = blob_bytes(ABF, SZ2 ? 1 : 0);
   const uint32_t units = p.a_nt * p.a_slices;
   const int g = lane >> 2, t = lane & 3;
@@ -373,6 +375,8 @@ __device__ __forceinline__ void run_a(const DecodeArgs& p, float* red, int warp,
   asm volatile("griddepcontrol.wait;" ::: "memory");
   if (tr && lane == 0) tr[1] = globaltimer_ns();
   const uint32_t launch = launch_number(p.launches);
+  unsigned long long seen = 0;
+  if (threadIdx.x == 0) seen = ld_volatile_u64(&g_last_entry);
   const uint16_t* xrow = reinterpret_cast<const uint16_t*>(p.x) + (size_t)(has ? g : 0) * p.d_in + 8 * t;
   int flip = 0;
   for (uint32_t u = blockIdx.x; u < units; u += p.n_a, flip ^= 1) {
@@ -428,6 +432,7 @@ __device__ __forceinline__ void run_a(const DecodeArgs& p, float* red, int warp,
     }
   }
   if (tr && lane == 0) tr[2] = globaltimer_ns();
+  return seen;
 }
 
 // One token: an SM has room for two CTAs, one of this launch and one of the launch behind it.  A CTA that holds A is done long before the
@@ -436,9 +441,9 @@ __device__ __forceinline__ void run_a(const DecodeArgs& p, float* red, int warp,
 // us instead of 15, four blocks 248 us enqueued against 178 in a graph.  So the CTA keeps its place until a launch has entered after its own, or the
 // first of the others is about to store its sums, or for kHoldNs (with many streams such CTAs could otherwise fill the chip).  Only timing
 // depends on it.  Kept always until the others' end, four blocks in a graph took 183 us instead of 178: the launch after next is placed later.
-__device__ unsigned long long g_last_entry;        // globaltimer when the last one-token launch on this device entered
 constexpr unsigned long long kHoldNs = 30000ull, kEntrySpreadNs = 1000ull;      // (CTAs of one launch enter within 0.6 us on a free chip)
-__device__ __forceinline__ void hold_place(const unsigned long long* launches, unsigned long long entry) {
+__device__ __forceinline__ void hold_place(const unsigned long long* launches, unsigned long long entry, unsigned long long seen) {
+  if (seen > entry + kEntrySpreadNs) return;
   const unsigned long long t0 = globaltimer_ns();
   while (ld_volatile_u64(&g_last_entry) <= entry + kEntrySpreadNs && (ld_volatile_u64(launches) & ((1ull << kLaunchShift) - 1)) == 0 &&
          globaltimer_ns() - t0 < kHoldNs) __nanosleep(100);
@@ -646,7 +651,7 @@ __global__ void __maxnreg__(120) k_decode(const __grid_constant__ DecodeArgs p) 
   asm volatile("griddepcontrol.launch_dependents;");
   touch_args(p);
   unsigned long long entry = 0;
-  if (MODE == 1 && threadIdx.x == 0) {
+  if (MODE == 1 && threadIdx.x == 0 && blockIdx.x < max(p.n_a, 1u)) {
     entry = globaltimer_ns();
     if (blockIdx.x == 0) asm volatile("st.volatile.global.u64 [%0], %1;" ::"l"(&g_last_entry), "l"(entry) : "memory");
   }
@@ -655,16 +660,17 @@ __global__ void __maxnreg__(120) k_decode(const __grid_constant__ DecodeArgs p) 
 
   if (blockIdx.x < p.n_a) {
     float* red = reinterpret_cast<float*>(smem);
+    unsigned long long seen = 0;
     switch (p.a_fmt) {
-      case FMT_F16: run_a<FMT_F16, false, kWarps>(p, red, warp, lane, tr); break;
-      case FMT_Q8: run_a<FMT_Q8, false, kWarps>(p, red, warp, lane, tr); break;
-      case FMT_Q4: if (p.a_sz2) run_a<FMT_Q4, true, kWarps>(p, red, warp, lane, tr); else run_a<FMT_Q4, false, kWarps>(p, red, warp, lane, tr); break;
-      case FMT_Q3: if (p.a_sz2) run_a<FMT_Q3, true, kWarps>(p, red, warp, lane, tr); else run_a<FMT_Q3, false, kWarps>(p, red, warp, lane, tr); break;
+      case FMT_F16: seen = run_a<FMT_F16, false, kWarps>(p, red, warp, lane, tr); break;
+      case FMT_Q8: seen = run_a<FMT_Q8, false, kWarps>(p, red, warp, lane, tr); break;
+      case FMT_Q4: if (p.a_sz2) seen = run_a<FMT_Q4, true, kWarps>(p, red, warp, lane, tr); else seen = run_a<FMT_Q4, false, kWarps>(p, red, warp, lane, tr); break;
+      case FMT_Q3: if (p.a_sz2) seen = run_a<FMT_Q3, true, kWarps>(p, red, warp, lane, tr); else seen = run_a<FMT_Q3, false, kWarps>(p, red, warp, lane, tr); break;
       default: break;
     }
     __syncthreads();                               // every thread of the CTA has read the launch counter
     if (threadIdx.x == 0) {
-      if constexpr (MODE == 1) hold_place(p.launches, entry);
+      if constexpr (MODE == 1) hold_place(p.launches, entry, seen);
       count_launch(p.launches);
     }
   } else {
