@@ -358,7 +358,12 @@ __global__ void __launch_bounds__(kThreads, 1) k_mid(const __grid_constant__ CUt
     for (uint32_t q = j; q < P; q += wpt) {
       if (ok && !mbar_try_wait_a(ring.bar, ring.parity) && !mbar_wait_lane(ring.bar, ring.parity, p.dev_status)) ok = false;
       if (ok && !mbar_try_wait_a(xfull + 8 * s, par) && !mbar_wait_lane(xfull + 8 * s, par, p.dev_status)) ok = false;
-      if (!__all_sync(0xffffffffu, ok)) { ok = false; break; }
+      if (!__all_sync(0xffffffffu, ok)) {          // gave up: what is in flight for this warp must land first, weights and the slots of X that it reads
+        ok = false;
+        for (uint32_t i = 0; i < slots; ++i) mbar_drain_warp(ring.bars + 8 * i, ring.bars + 8 * i < ring.bar ? ring.parity ^ 1u : ring.parity, lane);
+        for (uint32_t i = j; i < xslots; i += wpt) mbar_drain_warp(xfull + 8 * i, i < s ? par ^ 1u : par, lane);
+        break;
+      }
       const uint32_t src = ring.base + ring.so, x = xl + s * kXSlot;
       if (is_a) {
         product_a<NT, EXACT>(p.a_fmt, p.a_sz2, src, lane, x, acc[0]);
@@ -378,10 +383,6 @@ __global__ void __launch_bounds__(kThreads, 1) k_mid(const __grid_constant__ CUt
       ring_next(ring, slot_b);
       s += wpt;
       if (s >= xslots) { s = j; par ^= 1u; }
-    }
-    if (!ok) {                                     // gave up: what is in flight for this warp must land first, weights and the slots of X that it reads
-      for (uint32_t i = 0; i < slots; ++i) mbar_drain_warp(ring.bars + 8 * i, ring.bars + 8 * i < ring.bar ? ring.parity ^ 1u : ring.parity, lane);
-      for (uint32_t i = j; i < xslots; i += wpt) mbar_drain_warp(xfull + 8 * i, i < s ? par ^ 1u : par, lane);
     }
   }
 
