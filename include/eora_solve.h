@@ -19,8 +19,9 @@
  *
  * All pointers are DEVICE pointers to row-major fp32, 16-byte aligned, caller-owned; nothing is allocated, all work is
  * enqueued on `stream` and nothing synchronises.  `workspace` must hold eora_solve_workspace_bytes(cfg) bytes.
- * Arithmetic: fp32 products with fp32 accumulation for the large contractions, fp64 for the small (r + oversample)^2
- * problems (Gram matrices of the iterate, Cholesky factor, Jacobi eigenproblem).
+ * Arithmetic: products of fp32 accuracy for the large contractions (fp32 arithmetic, or three bf16 parts per value on the tensor
+ * cores with fp32 sums), fp64 for the small (r + oversample)^2 problems (Gram matrices of the iterate, Cholesky factor, Jacobi
+ * eigenproblem).  An infinity or NaN in the inputs, or a wait inside a kernel that ran out, shows as NaN in the results.
  *
  * Returns EORA_OK, or EORA_ERR_NULL_ARG / _BAD_SHAPE (d, k, n, rank < 1, rank + oversample > min(d, 512), workspace too
  * small) / _MISALIGNED / _CUDA (codes of eora_linear.h).

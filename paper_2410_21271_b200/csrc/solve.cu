@@ -10,14 +10,15 @@
 //       one-sided Jacobi,  U' = Y V[:, top r],  S' = sqrt(lam)
 //   6.  B' = U' S',  A = S'^{-1} U'^T dW
 //
-// Large contractions are tiled fp32 SGEMMs on the CUDA cores (fp32 because the quality of the eigenvectors near the cut
-// depends on the small differences between neighbouring eigenvalues); all matrices are padded with zeros to whole tiles, so
-// there is one form of each product.  The (r + oversample)^2 problems run in fp64.
-// Measured, 4096 x 4096 with 2048 calibration columns and rank 128: see k_sgemm_full and the kernels behind it.
+// The products are fp32 in accuracy, because the quality of the eigenvectors near the cut depends on the small differences between
+// neighbouring eigenvalues: the two large ones on the tensor cores with three bf16 numbers per value (solve_gemm.cu), those with the
+// iterates on the CUDA cores.  All matrices are padded with zeros to whole tiles, so there is one form of each product.  The
+// (r + oversample)^2 problems run in fp64.
 #include <cuda_runtime.h>
 #include <stdint.h>
 #include "../../include/eora_linear.h"
 #include "../../include/eora_solve.h"
+#include "solve_gemm.cuh"
 
 namespace {
 
@@ -94,49 +95,28 @@ __device__ __forceinline__ void ffma2(float2& d, const float2& a, const float2& 
   asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(dd) : "l"(reinterpret_cast<const unsigned long long&>(a)), "l"(reinterpret_cast<const unsigned long long&>(b)));
 }
 
-// The same product for whole tiles (M, N multiples of 128, P of 16, rows 16-byte aligned): 16-byte global loads, the
+// The same product for whole tiles, nothing transposed (M, N multiples of 128, P of 16, rows 16-byte aligned): 16-byte global loads, the
 // next k-slice fetched into registers while the current one is multiplied, 8 x 8 outputs per thread.
-// SYM: C = op(A) op(A)^T is symmetric; only the tiles on and below the diagonal are computed (grid: their number) and stored
-// to both places.
-template <bool TA, bool TB, bool SYM>
 __global__ void __launch_bounds__(256, 2) k_sgemm_full(int P, const float* __restrict__ A, int lda, const float* __restrict__ B, int ldb,
                                                     float* __restrict__ C, int ldc) {
   __shared__ __align__(16) float As[2][BKS][BM + PAD];
   __shared__ __align__(16) float Bs[2][BKS][BN + PAD];
   const int t = threadIdx.x, tx = t & 15, ty = t >> 4;
-  int by = blockIdx.y, bx = blockIdx.x;
-  if (SYM) {                                         // tile number -> (row, column <= row)
-    by = (int)((sqrtf(8.f * bx + 1.f) - 1.f) * 0.5f);
-    while ((by + 1) * (by + 2) / 2 <= bx) ++by;
-    while (by * (by + 1) / 2 > bx) --by;
-    bx -= by * (by + 1) / 2;
-  }
-  const int m0 = by * BM, n0 = bx * BN;
-  // this thread's two 16-byte pieces of each operand tile
-  // not transposed A / transposed B: tile rows (128) x 16 p: piece = (row, p4), 4 pieces per row;  else (p, col4), 32 per p
+  const int m0 = blockIdx.y * BM, n0 = blockIdx.x * BN;
+  // this thread's two 16-byte pieces of each operand tile: A 128 rows x 16 p, 4 pieces per row; B 16 p x 128 columns, 32 pieces per p
   int a_r[2], a_c[2], b_r[2], b_c[2];
 #pragma unroll
   for (int i = 0; i < 2; ++i) {
     const int e = t + 256 * i;
-    if (TA) { a_r[i] = e >> 5; a_c[i] = (e & 31) * 4; } else { a_r[i] = e >> 2; a_c[i] = (e & 3) * 4; }
-    if (TB) { b_r[i] = e >> 2; b_c[i] = (e & 3) * 4; } else { b_r[i] = e >> 5; b_c[i] = (e & 31) * 4; }
+    a_r[i] = e >> 2; a_c[i] = (e & 3) * 4;
+    b_r[i] = e >> 5; b_c[i] = (e & 31) * 4;
   }
-  auto load_a = [&](int p0, int i) -> float4 {
-    return TA ? *reinterpret_cast<const float4*>(A + (int64_t)(p0 + a_r[i]) * lda + m0 + a_c[i])
-              : *reinterpret_cast<const float4*>(A + (int64_t)(m0 + a_r[i]) * lda + p0 + a_c[i]);
-  };
-  auto load_b = [&](int p0, int i) -> float4 {
-    return TB ? *reinterpret_cast<const float4*>(B + (int64_t)(n0 + b_r[i]) * ldb + p0 + b_c[i])
-              : *reinterpret_cast<const float4*>(B + (int64_t)(p0 + b_r[i]) * ldb + n0 + b_c[i]);
-  };
+  auto load_a = [&](int p0, int i) -> float4 { return *reinterpret_cast<const float4*>(A + (int64_t)(m0 + a_r[i]) * lda + p0 + a_c[i]); };
+  auto load_b = [&](int p0, int i) -> float4 { return *reinterpret_cast<const float4*>(B + (int64_t)(p0 + b_r[i]) * ldb + n0 + b_c[i]); };
   auto store_a = [&](int buf, int i, const float4& v) {
-    if (TA) *reinterpret_cast<float4*>(&As[buf][a_r[i]][a_c[i]]) = v;
-    else { As[buf][a_c[i]][a_r[i]] = v.x; As[buf][a_c[i] + 1][a_r[i]] = v.y; As[buf][a_c[i] + 2][a_r[i]] = v.z; As[buf][a_c[i] + 3][a_r[i]] = v.w; }
+    As[buf][a_c[i]][a_r[i]] = v.x; As[buf][a_c[i] + 1][a_r[i]] = v.y; As[buf][a_c[i] + 2][a_r[i]] = v.z; As[buf][a_c[i] + 3][a_r[i]] = v.w;
   };
-  auto store_b = [&](int buf, int i, const float4& v) {
-    if (TB) { Bs[buf][b_c[i]][b_r[i]] = v.x; Bs[buf][b_c[i] + 1][b_r[i]] = v.y; Bs[buf][b_c[i] + 2][b_r[i]] = v.z; Bs[buf][b_c[i] + 3][b_r[i]] = v.w; }
-    else *reinterpret_cast<float4*>(&Bs[buf][b_r[i]][b_c[i]]) = v;
-  };
+  auto store_b = [&](int buf, int i, const float4& v) { *reinterpret_cast<float4*>(&Bs[buf][b_r[i]][b_c[i]]) = v; };
   float2 acc[8][4];
 #pragma unroll
   for (int i = 0; i < 8; ++i)
@@ -180,19 +160,6 @@ __global__ void __launch_bounds__(256, 2) k_sgemm_full(int P, const float* __res
     float* row = C + (int64_t)(m0 + (i & 3) + ty * 4 + (i & 4) * 16) * ldc + n0;
     *reinterpret_cast<float4*>(row + tx * 4) = make_float4(acc[i][0].x, acc[i][0].y, acc[i][1].x, acc[i][1].y);
     *reinterpret_cast<float4*>(row + 64 + tx * 4) = make_float4(acc[i][2].x, acc[i][2].y, acc[i][3].x, acc[i][3].y);
-  }
-  if (SYM && by != bx) {
-#pragma unroll
-    for (int j = 0; j < 8; ++j) {
-      float* row = C + (int64_t)(n0 + (j & 3) + tx * 4 + (j & 4) * 16) * ldc + m0;
-      const int q = j >> 1;
-#pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        const float4 v = (j & 1) ? make_float4(acc[4 * h][q].y, acc[4 * h + 1][q].y, acc[4 * h + 2][q].y, acc[4 * h + 3][q].y)
-                                 : make_float4(acc[4 * h][q].x, acc[4 * h + 1][q].x, acc[4 * h + 2][q].x, acc[4 * h + 3][q].x);
-        *reinterpret_cast<float4*>(row + 64 * h + ty * 4) = v;
-      }
-    }
   }
 }
 
@@ -337,7 +304,7 @@ cudaError_t sgemm(cudaStream_t st, int M, int N, int P, const float* A, int lda,
   dim3 grid((N + BN - 1) / BN, (M + BM - 1) / BM);
   const bool full = !ta && !tb && M % BM == 0 && N % BN == 0 && P % BKS == 0 && lda % 4 == 0 && ldb % 4 == 0 && ldc % 4 == 0 &&
                     ((reinterpret_cast<uintptr_t>(A) | reinterpret_cast<uintptr_t>(B) | reinterpret_cast<uintptr_t>(C)) & 15) == 0;
-  if (full) k_sgemm_full<false, false, false><<<grid, 256, 0, st>>>(P, A, lda, B, ldb, C, ldc);
+  if (full) k_sgemm_full<<<grid, 256, 0, st>>>(P, A, lda, B, ldb, C, ldc);
   else k_sgemm<<<grid, 256, 0, st>>>(M, N, P, A, lda, ta ? 1 : 0, B, ldb, tb ? 1 : 0, C, ldc);
   return cudaGetLastError();
 }
@@ -346,27 +313,6 @@ cudaError_t sgemm(cudaStream_t st, int M, int N, int P, const float* A, int lda,
 __global__ void k_sub(const float* __restrict__ a, const float* __restrict__ b, float* __restrict__ c, int64_t n) {
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) c[i] = a[i] - b[i];
 }
-// The same into a matrix padded with zeros ([rows_p][ld]); b == nullptr: a copy.
-__global__ void k_sub_pad(const float* __restrict__ a, const float* __restrict__ b, int rows, int cols, float* __restrict__ c, int rows_p, int ld) {
-  for (int r = blockIdx.x; r < rows_p; r += gridDim.x) {
-    const float* ar = a + (int64_t)r * cols;
-    const float* br = b ? b + (int64_t)r * cols : nullptr;
-    float* cr = c + (int64_t)r * ld;
-    if (cols % 4 == 0) {
-      for (int i = threadIdx.x * 4; i < ld; i += blockDim.x * 4) {
-        float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (r < rows && i < cols) {
-          v = *reinterpret_cast<const float4*>(ar + i);
-          if (br) { const float4 u = *reinterpret_cast<const float4*>(br + i); v.x -= u.x; v.y -= u.y; v.z -= u.z; v.w -= u.w; }
-        }
-        *reinterpret_cast<float4*>(cr + i) = v;
-      }
-    } else {
-      for (int i = threadIdx.x; i < ld; i += blockDim.x) cr[i] = r < rows && i < cols ? (br ? ar[i] - br[i] : ar[i]) : 0.f;
-    }
-  }
-}
-
 // A fixed start for the iteration: values in (-1, 1) from a counter hash (any full-rank start converges).  The iterate
 // is stored with a leading dimension ld >= m and rows_p >= rows rows (whole tiles); the padding is zero and stays zero.
 __global__ void k_init(float* y, int rows, int rows_p, int m, int ld) {
@@ -925,26 +871,60 @@ __global__ void __launch_bounds__(1024) k_jacobi64(double* H, int m, double* lam
   }
 }
 
-// sigma_i = sqrt(lam_i);  B'[row][i] = U[row][i] sigma_i  (U: [d][ld])
-__global__ void k_finish_b(const float* __restrict__ U, int ld, const double* __restrict__ lam, int d, int r, float* __restrict__ Bp, float* __restrict__ sigma) {
+// Sums of squares of the first r columns of V [v_rows][ld] and U [u_rows][ld], fp64: part z of the rows writes parts[z][0][r] and [z][1][r].
+constexpr int kSigmaParts = 32;
+__global__ void __launch_bounds__(256) k_colsq(const float* __restrict__ V, int v_rows, const float* __restrict__ U, int u_rows, int ld, int r, double* __restrict__ parts) {
+  __shared__ double sm[8][33];
+  const int c = threadIdx.x & 31, y = threadIdx.x >> 5, col = blockIdx.x * 32 + c;
+#pragma unroll
+  for (int w = 0; w < 2; ++w) {
+    const float* a = w ? U : V;
+    const int rows = w ? u_rows : v_rows, per = (rows + kSigmaParts - 1) / kSigmaParts, hi = min(rows, (int)(blockIdx.y + 1) * per);
+    double s = 0.0;
+    if (col < r)
+      for (int i = blockIdx.y * per + y; i < hi; i += 8) { const double v = a[(int64_t)i * ld + col]; s = fma(v, v, s); }
+    sm[y][c] = s;
+    __syncthreads();
+    if (y == 0 && col < r) {
+#pragma unroll
+      for (int i = 1; i < 8; ++i) s += sm[i][c];
+      parts[((int64_t)blockIdx.y * 2 + w) * r + col] = s;
+    }
+    __syncthreads();
+  }
+}
+// lam_i = |V_i|^2 / |U_i|^2
+__global__ void k_sigma(const double* __restrict__ parts, int r, double* __restrict__ lam) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= r) return;
+  double v = 0.0, u = 0.0;
+  for (int z = 0; z < kSigmaParts; ++z) { v += parts[(int64_t)z * 2 * r + i]; u += parts[((int64_t)z * 2 + 1) * r + i]; }
+  lam[i] = u > 0.0 ? v / u : 0.0;
+}
+// sigma_i = sqrt(lam_i);  B'[row][i] = U[row][i] sigma_i  (U: [d][ld]).  status: not zero if a product gave up; the results are then NaN.
+__global__ void k_finish_b(const float* __restrict__ U, int ld, const double* __restrict__ lam, int d, int r, float* __restrict__ Bp, float* __restrict__ sigma,
+                           const int* __restrict__ status) {
   const int64_t n = (int64_t)d * r;
+  const float bad = *status ? __int_as_float(0x7fffffff) : 0.f;
   for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < n; e += (int64_t)gridDim.x * blockDim.x) {
     const int i = (int)(e % r);
     const float s = (float)sqrt(fmax(lam[i], 0.0));
-    Bp[e] = U[e / r * ld + i] * s;
-    if (e < r) sigma[e] = (float)sqrt(fmax(lam[e], 0.0));
+    Bp[e] = U[e / r * ld + i] * s + bad;
+    if (e < r) sigma[e] = (float)sqrt(fmax(lam[e], 0.0)) + bad;
   }
 }
 // A[i][j] = T[j][i] / sigma_i  (T: [k][ld], holding dW^T U); 32 x 32 tiles through shared memory, 32 x 8 threads
-__global__ void k_finish_a(const float* __restrict__ T, int ld, const double* __restrict__ lam, int r, int k, float* __restrict__ A) {
+__global__ void k_finish_a(const float* __restrict__ T, int ld, const double* __restrict__ lam, int r, int k, float* __restrict__ A,
+                           const int* __restrict__ status) {
   __shared__ float tile[32][33];
+  const float bad = *status ? __int_as_float(0x7fffffff) : 0.f;
   const int j0 = blockIdx.x * 32, i0 = blockIdx.y * 32, x = threadIdx.x, y = threadIdx.y;
   for (int q = y; q < 32; q += 8) tile[q][x] = j0 + q < k && i0 + x < r ? T[(int64_t)(j0 + q) * ld + i0 + x] : 0.f;
   __syncthreads();
   for (int q = y; q < 32; q += 8) {
     if (i0 + q >= r || j0 + x >= k) continue;
     const double s = sqrt(fmax(lam[i0 + q], 0.0));
-    A[(int64_t)(i0 + q) * k + j0 + x] = s > 0.0 ? (float)((double)tile[x][q] / s) : 0.f;
+    A[(int64_t)(i0 + q) * k + j0 + x] = (s > 0.0 ? (float)((double)tile[x][q] / s) : 0.f) + bad;
   }
 }
 // sum of squares of a matrix, fp64, into *out (zeroed by the caller)
@@ -963,11 +943,12 @@ __global__ void k_axpy_neg(float* __restrict__ c, const float* __restrict__ a, i
 struct Plan {
   int d, k, n, r, m, iters;
   int dp, kp, np;             // d, k, n in whole 128-tiles
-  bool n_side, pad_x;         // iterate with P^T P instead of P P^T; X~ has to be copied into whole tiles
+  int kc;                     // of the reduction axis k: what is split at a time for P
+  bool n_side, pad_x;         // iterate with P^T P instead of P P^T; X~ is needed in whole tiles
   int s, sp;                  // size of the matrix that is iterated with, in whole tiles
   int w, ldm;                 // width of the skinny products' tiles, leading dimension of the iterates (a multiple of it)
   int wr, ldr;                // the same for the products with r columns
-  size_t off_dw, off_x, off_p, off_c, off_y, off_q, off_z, off_s, off_sp, off_d, off_h, off_lam, off_vf, total;
+  size_t off_dw, off_x, off_status, off_p, off_c, off_y, off_q, off_z, off_s, off_sp, off_d, off_h, off_lam, off_vf, total;
 };
 size_t up256(size_t v) { return (v + 255) & ~size_t(255); }
 int up128(int v) { return (v + 127) & ~127; }
@@ -1001,13 +982,21 @@ bool make_plan(const eora_solve_config* c, Plan& p) {
   const size_t c_el = (size_t)p.sp * p.sp, r_el = (size_t)p.d * p.k;
   p.off_dw = take((size_t)p.dp * p.kp * 4);
   p.off_x = take(p.pad_x ? (size_t)p.kp * p.np * 4 : 0);
+  p.off_status = take(4);
   p.off_p = take((size_t)p.dp * p.np * 4);                        // P = dW X~; the loss check keeps (dW - B'A) X~ here
-  p.off_c = take((c_el > r_el ? c_el : r_el) * 4);                // C; the loss check keeps dW - B'A here
+  // One region for what is not needed at the same time: dW and X~^T split, all of them or half of the reduction axis at a time (where all would take more than
+  // 32 MB); C, and P split for its square behind it; in the loss check dW - B'A.
+  p.kc = eora::split_bytes(p.dp, p.kp) + eora::split_bytes(p.np, p.kp) > (32u << 20) ? (p.kp / 128 + 1) / 2 * 128 : p.kp;
+  const size_t s_p = eora::split_bytes(p.dp, p.np);
+  size_t big = r_el * 4;
+  for (size_t v : {eora::split_bytes(p.dp, p.kc) + eora::split_bytes(p.np, p.kc), up256(c_el * 4) + s_p}) if (v > big) big = v;
+  p.off_c = take(big);
   p.off_y = take(rows * p.ldm * 4);
   p.off_q = take(rows * p.ldm * 4);
   p.off_z = take(tall * p.ldm * 4);
   p.off_s = take((size_t)p.m * p.m * 8);
-  p.off_sp = take((size_t)kGramParts * p.m * p.m * 8);
+  const size_t gram_el = (size_t)kGramParts * p.m * p.m, sig_el = (size_t)kSigmaParts * 2 * p.r;
+  p.off_sp = take((gram_el > sig_el ? gram_el : sig_el) * 8);
   p.off_d = take((size_t)((p.m + 15) / 16) * 256 * 8);
   p.off_h = take((size_t)p.m * p.m * 8);
   p.off_lam = take((size_t)(2 * p.m + 128) * 8);
@@ -1108,19 +1097,25 @@ int eora_solve(const eora_solve_config* cfg, const float* w, const float* w_hat,
   float* Vf = reinterpret_cast<float*>(ws + p.off_vf);
   const int dp = p.dp, kp = p.kp, np = p.np, sp = p.sp, ldm = p.ldm;
 
-  // step 1, and X~ in whole tiles
-  k_sub_pad<<<dp < 2368 ? dp : 2368, 256, 0, st>>>(w, w_hat, p.d, p.k, dW, dp, kp);
-  const float* x = x_tilde;
-  if (p.pad_x) {
-    float* xp = reinterpret_cast<float*>(ws + p.off_x);
-    k_sub_pad<<<kp < 2368 ? kp : 2368, 256, 0, st>>>(x_tilde, nullptr, p.k, p.n, xp, kp, np);
-    x = xp;
+  uint8_t* big = reinterpret_cast<uint8_t*>(ws + p.off_c);
+  uint8_t* behind_c = big + up256((size_t)p.sp * p.sp * 4);
+  int* status = reinterpret_cast<int*>(ws + p.off_status);
+  int device = 0, sms = 0;
+  CK(cudaGetDevice(&device));
+  CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device));
+  CK(cudaMemsetAsync(status, 0, 4, st));
+  // steps 1-4: dW, P = dW X~, and the smaller of P P^T and P^T P
+  float* xp = p.pad_x ? reinterpret_cast<float*>(ws + p.off_x) : nullptr;
+  for (int k0 = 0; k0 < kp; k0 += p.kc) {
+    const int kc = kp - k0 < p.kc ? kp - k0 : p.kc, kr = p.k - k0 < kc ? p.k - k0 : kc;      // columns of dW, without the padding
+    uint8_t* xs = big + eora::split_bytes(dp, p.kc);
+    CK(eora::split_rows(st, w + k0, w_hat + k0, p.d, kr, p.k, dp, kc, big, dW + k0, kp));
+    CK(eora::split_cols(st, x_tilde + (size_t)k0 * p.n, kr, p.n, p.n, kc, np, xs, xp ? xp + (size_t)k0 * np : nullptr));
+    CK(eora::split_gemm(st, big, xs, dp, np, kc, Pm, np, false, k0 > 0, sms, status));
   }
-  // steps 2-4: P = dW X~, and the smaller of P P^T and P^T P
-  k_sgemm_full<false, false, false><<<dim3(np / BN, dp / BM), 256, 0, st>>>(kp, dW, kp, x, np, Pm, np);
-  const int T = sp / BM;
-  if (p.n_side) k_sgemm_full<true, false, true><<<T * (T + 1) / 2, 256, 0, st>>>(dp, Pm, np, Pm, np, C, sp);
-  else k_sgemm_full<false, true, true><<<T * (T + 1) / 2, 256, 0, st>>>(np, Pm, np, Pm, np, C, sp);
+  if (p.n_side) CK(eora::split_cols(st, Pm, dp, np, np, dp, np, behind_c));
+  else CK(eora::split_rows(st, Pm, nullptr, dp, np, np, dp, np, behind_c, nullptr, 0));
+  CK(eora::split_gemm(st, behind_c, behind_c, sp, sp, p.n_side ? dp : np, C, sp, true, false, sms, status));
   // step 5: subspace iteration
   k_init<<<592, 256, 0, st>>>(Y, p.s, sp, p.m, ldm);
   CK(cudaGetLastError());
@@ -1152,10 +1147,14 @@ int eora_solve(const eora_solve_config* cfg, const float* w, const float* w_hat,
   CK(cudaMemsetAsync(Vf, 0, (size_t)ldm * ldm * 4, st));
   CK(jacobi(st, H, p.m, lam, Vf, ldm));
   CK(skinny<false>(st, p.wr, dp, ldm, Y, ldm, Vf, ldm, p.ldr, Q, ldm));       // U' = Y V[:, :r]
-  // step 6
-  k_finish_b<<<592, 256, 0, st>>>(Q, ldm, lam, p.d, p.r, b_prime, sigma);
+  // step 6.  The tensor cores' sums are 2e-7 too small (truncation), which the eigenvectors do not notice but the eigenvalues would (sigma 2e-7 off instead
+  // of 3e-8): sigma_i = |X~^T dW^T u_i| / |u_i| is taken from fp32 products on the CUDA cores.
   CK(skinny<true>(st, p.wr, kp, dp, dW, kp, Q, ldm, p.ldr, Z, ldm));          // dW^T U'
-  k_finish_a<<<dim3((p.k + 31) / 32, (p.r + 31) / 32), dim3(32, 8), 0, st>>>(Z, ldm, lam, p.r, p.k, a);
+  CK(skinny<true>(st, p.wr, np, kp, xp ? xp : x_tilde, np, Z, ldm, p.ldr, Y, ldm));
+  k_colsq<<<dim3((p.r + 31) / 32, kSigmaParts), 256, 0, st>>>(Y, np, Q, dp, ldm, p.r, Sp);
+  k_sigma<<<(p.r + 127) / 128, 128, 0, st>>>(Sp, p.r, lam);
+  k_finish_b<<<592, 256, 0, st>>>(Q, ldm, lam, p.d, p.r, b_prime, sigma, status);
+  k_finish_a<<<dim3((p.k + 31) / 32, (p.r + 31) / 32), dim3(32, 8), 0, st>>>(Z, ldm, lam, p.r, p.k, a, status);
   CK(cudaGetLastError());
   return EORA_OK;
 }

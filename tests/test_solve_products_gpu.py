@@ -1,0 +1,57 @@
+"""GPU parity of the offline solve where its tensor-core products can go wrong: both tile widths, fewer reduction elements than a chunk of the
+accumulators and a chunk with a remainder, padded sizes (X~ needed as whole tiles), iterates whose column tiles begin inside a block
+of 128, and values at the ends of the range that three bf16 parts cover.  The error has rank r plus noise a hundred times smaller, so the compensation B'A and the singular values are unique and comparable with the float64 oracle."""
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+from oracle import eora_solve_oracle as sol
+import eora_inputs as gen
+from test_solve_gpu import run_solve
+
+# fp32 accuracy of the products: 4096 terms carry at most 1e-6 relative (2-norm) into dW X~ and its square; over the gap of 100 between the
+# singular values on both sides of the cut that is far below the rounding of W - W^ itself (|W| / |dW| * 2^-24 < 1e-5).
+PRODUCT_RTOL = 1e-4
+SIGMA_RTOL = 1e-6
+
+
+@pytest.mark.parametrize("d,k,n,r", [
+    (4736, 256, 1024, 24),      # 37 x 8 tiles: the wide tile; n side
+    (128, 128, 128, 8),         # one tile, four stages
+    (300, 1100, 500, 40),       # padded everywhere; chunks of eight stages with a remainder
+    (1024, 320, 384, 100),      # iterate of 132 columns: two tiles of 96
+    (700, 640, 900, 250),       # 282 columns: three tiles of 96
+])
+def test_compensation_and_spectrum(d, k, n, r):
+    w, w_hat, x = gen.make_solve_case(41, d, k, n, kind="gap", rank_signal=r)
+    ref = sol.solve(w, w_hat, x, r)
+    b, a, s, _ = run_solve(w, w_hat, x, r)
+    want = ref["B"] @ ref["A"]
+    assert np.linalg.norm(b @ a - want) <= PRODUCT_RTOL * np.linalg.norm(want)
+    assert np.linalg.norm(s - ref["sigma"]) <= SIGMA_RTOL * np.linalg.norm(ref["sigma"])
+
+
+@pytest.mark.parametrize("scale", [2.0 ** -40, 2.0 ** 40])
+def test_scaled_activations_scale_sigma_alone(scale):
+    """Powers of two change no rounding anywhere: sigma scales with X~, B'A stays the same bit for bit."""
+    import torch
+    import paper_2410_21271_b200 as eora
+    d, k, n, r = 256, 384, 512, 32
+    w, w_hat, x = (torch.from_numpy(v).cuda() for v in gen.make_solve_case(42, d, k, n))
+    b0, a0, s0 = eora.solve(w, w_hat, x, r)
+    b1, a1, s1 = eora.solve(w, w_hat, x * scale, r)
+    torch.cuda.synchronize()
+    assert torch.equal(s0 * scale, s1)
+    assert torch.equal(b0 * scale, b1) and torch.equal(a0, a1 * scale)
+
+
+def test_not_a_number_in_not_a_number_out():
+    """One infinite activation makes every column of P that it meets infinite or NaN: nothing finite may be made up from it."""
+    import torch
+    import paper_2410_21271_b200 as eora
+    w, w_hat, x = (torch.from_numpy(v).cuda() for v in gen.make_solve_case(43, 128, 128, 256))
+    x[3, 5] = float("inf")
+    b, a, s = eora.solve(w, w_hat, x, 16)
+    torch.cuda.synchronize()
+    assert not bool(torch.isfinite(b @ a).all())
