@@ -608,7 +608,8 @@ __global__ void __launch_bounds__(256) k_trsm(const float* __restrict__ Y, const
 // meeting every column of one block is rotated against every column of the other, B disjoint pairs at a time whose latencies
 // overlap; the pairs inside a block take their turn once per sweep.  Squared norms are carried along (recomputed every
 // sweep), so a rotation needs one dot product.  The angle is computed in fp32 -- a rotation by a slightly different angle is
-// still a rotation, and the next sweep works on what it left -- its cosine in fp64.  One CTA that kept the columns in shared
+// still a rotation, and the next sweep works on what it left -- its cosine in fp64.  The last sweep is the one that finds every pair
+// orthogonal to 1e-8 before it rotates them (convergence is quadratic by then, and the results are fp32).  One CTA that kept the columns in shared
 // memory and went through it for every pair took 4.5 ms at m = 160.
 template <int B, int E>
 struct JacobiShape {
@@ -645,6 +646,7 @@ __global__ void __launch_bounds__(B == 4 ? 160 : 320, 1) k_jacobi_cl(const doubl
       }
     }
   if (t < 2) moved_s[t] = 0;
+  constexpr double kStop = 1e-16;
   int any = 0;
   auto norms = [&]() {
 #pragma unroll
@@ -661,7 +663,7 @@ __global__ void __launch_bounds__(B == 4 ? 160 : 320, 1) k_jacobi_cl(const doubl
   };
   auto rotate = [&](double (&x)[E], double (&y)[E], double& al, double& be, double ga) {
     if (ga * ga <= 1e-22 * al * be) return;          // orthogonal far beyond what the fp32 operands carry
-    any = 1;
+    if (ga * ga > kStop * al * be) any = 1;
     // both scaled by one power of two, so that fp32 neither overflows nor loses what is small
     const double zd = be - al, wd = 2.0 * ga;
     const int e_max = max(__double2hiint(zd) & 0x7ff00000, __double2hiint(wd) & 0x7ff00000);
@@ -711,18 +713,59 @@ __global__ void __launch_bounds__(B == 4 ? 160 : 320, 1) k_jacobi_cl(const doubl
           for (int b = 0; b < B; ++b) if ((b ^ k) > b) rotate(h[s][b], h[s][b ^ k], nrm[s][b], nrm[s][b ^ k], ga[s][b]);
       }
     }
+    // Meetings.  The B disjoint pairs of a round are dealt to B groups of lanes: their dot products are reduced into the groups
+    // (6 shuffles instead of 20 for B = 4), every group computes its pair's angle, all at the same time and without a branch, and
+    // keeps the squared norms of its two columns; cosines and sines are then read from the groups.  One pair after the other, each
+    // behind a branch, a round took 2.5 times as long.
+    constexpr int GL = 32 / B;                       // lanes of a group
+    const int pb = lane / GL;
+    double al = nrm[0][0], be = nrm[1][0];           // of column pb of the one block and column (pb + k) % B of the other
+#pragma unroll
+    for (int b = 1; b < B; ++b) if (pb == b) { al = nrm[0][b]; be = nrm[1][b]; }
     for (int step = 0; step < 2 * G - 1; ++step) {
 #pragma unroll
       for (int k = 0; k < B; ++k) {
         double ga[B];
 #pragma unroll
         for (int b = 0; b < B; ++b) ga[b] = dot(h[0][b], h[1][(b + k) % B]);
+        double g;
+        if constexpr (B == 4) {
+          const bool hi = lane & 16, odd = lane & 8;
+          double k0 = hi ? ga[2] : ga[0], k1 = hi ? ga[3] : ga[1];
+          k0 += __shfl_xor_sync(0xffffffffu, hi ? ga[0] : ga[2], 16);
+          k1 += __shfl_xor_sync(0xffffffffu, hi ? ga[1] : ga[3], 16);
+          g = (odd ? k1 : k0) + __shfl_xor_sync(0xffffffffu, odd ? k0 : k1, 8);
+        } else {
+          const bool hi = lane & 16;
+          g = (hi ? ga[1] : ga[0]) + __shfl_xor_sync(0xffffffffu, hi ? ga[0] : ga[1], 16);
+          g += __shfl_xor_sync(0xffffffffu, g, 8);
+        }
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1)
+        for (int o = 4; o > 0; o >>= 1) g += __shfl_xor_sync(0xffffffffu, g, o);
+        // (as in rotate above)
+        const double zd = be - al, wd = 2.0 * g;
+        const int e_max = max(__double2hiint(zd) & 0x7ff00000, __double2hiint(wd) & 0x7ff00000);
+        const bool act = g * g > 1e-22 * al * be && e_max >= 0x01000000;
+        const double unit = __hiloint2double(0x7fe00000 - e_max, 0);
+        const float z = (float)(zd * unit), w = (float)(wd * unit);
+        const float tf = act ? copysignf(w / (fabsf(z) + sqrtf(fmaf(z, z, w * w))), z >= 0.f ? w : -w) : 0.f;
+        const double tt = (double)tf, c = act ? rsqrt(fma(tt, tt, 1.0)) : 1.0, sn = c * tt;
+        if (__any_sync(0xffffffffu, act)) {
+          if (__any_sync(0xffffffffu, g * g > kStop * al * be)) any = 1;
+          const double c2 = c * c, s2 = sn * sn, cs2 = 2.0 * c * sn * g, na = c2 * al - cs2 + s2 * be, nb = s2 * al + cs2 + c2 * be;
+          al = na > 0.0 ? na : 0.0; be = nb > 0.0 ? nb : 0.0;
 #pragma unroll
-          for (int b = 0; b < B; ++b) ga[b] += __shfl_xor_sync(0xffffffffu, ga[b], o);
+          for (int b = 0; b < B; ++b) {
+            const double cb = __shfl_sync(0xffffffffu, c, b * GL), sb = __shfl_sync(0xffffffffu, sn, b * GL);
 #pragma unroll
-        for (int b = 0; b < B; ++b) rotate(h[0][b], h[1][(b + k) % B], nrm[0][b], nrm[1][(b + k) % B], ga[b]);
+            for (int e = 0; e < E; ++e) {
+              const double x = h[0][b][e], y = h[1][(b + k) % B][e];
+              h[0][b][e] = cb * x - sb * y;
+              h[1][(b + k) % B][e] = fma(sb, x, cb * y);
+            }
+          }
+        }
+        be = __shfl_sync(0xffffffffu, be, ((pb + 1) % B) * GL);
       }
       if (G == 1) break;
       // circle method: the top block of group 0 stays, the others move on by one place of the ring of blocks
@@ -740,9 +783,7 @@ __global__ void __launch_bounds__(B == 4 ? 160 : 320, 1) k_jacobi_cl(const doubl
 #pragma unroll
           for (int e = 0; e < E; ++e)
             asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(dst + (b * Sh::kElems + 32 * e) * 8), "d"(h[s][b][e]) : "memory");
-#pragma unroll
-        for (int b = 0; b < B; ++b)
-          if (lane == b) asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(dst + B * Sh::kElems * 8), "d"(nrm[s][b]) : "memory");
+        if (lane % GL == 0) asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(dst + (B * Sh::kElems + pb - lane) * 8), "d"(s ? be : al) : "memory");
       }
       cluster_sync_all();
 #pragma unroll
@@ -752,8 +793,7 @@ __global__ void __launch_bounds__(B == 4 ? 160 : 320, 1) k_jacobi_cl(const doubl
         for (int b = 0; b < B; ++b)
 #pragma unroll
           for (int e = 0; e < E; ++e) h[s][b][e] = src[b * Sh::kElems + 32 * e];
-#pragma unroll
-        for (int b = 0; b < B; ++b) nrm[s][b] = src[B * Sh::kElems + b - lane];
+        (s ? be : al) = src[B * Sh::kElems + pb - lane];
       }
     }
     // did anybody rotate?  every CTA's flag, by every warp that did
