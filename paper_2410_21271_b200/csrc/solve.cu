@@ -4,7 +4,8 @@
 //   2-4 the paper projects dW into the eigenspace of X~ X~^T, dW' = dW Q sqrt(L).  Only dW' dW'^T = P P^T with P = dW X~
 //       (d x n) is needed here.
 //   5.  top-r eigenpairs (U', S'^2) of P P^T by subspace iteration on m = r + oversample vectors:
-//         Y = C Q;  Q = orth(Y)  by Cholesky-QR (Gram matrix, factor and substitution in fp64);  repeated `iters` times.
+//         Y = C Q;  Q = orth(Y)  by Cholesky-QR (Gram matrix, factor and substitution in fp64);  repeated `iters` times, or by
+//       default fourteen times, the last ten of them with a Chebyshev filter (see eora_solve).
 //       C is the smaller of P P^T (d x d) and P^T P (n x n), whose leading eigenvectors P carries into each other.  Then a
 //       Rayleigh-Ritz step in the d-dimensional basis Y:  H = (P^T Y)^T (P^T Y)  (m x m, fp64),  H = V diag(lam) V^T by
 //       one-sided Jacobi,  U' = Y V[:, top r],  S' = sqrt(lam)
@@ -15,6 +16,7 @@
 // iterates on the CUDA cores.  All matrices are padded with zeros to whole tiles, so there is one form of each product.  The
 // (r + oversample)^2 problems run in fp64.
 #include <cuda_runtime.h>
+#include <math.h>
 #include <stdint.h>
 #include "../../include/eora_linear.h"
 #include "../../include/eora_solve.h"
@@ -168,9 +170,10 @@ __global__ void __launch_bounds__(256, 2) k_sgemm_full(int P, const float* __res
 // partial sums meet in distributed shared memory and are added in a fixed order, so the result does not depend on timing.
 // 4 x NC outputs per thread (two instructions' worth of shared-memory reads per ten of arithmetic at NC = 10; 2 x 10 was bound
 // by the reads), and enough CTAs without padding columns: 2048 x 2048 x 160 are 32 tiles, 128 CTAs.
+// shift (may be null; op(A) square): C = op(A) B - *shift B.
 template <int NC, bool TA>
 __global__ void __launch_bounds__(256) k_skinny(int P, const float* __restrict__ A, int lda, const float* __restrict__ B, int ldb,
-                                                float* __restrict__ C, int ldc) {
+                                                float* __restrict__ C, int ldc, const float* __restrict__ shift) {
   constexpr int W = 16 * NC, NP = NC / 2, RM = 64;
   constexpr int BQ = (BKS * W / 4 + 255) / 256;      // 16-byte pieces of the B slice per thread
   constexpr int kAb = 2 * BKS * (RM + PAD), kBb = 2 * BKS * (W + PAD), kSm = kAb + kBb > RM * W ? kAb + kBb : RM * W;
@@ -243,7 +246,17 @@ __global__ void __launch_bounds__(256) k_skinny(int P, const float* __restrict__
     buf ^= 1;
   }
   auto col = [&](int j) { return j / 2 < NC / 4 ? 64 * (j / 2) + tx * 4 + 2 * (j & 1) : 64 * (NC / 4) + tx * 2; };
+  const float rho = shift ? *shift : 0.f;
   if (ks == 1) {
+    if (shift) {
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int j = 0; j < NP; ++j) {
+          const float2 q = *reinterpret_cast<const float2*>(B + (int64_t)(m0 + ty * 4 + i) * ldb + n0 + col(j));
+          acc[i][j].x = fmaf(-rho, q.x, acc[i][j].x); acc[i][j].y = fmaf(-rho, q.y, acc[i][j].y);
+        }
+    }
 #pragma unroll
     for (int i = 0; i < 4; ++i)
 #pragma unroll
@@ -266,13 +279,18 @@ __global__ void __launch_bounds__(256) k_skinny(int P, const float* __restrict__
       asm volatile("ld.shared::cluster.v4.f32 {%0,%1,%2,%3}, [%4];" : "=f"(u.x), "=f"(u.y), "=f"(u.z), "=f"(u.w) : "r"(a));
       v.x += u.x; v.y += u.y; v.z += u.z; v.w += u.w;
     }
-    *reinterpret_cast<float4*>(C + (int64_t)(m0 + rank * per + e / (W / 4)) * ldc + n0 + (e % (W / 4)) * 4) = v;
+    const int row = m0 + rank * per + e / (W / 4), at = n0 + (e % (W / 4)) * 4;
+    if (shift) {
+      const float4 q = *reinterpret_cast<const float4*>(B + (int64_t)row * ldb + at);
+      v.x = fmaf(-rho, q.x, v.x); v.y = fmaf(-rho, q.y, v.y); v.z = fmaf(-rho, q.z, v.z); v.w = fmaf(-rho, q.w, v.w);
+    }
+    *reinterpret_cast<float4*>(C + (int64_t)row * ldc + at) = v;
   }
   cluster_sync_all();                                // nobody leaves while its sums are being read
 }
 
 template <int NC, bool TA>
-cudaError_t launch_skinny(cudaStream_t st, int M, int P, const float* A, int lda, const float* B, int ldb, int N, float* C, int ldc) {
+cudaError_t launch_skinny(cudaStream_t st, int M, int P, const float* A, int lda, const float* B, int ldb, int N, float* C, int ldc, const float* shift) {
   // as many CTAs per tile as there are SMs for, each with at least eight slices of P
   const int tiles = M / 64 * (N / (16 * NC));
   int ks = 4;
@@ -286,16 +304,16 @@ cudaError_t launch_skinny(cudaStream_t st, int M, int P, const float* A, int lda
   attr[0].val.clusterDim.x = ks; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, k_skinny<NC, TA>, P, A, lda, B, ldb, C, ldc);
+  return cudaLaunchKernelEx(&cfg, k_skinny<NC, TA>, P, A, lda, B, ldb, C, ldc, shift);
 }
 // N: a multiple of the width `w` (64, 96, 128 or 160) that make_plan chose.
 template <bool TA>
-cudaError_t skinny(cudaStream_t st, int w, int M, int P, const float* A, int lda, const float* B, int ldb, int N, float* C, int ldc) {
+cudaError_t skinny(cudaStream_t st, int w, int M, int P, const float* A, int lda, const float* B, int ldb, int N, float* C, int ldc, const float* shift = nullptr) {
   switch (w) {
-    case 64: return launch_skinny<4, TA>(st, M, P, A, lda, B, ldb, N, C, ldc);
-    case 96: return launch_skinny<6, TA>(st, M, P, A, lda, B, ldb, N, C, ldc);
-    case 128: return launch_skinny<8, TA>(st, M, P, A, lda, B, ldb, N, C, ldc);
-    default: return launch_skinny<10, TA>(st, M, P, A, lda, B, ldb, N, C, ldc);
+    case 64: return launch_skinny<4, TA>(st, M, P, A, lda, B, ldb, N, C, ldc, shift);
+    case 96: return launch_skinny<6, TA>(st, M, P, A, lda, B, ldb, N, C, ldc, shift);
+    case 128: return launch_skinny<8, TA>(st, M, P, A, lda, B, ldb, N, C, ldc, shift);
+    default: return launch_skinny<10, TA>(st, M, P, A, lda, B, ldb, N, C, ldc, shift);
   }
 }
 
@@ -402,6 +420,11 @@ cudaError_t gram64(cudaStream_t st, const float* A, int rows, int m, int ld, dou
   return cudaGetLastError();
 }
 
+// The power of two next to 1 / v.
+__device__ __forceinline__ float pow2_scale(double v) {
+  const int ex = min(max((__double2hiint(v) >> 20) - 1023, -120), 120);
+  return __int_as_float((127 - ex) << 23);
+}
 // 1 / sqrt(d) in fp64 from the fp32 value by Newton's method (each step doubles the digits; the argument's exponent is taken
 // out first, so every positive d works).
 __device__ __forceinline__ double rsqrt_newton(double d) {
@@ -427,7 +450,13 @@ constexpr int kCholSmem = 160;
 constexpr int kCholThreads = 512;
 __host__ __device__ constexpr int pan_pitch(int m) { return (m + 5) / 4 * 4 + 2; }      // (even, and rows of the panel on different banks)
 __host__ __device__ constexpr int chol_smem(int m) { return ((m <= kCholSmem ? m * (m | 1) : 0) + m + 16 * pan_pitch(m)) * 8 + 16; }
-__global__ void __launch_bounds__(kCholThreads) k_chol64(double* Sg, int m, double* __restrict__ Dinv) {
+//
+// f (may be null): the filter's state.  With prev the iterate went through a pair of products with (C - f->rho[0] I) and (C - f->rho[1] I), starting from
+// columns of norm 1 / f->scale, else through one with C: the diagonal of L then says where the eigenvalues of the iterate's columns are.
+// The next pair's shifts are lo and hi times the smallest of them.
+struct Filter { float rho[2]; double scale; };
+constexpr double kFilterEdge = 0.95;                 // the estimate comes from below, but not always (measured 0.8 to 1.07 of eigenvalue m after four steps)
+__global__ void __launch_bounds__(kCholThreads) k_chol64(double* Sg, int m, double* __restrict__ Dinv, Filter* f, bool prev, double lo, double hi) {
   extern __shared__ __align__(16) double sm[];
   __shared__ double dv[16][17];
   const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
@@ -535,6 +564,21 @@ __global__ void __launch_bounds__(kCholThreads) k_chol64(double* Sg, int m, doub
     }
     __syncthreads();
   }
+  if (f && warp == 0) {
+    double least_l = 1e300;
+    for (int i = lane; i < m; i += 32) least_l = fmin(least_l, S[(int64_t)i * ls + i]);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) least_l = fmin(least_l, __shfl_xor_sync(0xffffffffu, least_l, o));
+    if (lane == 0) {
+      double at = least_l;                           // (x - rho0)(x - rho1) = L f->scale
+      if (prev) {
+        const double r0 = f->rho[0], r1 = f->rho[1], half = 0.5 * (r0 - r1);
+        at = 0.5 * (r0 + r1) + sqrt(half * half + least_l * f->scale);
+      }
+      f->rho[0] = (float)(lo * kFilterEdge * at); f->rho[1] = (float)(hi * kFilterEdge * at);
+      f->scale = 1.0 / (double)pow2_scale(S[0]);
+    }
+  }
   if (in_smem)
     for (int i = warp; i < m; i += kCholThreads / 32)
       for (int j = lane; j <= i; j += 32) Sg[(int64_t)i * m + j] = S[i * ls + j];
@@ -569,8 +613,7 @@ __global__ void __launch_bounds__(256) k_trsm(const float* __restrict__ Y, const
   };
   fetch(0);
   float y = Y[row * ld + c];
-  const int ex = min(max((__double2hiint(L[0]) >> 20) - 1023, -120), 120);
-  const float scale = scaled ? __int_as_float((127 - ex) << 23) : 1.f;
+  const float scale = scaled ? pow2_scale(L[0]) : 1.f;
   for (int p = 0; p < np; ++p) {
     asm volatile("cp.async.wait_group 0;" ::: "memory");
     __syncthreads();                                 // panel p is there, and panel p - 1 has been read
@@ -981,14 +1024,15 @@ __global__ void k_axpy_neg(float* __restrict__ c, const float* __restrict__ a, i
 
 // ------------------------------------------------------------------------------------------------ workspace
 struct Plan {
-  int d, k, n, r, m, iters;
+  int d, k, n, r, m;
+  int iters;                  // plain products; 0: the filter
   int dp, kp, np;             // d, k, n in whole 128-tiles
   int kc;                     // of the reduction axis k: what is split at a time for P
   bool n_side, pad_x;         // iterate with P^T P instead of P P^T; X~ is needed in whole tiles
   int s, sp;                  // size of the matrix that is iterated with, in whole tiles
   int w, ldm;                 // width of the skinny products' tiles, leading dimension of the iterates (a multiple of it)
   int wr, ldr;                // the same for the products with r columns
-  size_t off_dw, off_x, off_status, off_p, off_c, off_y, off_q, off_z, off_s, off_sp, off_d, off_h, off_lam, off_vf, total;
+  size_t off_dw, off_x, off_status, off_filter, off_p, off_c, off_y, off_q, off_z, off_s, off_sp, off_d, off_h, off_lam, off_vf, total;
 };
 size_t up256(size_t v) { return (v + 255) & ~size_t(255); }
 int up128(int v) { return (v + 127) & ~127; }
@@ -1006,7 +1050,7 @@ bool make_plan(const eora_solve_config* c, Plan& p) {
   p.m = p.r + over;
   if (p.m > p.d) p.m = p.d;
   if (p.r > p.m || p.m > 512) return false;
-  p.iters = c->iters > 0 ? c->iters : 24;
+  p.iters = c->iters > 0 ? c->iters : 0;
   p.dp = up128(p.d); p.kp = up128(p.k); p.np = up128(p.n);
   p.pad_x = p.k % 128 || p.n % 128;
   // The smaller side (every iteration is a product with its square); it has to hold m directions.
@@ -1023,6 +1067,7 @@ bool make_plan(const eora_solve_config* c, Plan& p) {
   p.off_dw = take((size_t)p.dp * p.kp * 4);
   p.off_x = take(p.pad_x ? (size_t)p.kp * p.np * 4 : 0);
   p.off_status = take(4);
+  p.off_filter = take(sizeof(Filter));
   p.off_p = take((size_t)p.dp * p.np * 4);                        // P = dW X~; the loss check keeps (dW - B'A) X~ here
   // One region for what is not needed at the same time: dW and X~^T split, all of them or half of the reduction axis at a time (where all would take more than
   // 32 MB); C, and P split for its square behind it; in the loss check dW - B'A.
@@ -1066,11 +1111,11 @@ constexpr int kSingleSteps = 4;        // products that are orthogonalised one b
 
 // Q = orth(Y) by Cholesky-QR: Gram matrix, its factor and Q = Y L^{-T} in fp64.  Y, Q: [rows][ldm], rows a multiple of 16.
 int orthonormalise(cudaStream_t st, const Plan& p, int rows, const float* Y, float* Q, double* S, double* parts, double* D,
-                   bool scaled = false) {
+                   bool scaled = false, Filter* f = nullptr, bool prev = false, double lo = 0.0, double hi = 0.0) {
   CK(gram64<false>(st, Y, rows, p.m, p.ldm, parts, S));
   CK(allow_smem<k_chol64>(chol_smem(kCholSmem)));
   CK(allow_smem<k_trsm>(trsm_smem(512)));
-  k_chol64<<<1, kCholThreads, chol_smem(p.m), st>>>(S, p.m, D);
+  k_chol64<<<1, kCholThreads, chol_smem(p.m), st>>>(S, p.m, D, f, prev, lo, hi);
   k_trsm<<<rows / 16, 256, trsm_smem(p.m), st>>>(Y, S, D, p.m, p.ldm, Q, scaled);
   CK(cudaGetLastError());
   return EORA_OK;
@@ -1164,17 +1209,29 @@ int eora_solve(const eora_solve_config* cfg, const float* w, const float* w_hat,
   // eigenvector, which the first steps see to -- it is needed only every second product: the part of the larger eigenvectors that
   // rounding brings into a column stays in the span and is taken out with the next factor, and what lies outside the span
   // is damped by every product.  The iterate that goes through two products is scaled to norm 1 / lam_1, which keeps
-  // C C Q in the range of the products of one step.  Rank 128, 24 products: 27 -> 17 factorisations of 83 us.
-  for (int it = 0; it < p.iters;) {
-    const bool pair = it >= kSingleSteps && p.iters - it >= 2;
-    CK(skinny<true>(st, p.w, sp, sp, C, sp, Q, ldm, ldm, Y, ldm));            // Y = C Q (C is symmetric: read by columns)
+  // C C Q in the range of the products of one step.
+  //
+  // By default four single products are followed by kPairs pairs whose second factors are C - rho I with rho at the Chebyshev points of degree 2 kPairs
+  // of [0, lam_m]: what is left of an eigenvalue there is 1 / T_10(2 lam_r / lam_m - 1) of eigenvalue r's part instead of (lam_m / lam_r)^10.
+  // A pair takes a point and its mirror image, so no pair lets anything in the interval grow against what lies above it, whatever their order.  The
+  // diagonal of the factor says where lam_m is (k_chol64), each time anew.  14 products and 12 factorisations come as close as 24 and 17 of
+  // the plain iteration, or closer (error of the projector where the plain one has not converged: flat spectra 1.1e-2 -> 8e-4 and 2.1e-4 -> 3e-5).
+  const bool filter = p.iters == 0;
+  constexpr int kPairs = 5, kOrder[kPairs] = {3, 1, 4, 0, 2};
+  auto node = [&](int i) { return 0.5 + 0.5 * cos((2 * i + 1) * 3.14159265358979323846 / (4 * kPairs)); };
+  const int iters = filter ? kSingleSteps + 2 * kPairs : p.iters;
+  Filter* f = filter ? reinterpret_cast<Filter*>(ws + p.off_filter) : nullptr;
+  for (int it = 0, pairs = 0; it < iters;) {
+    const bool pair = it >= kSingleSteps && iters - it >= 2;
+    CK(skinny<true>(st, p.w, sp, sp, C, sp, Q, ldm, ldm, Y, ldm, pair && f ? f->rho : nullptr));      // Y = C Q (C is symmetric: read by columns)
     if (pair) {
-      CK(skinny<true>(st, p.w, sp, sp, C, sp, Y, ldm, ldm, Q, ldm));
+      CK(skinny<true>(st, p.w, sp, sp, C, sp, Y, ldm, ldm, Q, ldm, f ? f->rho + 1 : nullptr));
       float* y = Y; Y = Q; Q = y;
     }
     it += pair ? 2 : 1;
-    const bool next_pair = it >= kSingleSteps && p.iters - it >= 2;
-    if (int rc = orthonormalise(st, p, sp, Y, Q, S, Sp, D, next_pair)) return rc;
+    const bool next_pair = it >= kSingleSteps && iters - it >= 2;
+    const int i = next_pair && f ? kOrder[pairs++] : 0;
+    if (int rc = orthonormalise(st, p, sp, Y, Q, S, Sp, D, next_pair, next_pair ? f : nullptr, pair, node(i), node(2 * kPairs - 1 - i))) return rc;
   }
   if (p.n_side) {                                                             // to the d-dimensional side
     CK(skinny<false>(st, p.w, dp, np, Pm, np, Q, ldm, ldm, Y, ldm));
