@@ -12,8 +12,8 @@
 //   6.  B' = U' S',  A = S'^{-1} U'^T dW
 //
 // The products are fp32 in accuracy, because the quality of the eigenvectors near the cut depends on the small differences between
-// neighbouring eigenvalues: the two large ones on the tensor cores with three bf16 numbers per value (solve_gemm.cu), those with the
-// iterates on the CUDA cores.  All matrices are padded with zeros to whole tiles, so there is one form of each product.  The
+// neighbouring eigenvalues: on the tensor cores with three bf16 numbers per value (solve_gemm.cu), or, small ones and those with the
+// result's r columns, on the CUDA cores.  All matrices are padded with zeros to whole tiles, so there is one form of each product.  The
 // (r + oversample)^2 problems run in fp64.
 #include <cuda_runtime.h>
 #include <math.h>
@@ -291,10 +291,10 @@ __global__ void __launch_bounds__(256) k_skinny(int P, const float* __restrict__
 
 template <int NC, bool TA>
 cudaError_t launch_skinny(cudaStream_t st, int M, int P, const float* A, int lda, const float* B, int ldb, int N, float* C, int ldc, const float* shift) {
-  // as many CTAs per tile as there are SMs for, each with at least eight slices of P
+  // as many CTAs per tile as there is room for (two per SM), each with at least eight slices of P
   const int tiles = M / 64 * (N / (16 * NC));
   int ks = 4;
-  while (ks > 1 && (tiles * ks > 160 || P % (BKS * ks) || P / ks < 8 * BKS)) ks >>= 1;
+  while (ks > 1 && (tiles * ks > 300 || P % (BKS * ks) || P / ks < 8 * BKS)) ks >>= 1;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(ks, M / 64, N / (16 * NC));
   cfg.blockDim = dim3(256);
@@ -1070,11 +1070,13 @@ bool make_plan(const eora_solve_config* c, Plan& p) {
   p.off_filter = take(sizeof(Filter));
   p.off_p = take((size_t)p.dp * p.np * 4);                        // P = dW X~; the loss check keeps (dW - B'A) X~ here
   // One region for what is not needed at the same time: dW and X~^T split, all of them or half of the reduction axis at a time (where all would take more than
-  // 32 MB); C, and P split for its square behind it; in the loss check dW - B'A.
+  // 32 MB); C, and behind it P split for its square, then C and the iterate split; in the end P and the iterate split; in the loss check dW - B'A.
   p.kc = eora::split_bytes(p.dp, p.kp) + eora::split_bytes(p.np, p.kp) > (32u << 20) ? (p.kp / 128 + 1) / 2 * 128 : p.kp;
   const size_t s_p = eora::split_bytes(p.dp, p.np);
   size_t big = r_el * 4;
-  for (size_t v : {eora::split_bytes(p.dp, p.kc) + eora::split_bytes(p.np, p.kc), up256(c_el * 4) + s_p}) if (v > big) big = v;
+  const size_t s_q = eora::split_bytes(up128(p.ldm), p.dp > p.np ? p.dp : p.np);      // an iterate
+  for (size_t v : {eora::split_bytes(p.dp, p.kc) + eora::split_bytes(p.np, p.kc), up256(c_el * 4) + s_p, up256(c_el * 4) + eora::split_bytes(p.sp, p.sp) + s_q, s_p + s_q})
+    if (v > big) big = v;
   p.off_c = take(big);
   p.off_y = take(rows * p.ldm * 4);
   p.off_q = take(rows * p.ldm * 4);
@@ -1201,6 +1203,21 @@ int eora_solve(const eora_solve_config* cfg, const float* w, const float* w_hat,
   if (p.n_side) CK(eora::split_cols(st, Pm, dp, np, np, dp, np, behind_c));
   else CK(eora::split_rows(st, Pm, nullptr, dp, np, np, dp, np, behind_c, nullptr, 0));
   CK(eora::split_gemm(st, behind_c, behind_c, sp, sp, p.n_side ? dp : np, C, sp, true, false, sms, status));
+  // The products with an iterate: on the tensor cores, the iterate being split for each, or, small ones, on the CUDA cores in one launch.  512 x 512 x 64: 9
+  // against 6 us on the CUDA cores, 768 x 768 x 64 about even; 2048 x 2048 x 160: 21 against 50.
+  const bool tensor = (double)sp * sp * ldm >= 8e7;
+  if (tensor) CK(eora::split_rows(st, C, nullptr, sp, sp, sp, sp, sp, behind_c, nullptr, 0));
+  // V [rows_out][ldm] = M U - *shift U for an iterate U; M = mat split (rows_out x rows_in); sq: where U is split
+  auto product = [&](const uint8_t* mat, uint8_t* sq, int rows_out, int rows_in, const float* U, float* V, const float* shift) -> int {
+    CK(eora::split_cols(st, U, rows_in, ldm, ldm, rows_in, up128(ldm), sq));
+    CK(eora::split_skinny(st, p.w, mat, sq, rows_out, ldm, rows_in, V, ldm, U, shift, status));
+    return EORA_OK;
+  };
+  auto times_c = [&](const float* U, float* V, const float* shift) -> int {
+    if (tensor) return product(behind_c, behind_c + eora::split_bytes(sp, sp), sp, sp, U, V, shift);
+    CK(skinny<true>(st, p.w, sp, sp, C, sp, U, ldm, ldm, V, ldm, shift));      // (C is symmetric: read by columns)
+    return EORA_OK;
+  };
   // step 5: subspace iteration
   k_init<<<592, 256, 0, st>>>(Y, p.s, sp, p.m, ldm);
   CK(cudaGetLastError());
@@ -1223,9 +1240,9 @@ int eora_solve(const eora_solve_config* cfg, const float* w, const float* w_hat,
   Filter* f = filter ? reinterpret_cast<Filter*>(ws + p.off_filter) : nullptr;
   for (int it = 0, pairs = 0; it < iters;) {
     const bool pair = it >= kSingleSteps && iters - it >= 2;
-    CK(skinny<true>(st, p.w, sp, sp, C, sp, Q, ldm, ldm, Y, ldm, pair && f ? f->rho : nullptr));      // Y = C Q (C is symmetric: read by columns)
+    if (int rc = times_c(Q, Y, pair && f ? f->rho : nullptr)) return rc;
     if (pair) {
-      CK(skinny<true>(st, p.w, sp, sp, C, sp, Y, ldm, ldm, Q, ldm, f ? f->rho + 1 : nullptr));
+      if (int rc = times_c(Y, Q, f ? f->rho + 1 : nullptr)) return rc;
       float* y = Y; Y = Q; Q = y;
     }
     it += pair ? 2 : 1;
@@ -1234,12 +1251,22 @@ int eora_solve(const eora_solve_config* cfg, const float* w, const float* w_hat,
     if (int rc = orthonormalise(st, p, sp, Y, Q, S, Sp, D, next_pair, next_pair ? f : nullptr, pair, node(i), node(2 * kPairs - 1 - i))) return rc;
   }
   if (p.n_side) {                                                             // to the d-dimensional side
-    CK(skinny<false>(st, p.w, dp, np, Pm, np, Q, ldm, ldm, Y, ldm));
+    if (tensor) {
+      CK(eora::split_rows(st, Pm, nullptr, dp, np, np, dp, np, big, nullptr, 0));
+      if (int rc = product(big, big + eora::split_bytes(dp, np), dp, np, Q, Y, nullptr)) return rc;
+    } else {
+      CK(skinny<false>(st, p.w, dp, np, Pm, np, Q, ldm, ldm, Y, ldm));
+    }
     if (int rc = orthonormalise(st, p, dp, Y, Q, S, Sp, D)) return rc;
   }
   if (int rc = orthonormalise(st, p, dp, Q, Y, S, Sp, D)) return rc;          // second pass: orthogonal to fp32 rounding
   // Rayleigh-Ritz on span(Y)
-  CK(skinny<true>(st, p.w, np, dp, Pm, np, Y, ldm, ldm, Z, ldm));             // Z = P^T Y
+  if (tensor) {                                                               // Z = P^T Y
+    CK(eora::split_cols(st, Pm, dp, np, np, dp, np, big));
+    if (int rc = product(big, big + eora::split_bytes(dp, np), np, dp, Y, Z, nullptr)) return rc;
+  } else {
+    CK(skinny<true>(st, p.w, np, dp, Pm, np, Y, ldm, ldm, Z, ldm));
+  }
   CK(gram64<true>(st, Z, np, p.m, ldm, Sp, H));                               // H = Z^T Z = Y^T P P^T Y
   CK(cudaMemsetAsync(Vf, 0, (size_t)ldm * ldm * 4, st));
   CK(jacobi(st, H, p.m, lam, Vf, ldm));

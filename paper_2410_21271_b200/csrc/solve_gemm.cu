@@ -88,11 +88,17 @@ __global__ void __launch_bounds__(256) k_split_cols(const float* __restrict__ a,
                                                     float* __restrict__ copy) {
   __shared__ float s[kSplitCols][129];
   const int n0 = blockIdx.x * kSplitRows, k0 = blockIdx.y * kSplitCols;
-  for (int e = threadIdx.x; e < kSplitCols * kSplitRows; e += 256) {
-    const int k = e >> 7, n = e & 127;
-    const float v = k0 + k < rows && n0 + n < cols ? a[(int64_t)(k0 + k) * lda + n0 + n] : 0.f;
-    s[k][n] = v;
-    if (copy) copy[(int64_t)(k0 + k) * cols_p + n0 + n] = v;
+  float v[16];                                       // (all loads out together: the pass is latency)
+#pragma unroll
+  for (int i = 0; i < 16; ++i) {
+    const int k = (threadIdx.x >> 7) + 2 * i, n = threadIdx.x & 127;
+    v[i] = k0 + k < rows && n0 + n < cols ? a[(int64_t)(k0 + k) * lda + n0 + n] : 0.f;
+  }
+#pragma unroll
+  for (int i = 0; i < 16; ++i) {
+    const int k = (threadIdx.x >> 7) + 2 * i, n = threadIdx.x & 127;
+    s[k][n] = v[i];
+    if (copy) copy[(int64_t)(k0 + k) * cols_p + n0 + n] = v[i];
   }
   __syncthreads();
   const int c = threadIdx.x & 3;
@@ -100,10 +106,10 @@ __global__ void __launch_bounds__(256) k_split_cols(const float* __restrict__ a,
 #pragma unroll
   for (int i = 0; i < 2; ++i) {
     const int r = (threadIdx.x >> 2) + i * 64;
-    float v[8];
+    float w[8];
 #pragma unroll
-    for (int e = 0; e < 8; ++e) v[e] = s[8 * c + e][r];
-    store_piece(block, r, c, v);
+    for (int e = 0; e < 8; ++e) w[e] = s[8 * c + e][r];
+    store_piece(block, r, c, w);
   }
 }
 
@@ -126,15 +132,13 @@ __device__ __forceinline__ bool elect_one() {
   asm volatile("{\n\t.reg .pred q;\n\telect.sync _|q, 0xffffffff;\n\tselp.u32 %0, 1, 0, q;\n\t}" : "=r"(p));
   return p != 0;
 }
-__device__ __forceinline__ void tmem_add16(uint32_t taddr, float* acc) {
-  uint32_t v[16];
-  asm volatile("tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
-               : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]), "=r"(v[8]), "=r"(v[9]),
-                 "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15])
-               : "r"(taddr) : "memory");
+__device__ __forceinline__ void tmem_add8(uint32_t taddr, float* acc) {
+  uint32_t v[8];
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+               : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]) : "r"(taddr) : "memory");
   asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 #pragma unroll
-  for (int i = 0; i < 16; ++i) acc[i] += __uint_as_float(v[i]);
+  for (int i = 0; i < 8; ++i) acc[i] += __uint_as_float(v[i]);
 }
 // K-major, 64-byte swizzle operand descriptor: rows of 64 B, 8-row groups 512 B apart.
 __device__ __forceinline__ uint64_t make_desc64(uint32_t addr) {
@@ -143,13 +147,131 @@ __device__ __forceinline__ uint64_t make_desc64(uint32_t addr) {
   return ((uint64_t)hi << 32) | lo;
 }
 
+// The barriers of a CTA and its tensor memory: high x high in columns [0, NT), the rest in [256, 256 + NT).
+struct GemmShared { uint64_t full[4], empty[4], d0_full, d0_free, d1_full; uint32_t tmem; };
+constexpr uint32_t kSmallCol = 256;
+template <int S>
+__device__ __forceinline__ void gemm_setup(GemmShared& sh, int warp) {
+  if (threadIdx.x == 0) {
+    for (int i = 0; i < S; ++i) { mbar_init(sh.full + i, 1); mbar_init(sh.empty + i, 1); }
+    mbar_init(&sh.d0_full, 1); mbar_init(&sh.d0_free, 16); mbar_init(&sh.d1_full, 1);
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+  }
+  if (warp == 2) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&sh.tmem)), "r"(512u) : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  }
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  __syncthreads();
+  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+}
+__device__ __forceinline__ void gemm_release(GemmShared& sh, int warp) {
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  __syncthreads();
+  if (warp == 2) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(sh.tmem), "r"(512u) : "memory");
+}
+
+// The sums of a tile of 128 rows x NT columns over nkb stages.  ap: the row block of A at the first stage.  b: all of B; rows [n0, n0 + NT) of it, stages
+// from kb0 on, of nkb_b in all.  Warps 4..19 return the sums of row 32 (warp % 4) + lane and NT / 4 columns from (warp - 4) / 4 * NT / 4 on in acc
+// (warps whose wait ran out return false); the others take part.
+template <int NT, int S>
+__device__ __forceinline__ bool gemm_tile(GemmShared& sh, uint32_t smem, int warp, int lane, const uint8_t* ap, const uint8_t* b, int n0, int kb0,
+                                          int nkb_b, int nkb, int* status, float (&acc)[NT / 4]) {
+  constexpr int kStage = gemm_stage(NT), kA = kSplitBlock, kPlaneB = NT * 64;
+  if (warp == 0) {
+    if (lane == 0) {
+      int s = 0, wrap = 0, it = 0;
+      bool ok = true;
+      for (; it < nkb; ++it) {
+        if (wrap > 0 && !mbar_wait(sh.empty + s, (wrap - 1) & 1, status)) { ok = false; break; }
+        const uint32_t at = smem + s * kStage, bar = smem_u32(sh.full + s);
+        mbar_expect_tx_a(bar, kStage);
+        bulk_g2s_a(at, ap + (int64_t)it * kSplitBlock, kSplitBlock, bar);
+        for (int r = 0; r < NT;) {                   // the rows of B lie in one to three row blocks (n0 is a multiple of 32: the swizzle fits)
+          const int in = (n0 + r) % kSplitRows, cnt = min(kSplitRows - in, NT - r);
+          const uint8_t* src = b + ((int64_t)((n0 + r) / kSplitRows) * nkb_b + kb0 + it) * kSplitBlock + in * 64;
+          if (NT == kSplitRows && cnt == NT) {
+            bulk_g2s_a(at + kA, src, kSplitBlock, bar);
+          } else {
+#pragma unroll
+            for (int q = 0; q < 3; ++q) bulk_g2s_a(at + kA + q * kPlaneB + r * 64, src + q * kSplitPlane, cnt * 64, bar);
+          }
+          r += cnt;
+        }
+        if (++s == S) { s = 0; ++wrap; }
+      }
+      if (!ok) {                                     // gave up: what is in flight lands first
+        const int issued = it < S ? it : S;
+        for (int i = 0; i < issued; ++i) {
+          const int at_it = it - 1 - i, slot = at_it % S;
+          const unsigned long long t0 = globaltimer_ns();
+          while (!mbar_try_wait(sh.full + slot, (at_it / S) & 1) && globaltimer_ns() - t0 < 2000000ull) __nanosleep(200);
+        }
+      }
+    }
+  } else if (__shfl_sync(0xffffffffu, warp, 0) == 1) {
+    constexpr uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(NT >> 3) << 17) | ((128u >> 4) << 24);      // fp32 += bf16 x bf16
+    const bool elected = elect_one();
+    const uint32_t tmem = sh.tmem, small = tmem + kSmallCol;
+    const uint64_t a0 = make_desc64(smem), b0 = make_desc64(smem + kA);
+    constexpr uint32_t pa = kSplitPlane >> 4, pb = kPlaneB >> 4;
+    bool ok = true;
+    uint32_t s = 0, ph = 0;
+    for (int it = 0, pos = 0; it < nkb; ++it) {
+      if (!mbar_try_wait_a(smem_u32(sh.full + s), ph)) ok = mbar_wait(sh.full + s, ph, status);
+      if (ok && pos == 0 && it > 0) ok = mbar_wait(&sh.d0_free, (it / kChunk - 1) & 1, status);
+      if (!__all_sync(0xffffffffu, ok)) break;
+      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+      const uint64_t ad = a0 + s * (kStage >> 4), bd = b0 + s * (kStage >> 4);
+      const bool last = pos == kChunk - 1 || it == nkb - 1;
+      if (elected) {
+#pragma unroll
+        for (int k = 0; k < 2; ++k) umma_bf16(tmem, ad + 2 * k, bd + 2 * k, idesc, pos > 0 || k > 0 ? 1u : 0u);
+        if (last) umma_commit(&sh.d0_full);
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+          umma_bf16(small, ad + 2 * k, bd + pb + 2 * k, idesc, it > 0 || k > 0 ? 1u : 0u);
+          umma_bf16(small, ad + pa + 2 * k, bd + 2 * k, idesc, 1u);
+          umma_bf16(small, ad + 2 * k, bd + 2 * pb + 2 * k, idesc, 1u);
+          umma_bf16(small, ad + 2 * pa + 2 * k, bd + 2 * k, idesc, 1u);
+          umma_bf16(small, ad + pa + 2 * k, bd + pb + 2 * k, idesc, 1u);
+        }
+        umma_commit(sh.empty + s);
+      }
+      if (++pos == kChunk) pos = 0;
+      if (++s == (uint32_t)S) { s = 0; ph ^= 1u; }
+    }
+    if (elected) umma_commit(&sh.d1_full);
+    __syncwarp();
+  } else if (warp >= 4) {
+    constexpr int W = NT / 4;                        // columns of a warp: a quarter of the tile's, of the 32 rows its number selects
+    const uint32_t at = sh.tmem + ((uint32_t)((warp & 3) * 32) << 16) + ((warp - 4) >> 2) * W;
+#pragma unroll
+    for (int i = 0; i < W; ++i) acc[i] = 0.f;
+    const int chunks = (nkb + kChunk - 1) / kChunk;
+    for (int ch = 0; ch < chunks; ++ch) {
+      if (!mbar_wait_warp_fast(&sh.d0_full, ch & 1, status, lane)) return false;
+      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+#pragma unroll
+      for (int i = 0; i < W; i += 8) tmem_add8(at + i, acc + i);
+      asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+      __syncwarp();
+      if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(&sh.d0_free)) : "memory");
+    }
+    if (!mbar_wait_warp_fast(&sh.d1_full, 0, status, lane)) return false;
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+#pragma unroll
+    for (int i = 0; i < W; i += 8) tmem_add8(at + kSmallCol + i, acc + i);
+  }
+  return true;
+}
+
 template <int NT, bool SYM>
 __global__ void __launch_bounds__(kGemmThreads, 1) k_split_gemm(const uint8_t* __restrict__ a, const uint8_t* __restrict__ b, int nkb,
                                                                  float* __restrict__ c, int ldc, bool add, int* status) {
-  constexpr int S = gemm_stages(NT), kStage = gemm_stage(NT), kA = kSplitBlock, kPlaneB = NT * 64;
   extern __shared__ __align__(1024) uint8_t smem_raw[];
-  __shared__ __align__(8) uint64_t full[S], empty[S], d0_full, d0_free, d1_full;
-  __shared__ uint32_t tmem_s;
+  __shared__ __align__(8) GemmShared sh;
   const uint32_t smem = (smem_u32(smem_raw) + 1023u) & ~1023u;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   int by = blockIdx.y, bx = blockIdx.x;
@@ -159,127 +281,75 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_split_gemm(const uint8_t* _
     while (by * (by + 1) / 2 > bx) --by;
     bx -= by * (by + 1) / 2;
   }
-  if (threadIdx.x == 0) {
-    for (int i = 0; i < S; ++i) { mbar_init(full + i, 1); mbar_init(empty + i, 1); }
-    mbar_init(&d0_full, 1); mbar_init(&d0_free, 16); mbar_init(&d1_full, 1);
-    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+  gemm_setup<gemm_stages(NT)>(sh, warp);
+  float acc[NT / 4];
+  const bool ok = gemm_tile<NT, gemm_stages(NT)>(sh, smem, warp, lane, a + (int64_t)by * nkb * kSplitBlock, b, bx * NT, 0, nkb, nkb, status, acc);
+  if (warp >= 4 && ok) {
+    const int64_t row = (int64_t)by * 128 + (warp & 3) * 32 + lane, col = (int64_t)bx * NT + ((warp - 4) >> 2) * (NT / 4);
+    float4* to = reinterpret_cast<float4*>(c + row * ldc + col);
+    if (add) {
+#pragma unroll
+      for (int i = 0; i < NT / 16; ++i) {
+        const float4 o = to[i];
+        acc[4 * i] += o.x; acc[4 * i + 1] += o.y; acc[4 * i + 2] += o.z; acc[4 * i + 3] += o.w;
+      }
+    }
+#pragma unroll
+    for (int i = 0; i < NT / 16; ++i) to[i] = make_float4(acc[4 * i], acc[4 * i + 1], acc[4 * i + 2], acc[4 * i + 3]);
+    if (SYM && by != bx) {
+#pragma unroll
+      for (int i = 0; i < NT / 4; ++i) c[(col + i) * ldc + row] = acc[i];
+    }
   }
-  if (warp == 2) {                                   // high x high in columns [0, NT), the rest in [NT, 2 NT)
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_s)), "r"(2u * NT) : "memory");
-    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
-  }
-  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-  __syncthreads();
-  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-  const uint32_t tmem = tmem_s;
+  gemm_release(sh, warp);
+}
 
-  if (warp == 0) {
-    if (lane == 0) {
-      const uint8_t* ap = a + (int64_t)by * nkb * kSplitBlock;
-      const uint8_t* bp = b + (int64_t)bx * (NT / kSplitRows) * nkb * kSplitBlock;
-      int s = 0, wrap = 0, it = 0;
-      bool ok = true;
-      for (; it < nkb; ++it) {
-        if (wrap > 0 && !mbar_wait(empty + s, (wrap - 1) & 1, status)) { ok = false; break; }
-        const uint32_t at = smem + s * kStage, bar = smem_u32(full + s);
-        mbar_expect_tx_a(bar, kStage);
-        bulk_g2s_a(at, ap + (int64_t)it * kSplitBlock, kSplitBlock, bar);
-        if (NT == kSplitRows) {
-          bulk_g2s_a(at + kA, bp + (int64_t)it * kSplitBlock, kSplitBlock, bar);
-        } else {                                     // a plane of both row blocks, one behind the other
+// Products with an iterate: C [m][ldc] = A B^T - *shift Y, B having a few hundred rows (the iterate's columns), of which a CTA takes NT.  A cluster
+// shares a tile of 128 rows along the reduction axis; the parts meet in distributed shared memory and are added in a fixed order.
+// 2048 x 2048 x 160 are 16 tiles, 64 CTAs of sixteen stages.
+constexpr int kPartPad = 4;                          // floats between the rows of a part (16-byte stores of 32 rows hit all banks)
+template <int NT>
+__global__ void __launch_bounds__(kGemmThreads, 1) k_split_skinny(const uint8_t* __restrict__ a, const uint8_t* __restrict__ b, int nkb,
+                                                                   float* __restrict__ c, int ldc, const float* __restrict__ y, const float* __restrict__ shift, int* status) {
+  constexpr int S = 3, pitch = NT + kPartPad;
+  extern __shared__ __align__(1024) uint8_t smem_raw[];
+  __shared__ __align__(8) GemmShared sh;
+  uint8_t* base = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
+  const uint32_t smem = smem_u32(base);
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, ks = gridDim.x, rank = blockIdx.x;
+  const int n0 = blockIdx.z * NT, lo = rank * nkb / ks, hi = (rank + 1) * nkb / ks;
+  gemm_setup<S>(sh, warp);
+  float acc[NT / 4];
+  const bool ok = gemm_tile<NT, S>(sh, smem, warp, lane, a + ((int64_t)blockIdx.y * nkb + lo) * kSplitBlock, b, n0, lo, nkb, hi - lo, status, acc);
+  // (every MMA has completed when a warp has its sums, so the stages may be overwritten; a CTA that gave up sends what it has: the status says so)
+  float* part = reinterpret_cast<float*>(base);
+  if (warp >= 4 && ok) {
+    float4* to = reinterpret_cast<float4*>(part + ((warp & 3) * 32 + lane) * pitch + ((warp - 4) >> 2) * (NT / 4));
 #pragma unroll
-          for (int q = 0; q < 6; ++q)
-            bulk_g2s_a(at + kA + (q >> 1) * kPlaneB + (q & 1) * kSplitPlane, bp + ((int64_t)(q & 1) * nkb + it) * kSplitBlock + (q >> 1) * kSplitPlane, kSplitPlane, bar);
-        }
-        if (++s == S) { s = 0; ++wrap; }
-      }
-      if (!ok) {                                     // gave up: what is in flight lands first
-        const int issued = it < S ? it : S;
-        for (int i = 0; i < issued; ++i) {
-          const int at_it = it - 1 - i, slot = at_it % S;
-          const unsigned long long t0 = globaltimer_ns();
-          while (!mbar_try_wait(full + slot, (at_it / S) & 1) && globaltimer_ns() - t0 < 2000000ull) __nanosleep(200);
-        }
-      }
-    }
-  } else if (__shfl_sync(0xffffffffu, warp, 0) == 1) {
-    constexpr uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(NT >> 3) << 17) | ((128u >> 4) << 24);      // fp32 += bf16 x bf16
-    const bool elected = elect_one();
-    const uint64_t a0 = make_desc64(smem), b0 = make_desc64(smem + kA);
-    constexpr uint32_t pa = kSplitPlane >> 4, pb = kPlaneB >> 4;
-    bool ok = true;
-    uint32_t s = 0, ph = 0;
-    for (int it = 0, pos = 0; it < nkb; ++it) {
-      if (!mbar_try_wait_a(smem_u32(full + s), ph)) ok = mbar_wait(full + s, ph, status);
-      if (ok && pos == 0 && it > 0) ok = mbar_wait(&d0_free, (it / kChunk - 1) & 1, status);
-      if (!__all_sync(0xffffffffu, ok)) break;
-      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-      const uint64_t ad = a0 + s * (kStage >> 4), bd = b0 + s * (kStage >> 4);
-      const bool last = pos == kChunk - 1 || it == nkb - 1;
-      if (elected) {
-#pragma unroll
-        for (int k = 0; k < 2; ++k) umma_bf16(tmem, ad + 2 * k, bd + 2 * k, idesc, pos > 0 || k > 0 ? 1u : 0u);
-        if (last) umma_commit(&d0_full);
-#pragma unroll
-        for (int k = 0; k < 2; ++k) {
-          umma_bf16(tmem + NT, ad + 2 * k, bd + pb + 2 * k, idesc, it > 0 || k > 0 ? 1u : 0u);
-          umma_bf16(tmem + NT, ad + pa + 2 * k, bd + 2 * k, idesc, 1u);
-          umma_bf16(tmem + NT, ad + 2 * k, bd + 2 * pb + 2 * k, idesc, 1u);
-          umma_bf16(tmem + NT, ad + 2 * pa + 2 * k, bd + 2 * k, idesc, 1u);
-          umma_bf16(tmem + NT, ad + pa + 2 * k, bd + pb + 2 * k, idesc, 1u);
-        }
-        umma_commit(empty + s);
-      }
-      if (++pos == kChunk) pos = 0;
-      if (++s == (uint32_t)S) { s = 0; ph ^= 1u; }
-    }
-    if (elected) umma_commit(&d1_full);
-    __syncwarp();
-  } else if (warp >= 4) {
-    constexpr int W = NT / 4;                        // columns of a warp: a quarter of the tile's, of the 32 rows its number selects
-    const int lq = warp & 3, cg = (warp - 4) >> 2;
-    const uint32_t at = tmem + ((uint32_t)(lq * 32) << 16) + cg * W;
-    float acc[W];
-#pragma unroll
-    for (int i = 0; i < W; ++i) acc[i] = 0.f;
-    bool ok = true;
-    const int chunks = (nkb + kChunk - 1) / kChunk;
-    for (int ch = 0; ch < chunks && ok; ++ch) {
-      ok = mbar_wait_warp_fast(&d0_full, ch & 1, status, lane);
-      if (!ok) break;
-      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-#pragma unroll
-      for (int i = 0; i < W; i += 16) tmem_add16(at + i, acc + i);
-      asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-      __syncwarp();
-      if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(&d0_free)) : "memory");
-    }
-    if (ok) ok = mbar_wait_warp_fast(&d1_full, 0, status, lane);
-    if (ok) {
-      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-#pragma unroll
-      for (int i = 0; i < W; i += 16) tmem_add16(at + NT + i, acc + i);
-      const int64_t row = (int64_t)by * 128 + lq * 32 + lane, col = (int64_t)bx * NT + cg * W;
-      float4* to = reinterpret_cast<float4*>(c + row * ldc + col);
-      if (add) {
-#pragma unroll
-        for (int i = 0; i < W / 4; ++i) {
-          const float4 o = to[i];
-          acc[4 * i] += o.x; acc[4 * i + 1] += o.y; acc[4 * i + 2] += o.z; acc[4 * i + 3] += o.w;
-        }
-      }
-#pragma unroll
-      for (int i = 0; i < W / 4; ++i) to[i] = make_float4(acc[4 * i], acc[4 * i + 1], acc[4 * i + 2], acc[4 * i + 3]);
-      if (SYM && by != bx) {
-#pragma unroll
-        for (int i = 0; i < W; ++i) c[(col + i) * ldc + row] = acc[i];
-      }
-    }
+    for (int i = 0; i < NT / 16; ++i) to[i] = make_float4(acc[4 * i], acc[4 * i + 1], acc[4 * i + 2], acc[4 * i + 3]);
   }
-  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-  __syncthreads();
-  if (warp == 2) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(2u * NT) : "memory");
+  __syncwarp();
+  cluster_arrive(); cluster_wait();
+  const int per = 128 / ks;                          // rows of the tile that this CTA adds up
+  const float rho = shift ? *shift : 0.f;
+  for (int e = threadIdx.x; e < per * (NT / 4); e += kGemmThreads) {
+    const int r = rank * per + e / (NT / 4), q = (e % (NT / 4)) * 4;
+    const uint32_t at = smem + (r * pitch + q) * 4;
+    float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int k = 0; k < ks; ++k) {
+      float4 u;
+      asm volatile("ld.shared::cluster.v4.f32 {%0,%1,%2,%3}, [%4];" : "=f"(u.x), "=f"(u.y), "=f"(u.z), "=f"(u.w) : "r"(mapa(at, (uint32_t)k)));
+      v.x += u.x; v.y += u.y; v.z += u.z; v.w += u.w;
+    }
+    const int64_t to = ((int64_t)blockIdx.y * 128 + r) * ldc + n0 + q;
+    if (shift) {
+      const float4 u = *reinterpret_cast<const float4*>(y + to);
+      v.x = fmaf(-rho, u.x, v.x); v.y = fmaf(-rho, u.y, v.y); v.z = fmaf(-rho, u.z, v.z); v.w = fmaf(-rho, u.w, v.w);
+    }
+    *reinterpret_cast<float4*>(c + to) = v;
+  }
+  cluster_arrive(); cluster_wait();                  // nobody leaves while its sums are being read
+  gemm_release(sh, warp);
 }
 
 template <int NT, bool SYM>
@@ -316,6 +386,49 @@ cudaError_t split_gemm(cudaStream_t st, const uint8_t* a, const uint8_t* b, int 
   const int waves256 = (mt * (nt / 2) + sm_count - 1) / sm_count, waves128 = (mt * nt + sm_count - 1) / sm_count;
   if (nt % 2 == 0 && waves256 * 1536 <= waves128 * 900) return launch_gemm<256, false>(dim3(nt / 2, mt), st, a, b, k, c, ldc, add, status);
   return launch_gemm<128, false>(dim3(nt, mt), st, a, b, k, c, ldc, add, status);
+}
+
+namespace {
+template <int NT>
+cudaError_t launch_skinny(cudaStream_t st, const uint8_t* a, const uint8_t* b, int m, int n, int k, float* c, int ldc, const float* y, const float* shift, int* status) {
+  constexpr int smem = 3 * gemm_stage(NT) + 1024;
+  static_assert(128 * (NT + kPartPad) * 4 <= 3 * gemm_stage(NT), "a CTA's sums take the place of its stages");
+  static bool set[64] = {};                          // per device
+  int device = 0;
+  cudaError_t e = cudaGetDevice(&device);
+  if (e != cudaSuccess) return e;
+  if (device < 0 || device >= 64) return cudaErrorInvalidDevice;
+  if (!set[device]) {
+    e = cudaFuncSetAttribute(k_split_skinny<NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    if (e != cudaSuccess) return e;
+    set[device] = true;
+  }
+  // as many CTAs per tile as run at once (15 clusters of eight, 33 of four, 74 of two, measured with one CTA per SM), each with at least four stages.  (A
+  // sixteenth cluster of eight waits for the others: 25 us instead of 17.)
+  const int tiles = m / 128 * (n / NT), nkb = k / kSplitCols;
+  int ks = 8;
+  while (ks > 1 && (tiles > (ks == 8 ? 15 : ks == 4 ? 33 : 74) || nkb / ks < 4)) ks >>= 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(ks, m / 128, n / NT);
+  cfg.blockDim = dim3(kGemmThreads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = ks; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, k_split_skinny<NT>, a, b, nkb, c, ldc, y, shift, status);
+}
+}  // namespace
+
+cudaError_t split_skinny(cudaStream_t st, int width, const uint8_t* a, const uint8_t* b, int m, int n, int k, float* c, int ldc, const float* y, const float* shift, int* status) {
+  switch (width) {
+    case 64: return launch_skinny<64>(st, a, b, m, n, k, c, ldc, y, shift, status);
+    case 96: return launch_skinny<96>(st, a, b, m, n, k, c, ldc, y, shift, status);
+    case 128: return launch_skinny<128>(st, a, b, m, n, k, c, ldc, y, shift, status);
+    default: return launch_skinny<160>(st, a, b, m, n, k, c, ldc, y, shift, status);
+  }
 }
 
 }  // namespace eora

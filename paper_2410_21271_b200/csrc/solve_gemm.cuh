@@ -23,4 +23,9 @@ cudaError_t split_cols(cudaStream_t st, const float* a, int rows, int cols, int 
 cudaError_t split_gemm(cudaStream_t st, const uint8_t* a, const uint8_t* b, int m, int n, int k, float* c, int ldc, bool sym, bool add, int sm_count,
                        int* status);
 
+// The same for B with n (a multiple of `width`: 64, 96, 128 or 160) rows, split as a matrix of whole blocks: C [m][ldc] = A B^T - *shift Y
+// (shift, Y [m][ldc]: may be null; Y must not be C).
+cudaError_t split_skinny(cudaStream_t st, int width, const uint8_t* a, const uint8_t* b, int m, int n, int k, float* c, int ldc, const float* y,
+                         const float* shift, int* status);
+
 }  // namespace eora
