@@ -444,35 +444,55 @@ __device__ __forceinline__ double rsqrt_newton(double d) {
 // The chain of (A)s is what bounds it: a pivot, its root, a column and an update, 16 times per panel.
 // Writes L over S (lower triangle, global) and the inverses of the diagonal blocks; Q = Y L^{-T} follows by k_trsm.  Every diagonal
 // element first grows by 1e-13 of itself, so that a rank-deficient iterate still factors; relative to itself, because the columns of
-// an iterate are graded (column j has about the norm of the j-th eigenvalue, or of its square).  In shared memory up to
-// m = kCholSmem, else in place in global memory (L2).  m = 160: 300 us with an explicit inverse and unblocked updates before.
+// an iterate are graded (column j has about the norm of the j-th eigenvalue, or of its square).
+// L0: the whole matrix, rows ld apart; this launch factors the m x m block (m <= kCholSmem, what shared memory holds) whose first row and column
+// are j_base, of m_all; least_g: [m_all], the smallest pivots of later blocks.  Larger matrices go block by block (orthonormalise).
 constexpr int kCholSmem = 160;
 constexpr int kCholThreads = 512;
 __host__ __device__ constexpr int pan_pitch(int m) { return (m + 5) / 4 * 4 + 2; }      // (even, and rows of the panel on different banks)
-__host__ __device__ constexpr int chol_smem(int m) { return ((m <= kCholSmem ? m * (m | 1) : 0) + m + 16 * pan_pitch(m)) * 8 + 16; }
+__host__ __device__ constexpr int chol_smem(int m) { return (m * (m | 1) + m + 16 * pan_pitch(m)) * 8 + 16; }
 //
 // f (may be null): the filter's state.  With prev the iterate went through a pair of products with (C - f->rho[0] I) and (C - f->rho[1] I), starting from
 // columns of norm 1 / f->scale, else through one with C: the diagonal of L then says where the eigenvalues of the iterate's columns are.
 // The next pair's shifts are lo and hi times the smallest of them.
 struct Filter { float rho[2]; double scale; };
 constexpr double kFilterEdge = 0.95;                 // the estimate comes from below, but not always (measured 0.8 to 1.07 of eigenvalue m after four steps)
-__global__ void __launch_bounds__(kCholThreads) k_chol64(double* Sg, int m, double* __restrict__ Dinv, Filter* f, bool prev, double lo, double hi) {
+__global__ void __launch_bounds__(kCholThreads) k_chol64(double* L0, int ld, int m_all, int j_base, int m, double* __restrict__ Dinv, double* least_g, Filter* f, bool prev, double lo, double hi) {
   extern __shared__ __align__(16) double sm[];
   __shared__ double dv[16][17];
   const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
-  const bool in_smem = m <= kCholSmem;
-  const int ls = in_smem ? (m | 1) : m, lp = pan_pitch(m);
+  double* Sg = L0 + (int64_t)j_base * (ld + 1);
+  const int ls = m | 1, lp = pan_pitch(m);
   double* pan = sm;                                  // [16][lp]: the panel by columns
   double* least = sm + 16 * lp;                      // [m]: the smallest pivot of a column that is taken as it is
-  double* S = in_smem ? least + m : Sg;
-  if (in_smem)
-    for (int i = warp; i < m; i += kCholThreads / 32)
-      for (int j = lane; j <= i; j += 32) S[i * ls + j] = Sg[(int64_t)i * m + j];
+  double* S = least + m;
+  for (int i = warp; i < m; i += 2 * (kCholThreads / 32)) {      // two rows' loads go out together (one at a time each was a round trip to L2: 20 us)
+    double v[2][kCholSmem / 32];
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+#pragma unroll
+      for (int k = 0; k < kCholSmem / 32; ++k) {
+        const int r = i + h * (kCholThreads / 32), j = lane + 32 * k;
+        v[h][k] = r < m && j <= r ? Sg[(int64_t)r * ld + j] : 0.0;
+      }
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+#pragma unroll
+      for (int k = 0; k < kCholSmem / 32; ++k) {
+        const int r = i + h * (kCholThreads / 32), j = lane + 32 * k;
+        if (r < m && j <= r) S[r * ls + j] = v[h][k];
+      }
+  }
   __syncthreads();
-  for (int i = t; i < m; i += kCholThreads) {
-    const double shift = 1e-13 * S[(int64_t)i * ls + i] + 1e-300;
-    S[(int64_t)i * ls + i] += shift;
-    least[i] = 1e-3 * shift;
+  if (j_base == 0) {                                 // (for all blocks: a later one's diagonal is a difference by then)
+    for (int i = t; i < m_all; i += kCholThreads) {
+      double& d = i < m ? S[(int64_t)i * ls + i] : L0[(int64_t)i * (ld + 1)];
+      const double shift = 1e-13 * d + 1e-300;
+      d += shift;
+      if (i < m) least[i] = 1e-3 * shift; else least_g[i] = 1e-3 * shift;
+    }
+  } else {
+    for (int i = t; i < m; i += kCholThreads) least[i] = least_g[j_base + i];
   }
   __syncthreads();
   auto diagonal = [&](int j0) {                      // (A), one warp; lanes 16..31 repeat lanes 0..15
@@ -567,6 +587,7 @@ __global__ void __launch_bounds__(kCholThreads) k_chol64(double* Sg, int m, doub
   if (f && warp == 0) {
     double least_l = 1e300;
     for (int i = lane; i < m; i += 32) least_l = fmin(least_l, S[(int64_t)i * ls + i]);
+    for (int i = lane; i < j_base; i += 32) least_l = fmin(least_l, L0[(int64_t)i * (ld + 1)]);
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) least_l = fmin(least_l, __shfl_xor_sync(0xffffffffu, least_l, o));
     if (lane == 0) {
@@ -576,21 +597,22 @@ __global__ void __launch_bounds__(kCholThreads) k_chol64(double* Sg, int m, doub
         at = 0.5 * (r0 + r1) + sqrt(half * half + least_l * f->scale);
       }
       f->rho[0] = (float)(lo * kFilterEdge * at); f->rho[1] = (float)(hi * kFilterEdge * at);
-      f->scale = 1.0 / (double)pow2_scale(S[0]);
+      f->scale = 1.0 / (double)pow2_scale(j_base ? L0[0] : S[0]);
     }
   }
-  if (in_smem)
-    for (int i = warp; i < m; i += kCholThreads / 32)
-      for (int j = lane; j <= i; j += 32) Sg[(int64_t)i * m + j] = S[i * ls + j];
+  for (int i = warp; i < m; i += kCholThreads / 32)
+    for (int j = lane; j <= i; j += 32) Sg[(int64_t)i * ld + j] = S[i * ls + j];
 }
 
 // Q = Y L^{-T}, row by row (fp64 inside): a CTA takes 16 rows, half a warp each (lane = column of the panel); panel by panel of 16
 // columns  q_p = (y_p - sum_{c < 16 p} q_c L[p][c]^T) Dinv_p^T.  A panel's 16 rows of L and its Dinv come by cp.async, one panel
 // ahead, its column of Y by a load one panel ahead.  With `scaled`, Q is divided by the power of two next to L[0][0].
+// T: float (an iterate; rows are a multiple of 16 and Q's columns past m become zero) or double (rows of the Gram matrix below a block, in place).
 __host__ __device__ constexpr int trsm_pitch(int m) { return (m + 15) / 16 * 16 + 2; }
 __host__ __device__ constexpr int trsm_smem(int m) { return (3 * 16 * trsm_pitch(m) + 2 * 16 * 18) * 8; }
-__global__ void __launch_bounds__(256) k_trsm(const float* __restrict__ Y, const double* __restrict__ L, const double* __restrict__ Dinv, int m, int ld,
-                                              float* __restrict__ Q, bool scaled) {
+template <typename T>
+__global__ void __launch_bounds__(256) k_trsm(const T* Y, const double* __restrict__ L, int ll, const double* __restrict__ Dinv, int m, int ld, int rows,
+                                              T* Q, bool scaled) {
   extern __shared__ __align__(16) double smt[];
   const int lq = trsm_pitch(m);
   double* qd = smt;                                  // [16][lq]
@@ -606,20 +628,21 @@ __global__ void __launch_bounds__(256) k_trsm(const float* __restrict__ Y, const
     double* dst = lp + (p & 1) * 16 * lq;
     copy8(di + (p & 1) * 16 * 18 + r * 18 + c, Dinv + (int64_t)(16 * p + r) * 16 + c);
     for (int q = c; q < 16 * p; q += 16) {
-      if (16 * p + r < m) copy8(dst + r * lq + q, L + (int64_t)(16 * p + r) * m + q);
+      if (16 * p + r < m) copy8(dst + r * lq + q, L + (int64_t)(16 * p + r) * ll + q);
       else dst[r * lq + q] = 0.0;
     }
     asm volatile("cp.async.commit_group;" ::: "memory");
   };
   fetch(0);
-  float y = Y[row * ld + c];
+  const bool live = row < rows;
+  T y = live ? Y[row * ld + c] : (T)0;
   const float scale = scaled ? pow2_scale(L[0]) : 1.f;
   for (int p = 0; p < np; ++p) {
     asm volatile("cp.async.wait_group 0;" ::: "memory");
     __syncthreads();                                 // panel p is there, and panel p - 1 has been read
     if (p + 1 < np) fetch(p + 1);
     double v[4] = {(double)y, 0.0, 0.0, 0.0};
-    if (p + 1 < np) y = Y[row * ld + 16 * (p + 1) + c];
+    if (live && p + 1 < np) y = Y[row * ld + 16 * (p + 1) + c];
     const double* lr = lp + (p & 1) * 16 * lq + c * lq;
     const double* qr = qd + r * lq;
 #pragma unroll 4
@@ -635,10 +658,45 @@ __global__ void __launch_bounds__(256) k_trsm(const float* __restrict__ Y, const
     for (int q = 0; q < 16; ++q) o[q & 3] = fma(__shfl_sync(0xffffffffu, w, q, 16), dr[q], o[q & 3]);      // (Dinv is lower triangular: zeros past c)
     const double res = (o[0] + o[1]) + (o[2] + o[3]);
     qd[r * lq + 16 * p + c] = res;
-    Q[row * ld + 16 * p + c] = (float)res * scale;
+    if (live) Q[row * ld + 16 * p + c] = (T)res * (T)scale;
     __syncwarp();
   }
-  for (int i = 16 * np + c; i < ld; i += 16) Q[row * ld + i] = 0.f;
+  if constexpr (sizeof(T) == 4)
+    for (int i = 16 * np + c; i < ld; i += 16) Q[row * ld + i] = 0.f;
+}
+
+// S22 -= L21 L21^T, lower triangle: rows [j1, m) of the matrix, the block's columns [j0, j1) (a multiple of 32 of them).  One CTA per 32 x 32 tile.
+__global__ void __launch_bounds__(256) k_syrk64(double* __restrict__ S, int ld, int m, int j0, int j1) {
+  __shared__ double sa[32][33], sb[32][33];
+  int bi = (int)((sqrtf(8.f * blockIdx.x + 1.f) - 1.f) * 0.5f);
+  while ((bi + 1) * (bi + 2) / 2 <= (int)blockIdx.x) ++bi;
+  while (bi * (bi + 1) / 2 > (int)blockIdx.x) --bi;
+  const int bj = blockIdx.x - bi * (bi + 1) / 2;
+  const int t = threadIdx.x, x = t & 31, y = t >> 5, ti = t >> 4, tj = t & 15;
+  double acc[2][2] = {{0.0, 0.0}, {0.0, 0.0}};
+  for (int q0 = j0; q0 < j1; q0 += 32) {
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const int i = j1 + bi * 32 + y + 8 * k, j = j1 + bj * 32 + y + 8 * k;
+      sa[y + 8 * k][x] = i < m ? S[(int64_t)i * ld + q0 + x] : 0.0;
+      sb[y + 8 * k][x] = j < m ? S[(int64_t)j * ld + q0 + x] : 0.0;
+    }
+    __syncthreads();
+#pragma unroll 8
+    for (int q = 0; q < 32; ++q) {
+      const double a0 = sa[2 * ti][q], a1 = sa[2 * ti + 1][q], b0 = sb[2 * tj][q], b1 = sb[2 * tj + 1][q];
+      acc[0][0] = fma(a0, b0, acc[0][0]); acc[0][1] = fma(a0, b1, acc[0][1]);
+      acc[1][0] = fma(a1, b0, acc[1][0]); acc[1][1] = fma(a1, b1, acc[1][1]);
+    }
+    __syncthreads();
+  }
+#pragma unroll
+  for (int i = 0; i < 2; ++i)
+#pragma unroll
+    for (int j = 0; j < 2; ++j) {
+      const int gi = j1 + bi * 32 + 2 * ti + i, gj = j1 + bj * 32 + 2 * tj + j;
+      if (gi < m && gj <= gi) S[(int64_t)gi * ld + gj] -= acc[i][j];
+    }
 }
 
 // Symmetric positive semi-definite eigenproblem H = V diag(lam) V^T, m x m, fp64, by one-sided (Hestenes) Jacobi: pairs of
@@ -1084,7 +1142,7 @@ bool make_plan(const eora_solve_config* c, Plan& p) {
   p.off_s = take((size_t)p.m * p.m * 8);
   const size_t gram_el = (size_t)kGramParts * p.m * p.m, sig_el = (size_t)kSigmaParts * 2 * p.r;
   p.off_sp = take((gram_el > sig_el ? gram_el : sig_el) * 8);
-  p.off_d = take((size_t)((p.m + 15) / 16) * 256 * 8);
+  p.off_d = take((size_t)((p.m + 15) / 16) * 256 * 8 + (size_t)p.m * 8);      // the diagonal blocks' inverses, the smallest pivots
   p.off_h = take((size_t)p.m * p.m * 8);
   p.off_lam = take((size_t)(2 * p.m + 128) * 8);
   p.off_vf = take((size_t)p.ldm * p.ldm * 4);
@@ -1116,9 +1174,21 @@ int orthonormalise(cudaStream_t st, const Plan& p, int rows, const float* Y, flo
                    bool scaled = false, Filter* f = nullptr, bool prev = false, double lo = 0.0, double hi = 0.0) {
   CK(gram64<false>(st, Y, rows, p.m, p.ldm, parts, S));
   CK(allow_smem<k_chol64>(chol_smem(kCholSmem)));
-  CK(allow_smem<k_trsm>(trsm_smem(512)));
-  k_chol64<<<1, kCholThreads, chol_smem(p.m), st>>>(S, p.m, D, f, prev, lo, hi);
-  k_trsm<<<rows / 16, 256, trsm_smem(p.m), st>>>(Y, S, D, p.m, p.ldm, Q, scaled);
+  CK(allow_smem<k_trsm<float>>(trsm_smem(512)));
+  CK(allow_smem<k_trsm<double>>(trsm_smem(kCholSmem)));
+  // Up to 160 columns one CTA factors the matrix in shared memory.  More go in blocks of 160: factor, rows below, update of the rest (2048 x 3072, n 2048, 288
+  // columns: 6.28 ms, with one CTA that kept such a matrix in L2 7.72).
+  for (int j0 = 0; j0 < p.m; j0 += kCholSmem) {
+    const int w = p.m - j0 < kCholSmem ? p.m - j0 : kCholSmem, j1 = j0 + w, below = p.m - j1;
+    k_chol64<<<1, kCholThreads, chol_smem(w), st>>>(S, p.m, p.m, j0, w, D + j0 * 16, D + (size_t)((p.m + 15) / 16) * 256, below ? nullptr : f, prev, lo, hi);
+    if (below > 0) {
+      double* l21 = S + (int64_t)j1 * p.m + j0;
+      k_trsm<double><<<(below + 15) / 16, 256, trsm_smem(w), st>>>(l21, S + (int64_t)j0 * (p.m + 1), p.m, D + j0 * 16, w, p.m, below, l21, false);
+      const int nb = (below + 31) / 32;
+      k_syrk64<<<nb * (nb + 1) / 2, 256, 0, st>>>(S, p.m, p.m, j0, j1);
+    }
+  }
+  k_trsm<float><<<rows / 16, 256, trsm_smem(p.m), st>>>(Y, S, p.m, D, p.m, p.ldm, rows, Q, scaled);
   CK(cudaGetLastError());
   return EORA_OK;
 }

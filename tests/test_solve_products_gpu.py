@@ -1,6 +1,6 @@
 """GPU parity of the offline solve where its tensor-core products can go wrong: both tile widths, fewer reduction elements than a chunk of the
 accumulators and a chunk with a remainder, padded sizes (X~ needed as whole tiles), iterates whose column tiles begin inside a block
-of 128, and values at the ends of the range that three bf16 parts cover.  The error has rank r plus noise a hundred times smaller, so the compensation B'A and the singular values are unique and comparable with the float64 oracle."""
+of 128, one to four blocks of the Cholesky factor, and values at the ends of the range that three bf16 parts cover.  The error has rank r plus noise a hundred times smaller, so the compensation B'A and the singular values are unique and comparable with the float64 oracle."""
 import numpy as np
 import pytest
 
@@ -21,7 +21,9 @@ SIGMA_RTOL = 1e-6
     (128, 128, 128, 8),         # one tile, four stages
     (300, 1100, 500, 40),       # padded everywhere; chunks of eight stages with a remainder
     (1024, 320, 384, 100),      # iterate of 132 columns: two tiles of 96
-    (700, 640, 900, 250),       # 282 columns: three tiles of 96
+    (700, 640, 900, 250),       # 282 columns: three tiles of 96, two blocks of the factor
+    (640, 600, 700, 400),       # 432 columns: three blocks of the factor
+    (1000, 1000, 1100, 480),    # 512 columns: four
 ])
 def test_compensation_and_spectrum(d, k, n, r):
     w, w_hat, x = gen.make_solve_case(41, d, k, n, kind="gap", rank_signal=r)
