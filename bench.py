@@ -491,9 +491,9 @@ FP32_PEAK_TFLOPS = 148 * 128 * 2 * 1.965e9 / 1e12
 
 def time_solve(device: str, d: int = 4096, k: int = 4096, n: int = 2048, r: int = 128, reps: int = 3, cpu: bool = True):
     """Extra: the offline solve (Algorithm 1 steps 1-6) of one q-shaped layer: weight 4096 x 4096, 2048 calibration
-    columns, rank 128, library defaults (32 extra vectors, 24 iterations).  Flops = those of the contractions the
-    library runs, without padding: P = dW X~, the lower half of its smaller square, one product with that per iteration, the way to the d side, P^T Y,
-    Y V and dW^T U'; the factorisations and the small fp64 problems are not counted."""
+    columns, rank 128, library defaults (32 extra vectors, 14 products with the square).  Flops = those of the contractions the
+    library runs, without padding: P = dW X~, the lower half of its smaller square, fourteen products with that, the way to the d side, P^T Y,
+    Y V, dW^T U' and X~^T dW^T U'; the factorisations and the small fp64 problems are not counted."""
     import torch
     import paper_2410_21271_b200 as eora
     w, w_hat, x = gen.make_solve_case(31, d, k, n)
@@ -507,10 +507,10 @@ def time_solve(device: str, d: int = 4096, k: int = 4096, n: int = 2048, r: int 
     e1.record()
     torch.cuda.synchronize()
     ms = e0.elapsed_time(e1) / reps
-    m, iters = r + 32, 24
+    m, iters = r + 32, 14
     side, other = (n, d) if m <= n < d else (d, n)        # the library iterates with the smaller square that holds m directions
     flops = 2.0 * d * k * n + 1.0 * side * side * other + iters * 2.0 * side * side * m + (2.0 * d * n * m if side == n else 0.0) \
-        + 2.0 * d * n * m + 2.0 * d * m * r + 2.0 * r * d * k
+        + 2.0 * d * n * m + 2.0 * d * m * r + 2.0 * r * d * k + 2.0 * r * k * n
     loss = eora.solve_loss(tw, th, tx, b, a)
     uncompensated = float(torch.linalg.norm((tw - th).double() @ tx.double()))
     out = {"workload": f"one layer {d}x{k}, {n} calibration columns, rank {r}", "ms": ms, "layers_per_s": 1e3 / ms,

@@ -391,7 +391,9 @@ cudaError_t split_gemm(cudaStream_t st, const uint8_t* a, const uint8_t* b, int 
 namespace {
 template <int NT>
 cudaError_t launch_skinny(cudaStream_t st, const uint8_t* a, const uint8_t* b, int m, int n, int k, float* c, int ldc, const float* y, const float* shift, int* status) {
-  constexpr int smem = 3 * gemm_stage(NT) + 1024;
+  // More than half of an SM's shared memory, so that no two such CTAs (of solves on different streams) share an SM: each takes all of tensor memory, and
+  // clusters whose CTAs wait for one another's would wait for good.
+  constexpr int own = 3 * gemm_stage(NT) + 1024, smem = own > 120 * 1024 ? own : 120 * 1024;
   static_assert(128 * (NT + kPartPad) * 4 <= 3 * gemm_stage(NT), "a CTA's sums take the place of its stages");
   static bool set[64] = {};                          // per device
   int device = 0;
