@@ -5,9 +5,9 @@
 // contraction, so it runs on the 5th-generation tensor cores.  The product is computed transposed,
 // Yt[n][m] = sum_k w[n][k] X[m][k], so that the operand that has to be produced on chip is the small one:
 //   * MMA "A" operand (128 rows): a tile of 128 output columns n of the weights.  Sixteen dequant warps
-//     read the packed tiles of the shared layout straight from global memory (512 contiguous bytes per
-//     warp), turn them into fp16 RN((q - z) * s) in registers and store them as a K-major,
-//     128-byte-swizzled operand tile (bank-conflict-free stores);
+//     turn the packed tiles of the shared layout into fp16 RN((q - z) * s) in registers and store them in tensor memory (TM, see
+//     tm_tile), or, where the accumulators fill that (256 rows x more than 160 tokens), as a K-major,
+//     128-byte-swizzled operand tile in shared memory (bank-conflict-free stores);
 //   * MMA "B" operand (up to 256 rows): a tile of tokens of X, K-major, brought in by TMA
 //     (cp.async.bulk.tensor, 128-byte swizzle, no multicast) into the same ring of k-block stages as
 //     the dequantised weight tile;
@@ -54,6 +54,9 @@ struct PrefillArgs {
   int nkb_w, nkb_b;  // k-blocks of each part
   int sw;            // stages of the ring (token tiles first, weight tiles from w_off on)
   int w_off, w_slot; // byte offset of the weight ring (after sw token tiles of bt*128 bytes), bytes of a weight tile (rows * 128)
+  // Weights in tensor memory (TM): the warps' rings of packed weights start at w_off, w_slot bytes apart; columns of tensor memory from one 128-row
+  // half's accumulator to the next; first column of the ring of weight tiles, columns of a stage (32 per half).
+  int acc_cols, a_col0, a_cols;
   // Where the tiles leave SMs idle, the reduction axis of a tile is split over the ksplit CTAs of a cluster (the first one
   // also takes the K-extension; split_lo says which backbone k-blocks are whose).  The
   // partial accumulators meet in distributed shared memory: every CTA finishes every ksplit-th chunk of 32 tokens.
@@ -95,6 +98,17 @@ __device__ __forceinline__ void tma_load_2d(void* dst, const CUtensorMap* tm, in
 __device__ __forceinline__ void umma_f16(uint32_t tmem_d, uint64_t adesc, uint64_t bdesc, uint32_t idesc, uint32_t accumulate) {
   asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\ttcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
                ::"r"(tmem_d), "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate) : "memory");
+}
+// The same with the 128-row operand in tensor memory: lane = row, one 32-bit column = two reduction elements.
+__device__ __forceinline__ void umma_f16_ts(uint32_t tmem_d, uint32_t tmem_a, uint64_t bdesc, uint32_t idesc, uint32_t accumulate) {
+  asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\ttcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}"
+               ::"r"(tmem_d), "r"(tmem_a), "l"(bdesc), "r"(idesc), "r"(accumulate) : "memory");
+}
+// 16 lanes x 32 columns as fragments of 8 x 8 blocks (the inverse of tmem_ld16x32 below).
+__device__ __forceinline__ void tmem_st16x32(uint32_t taddr, const uint32_t (&v)[16]) {
+  asm volatile("tcgen05.st.sync.aligned.16x256b.x4.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, %16};"
+               ::"r"(taddr), "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]), "r"(v[4]), "r"(v[5]), "r"(v[6]), "r"(v[7]), "r"(v[8]), "r"(v[9]),
+                 "r"(v[10]), "r"(v[11]), "r"(v[12]), "r"(v[13]), "r"(v[14]), "r"(v[15]) : "memory");
 }
 __device__ __forceinline__ void umma_commit(uint64_t* bar) {
   asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar)) : "memory");
@@ -414,7 +428,213 @@ __device__ __forceinline__ bool dequant_part(const WMat& mat, int n0, int kb_lo,
   }
 }
 
-template <int WF, int BF>
+// ---------------------------------------------------------------------------------------------- weights in tensor memory
+// Up to 160 tokens (256 with 128 rows) the accumulators leave tensor memory for the dequantised weights.  Through shared memory a k-block of 256 rows x
+// 64 tokens moved 32 KB of weights in and out of it, 512 cycles of its bandwidth, and each hand-over waited for the stores to become visible to the
+// MMAs (1215 cycles a k-block); here the weights go from registers to tensor memory and the MMAs read only the tokens from shared memory (790).  Three
+// LLaMA3-8B blocks of 64 tokens, 4-bit, 8-bit adapters of rank 512: 419 -> 358 us; a block of 128 tokens 124 -> 105, of a prompt of 333 232 -> 214.
+// Tried and not kept: two chains of MMAs with accumulators of their own (128 rows 515 -> 562 cycles).
+//
+// tcgen05.st writes a tile of 16 rows x 64 reduction elements as fragments of 8 x 8 32-bit blocks: lane (g, t) holds, for each of the four MMAs j of a
+// k-block, elements 16 j + 4 t .. + 3 of rows g and g + 8.  In the packed layout these are half (t & 1) of the eight codes that
+// lane (g, 2 (j & 1) + (t >> 1)) owns of the 32-element block j / 2.  So every warp brings its blobs to shared memory (a ring of its own,
+// asked for before anything else in the kernel) and its lanes read the words of those two lanes.
+// out[4 j + 2 hf + i]: elements 16 j + 4 t + 2 i, + 1 of row g + 8 hf, as fp16 RN((q - z) * s).
+template <int FMT>
+__device__ __forceinline__ void tm_tile(uint32_t tile, int lane, const ZC& zc, uint32_t s_a, uint32_t s_b, uint32_t (&out)[16]) {
+  const int g = lane >> 2, t = lane & 3, half = t & 1;
+  const uint32_t at = (uint32_t)(g * 4 + (t >> 1));  // lane of the packed layout for even j; two further for odd j
+  auto put = [&](int j, int hf, uint32_t a, uint32_t b) {
+    out[4 * j + 2 * hf] = h2mul(a, hf ? s_b : s_a); out[4 * j + 2 * hf + 1] = h2mul(b, hf ? s_b : s_a);
+  };
+  if constexpr (FMT == FMT_Q4) {
+#pragma unroll
+    for (int jj = 0; jj < 2; ++jj) {
+      const uint4 u = lds_u4(tile + (at + 2 * jj) * 16);
+      const uint32_t w[4] = {u.x, u.y, u.z, u.w};
+#pragma unroll
+      for (int part = 0; part < 4; ++part) {
+        const int hf = part & 1;
+        const uint32_t v = w[part] >> (8 * half);
+        put(2 * (part >> 1) + jj, hf, h2sub(and_or(v, 0x000f000fu, kMagic), zc.c[hf][0]), h2fma(and_or(v, 0x00f000f0u, kMagic), 0x2C002C00u, zc.c[hf][1]));
+      }
+    }
+  } else if constexpr (FMT == FMT_Q3) {
+#pragma unroll
+    for (int jj = 0; jj < 2; ++jj) {
+      const uint2 u = lds_u2(tile + (at + 2 * jj) * 8);
+      const uint32_t w2 = lds_u1(tile + 256 + (at + 2 * jj) * 4), w[3] = {u.x, u.y, w2};
+#pragma unroll
+      for (int part = 0; part < 4; ++part) {
+        const int hf = part & 1;
+        const uint32_t q = part < 3 ? (w[part < 3 ? part : 0] >> (3 * half)) & 0x07070707u
+                                    : and_or(w2 >> (4 + half), 0x04040404u, ((half ? u.y : u.x) >> 6) & 0x03030303u);
+        put(2 * (part >> 1) + jj, hf, h2sub(quad_pair(q, 0), zc.c[hf][0]), h2sub(quad_pair(q, 1), zc.c[hf][0]));
+      }
+    }
+  } else if constexpr (FMT == FMT_Q8) {
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+#pragma unroll
+      for (int hf = 0; hf < 2; ++hf) {
+        const uint32_t w = lds_u1(tile + (j >> 1) * 512 + (at + 2 * (j & 1)) * 16 + hf * 8 + half * 4);
+        put(j, hf, h2sub(and_or(w, 0x00ff00ffu, kMagic), zc.c[hf][0]), h2sub(and_or(w >> 8, 0x00ff00ffu, kMagic), zc.c[hf][0]));
+      }
+  } else if constexpr (FMT == FMT_F16) {
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+#pragma unroll
+      for (int hf = 0; hf < 2; ++hf) {
+        const uint2 w = lds_u2(tile + (2 * (j >> 1) + hf) * 512 + (at + 2 * (j & 1)) * 16 + half * 8);
+        out[4 * j + 2 * hf] = w.x; out[4 * j + 2 * hf + 1] = w.y;
+      }
+  } else {                                           // 2:4 formats: the quad `half` of each part (selectors as in dequant_store)
+#pragma unroll
+    for (int jj = 0; jj < 2; ++jj) {
+      const uint32_t meta = lds_u1(tile + (FMT == FMT_SP24 ? 1024 : 256) + (at + 2 * jj) * 4) >> (4 * half);
+      const uint32_t at0 = (meta << 3) & 0x18181818u, at1 = (meta << 1) & 0x18181818u;
+      uint2 u = make_uint2(0u, 0u);
+      if constexpr (FMT == FMT_SQ4) { u = lds_u2(tile + (at + 2 * jj) * 8); u.x >>= 4 * half; u.y >>= 4 * half; }
+#pragma unroll
+      for (int part = 0; part < 4; ++part) {
+        const int hf = part & 1, j = 2 * (part >> 1) + jj;
+        uint32_t v;
+        if constexpr (FMT == FMT_SP24) v = lds_u1(tile + (part >> 1) * 512 + (at + 2 * jj) * 16 + hf * 8 + half * 4);
+        else v = h2mul(h2sub(and_or(((part >> 1) ? u.y : u.x) >> (8 * hf), 0x000f000fu, kMagic), zc.c[hf][0]), hf ? s_b : s_a);
+        const uint32_t sel = 0x44444444u ^ __funnelshift_l(0u, 0x54u, at0 >> (8 * part)) ^ __funnelshift_l(0u, 0x76u, at1 >> (8 * part));
+        out[4 * j + 2 * hf] = prmt(v, 0u, sel); out[4 * j + 2 * hf + 1] = prmt(v, 0u, sel >> 16);
+      }
+    }
+  }
+}
+
+// Weights to shared memory, 16 bytes a lane and instruction; a group per slot of a ring.
+__device__ __forceinline__ void cp16(uint32_t dst, const void* src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
+}
+__device__ __forceinline__ void cp_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+// All but the PENDING newest groups have landed, for every lane of the warp.
+template <int PENDING>
+__device__ __forceinline__ void cp_wait() {
+  asm volatile("cp.async.wait_group %0;" ::"n"(PENDING) : "memory");
+  __syncwarp();
+}
+// BYTES (a multiple of 16) by a warp.
+template <int BYTES>
+__device__ __forceinline__ void cp_block(uint32_t dst, const uint8_t* src, int lane) {
+#pragma unroll
+  for (int o = 0; o < BYTES; o += 512)
+    if (o + 512 <= BYTES || o + lane * 16 < BYTES) cp16(dst + o + lane * 16, src + o + lane * 16);
+}
+
+// A warp's ring of packed weights: slots of one unit (a blob, or one tile where there are no scales), one group of copies each.
+template <int FMT> constexpr int tm_tiles = fmt_quantised(FMT) ? 2 : 1;        // tiles of a unit
+__host__ __device__ constexpr int tm_unit_most(int fmt) { return fmt == FMT_NONE ? 0 : fmt_quantised(fmt) ? blob_bytes(fmt, 1) : tile_bytes(fmt); }
+__host__ __device__ constexpr int tm_slots(int fmt) { return tm_unit_most(fmt) <= 1536 ? 4 : 2; }      // (16 warps: 68 KB of 4-bit weights, 64 KB of fp16 in flight)
+__host__ __device__ constexpr int tm_ring(int fmt) { return tm_slots(fmt) * tm_unit_most(fmt); }
+
+// The counterpart of dequant_part: the same units, in the same order.  `tile`: row tile of the CTA's 256 weight rows.  ring: the warp's ring.  The loop
+// is bound by its instructions (130 a tile took 907 cycles per k-block of 256 rows, of which the arithmetic is 150), so it carries nothing that could be
+// worked out before.
+template <int FMT>
+__device__ __forceinline__ bool dequant_part_tm(const WMat& mat, int n0, int kb_lo, int kb_hi, int it0, int tile, int phase, int step, int lane,
+                                                const PrefillArgs& p, uint32_t ring, uint32_t tmem_a, uint64_t* full_w, uint64_t* empty_w) {
+  if constexpr (FMT == FMT_NONE) {
+    return true;
+  } else {
+    constexpr int U = tm_tiles<FMT>, D = tm_slots(FMT), tb = tile_bytes(FMT);
+    constexpr bool quant = fmt_quantised(FMT);
+    constexpr int kUnit = quant ? blob_bytes(FMT, 0) : tb;
+    const int rt = (n0 >> 4) + tile;
+    const bool active = rt < mat.nt;                     // (else: rows past the matrix, zeros keep the operand finite)
+    const bool two = quant && mat.sz2 != 0;
+    const uint32_t unit_b = quant ? (uint32_t)mat.blob : (uint32_t)tb, ring_b = D * unit_b;
+    const int u_lo = kb_lo / U + phase, u_hi = kb_hi / U;
+    // the next unit to ask for, and where it is; where the second half of the pairs begins, it is elsewhere
+    int u_next = active ? u_lo : u_hi;
+    const uint8_t* next = wmat_blob(mat, rt, u_next * U / 2) + (U == 1 ? (u_next & 1) * tb : 0);
+    const int64_t to_second = wmat_blob(mat, rt, mat.half) - (wmat_blob(mat, rt, 0) + (int64_t)mat.half * mat.blob);
+    int cross = u_next * U / 2 < mat.half ? 2 * mat.half / U : 0x7fffffff;
+    const int stride = U == 1 ? (step == 2 ? mat.blob : tb) : step * mat.blob;      // (two tiles of an unquantised blob are contiguous, and so are its blobs)
+    auto ask = [&](uint32_t to) {
+      if (u_next < u_hi) {
+        if (u_next >= cross) { next += to_second; cross = 0x7fffffff; }
+        cp_block<kUnit>(to, next, lane);
+        if (two && lane < kSzEntryBytes / 16) cp16(to + kUnit + lane * 16, next + kUnit + lane * 16);
+        u_next += step;
+        next += stride;
+      }
+      cp_commit();                                       // (also if there is nothing left: the count of groups stays in step)
+    };
+#pragma unroll 1
+    for (uint32_t o = 0; o < ring_b; o += unit_b) ask(ring + o);
+    const uint32_t sz_at = 2 * tb + 4 * (lane >> 2), zz_at = 2 * tb + 32 + 2 * (lane >> 2);
+    const int stages = p.sw;
+    const uint32_t cols = p.a_cols;
+    int s = (it0 + phase * U) % stages;
+    uint32_t ph = (uint32_t)((it0 + phase * U) / stages) & 1u;
+    uint32_t full = smem_u32(full_w) + 8 * s, empty = smem_u32(empty_w) + 8 * s, at = tmem_a + s * cols;      // of stage s
+    auto advance = [&](int by) {
+      s += by; full += 8 * by; empty += 8 * by; at += by * cols;
+      if (s >= stages) { s -= stages; full -= 8 * stages; empty -= 8 * stages; at -= stages * cols; ph ^= 1u; }
+    };
+    const bool traced = p.trace && blockIdx.x == 0 && tile == 0 && lane == 0;
+    int it = it0 + phase * U;
+    // A tile is handed over when the next one has been dequantised: by then its way to tensor memory, some hundred cycles, is over.
+    uint32_t sent = 0;                                   // its stage's barrier, 0: none
+    auto hand_over = [&]() {
+      asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+      asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+      __syncwarp();
+      if (lane == 0 && sent) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(sent) : "memory");
+    };
+    uint32_t so = 0;                                     // slot of the unit
+    bool ok = true;
+#pragma unroll 1
+    for (int u = u_lo; u < u_hi; u += step) {
+      cp_wait<D - 1>();
+      const uint32_t src = ring + so;
+      ZC zc;
+      uint32_t s_a = 0u, s_b = 0u;
+#pragma unroll
+      for (int c = 0; c < U; ++c) {
+        uint32_t out[16];
+        if (active) {
+          if constexpr (quant) {
+            if (c == 0 || two) {
+              const uint32_t sc2 = lds_u1(src + sz_at + (c ? kSzEntryBytes : 0)), zz = lds_u16(src + zz_at + (c ? kSzEntryBytes : 0));
+              s_a = prmt(sc2, 0u, 0x1010u); s_b = prmt(sc2, 0u, 0x3232u);
+              make_zc_p<FMT>(zc, zz);
+            }
+          }
+          tm_tile<FMT>(src + c * tb, lane, zc, s_a, s_b, out);
+        } else {
+#pragma unroll
+          for (int i = 0; i < 16; ++i) out[i] = 0u;
+        }
+        hand_over();
+        if (!__all_sync(0xffffffffu, mbar_try_wait_a(empty, ph ^ 1u)) && !mbar_wait_warp_fast(empty_w + s, ph ^ 1u, p.dev_status, lane)) { ok = false; break; }
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        tmem_st16x32(at, out);
+        sent = full;
+        if (traced) p.trace[it * 4 + 1] = clock64();
+        it += c + 1 < U ? 1 : step * U - U + 1;
+        advance(c + 1 < U ? 1 : step * U - U + 1);       // (by at most 3 <= stages)
+      }
+      if (!ok) break;
+      __syncwarp();                                      // every lane has read the slot
+      ask(src);
+      so += unit_b;
+      if (so == ring_b) so = 0;
+    }
+    if (ok) hand_over();
+    else cp_wait<0>();                                   // gave up: what is in flight lands first
+    return ok;
+  }
+}
+
+// TM: the dequantised weights go to tensor memory instead of shared memory.
+template <int WF, int BF, bool TM>
 __global__ void __launch_bounds__(kThreadsP, 1) k_prefill(const __grid_constant__ CUtensorMap tm_x,
                                                           const __grid_constant__ CUtensorMap tm_t,
                                                           const __grid_constant__ CUtensorMap tm_x_small,
@@ -461,10 +681,14 @@ __global__ void __launch_bounds__(kThreadsP, 1) k_prefill(const __grid_constant_
   const uint32_t xbytes = (uint32_t)bt * 128;               // bytes of a token tile; the ring's slots are p.bt * 128 apart
   const uint32_t xslot = (uint32_t)p.bt * 128;
 
-  if constexpr (WF == FMT_SQ4) {
+  if constexpr (WF == FMT_SQ4 && !TM) {
     if (threadIdx.x >= 32 && threadIdx.x < 48) sp_lut[threadIdx.x - 32] = sp24_selectors(threadIdx.x - 32);
   }
   const uint32_t lut = smem_u32(sp_lut);
+  if (threadIdx.x == 96) {                                  // (their first use would pay for a trip to L2)
+    asm volatile("prefetch.tensormap [%0];" ::"l"(map_x) : "memory");
+    if (nkb_ext > 0) asm volatile("prefetch.tensormap [%0];" ::"l"(map_t) : "memory");
+  }
   if (threadIdx.x == 0) {
     PTRACE(nkb, 0);
     fail_s = 0;
@@ -483,6 +707,14 @@ __global__ void __launch_bounds__(kThreadsP, 1) k_prefill(const __grid_constant_
   const uint32_t tmem_d = tmem_base_s;
   if (threadIdx.x == 0) PTRACE(nkb, 1);
 
+  if constexpr (TM && BF != FMT_NONE) {                     // the CTA's blobs of B towards L2: they are needed at once, at the end
+    if (warp == 3 && nkb_ext > 0) {
+      const int t_lo = n0 >> 4, t_n = min(8 * nh, p.b.nt - t_lo);
+      const uint8_t* src = wmat_blob(p.b, t_lo, 0);
+      const int64_t bytes = (int64_t)t_n * p.b.np * p.b.blob;
+      for (int64_t o = (int64_t)lane << 13; o < bytes; o += 32 << 13) prefetch_l2(src + o, (uint32_t)(bytes - o < 8192 ? bytes - o : 8192));
+    }
+  }
   if (warp == 0) {
     // ------------------------------------------------------------------ TMA producer (token tiles)
     if (lane == 0) {
@@ -532,8 +764,12 @@ __global__ void __launch_bounds__(kThreadsP, 1) k_prefill(const __grid_constant_
           // half j / 4 of the weight rows is 128 rows = 16 KB further (+1024 in the address field), each K step of
           // 16 fp16 is 32 bytes further (+2)
           if (j < 4 * nh)
-            umma_f16(tmem_d + (j >> 2) * 256, adesc + (uint64_t)((j >> 2) * ((BN_W * 128) >> 4) + 2 * (j & 3)), bdesc + 2 * (j & 3),
-                     idesc, (it > 0 || (j & 3) > 0) ? 1u : 0u);
+            if constexpr (TM)                           // (16 reduction elements are 8 columns)
+              umma_f16_ts(tmem_d + (j >> 2) * p.acc_cols, tmem_d + p.a_col0 + sw * p.a_cols + (j >> 2) * 32 + 8 * (j & 3), bdesc + 2 * (j & 3),
+                          idesc, (it > 0 || (j & 3) > 0) ? 1u : 0u);
+            else
+              umma_f16(tmem_d + (j >> 2) * 256, adesc + (uint64_t)((j >> 2) * ((BN_W * 128) >> 4) + 2 * (j & 3)), bdesc + 2 * (j & 3),
+                       idesc, (it > 0 || (j & 3) > 0) ? 1u : 0u);
         }
         umma_commit_a(empty0 + 8 * sw);             // arrives when these MMAs have finished reading their operands
         PTRACE(it, 3);
@@ -546,7 +782,16 @@ __global__ void __launch_bounds__(kThreadsP, 1) k_prefill(const __grid_constant_
     // ------------------------------------------------------------------ dequant warps, then epilogue
     const int dw = warp - 4;
     bool ok = true;
-    {
+    if constexpr (TM) {
+      // A warp writes to the quarter of the lanes that its number selects: row tiles 2 (warp % 4) and the next one of each half.  Two halves: one
+      // row tile per warp; one half: two warps per row tile, alternating units.
+      const int q = dw >> 2, kstep = 3 - nh, kphase = nh == 2 ? 0 : q >> 1;
+      const int in_half = 2 * (dw & 3) + (q & 1), hh = nh == 2 ? q >> 1 : 0, tile = hh * 8 + in_half;
+      const uint32_t ring = smem_u32(smem + p.w_off) + (uint32_t)(dw * p.w_slot);
+      const uint32_t tmem_a = tmem_d + ((uint32_t)(in_half * 16) << 16) + p.a_col0 + hh * 32;
+      ok = dequant_part_tm<WF>(p.w, n0, kw_lo, kw_hi, 0, tile, kphase, kstep, lane, p, ring, tmem_a, full_w, empty_w);
+      if (ok && nkb_ext > 0) ok = dequant_part_tm<BF>(p.b, n0, 0, nkb_ext, nkw, tile, kphase, kstep, lane, p, ring, tmem_a, full_w, empty_w);
+    } else {
       // two halves: one row tile per warp; one half: two warps per row tile, alternating k-blocks
       const int kstep = 3 - nh, tile = nh == 2 ? dw : (dw & 7), kphase = nh == 2 ? 0 : (dw >> 3);
       ok = dequant_part<WF>(p.w, n0, kw_lo, kw_hi, 0, tile, kphase, kstep, lane, smem, p, full_w, empty_w, lut);
@@ -567,6 +812,7 @@ __global__ void __launch_bounds__(kThreadsP, 1) k_prefill(const __grid_constant_
   const int nl = lq * 32 + lane;                         // local weight row inside the half = thread index inside the group
   const int nchunk = (bt + 31) >> 5, units = nh * nchunk;
   const uint32_t lane_base = tmem_d + ((uint32_t)(lq * 32) << 16);
+  const uint32_t acc_cols = TM ? (uint32_t)p.acc_cols : 256u;
   const uint32_t parts = smem_u32(smem) + 65536;         // split: the other CTAs' shares of this CTA's units, 16 KB each
   const bool out16 = p.out_dtype != EORA_Y_F32;
   // A unit's accumulators: for a 16-bit Y as fragments of 8 x 8 blocks, for a float Y one row of W per lane (32 tokens).
@@ -588,7 +834,7 @@ __global__ void __launch_bounds__(kThreadsP, 1) k_prefill(const __grid_constant_
       if (owner == split) continue;
       const int hh = u / nchunk, c0 = (u - hh * nchunk) * 32;
       uint32_t v[32];
-      load_unit(lane_base + hh * 256 + (uint32_t)c0, v);
+      load_unit(lane_base + hh * acc_cols + (uint32_t)c0, v);
       const int slot = (u / p.ksplit) * (p.ksplit - 1) + (split < owner ? split : split - 1);
       const uint32_t to = mapa(parts + slot * 16384 + nl * 16, (uint32_t)owner);      // (the same thread of the owner adds it to the same registers)
 #pragma unroll
@@ -614,7 +860,7 @@ __global__ void __launch_bounds__(kThreadsP, 1) k_prefill(const __grid_constant_
       const uint32_t tbuf = gbuf + flip * 16384;
       if (p.ksplit == 1) flip ^= 1;
       uint32_t v[32];
-      load_unit(lane_base + hh * 256 + (uint32_t)c0, v);
+      load_unit(lane_base + hh * acc_cols + (uint32_t)c0, v);
       for (int q = 0; q < p.ksplit - 1; ++q) {
         const uint32_t src = parts + (i * (p.ksplit - 1) + q) * 16384 + nl * 16;
 #pragma unroll
@@ -742,15 +988,20 @@ cudaError_t launch_p(dim3 grid, int smem, cudaStream_t st, const CUtensorMap& tx
   return cudaLaunchKernelEx(&cfg, KERNEL, tx, tt, txs, tts, a);
 }
 
+template <int WF, int BF>
+cudaError_t launch_tm(dim3 grid, int smem, cudaStream_t st, const CUtensorMap& tx, const CUtensorMap& tt, const CUtensorMap& txs, const CUtensorMap& tts,
+                      const PrefillArgs& a) {
+  return a.a_cols ? launch_p<k_prefill<WF, BF, true>>(grid, smem, st, tx, tt, txs, tts, a) : launch_p<k_prefill<WF, BF, false>>(grid, smem, st, tx, tt, txs, tts, a);
+}
 template <int WF>
 cudaError_t launch_bf(int bf, dim3 grid, int smem, cudaStream_t st, const CUtensorMap& tx, const CUtensorMap& tt,
                       const CUtensorMap& txs, const CUtensorMap& tts, const PrefillArgs& a) {
   switch (bf) {
-    case FMT_F16: return launch_p<k_prefill<WF, FMT_F16>>(grid, smem, st, tx, tt, txs, tts, a);
-    case FMT_Q4: return launch_p<k_prefill<WF, FMT_Q4>>(grid, smem, st, tx, tt, txs, tts, a);
-    case FMT_Q8: return launch_p<k_prefill<WF, FMT_Q8>>(grid, smem, st, tx, tt, txs, tts, a);
-    case FMT_Q3: return launch_p<k_prefill<WF, FMT_Q3>>(grid, smem, st, tx, tt, txs, tts, a);
-    default: return launch_p<k_prefill<WF, FMT_NONE>>(grid, smem, st, tx, tt, txs, tts, a);
+    case FMT_F16: return launch_tm<WF, FMT_F16>(grid, smem, st, tx, tt, txs, tts, a);
+    case FMT_Q4: return launch_tm<WF, FMT_Q4>(grid, smem, st, tx, tt, txs, tts, a);
+    case FMT_Q8: return launch_tm<WF, FMT_Q8>(grid, smem, st, tx, tt, txs, tts, a);
+    case FMT_Q3: return launch_tm<WF, FMT_Q3>(grid, smem, st, tx, tt, txs, tts, a);
+    default: return launch_tm<WF, FMT_NONE>(grid, smem, st, tx, tt, txs, tts, a);
   }
 }
 
@@ -762,13 +1013,32 @@ cudaError_t launch_any(int wf, int bf, dim3 grid, int smem, cudaStream_t st, con
     case FMT_SP24: return launch_bf<FMT_SP24>(bf, grid, smem, st, tx, tt, txs, tts, a);
     case FMT_SQ4: return launch_bf<FMT_SQ4>(bf, grid, smem, st, tx, tt, txs, tts, a);
     // A as the weight of the first launch (t = X.A): no K-extension there
-    case FMT_F16: return launch_p<k_prefill<FMT_F16, FMT_NONE>>(grid, smem, st, tx, tt, txs, tts, a);
-    case FMT_Q8: return launch_p<k_prefill<FMT_Q8, FMT_NONE>>(grid, smem, st, tx, tt, txs, tts, a);
+    case FMT_F16: return launch_tm<FMT_F16, FMT_NONE>(grid, smem, st, tx, tt, txs, tts, a);
+    case FMT_Q8: return launch_tm<FMT_Q8, FMT_NONE>(grid, smem, st, tx, tt, txs, tts, a);
     default: return cudaErrorInvalidValue;
   }
 }
 
+// Weights in tensor memory: beside the accumulators there is room for at least kTmLeast stages of the tile's weights.
+constexpr int kTmLeast = 3;
+bool tm_fits(int rows, int bt) { return rows / BN_W * (bt + kTmLeast * 32) <= 512; }
+
 int fill_stages(PrefillArgs& a) {      // returns the dynamic shared memory to request
+  if (tm_fits(a.rows, a.bt)) {
+    const int nh = a.rows / BN_W;
+    a.acc_cols = a.bt; a.a_col0 = nh * a.bt; a.a_cols = 32 * nh;
+    // stages as tensor memory has room for, if the warps' rings fit beside their token tiles
+    const int w_ring = tm_ring(a.w.fmt), b_ring = tm_ring(a.b.fmt);
+    a.w_slot = w_ring > b_ring ? w_ring : b_ring;
+    a.sw = (512 - a.a_col0) / a.a_cols;
+    if (a.sw > kMaxWStages) a.sw = kMaxWStages;
+    while (a.sw > kTmLeast && a.sw * a.bt * 128 + kDqWarps * a.w_slot > kSmemP - 1024) --a.sw;
+    a.w_off = a.sw * a.bt * 128;
+    const int smem = a.w_off + kDqWarps * a.w_slot, units = nh * ((a.bt + 31) / 32);
+    const int out = a.ksplit > 1 ? 65536 + (units + a.ksplit - 1) / a.ksplit * (a.ksplit - 1) * 16384 : 131072;      // the epilogue's
+    return (out > smem ? out : smem) + 1024;
+  }
+  a.a_cols = 0;
   a.w_slot = a.rows * 128;
   const int stage = a.bt * 128 + a.w_slot;             // token tile + weight tile of one k-block
   a.sw = (kSmemP - 1024) / stage;
@@ -791,11 +1061,12 @@ bool split_fits(int rows, int bt, int ks) {
 // CTAs of clusters of ks that run at once, one per SM (measured: 74 clusters of two, 33 of four, 15 of eight; 148 SMs).
 int at_once(int ks, int sm_count) { return ks == 1 ? sm_count : ks == 2 ? sm_count / 2 * 2 : ks == 4 ? sm_count * 33 / 148 * 4 : sm_count * 15 / 148 * 8; }
 
-// Cycles of a k-block: the dequantisation of the CTA's rows bounds it whatever the tokens (128 rows 525, 256 rows 1030; measured with
-// 64 to 512 tokens) up to 192 of them.  With 256 the eight MMAs of 256 rows alone take 1024 (1150 in all), and the token tiles of
-// 128 rows come close to what L2 delivers (600 in one wave, 740 when the SMs are full throughout several).
+// Cycles of a k-block, measured with 64 to 256 tokens.  Weights in tensor memory: 128 rows 515 whatever the tokens, 256 rows 790, which is as long as
+// sixteen warps take to dequantise them.  Through shared memory, where the accumulators leave no room: 256 rows 1100, and with 256 tokens, whose eight MMAs
+// alone take 1024, 1150.  Many tokens come close to what L2 delivers when the SMs are full throughout several waves (128 rows x 256 tokens: 740).
 float kblock_cycles(const Tiling& t, bool one_wave) {
-  return t.rows == BN_W ? (t.bt <= 192 ? 525.f : one_wave ? 600.f : 740.f) : (t.bt <= 192 ? 1030.f : 1150.f);
+  if (t.rows == BN_W) return one_wave || t.bt <= 176 ? (t.bt <= 224 ? 515.f : 540.f) : 2.9f * (float)t.bt;
+  return tm_fits(t.rows, t.bt) ? 790.f : t.bt <= 192 ? 1100.f : 1150.f;
 }
 // Estimated cycles of a launch: its k-blocks, set-up and first operands 3200, the epilogue 900 and 5000 per 256 x 256 of the tile; sharing a
 // reduction axis costs two cluster barriers and the way of the tile's sums through distributed shared memory, 1000 + 1600 per
@@ -826,8 +1097,10 @@ template <typename F>
 void each_tiling(int n_rows, int m, int nkb_w, int sm_count, bool only128, F f) {
   // Even tiles up to 1024 tokens, whole ones beyond.  Beyond, even ones are 1 to 3 % faster up to 1100 tokens (4096 x 14336 at 1025: 103.3 against
   // 106.9 us), within 2 % from there on and 5 % slower at 1800 to 1900 of that shape (198.9 against 188.4).
-  const int bt = m > 1024 ? 256 : token_tile(m, 256);
-  for (int rows = BN_W; rows <= (only128 ? BN_W : 2 * BN_W); rows += BN_W)
+  // Or tiles of at most 160, where the weights of 256 rows fit into tensor memory.
+  const int wide = m > 1024 ? 256 : token_tile(m, 256), narrow = m > 1024 ? 256 : token_tile(m, 160);
+  for (int bt = wide; bt == wide || bt == narrow; bt = bt == narrow ? 0 : narrow)
+   for (int rows = BN_W; rows <= (only128 ? BN_W : 2 * BN_W); rows += BN_W)
     for (int ks = 1; ks <= 8 && (ks == 1 || (nkb_w / ks >= 4 && split_fits(rows, bt, ks))); ks *= 2)
       if (ks == 1 || (n_rows + rows - 1) / rows * ((m + bt - 1) / bt) * ks <= at_once(ks, sm_count)) f(Tiling{rows, bt, ks});
 }

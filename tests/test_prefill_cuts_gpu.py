@@ -53,3 +53,24 @@ def test_prefill_fused_calls_in_a_row(M):
         check_parity(ys[i].float().cpu().numpy().astype(np.float64), orc.forward(x2, "f16", *case), f"layer {i}")
     F.close()
     one.close()
+
+
+@pytest.mark.parametrize("w,ab,K,N,r,M,group", [
+    ("q4", "f16", 256, 38144, 64, 160, 128),   # 256 rows x 160 tokens: the accumulators leave tensor memory for three stages of weights
+    ("q4", "f16", 256, 38144, 64, 161, 128),   # one token more: narrower tiles, or the weights through shared memory
+    ("q4", "f16", 256, 38144, 64, 352, 128),
+    ("sp24", "q8", 384, 38144, 128, 64, 128),  # units of one tile (2:4) and of two (8-bit)
+    ("q3", "q3", 640, 18944, 256, 224, 128),   # 128 rows x 224 tokens
+    ("sq4", "q4", 256, 288, 64, 40, 128),      # row tiles past the matrix
+    ("q4", "f16", 128, 2048, 64, 34, 128),     # fewer units than a warp's ring has slots
+    ("q4", "f16", 640, 544, 64, 50, 64),       # a scale entry per tile
+    ("q3", "q8", 4096, 2176, 512, 100, 64),    # clusters; the halves of the reduction axis; rings that go round
+])
+def test_prefill_weights_in_tensor_memory(w, ab, K, N, r, M, group):
+    """Where the dequantised weights go to tensor memory and where they do not: tiles of weight rows and tokens around the limit, rows past the
+    matrix, rings that are not filled and rings that go round, both sizes of a unit of work, one or two scale entries."""
+    wf, af, bf = make_case(77, K, N, r, w=w, ab=ab, group=group)
+    x = gen.make_x(78, M, K, "f16")
+    L = eora.Layer(wf, af, bf, max_m=M)
+    check_parity(run_layer(L, x, "f16"), orc.forward(x, "f16", wf, af, bf), f"{w}/{ab} K{K} N{N} r{r} M{M}")
+    L.close()
