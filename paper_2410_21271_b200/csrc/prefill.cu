@@ -13,7 +13,7 @@
 //     the dequantised weight tile;
 //   * an elected lane of one warp issues tcgen05.mma (M = 128, N = tokens, K = 16) with the fp32 accumulator in
 //     tensor memory; tcgen05.commit releases the ring slots when the MMAs have drained;
-//   * where whole tiles would leave SMs idle, a cluster of two, four or eight CTAs shares a tile's reduction axis and
+//   * where whole tiles would leave SMs idle, a cluster of two to eight CTAs shares a tile's reduction axis and
 //     adds its parts through distributed shared memory (pick_tilings chooses tile and cluster for both launches);
 //   * the low-rank term is a K-extension: after the d_in/64 backbone k-blocks come r/64 k-blocks whose
 //     token operand is t = X.A (fp16, from a first launch of the same kernel with A as the weight) and
@@ -25,6 +25,7 @@
 // when X is bf16 (the f16 MMA kind needs both operands in fp16; weights are kept fp16 because
 // bf16 weights alone cost 1.7e-3 of the 2e-3 error budget).
 #include <cuda.h>
+#include <math.h>
 #include "decode_common.cuh"
 
 namespace eora {
@@ -1058,8 +1059,11 @@ bool split_fits(int rows, int bt, int ks) {
   const int units = rows / BN_W * ((bt + 31) / 32);
   return 65536 + (units + ks - 1) / ks * (ks - 1) * 16384 <= kSmemP - 1024;
 }
-// CTAs of clusters of ks that run at once, one per SM (measured: 74 clusters of two, 33 of four, 15 of eight; 148 SMs).
-int at_once(int ks, int sm_count) { return ks == 1 ? sm_count : ks == 2 ? sm_count / 2 * 2 : ks == 4 ? sm_count * 33 / 148 * 4 : sm_count * 15 / 148 * 8; }
+// CTAs of clusters of ks that run at once, one per SM (the occupancy calculator's figures for 148 SMs; of seven only 15 clusters).
+int at_once(int ks, int sm_count) {
+  constexpr int clusters[9] = {0, 148, 74, 45, 33, 26, 22, 15, 15};
+  return sm_count * clusters[ks] / 148 * ks;
+}
 
 // Cycles of a k-block, measured with 64 to 256 tokens.  Weights in tensor memory: 128 rows 515 whatever the tokens, 256 rows 790, which is as long as
 // sixteen warps take to dequantise them.  Through shared memory, where the accumulators leave no room: 256 rows 1100, and with 256 tokens, whose eight MMAs
@@ -1077,9 +1081,11 @@ float tiling_cost(const Tiling& t, int n_rows, int m, int nkb, int sm_count) {
   float waves = (float)((ctas + cap - 1) / cap);
   const int over = tiles % sm_count;
   if (t.ks == 1 && t.rows == 2 * BN_W && t.bt == 256 && tiles > sm_count && over > 0 && 4 * over <= sm_count) waves -= 0.5f;
-  const float area = (float)(t.rows * t.bt) / 65536.f, doublings = t.ks == 1 ? 0.f : t.ks == 2 ? 1.f : t.ks == 4 ? 2.f : 3.f;
+  const float area = (float)(t.rows * t.bt) / 65536.f, doublings = log2f((float)t.ks);
+  // Three, five, six or seven CTAs deal a tile's units unevenly (q|k|v at 100 tokens with five 21.4 us, with two CTAs of half the rows 19.5, estimated 4 % slower).
+  const float uneven = t.ks & (t.ks - 1) ? 2500.f : 0.f;
   return waves * ((float)((nkb + t.ks - 1) / t.ks) * kblock_cycles(t, ctas <= cap) + 4100.f + 5000.f * area +
-                  (t.ks > 1 ? 1000.f + 1600.f * doublings + 5500.f * area : 0.f));
+                  (t.ks > 1 ? 1000.f + 1600.f * doublings + 5500.f * area + uneven : 0.f));
 }
 
 int token_tile(int m, int most) {      // the MMA N: a multiple of 16 up to `most`, even tiles
@@ -1101,8 +1107,8 @@ void each_tiling(int n_rows, int m, int nkb_w, int sm_count, bool only128, F f) 
   const int wide = m > 1024 ? 256 : token_tile(m, 256), narrow = m > 1024 ? 256 : token_tile(m, 160);
   for (int bt = wide; bt == wide || bt == narrow; bt = bt == narrow ? 0 : narrow)
    for (int rows = BN_W; rows <= (only128 ? BN_W : 2 * BN_W); rows += BN_W)
-    for (int ks = 1; ks <= 8 && (ks == 1 || (nkb_w / ks >= 4 && split_fits(rows, bt, ks))); ks *= 2)
-      if (ks == 1 || (n_rows + rows - 1) / rows * ((m + bt - 1) / bt) * ks <= at_once(ks, sm_count)) f(Tiling{rows, bt, ks});
+    for (int ks = 1; ks <= 8 && (ks == 1 || nkb_w / ks >= 4); ++ks)
+      if (ks == 1 || (split_fits(rows, bt, ks) && (n_rows + rows - 1) / rows * ((m + bt - 1) / bt) * ks <= at_once(ks, sm_count))) f(Tiling{rows, bt, ks});
 }
 Tilings pick_tilings(int n_rows, int t_cols, int m, int nkb_w, int nkb_b, int sm_count, bool only128) {
   Tilings best = {};
