@@ -432,8 +432,8 @@ __device__ __forceinline__ bool dequant_part(const WMat& mat, int n0, int kb_lo,
 // ---------------------------------------------------------------------------------------------- weights in tensor memory
 // Up to 160 tokens (256 with 128 rows) the accumulators leave tensor memory for the dequantised weights.  Through shared memory a k-block of 256 rows x
 // 64 tokens moved 32 KB of weights in and out of it, 512 cycles of its bandwidth, and each hand-over waited for the stores to become visible to the
-// MMAs (1215 cycles a k-block); here the weights go from registers to tensor memory and the MMAs read only the tokens from shared memory (790).  Three
-// LLaMA3-8B blocks of 64 tokens, 4-bit, 8-bit adapters of rank 512: 419 -> 358 us; a block of 128 tokens 124 -> 105, of a prompt of 333 232 -> 214.
+// MMAs (1215 cycles a k-block); here the weights go from registers to tensor memory and the MMAs read only the tokens from shared memory (790).  A 4-bit
+// LLaMA3-8B block of 64 tokens with 8-bit adapters of rank 512: 139 -> 114 us; of 128 tokens, rank 128, 124 -> 105; of a prompt of 333 235 -> 204.
 // Tried and not kept: two chains of MMAs with accumulators of their own (128 rows 515 -> 562 cycles).
 //
 // tcgen05.st writes a tile of 16 rows x 64 reduction elements as fragments of 8 x 8 32-bit blocks: lane (g, t) holds, for each of the four MMAs j of a
@@ -1083,7 +1083,7 @@ float tiling_cost(const Tiling& t, int n_rows, int m, int nkb, int sm_count) {
   if (t.ks == 1 && t.rows == 2 * BN_W && t.bt == 256 && tiles > sm_count && over > 0 && 4 * over <= sm_count) waves -= 0.5f;
   const float area = (float)(t.rows * t.bt) / 65536.f, doublings = log2f((float)t.ks);
   // Three, five, six or seven CTAs deal a tile's units unevenly (q|k|v at 100 tokens with five 21.4 us, with two CTAs of half the rows 19.5, estimated 4 % slower).
-  const float uneven = t.ks & (t.ks - 1) ? 2500.f : 0.f;
+  const float uneven = t.ks & (t.ks - 1) ? 2000.f : 0.f;
   return waves * ((float)((nkb + t.ks - 1) / t.ks) * kblock_cycles(t, ctas <= cap) + 4100.f + 5000.f * area +
                   (t.ks > 1 ? 1000.f + 1600.f * doublings + 5500.f * area + uneven : 0.f));
 }
@@ -1123,7 +1123,8 @@ Tilings pick_tilings(int n_rows, int t_cols, int m, int nkb_w, int nkb_b, int sm
       const float ct = tiling_cost(t, t_cols, m, nkb_w, sm_count), tail = (float)nkb_b * kblock_cycles(a, true);
       const int tc = ctas_of(t, t_cols), one_wave = ctas <= at_once(a.ks, sm_count);
       const bool beside = one_wave && ctas + tc <= at_once(a.ks > t.ks ? a.ks : t.ks, sm_count);
-      take(t, beside ? (cm > ct + tail ? cm : ct + tail) : one_wave ? cm + ct : cm + ct * (float)tc / (float)sm_count);
+      // (of equal ones the earlier t: three blocks of 64 tokens with adapters of rank 512, down 31.6 -> 28.6 us)
+      take(t, 0.02f * ct + (beside ? (cm > ct + tail ? cm : ct + tail) : one_wave ? cm + ct : cm + ct * (float)tc / (float)sm_count));
     });
   });
   return best;
