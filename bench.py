@@ -514,7 +514,8 @@ def time_solve(device: str, d: int = 4096, k: int = 4096, n: int = 2048, r: int 
     loss = eora.solve_loss(tw, th, tx, b, a)
     uncompensated = float(torch.linalg.norm((tw - th).double() @ tx.double()))
     out = {"workload": f"one layer {d}x{k}, {n} calibration columns, rank {r}", "ms": ms, "layers_per_s": 1e3 / ms,
-           "gflop": flops / 1e9, "tflops": flops / ms / 1e9, "bound": "alu", "peak_tflops_fp32": FP32_PEAK_TFLOPS,
+           "gflop": flops / 1e9, "tflops": flops / ms / 1e9, "bound": "latency", "peak_tflops_fp32": FP32_PEAK_TFLOPS,
+           "products": "fp32 accuracy, large ones as three bf16 parts per value on the tensor cores: not bounded by the fp32 FMA peak",
            "frac_of_fp32_peak": flops / ms / 1e9 / FP32_PEAK_TFLOPS,
            "remaining_loss_over_uncompensated": loss / uncompensated, "dtype": "f32 (f64 for the small problems)"}
     # Independent layers (q, k, v share one input; gate and up another) can be solved side by side: each solve is a
