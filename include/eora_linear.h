@@ -242,6 +242,20 @@ int eora_linear_decode_grid(eora_linear_t h, int32_t m);
 int eora_linear_set_trace(eora_linear_t h, void* trace_buf);
 
 /*
+ * Diagnostics: the tiles that the tensor-core family for more than 32 tokens (9 to 32 where a layer does not fit the kernel for
+ * those) gives a forward(m) of n_layers (1: a plain layer, 2..4: a fused group) on a GPU of sm_count SMs.  Host arithmetic only: no device
+ * is needed.  out[0]: the main product, out[1]: t = X.A (zeros without an adapter).  EORA_ERR_UNSUPPORTED: this family does not serve them.
+ */
+typedef struct {
+  int32_t rows, tokens;       /* weight rows and tokens of a tile */
+  int32_t cluster;            /* CTAs that share a tile's reduction axis */
+  int32_t stages;             /* k-blocks in the ring */
+  int32_t in_tensor_memory;   /* 1: the dequantised weights go through tensor memory, 0: through shared memory */
+  int32_t longest_step;       /* k-blocks from one that a dequantising warp takes to the next it takes, at most: never more than `stages` */
+} eora_prefill_tiling;
+int eora_linear_prefill_plan(const eora_linear_config* cfgs, int32_t n_layers, int32_t m, int32_t sm_count, eora_prefill_tiling* out);
+
+/*
  * The same layer for callers that cannot allocate device memory.  (The paper has no counterpart:
  * this is a deployment convenience of the library.)
  *

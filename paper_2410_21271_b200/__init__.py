@@ -36,6 +36,10 @@ class eora_linear_weights(Structure):
                                         "b", "b_scales", "b_zeros", "w_meta")]
 
 
+class eora_prefill_tiling(Structure):
+    _fields_ = [(n, c_int32) for n in ("rows", "tokens", "cluster", "stages", "in_tensor_memory", "longest_step")]
+
+
 class eora_solve_config(Structure):
     _fields_ = [("d", c_int32), ("k", c_int32), ("n", c_int32), ("rank", c_int32), ("oversample", c_int32), ("iters", c_int32)]
 
@@ -98,6 +102,8 @@ def lib() -> ctypes.CDLL:
         L.eora_linear_set_trace.restype = c_int
         L.eora_linear_decode_grid.argtypes = [c_void_p, c_int32]
         L.eora_linear_decode_grid.restype = c_int
+        L.eora_linear_prefill_plan.argtypes = [POINTER(eora_linear_config), c_int32, c_int32, c_int32, POINTER(eora_prefill_tiling)]
+        L.eora_linear_prefill_plan.restype = c_int
         L.eora_linear_forward_noalloc.argtypes = [POINTER(eora_linear_config), POINTER(eora_linear_weights), c_void_p,
                                                   c_int32, c_void_p, c_void_p]
         L.eora_linear_forward_noalloc.restype = c_int
@@ -301,6 +307,16 @@ def eora_linear_set_trace(handle: int, buf) -> int:
 
 def eora_linear_decode_grid(handle: int, m: int) -> int:
     return lib().eora_linear_decode_grid(handle, int(m))
+
+
+def eora_linear_prefill_plan(cfgs, m: int, sm_count: int = 148) -> list:
+    """Tiles of a forward of `cfgs` (one config, or those of a fused group) by the tensor-core family: [main product, t = X.A]."""
+    arr = (eora_linear_config * len(cfgs))(*cfgs)
+    out = (eora_prefill_tiling * 2)()
+    st = lib().eora_linear_prefill_plan(arr, len(cfgs), int(m), int(sm_count), out)
+    if st != EORA_OK:
+        raise EoraError(st, "eora_linear_prefill_plan")
+    return list(out)
 
 
 EORA_NOALLOC_MAX_T_ELEMS = 65536

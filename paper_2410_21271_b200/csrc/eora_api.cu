@@ -161,52 +161,20 @@ WMat pair_view(const WMat& m, int p0, int n_pairs) {
   return v;
 }
 
-// One backbone with n adapters (decode only): cfg is the layer's, wts[j] carries adapter j (the backbone
-// pointers are taken from wts[0]).
-int create_multi_impl(const eora_linear_config* cfg, const eora_linear_weights* wts, int n, void* stream, eora_linear_t* out);
-
-// One layer (n == 1) or n layers that share X, stacked along the output axis (fused).
-int create_impl(const eora_linear_config* cfgs, const eora_linear_weights* wts, int n, void* stream, eora_linear_t* out) {
-  if (out) *out = nullptr;
-  if (!cfgs || !wts || !out) return EORA_ERR_NULL_ARG;
-  if (n < 1 || n > 4) return EORA_ERR_BAD_SHAPE;
+// Layers that can be fused differ in d_out only.
+bool same_layer_kind(const eora_linear_config& ci, const eora_linear_config& c) {
+  return ci.d_in == c.d_in && ci.rank == c.rank && ci.w_format == c.w_format && ci.w_bits == c.w_bits && ci.w_group == c.w_group &&
+         ci.ab_format == c.ab_format && ci.ab_group == c.ab_group && ci.x_dtype == c.x_dtype && ci.y_dtype == c.y_dtype &&
+         ci.max_m == c.max_m && ci.kernel_policy == c.kernel_policy;
+}
+eora_linear_config joined_config(const eora_linear_config* cfgs, int n) {
   eora_linear_config c = cfgs[0];
-  int d_out_total = 0;
-  for (int i = 0; i < n; ++i) {
-    int st = check_config(cfgs[i]);
-    if (st != EORA_OK) return st;
-    st = check_weights(cfgs[i], wts[i]);
-    if (st != EORA_OK) return st;
-    const eora_linear_config& ci = cfgs[i];
-    if (ci.d_in != c.d_in || ci.rank != c.rank || ci.w_format != c.w_format || ci.w_bits != c.w_bits || ci.w_group != c.w_group ||
-        ci.ab_format != c.ab_format || ci.ab_group != c.ab_group || ci.x_dtype != c.x_dtype || ci.y_dtype != c.y_dtype ||
-        ci.max_m != c.max_m || ci.kernel_policy != c.kernel_policy)
-      return EORA_ERR_BAD_SHAPE;
-    d_out_total += ci.d_out;
-  }
-  const bool fused = n > 1;
-  if (fused && c.kernel_policy == EORA_POLICY_GENERIC) return EORA_ERR_UNSUPPORTED;
-  c.d_out = d_out_total;
-
-  eora_linear* obj = new (std::nothrow) eora_linear();
-  if (!obj) return EORA_ERR_CUDA;
-  Handle* h = &obj->h;
-  *h = Handle();
+  for (int i = 1; i < n; ++i) c.d_out += cfgs[i].d_out;
+  return c;
+}
+// The shapes of a handle of n layers: c is the layers' common config with all their outputs.
+void shape_handle(Handle* h, const eora_linear_config& c, const eora_linear_config* cfgs, int n) {
   h->cfg = c;
-  cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
-  auto fail = [&](int code) {
-    if (h->prefill_state) prefill_free(h);
-    if (h->tc_state) decode_tc_free(h);
-    if (h->stage_mem) cudaFree(h->stage_mem);
-    if (h->weight_mem) cudaFree(h->weight_mem);
-    if (h->scratch_mem) cudaFree(h->scratch_mem);
-    delete obj;
-    return code;
-  };
-  if (cudaGetDevice(&h->device) != cudaSuccess) return fail(EORA_ERR_CUDA);
-  if (cudaDeviceGetAttribute(&h->sm_count, cudaDevAttrMultiProcessorCount, h->device) != cudaSuccess) return fail(EORA_ERR_CUDA);
-
-  h->wait_limit_ns = 1000000000ull;
   h->r_pad = (int)align_up(c.rank, 128);
   h->n_sub = n;
   h->n_adapters = 1;
@@ -224,12 +192,53 @@ int create_impl(const eora_linear_config* cfgs, const eora_linear_weights* wts, 
   if (c.rank > 0) {
     int ga = ab_grouped ? c.ab_group : 0;
     int gb = ab_grouped ? (c.ab_group < c.rank ? c.ab_group : c.rank) : 0;
-    wmat_shape(h->a, ab_fmt, fused ? n * h->r_pad : c.rank, c.d_in, ga);   // fused: layer i owns rows [i r_pad, (i+1) r_pad)
+    wmat_shape(h->a, ab_fmt, n > 1 ? n * h->r_pad : c.rank, c.d_in, ga);   // fused: layer i owns rows [i r_pad, (i+1) r_pad)
     wmat_shape(h->b, ab_fmt, c.d_out, h->r_pad, gb);
   } else {
     wmat_shape(h->a, FMT_NONE, 0, 0, 0);
     wmat_shape(h->b, FMT_NONE, 0, 0, 0);
   }
+}
+
+// One backbone with n adapters (decode only): cfg is the layer's, wts[j] carries adapter j (the backbone
+// pointers are taken from wts[0]).
+int create_multi_impl(const eora_linear_config* cfg, const eora_linear_weights* wts, int n, void* stream, eora_linear_t* out);
+
+// One layer (n == 1) or n layers that share X, stacked along the output axis (fused).
+int create_impl(const eora_linear_config* cfgs, const eora_linear_weights* wts, int n, void* stream, eora_linear_t* out) {
+  if (out) *out = nullptr;
+  if (!cfgs || !wts || !out) return EORA_ERR_NULL_ARG;
+  if (n < 1 || n > 4) return EORA_ERR_BAD_SHAPE;
+  for (int i = 0; i < n; ++i) {
+    int st = check_config(cfgs[i]);
+    if (st != EORA_OK) return st;
+    st = check_weights(cfgs[i], wts[i]);
+    if (st != EORA_OK) return st;
+    if (!same_layer_kind(cfgs[i], cfgs[0])) return EORA_ERR_BAD_SHAPE;
+  }
+  const eora_linear_config c = joined_config(cfgs, n);
+  const bool fused = n > 1;
+  if (fused && c.kernel_policy == EORA_POLICY_GENERIC) return EORA_ERR_UNSUPPORTED;
+
+  eora_linear* obj = new (std::nothrow) eora_linear();
+  if (!obj) return EORA_ERR_CUDA;
+  Handle* h = &obj->h;
+  *h = Handle();
+  cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
+  auto fail = [&](int code) {
+    if (h->prefill_state) prefill_free(h);
+    if (h->tc_state) decode_tc_free(h);
+    if (h->stage_mem) cudaFree(h->stage_mem);
+    if (h->weight_mem) cudaFree(h->weight_mem);
+    if (h->scratch_mem) cudaFree(h->scratch_mem);
+    delete obj;
+    return code;
+  };
+  if (cudaGetDevice(&h->device) != cudaSuccess) return fail(EORA_ERR_CUDA);
+  if (cudaDeviceGetAttribute(&h->sm_count, cudaDevAttrMultiProcessorCount, h->device) != cudaSuccess) return fail(EORA_ERR_CUDA);
+
+  h->wait_limit_ns = 1000000000ull;
+  shape_handle(h, c, cfgs, n);
 
   // ---- weights: one allocation
   Carve sizing{nullptr, 0};
@@ -263,6 +272,7 @@ int create_impl(const eora_linear_config* cfgs, const eora_linear_weights* wts, 
   if (cudaMemsetAsync(h->scratch_mem, 0, (size_t)h->scratch_bytes, s) != cudaSuccess) return fail(EORA_ERR_CUDA);
 
   // ---- re-tile, layer by layer into its range of row tiles
+  const bool ab_grouped = c.ab_format == EORA_AB_Q4 || c.ab_format == EORA_AB_Q3;
   cudaError_t e = cudaSuccess;
   for (int i = 0; i < n && e == cudaSuccess; ++i) {
     const eora_linear_weights& w = wts[i];
@@ -677,6 +687,20 @@ int eora_linear_decode_grid(eora_linear_t obj, int32_t m) {
   if (decode_tc_supported(&obj->h, m)) return decode_tc_grid(&obj->h);
   if (multi_takes_mid(&obj->h, m)) return mid_grid(&obj->h, m);
   return decode_grid(&obj->h, m);
+}
+
+int eora_linear_prefill_plan(const eora_linear_config* cfgs, int32_t n_layers, int32_t m, int32_t sm_count, eora_prefill_tiling* out) {
+  if (!cfgs || !out) return EORA_ERR_NULL_ARG;
+  if (n_layers < 1 || n_layers > 4 || m < 9 || sm_count < 1) return EORA_ERR_BAD_SHAPE;
+  for (int i = 0; i < n_layers; ++i) {
+    const int st = check_config(cfgs[i]);
+    if (st != EORA_OK) return st;
+    if (!same_layer_kind(cfgs[i], cfgs[0])) return EORA_ERR_BAD_SHAPE;
+  }
+  Handle h = Handle();
+  h.sm_count = sm_count;
+  shape_handle(&h, joined_config(cfgs, n_layers), cfgs, n_layers);
+  return prefill_plan(&h, m, out);
 }
 
 int64_t eora_linear_weight_bytes(eora_linear_t obj) { return obj ? obj->h.weight_bytes + decode_tc_weight_bytes(&obj->h) : 0; }

@@ -265,5 +265,6 @@ cudaError_t prefill_init(Handle* h);
 void prefill_free(Handle* h);
 cudaError_t launch_prefill_forward(const Handle* h, const void* x, int m, void* const* ys, cudaStream_t st);
 int prefill_launch_count(const Handle* h, int m);
+int prefill_plan(const Handle* h, int m, eora_prefill_tiling* out);      // host arithmetic only; out: the main product, t = X.A
 
 }  // namespace eora

@@ -84,12 +84,19 @@ struct PrefillState {
 
 // First backbone k-block of split s: even shares of all k-blocks, the extension being part of the first; if the extension is more than
 // a share, the others share the backbone.  (each_tiling sees to it that every split has some.)
-__device__ __forceinline__ int split_lo(const PrefillArgs& p, int s) {
+__host__ __device__ __forceinline__ int split_lo(const PrefillArgs& p, int s) {
   if (s <= 0) return 0;
   if (s >= p.ksplit) return p.nkb_w;
   const int w = p.nkb_w / 2, b = p.nkb_b / 2, total = w + b;      // in pairs: a blob is not split
   return 2 * (b > total / p.ksplit ? (s - 1) * w / (p.ksplit - 1) : s * total / p.ksplit - b);
 }
+
+// k-blocks of a dequant warp's unit of work: a blob, or one tile where the blob has no scales (TM) or is 32 registers.
+__host__ __device__ constexpr int unit_blocks(int fmt, bool tm) { return tm ? (fmt_quantised(fmt) ? 2 : 1) : fmt == FMT_F16 ? 1 : 2; }
+// Two warps that share a row tile take its units alternately, and go on alternately from W's last unit to B's first: the first unit of B of the warp that
+// began W with unit `phase`.  So no warp passes over more than one unit of the other, three k-blocks at most from one of its own to the next; a wait by
+// parity cannot tell a stage's phase from the one two before, which a longer step than there are stages would ask of it.
+__host__ __device__ constexpr int b_phase(int phase, int step, int units_w) { return step == 2 ? (units_w + phase) & 1 : 0; }
 
 // ---------------------------------------------------------------------------------------------- PTX
 __device__ __forceinline__ void tma_load_2d(void* dst, const CUtensorMap* tm, int c0, int c1, uint64_t* bar) {
@@ -351,7 +358,7 @@ __device__ __forceinline__ bool dequant_part(const WMat& mat, int n0, int kb_lo,
   if constexpr (FMT == FMT_NONE) {
     return true;
   } else {
-    constexpr int U = FMT == FMT_F16 ? 1 : 2, PF = FMT == FMT_F16 ? 3 : 2;
+    constexpr int U = unit_blocks(FMT, false), PF = FMT == FMT_F16 ? 3 : 2;
     constexpr bool quant = fmt_quantised(FMT);
     constexpr int tb = tile_bytes(FMT);
     const int rt = (n0 >> 4) + tile;                     // this warp's row tile of the matrix
@@ -391,7 +398,7 @@ __device__ __forceinline__ bool dequant_part(const WMat& mat, int n0, int kb_lo,
     for (int j = 0; j < PF; ++j) issue(j);
     int it = it0 + phase * U;
     int s = it % p.sw, wrap = it / p.sw;                 // ring slot of iteration `it`, and how often it has been used before
-    auto advance = [&](int by) {                         // by <= 3 <= stages
+    auto advance = [&](int by) {                         // by <= 3 <= stages (b_phase: across the seam too)
       it += by;
       s += by;
       if (s >= p.sw) { s -= p.sw; ++wrap; }
@@ -529,7 +536,6 @@ __device__ __forceinline__ void cp_block(uint32_t dst, const uint8_t* src, int l
 }
 
 // A warp's ring of packed weights: slots of one unit (a blob, or one tile where there are no scales), one group of copies each.
-template <int FMT> constexpr int tm_tiles = fmt_quantised(FMT) ? 2 : 1;        // tiles of a unit
 __host__ __device__ constexpr int tm_unit_most(int fmt) { return fmt == FMT_NONE ? 0 : fmt_quantised(fmt) ? blob_bytes(fmt, 1) : tile_bytes(fmt); }
 __host__ __device__ constexpr int tm_slots(int fmt) { return tm_unit_most(fmt) <= 1536 ? 4 : 2; }      // (16 warps: 68 KB of 4-bit weights, 64 KB of fp16 in flight)
 __host__ __device__ constexpr int tm_ring(int fmt) { return tm_slots(fmt) * tm_unit_most(fmt); }
@@ -543,7 +549,7 @@ __device__ __forceinline__ bool dequant_part_tm(const WMat& mat, int n0, int kb_
   if constexpr (FMT == FMT_NONE) {
     return true;
   } else {
-    constexpr int U = tm_tiles<FMT>, D = tm_slots(FMT), tb = tile_bytes(FMT);
+    constexpr int U = unit_blocks(FMT, true), D = tm_slots(FMT), tb = tile_bytes(FMT);
     constexpr bool quant = fmt_quantised(FMT);
     constexpr int kUnit = quant ? blob_bytes(FMT, 0) : tb;
     const int rt = (n0 >> 4) + tile;
@@ -620,7 +626,7 @@ __device__ __forceinline__ bool dequant_part_tm(const WMat& mat, int n0, int kb_
         sent = full;
         if (traced) p.trace[it * 4 + 1] = clock64();
         it += c + 1 < U ? 1 : step * U - U + 1;
-        advance(c + 1 < U ? 1 : step * U - U + 1);       // (by at most 3 <= stages)
+        advance(c + 1 < U ? 1 : step * U - U + 1);       // (by at most 3 <= stages; b_phase: across the seam too)
       }
       if (!ok) break;
       __syncwarp();                                      // every lane has read the slot
@@ -791,12 +797,14 @@ __global__ void __launch_bounds__(kThreadsP, 1) k_prefill(const __grid_constant_
       const uint32_t ring = smem_u32(smem + p.w_off) + (uint32_t)(dw * p.w_slot);
       const uint32_t tmem_a = tmem_d + ((uint32_t)(in_half * 16) << 16) + p.a_col0 + hh * 32;
       ok = dequant_part_tm<WF>(p.w, n0, kw_lo, kw_hi, 0, tile, kphase, kstep, lane, p, ring, tmem_a, full_w, empty_w);
-      if (ok && nkb_ext > 0) ok = dequant_part_tm<BF>(p.b, n0, 0, nkb_ext, nkw, tile, kphase, kstep, lane, p, ring, tmem_a, full_w, empty_w);
+      if (ok && nkb_ext > 0)
+        ok = dequant_part_tm<BF>(p.b, n0, 0, nkb_ext, nkw, tile, b_phase(kphase, kstep, nkw / unit_blocks(WF, true)), kstep, lane, p, ring, tmem_a, full_w, empty_w);
     } else {
       // two halves: one row tile per warp; one half: two warps per row tile, alternating k-blocks
       const int kstep = 3 - nh, tile = nh == 2 ? dw : (dw & 7), kphase = nh == 2 ? 0 : (dw >> 3);
       ok = dequant_part<WF>(p.w, n0, kw_lo, kw_hi, 0, tile, kphase, kstep, lane, smem, p, full_w, empty_w, lut);
-      if (ok && nkb_ext > 0) ok = dequant_part<BF>(p.b, n0, 0, nkb_ext, nkw, tile, kphase, kstep, lane, smem, p, full_w, empty_w, lut);
+      if (ok && nkb_ext > 0)
+        ok = dequant_part<BF>(p.b, n0, 0, nkb_ext, nkw, tile, b_phase(kphase, kstep, nkw / unit_blocks(WF, false)), kstep, lane, smem, p, full_w, empty_w, lut);
     }
     if (ok) ok = mbar_wait_warp(&acc_full, 0, p.dev_status, lane);
     // the warps meet at barriers below: they must all take the same way
@@ -1130,7 +1138,57 @@ Tilings pick_tilings(int n_rows, int t_cols, int m, int nkb_w, int nkb_b, int sm
   return best;
 }
 
+Tilings plan_tilings(const Handle* h, int m) {
+  const bool ab = h->cfg.rank > 0;
+  const int n_rows = h->n_sub > 1 ? 16 * h->sub_tile0[h->n_sub] : h->cfg.d_out;
+  bool only128 = false;                                       // fused layers: every layer a whole number of tiles
+  for (int i = 0; i < h->n_sub && h->n_sub > 1; ++i) only128 = only128 || h->sub_dout[i] % (2 * BN_W) != 0;
+  return pick_tilings(n_rows, ab ? h->t_cols : 0, m, h->cfg.d_in / BK, ab ? h->r_pad / BK : 0, h->sm_count, only128);
+}
+
+// The most k-blocks from one that a dequant warp takes to the next it takes, over the CTAs of a launch whose rows end in a tile of one half.
+int longest_step(const PrefillArgs& a) {
+  const bool tm = a.a_cols > 0;
+  const int uw = unit_blocks(a.w.fmt, tm), ub = unit_blocks(a.b.fmt, tm);
+  int longest = 1;
+  for (int split = 0; split < a.ksplit; ++split)
+    for (int phase = 0; phase < 2; ++phase) {
+      const int nkw = split_lo(a, split + 1) - split_lo(a, split), nb = split == 0 ? a.nkb_b : 0;
+      int last = -1;                                     // (the first ones need no wait: as if the k-block in front of the first were this warp's)
+      auto part = [&](int it0, int units, int u, int from) {
+        for (int i = from; i < units; i += 2) {
+          if (it0 + i * u - last > longest) longest = it0 + i * u - last;
+          last = it0 + i * u + u - 1;
+        }
+      };
+      part(0, nkw / uw, uw, phase);
+      if (nb > 0) part(nkw, nb / ub, ub, b_phase(phase, 2, nkw / uw));
+    }
+  return longest;
+}
+
 }  // namespace
+
+int prefill_plan(const Handle* h, int m, eora_prefill_tiling* out) {
+  if (h->multi || h->w.group % 64) return EORA_ERR_UNSUPPORTED;
+  for (int i = 0; i < h->n_sub && h->n_sub > 1; ++i)
+    if (h->sub_dout[i] % BN_W) return EORA_ERR_UNSUPPORTED;
+  const Tilings tls = plan_tilings(h, m);
+  for (int i = 0; i < 2; ++i) {
+    out[i] = eora_prefill_tiling();
+    if (i == 1 && h->cfg.rank == 0) break;
+    const Tiling& t = i ? tls.t : tls.main;
+    PrefillArgs a = {};
+    a.w.fmt = i ? h->a.fmt : h->w.fmt;
+    a.b.fmt = i || h->cfg.rank == 0 ? FMT_NONE : h->b.fmt;
+    a.rows = t.rows; a.bt = t.bt; a.ksplit = t.ks;
+    a.nkb_w = h->cfg.d_in / BK; a.nkb_b = i || h->cfg.rank == 0 ? 0 : h->r_pad / BK;
+    fill_stages(a);
+    out[i].rows = t.rows; out[i].tokens = t.bt; out[i].cluster = t.ks;
+    out[i].stages = a.sw; out[i].in_tensor_memory = a.a_cols > 0; out[i].longest_step = longest_step(a);
+  }
+  return EORA_OK;
+}
 
 bool prefill_supported(const Handle* h, int m) {
   if (m <= 8) return false;              // one decode pass is always cheaper
@@ -1191,11 +1249,7 @@ cudaError_t launch_prefill_forward(const Handle* h, const void* x, int m, void* 
   }
   if (mid_supported(h, m)) return launch_mid_forward(h, x16, m, ys, st);
   const bool ab = c.rank > 0;
-  const int nkb_w = c.d_in / BK, nkb_b = ab ? h->r_pad / BK : 0;
-  const int n_rows_all = h->n_sub > 1 ? 16 * h->sub_tile0[h->n_sub] : c.d_out;
-  bool only128 = false;                                       // fused layers: every layer a whole number of tiles
-  for (int i = 0; i < h->n_sub && h->n_sub > 1; ++i) only128 = only128 || h->sub_dout[i] % (2 * BN_W) != 0;
-  const Tilings tls = pick_tilings(n_rows_all, ab ? h->t_cols : 0, m, nkb_w, nkb_b, h->sm_count, only128);
+  const Tilings tls = plan_tilings(h, m);
   const Tiling tl = tls.main;
   const int bt = tl.bt;
   CUtensorMap tm_x, tm_t;

@@ -58,3 +58,15 @@ def expected_family(M, K):
     if M > 64 or (M > 16 and ((M + 7) // 8) * 30 > K // 64):
         return eora.EORA_PATH_PREFILL
     return eora.EORA_PATH_DECODE
+
+
+def prefill_plan(w, ab, K, N, r, M, group=128):
+    """Tiles of a plain layer's forward by the tensor-core path (main product, t = X.A) on a GPU of 148 SMs."""
+    import paper_2410_21271_b200 as eora
+    c = eora.eora_linear_config()
+    c.d_in, c.d_out, c.rank, c.max_m = K, N, r, M
+    c.w_format = {"sp24": eora.EORA_W_SPARSE24, "sq4": eora.EORA_W_SPARSE24_Q4}.get(w, eora.EORA_W_QUANT)
+    c.w_bits, c.w_group = 3 if w == "q3" else 4, group
+    c.ab_format = {"f16": eora.EORA_AB_F16, "q4": eora.EORA_AB_Q4, "q3": eora.EORA_AB_Q3, "q8": eora.EORA_AB_Q8}[ab]
+    c.ab_group = 128
+    return eora.eora_linear_prefill_plan([c], M)

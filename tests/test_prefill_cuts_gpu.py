@@ -9,7 +9,7 @@ pytestmark = pytest.mark.gpu
 from oracle import eora_oracle as orc
 import eora_inputs as gen
 import paper_2410_21271_b200 as eora
-from helpers import make_case, run_layer, check_parity, x_to_torch
+from helpers import make_case, run_layer, check_parity, x_to_torch, prefill_plan
 
 
 @pytest.mark.parametrize("w,ab,K,N,r,M,xd,yd,group", [
@@ -73,4 +73,28 @@ def test_prefill_weights_in_tensor_memory(w, ab, K, N, r, M, group):
     x = gen.make_x(78, M, K, "f16")
     L = eora.Layer(wf, af, bf, max_m=M)
     check_parity(run_layer(L, x, "f16"), orc.forward(x, "f16", wf, af, bf), f"{w}/{ab} K{K} N{N} r{r} M{M}")
+    L.close()
+
+
+@pytest.mark.parametrize("w,ab,K,N,r,M,stages,tm", [
+    ("q4", "q4", 640, 3936, 256, 1100, 3, 0),     # 256 rows x 256 tokens, five units of W and two of B
+    ("q4", "f16", 640, 3936, 64, 1100, 3, 0),     # units of B of one k-block
+    ("q4", "f16", 512, 3936, 64, 1100, 3, 0),     # an even number of units
+    ("q4", "q4", 640, 19040, 256, 143, 3, 1),     # weights in tensor memory
+    ("q3", "f16", 384, 19040, 128, 143, 3, 1),
+    ("q4", "q8", 256, 19040, 256, 143, 3, 1),
+    ("sp24", "q4", 640, 19040, 256, 143, 3, 1),   # units of W of one k-block
+    ("q4", "q3", 640, 19040, 256, 100, 4, 1),
+    ("sq4", "q8", 640, 544, 256, 1100, 4, 1),     # 128 rows x 256 tokens
+])
+def test_prefill_short_rings(w, ab, K, N, r, M, stages, tm):
+    """The shortest rings, with tiles of one half (two warps to a row tile): odd and even numbers of units in front of the extension's."""
+    main = prefill_plan(w, ab, K, N, r, M)[0]
+    assert (main.stages, main.in_tensor_memory) == (stages, tm) and 0 < (N - 1) % main.rows + 1 <= 128
+    wf, af, bf = make_case(79, K, N, r, w=w, ab=ab)
+    x = gen.make_x(80, M, K, "f16")
+    L = eora.Layer(wf, af, bf, max_m=M)
+    ref = orc.forward(x, "f16", wf, af, bf)
+    for rep in range(3):
+        check_parity(run_layer(L, x, "f16"), ref, f"{w}/{ab} K{K} N{N} r{r} M{M} call {rep}")
     L.close()
