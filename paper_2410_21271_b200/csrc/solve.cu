@@ -1034,13 +1034,13 @@ __global__ void __launch_bounds__(256) k_colsq(const float* __restrict__ V, int 
     __syncthreads();
   }
 }
-// lam_i = |V_i|^2 / |U_i|^2
+// lam_i = |V_i|^2 / |U_i|^2; zero for a direction that is zero, and NaN where either is NaN (so no comparison that a NaN would fail decides here or below).
 __global__ void k_sigma(const double* __restrict__ parts, int r, double* __restrict__ lam) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= r) return;
   double v = 0.0, u = 0.0;
   for (int z = 0; z < kSigmaParts; ++z) { v += parts[(int64_t)z * 2 * r + i]; u += parts[((int64_t)z * 2 + 1) * r + i]; }
-  lam[i] = u > 0.0 ? v / u : 0.0;
+  lam[i] = u == 0.0 ? 0.0 : v / u;
 }
 // sigma_i = sqrt(lam_i);  B'[row][i] = U[row][i] sigma_i  (U: [d][ld]).  status: not zero if a product gave up; the results are then NaN.
 __global__ void k_finish_b(const float* __restrict__ U, int ld, const double* __restrict__ lam, int d, int r, float* __restrict__ Bp, float* __restrict__ sigma,
@@ -1049,9 +1049,8 @@ __global__ void k_finish_b(const float* __restrict__ U, int ld, const double* __
   const float bad = *status ? __int_as_float(0x7fffffff) : 0.f;
   for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < n; e += (int64_t)gridDim.x * blockDim.x) {
     const int i = (int)(e % r);
-    const float s = (float)sqrt(fmax(lam[i], 0.0));
-    Bp[e] = U[e / r * ld + i] * s + bad;
-    if (e < r) sigma[e] = (float)sqrt(fmax(lam[e], 0.0)) + bad;
+    Bp[e] = U[e / r * ld + i] * (float)sqrt(lam[i]) + bad;
+    if (e < r) sigma[e] = (float)sqrt(lam[e]) + bad;
   }
 }
 // A[i][j] = T[j][i] / sigma_i  (T: [k][ld], holding dW^T U); 32 x 32 tiles through shared memory, 32 x 8 threads
@@ -1064,8 +1063,8 @@ __global__ void k_finish_a(const float* __restrict__ T, int ld, const double* __
   __syncthreads();
   for (int q = y; q < 32; q += 8) {
     if (i0 + q >= r || j0 + x >= k) continue;
-    const double s = sqrt(fmax(lam[i0 + q], 0.0));
-    A[(int64_t)(i0 + q) * k + j0 + x] = (s > 0.0 ? (float)((double)tile[x][q] / s) : 0.f) + bad;
+    const double s = sqrt(lam[i0 + q]);
+    A[(int64_t)(i0 + q) * k + j0 + x] = (s == 0.0 ? 0.f : (float)((double)tile[x][q] / s)) + bad;
   }
 }
 // sum of squares of a matrix, fp64, into *out (zeroed by the caller)

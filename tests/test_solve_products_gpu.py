@@ -57,3 +57,17 @@ def test_not_a_number_in_not_a_number_out():
     b, a, s = eora.solve(w, w_hat, x, 16)
     torch.cuda.synchronize()
     assert not bool(torch.isfinite(b @ a).all())
+
+
+@pytest.mark.parametrize("d,k,n,r", [(256, 256, 512, 16), (1024, 512, 1024, 64), (640, 384, 600, 350)])      # the last: eigenproblem in one CTA
+@pytest.mark.parametrize("where,value", [("w", "nan"), ("w_hat", "inf"), ("x", "nan"), ("x", "-inf")])
+def test_what_is_not_finite_shows_in_every_result(d, k, n, r, where, value):
+    """sigma and A are not zero ("no error to compensate") where B' is not a number: every element of all three is not finite."""
+    import torch
+    import paper_2410_21271_b200 as eora
+    t = dict(zip(("w", "w_hat", "x"), (torch.from_numpy(v).cuda() for v in gen.make_solve_case(44, d, k, n))))
+    t[where][5, 7] = float(value)
+    b, a, s = eora.solve(t["w"], t["w_hat"], t["x"], r)
+    torch.cuda.synchronize()
+    for name, v in (("B'", b), ("A", a), ("sigma", s)):
+        assert not bool(torch.isfinite(v).any()), name
