@@ -25,7 +25,6 @@
 // when X is bf16 (the f16 MMA kind needs both operands in fp16; weights are kept fp16 because
 // bf16 weights alone cost 1.7e-3 of the 2e-3 error budget).
 #include <cuda.h>
-#include <math.h>
 #include "decode_common.cuh"
 
 namespace eora {
@@ -1089,7 +1088,8 @@ float tiling_cost(const Tiling& t, int n_rows, int m, int nkb, int sm_count) {
   float waves = (float)((ctas + cap - 1) / cap);
   const int over = tiles % sm_count;
   if (t.ks == 1 && t.rows == 2 * BN_W && t.bt == 256 && tiles > sm_count && over > 0 && 4 * over <= sm_count) waves -= 0.5f;
-  const float area = (float)(t.rows * t.bt) / 65536.f, doublings = log2f((float)t.ks);
+  constexpr float log2s[9] = {0.f, 0.f, 1.f, 1.5849625f, 2.f, 2.3219281f, 2.5849625f, 2.807355f, 3.f};
+  const float area = (float)(t.rows * t.bt) / 65536.f, doublings = log2s[t.ks];
   // Three, five, six or seven CTAs deal a tile's units unevenly (q|k|v at 100 tokens with five 21.4 us, with two CTAs of half the rows 19.5, estimated 4 % slower).
   const float uneven = t.ks & (t.ks - 1) ? 2000.f : 0.f;
   return waves * ((float)((nkb + t.ks - 1) / t.ks) * kblock_cycles(t, ctas <= cap) + 4100.f + 5000.f * area +
@@ -1107,34 +1107,51 @@ int token_tile(int m, int most) {      // the MMA N: a multiple of 16 up to `mos
 struct Tilings { Tiling main, t; };
 // A reduction axis is shared only by clusters that all run at once: in a second wave a cluster waits for SMs side by side (192 CTAs
 // in pairs take 50 us where 96 take 27).
-template <typename F>
-void each_tiling(int n_rows, int m, int nkb_w, int sm_count, bool only128, F f) {
+// A tiling that can be taken, its CTAs and its time.
+struct Candidate { Tiling t; int ctas; float cost; };
+constexpr int kMaxCandidates = 32;                   // two token tiles x two row sizes x eight cluster sizes
+int candidates(int n_rows, int m, int nkb_w, int nkb, int sm_count, bool only128, Candidate (&out)[kMaxCandidates]) {
   // Even tiles up to 1024 tokens, whole ones beyond.  Beyond, even ones are 1 to 3 % faster up to 1100 tokens (4096 x 14336 at 1025: 103.3 against
   // 106.9 us), within 2 % from there on and 5 % slower at 1800 to 1900 of that shape (198.9 against 188.4).
   // Or tiles of at most 160, where the weights of 256 rows fit into tensor memory.
   const int wide = m > 1024 ? 256 : token_tile(m, 256), narrow = m > 1024 ? 256 : token_tile(m, 160);
-  for (int bt = wide; bt == wide || bt == narrow; bt = bt == narrow ? 0 : narrow)
-   for (int rows = BN_W; rows <= (only128 ? BN_W : 2 * BN_W); rows += BN_W)
-    for (int ks = 1; ks <= 8 && (ks == 1 || nkb_w / ks >= 4); ++ks)
-      if (ks == 1 || (split_fits(rows, bt, ks) && (n_rows + rows - 1) / rows * ((m + bt - 1) / bt) * ks <= at_once(ks, sm_count))) f(Tiling{rows, bt, ks});
+  int n = 0;
+  for (int bt = wide; bt == wide || bt == narrow; bt = bt == narrow ? 0 : narrow) {
+    for (int rows = BN_W; rows <= (only128 ? BN_W : 2 * BN_W); rows += BN_W) {
+      const int tiles = (n_rows + rows - 1) / rows * ((m + bt - 1) / bt);
+      for (int ks = 1; ks <= 8 && (ks == 1 || nkb_w / ks >= 4); ++ks) {
+        const Tiling t{rows, bt, ks};
+        if (ks == 1 || (split_fits(rows, bt, ks) && tiles * ks <= at_once(ks, sm_count))) out[n++] = {t, tiles * ks, tiling_cost(t, n_rows, m, nkb, sm_count)};
+      }
+    }
+  }
+  return n;
 }
+// This runs in every call: each candidate's time is worked out once, and a main product that alone takes as long as the best pair does is not paired
+// (200 tokens, 1024 outputs, rank 512: 17 us with the times worked out for every pair, now 1.5).
 Tilings pick_tilings(int n_rows, int t_cols, int m, int nkb_w, int nkb_b, int sm_count, bool only128) {
+  Candidate mains[kMaxCandidates], ts[kMaxCandidates];
+  const int n_main = candidates(n_rows, m, nkb_w, nkb_w + nkb_b, sm_count, only128, mains);
+  const int n_t = t_cols > 0 ? candidates(t_cols, m, nkb_w, nkb_w, sm_count, t_cols <= BN_W, ts) : 0;
+  int room[9] = {};
+  for (int ks = 1; ks <= 8; ++ks) room[ks] = at_once(ks, sm_count);
   Tilings best = {};
   float best_c = -1.f;
-  auto ctas_of = [&](const Tiling& t, int rows) { return (rows + t.rows - 1) / t.rows * ((m + t.bt - 1) / t.bt) * t.ks; };
-  each_tiling(n_rows, m, nkb_w, sm_count, only128, [&](const Tiling& a) {
-    const float cm = tiling_cost(a, n_rows, m, nkb_w + nkb_b, sm_count);
-    const int ctas = ctas_of(a, n_rows);
-    auto take = [&](const Tiling& t, float c) { if (best_c < 0.f || c < best_c) { best_c = c; best = {a, t}; } };
-    if (t_cols == 0) { take(a, cm); return; }
-    each_tiling(t_cols, m, nkb_w, sm_count, t_cols <= BN_W, [&](const Tiling& t) {
-      const float ct = tiling_cost(t, t_cols, m, nkb_w, sm_count), tail = (float)nkb_b * kblock_cycles(a, true);
-      const int tc = ctas_of(t, t_cols), one_wave = ctas <= at_once(a.ks, sm_count);
-      const bool beside = one_wave && ctas + tc <= at_once(a.ks > t.ks ? a.ks : t.ks, sm_count);
+  for (int i = 0; i < n_main; ++i) {
+    const Candidate& a = mains[i];
+    const float cm = a.cost, tail = (float)nkb_b * kblock_cycles(a.t, true);
+    if (best_c >= 0.f && cm >= best_c) continue;
+    if (n_t == 0) { best_c = cm; best = {a.t, Tiling{}}; continue; }
+    const bool one_wave = a.ctas <= room[a.t.ks];
+    for (int j = 0; j < n_t; ++j) {
+      const Candidate& t = ts[j];
+      const float ct = t.cost;
+      const bool beside = one_wave && a.ctas + t.ctas <= room[a.t.ks > t.t.ks ? a.t.ks : t.t.ks];
       // (of equal ones the earlier t: three blocks of 64 tokens with adapters of rank 512, down 31.6 -> 28.6 us)
-      take(t, 0.02f * ct + (beside ? (cm > ct + tail ? cm : ct + tail) : one_wave ? cm + ct : cm + ct * (float)tc / (float)sm_count));
-    });
-  });
+      const float c = 0.02f * ct + (beside ? (cm > ct + tail ? cm : ct + tail) : one_wave ? cm + ct : cm + ct * (float)t.ctas / (float)sm_count);
+      if (best_c < 0.f || c < best_c) { best_c = c; best = {a.t, t.t}; }
+    }
+  }
   return best;
 }
 

@@ -36,3 +36,21 @@ def test_no_shape_lets_a_warp_pass_over_a_whole_ring():
             assert t.longest_step <= 3 and t.longest_step <= max(t.stages, 1), (w, ab, K, N, r, M, t.rows, t.tokens, t.stages, t.longest_step)
             short += 0 < t.stages <= 4
     assert short > 200
+
+
+def test_planning_takes_no_longer_with_many_tilings_to_choose_from():
+    """A forward plans its tiles in every call.  200 tokens with adapters of rank 512 have the most tilings (hundreds of pairs of a main product's and
+    one for t), 2048 tokens the fewest."""
+    import time
+
+    def best(*shape):
+        times = []
+        for _ in range(30):
+            t = time.perf_counter()
+            for _ in range(50):
+                plan(*shape)
+            times.append(time.perf_counter() - t)
+        return min(times)
+
+    few, many = best("q4", "f16", 4096, 1024, 128, 2048), best("q4", "f16", 4096, 1024, 512, 200)
+    assert many < 1.5 * few
