@@ -20,6 +20,8 @@
  *
  * All pointers are DEVICE pointers to row-major fp32, 16-byte aligned, caller-owned; nothing is allocated, all work is
  * enqueued on `stream` and nothing synchronises.  `workspace` must hold eora_solve_workspace_bytes(cfg) bytes.
+ * (A smaller workspace is taken too, down to one that holds dW, P = dW X~, the smaller square of P, the iterates and, where k or n is no multiple
+ * of 128, a copy of X~: products then go in more parts and, where k is far below min(d, n), those with the iterates are slower.)
  * Arithmetic: products of fp32 accuracy for the large contractions (fp32 arithmetic, or three bf16 parts per value on the tensor
  * cores with fp32 sums), fp64 for the small (r + oversample)^2 problems (Gram matrices of the iterate, Cholesky factor, Jacobi
  * eigenproblem).  An infinity or NaN in the inputs, or a wait inside a kernel that ran out, shows as NaN in the results.

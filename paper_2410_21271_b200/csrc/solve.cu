@@ -1084,12 +1084,15 @@ struct Plan {
   int d, k, n, r, m;
   int iters;                  // plain products; 0: the filter
   int dp, kp, np;             // d, k, n in whole 128-tiles
-  int kc;                     // of the reduction axis k: what is split at a time for P
+  bool tensor;                // products with the iterate on the tensor cores (with C's three parts in the workspace)
+  bool keep_dw;               // dW stays where P's product leaves it; else its place is used in between, and it is formed again for step 6
+  int kc, lc;                 // of the reduction axes of P and of its square: what is split at a time
+  int py, pz;                 // rows of P, and columns of it, that are split at a time for the products with the iterate
   bool n_side, pad_x;         // iterate with P^T P instead of P P^T; X~ is needed in whole tiles
   int s, sp;                  // size of the matrix that is iterated with, in whole tiles
   int w, ldm;                 // width of the skinny products' tiles, leading dimension of the iterates (a multiple of it)
   int wr, ldr;                // the same for the products with r columns
-  size_t off_dw, off_x, off_status, off_filter, off_p, off_c, off_y, off_q, off_z, off_s, off_sp, off_d, off_h, off_lam, off_vf, total;
+  size_t off_x, off_p, off_dw, off_big, off_c, off_parts, off_sq, off_it, off_y, off_q, off_z, off_s, off_sp, off_d, off_h, off_lam, off_vf, total;
 };
 size_t up256(size_t v) { return (v + 255) & ~size_t(255); }
 int up128(int v) { return (v + 127) & ~127; }
@@ -1100,7 +1103,82 @@ int pick_width(int cols) {
     if ((cols + w - 1) / w * w < (cols + best - 1) / best * best) best = w;
   return best;
 }
-bool make_plan(const eora_solve_config* c, Plan& p) {
+// What the workspace has room for.  ROOMY: what makes no product go in more parts than is good for it, or as much of that as kRoomy or a quarter of the
+// matrices themselves.  TIGHT: the matrices (and C's three parts where they are larger).  LEAN: the matrices; products with the iterate on the CUDA cores.
+// Parts cost some 10 us each in a small solve, 2 to 4 % of it, and 80 us at 4096 x 4096 x 16384 (seven parts 8.26 ms, one 7.7, with 330 MB more; three, with 110 MB more, 7.8).
+enum Room { ROOMY, TIGHT, LEAN };
+constexpr size_t kRoomy = 48u << 20;
+constexpr size_t kSmall = 8u << 20;                  // (one or two parts more at most; the reported workspace is the smallest one then)
+
+// Offsets and parts for a given region `big`; whole: nothing goes in more parts than is good for it.
+bool lay_out(Plan& p, size_t big, bool& whole) {
+  size_t o = 0;
+  auto take = [&](size_t bytes) { size_t at = o; o += up256(bytes); return at; };
+  const size_t rows = p.dp > p.np ? p.dp : p.np, tall = rows > (size_t)p.kp ? rows : p.kp, c_b = (size_t)p.sp * p.sp * 4;
+  p.off_x = take(p.pad_x ? (size_t)p.kp * p.np * 4 : 0);
+  p.off_p = take((size_t)p.dp * p.np * 4);                        // P = dW X~; the loss check keeps (dW - B'A) X~ here
+  p.off_dw = take((size_t)p.dp * p.kp * 4);
+  // One region for what is not needed at the same time, with room for C or, in the loss check, dW - B'A:
+  //   dW and X~^T split, as much of the reduction axis at a time as there is room for up to off_lam (at least two parts where all would take more than 32 MB);
+  //   C at the region's end, and P split for its square in front of it or behind it;
+  //   C split from the region's front on, over C itself (slabs of rows, in order);
+  //   in the end P split, as many of the result's rows at a time as there is room for.
+  // Without keep_dw it begins with dW's place.  An iterate's parts are at its end, or, if they fit there, among the small problems, which are not in use when it is
+  // multiplied with.
+  p.off_big = take(big);
+  p.off_c = p.off_big + big - c_b;
+  const size_t end = o;
+  p.off_y = take(rows * p.ldm * 4);
+  p.off_q = take(rows * p.ldm * 4);
+  p.off_z = take(tall * p.ldm * 4);
+  p.off_s = take((size_t)p.m * p.m * 8);                          // (in the end, with the next one: 64 r partial sums for sigma)
+  p.off_sp = take((size_t)kGramParts * p.m * p.m * 8);
+  p.off_d = take((size_t)((p.m + 15) / 16) * 256 * 8);
+  p.off_h = take((size_t)p.m * p.m * 8);
+  p.off_lam = take((size_t)(2 * p.m + 128) * 8);                  // (the last 32 doubles: status and the filter's state)
+  p.off_vf = take((size_t)p.ldm * p.ldm * 4);
+  p.total = o;
+  p.off_it = p.keep_dw ? p.off_big : p.off_dw;
+  size_t s_q = eora::split_bytes(up128(p.ldm), p.dp);             // an iterate of either side (np <= dp with n_side)
+  const bool among = s_q <= p.off_lam - p.off_s;
+  p.off_sq = among ? p.off_s : end - s_q;
+  if (among) s_q = 0;
+  // How much at a time.
+  auto in_parts = [](int len, int parts) { return ((len / 128 + parts - 1) / parts) * 128; };
+  auto at_once = [&](int len, size_t each, size_t room, int least) {      // (each: bytes of 128 of len)
+    const size_t most = room / each;
+    if (most < 1) return 0;
+    int parts = least;
+    while ((size_t)in_parts(len, parts) > most * 128) ++parts;
+    return in_parts(len, parts);
+  };
+  const size_t dx = eora::split_bytes(p.dp, 128) + eora::split_bytes(p.np, 128);
+  const int halves = dx * (p.kp / 128) > (32u << 20) ? 2 : 1;
+  p.kc = at_once(p.kp, dx, p.off_lam - p.off_it, halves);
+  const int len = p.n_side ? p.dp : p.np;                         // reduction axis of P's square
+  const size_t front = p.off_c - p.off_it, behind = p.off_lam - p.off_y;
+  p.off_parts = front >= behind ? p.off_it : p.off_y;
+  p.lc = at_once(len, eora::split_bytes(p.sp, 128), front >= behind ? front : behind, 1);
+  if (p.kc < 1 || p.lc < 1) return false;
+  whole = p.kc == in_parts(p.kp, halves) && p.lc == len;
+  p.py = p.pz = 0;
+  if (p.tensor) {
+    if (end - p.off_it < s_q || eora::split_bytes(p.sp, p.sp) > end - p.off_it - s_q) return false;
+    // (a slab of C takes at least one row block: the last one with what C's rows in front of it have left)
+    if (front + (size_t)(p.sp - 128) * p.sp * 4 < eora::split_bytes(p.sp, p.sp)) return false;
+    const size_t room = end - p.off_it - s_q;
+    p.pz = at_once(p.np, eora::split_bytes(128, p.dp), room, 1);
+    if (p.pz < 1) return false;
+    whole = whole && p.pz == p.np;
+    if (p.n_side) {
+      p.py = at_once(p.dp, eora::split_bytes(128, p.np), room, 1);
+      if (p.py < 1) return false;
+      whole = whole && p.py == p.dp;
+    }
+  }
+  return true;
+}
+bool make_plan(const eora_solve_config* c, Plan& p, Room room) {
   if (!c || c->d < 1 || c->k < 1 || c->n < 1 || c->rank < 1) return false;
   p.d = c->d; p.k = c->k; p.n = c->n; p.r = c->rank;
   int over = c->oversample > 0 ? c->oversample : 32;
@@ -1117,36 +1195,40 @@ bool make_plan(const eora_solve_config* c, Plan& p) {
   p.w = pick_width(p.m); p.ldm = (p.m + p.w - 1) / p.w * p.w;
   p.wr = pick_width(p.r); p.ldr = (p.r + p.wr - 1) / p.wr * p.wr;
   if (p.ldr > p.ldm) { p.wr = p.w; p.ldr = p.ldm; }
-  size_t o = 0;
-  auto take = [&](size_t bytes) { size_t at = o; o += up256(bytes); return at; };
-  const size_t rows = p.dp > p.np ? p.dp : p.np, tall = rows > (size_t)p.kp ? rows : p.kp;
-  const size_t c_el = (size_t)p.sp * p.sp, r_el = (size_t)p.d * p.k;
-  p.off_dw = take((size_t)p.dp * p.kp * 4);
-  p.off_x = take(p.pad_x ? (size_t)p.kp * p.np * 4 : 0);
-  p.off_status = take(4);
-  p.off_filter = take(sizeof(Filter));
-  p.off_p = take((size_t)p.dp * p.np * 4);                        // P = dW X~; the loss check keeps (dW - B'A) X~ here
-  // One region for what is not needed at the same time: dW and X~^T split, all of them or half of the reduction axis at a time (where all would take more than
-  // 32 MB); C, and behind it P split for its square, then C and the iterate split; in the end P and the iterate split; in the loss check dW - B'A.
-  p.kc = eora::split_bytes(p.dp, p.kp) + eora::split_bytes(p.np, p.kp) > (32u << 20) ? (p.kp / 128 + 1) / 2 * 128 : p.kp;
-  const size_t s_p = eora::split_bytes(p.dp, p.np);
-  size_t big = r_el * 4;
-  const size_t s_q = eora::split_bytes(up128(p.ldm), p.dp > p.np ? p.dp : p.np);      // an iterate
-  for (size_t v : {eora::split_bytes(p.dp, p.kc) + eora::split_bytes(p.np, p.kc), up256(c_el * 4) + s_p, up256(c_el * 4) + eora::split_bytes(p.sp, p.sp) + s_q, s_p + s_q})
-    if (v > big) big = v;
-  p.off_c = take(big);
-  p.off_y = take(rows * p.ldm * 4);
-  p.off_q = take(rows * p.ldm * 4);
-  p.off_z = take(tall * p.ldm * 4);
-  p.off_s = take((size_t)p.m * p.m * 8);
-  const size_t gram_el = (size_t)kGramParts * p.m * p.m, sig_el = (size_t)kSigmaParts * 2 * p.r;
-  p.off_sp = take((gram_el > sig_el ? gram_el : sig_el) * 8);
-  p.off_d = take((size_t)((p.m + 15) / 16) * 256 * 8 + (size_t)p.m * 8);      // the diagonal blocks' inverses, the smallest pivots
-  p.off_h = take((size_t)p.m * p.m * 8);
-  p.off_lam = take((size_t)(2 * p.m + 128) * 8);
-  p.off_vf = take((size_t)p.ldm * p.ldm * 4);
-  p.total = o;
-  return true;
+  // The products with an iterate: on the tensor cores, the iterate being split for each, or, small ones, on the CUDA cores in one launch.  512 x 512 x 64: 9
+  // against 6 us on the CUDA cores, 768 x 768 x 64 about even; 2048 x 2048 x 160: 21 against 50.
+  p.tensor = room != LEAN && (double)p.sp * p.sp * p.ldm >= 8e7;
+  const size_t c_b = (size_t)p.sp * p.sp * 4, e_b = (size_t)p.d * p.k * 4, least = up256(c_b > e_b ? c_b : e_b);
+  // The matrices' own size if that will do, with dW left alone or formed again; else a larger one.
+  bool whole = false;
+  p.keep_dw = true;
+  if (lay_out(p, least, whole) && whole) return true;
+  if (room == ROOMY && p.total >= kSmall) {
+    // what is asked of the region: dW and X~^T split, C and P split, C's three parts, each with an iterate's
+    const int len = p.n_side ? p.dp : p.np;
+    const size_t sq = eora::split_bytes(up128(p.ldm), p.dp), c_p = c_b + eora::split_bytes(p.sp, len), c_3 = eora::split_bytes(p.sp, p.sp) + sq;
+    const int kh = eora::split_bytes(p.dp, p.kp) + eora::split_bytes(p.np, p.kp) > (32u << 20) ? (p.kp / 128 + 1) / 2 * 128 : p.kp;
+    const size_t a = eora::split_bytes(p.dp, kh) + eora::split_bytes(p.np, kh), own = p.off_lam - p.off_y, p_3 = eora::split_bytes(p.dp, p.np) + sq;
+    size_t need = least;
+    for (size_t v : {a > own ? a - own : 0, c_p, p.tensor ? c_3 : 0, p.tensor ? p_3 : 0})
+      if (up256(v) > need) need = up256(v);
+    const size_t most = p.total / 4 > kRoomy ? up256(p.total / 4) : kRoomy;
+    if (need - least <= most && lay_out(p, need, whole) && whole) return true;
+    p.keep_dw = false;
+    const size_t dw_b = up256((size_t)p.dp * p.kp * 4);
+    if (lay_out(p, least, whole) && whole) return true;
+    const size_t more = need > dw_b ? need - dw_b : 0;
+    if (more > least && lay_out(p, more - least <= most ? more : least + most, whole)) return true;
+  }
+  // In parts.
+  for (int i = 0; i < 2; ++i) {
+    p.keep_dw = i == 0 && !p.tensor;
+    if (lay_out(p, least, whole)) return true;
+  }
+  // C's three parts are larger than C and dW (14336 x 4096, n 16384).
+  const size_t three = up256(eora::split_bytes(p.sp, p.sp) + eora::split_bytes(up128(p.ldm), p.dp) + eora::split_bytes(128, p.dp)), dw_b = up256((size_t)p.dp * p.kp * 4);
+  p.keep_dw = false;
+  return lay_out(p, three - dw_b, whole);
 }
 inline bool aligned16(const void* q) { return (reinterpret_cast<uintptr_t>(q) & 15) == 0; }
 
@@ -1168,7 +1250,8 @@ cudaError_t allow_smem(int bytes) {
 
 constexpr int kSingleSteps = 4;        // products that are orthogonalised one by one before the pairs begin
 
-// Q = orth(Y) by Cholesky-QR: Gram matrix, its factor and Q = Y L^{-T} in fp64.  Y, Q: [rows][ldm], rows a multiple of 16.
+// Q = orth(Y) by Cholesky-QR: Gram matrix, its factor and Q = Y L^{-T} in fp64.  Y, Q: [rows][ldm], rows a multiple of 16.  parts: the Gram matrix's
+// partial sums, then the smallest pivots.
 int orthonormalise(cudaStream_t st, const Plan& p, int rows, const float* Y, float* Q, double* S, double* parts, double* D,
                    bool scaled = false, Filter* f = nullptr, bool prev = false, double lo = 0.0, double hi = 0.0) {
   CK(gram64<false>(st, Y, rows, p.m, p.ldm, parts, S));
@@ -1179,7 +1262,7 @@ int orthonormalise(cudaStream_t st, const Plan& p, int rows, const float* Y, flo
   // columns: 6.28 ms, with one CTA that kept such a matrix in L2 7.72).
   for (int j0 = 0; j0 < p.m; j0 += kCholSmem) {
     const int w = p.m - j0 < kCholSmem ? p.m - j0 : kCholSmem, j1 = j0 + w, below = p.m - j1;
-    k_chol64<<<1, kCholThreads, chol_smem(w), st>>>(S, p.m, p.m, j0, w, D + j0 * 16, D + (size_t)((p.m + 15) / 16) * 256, below ? nullptr : f, prev, lo, hi);
+    k_chol64<<<1, kCholThreads, chol_smem(w), st>>>(S, p.m, p.m, j0, w, D + j0 * 16, parts, below ? nullptr : f, prev, lo, hi);
     if (below > 0) {
       double* l21 = S + (int64_t)j1 * p.m + j0;
       k_trsm<double><<<(below + 15) / 16, 256, trsm_smem(w), st>>>(l21, S + (int64_t)j0 * (p.m + 1), p.m, D + j0 * 16, w, p.m, below, l21, false);
@@ -1228,14 +1311,16 @@ extern "C" {
 
 size_t eora_solve_workspace_bytes(const eora_solve_config* cfg) {
   Plan p;
-  return make_plan(cfg, p) ? p.total : 0;
+  return make_plan(cfg, p, ROOMY) ? p.total : 0;
 }
 
 int eora_solve(const eora_solve_config* cfg, const float* w, const float* w_hat, const float* x_tilde, float* b_prime, float* a,
                float* sigma, void* workspace, size_t workspace_bytes, void* stream) {
   if (!cfg || !w || !w_hat || !x_tilde || !b_prime || !a || !sigma || !workspace) return EORA_ERR_NULL_ARG;
   Plan p;
-  if (!make_plan(cfg, p) || workspace_bytes < p.total) return EORA_ERR_BAD_SHAPE;
+  bool fits = false;
+  for (Room room : {ROOMY, TIGHT, LEAN}) fits = fits || (make_plan(cfg, p, room) && workspace_bytes >= p.total);
+  if (!fits) return EORA_ERR_BAD_SHAPE;
   if (!aligned16(w) || !aligned16(w_hat) || !aligned16(x_tilde) || !aligned16(b_prime) || !aligned16(a) || !aligned16(workspace)) return EORA_ERR_MISALIGNED;
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
   char* ws = reinterpret_cast<char*>(workspace);
@@ -1253,9 +1338,10 @@ int eora_solve(const eora_solve_config* cfg, const float* w, const float* w_hat,
   float* Vf = reinterpret_cast<float*>(ws + p.off_vf);
   const int dp = p.dp, kp = p.kp, np = p.np, sp = p.sp, ldm = p.ldm;
 
-  uint8_t* big = reinterpret_cast<uint8_t*>(ws + p.off_c);
-  uint8_t* behind_c = big + up256((size_t)p.sp * p.sp * 4);
-  int* status = reinterpret_cast<int*>(ws + p.off_status);
+  uint8_t* it_mem = reinterpret_cast<uint8_t*>(ws + p.off_it);
+  uint8_t* parts = reinterpret_cast<uint8_t*>(ws + p.off_parts);
+  int* status = reinterpret_cast<int*>(lam + 2 * p.m + 96);
+  static_assert(sizeof(Filter) <= 30 * 8, "behind the eigenvalues");
   int device = 0, sms = 0;
   CK(cudaGetDevice(&device));
   CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device));
@@ -1264,26 +1350,40 @@ int eora_solve(const eora_solve_config* cfg, const float* w, const float* w_hat,
   float* xp = p.pad_x ? reinterpret_cast<float*>(ws + p.off_x) : nullptr;
   for (int k0 = 0; k0 < kp; k0 += p.kc) {
     const int kc = kp - k0 < p.kc ? kp - k0 : p.kc, kr = p.k - k0 < kc ? p.k - k0 : kc;      // columns of dW, without the padding
-    uint8_t* xs = big + eora::split_bytes(dp, p.kc);
-    CK(eora::split_rows(st, w + k0, w_hat + k0, p.d, kr, p.k, dp, kc, big, dW + k0, kp));
+    uint8_t* xs = it_mem + eora::split_bytes(dp, p.kc);
+    CK(eora::split_rows(st, w + k0, w_hat + k0, p.d, kr, p.k, dp, kc, it_mem, p.keep_dw ? dW + k0 : nullptr, kp));
     CK(eora::split_cols(st, x_tilde + (size_t)k0 * p.n, kr, p.n, p.n, kc, np, xs, xp ? xp + (size_t)k0 * np : nullptr));
-    CK(eora::split_gemm(st, big, xs, dp, np, kc, Pm, np, false, k0 > 0, sms, status));
+    CK(eora::split_gemm(st, it_mem, xs, dp, np, kc, Pm, np, false, k0 > 0, sms, status));
   }
-  if (p.n_side) CK(eora::split_cols(st, Pm, dp, np, np, dp, np, behind_c));
-  else CK(eora::split_rows(st, Pm, nullptr, dp, np, np, dp, np, behind_c, nullptr, 0));
-  CK(eora::split_gemm(st, behind_c, behind_c, sp, sp, p.n_side ? dp : np, C, sp, true, false, sms, status));
-  // The products with an iterate: on the tensor cores, the iterate being split for each, or, small ones, on the CUDA cores in one launch.  512 x 512 x 64: 9
-  // against 6 us on the CUDA cores, 768 x 768 x 64 about even; 2048 x 2048 x 160: 21 against 50.
-  const bool tensor = (double)sp * sp * ldm >= 8e7;
-  if (tensor) CK(eora::split_rows(st, C, nullptr, sp, sp, sp, sp, sp, behind_c, nullptr, 0));
-  // V [rows_out][ldm] = M U - *shift U for an iterate U; M = mat split (rows_out x rows_in); sq: where U is split
-  auto product = [&](const uint8_t* mat, uint8_t* sq, int rows_out, int rows_in, const float* U, float* V, const float* shift) -> int {
-    CK(eora::split_cols(st, U, rows_in, ldm, ldm, rows_in, up128(ldm), sq));
-    CK(eora::split_skinny(st, p.w, mat, sq, rows_out, ldm, rows_in, V, ldm, U, shift, status));
+  const int len = p.n_side ? dp : np;
+  for (int l0 = 0; l0 < len; l0 += p.lc) {
+    const int lc = len - l0 < p.lc ? len - l0 : p.lc;
+    if (p.n_side) CK(eora::split_cols(st, Pm + (size_t)l0 * np, lc, np, np, lc, np, parts));
+    else CK(eora::split_rows(st, Pm + l0, nullptr, dp, lc, np, dp, lc, parts, nullptr, 0));
+    CK(eora::split_gemm(st, parts, parts, sp, sp, lc, C, sp, true, l0 > 0, sms, status));
+  }
+  uint8_t* sq = reinterpret_cast<uint8_t*>(ws + p.off_sq);
+  if (p.tensor) {
+    // C's parts take 6 bytes where C has 4: a slab of rows ends before the first row that is not yet split.
+    for (int r0 = 0; r0 < sp;) {
+      const size_t room = p.off_c - p.off_it + (size_t)r0 * sp * 4;
+      const int most = (int)(room / eora::split_bytes(128, sp) < (size_t)sp / 128 ? room / eora::split_bytes(128, sp) : (size_t)sp / 128) * 128, r1 = most < sp ? most : sp;
+      if (r1 <= r0) return EORA_ERR_BAD_SHAPE;       // (never: lay_out has seen to it)
+      CK(eora::split_rows(st, C + (size_t)r0 * sp, nullptr, r1 - r0, sp, sp, r1 - r0, sp, it_mem + eora::split_bytes(r0, sp), nullptr, 0));
+      r0 = r1;
+    }
+  }
+  // V [rows_out][ldm] = M U - *shift U for an iterate U; M = mat split (rows_out x rows_in); to: where U is split
+  auto product = [&](const uint8_t* mat, const uint8_t* u_split, int rows_out, int rows_in, const float* U, float* V, const float* shift) -> int {
+    CK(eora::split_skinny(st, p.w, mat, u_split, rows_out, ldm, rows_in, V, ldm, U, shift, status));
     return EORA_OK;
   };
+  auto split_iterate = [&](const float* U, int rows_in, uint8_t* to) { return eora::split_cols(st, U, rows_in, ldm, ldm, rows_in, up128(ldm), to); };
   auto times_c = [&](const float* U, float* V, const float* shift) -> int {
-    if (tensor) return product(behind_c, behind_c + eora::split_bytes(sp, sp), sp, sp, U, V, shift);
+    if (p.tensor) {
+      CK(split_iterate(U, sp, sq));
+      return product(it_mem, sq, sp, sp, U, V, shift);
+    }
     CK(skinny<true>(st, p.w, sp, sp, C, sp, U, ldm, ldm, V, ldm, shift));      // (C is symmetric: read by columns)
     return EORA_OK;
   };
@@ -1306,7 +1406,7 @@ int eora_solve(const eora_solve_config* cfg, const float* w, const float* w_hat,
   constexpr int kPairs = 5, kOrder[kPairs] = {3, 1, 4, 0, 2};
   auto node = [&](int i) { return 0.5 + 0.5 * cos((2 * i + 1) * 3.14159265358979323846 / (4 * kPairs)); };
   const int iters = filter ? kSingleSteps + 2 * kPairs : p.iters;
-  Filter* f = filter ? reinterpret_cast<Filter*>(ws + p.off_filter) : nullptr;
+  Filter* f = filter ? reinterpret_cast<Filter*>(lam + 2 * p.m + 98) : nullptr;
   for (int it = 0, pairs = 0; it < iters;) {
     const bool pair = it >= kSingleSteps && iters - it >= 2;
     if (int rc = times_c(Q, Y, pair && f ? f->rho : nullptr)) return rc;
@@ -1320,9 +1420,13 @@ int eora_solve(const eora_solve_config* cfg, const float* w, const float* w_hat,
     if (int rc = orthonormalise(st, p, sp, Y, Q, S, Sp, D, next_pair, next_pair ? f : nullptr, pair, node(i), node(2 * kPairs - 1 - i))) return rc;
   }
   if (p.n_side) {                                                             // to the d-dimensional side
-    if (tensor) {
-      CK(eora::split_rows(st, Pm, nullptr, dp, np, np, dp, np, big, nullptr, 0));
-      if (int rc = product(big, big + eora::split_bytes(dp, np), dp, np, Q, Y, nullptr)) return rc;
+    if (p.tensor) {
+      CK(split_iterate(Q, np, sq));
+      for (int r0 = 0; r0 < dp; r0 += p.py) {
+        const int rc = dp - r0 < p.py ? dp - r0 : p.py;
+        CK(eora::split_rows(st, Pm + (size_t)r0 * np, nullptr, rc, np, np, rc, np, it_mem, nullptr, 0));
+        if (int e = product(it_mem, sq, rc, np, Q, Y + (size_t)r0 * ldm, nullptr)) return e;
+      }
     } else {
       CK(skinny<false>(st, p.w, dp, np, Pm, np, Q, ldm, ldm, Y, ldm));
     }
@@ -1330,9 +1434,13 @@ int eora_solve(const eora_solve_config* cfg, const float* w, const float* w_hat,
   }
   if (int rc = orthonormalise(st, p, dp, Q, Y, S, Sp, D)) return rc;          // second pass: orthogonal to fp32 rounding
   // Rayleigh-Ritz on span(Y)
-  if (tensor) {                                                               // Z = P^T Y
-    CK(eora::split_cols(st, Pm, dp, np, np, dp, np, big));
-    if (int rc = product(big, big + eora::split_bytes(dp, np), np, dp, Y, Z, nullptr)) return rc;
+  if (p.tensor) {                                                             // Z = P^T Y
+    CK(split_iterate(Y, dp, sq));
+    for (int n0 = 0; n0 < np; n0 += p.pz) {
+      const int nc = np - n0 < p.pz ? np - n0 : p.pz;
+      CK(eora::split_cols(st, Pm + n0, dp, nc, np, dp, nc, it_mem));
+      if (int e = product(it_mem, sq, nc, dp, Y, Z + (size_t)n0 * ldm, nullptr)) return e;
+    }
   } else {
     CK(skinny<true>(st, p.w, np, dp, Pm, np, Y, ldm, ldm, Z, ldm));
   }
@@ -1342,10 +1450,11 @@ int eora_solve(const eora_solve_config* cfg, const float* w, const float* w_hat,
   CK(skinny<false>(st, p.wr, dp, ldm, Y, ldm, Vf, ldm, p.ldr, Q, ldm));       // U' = Y V[:, :r]
   // step 6.  The tensor cores' sums are 2e-7 too small (truncation), which the eigenvectors do not notice but the eigenvalues would (sigma 2e-7 off instead
   // of 3e-8): sigma_i = |X~^T dW^T u_i| / |u_i| is taken from fp32 products on the CUDA cores.
+  if (!p.keep_dw) CK(eora::split_rows(st, w, w_hat, p.d, p.k, p.k, dp, kp, nullptr, dW, kp));
   CK(skinny<true>(st, p.wr, kp, dp, dW, kp, Q, ldm, p.ldr, Z, ldm));          // dW^T U'
   CK(skinny<true>(st, p.wr, np, kp, xp ? xp : x_tilde, np, Z, ldm, p.ldr, Y, ldm));
-  k_colsq<<<dim3((p.r + 31) / 32, kSigmaParts), 256, 0, st>>>(Y, np, Q, dp, ldm, p.r, Sp);
-  k_sigma<<<(p.r + 127) / 128, 128, 0, st>>>(Sp, p.r, lam);
+  k_colsq<<<dim3((p.r + 31) / 32, kSigmaParts), 256, 0, st>>>(Y, np, Q, dp, ldm, p.r, S);
+  k_sigma<<<(p.r + 127) / 128, 128, 0, st>>>(S, p.r, lam);
   k_finish_b<<<592, 256, 0, st>>>(Q, ldm, lam, p.d, p.r, b_prime, sigma, status);
   k_finish_a<<<dim3((p.k + 31) / 32, (p.r + 31) / 32), dim3(32, 8), 0, st>>>(Z, ldm, lam, p.r, p.k, a, status);
   CK(cudaGetLastError());
@@ -1356,11 +1465,11 @@ int eora_solve_loss(const eora_solve_config* cfg, const float* w, const float* w
                     const float* a, double* loss_sq, void* workspace, size_t workspace_bytes, void* stream) {
   if (!cfg || !w || !w_hat || !x_tilde || !b_prime || !a || !loss_sq || !workspace) return EORA_ERR_NULL_ARG;
   Plan p;
-  if (!make_plan(cfg, p) || workspace_bytes < p.total) return EORA_ERR_BAD_SHAPE;
+  if (!make_plan(cfg, p, LEAN) || workspace_bytes < p.total) return EORA_ERR_BAD_SHAPE;
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
   char* ws = reinterpret_cast<char*>(workspace);
   float* dW = reinterpret_cast<float*>(ws + p.off_dw);
-  float* R = reinterpret_cast<float*>(ws + p.off_c);       // B'A, then the residual
+  float* R = reinterpret_cast<float*>(ws + p.off_big);     // B'A, then the residual
   float* E = reinterpret_cast<float*>(ws + p.off_p);       // (dW - B'A) X~  (d x n)
   k_sub<<<592, 256, 0, st>>>(w, w_hat, dW, (int64_t)p.d * p.k);
   CK(sgemm(st, p.d, p.k, p.r, b_prime, p.r, false, a, p.k, false, R, p.k));    // B' A

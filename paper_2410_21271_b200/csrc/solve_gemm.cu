@@ -78,7 +78,7 @@ __global__ void __launch_bounds__(256) k_split_rows(const float* __restrict__ a,
       float4* to = reinterpret_cast<float4*>(copy + row * ld_copy + k0);
       to[0] = make_float4(v[0], v[1], v[2], v[3]); to[1] = make_float4(v[4], v[5], v[6], v[7]);
     }
-    store_piece(out + ((int64_t)blockIdx.y * (cols_p / kSplitCols) + kb) * kSplitBlock, r, c, v);
+    if (out) store_piece(out + ((int64_t)blockIdx.y * (cols_p / kSplitCols) + kb) * kSplitBlock, r, c, v);
   }
 }
 

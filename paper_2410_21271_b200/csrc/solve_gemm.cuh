@@ -11,7 +11,7 @@ namespace eora {
 constexpr int kSplitRows = 128, kSplitCols = 32, kSplitPlane = kSplitRows * kSplitCols * 2, kSplitBlock = 3 * kSplitPlane;
 inline size_t split_bytes(int rows, int cols) { return (size_t)(rows / kSplitRows) * (cols / kSplitCols) * kSplitBlock; }
 
-// out = split(a - b) (b may be null) of [rows][cols] fp32, leading dimension lda (multiple of 4), padded with zeros to rows_p x cols_p.  copy
+// out (may be null) = split(a - b) (b may be null) of [rows][cols] fp32, leading dimension lda, padded with zeros to rows_p x cols_p.  copy
 // (may be null): a - b itself, padded, as [rows_p][cols_p] fp32, rows ld_copy apart.
 cudaError_t split_rows(cudaStream_t st, const float* a, const float* b, int rows, int cols, int lda, int rows_p, int cols_p, uint8_t* out, float* copy,
                        int ld_copy);
@@ -19,7 +19,7 @@ cudaError_t split_rows(cudaStream_t st, const float* a, const float* b, int rows
 cudaError_t split_cols(cudaStream_t st, const float* a, int rows, int cols, int lda, int rows_p, int cols_p, uint8_t* out, float* copy = nullptr);
 
 // C [m][ldc] = A B^T with A [m][k] and B [n][k] split as above; m, n, k multiples of 128.  sym: A and B are the same operand, and only tiles
-// on and below the diagonal are computed and stored to both places.  add: C += instead (not with sym).  status: set to 1 if a wait inside the kernel ran out.
+// on and below the diagonal are computed and stored to both places.  add: C += instead.  status: not zero if a wait inside the kernel ran out.
 cudaError_t split_gemm(cudaStream_t st, const uint8_t* a, const uint8_t* b, int m, int n, int k, float* c, int ldc, bool sym, bool add, int sm_count,
                        int* status);
 

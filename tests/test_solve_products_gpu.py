@@ -71,3 +71,35 @@ def test_what_is_not_finite_shows_in_every_result(d, k, n, r, where, value):
     torch.cuda.synchronize()
     for name, v in (("B'", b), ("A", a), ("sigma", s)):
         assert not bool(torch.isfinite(v).any()), name
+
+
+@pytest.mark.parametrize("d,k,n,r", [
+    (1024, 1024, 4000, 60),     # without room beyond the matrices: dW's place used in between, every product but C's own in parts
+    (1500, 1024, 1000, 60),     # the same on the n side
+    (1500, 300, 1000, 60),      # few inputs: C split over itself in slabs; in the smallest workspace products with C itself
+    (1100, 200, 1300, 60),      # the same on the d side
+    (1700, 300, 1300, 30),      # an iterate's parts among the matrices', not among the small problems
+    (60, 40, 3000, 20),         # small matrices, many columns
+])
+def test_workspaces_down_to_the_matrices_alone(d, k, n, r):
+    """The reported workspace, less than that, and one that holds dW, P, C and the iterates and nothing else: results as ever, and nothing behind it is touched."""
+    import torch
+    import paper_2410_21271_b200 as eora
+    from test_solve_plan_cpu import matrices
+    w, w_hat, x = gen.make_solve_case(45, d, k, n, kind="gap", rank_signal=r)
+    ref = sol.solve(w, w_hat, x, r)
+    want = ref["B"] @ ref["A"]
+    cfg = eora.eora_solve_config(d, k, n, r, 0, 0)
+    tw, th, tx = (torch.from_numpy(v).cuda() for v in (w, w_hat, x))
+    most = eora.eora_solve_workspace_bytes(cfg)
+    for size in sorted({most, max(most - 1, matrices(d, k, n, r)), matrices(d, k, n, r)}):
+        ws = torch.full((size + 65536,), 0xA5, dtype=torch.uint8, device="cuda:0")
+        b, a, s = torch.empty((d, r), device="cuda:0"), torch.empty((r, k), device="cuda:0"), torch.empty(r, device="cuda:0")
+        loss = torch.zeros(1, dtype=torch.float64, device="cuda:0")
+        eora.eora_solve(cfg, tw, th, tx, b, a, s, ws[:size])
+        eora.eora_solve_loss(cfg, tw, th, tx, b, a, loss, ws[:size])
+        torch.cuda.synchronize()
+        assert bool((ws[size:] == 0xA5).all())
+        got = b.cpu().numpy().astype(np.float64) @ a.cpu().numpy()
+        assert np.linalg.norm(got - want) <= PRODUCT_RTOL * np.linalg.norm(want)
+        assert np.linalg.norm(s.cpu().numpy() - ref["sigma"]) <= SIGMA_RTOL * np.linalg.norm(ref["sigma"])
