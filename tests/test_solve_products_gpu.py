@@ -17,13 +17,14 @@ SIGMA_RTOL = 1e-6
 
 
 @pytest.mark.parametrize("d,k,n,r", [
-    (4736, 256, 1024, 24),      # 37 x 8 tiles: the wide tile; n side
+    (4736, 256, 1024, 24),      # 37 x 8 tiles: the wide tile; n side, an iterate of 56 columns on the CUDA cores
     (128, 128, 128, 8),         # one tile, four stages
     (300, 1100, 500, 40),       # padded everywhere; chunks of eight stages with a remainder
-    (1024, 320, 384, 100),      # iterate of 132 columns: two tiles of 96
+    (1024, 320, 384, 100),      # iterate of 132 columns: two tiles of 96, on the CUDA cores
     (700, 640, 900, 250),       # 282 columns: three tiles of 96, two blocks of the factor
     (640, 600, 700, 400),       # 432 columns: three blocks of the factor
     (1000, 1000, 1100, 480),    # 512 columns: four
+    (512, 520, 600, 268),       # 300 columns on the tensor cores: two tiles of 160, the second beginning inside a block
 ])
 def test_compensation_and_spectrum(d, k, n, r):
     w, w_hat, x = gen.make_solve_case(41, d, k, n, kind="gap", rank_signal=r)
@@ -103,3 +104,33 @@ def test_workspaces_down_to_the_matrices_alone(d, k, n, r):
         got = b.cpu().numpy().astype(np.float64) @ a.cpu().numpy()
         assert np.linalg.norm(got - want) <= PRODUCT_RTOL * np.linalg.norm(want)
         assert np.linalg.norm(s.cpu().numpy() - ref["sigma"]) <= SIGMA_RTOL * np.linalg.norm(ref["sigma"])
+
+
+def test_more_tiles_than_clusters_of_two():
+    """An iterate of 512 columns with 2432 rows: 76 tiles of its product with C, a CTA each."""
+    d, k, n, r = 2432, 600, 2500, 32
+    w, w_hat, x = gen.make_solve_case(46, d, k, n, kind="gap", rank_signal=r)
+    ref = sol.solve(w, w_hat, x, r)
+    want = ref["B"] @ ref["A"]
+    b, a, s, _ = run_solve(w, w_hat, x, r, oversample=480)
+    assert np.linalg.norm(b @ a - want) <= PRODUCT_RTOL * np.linalg.norm(want)
+    assert np.linalg.norm(s - ref["sigma"]) <= SIGMA_RTOL * np.linalg.norm(ref["sigma"])
+
+
+def test_tensor_core_products_side_by_side_on_three_streams():
+    """Three solves whose clusters share the GPU: every one gives what it gives alone, bit for bit."""
+    import torch
+    import paper_2410_21271_b200 as eora
+    cases = [(1024, 900, 1100, 64), (1500, 1024, 1024, 100), (900, 1024, 1000, 128)]
+    ins = [(tuple(torch.from_numpy(v).cuda() for v in gen.make_solve_case(47 + i, d, k, n)), r) for i, (d, k, n, r) in enumerate(cases)]
+    alone = [eora.solve(*t, r) for t, r in ins]
+    torch.cuda.synchronize()
+    streams = [torch.cuda.Stream() for _ in cases]
+    for rep in range(3):
+        outs = []
+        for st, (t, r) in zip(streams, ins):
+            with torch.cuda.stream(st):
+                outs.append(eora.solve(*t, r, stream=st))
+    torch.cuda.synchronize()
+    for one, other in zip(alone, outs):
+        assert all(torch.equal(u, v) for u, v in zip(one, other))
