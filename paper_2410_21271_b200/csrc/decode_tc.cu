@@ -35,6 +35,7 @@
 #include <type_traits>
 #include <vector>
 #include "decode_common.cuh"
+#include "tcgen05.cuh"
 #include "tmat.cuh"
 
 namespace eora {
@@ -97,9 +98,6 @@ __device__ __forceinline__ void issue_unit(uint32_t d, uint32_t a, uint32_t blo,
   issue_one<I8, 1>(d, a, blo, bhi, idesc);
   if constexpr (N > 2) { issue_one<I8, 2>(d, a, blo, bhi, idesc); issue_one<I8, 3>(d, a, blo, bhi, idesc); }
 }
-__device__ __forceinline__ void umma_commit_tc(uint64_t* bar) {
-  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar)) : "memory");
-}
 __device__ __forceinline__ void tmem_st8(uint32_t taddr, const uint32_t* r) {
   asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};"
                ::"r"(taddr), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]) : "memory");
@@ -127,12 +125,6 @@ __device__ __forceinline__ void st_shared_v4u(uint32_t addr, uint4 v) {
   asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w) : "memory");
 }
 
-// K-major, 128-byte swizzle operand descriptor: rows of 128 B, 8-row groups 1024 B apart (the activation operand).
-__device__ __forceinline__ uint64_t make_desc_tc(uint32_t addr) {
-  const uint32_t lo = ((addr & 0x3FFFFu) >> 4) | (1u << 16);
-  const uint32_t hi = (1024u >> 4) | (1u << 14) | (2u << 29);
-  return ((uint64_t)hi << 32) | lo;
-}
 // byte offset of byte kb (0..127) of row n inside an activation stage (128-byte swizzle)
 __device__ __forceinline__ uint32_t x_off(uint32_t n, uint32_t kb) {
   return (n >> 3) * 1024u + (n & 7u) * 128u + ((((kb >> 4) ^ (n & 7u)) << 4) | (kb & 15u));
@@ -673,7 +665,7 @@ __global__ void __launch_bounds__(TcShape<MT>::kThreads, TcShape<MT>::kCtasPerSm
     const int set = warp >> 2, quad = warp & 3;
     const int rr = quad * 32 + lane;                      // this thread's row of every unit
     const uint32_t lane_base = tmem + ((uint32_t)(quad * 32) << 16) + set * kSetCols;
-    const uint64_t bdesc0 = make_desc_tc(smem_u32(xst));
+    const uint64_t bdesc0 = make_desc<128>(smem_u32(xst));
     const uint32_t blo0 = (uint32_t)bdesc0, bhi = (uint32_t)(bdesc0 >> 32);
     float acc[MT];
 #pragma unroll
@@ -766,7 +758,7 @@ __global__ void __launch_bounds__(TcShape<MT>::kThreads, TcShape<MT>::kCtasPerSm
           const uint32_t a = tmem + set * kSetCols, d = a + kACols, blo = blo0 + sx * (kXStage >> 4);
           if (seg == SEG_W) issue_unit<WF, NCOL>(d, a, blo, bhi);
           else if constexpr (ABF != FMT_NONE) issue_unit<ABF, NCOL>(d, a, blo, bhi);
-          umma_commit_tc(sh.mma_done + set);
+          umma_commit(sh.mma_done + set);
         }
       }
       // ---- read the rows back

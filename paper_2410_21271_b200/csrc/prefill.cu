@@ -26,6 +26,7 @@
 // bf16 weights alone cost 1.7e-3 of the 2e-3 error budget).
 #include <cuda.h>
 #include "decode_common.cuh"
+#include "tcgen05.cuh"
 
 namespace eora {
 using namespace dec;
@@ -102,10 +103,6 @@ __device__ __forceinline__ void tma_load_2d(void* dst, const CUtensorMap* tm, in
   asm volatile("cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];"
                ::"r"(smem_u32(dst)), "l"(tm), "r"(c0), "r"(c1), "r"(smem_u32(bar)) : "memory");
 }
-__device__ __forceinline__ void umma_f16(uint32_t tmem_d, uint64_t adesc, uint64_t bdesc, uint32_t idesc, uint32_t accumulate) {
-  asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\ttcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
-               ::"r"(tmem_d), "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate) : "memory");
-}
 // The same with the 128-row operand in tensor memory: lane = row, one 32-bit column = two reduction elements.
 __device__ __forceinline__ void umma_f16_ts(uint32_t tmem_d, uint32_t tmem_a, uint64_t bdesc, uint32_t idesc, uint32_t accumulate) {
   asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\ttcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}"
@@ -116,17 +113,6 @@ __device__ __forceinline__ void tmem_st16x32(uint32_t taddr, const uint32_t (&v)
   asm volatile("tcgen05.st.sync.aligned.16x256b.x4.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, %16};"
                ::"r"(taddr), "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]), "r"(v[4]), "r"(v[5]), "r"(v[6]), "r"(v[7]), "r"(v[8]), "r"(v[9]),
                  "r"(v[10]), "r"(v[11]), "r"(v[12]), "r"(v[13]), "r"(v[14]), "r"(v[15]) : "memory");
-}
-__device__ __forceinline__ void umma_commit(uint64_t* bar) {
-  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar)) : "memory");
-}
-__device__ __forceinline__ void umma_commit_a(uint32_t bar) {
-  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
-}
-__device__ __forceinline__ bool elect_one() {
-  uint32_t p;
-  asm volatile("{\n\t.reg .pred q;\n\telect.sync _|q, 0xffffffff;\n\tselp.u32 %0, 1, 0, q;\n\t}" : "=r"(p));
-  return p != 0;
 }
 // 16 lanes x 32 columns as fragments of 8 x 8 blocks: registers 4 c .. 4 c + 3 hold columns 8 c + 2 (lane % 4) and the next one of
 // lane lane / 4, then of lane lane / 4 + 8.
@@ -152,14 +138,6 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&v)[32]) {
                  "=r"(v[17]), "=r"(v[18]), "=r"(v[19]), "=r"(v[20]), "=r"(v[21]), "=r"(v[22]), "=r"(v[23]), "=r"(v[24]),
                  "=r"(v[25]), "=r"(v[26]), "=r"(v[27]), "=r"(v[28]), "=r"(v[29]), "=r"(v[30]), "=r"(v[31])
                : "r"(taddr) : "memory");
-}
-
-// K-major, 128-byte swizzle operand descriptor: rows of 128 B, 8-row groups 1024 B apart.
-__device__ __forceinline__ uint64_t make_desc(const void* smem_ptr) {
-  const uint32_t addr = smem_u32(smem_ptr);
-  const uint32_t lo = ((addr & 0x3FFFFu) >> 4) | (1u << 16);            // start address, leading byte offset (unused) = 1
-  const uint32_t hi = (1024u >> 4) | (1u << 14) | (2u << 29);           // stride byte offset, descriptor version 1, SWIZZLE_128B
-  return ((uint64_t)hi << 32) | lo;
 }
 
 // packed tile payload of one lane, by format
@@ -752,7 +730,7 @@ __global__ void __launch_bounds__(kThreadsP, 1) k_prefill(const __grid_constant_
     // instruction descriptor: fp32 accumulate, fp16 x fp16, both operands K-major, M = 128 weight rows, N = bt tokens
     const uint32_t idesc = (1u << 4) | ((uint32_t)(bt >> 3) << 17) | ((uint32_t)(BN_W >> 4) << 24);
     const bool elected = elect_one();
-    const uint64_t bdesc0 = make_desc(smem), adesc0 = make_desc(smem + p.w_off);
+    const uint64_t bdesc0 = make_desc<128>(smem_u32(smem)), adesc0 = make_desc<128>(smem_u32(smem + p.w_off));
     const uint32_t bstep = xslot >> 4, astep = (uint32_t)p.w_slot >> 4;       // from one ring slot to the next, in 16-byte units
     const uint32_t full0 = smem_u32(full_w), empty0 = smem_u32(empty_w);
     bool ok = true;

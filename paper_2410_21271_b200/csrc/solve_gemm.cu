@@ -15,6 +15,7 @@
 // Operands are split and laid out as the tensor core reads them by a pass of their own (2 x 3 x 2 bytes per value, 15 to 35 us).
 #include <cuda_bf16.h>
 #include "decode_common.cuh"
+#include "tcgen05.cuh"
 #include "solve_gemm.cuh"
 
 namespace eora {
@@ -120,18 +121,6 @@ __host__ __device__ constexpr int gemm_stage(int nt) { return (kSplitRows + nt) 
 __host__ __device__ constexpr int gemm_stages(int nt) { return nt == 256 ? 3 : 4; }
 constexpr int gemm_smem(int nt) { return gemm_stage(nt) * gemm_stages(nt) + 1024; }
 
-__device__ __forceinline__ void umma_bf16(uint32_t tmem_d, uint64_t adesc, uint64_t bdesc, uint32_t idesc, uint32_t accumulate) {
-  asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\ttcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
-               ::"r"(tmem_d), "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate) : "memory");
-}
-__device__ __forceinline__ void umma_commit(uint64_t* bar) {
-  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar)) : "memory");
-}
-__device__ __forceinline__ bool elect_one() {
-  uint32_t p;
-  asm volatile("{\n\t.reg .pred q;\n\telect.sync _|q, 0xffffffff;\n\tselp.u32 %0, 1, 0, q;\n\t}" : "=r"(p));
-  return p != 0;
-}
 __device__ __forceinline__ void tmem_add8(uint32_t taddr, float* acc) {
   uint32_t v[8];
   asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
@@ -139,12 +128,6 @@ __device__ __forceinline__ void tmem_add8(uint32_t taddr, float* acc) {
   asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 #pragma unroll
   for (int i = 0; i < 8; ++i) acc[i] += __uint_as_float(v[i]);
-}
-// K-major, 64-byte swizzle operand descriptor: rows of 64 B, 8-row groups 512 B apart.
-__device__ __forceinline__ uint64_t make_desc64(uint32_t addr) {
-  const uint32_t lo = ((addr & 0x3FFFFu) >> 4) | (1u << 16);
-  const uint32_t hi = (512u >> 4) | (1u << 14) | (4u << 29);
-  return ((uint64_t)hi << 32) | lo;
 }
 
 // The barriers of a CTA and its tensor memory: high x high in columns [0, NT), the rest in [256, 256 + NT).
@@ -214,7 +197,7 @@ __device__ __forceinline__ bool gemm_tile(GemmShared& sh, uint32_t smem, int war
     constexpr uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(NT >> 3) << 17) | ((128u >> 4) << 24);      // fp32 += bf16 x bf16
     const bool elected = elect_one();
     const uint32_t tmem = sh.tmem, small = tmem + kSmallCol;
-    const uint64_t a0 = make_desc64(smem), b0 = make_desc64(smem + kA);
+    const uint64_t a0 = make_desc<64>(smem), b0 = make_desc<64>(smem + kA);
     constexpr uint32_t pa = kSplitPlane >> 4, pb = kPlaneB >> 4;
     bool ok = true;
     uint32_t s = 0, ph = 0;
@@ -227,15 +210,15 @@ __device__ __forceinline__ bool gemm_tile(GemmShared& sh, uint32_t smem, int war
       const bool last = pos == kChunk - 1 || it == nkb - 1;
       if (elected) {
 #pragma unroll
-        for (int k = 0; k < 2; ++k) umma_bf16(tmem, ad + 2 * k, bd + 2 * k, idesc, pos > 0 || k > 0 ? 1u : 0u);
+        for (int k = 0; k < 2; ++k) umma_f16(tmem, ad + 2 * k, bd + 2 * k, idesc, pos > 0 || k > 0 ? 1u : 0u);
         if (last) umma_commit(&sh.d0_full);
 #pragma unroll
         for (int k = 0; k < 2; ++k) {
-          umma_bf16(small, ad + 2 * k, bd + pb + 2 * k, idesc, it > 0 || k > 0 ? 1u : 0u);
-          umma_bf16(small, ad + pa + 2 * k, bd + 2 * k, idesc, 1u);
-          umma_bf16(small, ad + 2 * k, bd + 2 * pb + 2 * k, idesc, 1u);
-          umma_bf16(small, ad + 2 * pa + 2 * k, bd + 2 * k, idesc, 1u);
-          umma_bf16(small, ad + pa + 2 * k, bd + pb + 2 * k, idesc, 1u);
+          umma_f16(small, ad + 2 * k, bd + pb + 2 * k, idesc, it > 0 || k > 0 ? 1u : 0u);
+          umma_f16(small, ad + pa + 2 * k, bd + 2 * k, idesc, 1u);
+          umma_f16(small, ad + 2 * k, bd + 2 * pb + 2 * k, idesc, 1u);
+          umma_f16(small, ad + 2 * pa + 2 * k, bd + 2 * k, idesc, 1u);
+          umma_f16(small, ad + pa + 2 * k, bd + pb + 2 * k, idesc, 1u);
         }
         umma_commit(sh.empty + s);
       }
