@@ -485,10 +485,6 @@ def time_single_layer(device: str, K: int, N: int, w: str, r: int, M: int, copie
     return e0.elapsed_time(e1) / (iters * copies)
 
 
-# Peak of the fp32 FMA pipe: 148 SMs x 128 lanes x 2 flops x 1.965 GHz (unit counts and maximum clock of the part).
-FP32_PEAK_TFLOPS = 148 * 128 * 2 * 1.965e9 / 1e12
-
-
 def time_solve(device: str, d: int = 4096, k: int = 4096, n: int = 2048, r: int = 128, reps: int = 3, cpu: bool = True):
     """Extra: the offline solve (Algorithm 1 steps 1-6) of one q-shaped layer: weight 4096 x 4096, 2048 calibration
     columns, rank 128, library defaults (32 extra vectors, 14 products with the square).  Flops = those of the contractions the
@@ -511,12 +507,13 @@ def time_solve(device: str, d: int = 4096, k: int = 4096, n: int = 2048, r: int 
     side, other = (n, d) if m <= n < d else (d, n)        # the library iterates with the smaller square that holds m directions
     flops = 2.0 * d * k * n + 1.0 * side * side * other + iters * 2.0 * side * side * m + (2.0 * d * n * m if side == n else 0.0) \
         + 2.0 * d * n * m + 2.0 * d * m * r + 2.0 * r * d * k + 2.0 * r * k * n
+    peak = measured_peaks()[0]["bf16_tflops"] / 6          # six bf16 MMAs per fp32 product
     loss = eora.solve_loss(tw, th, tx, b, a)
     uncompensated = float(torch.linalg.norm((tw - th).double() @ tx.double()))
     out = {"workload": f"one layer {d}x{k}, {n} calibration columns, rank {r}", "ms": ms, "layers_per_s": 1e3 / ms,
-           "gflop": flops / 1e9, "tflops": flops / ms / 1e9, "bound": "latency", "peak_tflops_fp32": FP32_PEAK_TFLOPS,
-           "products": "fp32 accuracy, large ones as three bf16 parts per value on the tensor cores: not bounded by the fp32 FMA peak",
-           "frac_of_fp32_peak": flops / ms / 1e9 / FP32_PEAK_TFLOPS,
+           "gflop": flops / 1e9, "tflops": flops / ms / 1e9, "bound": "latency",
+           "products": "fp32 accuracy: three bf16 parts per value and six MMAs per product on the tensor cores, small ones on the CUDA cores",
+           "peak_tflops": peak, "frac_of_peak": flops / ms / 1e9 / peak,
            "remaining_loss_over_uncompensated": loss / uncompensated, "dtype": "f32 (f64 for the small problems)"}
     # Independent layers (q, k, v share one input; gate and up another) can be solved side by side: each solve is a
     # chain of launches on its own stream with its own workspace, and the one-CTA factorisations of one layer run beside
@@ -544,7 +541,7 @@ def time_solve(device: str, d: int = 4096, k: int = 4096, n: int = 2048, r: int 
     ms_c = e0.elapsed_time(e1) / (n_streams * per_stream)
     same = all(bool(torch.equal(bb, b)) and bool(torch.equal(aa, a)) for _, bb, aa, _ in bufs)
     out["side_by_side"] = {"streams": n_streams, "solves": n_streams * per_stream, "ms_per_layer": ms_c, "layers_per_s": 1e3 / ms_c,
-                           "tflops": flops / ms_c / 1e9, "frac_of_fp32_peak": flops / ms_c / 1e9 / FP32_PEAK_TFLOPS,
+                           "tflops": flops / ms_c / 1e9, "frac_of_peak": flops / ms_c / 1e9 / peak,
                            "results_equal_to_the_single_stream_solve": same}
     del bufs
     if cpu:

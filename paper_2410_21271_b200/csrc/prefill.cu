@@ -417,13 +417,13 @@ __device__ __forceinline__ bool dequant_part(const WMat& mat, int n0, int kb_lo,
 // Up to 160 tokens (256 with 128 rows) the accumulators leave tensor memory for the dequantised weights.  Through shared memory a k-block of 256 rows x
 // 64 tokens moved 32 KB of weights in and out of it, 512 cycles of its bandwidth, and each hand-over waited for the stores to become visible to the
 // MMAs (1215 cycles a k-block); here the weights go from registers to tensor memory and the MMAs read only the tokens from shared memory (790).  A 4-bit
-// LLaMA3-8B block of 64 tokens with 8-bit adapters of rank 512: 139 -> 114 us; of 128 tokens, rank 128, 124 -> 105; of a prompt of 333 235 -> 204.
+// LLaMA3-8B block of 64 tokens with 8-bit adapters of rank 512: 139 -> 114 us; of 128 tokens, rank 128, 124 -> 105; of a prompt of 333 238 -> 218.
 // Tried and not kept: two chains of MMAs with accumulators of their own (128 rows 515 -> 562 cycles).
 //
 // tcgen05.st writes a tile of 16 rows x 64 reduction elements as fragments of 8 x 8 32-bit blocks: lane (g, t) holds, for each of the four MMAs j of a
 // k-block, elements 16 j + 4 t .. + 3 of rows g and g + 8.  In the packed layout these are half (t & 1) of the eight codes that
-// lane (g, 2 (j & 1) + (t >> 1)) owns of the 32-element block j / 2.  So every warp brings its blobs to shared memory (a ring of its own,
-// asked for before anything else in the kernel) and its lanes read the words of those two lanes.
+// lane (g, 2 (j & 1) + (t >> 1)) owns of the 32-element block j / 2.  So every warp brings its blobs to shared memory (a ring of its own;
+// the first of W are asked for as soon as the barriers and tensor memory are set up, those of B behind all of W) and its lanes read the words of those two lanes.
 // out[4 j + 2 hf + i]: elements 16 j + 4 t + 2 i, + 1 of row g + 8 hf, as fp16 RN((q - z) * s).
 template <int FMT>
 __device__ __forceinline__ void tm_tile(uint32_t tile, int lane, const ZC& zc, uint32_t s_a, uint32_t s_b, uint32_t (&out)[16]) {

@@ -1,6 +1,6 @@
 // Offline EoRA solve (Algorithm 1, steps 1-6) on the GPU; the interface and the mathematics are in eora_solve.h.
 //
-//   1.  dW = W - W^                                                    (k_sub)
+//   1.  dW = W - W^                                                    (k_split_rows, on the way to its three parts)
 //   2-4 the paper projects dW into the eigenspace of X~ X~^T, dW' = dW Q sqrt(L).  Only dW' dW'^T = P P^T with P = dW X~
 //       (d x n) is needed here.
 //   5.  top-r eigenpairs (U', S'^2) of P P^T by subspace iteration on m = r + oversample vectors:
@@ -456,7 +456,7 @@ __host__ __device__ constexpr int chol_smem(int m) { return (m * (m | 1) + m + 1
 // columns of norm 1 / f->scale, else through one with C: the diagonal of L then says where the eigenvalues of the iterate's columns are.
 // The next pair's shifts are lo and hi times the smallest of them.
 struct Filter { float rho[2]; double scale; };
-constexpr double kFilterEdge = 0.95;                 // the estimate comes from below, but not always (measured 0.8 to 1.07 of eigenvalue m after four steps)
+constexpr double kFilterEdge = 0.95;                 // the estimate comes from below, but not always (measured 0.8 to 1.07 of eigenvalue m after four steps; 1.3 on a plateau with few extra vectors, where the points then lie a little high and the loss is still half the plain iteration's)
 __global__ void __launch_bounds__(kCholThreads) k_chol64(double* L0, int ld, int m_all, int j_base, int m, double* __restrict__ Dinv, double* least_g, Filter* f, bool prev, double lo, double hi) {
   extern __shared__ __align__(16) double sm[];
   __shared__ double dv[16][17];
